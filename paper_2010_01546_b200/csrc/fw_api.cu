@@ -609,8 +609,6 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
   st = resync_phiy(L, n);
   if (st != FW_OK) return st;
   if (K == 0) return FW_OK;      // no step: Phi_y has been brought up to date, nothing else changes
-  GroupDev g; int max_M, max_N;
-  fill_group(L, n, g, max_M, max_N);
   // small layers: the whole K-step recursion runs on chip, a layer on 1 to 16 CTAs of a cluster;
   // the rest takes the multi-launch path (one launch per pass, batched over layers)
   GroupDev gc, gl; PtrTable tc, tl;
@@ -678,7 +676,7 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
   }
   bool any_beta = false;
   for (int i = 0; i < n; ++i) any_beta |= (L[i]->d.beta > 0.f);
-  if (any_beta) FW_CUDA(launch_smooth(g, max_M, s), "smooth");
+  if (gl.n && any_beta) FW_CUDA(launch_smooth(gl, ml, s), "smooth");
   for (int i = 0; i < n; ++i) L[i]->t_identity = false;
   return FW_OK;
 }

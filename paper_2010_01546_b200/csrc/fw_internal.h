@@ -222,6 +222,7 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
 bool recursion_cluster_supported(int M);
 // CTAs of a 16-CTA cluster the on-chip recursion gives a layer of size M (1, 2, 4, 8, 16; 0: not on chip)
 int recursion_cluster_ctas(int M);
+// All K steps of a call for layers that fit on chip, T, Q and Qs included
 cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
                                      cudaStream_t s);
 // All K steps of a group of large gamma = 1 layers as one persistent cooperative launch.  bar_words: two ints in the

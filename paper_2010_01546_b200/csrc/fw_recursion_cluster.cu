@@ -1,32 +1,35 @@
-// On-chip recursion for small layers (Sec. 4): a layer's whitened covariance
-// Phi_y AND its transform T^T stay resident in distributed shared memory for
-// all K steps of a call.  The launch uses thread-block clusters of 16 CTAs; a
-// layer takes n = 1 ... 16 consecutive CTAs of one cluster (at least as many
-// as its slabs need; more while the clusters of one wave allow and the layer
-// is the launch's slowest), so a cluster carries one large layer or several
-// small ones and every SM does a similar amount of work per pass.  CTA `sub`
-// of a layer owns a slab of rows of both matrices; every pass of a step is a
-// slab-times-vector product out of shared memory.  The passes are chained as a
-// dataflow: each CTA pushes its slice of a result straight into all peers'
-// copies of the vector with asynchronous remote stores that count bytes on the
-// receiver's mbarrier, and every CTA waits only on its own barrier.  No
-// cluster-wide barrier is taken inside a step, and the partial sums a pass
-// needs next (squared norm, v.u) travel with the slices.  Global memory is
-// touched three times per call: the slabs come in, the slabs go out, and Q
-// takes the rank-one terms of the steps (Eq. 44) a few steps at a time -- the
-// recursion itself never reads Q.
+// On-chip recursion for small layers (Sec. 4): a layer's whitened covariance Phi_y
+// stays on chip for all steps of a launch, each warp's rows in its registers, with
+// a copy in shared memory for the row m' a step sends round.  The launch uses
+// thread-block clusters; a layer takes n = 1 ... 16 consecutive CTAs of one
+// cluster (at least as many as its rows need; more while the clusters of one wave
+// allow and the layer is the launch's slowest).  CTA `sub` of a layer owns a slab
+// of rows; every pass of a step is a slab-times-vector product.  The passes are
+// chained as a dataflow: each warp pushes its slice of a result straight into all
+// CTAs' copies of the vector with asynchronous remote stores that count bytes on
+// the receiver's mbarrier, and every warp waits on its own CTA's barrier -- no
+// block or cluster barrier separates the power iterations.  T and Q are not
+// needed by a step, so a step only records its v_e and a_e; after the last step
+// (or every KH) each warp loads its rows of T^T, forms t = T^T v_e step by step,
+// and T and Q take the rank-one terms (Eqs. 42, 44) in step order: the product
+// T^T v is out of the chain and the rows of T^T out of shared memory.
 //
-// Buffer reuse is safe without further synchronisation: a peer can send
-// exchange e + 1 only after it received this CTA's slice of exchange e, so
-// while this CTA works between its sends e and e + 1 only the target of
-// exchange e + 1 can change under it, and that buffer is never read in that
-// window (vectors alternate, partial-sum slots and barriers are double-buffered).
+// What bounds it: the chain of P + 5 dependent exchanges per step.  A pass reads
+// only the vector from shared memory (rows in registers: at M = 576 the slab's 83
+// KB per pass alone would take 0.35 us of shared-memory bandwidth), so what is
+// left is the latency of the reduction, the remote store and the wait.
 //
-// The arithmetic is that of the multi-launch path in fw_recursion.cu (same
-// passes, symmetric evaluation of the rank updates); dot products are accumulated
-// in fp32 here (rows are at most ~600 long and split over two accumulators).
+// Buffer reuse is safe without further synchronisation: a CTA can send exchange
+// e + 1 only after it received every warp's slice of exchange e, and a warp sends
+// its slice after its last read of the pass's input; vectors alternate and the
+// barriers are double-buffered.  Warps that own no rows take no part in the steps.
+//
+// Dot products are accumulated in fp32 (rows are at most 624 long and split over
+// two accumulators per lane); rank updates are evaluated symmetrically.
 #include <cooperative_groups.h>
+#include <algorithm>
 #include <cstring>
+#include <mutex>
 
 #include "fw_internal.h"
 #include "fw_sm100.cuh"
@@ -38,21 +41,23 @@ namespace {
 
 using sm100::smem_u32;
 
-constexpr int CL = 16;             // CTAs per cluster of the launch
+constexpr int CLMAX = 16;          // largest cluster (beyond 8: non-portable size)
 constexpr int CT = 512;            // threads per CTA
 constexpr int CW = CT / 32;        // warps per CTA
-constexpr int MAXGPW = 2;          // groups of four rows per warp, at most (rows per CTA <= 128); three were
-                                   // measured: twelve rows per warp cost 1.8 us per pass (13 values through five
-                                   // shuffle rounds) against 1.1 us for eight
-constexpr int kMaxIt = 5;          // float4 columns per lane, at most (rows of at most 640 entries)
-constexpr int KQ = 4;              // steps whose rank-one terms of Q are applied together
-constexpr size_t kSmemLimit = 226 * 1024;   // plus the static variables below: within the 227 KB of a CTA
+constexpr int kMaxIt = 5;          // float4 columns per lane, at most
+constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take the fp64 passes
+constexpr int KH = 8;              // steps between two updates of T and Q
+constexpr size_t kSmemLimit = 226 * 1024 - 512;   // plus the static variables below: within the 227 KB of a CTA
+
+// A warp owns one group of four rows (up to kMaxIt float4 columns per lane: 80 registers) or, for rows of at most 256
+// entries, two (64 registers).
+__host__ __device__ constexpr int max_groups(int it) { return it <= 2 ? 2 : 1; }
 
 struct ClusterArgs {
   GroupDev g;
   PtrTable traces;
   int32_t first_cta[FW_MAX_GROUP];   // first CTA of each layer (a layer never straddles a cluster)
-  int32_t ncta[FW_MAX_GROUP];        // CTAs of each layer: 1 ... 16
+  int32_t ncta[FW_MAX_GROUP];        // CTAs of each layer: 1 ... cluster size
   int32_t K, P;
 };
 
@@ -62,9 +67,9 @@ __device__ __forceinline__ uint32_t map_cluster(uint32_t saddr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
-// asynchronous 16-byte store into a peer's shared memory; the peer's mbarrier counts the bytes.  One message
-// carries four results: the receiver's barrier takes a few clocks per message, so the count of messages, not
-// their size, is what an exchange costs.
+// asynchronous 16-byte store into a CTA's shared memory; its mbarrier counts the bytes.  One message carries four
+// results: the receiver's barrier takes a few clocks per message, so the count of messages, not their size, is what
+// an exchange costs.
 __device__ __forceinline__ void st_async_v4(uint32_t raddr, float4 v, uint32_t rbar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                ::"r"(raddr), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
@@ -73,38 +78,30 @@ __device__ __forceinline__ void st_async_v4(uint32_t raddr, float4 v, uint32_t r
 __device__ __forceinline__ void cp_async16(uint32_t saddr, const float* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(g) : "memory");
 }
-__device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Bounded wait of the whole CTA for an exchange to land; the verdict is uniform over the CTA.
-// The block barrier inside also publishes the slice this CTA stored into its own copy.
-// Only the first warp polls (the others sleep at the block barrier and leave the issue slots to the warps
-// still at work); its acquire together with the barrier makes the received data visible to every thread.
-__device__ __forceinline__ bool exchange_wait(uint32_t bar, uint32_t parity) {
-  bool ok = true;
-  if (threadIdx.x < 32) {
-    ok = false;
-    for (uint32_t i = 0; i < sm100::kSpinLimit; ++i)
-      if (try_wait_cluster(bar, parity)) { ok = true; break; }
-  }
-  return __syncthreads_and(ok) != 0;
-}
 
+// What a CTA knows about its layer; lives in shared memory (the threads' registers hold matrix rows).
 struct Slab {
   float* phi;     // my rows of Phi_y in shared memory, leading dimension Mp
-  float* tt;      // my rows of T^T, same shape
+  float* xi2; float* cvec; float* wvec; float* buf0; float* uvec;   // vectors of Mv floats; buf0: two, Mv apart
+  float* vh; float* th;   // v_e and t of the recorded steps, KH vectors each
   int M, Mp;      // matrix size, padded row length
+  int Mv;         // vector length in shared memory
   int R;          // rows per CTA, a multiple of four (rows past the matrix are zero rows)
   int row0, nrows;  // my first row; how many of my rows are rows of the matrix
   int n;          // CTAs of this layer
   int sub;        // my index among them
-  uint32_t rdelta;  // lane p < n: cluster address of peer p's shared memory minus this CTA's own
+  uint32_t tx;    // bytes of one exchanged vector
+  int maxcol;     // start vector: largest column instead of the alignment
+  float c_rel, c_abs, delta, eps, lam_bar;
+  float ah[KH];   // a_e of the recorded steps
+  int fail;       // set once a bounded wait of this CTA gave up
+};
+// The parts of it every pass needs, in registers.
+struct Link {
+  uint32_t rdelta;  // lane p < n: cluster address of CTA p's shared memory minus this CTA's own
+  uint32_t bar0;    // two exchange barriers, 8 bytes apart
+  int n;
+  int active;       // threads of the warps that own rows; the others take no part in the steps
 };
 
 // 1/sqrt(n2) refined by one Newton step, 0 when n2 is not a positive finite number
@@ -112,84 +109,442 @@ __device__ __forceinline__ float inv_norm(float n2) {
   float inv = (n2 > 0.f && isfinite(n2)) ? rsqrtf(n2) : 0.f;
   return inv > 0.f ? inv * (1.5f - 0.5f * n2 * inv * inv) : 0.f;
 }
-
-// x . y over the first Mp entries, by one warp; every warp of every CTA of a layer adds in the same order, so all
-// of them hold the same bits
-__device__ __forceinline__ float warp_dot(const float* x, const float* y, int Mp) {
-  const int lane = threadIdx.x & 31;
-  const float4* x4 = reinterpret_cast<const float4*>(x);
-  const float4* y4 = reinterpret_cast<const float4*>(y);
-  float a0 = 0.f, a1 = 0.f;
-  for (int c = lane; c < (Mp >> 2); c += 32) {
-    const float4 a = x4[c], b = y4[c];
-    a0 = fmaf(a.x, b.x, a0); a1 = fmaf(a.y, b.y, a1);
-    a0 = fmaf(a.z, b.z, a0); a1 = fmaf(a.w, b.w, a1);
-  }
-  float t = a0 + a1;
+__device__ __forceinline__ float warp_sum(float x) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
 }
 
-// y[row0 + r] = scale * dot(A[r,:], x) for my rows; A rows live in shared memory.  POWER: the pass of a power
-// iteration, where the scale is 1 / ||x||: the squared norm is summed from the values of x the pass loads anyway
-// and reduced in the same shuffle rounds as the row sums, so normalising adds no latency of its own.
-// Each result is sent into `dst` (a shared-memory vector) of every CTA of the layer.  A warp owns groups of four
-// consecutive rows (groups warp, warp + CW, ...: NG of them) and works on all of them at once; lane p < n sends
-// each group's four results to peer p as one 16-byte message.  The code is specialised on NG and loops over the
-// columns at run time: the passes of small layers are bound by instruction issue and latency, so no instruction is
-// spent on rows or columns a layer does not have.
-template <bool SELF, int NG, bool POWER = false>
-__device__ __forceinline__ void gemv_send_rows(const float* A, int lda, const float* x, const Slab& s, float scale,
-                                               float* dst, uint32_t bar) {
-  constexpr int NQ = 4 * NG;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (NG == 0) return;
-  const int M4 = s.Mp >> 2;
-  const int ld4 = lda >> 2;
+// Sums of four values over the warp in 6 shuffles instead of 20: halves of the warp keep two of the values, quarters
+// one, and the four totals are handed to every lane.
+__device__ __forceinline__ float4 warp_sum4(float y0, float y1, float y2, float y3) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
+  float u0 = hi ? y2 : y0, u1 = hi ? y3 : y1;
+  u0 += __shfl_xor_sync(0xffffffffu, hi ? y0 : y2, 16);
+  u1 += __shfl_xor_sync(0xffffffffu, hi ? y1 : y3, 16);
+  float z = mid ? u1 : u0;
+  z += __shfl_xor_sync(0xffffffffu, mid ? u0 : u1, 8);
+  z += __shfl_xor_sync(0xffffffffu, z, 4);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
+  return make_float4(__shfl_sync(0xffffffffu, z, 0), __shfl_sync(0xffffffffu, z, 8), __shfl_sync(0xffffffffu, z, 16),
+                     __shfl_sync(0xffffffffu, z, 24));
+}
+
+// barriers among the warps that own rows
+__device__ __forceinline__ void rows_sync(const Link& l) { asm volatile("bar.sync 1, %0;" ::"r"(l.active) : "memory"); }
+
+// Arms the barrier of exchange e (one thread) ahead of the pass, off the chain.
+__device__ __forceinline__ void arm(const Link& l, uint32_t e, uint32_t bytes) {
+  if (l.n > 1 && threadIdx.x == 0) sm100::mbar_expect_tx(l.bar0 + ((e & 1) << 3), bytes);
+}
+// Bounded wait for exchange e.  Every warp waits for itself.  Once a wait has given up no later wait of the CTA
+// blocks: the CTA runs on with stale data to the end of the call, so that its block barriers and its peers stay in
+// step, and reports the time-out there.  A layer on one CTA exchanges through its own shared memory.
+__device__ __forceinline__ void wait_exchange(const Link& l, uint32_t e, int* fail) {
+  if (l.n == 1) { rows_sync(l); return; }
+  const uint32_t bar = l.bar0 + ((e & 1) << 3), parity = (e >> 1) & 1;
+  if (sm100::mbar_try_wait(bar, parity)) return;
+  if (*(volatile int*)fail) return;
+  for (uint32_t i = 0; i < sm100::kSpinLimit; ++i)
+    if (sm100::mbar_try_wait(bar, parity)) return;
+  *(volatile int*)fail = 1;
+}
+// four results of a group into `tgt` of every CTA of the layer
+__device__ __forceinline__ void send4(const Link& l, float* tgt, float4 v, uint32_t e) {
+  const int lane = threadIdx.x & 31;
+  if (l.n == 1) {
+    if (lane == 0) *reinterpret_cast<float4*>(tgt) = v;
+  } else if (lane < l.n) {
+    st_async_v4(smem_u32(tgt) + l.rdelta, v, l.bar0 + ((e & 1) << 3) + l.rdelta);
+  }
+}
+
+// One pass: y = scale * (my rows) x, sent to `dst` (the slot of the warp's first
+// group in the result vector) of every CTA of the layer.  NORM: scale = 1 / ||x||, summed from
+// the values of x the pass loads anyway; returns ||x||^2.  SELF: squared norms of the rows themselves.
+enum { PASS_SELF, PASS_SCALE, PASS_NORM };
+template <int MODE, int NG, int IT>
+__device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float* x, float scale, const Link& l,
+                                      float* dst, uint32_t e) {
+  const int lane = threadIdx.x & 31;
   const float4* x4 = reinterpret_cast<const float4*>(x);
-  const float4* A4 = reinterpret_cast<const float4*>(A) + (size_t)(4 * warp) * ld4;
-  float acc[NQ > 0 ? NQ : 1][2];
+  float acc[4 * NG][2];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) acc[q][0] = acc[q][1] = 0.f;
+  for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
   float n0 = 0.f, n1 = 0.f;
-#pragma unroll 2
-  for (int c = lane; c < M4; c += 32) {
-    float4 a[NQ > 0 ? NQ : 1];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) a[q] = A4[((q >> 2) * 4 * CW + (q & 3)) * ld4 + c];
+  for (int k = 0; k < IT; ++k) {
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!SELF) b = x4[c];
-    if (POWER) {
+    if (MODE != PASS_SELF) b = x4[lane + 32 * k];
+    if (MODE == PASS_NORM) {
       n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
       n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
     }
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      const float4 bb = SELF ? a[q] : b;
-      acc[q][0] = fmaf(a[q].x, bb.x, acc[q][0]); acc[q][1] = fmaf(a[q].y, bb.y, acc[q][1]);
-      acc[q][0] = fmaf(a[q].z, bb.z, acc[q][0]); acc[q][1] = fmaf(a[q].w, bb.w, acc[q][1]);
+    for (int q = 0; q < 4 * NG; ++q) {
+      const float4 v = a[q][k];
+      const float4 bb = MODE == PASS_SELF ? v : b;
+      acc[q][0] = fmaf(v.x, bb.x, acc[q][0]); acc[q][1] = fmaf(v.y, bb.y, acc[q][1]);
+      acc[q][0] = fmaf(v.z, bb.z, acc[q][0]); acc[q][1] = fmaf(v.w, bb.w, acc[q][1]);
     }
   }
-  float y[NQ > 0 ? NQ : 1];
+  float n2 = 0.f;
+  if (MODE == PASS_NORM) { n2 = warp_sum(n0 + n1); scale = inv_norm(n2); }
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) y[q] = acc[q][0] + acc[q][1];
-  float nin = n0 + n1;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
-    if (POWER) nin += __shfl_xor_sync(0xffffffffu, nin, o);
+  for (int g = 0; g < NG; ++g) {
+    float4 v = warp_sum4(acc[4 * g][0] + acc[4 * g][1], acc[4 * g + 1][0] + acc[4 * g + 1][1],
+                         acc[4 * g + 2][0] + acc[4 * g + 2][1], acc[4 * g + 3][0] + acc[4 * g + 3][1]);
+    v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale;
+    send4(l, dst + 4 * CW * g, v, e);
   }
-  if (POWER) scale = inv_norm(nin);
-  if (lane < s.n) {
-#pragma unroll
-    for (int k = 0; k < NG; ++k) {
-      const float4 v = make_float4(y[4 * k] * scale, y[4 * k + 1] * scale, y[4 * k + 2] * scale, y[4 * k + 3] * scale);
-      float* tgt = dst + s.row0 + 4 * (warp + CW * k);
-      if (lane == s.sub) *reinterpret_cast<float4*>(tgt) = v;
-      else st_async_v4(smem_u32(tgt) + s.rdelta, v, bar + s.rdelta);
+  return n2;
+}
+
+// m' = argmax xi, lowest index on ties (Eq. 46).  Every warp finds it for itself: squared norms are not negative, so
+// their bit patterns are ordered; a NaN never wins.
+__device__ __forceinline__ int argmax_xi(const Slab& s) {
+  const int lane = threadIdx.x & 31;
+  uint32_t best = 0, bi = 0;
+  for (int c = lane; c < (s.Mp >> 2); c += 32) {
+    const float4 x = reinterpret_cast<const float4*>(s.xi2)[c];
+#define FW_CAND(X, o)                                                                                     \
+    {                                                                                                     \
+      const uint32_t k = (X) >= 0.f && 4 * c + (o) < s.M ? __float_as_uint(X) + 1u : 0u;                   \
+      if (k > best) { best = k; bi = 4 * c + (o); }                                                       \
     }
+    FW_CAND(x.x, 0) FW_CAND(x.y, 1) FW_CAND(x.z, 2) FW_CAND(x.w, 3)
+#undef FW_CAND
+  }
+  const uint32_t top = __reduce_max_sync(0xffffffffu, best);
+  bi = __reduce_min_sync(0xffffffffu, best == top ? bi : 0xffffffffu);
+  return top == 0 || bi >= (uint32_t)s.M ? 0 : (int)bi;
+}
+
+// Row m' of Phi_y into wvec of every CTA of the layer: the CTA that owns it sends it (exchange e).  A CTA that holds all
+// rows reads the row where it is.
+__device__ __forceinline__ const float* row_exchange(Slab& s, const Link& l, int mp, uint32_t e) {
+  const int owner = mp / s.R;
+  const float* row = s.phi + (size_t)(mp - owner * s.R) * s.Mp;
+  if (l.n == 1) return row;
+  arm(l, e, (uint32_t)s.Mp * 4u);
+  if (owner == s.sub) {
+    const uint32_t bar = l.bar0 + ((e & 1) << 3);
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < (s.Mp >> 2); c += l.active >> 5) {
+      // a lane per peer: the lanes' copies of one float4 go out together
+      const float4 v = reinterpret_cast<const float4*>(row)[c];
+      if (lane < l.n) st_async_v4(smem_u32(s.wvec + 4 * c) + l.rdelta, v, bar + l.rdelta);
+    }
+  }
+  wait_exchange(l, e, &s.fail);
+  return s.wvec;
+}
+
+// Weights of the coherent set into wvec (Eqs. 48-49); returns the size of the set
+__device__ __forceinline__ int align_weights(Slab& s, const Link& l, int mp) {
+  if (s.maxcol) {
+    rows_sync(l);                     // wvec may still be read by a slower warp
+    for (int m = threadIdx.x; m < s.Mp; m += l.active) s.wvec[m] = (m == mp) ? 1.f : 0.f;
+    rows_sync(l);
+    return 1;
+  }
+  const float xi_mp = sqrtf(s.xi2[mp]), c_rel = s.c_rel, c_abs = s.c_abs;
+  int cnt = 0;
+  for (int base = 0; base < s.Mp; base += l.active) {
+    const int m = base + (int)threadIdx.x;
+    int in = 0;
+    if (m < s.Mp) {
+      float wv = 0.f;
+      if (m < s.M) {
+        const float c = s.cvec[m];
+        const float thr = fmaxf(c_rel * xi_mp * sqrtf(s.xi2[m]), c_abs);
+        in = fabsf(c) >= thr;       // false for NaN
+        wv = in ? (1.f / c) : 0.f;
+      }
+      s.wvec[m] = wv;
+    }
+    int n;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %1, 0;\n\tbarrier.cta.red.popc.aligned.u32 %0, 1, %2, p;\n\t}"
+                 : "=r"(n) : "r"(in), "r"(l.active) : "memory");
+    cnt += n;
+  }
+  return cnt;
+}
+
+// rows of a row-major matrix in global memory <-> the registers of the warp that owns them; V4: rows of whole float4s
+template <int NG, int IT, bool V4>
+__device__ __forceinline__ void load_rows(float4 (&a)[4 * NG][IT], const float* G, const Slab& s) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int M = s.M;
+#pragma unroll
+  for (int q = 0; q < 4 * NG; ++q) {
+    const int i = s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3);
+    const float* row = G + (size_t)i * M;
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int c = lane + 32 * k;
+      a[q][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i >= M) continue;
+      if (V4) {
+        if (4 * c < M) a[q][k] = reinterpret_cast<const float4*>(row)[c];
+      } else {
+        if (4 * c < M) a[q][k].x = row[4 * c];
+        if (4 * c + 1 < M) a[q][k].y = row[4 * c + 1];
+        if (4 * c + 2 < M) a[q][k].z = row[4 * c + 2];
+        if (4 * c + 3 < M) a[q][k].w = row[4 * c + 3];
+      }
+    }
+  }
+}
+template <int NG, int IT, bool V4>
+__device__ __forceinline__ void store_rows(const float4 (&a)[4 * NG][IT], float* G, const Slab& s) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int M = s.M;
+#pragma unroll
+  for (int q = 0; q < 4 * NG; ++q) {
+    const int i = s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3);
+    if (i >= M) continue;
+    float* row = G + (size_t)i * M;
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int c = lane + 32 * k;
+      if (V4) {
+        if (4 * c < M) reinterpret_cast<float4*>(row)[c] = a[q][k];
+      } else {
+        if (4 * c < M) row[4 * c] = a[q][k].x;
+        if (4 * c + 1 < M) row[4 * c + 1] = a[q][k].y;
+        if (4 * c + 2 < M) row[4 * c + 2] = a[q][k].z;
+        if (4 * c + 3 < M) row[4 * c + 3] = a[q][k].w;
+      }
+    }
+  }
+}
+
+// The recorded steps in T and Q, one exchange in all.  T first (t of step k comes from T after step k - 1), then Q, with
+// the operations on every element in step order; smooth: Qs <- beta Qs + (1 - beta) Q (Eq. 35).
+template <int NG, int IT, bool V4>
+__device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* L, int steps, bool smooth, uint32_t e) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float4 a[4 * NG][IT];
+  float* th = s.th + s.row0 + 4 * warp;
+  int live = 0;
+#pragma unroll 1
+  for (int k = 0; k < steps; ++k) live += s.ah[k] != 0.f ? 1 : 0;
+  if (live) {
+    load_rows<NG, IT, V4>(a, L->Tt, s);
+    arm(l, e, (uint32_t)live * s.tx);
+#pragma unroll 1
+    for (int k = 0; k < steps; ++k) {
+      const float ak = s.ah[k];
+      if (ak == 0.f) continue;
+      const float4* v4 = reinterpret_cast<const float4*>(s.vh + k * s.Mv);
+      float acc[4 * NG][2];
+#pragma unroll
+      for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const float4 b = v4[lane + 32 * it];
+#pragma unroll
+        for (int q = 0; q < 4 * NG; ++q) {
+          acc[q][0] = fmaf(a[q][it].x, b.x, acc[q][0]); acc[q][1] = fmaf(a[q][it].y, b.y, acc[q][1]);
+          acc[q][0] = fmaf(a[q][it].z, b.z, acc[q][0]); acc[q][1] = fmaf(a[q][it].w, b.w, acc[q][1]);
+        }
+      }
+      float at[4 * NG];
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        const float4 t = warp_sum4(acc[4 * g][0] + acc[4 * g][1], acc[4 * g + 1][0] + acc[4 * g + 1][1],
+                                   acc[4 * g + 2][0] + acc[4 * g + 2][1], acc[4 * g + 3][0] + acc[4 * g + 3][1]);
+        send4(l, th + k * s.Mv + 4 * CW * g, t, e);
+        at[4 * g] = ak * t.x; at[4 * g + 1] = ak * t.y; at[4 * g + 2] = ak * t.z; at[4 * g + 3] = ak * t.w;
+      }
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const float4 b = v4[lane + 32 * it];
+#pragma unroll
+        for (int q = 0; q < 4 * NG; ++q) {
+          a[q][it].x = fmaf(at[q], b.x, a[q][it].x); a[q][it].y = fmaf(at[q], b.y, a[q][it].y);
+          a[q][it].z = fmaf(at[q], b.z, a[q][it].z); a[q][it].w = fmaf(at[q], b.w, a[q][it].w);
+        }
+      }
+    }
+    store_rows<NG, IT, V4>(a, L->Tt, s);
+  } else {
+    arm(l, e, 0u);
+  }
+  load_rows<NG, IT, V4>(a, L->Q, s);
+  wait_exchange(l, e, &s.fail);
+  if (live) {
+#pragma unroll 1
+    for (int k = 0; k < steps; ++k) {
+      const float ak = s.ah[k];
+      if (ak == 0.f) continue;
+      const float aq = ak * (ak + 2.f);
+      const float* tk = s.th + k * s.Mv;
+      float ti[4 * NG];
+#pragma unroll
+      for (int q = 0; q < 4 * NG; ++q) ti[q] = tk[s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3)];
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const float4 b = reinterpret_cast<const float4*>(tk)[lane + 32 * it];
+#pragma unroll
+        for (int q = 0; q < 4 * NG; ++q) {
+          a[q][it].x = __fadd_rn(a[q][it].x, __fmul_rn(aq, __fmul_rn(ti[q], b.x)));
+          a[q][it].y = __fadd_rn(a[q][it].y, __fmul_rn(aq, __fmul_rn(ti[q], b.y)));
+          a[q][it].z = __fadd_rn(a[q][it].z, __fmul_rn(aq, __fmul_rn(ti[q], b.z)));
+          a[q][it].w = __fadd_rn(a[q][it].w, __fmul_rn(aq, __fmul_rn(ti[q], b.w)));
+        }
+      }
+    }
+    if (!*(volatile int*)&s.fail) store_rows<NG, IT, V4>(a, L->Q, s);
+  }
+  if (smooth) {
+    const float beta = L->beta, ob = 1.f - beta;
+    const int M = s.M;
+    float* Qs = L->Qs;
+#pragma unroll
+    for (int q = 0; q < 4 * NG; ++q) {
+      const int i = s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3);
+      if (i >= M) continue;
+      float* row = Qs + (size_t)i * M;
+      if (V4) {
+#pragma unroll
+        for (int it = 0; it < IT; ++it) {
+          const int c = lane + 32 * it;
+          if (4 * c >= M) continue;
+          float4 o = reinterpret_cast<float4*>(row)[c];
+          o.x = fmaf(beta, o.x, ob * a[q][it].x); o.y = fmaf(beta, o.y, ob * a[q][it].y);
+          o.z = fmaf(beta, o.z, ob * a[q][it].z); o.w = fmaf(beta, o.w, ob * a[q][it].w);
+          reinterpret_cast<float4*>(row)[c] = o;
+        }
+      } else {
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const int c = 4 * (lane + 32 * it);
+        if (c < M) row[c] = fmaf(beta, row[c], ob * a[q][it].x);
+        if (c + 1 < M) row[c + 1] = fmaf(beta, row[c + 1], ob * a[q][it].y);
+        if (c + 2 < M) row[c + 2] = fmaf(beta, row[c + 2], ob * a[q][it].z);
+        if (c + 3 < M) row[c + 3] = fmaf(beta, row[c + 3], ob * a[q][it].w);
+      }
+      }
+    }
+  }
+}
+
+// Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane.
+template <int NG, int IT>
+__device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L, float* tr, int k0, int k1, int P,
+                                       bool last, uint32_t e) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slot = s.row0 + 4 * warp;       // the warp's first group in a result vector
+  const uint32_t tx = s.tx;
+  float4 a[4 * NG][IT];
+#pragma unroll
+  for (int q = 0; q < 4 * NG; ++q) {
+    const float4* r4 = reinterpret_cast<const float4*>(s.phi + (size_t)(4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp);
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int c = lane + 32 * k;
+      a[q][k] = c < (s.Mp >> 2) ? r4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  for (int step = k0; step < k1; ++step) {
+    // S1: squared column norms (= row norms, Phi_y is exactly symmetric)             (Eq. 45)
+    arm(l, e, tx);
+    pass<PASS_SELF, NG, IT>(a, nullptr, 1.f, l, s.xi2 + slot, e);
+    wait_exchange(l, e, &s.fail); ++e;
+    // S2: m' = argmax xi, x = row m' of Phi_y, c = Phi_y x                            (Eqs. 46-47)
+    const int mp = argmax_xi(s);
+    const float* row = row_exchange(s, l, mp, e); ++e;
+    arm(l, e, tx);
+    pass<PASS_SCALE, NG, IT>(a, row, 1.f, l, s.cvec + slot, e);
+    wait_exchange(l, e, &s.fail); ++e;
+    // S3: coherent set and aligned average                                          (Eqs. 48-49)
+    arm(l, e, tx);
+    const int cnt = align_weights(s, l, mp);
+    pass<PASS_SCALE, NG, IT>(a, s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, l, s.buf0 + slot, e);
+    wait_exchange(l, e, &s.fail); ++e;
+    // S4: P power iterations u = Phi_y (prev / ||prev||)
+    float* x = s.buf0;
+    float* y = x + s.Mv;
+    for (int p = 0; p < P; ++p) {
+      arm(l, e, tx);
+      pass<PASS_NORM, NG, IT>(a, x, 0.f, l, y + slot, e);
+      wait_exchange(l, e, &s.fail); ++e;
+      float* t = x; x = y; y = t;
+    }
+    // S5: v = prev/||prev|| (Eq. 50), u = Phi_y v, lambda_e = v.u (Eq. 36)
+    arm(l, e, tx);
+    const float n2 = pass<PASS_NORM, NG, IT>(a, x, 0.f, l, s.uvec + slot, e);
+    const float inv = inv_norm(n2);
+    float* vh = s.vh + (step - k0) * s.Mv;
+    wait_exchange(l, e, &s.fail); ++e;
+    float l0 = 0.f, l1 = 0.f;
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    const float4* u4 = reinterpret_cast<const float4*>(s.uvec);
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const float4 xv = x4[lane + 32 * k], uv = u4[lane + 32 * k];
+      const float4 vv = make_float4(xv.x * inv, xv.y * inv, xv.z * inv, xv.w * inv);
+      l0 = fmaf(vv.x, uv.x, l0); l1 = fmaf(vv.y, uv.y, l1);
+      l0 = fmaf(vv.z, uv.z, l0); l1 = fmaf(vv.w, uv.w, l1);
+      if (warp == 0) reinterpret_cast<float4*>(vh)[lane + 32 * k] = vv;      // every CTA records the whole vector
+    }
+    const float lam_e = warp_sum(l0 + l1);
+    // S6: g_e, a_e (Eqs. 40-41), rank update of Phi_y.  All warps of all CTAs sum in the same order, so they hold the
+    // same bits.
+    const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
+    float g_e = 1.f, aa = 0.f;
+    if (ok) {
+      g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);
+      aa = sqrtf(g_e) - 1.f;
+    }
+    // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T = v w^T + w v^T with w = a u + (a^2 lambda_e / 2) v: four operations
+    // an element, symmetric in (i, j)
+    if (aa != 0.f) {
+      const float hl = 0.5f * aa * aa * lam_e;
+      float vi[4 * NG], wi[4 * NG];
+#pragma unroll
+      for (int q = 0; q < 4 * NG; ++q) {
+        const int i = slot + 4 * CW * (q >> 2) + (q & 3);
+        vi[q] = x[i] * inv;
+        wi[q] = __fadd_rn(__fmul_rn(aa, s.uvec[i]), __fmul_rn(hl, vi[q]));
+      }
+#pragma unroll
+      for (int k = 0; k < IT; ++k) {
+        const int c = lane + 32 * k;
+        float4 vj = x4[c], wj = u4[c];
+        vj.x *= inv; vj.y *= inv; vj.z *= inv; vj.w *= inv;
+        wj.x = __fadd_rn(__fmul_rn(aa, wj.x), __fmul_rn(hl, vj.x)); wj.y = __fadd_rn(__fmul_rn(aa, wj.y), __fmul_rn(hl, vj.y));
+        wj.z = __fadd_rn(__fmul_rn(aa, wj.z), __fmul_rn(hl, vj.z)); wj.w = __fadd_rn(__fmul_rn(aa, wj.w), __fmul_rn(hl, vj.w));
+#pragma unroll
+        for (int q = 0; q < 4 * NG; ++q) {
+          a[q][k].x = __fadd_rn(a[q][k].x, __fadd_rn(__fmul_rn(vi[q], wj.x), __fmul_rn(wi[q], vj.x)));
+          a[q][k].y = __fadd_rn(a[q][k].y, __fadd_rn(__fmul_rn(vi[q], wj.y), __fmul_rn(wi[q], vj.y)));
+          a[q][k].z = __fadd_rn(a[q][k].z, __fadd_rn(__fmul_rn(vi[q], wj.z), __fmul_rn(wi[q], vj.z)));
+          a[q][k].w = __fadd_rn(a[q][k].w, __fadd_rn(__fmul_rn(vi[q], wj.w), __fmul_rn(wi[q], vj.w)));
+          if (c < (s.Mp >> 2))
+            reinterpret_cast<float4*>(s.phi + (size_t)(4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp)[c] = a[q][k];
+        }
+      }
+    }
+    if (threadIdx.x == 0) {
+      s.ah[step - k0] = aa;
+      if (s.sub == 0) {
+        if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
+        if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
+        if (tr) {
+          tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
+        }
+        if (last && step + 1 == k1) {
+          L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
+          L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
+        }
+      }
+    }
+    rows_sync(l);       // the slab is complete (any warp may send its row m' next), ah and vh for apply_steps
   }
 }
 
@@ -199,101 +554,32 @@ __device__ __forceinline__ int warp_groups(int R) {
   return ng > warp ? (ng - warp + CW - 1) / CW : 0;
 }
 
-template <bool SELF>
-__device__ __noinline__ void slab_gemv_send(const float* A, int lda, const float* x, const Slab s, float scale,
-                                            float* dst, uint32_t bar) {
-  static_assert(MAXGPW == 2, "specialisations below");
-  switch (warp_groups(s.R)) {
-    case 1: gemv_send_rows<SELF, 1>(A, lda, x, s, scale, dst, bar); break;
-    case 2: gemv_send_rows<SELF, 2>(A, lda, x, s, scale, dst, bar); break;
-    default: break;
-  }
-}
-
-// The P power iterations of a step (S4) as one specialised loop: the pass, its exchange and the next pass
-// follow each other without a call or a dispatch in between, and everything that does not change from pass to
-// pass stays in registers.  Returns false when a wait gave up.
-template <int NG>
-__device__ __forceinline__ bool power_loop_rows(const Slab& s, float* buf0, int Mv, uint32_t bar0, uint32_t& e, int P,
-                                                int& cur, uint32_t tx_bytes) {
-  for (int p = 0; p < P; ++p) {
-    const uint32_t bar = bar0 + ((e & 1) << 3);
-    if (threadIdx.x == 0) sm100::mbar_expect_tx(bar, tx_bytes);     // armed ahead of the pass, off the chain
-    gemv_send_rows<false, NG, true>(s.phi, s.Mp, buf0 + cur * Mv, s, 0.f, buf0 + (cur ^ 1) * Mv, bar);
-    if (!exchange_wait(bar, (e >> 1) & 1)) return false;
-    ++e;
-    cur ^= 1;
-  }
-  return true;
-}
-
-__device__ __noinline__ bool power_loop(const Slab s, float* buf0, int Mv, uint32_t bar0, uint32_t& e, int P,
-                                        int& cur, uint32_t tx_bytes) {
-  switch (warp_groups(s.R)) {
-    case 0: return power_loop_rows<0>(s, buf0, Mv, bar0, e, P, cur, tx_bytes);
-    case 1: return power_loop_rows<1>(s, buf0, Mv, bar0, e, P, cur, tx_bytes);
-    case 2: return power_loop_rows<2>(s, buf0, Mv, bar0, e, P, cur, tx_bytes);
-    default: return true;
-  }
-}
-
-// Q <- Q + aq t t^T on my rows for the pending steps (Eq. 44), in step order, each with the roundings of a step
-// applied alone.  A thread has all its loads of a round in flight before it uses the first.
-__device__ __noinline__ void flush_q(float* Q, const Slab s, const float* tk, int Mv, const float* aq, int pending) {
-  const int M = s.M;
-  if ((M & 3) == 0) {
-    constexpr int U = 6;
-    const int M4 = M >> 2, total = s.nrows * M4;
-    float4* Q4 = reinterpret_cast<float4*>(Q + (size_t)s.row0 * M);
-    for (int base = threadIdx.x; base < total; base += CT * U) {
-      float4 q[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (base + u * CT < total) q[u] = Q4[base + u * CT];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = base + u * CT;
-        if (i < total) {
-          const int r = i / M4, c = i - r * M4;
-          for (int k = 0; k < pending; ++k) {
-            const float ti = tk[k * Mv + s.row0 + r], ak = aq[k];
-            const float4 tj = reinterpret_cast<const float4*>(tk + k * Mv)[c];
-            q[u].x = __fadd_rn(q[u].x, __fmul_rn(ak, __fmul_rn(ti, tj.x)));
-            q[u].y = __fadd_rn(q[u].y, __fmul_rn(ak, __fmul_rn(ti, tj.y)));
-            q[u].z = __fadd_rn(q[u].z, __fmul_rn(ak, __fmul_rn(ti, tj.z)));
-            q[u].w = __fadd_rn(q[u].w, __fmul_rn(ak, __fmul_rn(ti, tj.w)));
-          }
-          Q4[i] = q[u];
-        }
-      }
-    }
-  } else {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int r = warp; r < s.nrows; r += CW) {
-      const int i = s.row0 + r;
-      float* Qr = Q + (size_t)i * M;
-      for (int c = lane; c < M; c += 32) {
-        float q = Qr[c];
-        for (int k = 0; k < pending; ++k)
-          q = __fadd_rn(q, __fmul_rn(aq[k], __fmul_rn(tk[k * Mv + i], tk[k * Mv + c])));
-        Qr[c] = q;
-      }
-    }
-  }
-}
-
-// dynamic shared memory (Mv = n R >= Mp: the length of a vector that n slices of R results fill):
-// [phi slab R x Mp][tt slab R x Mp][xi2][cvec][wvec][bufA][bufB][vvec][uvec][tvec][tk: KQ x Mv]
+// dynamic shared memory: [phi slab R x Mp][xi2][cvec][wvec][two power-iteration vectors][uvec][vh: KH][th: KH], vectors
+// of Mv floats: what n slices of R results fill, and at least whole trips of a warp over the columns
 extern __shared__ __align__(16) float csm[];
 
 __host__ __device__ inline int slab_rows(int M, int n) { return (((M + n - 1) / n) + 3) & ~3; }
+__host__ __device__ inline int slab_trips(int M) { return (((M + 3) >> 2) + 31) / 32; }
+__host__ __device__ inline int slab_vec(int M, int n) {
+  const int a = n * slab_rows(M, n), b = 128 * slab_trips(M);
+  return a > b ? a : b;
+}
+constexpr int kVecs = 6 + 2 * KH;
 
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(CT, 1)
-recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
+template <int NG, int IT>
+__device__ __forceinline__ void run_chunk(Slab& s, const Link& l, const LayerDev* L, float* tr, int k0, int k1, int P,
+                                          bool last, bool smooth, uint32_t e) {
+  run_steps<NG, IT>(s, l, L, tr, k0, k1, P, last, e);
+  e += (uint32_t)(k1 - k0) * (uint32_t)(P + 5);
+  if ((s.M & 3) == 0) apply_steps<NG, IT, true>(s, l, L, k1 - k0, smooth, e);
+  else apply_steps<NG, IT, false>(s, l, L, k1 - k0, smooth, e);
+}
+
+__global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // my layer: the one whose CTA range holds this CTA (none: a filler CTA of the last cluster)
+  const int lane = threadIdx.x & 31;
+  // my layer: the one whose CTA range holds this CTA (none: a filler CTA of a cluster)
   int layer = -1;
 #pragma unroll 1
   for (int l = 0; l < a.g.n; ++l)
@@ -304,273 +590,100 @@ recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
     return;
   }
   const LayerDev* L = a.g.layer[layer];
-  const int K = a.K, P = a.P;
-  const int n = a.ncta[layer];
-  const int sub = (int)blockIdx.x - a.first_cta[layer];
-  const int rank0 = rank - sub;                 // cluster rank of the layer's first CTA
-  const int M = L->M;
-  const int Mp = (M + 3) & ~3;
-  const int R = slab_rows(M, n);
-  const int Mv = n * R;
-  Slab s;
-  s.M = M; s.Mp = Mp; s.R = R; s.n = n; s.sub = sub;
-  s.row0 = sub * R;
-  s.nrows = max(0, min(R, M - s.row0));
-  s.phi = csm;
-  s.tt = csm + (size_t)R * Mp;
-  float* xi2 = csm + 2 * (size_t)R * Mp;
-  float* cvec = xi2 + Mv;
-  float* wvec = cvec + Mv;
-  float* buf0 = wvec + Mv;           // two alternating power-iteration vectors, Mv apart
-  float* vvec = wvec + 3 * Mv;
-  float* uvec = vvec + Mv;
-  float* tvec = uvec + Mv;
-  float* tk = tvec + Mv;             // the vectors t of the steps whose Q terms are pending
   __shared__ __align__(8) uint64_t xbar[2];
-  __shared__ float sredf[CW];
-  __shared__ int sredi[CW + 1];
-  __shared__ float s_aq[KQ];
-
-  // ---- load my rows of Phi_y and T^T (padded with zeros to R rows of Mp); clear the vectors ----
-  for (int which = 0; which < 2; ++which) {
-    const float* G = which ? L->Tt : L->Phiy;
-    float* S = which ? s.tt : s.phi;
-    if ((M & 3) == 0) {
-      // 16-byte asynchronous copies, every one of a thread in flight at once: the load costs one trip to
-      // memory, not one per row
-      const int M4 = M >> 2;
-      for (int i = threadIdx.x; i < R * M4; i += CT) {
-        const int r = i / M4, c = i - r * M4;
-        float* d = S + (size_t)r * Mp + 4 * c;
-        if (r < s.nrows) cp_async16(smem_u32(d), G + (size_t)(s.row0 + r) * M + 4 * c);
-        else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    } else {
-      for (int i = threadIdx.x; i < R * Mp; i += CT) {
-        const int r = i / Mp, c = i - r * Mp;
-        S[i] = (c < M && r < s.nrows) ? G[(size_t)(s.row0 + r) * M + c] : 0.f;
-      }
-    }
-  }
-  for (int i = threadIdx.x; i < (8 + KQ) * Mv; i += CT) xi2[i] = 0.f;
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __shared__ Slab s;
+  Link l;
+  l.n = a.ncta[layer];
+  l.active = 0;
+  l.bar0 = smem_u32(&xbar[0]);                       // the two barriers are 8 bytes apart
   if (threadIdx.x == 0) {
-    sm100::mbar_init(smem_u32(&xbar[0]), 1);
-    sm100::mbar_init(smem_u32(&xbar[1]), 1);
+    const int M = L->M, n = l.n;
+    s.M = M; s.Mp = (M + 3) & ~3; s.R = slab_rows(M, n); s.n = n;
+    s.Mv = slab_vec(M, n);
+    s.sub = (int)blockIdx.x - a.first_cta[layer];
+    s.row0 = s.sub * s.R;
+    s.nrows = max(0, min(s.R, M - s.row0));
+    s.phi = csm;
+    s.xi2 = csm + (size_t)s.R * s.Mp;
+    s.cvec = s.xi2 + s.Mv; s.wvec = s.cvec + s.Mv; s.buf0 = s.wvec + s.Mv; s.uvec = s.buf0 + 2 * s.Mv;
+    s.vh = s.uvec + s.Mv; s.th = s.vh + KH * s.Mv;
+    s.tx = (uint32_t)n * (uint32_t)s.R * 4u;
+    s.maxcol = L->init == FW_INIT_MAXCOL;
+    s.c_rel = L->c_rel; s.c_abs = L->c_abs; s.delta = L->delta; s.eps = L->eps;
+    s.lam_bar = L->scal[SC_LAMBDA_BAR];
+    s.fail = 0;
+    sm100::mbar_init(l.bar0, 1);
+    sm100::mbar_init(l.bar0 + 8, 1);
     sm100::mbar_fence_init();
   }
-  const uint32_t bar0 = smem_u32(&xbar[0]);                       // the two barriers are 8 bytes apart
-  // A peer's window of the cluster address space is this CTA's window shifted by a constant; the stores
-  // below rely on it, so it is checked on two addresses far apart before anything is sent.
-  const uint32_t peer_rank = (uint32_t)(rank0 + min(lane, n - 1));
-  s.rdelta = map_cluster(bar0, peer_rank) - bar0;
-  const bool linear = (map_cluster(smem_u32(tk), peer_rank) - smem_u32(tk)) == s.rdelta;
-  bool failed = __syncthreads_or(!linear) != 0;
+  __syncthreads();
+  const int M = s.M, R = s.R, nrows = s.nrows;
+  l.active = 32 * min(CW, R >> 2);
+
+  // ---- load my rows of Phi_y (padded with zeros to R rows of Mp); clear the vectors ----
+  if ((M & 3) == 0) {
+    // 16-byte asynchronous copies, every one of a thread in flight at once: one trip to memory
+    const int M4 = M >> 2;
+    for (int i = threadIdx.x; i < R * M4; i += CT) {
+      const int r = i / M4, c = i - r * M4;
+      float* d = csm + (size_t)r * M + 4 * c;
+      if (r < nrows) cp_async16(smem_u32(d), L->Phiy + (size_t)(s.row0 + r) * M + 4 * c);
+      else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  } else {
+    for (int i = threadIdx.x; i < R * s.Mp; i += CT) {
+      const int r = i / s.Mp, c = i - r * s.Mp;
+      csm[i] = (c < M && r < nrows) ? L->Phiy[(size_t)(s.row0 + r) * M + c] : 0.f;
+    }
+  }
+  for (int i = threadIdx.x; i < kVecs * s.Mv; i += CT) s.xi2[i] = 0.f;
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  // A CTA's window of the cluster address space is this CTA's window shifted by a constant; the stores rely on it,
+  // so it is checked on two addresses far apart before anything is sent.
+  const uint32_t peer_rank = (uint32_t)(rank - s.sub + min(lane, l.n - 1));
+  l.rdelta = map_cluster(l.bar0, peer_rank) - l.bar0;
+  const bool linear = (map_cluster(smem_u32(s.th), peer_rank) - smem_u32(s.th)) == l.rdelta;
+  const bool usable = __syncthreads_or(!linear) == 0;
   cluster.sync();   // every barrier is initialised before the first remote store can arrive
 
-  const uint32_t vec_bytes = (uint32_t)(n - 1) * (uint32_t)R * 4u;   // one vector's slices from the n - 1 peers
-  uint32_t e = 0;                                                 // exchanges completed so far
-  int pending = 0;                                                // steps whose Q terms wait in tk
-  // arm the barrier of the current exchange for `nvec` vectors, wait for it, advance
-#define FW_BAR (bar0 + ((e & 1) << 3))
-#define FW_EXCHANGE(nvec)                                                    \
-  {                                                                          \
-    if (threadIdx.x == 0) sm100::mbar_expect_tx(FW_BAR, (nvec) * vec_bytes); \
-    if (!exchange_wait(FW_BAR, (e >> 1) & 1)) { failed = true; goto done; }  \
-    ++e;                                                                     \
-  }
-#define FW_FLUSH_Q()                                   \
-  {                                                    \
-    if (pending > 0) {                                 \
-      flush_q(L->Q, s, tk, Mv, s_aq, pending);         \
-      __syncthreads();                                 \
-      pending = 0;                                     \
-    }                                                  \
-  }
-  if (failed) goto done;
-
-  {
-  float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
-  const float c_rel = L->c_rel, c_abs = L->c_abs, delta = L->delta, eps = L->eps;
-  const float lam_bar = L->scal[SC_LAMBDA_BAR];
-  const bool maxcol = (L->init == FW_INIT_MAXCOL);
-  bool any_nosub = false, any_nonfinite = false;
-
-  for (int step = 0; step < K; ++step) {
-    // S1: squared column norms (= row norms, Phi_y is exactly symmetric)             (Eq. 45)
-    slab_gemv_send<true>(s.phi, Mp, nullptr, s, 1.f, xi2, FW_BAR);
-    FW_EXCHANGE(1u)
-    // S2: m' = argmax xi (lowest index on ties), x = row m' of Phi_y, c = Phi_y x    (Eqs. 46-47)
-    {
-      float best = -1.f;
-      int bi = 0x7fffffff;
-      for (int m = threadIdx.x; m < M; m += CT) {
-        const float x = xi2[m];
-        if (x > best) { best = x; bi = m; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float xo = __shfl_xor_sync(0xffffffffu, best, o);
-        const int io = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (xo > best || (xo == best && io < bi)) { best = xo; bi = io; }
-      }
-      if (lane == 0) { sredf[warp] = best; sredi[warp] = bi; }
-      __syncthreads();
-      if (threadIdx.x < 32) {
-        best = threadIdx.x < CW ? sredf[threadIdx.x] : -1.f;
-        bi = threadIdx.x < CW ? sredi[threadIdx.x] : 0x7fffffff;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float xo = __shfl_xor_sync(0xffffffffu, best, o);
-          const int io = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (xo > best || (xo == best && io < bi)) { best = xo; bi = io; }
+  if (usable) {
+    float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
+    const int it = slab_trips(M), ng = warp_groups(R);
+    uint32_t e = 0;                        // exchanges so far
+    for (int k0 = 0; k0 < a.K; k0 += KH) {
+      const int k1 = min(a.K, k0 + KH);
+      const bool last = k1 == a.K, smooth = last && L->Qs != L->Q;
+      if (ng == 1) {
+        switch (it) {
+          case 1: run_chunk<1, 1>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
+          case 2: run_chunk<1, 2>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
+          case 3: run_chunk<1, 3>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
+          case 4: run_chunk<1, 4>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
+          default: run_chunk<1, 5>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
         }
-        if (threadIdx.x == 0) sredi[CW] = bi;
-      }
-      __syncthreads();
-    }
-    int mp = sredi[CW];
-    if (mp < 0 || mp >= M) mp = 0;
-    {
-      // the owner's slab is current: its updates of the previous step precede its S1 sends, which this
-      // CTA has received
-      const int owner = mp / R;
-      const float* rphi = cluster.map_shared_rank(s.phi, rank0 + owner) + (size_t)(mp - owner * R) * Mp;
-      for (int m = threadIdx.x; m < Mp; m += CT) wvec[m] = rphi[m];
-    }
-    __syncthreads();
-    slab_gemv_send<false>(s.phi, Mp, wvec, s, 1.f, cvec, FW_BAR);
-    FW_EXCHANGE(1u)
-    // S3: coherent set and aligned average                                          (Eqs. 48-49)
-    int cnt = 0;
-    if (maxcol) {
-      for (int m = threadIdx.x; m < Mp; m += CT) wvec[m] = (m == mp) ? 1.f : 0.f;
-      cnt = 1;
-      __syncthreads();
-    } else {
-      const float xi_mp = sqrtf(xi2[mp]);
-      for (int base = 0; base < Mp; base += CT) {
-        const int m = base + threadIdx.x;
-        bool in = false;
-        if (m < Mp) {
-          float wv = 0.f;
-          if (m < M) {
-            const float c = cvec[m];
-            const float thr = fmaxf(c_rel * xi_mp * sqrtf(xi2[m]), c_abs);
-            in = fabsf(c) >= thr;
-            wv = in ? (1.f / c) : 0.f;
-          }
-          wvec[m] = wv;
-        }
-        cnt += __syncthreads_count(in);
-      }
-      if (sub == 0)
-        for (int m = threadIdx.x; m < M; m += CT) L->wvec[m] = wvec[m];
-    }
-    const float inv_cnt = cnt > 0 ? 1.f / (float)cnt : 0.f;
-    slab_gemv_send<false>(s.phi, Mp, wvec, s, inv_cnt, buf0, FW_BAR);
-    FW_EXCHANGE(1u)
-    // S4: P power iterations u = Phi_y (prev / ||prev||)
-    int cur = 0;
-    if (!power_loop(s, buf0, Mv, bar0, e, P, cur, vec_bytes)) { failed = true; goto done; }
-    // S5: v = prev/||prev|| (Eq. 50), u = Phi_y v, t = T^T v; lambda_e = v.u (Eq. 36)
-    const float n2 = warp_dot(buf0 + cur * Mv, buf0 + cur * Mv, Mp);
-    const float inv = inv_norm(n2);
-    for (int m = threadIdx.x; m < Mp; m += CT) vvec[m] = buf0[cur * Mv + m] * inv;
-    __syncthreads();
-    slab_gemv_send<false>(s.phi, Mp, vvec, s, 1.f, uvec, FW_BAR);
-    slab_gemv_send<false>(s.tt, Mp, vvec, s, 1.f, tvec, FW_BAR);
-    FW_EXCHANGE(2u)
-    const float lam_e = warp_dot(vvec, uvec, Mp);
-    // S6: g_e, a_e (Eqs. 40-41), rank updates (Eqs. 42, 44)
-    const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
-    float g_e = 1.f, aa = 0.f;
-    if (ok) {
-      g_e = delta * lam_bar / fmaxf(lam_e, eps);
-      aa = sqrtf(g_e) - 1.f;
-    }
-    any_nosub |= !ok;
-    any_nonfinite |= !isfinite(n2) || !isfinite(lam_e);
-    if (sub == 0 && threadIdx.x == 0) {
-      L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
-      L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
-      if (tr) {
-        tr[4 * step + 0] = lam_e; tr[4 * step + 1] = g_e;
-        tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
-      }
-    }
-    if (aa != 0.f) {
-      const float a2l = aa * aa * lam_e;
-      // both slabs in shared memory: a warp walks its rows, a lane its float4 columns (the padding columns
-      // hold zeros in every vector, so they stay zero in the slabs)
-      // a lane's entries of v and u are the same for every row: they stay in registers
-      const int M4 = Mp >> 2;
-      float4 vj[kMaxIt], uj[kMaxIt];
-#pragma unroll
-      for (int k = 0; k < kMaxIt; ++k) {
-        const int c = lane + 32 * k;
-        vj[k] = uj[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < M4) { vj[k] = reinterpret_cast<const float4*>(vvec)[c]; uj[k] = reinterpret_cast<const float4*>(uvec)[c]; }
-      }
-      for (int r = warp; r < s.nrows; r += CW) {
-        const int i = s.row0 + r;
-        const float vi = vvec[i], ui = uvec[i], ti = tvec[i];
-        const float ati = aa * ti;
-        float4* T4 = reinterpret_cast<float4*>(s.tt + (size_t)r * Mp);
-        float4* P4 = reinterpret_cast<float4*>(s.phi + (size_t)r * Mp);
-#pragma unroll
-        for (int k = 0; k < kMaxIt; ++k) {
-          const int c = lane + 32 * k;
-          if (c < M4) {
-            float4 tt = T4[c], p = P4[c];
-#define FW_UPD(X)                                                                                                  \
-            tt.X = fmaf(ati, vj[k].X, tt.X);                                                                       \
-            p.X = __fadd_rn(p.X, __fadd_rn(__fmul_rn(aa, __fadd_rn(__fmul_rn(vi, uj[k].X), __fmul_rn(ui, vj[k].X))), \
-                                           __fmul_rn(a2l, __fmul_rn(vi, vj[k].X))));
-            FW_UPD(x) FW_UPD(y) FW_UPD(z) FW_UPD(w)
-#undef FW_UPD
-            T4[c] = tt; P4[c] = p;
-          }
+      } else if (ng == 2) {
+        switch (it) {
+          case 1: run_chunk<2, 1>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
+          default: run_chunk<2, 2>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
         }
       }
-      // the step's term of Q (Eq. 44) waits: the recursion does not read Q
-      for (int m = threadIdx.x; m < Mp; m += CT) tk[pending * Mv + m] = tvec[m];
-      if (threadIdx.x == 0) s_aq[pending] = aa * (aa + 2.f);
-      __syncthreads();
-      ++pending;
-      if (pending == KQ) FW_FLUSH_Q()
+      e += (uint32_t)(k1 - k0) * (uint32_t)(a.P + 5) + 1u;
     }
-    // the slab updates are ordered before this CTA's next sends, whose receipt lets a peer read the slab
-    asm volatile("fence.acq_rel.cluster;" ::: "memory");
-    __syncthreads();
   }
-  FW_FLUSH_Q()
-  if (any_nosub && sub == 0 && threadIdx.x == 0) L->iscal[IS_STATUS_NOSUB] = 1;
-  if (any_nonfinite && sub == 0 && threadIdx.x == 0) L->iscal[IS_STATUS_NONFINITE] = 1;
-  }
-done:
-#undef FW_EXCHANGE
-#undef FW_FLUSH_Q
-#undef FW_BAR
-  if (failed) {
+  __syncthreads();
+  if (s.fail || !usable) {
     // a wait gave up: the state of this layer is not to be trusted; report and leave in step with the peers
     if (threadIdx.x == 0) L->iscal[IS_STATUS_TIMEOUT] = 1;
   } else {
-    // ---- write my rows of Phi_y and T^T back ----
-    for (int which = 0; which < 2; ++which) {
-      float* G = which ? L->Tt : L->Phiy;
-      const float* S = which ? s.tt : s.phi;
-      if ((M & 3) == 0) {
-        for (int r = warp; r < s.nrows; r += CW) {
-          float4* dstp = reinterpret_cast<float4*>(G + (size_t)(s.row0 + r) * M);
-          const float4* src = reinterpret_cast<const float4*>(S + (size_t)r * Mp);
-          for (int c = lane; c < (M >> 2); c += 32) dstp[c] = src[c];
-        }
-      } else {
-        for (int i = threadIdx.x; i < s.nrows * Mp; i += CT) {
-          const int r = i / Mp, c = i - r * Mp;
-          if (c < M) G[(size_t)(s.row0 + r) * M + c] = S[i];
-        }
+    if (s.sub == 0 && !s.maxcol)
+      for (int m = threadIdx.x; m < M; m += CT) L->wvec[m] = s.wvec[m];    // alignment weights of the last step
+    if ((M & 3) == 0) {
+      float4* dst = reinterpret_cast<float4*>(L->Phiy + (size_t)s.row0 * M);
+      for (int i = threadIdx.x; i < nrows * (M >> 2); i += CT) dst[i] = reinterpret_cast<const float4*>(csm)[i];
+    } else {
+      for (int i = threadIdx.x; i < nrows * s.Mp; i += CT) {
+        const int r = i / s.Mp, c = i - r * s.Mp;
+        if (c < M) L->Phiy[(size_t)(s.row0 + r) * M + c] = csm[i];
       }
     }
   }
@@ -578,25 +691,24 @@ done:
 }
 
 size_t cluster_smem(int M, int n) {
-  const int Mp = (M + 3) & ~3;
-  const int R = slab_rows(M, n);
-  return (2 * (size_t)R * Mp + (8 + KQ) * (size_t)n * R) * sizeof(float);
+  return ((size_t)slab_rows(M, n) * ((M + 3) & ~3) + (size_t)kVecs * slab_vec(M, n)) * sizeof(float);
 }
-
 
 bool cluster_fits(int M, int n) {
-  return cluster_smem(M, n) <= kSmemLimit && slab_rows(M, n) <= 4 * MAXGPW * CW && M <= 128 * kMaxIt;
+  const int it = slab_trips(M);
+  return M <= kMaxM && it <= kMaxIt && slab_rows(M, n) <= 4 * CW * max_groups(it) && cluster_smem(M, n) <= kSmemLimit;
 }
 
-// what a pass costs the busiest warp of a layer on n CTAs: its groups of four rows times the trips over the columns
+// What a pass costs a layer on n CTAs, in units of the work of one group of four rows and one trip over the columns:
+// the work of the busiest of the four SM partitions, and the fixed part of an exchange (less within one CTA).
 int cluster_cost(int M, int n) {
   const int groups = slab_rows(M, n) / 4;
-  return ((groups + CW - 1) / CW) * ((((M + 3) >> 2) + 31) / 32);
+  return ((groups + 3) / 4) * slab_trips(M) + (n > 1 ? 20 : 8);
 }
 
-// first-fit of the layers' CTA counts (largest first) into clusters of CL: the clusters needed; first[i] (optional)
+// first-fit of the layers' CTA counts (largest first) into clusters of cl: the clusters needed; first[i] (optional)
 // receives the first CTA of layer i.  A layer never straddles a cluster.
-int cluster_pack(const int* cnt, int n, int32_t* first) {
+int cluster_pack(const int* cnt, int n, int cl, int32_t* first) {
   int order[FW_MAX_GROUP], used[FW_MAX_GROUP];
   for (int i = 0; i < n; ++i) { order[i] = i; used[i] = 0; }
   for (int i = 1; i < n; ++i)                       // insertion sort, stable
@@ -607,20 +719,57 @@ int cluster_pack(const int* cnt, int n, int32_t* first) {
   for (int oi = 0; oi < n; ++oi) {
     const int i = order[oi];
     int b = 0;
-    while (b < bins && used[b] + cnt[i] > CL) ++b;
+    while (b < bins && used[b] + cnt[i] > cl) ++b;
     if (b == bins) ++bins;
-    if (first) first[i] = b * CL + used[b];
+    if (first) first[i] = b * cl + used[b];
     used[b] += cnt[i];
   }
   return bins;
 }
 
+// CTA counts of the layers in clusters of cl, of which `resident` run together.  Every layer starts on the fewest CTAs
+// that hold it; then, while the clusters of one wave allow, the layer whose passes cost most is spread over more CTAs
+// (the launch ends with its slowest layer).  Returns the cost of the launch: waves x slowest layer; 0: does not fit.
+int cluster_plan(const int* layer_M, int n, int cl, int resident, int* cnt) {
+  for (int i = 0; i < n; ++i) {
+    cnt[i] = recursion_cluster_ctas(layer_M[i]);
+    if (cnt[i] == 0 || cnt[i] > cl) return 0;
+  }
+  for (int round = 0; round < 16 * FW_MAX_GROUP; ++round) {
+    int worst_cost = 0;
+    for (int i = 0; i < n; ++i) worst_cost = std::max(worst_cost, cluster_cost(layer_M[i], cnt[i]));
+    // all layers at the worst cost have to improve for the launch to gain: try them together
+    int trial[FW_MAX_GROUP];
+    bool improved = true;
+    for (int i = 0; i < n && improved; ++i) {
+      trial[i] = cnt[i];
+      if (cluster_cost(layer_M[i], cnt[i]) != worst_cost) continue;
+      int n2 = cnt[i] + 1;
+      while (n2 <= cl && !(cluster_fits(layer_M[i], n2) && cluster_cost(layer_M[i], n2) < worst_cost)) ++n2;
+      improved = n2 <= cl;                           // else this layer cannot get cheaper: the maximum stays
+      trial[i] = n2;
+    }
+    if (!improved || cluster_pack(trial, n, cl, nullptr) > resident) break;
+    for (int i = 0; i < n; ++i) cnt[i] = trial[i];
+  }
+  int worst = 0;
+  for (int i = 0; i < n; ++i) worst = std::max(worst, cluster_cost(layer_M[i], cnt[i]));
+  const int bins = cluster_pack(cnt, n, cl, nullptr);
+  return worst * ((bins + resident - 1) / resident);
+}
+
+// The plan of the last set of layers a thread launched (a training loop repeats one set).
+struct ClusterPlan {
+  int dev = -1, n = 0, cl = 0, bins = 0;
+  int dims[FW_MAX_GROUP], cnt[FW_MAX_GROUP];
+  int32_t first[FW_MAX_GROUP];
+};
+
 }  // namespace
 
-// CTAs a layer of size M needs at least: the smallest count whose slabs of Phi_y and T^T fit a CTA's shared memory
-// with at most MAXGPW groups of four rows per warp; 0: the layer does not fit on chip
+// CTAs a layer of size M needs at least: the smallest count whose slab of Phi_y fits a CTA; 0: not on chip
 int recursion_cluster_ctas(int M) {
-  for (int n = 1; n <= CL; ++n)
+  for (int n = 1; n <= CLMAX; ++n)
     if (cluster_fits(M, n)) return n;
   return 0;
 }
@@ -630,75 +779,66 @@ bool recursion_cluster_supported(int M) { return recursion_cluster_ctas(M) > 0; 
 cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
                                      cudaStream_t s) {
   static SmemAttrCache attr;
-  static bool nonportable_set[64] = {false};
-  static int max_clusters[64] = {0};
+  static std::mutex mu;
+  static int resident[64][5];        // clusters of 1, 2, 4, 8, 16 CTAs that run together (16: 7 on a B200)
+  thread_local ClusterPlan plan;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); dev = 0; }
-  if (!nonportable_set[dev]) {
-    // clusters of 16 CTAs are beyond the portable size of 8
-    cudaError_t e = cudaFuncSetAttribute(recursion_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    nonportable_set[dev] = true;
-  }
-  cudaError_t e = ensure_dyn_smem(recursion_cluster_kernel, kSmemLimit, attr);
-  if (e != cudaSuccess) return e;
-  if (max_clusters[dev] == 0) {
-    // clusters of 16 that can be resident together (7 on a B200): the plan below stays within one wave of them
-    cudaLaunchConfig_t cfg;
+  auto config = [&](cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cl, int ctas, size_t smem) {
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(CL * 64); cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = kSmemLimit;
-    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[0].val.clusterDim.x = cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, recursion_cluster_kernel, &cfg) != cudaSuccess || nc < 1) {
-      cudaGetLastError();
-      nc = 1;
+  };
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (resident[dev][0] == 0) {
+      // clusters of 16 CTAs are beyond the portable size of 8
+      cudaError_t e = cudaFuncSetAttribute(recursion_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) e = ensure_dyn_smem(recursion_cluster_kernel, kSmemLimit, attr);
+      if (e != cudaSuccess) return e;
+      for (int b = 4; b >= 0; --b) {
+        int nc = 0;
+        config(cfg, at, 1 << b, CLMAX * 64, kSmemLimit);
+        if (cudaOccupancyMaxActiveClusters(&nc, recursion_cluster_kernel, &cfg) != cudaSuccess || nc < 1) {
+          cudaGetLastError();
+          nc = 1;
+        }
+        resident[dev][b] = nc;
+      }
     }
-    max_clusters[dev] = nc;
+  }
+  if (plan.dev != dev || plan.n != g.n || memcmp(plan.dims, layer_M, g.n * sizeof(int)) != 0) {
+    // the cluster size whose plan costs least; the larger one where two tie (layers can spread further)
+    int best = 0;
+    plan.dev = -1;
+    for (int b = 4; b >= 0; --b) {
+      int cnt[FW_MAX_GROUP];
+      const int c = cluster_plan(layer_M, g.n, 1 << b, resident[dev][b], cnt);
+      if (c == 0 || (best != 0 && c >= best)) continue;
+      best = c;
+      plan.cl = 1 << b;
+      memcpy(plan.cnt, cnt, g.n * sizeof(int));
+    }
+    if (best == 0) return cudaErrorInvalidValue;
+    plan.bins = cluster_pack(plan.cnt, g.n, plan.cl, plan.first);
+    memcpy(plan.dims, layer_M, g.n * sizeof(int));
+    plan.n = g.n; plan.dev = dev;
   }
   ClusterArgs a;
   memset(&a, 0, sizeof(a));
   a.g = g; a.traces = traces; a.K = K; a.P = P;
-  // Every layer starts on the fewest CTAs that hold it; then, while the clusters of one wave allow, the layer whose
-  // busiest warp has the most work per pass is spread over more CTAs (the launch ends with its slowest layer).
-  int cnt[FW_MAX_GROUP];
-  for (int i = 0; i < g.n; ++i) {
-    cnt[i] = recursion_cluster_ctas(layer_M[i]);
-    if (cnt[i] == 0) return cudaErrorInvalidValue;
-  }
-  for (int round = 0; round < 16 * FW_MAX_GROUP; ++round) {
-    int worst = -1, worst_cost = 0;
-    for (int i = 0; i < g.n; ++i) {
-      const int c = cluster_cost(layer_M[i], cnt[i]);
-      if (c > worst_cost) { worst_cost = c; worst = i; }
-    }
-    if (worst < 0) break;
-    // all layers at the worst cost have to improve for the launch to gain: try them in turn
-    bool improved = false;
-    for (int i = 0; i < g.n && !improved; ++i) {
-      if (cluster_cost(layer_M[i], cnt[i]) != worst_cost) continue;
-      int n2 = cnt[i] + 1;
-      while (n2 <= CL && !(cluster_fits(layer_M[i], n2) && cluster_cost(layer_M[i], n2) < worst_cost)) ++n2;
-      if (n2 > CL) { improved = false; break; }       // this layer cannot get cheaper: the maximum stays
-      const int keep = cnt[i];
-      cnt[i] = n2;
-      if (cluster_pack(cnt, g.n, nullptr) > max_clusters[dev]) { cnt[i] = keep; break; }
-      improved = true;
-    }
-    if (!improved) break;
-  }
-  const int bins = cluster_pack(cnt, g.n, a.first_cta);
-  for (int i = 0; i < g.n; ++i) a.ncta[i] = cnt[i];
   size_t smem = 0;
   for (int i = 0; i < g.n; ++i) {
-    const size_t need = cluster_smem(layer_M[i], cnt[i]);
-    if (need > smem) smem = need;
+    a.first_cta[i] = plan.first[i]; a.ncta[i] = plan.cnt[i];
+    smem = std::max(smem, cluster_smem(layer_M[i], plan.cnt[i]));
   }
+  config(cfg, at, plan.cl, plan.bins * plan.cl, smem);
   ProfScope ps(FW_PROF_RECUR_CHIP, s);
-  recursion_cluster_kernel<<<bins * CL, CT, smem, s>>>(a);
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, recursion_cluster_kernel, a);
 }
 
 }  // namespace fw

@@ -1,0 +1,73 @@
+"""On-chip recursion at the edges of its register tiles (rows of 128 entries per trip, one or two groups of four rows
+per warp, one or several CTAs per layer) and of its step batches (T and Q take eight steps at a time)."""
+import numpy as np
+import pytest
+
+from oracle import fw_oracle as O
+from paper_2010_01546_b200 import synth
+
+from fwtest_util import TOL_FP32, group_reduce_with_replay, oracle_hyper, reduce_with_replay, rel_fro, t2n
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    from paper_2010_01546_b200 import binding as B, build
+    build.build_library()
+    return torch, B
+
+
+def spd32(M, cond, seed):
+    Phi, _, _ = synth.spd_with_spectrum(M, cond, seed, basis="qr" if M <= 300 else "householder")
+    P = Phi.astype(np.float32)
+    return np.triu(P) + np.triu(P, 1).T
+
+
+def check(L, Lo, B):
+    for f, ref in ((B.FW_F_T, Lo.T), (B.FW_F_Q, Lo.Q), (B.FW_F_QS, Lo.Qs), (B.FW_F_PHIY, Lo.phiy())):
+        assert rel_fro(t2n(L.get(f)).reshape(ref.shape), ref) <= TOL_FP32
+
+
+@pytest.mark.parametrize("M", [1, 4, 63, 64, 65, 128, 129, 255, 256, 257, 384, 513, 624])
+def test_tile_edges(env, M):
+    torch, B = env
+    Phi = spd32(M, 1e2, 900 + M)
+    La, Lb = B.Layer(M, 4, beta=0.2, gamma=1.0), B.Layer(M, 4, beta=0.2, gamma=1.0)
+    Lo = O.Layer(M, 4, oracle_hyper(La.desc))
+    for L in (La, Lb):
+        L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda())
+    Lo.set_phix(Phi)
+    reduce_with_replay(La, Lo, 2, 3, B, torch)
+    check(La, Lo, B)
+    # 18 steps of one call (batches of 8, 8 and 2) are those of single calls, Q_s apart (smoothed once per call)
+    for _ in range(16):
+        La.cond_reduce(1, 3)
+    Lb.cond_reduce(18, 3)
+    for f in (B.FW_F_T, B.FW_F_Q, B.FW_F_PHIY, B.FW_F_ALIGN_W):
+        assert torch.equal(La.get(f), Lb.get(f))
+    assert La.sync_status() in (B.FW_OK, B.FW_WARN_NO_SUBSPACE)
+
+
+@pytest.mark.parametrize("dims", [[256] * 64, [620, 577, 300, 145, 64, 33, 1], [128, 12]])
+def test_groups(env, dims):
+    torch, B = env
+    Ls, Los = [], []
+    for i, M in enumerate(dims):
+        Phi = spd32(M, 1e2, 40 + i)
+        L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+        Lo = O.Layer(M, 4, oracle_hyper(L.desc))
+        L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda()); Lo.set_phix(Phi)
+        Ls.append(L); Los.append(Lo)
+    if len(dims) > 8:                       # a full group: every layer must come out as it does alone
+        B.fw_group_cond_reduce([L.handle for L in Ls], 2, 4)
+        for i in (0, 27, 28, 63):
+            L = B.Layer(dims[i], 4, beta=0.0, gamma=1.0)
+            L.set(B.FW_F_PHIX, torch.from_numpy(spd32(dims[i], 1e2, 40 + i)).cuda())
+            L.cond_reduce(2, 4)
+            assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), t2n(L.get(B.FW_F_T))) <= TOL_FP32
+        return
+    group_reduce_with_replay(Ls, Los, 2, 4, B, torch)
+    for L, Lo in zip(Ls, Los):
+        check(L, Lo, B)
