@@ -28,7 +28,7 @@ struct fw_layer {
   bool block_open;     // earlier calls of the current block left their sums in the accumulators (FW_COV_ACCUMULATE)
   bool block_shifted;  // the current block is centred on the pilot mean taken from its first call
   int64_t acc_rows;    // rows accumulated by those calls
-  uint32_t bar_base;   // arrivals so far at this layer's grid-barrier counter (persistent recursion launches it led)
+  uint32_t epoch;      // packet exchanges of this layer so far (recursion of large layers)
   float* W;
   float* b;
 };
@@ -101,6 +101,9 @@ size_t carve(const fw_layer_desc& d, char* base, LayerDev* h) {
   L.colsum_acc = (float*)take(vec);
   L.gq_tmp = (float*)take((size_t)d.N * vec);
   L.pmean = (float*)take(vec);
+  L.vh = (float*)take(kHist * vec); L.th = (float*)take(kHist * vec);
+  L.ah = (float*)take(kHist * sizeof(float));
+  L.px = (unsigned long long*)take(3 * ((M + 15) & ~(size_t)15) * sizeof(unsigned long long));
   return off;
 }
 
@@ -222,7 +225,6 @@ const Tuning& tuning() {
     v.pair_splits = geti("FW_PAIR_SPLITS", 0);
     v.pair_debug = getenv("FW_PAIR_DEBUG") ? 1 : 0;
     v.pass_shape = geti("FW_PASS_SHAPE", 0);
-    v.persist_max_mb = geti("FW_PERSIST_MAX_MB", 512);
     v.gram_waves_pct = geti("FW_GRAM_WAVES_PCT", 200);
     if (v.gram_waves_pct < 50 || v.gram_waves_pct > 1600) v.gram_waves_pct = 200;
     return v;
@@ -327,7 +329,7 @@ fw_status fw_layer_create(const fw_layer_desc* d, void* dev_workspace, size_t by
   L->dev = (LayerDev*)dev_workspace;
   L->have_cov = false; L->first_block = true; L->phiy_stale = true; L->t_identity = true;
   L->shift_zero = false;               // cleared by init_identity, but the first block settles it either way
-  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->bar_base = 0;
+  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->epoch = 0;
   cudaError_t e = cudaMemcpyAsync(L->dev, &L->h, sizeof(LayerDev), cudaMemcpyHostToDevice, L->stream);
   if (e == cudaSuccess) e = launch_init_identity(L->dev, d->M, L->stream);
   if (e != cudaSuccess) { delete L; return cuda_fail(e, "fw_layer_create"); }
@@ -346,7 +348,7 @@ fw_status fw_layer_reset(fw_layer* L) {
   FW_CUDA(launch_init_identity(L->dev, L->d.M, L->stream), "fw_layer_reset");
   L->have_cov = false; L->first_block = true; L->phiy_stale = true; L->t_identity = true;
   L->shift_zero = true;                // init_identity clears the shift vector
-  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->bar_base = 0;
+  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->epoch = 0;
   return FW_OK;
 }
 
@@ -609,73 +611,45 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
   st = resync_phiy(L, n);
   if (st != FW_OK) return st;
   if (K == 0) return FW_OK;      // no step: Phi_y has been brought up to date, nothing else changes
-  // small layers: the whole K-step recursion runs on chip, a layer on 1 to 16 CTAs of a cluster;
-  // the rest takes the multi-launch path (one launch per pass, batched over layers)
-  GroupDev gc, gl; PtrTable tc, tl;
-  memset(&tc, 0, sizeof(tc)); memset(&tl, 0, sizeof(tl));
-  gc.n = gl.n = 0; gc.pad = gl.pad = 0;
-  int ml = 0;
-  int dims_c[FW_MAX_GROUP];
-  // largest layers first: CTAs are handed out in launch order, so the long row blocks start early and the
-  // short ones fill the end of every pass
-  std::vector<int> order(n);
+  // small layers: a layer on 1 to 16 CTAs of a cluster; large ones on teams of CTAs of a cooperative launch; leaky ones
+  // (gamma < 1) one launch per pass, batched over the layers
+  GroupDev gc, gp, gl; PtrTable tc, tp, tl;
+  memset(&tc, 0, sizeof(tc)); memset(&tp, 0, sizeof(tp)); memset(&tl, 0, sizeof(tl));
+  gc.n = gp.n = gl.n = 0; gc.pad = gp.pad = gl.pad = 0;
+  int dims_c[FW_MAX_GROUP], dims_p[FW_MAX_GROUP], ml = 0, row_blocks = 0;
+  fw_layer* team[FW_MAX_GROUP];
+  // largest layers first: CTAs are handed out in launch order, so the long row blocks start early
+  int order[FW_MAX_GROUP];
   for (int i = 0; i < n; ++i) order[i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return L[a]->d.M > L[b]->d.M; });
+  std::stable_sort(order, order + n, [&](int a, int b) { return L[a]->d.M > L[b]->d.M; });
   for (int oi = 0; oi < n; ++oi) {
-    const int i = order[oi];
-    float* t = traces_or_null ? traces_or_null[i] : nullptr;
-    if (L[i]->d.gamma == 1.0f && recursion_cluster_supported(L[i]->d.M)) {
-      gc.layer[gc.n] = L[i]->dev; tc.p[gc.n] = t; dims_c[gc.n] = L[i]->d.M; ++gc.n;
+    fw_layer* l = L[order[oi]];
+    float* t = traces_or_null ? traces_or_null[order[oi]] : nullptr;
+    const int M = l->d.M;
+    if (l->d.gamma != 1.0f) {
+      gl.layer[gl.n] = l->dev; tl.p[gl.n] = t; ++gl.n;
+      ml = std::max(ml, M);
+      row_blocks += (M + kGemvRowsPerBlock - 1) / kGemvRowsPerBlock;
+    } else if (recursion_cluster_supported(M)) {
+      gc.layer[gc.n] = l->dev; tc.p[gc.n] = t; dims_c[gc.n] = M; ++gc.n;
     } else {
-      gl.layer[gl.n] = L[i]->dev; tl.p[gl.n] = t; ++gl.n;
-      if (L[i]->d.M > ml) ml = L[i]->d.M;
+      gp.layer[gp.n] = l->dev; tp.p[gp.n] = t; dims_p[gp.n] = M; team[gp.n] = l; ++gp.n;
     }
   }
   if (gc.n) FW_CUDA(launch_recursion_cluster(gc, tc, dims_c, K, P, s), "recursion (cluster)");
-  if (gl.n) {
-    // large layers: gamma = 1 layers with 16-byte rows take all K steps in one persistent cooperative launch;
-    // leaky layers (their update needs transposed tiles) and odd sizes take one launch per pass
-    GroupDev gp, go; PtrTable tp, to;
-    memset(&tp, 0, sizeof(tp)); memset(&to, 0, sizeof(to));
-    gp.n = go.n = 0; gp.pad = go.pad = 0;
-    int dims_p[FW_MAX_GROUP];
-    fw_layer* leader = nullptr;
-    int mo = 0, row_blocks = 0;
-    bool any_leaky = false;
-    // The persistent launch wins where a pass is short against a kernel boundary (a handful of layers, up to a few
-    // hundred MB of state in all); past that the statically split rows stream a few percent below the many small
-    // CTAs of the per-pass launches, which the hardware balances as it goes.
-    double state_mb = 0;
-    for (int i = 0; i < n; ++i)
-      if (!(L[i]->d.gamma == 1.0f && recursion_cluster_supported(L[i]->d.M)))
-        state_mb += 4.0 * L[i]->d.M * (double)L[i]->d.M / 1e6;
-    const bool persist_ok = state_mb <= (double)tuning().persist_max_mb;
-    for (int oi = 0; oi < n; ++oi) {
-      const int i = order[oi];
-      if (L[i]->d.gamma == 1.0f && recursion_cluster_supported(L[i]->d.M)) continue;
-      float* t = traces_or_null ? traces_or_null[i] : nullptr;
-      const int Mi = L[i]->d.M;
-      const float gi = L[i]->d.gamma;
-      if (persist_ok && recursion_persist_supported(&Mi, &gi, 1)) {
-        if (!leader) leader = L[i];
-        dims_p[gp.n] = Mi;
-        gp.layer[gp.n] = L[i]->dev; tp.p[gp.n] = t; ++gp.n;
-      } else {
-        go.layer[go.n] = L[i]->dev; to.p[go.n] = t; ++go.n;
-        if (Mi > mo) mo = Mi;
-        row_blocks += (Mi + kGemvRowsPerBlock - 1) / kGemvRowsPerBlock;
-        any_leaky |= (gi != 1.0f);
-      }
-    }
-    if (gp.n)
-      FW_CUDA(launch_recursion_persist(gp, tp, dims_p, K, P, leader->h.iscal + IS_GRID_BAR,
-                                       leader->h.iscal + IS_STATUS_TIMEOUT, &leader->bar_base, s),
-              "recursion (persistent)");
-    for (int k = 0; k < K && go.n; ++k)
-      FW_CUDA(launch_recursion_step(go, P, k, to, mo, any_leaky, row_blocks, s), "recursion step");
-  }
   bool any_beta = false;
   for (int i = 0; i < n; ++i) any_beta |= (L[i]->d.beta > 0.f);
+  // large layers: teams of CTAs; T and Q take the recorded steps, up to kHist at a time
+  for (int k0 = 0; k0 < K && gp.n; k0 += kHist) {
+    const int kc = std::min(kHist, K - k0);
+    uint32_t epoch[FW_MAX_GROUP];
+    for (int i = 0; i < gp.n; ++i) { epoch[i] = team[i]->epoch; team[i]->epoch += (uint32_t)team_exchanges(kc, P); }
+    FW_CUDA(launch_recursion_team(gp, tp, dims_p, epoch, k0, kc, P, k0 + kc == K, s), "recursion (teams)");
+    FW_CUDA(launch_recursion_apply(gp, dims_p, kc, any_beta && k0 + kc == K, s), "recursion (T, Q)");
+  }
+  // leaky layers (their update needs transposed tiles): one launch per pass
+  for (int k = 0; k < K && gl.n; ++k)
+    FW_CUDA(launch_recursion_step(gl, P, k, tl, ml, row_blocks, s), "recursion step");
   if (gl.n && any_beta) FW_CUDA(launch_smooth(gl, ml, s), "smooth");
   for (int i = 0; i < n; ++i) L[i]->t_identity = false;
   return FW_OK;
@@ -988,11 +962,6 @@ fw_status fw_layer_sync_status(fw_layer* L) {
   FW_CUDA(cudaStreamSynchronize(L->stream), "status sync");
   if (is[IS_STATUS_NONFINITE] || is[IS_STATUS_NOSUB] || is[IS_STATUS_TIMEOUT]) {
     FW_CUDA(cudaMemsetAsync(L->h.iscal + IS_STATUS_NOSUB, 0, 3 * sizeof(int32_t), L->stream), "status clear");
-  }
-  if (is[IS_STATUS_TIMEOUT]) {
-    // a persistent launch this layer led may have left its barrier counter short: start it afresh
-    FW_CUDA(cudaMemsetAsync(L->h.iscal + IS_GRID_BAR, 0, 2 * sizeof(int32_t), L->stream), "barrier clear");
-    L->bar_base = 0;
   }
   if (is[IS_STATUS_TIMEOUT]) return FW_ERR_TIMEOUT;
   if (is[IS_STATUS_NONFINITE]) return FW_WARN_NONFINITE;

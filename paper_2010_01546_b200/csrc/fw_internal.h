@@ -59,7 +59,14 @@ struct LayerDev {
   // pilot mean of an unshifted tensor-core block: its outer product is taken out of the Gram accumulators as the
   // rows go by (and put back by the moment kernels), so that the accumulators hold centred sums
   float* pmean;         // M
+  // recursion of large layers (fw_recursion_team.cu): steps whose rank-one terms T, Q have not taken yet, and the packets
+  // {value, exchange number} the CTAs of a layer exchange
+  float* vh;            // kHist x M  unit vectors v_e of the steps
+  float* th;            // kHist x M  t = T^T v_e of the steps
+  float* ah;            // kHist      a_e of the steps
+  unsigned long long* px;   // 3 x M (rounded up to even)
 };
+constexpr int kHist = 16;   // steps of a call between two updates of T and Q
 
 // The pilot mean as the tensor core reads it: rounded to bf16 (nearest even) for bf16 X, truncated to TF32 for
 // fp32 X.  The Gram kernel that subtracts n c c^T and the moment kernels that add it back both use this value.
@@ -74,8 +81,7 @@ constexpr int kCorrEveryStages = 8;   // CTA-pair Gram: one correction MMA per a
 
 
 enum { SC_LAMBDA_BAR = 0, SC_LAMBDA_E = 1, SC_G_E = 2, SC_A_E = 3, SC_LAST_NORM2 = 4, SC_COUNT = 8 };
-enum { IS_MPRIME = 0, IS_SETSIZE = 1, IS_STATUS_NOSUB = 2, IS_STATUS_NONFINITE = 3, IS_STATUS_TIMEOUT = 4,
-       IS_GRID_BAR = 5 /* grid-barrier counter and, after it, the abort flag of the persistent recursion */, IS_COUNT = 8 };
+enum { IS_MPRIME = 0, IS_SETSIZE = 1, IS_STATUS_NOSUB = 2, IS_STATUS_NONFINITE = 3, IS_STATUS_TIMEOUT = 4, IS_COUNT = 8 };
 
 constexpr int kGemvRowsPerBlock = 32;   // rows of a matrix handled by one CTA of a GEMV pass (default shape)
 constexpr int kGemvMinRowsPerBlock = 8; // smallest pass shape: sizes the per-block partial sums
@@ -179,8 +185,6 @@ struct Tuning {
   int pair_splits;     // FW_PAIR_SPLITS  row slabs per problem of the CTA-pair kernels (0: chosen by the scheduler)
   int pair_debug;      // FW_PAIR_DEBUG   print the chosen slabs
   int pass_shape;      // FW_PASS_SHAPE   42 / 24 / 18 / 41: shape of the streaming recursion passes (0: automatic)
-  int persist_max_mb;  // FW_PERSIST_MAX_MB  largest total state (MB of 4 M^2 over the large layers of a call) the
-                       //                 persistent recursion launch takes (default 512; 0: never)
   int gram_waves_pct;  // FW_GRAM_WAVES_PCT  CTAs of a single-CTA Gram launch, in percent of the SM count (default 200)
 };
 const Tuning& tuning();
@@ -210,8 +214,9 @@ cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t*
 // fresh[i] != 0: the first call of the block, acc is overwritten
 cudaError_t launch_accumulate(const GroupDev& g, const int32_t* splits, const int32_t* fresh, const float* corr,
                               const int32_t* layer_M, cudaStream_t s);
+// one step of leaky layers (gamma < 1), a launch per pass
 cudaError_t launch_recursion_step(const GroupDev& g, int P, int step, const PtrTable& traces, int max_M,
-                                  bool any_leaky, int row_blocks, cudaStream_t s);
+                                  int row_blocks, cudaStream_t s);
 cudaError_t launch_smooth(const GroupDev& g, int max_M, cudaStream_t s);
 // Whitening from the eigenvalue decomposition (fw_evd.cu): one-sided Jacobi in fp64 on src[i], then (with_v) T, Q, Phi_y
 size_t evd_scratch_bytes(int M);
@@ -225,12 +230,14 @@ int recursion_cluster_ctas(int M);
 // All K steps of a call for layers that fit on chip, T, Q and Qs included
 cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
                                      cudaStream_t s);
-// All K steps of a group of large gamma = 1 layers as one persistent cooperative launch.  bar_words: two ints in the
-// leading layer's workspace (barrier counter, abort flag); bar_base_host: the host's count of arrivals at that
-// counter so far, advanced by the launch.
-bool recursion_persist_supported(const int* layer_M, const float* layer_gamma, int n);
-cudaError_t launch_recursion_persist(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
-                                     int32_t* bar_words, int32_t* status, uint32_t* bar_base_host, cudaStream_t s);
+// Steps k0 ... k0 + K - 1 (K <= kHist) of a call for large gamma = 1 layers, as one cooperative launch; v_e, a_e of the
+// steps are left in vh, ah.  epoch[i]: number of the layer's last packet exchange, advanced by team_exchanges(K, P) a
+// launch.  last: the launch ends the call.
+int team_exchanges(int K, int P);
+cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, const uint32_t* epoch,
+                                  int k0, int K, int P, bool last, cudaStream_t s);
+// T, Q take the K steps recorded in vh, ah (Eqs. 42, 44), in step order; smooth: Qs <- beta Qs + (1 - beta) Q after them
+cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K, bool smooth, cudaStream_t s);
 // zero-padded copies [B][H + 2][W + 2][C] of n NHWC fp32 activations in one launch; dst_floats[i] (a multiple of 4)
 // floats of dst[i] are written in all
 cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, const int* B, const int* H, const int* W,

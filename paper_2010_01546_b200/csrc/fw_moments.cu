@@ -336,6 +336,7 @@ __global__ void init_identity_kernel(const LayerDev* L) {
     for (int m = threadIdx.x; m < M; m += blockDim.x) {
       L->mu[m] = 0.f; L->mu_prev[m] = 0.f; L->phi[m] = 0.f; L->shift[m] = 0.f;
     }
+    for (int m = threadIdx.x; m < 3 * ((M + 15) & ~15); m += blockDim.x) L->px[m] = 0;     // no exchange has this number
     if (threadIdx.x < SC_COUNT) L->scal[threadIdx.x] = 0.f;
     if (threadIdx.x < IS_COUNT) L->iscal[threadIdx.x] = 0;
   }

@@ -1,5 +1,6 @@
-// Recursive condition-number reduction (Sec. 4): one step is a fixed sequence
-// of passes over the layer's M x M state, each pass one launch batched over all
+// Recursive condition-number reduction (Sec. 4) of layers with a leaky transform
+// (gamma < 1; the others run in fw_recursion_cluster.cu and fw_recursion_team.cu):
+// one step is a fixed sequence of passes over the layer's M x M state, each pass one launch batched over all
 // layers of the group (grid.y = layer).  Every pass is a row-wise product
 // y = A x with A row-major: a warp owns rows, lanes stride the columns with
 // 128-bit loads, partial sums are reduced by warp shuffles.  Scalars (m',
@@ -19,7 +20,6 @@
 namespace fw {
 namespace {
 
-constexpr int RB = kGemvRowsPerBlock;      // rows per CTA of the update kernel and of the default pass shape
 constexpr int WARPS = kGemvThreads / 32;   // 8
 // Pass shapes (rows per warp R, column positions per trip C); a CTA covers 8 R rows.  Measured:
 //   (4, 1)  many CTAs per SM (64 layers of the stress sweep): the lightest loop at four CTAs per SM
@@ -126,10 +126,9 @@ __global__ void __launch_bounds__(kGemvThreads, (C == 1) ? 4 : 2) recursion_pass
   constexpr int RBk = WARPS * R;                // rows per CTA of this shape
   const int row0 = blockIdx.x * RBk;
   if (row0 >= M) return;
-  // FINAL only: blockIdx.z == 1 is the product t = T^T v, blockIdx.z == 2 (leaky layers) q = P^T v
+  // FINAL only: blockIdx.z == 1 is the product t = T^T v, blockIdx.z == 2 q = P^T v
   const int zi = (PASS == PASS_FINAL) ? (int)blockIdx.z : 0;
   const bool second = zi != 0;
-  if (zi == 2 && L->gamma == 1.f) return;
   const int nblk = (M + RBk - 1) / RBk;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ float red[WARPS];
@@ -310,21 +309,15 @@ __global__ void __launch_bounds__(kGemvThreads, (C == 1) ? 4 : 2) recursion_pass
   }
 }
 
-// Rank updates at gamma == 1 for a block of rows.  Element-wise, 128-bit accesses.
-//   Q   += a (a + 2) t t^T                               (Eq. 44)
-//   T^T += a t v^T            i.e. T += a v t^T          (Eq. 42)
-//   Phiy += a (v u^T + u v^T) + a^2 lambda_e v v^T        (from Phiy = T Phix T^T)
-// The Phiy and Q terms are evaluated symmetrically in (i, j) so both stay exactly symmetric.
-__global__ void __launch_bounds__(kGemvThreads) recursion_update_kernel(const __grid_constant__ GroupDev g,
-                                                                        const __grid_constant__ PtrTable traces,
-                                                                        int step, int pass_rows) {
-  const LayerDev* L = g.layer[blockIdx.y];
-  const int M = L->M;
-  const int row0 = blockIdx.x * RB;
-  if (row0 >= M) return;
-  const int nblk = (M + pass_rows - 1) / pass_rows;   // partials of lambda_e: one per CTA of the FINAL pass
+// lambda_e, g_e, a_e of the step (Eqs. 36, 40-41); one CTA per layer
+__global__ void __launch_bounds__(kGemvThreads) recursion_scalars_kernel(const __grid_constant__ GroupDev g,
+                                                                         const __grid_constant__ PtrTable traces,
+                                                                         int step, int pass_rows) {
+  const LayerDev* L = g.layer[blockIdx.x];
+  const int nblk = (L->M + pass_rows - 1) / pass_rows;   // partials of lambda_e: one per CTA of the FINAL pass
   __shared__ float red[WARPS];
   const float lam_e = block_sum_partials(L->part + 2 * L->part_stride, nblk, red);
+  if (threadIdx.x != 0) return;
   const float n2 = L->scal[SC_LAST_NORM2];
   const int cnt = L->iscal[IS_SETSIZE];
   const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
@@ -333,80 +326,15 @@ __global__ void __launch_bounds__(kGemvThreads) recursion_update_kernel(const __
     g_e = L->delta * L->scal[SC_LAMBDA_BAR] / fmaxf(lam_e, L->eps);   // Eq. 40
     a = sqrtf(g_e) - 1.f;                                             // Eq. 41
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = a;
-    if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
-    if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;   // NaN / Inf in the state
-    float* tr = const_cast<float*>(reinterpret_cast<const float*>(traces.p[blockIdx.y]));
-    if (tr) {
-      tr[4 * step + 0] = lam_e; tr[4 * step + 1] = g_e;
-      tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)L->iscal[IS_MPRIME];
-    }
-  }
-  if (L->gamma != 1.f) return;   // leaky layers are updated by recursion_update_leaky_kernel
-  if (a == 0.f) return;          // gamma == 1 and a == 0: nothing changes
-  const float aq = a * (a + 2.f);
-  const float a2l = a * a * lam_e;
-  const float* v = L->v; const float* u = L->u; const float* t = L->t;
-  const int rows = min(RB, M - row0);
-  if ((M & 3) == 0) {
-    const int M4 = M >> 2;
-    const int total = rows * M4;
-    // two elements per trip, all six matrix loads issued before any is used: with few CTAs per SM (a handful of
-    // layers) the bytes a thread keeps in flight set the bandwidth the kernel reaches
-    for (int e0 = threadIdx.x; e0 < total; e0 += 2 * blockDim.x) {
-      float4 q[2], tt[2], p[2];
-      int64_t off[2];
-      int ri[2], cj[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int e = e0 + h * blockDim.x;
-        const bool in = e < total;
-        const int r = in ? e / M4 : 0, c4 = in ? e - r * M4 : 0;
-        ri[h] = in ? row0 + r : -1; cj[h] = c4;
-        off[h] = (int64_t)(row0 + r) * M4 + c4;
-        if (in) {
-          q[h] = reinterpret_cast<const float4*>(L->Q)[off[h]];
-          tt[h] = reinterpret_cast<const float4*>(L->Tt)[off[h]];
-          p[h] = reinterpret_cast<const float4*>(L->Phiy)[off[h]];
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (ri[h] < 0) continue;
-        const int i = ri[h];
-        const float vi = v[i], ui = u[i], ti = t[i];
-        const float4 vj = reinterpret_cast<const float4*>(v)[cj[h]];
-        const float4 uj = reinterpret_cast<const float4*>(u)[cj[h]];
-        const float4 tj = reinterpret_cast<const float4*>(t)[cj[h]];
-#define FW_UPD(X)                                                                              \
-        q[h].X = __fadd_rn(q[h].X, __fmul_rn(aq, __fmul_rn(ti, tj.X)));                          \
-        tt[h].X = fmaf(a * ti, vj.X, tt[h].X);                                                   \
-        p[h].X = __fadd_rn(p[h].X, __fadd_rn(__fmul_rn(a, __fadd_rn(__fmul_rn(vi, uj.X), __fmul_rn(ui, vj.X))), \
-                                             __fmul_rn(a2l, __fmul_rn(vi, vj.X))));
-        FW_UPD(x) FW_UPD(y) FW_UPD(z) FW_UPD(w)
-#undef FW_UPD
-        reinterpret_cast<float4*>(L->Q)[off[h]] = q[h];
-        reinterpret_cast<float4*>(L->Tt)[off[h]] = tt[h];
-        reinterpret_cast<float4*>(L->Phiy)[off[h]] = p[h];
-      }
-    }
-  } else {
-    const int total = rows * M;
-    for (int e = threadIdx.x; e < total; e += blockDim.x) {
-      const int r = e / M, j = e - r * M;
-      const int i = row0 + r;
-      const float vi = v[i], ui = u[i], ti = t[i];
-      const int64_t off = (int64_t)i * M + j;
-      L->Q[off] = __fadd_rn(L->Q[off], __fmul_rn(aq, __fmul_rn(ti, t[j])));
-      L->Tt[off] = fmaf(a * ti, v[j], L->Tt[off]);
-      L->Phiy[off] = __fadd_rn(L->Phiy[off],
-                               __fadd_rn(__fmul_rn(a, __fadd_rn(__fmul_rn(vi, u[j]), __fmul_rn(ui, v[j]))),
-                                         __fmul_rn(a2l, __fmul_rn(vi, v[j]))));
-    }
+  L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = a;
+  if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
+  if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;   // NaN / Inf in the state
+  float* tr = const_cast<float*>(reinterpret_cast<const float*>(traces.p[blockIdx.x]));
+  if (tr) {
+    tr[4 * step + 0] = lam_e; tr[4 * step + 1] = g_e;
+    tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)L->iscal[IS_MPRIME];
   }
 }
-
 
 // Rank updates with leakage gamma < 1 (Eqs. 42, 44).  With P = T Phix kept as Pt = P^T and q = P^T v:
 //   Q    <- g^2 (Q + a(a+2) t t^T) + (1-g)^2 I + g(1-g) (a (v t^T + t v^T) + T + T^T)
@@ -418,7 +346,6 @@ __global__ void __launch_bounds__(kGemvThreads) recursion_update_kernel(const __
 __global__ void __launch_bounds__(256) recursion_update_leaky_kernel(const __grid_constant__ GroupDev g) {
   const LayerDev* L = g.layer[blockIdx.z];
   const float gm = L->gamma;
-  if (gm == 1.f) return;
   const int M = L->M;
   const int bi = blockIdx.y, bj = blockIdx.x;
   if (bj < bi || bi * 32 >= M || bj * 32 >= M) return;
@@ -500,7 +427,7 @@ __global__ void __launch_bounds__(256) smooth_kernel(const __grid_constant__ Gro
 
 template <int R, int C>
 static cudaError_t recursion_step_launches(const GroupDev& g, int P, int step, const PtrTable& traces, int max_M,
-                                           bool any_leaky, cudaStream_t s) {
+                                           cudaStream_t s) {
   constexpr int RBk = WARPS * R;
   const int nblk = (max_M + RBk - 1) / RBk;
   const size_t shm = (size_t)((max_M + 3) & ~3) * sizeof(float);
@@ -514,11 +441,10 @@ static cudaError_t recursion_step_launches(const GroupDev& g, int P, int step, c
     recursion_pass_kernel<PASS_POWER, R, C><<<grid, block, shm, s>>>(g, cur, cur ^ 1);
     cur ^= 1;
   }
-  dim3 grid2(nblk, g.n, any_leaky ? 3 : 2);
+  dim3 grid2(nblk, g.n, 3);
   { ProfScope ps(FW_PROF_RECUR_MV, s); recursion_pass_kernel<PASS_FINAL, R, C><<<grid2, block, shm, s>>>(g, cur, 0); }
-  dim3 gridu((max_M + RB - 1) / RB, g.n);
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); recursion_update_kernel<<<gridu, block, 0, s>>>(g, traces, step, RBk); }
-  if (any_leaky) {
+  { ProfScope ps(FW_PROF_RECUR_UPD, s); recursion_scalars_kernel<<<g.n, block, 0, s>>>(g, traces, step, RBk); }
+  {
     const int t32 = (max_M + 31) / 32;
     ProfScope ps(FW_PROF_RECUR_UPD, s);
     recursion_update_leaky_kernel<<<dim3(t32, t32, g.n), dim3(32, 8), 0, s>>>(g);
@@ -528,15 +454,15 @@ static cudaError_t recursion_step_launches(const GroupDev& g, int P, int step, c
 
 // row_blocks: 32-row blocks that have rows to work on, summed over the group's layers
 cudaError_t launch_recursion_step(const GroupDev& g, int P, int step, const PtrTable& traces, int max_M,
-                                  bool any_leaky, int row_blocks, cudaStream_t s) {
+                                  int row_blocks, cudaStream_t s) {
   const int forced = tuning().pass_shape;   // tuning aid
-  if (forced == 42) return recursion_step_launches<4, 2>(g, P, step, traces, max_M, any_leaky, s);
-  if (forced == 24) return recursion_step_launches<2, 4>(g, P, step, traces, max_M, any_leaky, s);
-  if (forced == 18) return recursion_step_launches<1, 8>(g, P, step, traces, max_M, any_leaky, s);
-  if (forced == 41) return recursion_step_launches<4, 1>(g, P, step, traces, max_M, any_leaky, s);
-  if (row_blocks < 148) return recursion_step_launches<2, 4>(g, P, step, traces, max_M, any_leaky, s);
-  if (row_blocks < 8 * 148) return recursion_step_launches<4, 2>(g, P, step, traces, max_M, any_leaky, s);
-  return recursion_step_launches<4, 1>(g, P, step, traces, max_M, any_leaky, s);
+  if (forced == 42) return recursion_step_launches<4, 2>(g, P, step, traces, max_M, s);
+  if (forced == 24) return recursion_step_launches<2, 4>(g, P, step, traces, max_M, s);
+  if (forced == 18) return recursion_step_launches<1, 8>(g, P, step, traces, max_M, s);
+  if (forced == 41) return recursion_step_launches<4, 1>(g, P, step, traces, max_M, s);
+  if (row_blocks < 148) return recursion_step_launches<2, 4>(g, P, step, traces, max_M, s);
+  if (row_blocks < 8 * 148) return recursion_step_launches<4, 2>(g, P, step, traces, max_M, s);
+  return recursion_step_launches<4, 1>(g, P, step, traces, max_M, s);
 }
 
 cudaError_t launch_smooth(const GroupDev& g, int max_M, cudaStream_t s) {

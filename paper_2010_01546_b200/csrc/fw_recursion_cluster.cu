@@ -79,11 +79,15 @@ __device__ __forceinline__ void cp_async16(uint32_t saddr, const float* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(g) : "memory");
 }
 
+// dynamic shared memory: [phi slab R x Mp][xi2][cvec][wvec][two power-iteration vectors][uvec][vh: KH][th: KH], vectors
+// of Mv floats: what n slices of R results fill, and at least whole trips of a warp over the columns
+extern __shared__ __align__(16) float csm[];
+
 // What a CTA knows about its layer; lives in shared memory (the threads' registers hold matrix rows).
 struct Slab {
-  float* phi;     // my rows of Phi_y in shared memory, leading dimension Mp
-  float* xi2; float* cvec; float* wvec; float* buf0; float* uvec;   // vectors of Mv floats; buf0: two, Mv apart
-  float* vh; float* th;   // v_e and t of the recorded steps, KH vectors each
+  // offsets into the dynamic shared memory (not pointers: the compiler then knows which memory they point to)
+  int xi2, cvec, wvec, buf0, uvec;   // vectors of Mv floats; buf0: two, Mv apart.  My rows of Phi_y are at 0, Mp apart
+  int vh, th;     // v_e and t of the recorded steps, KH vectors each
   int M, Mp;      // matrix size, padded row length
   int Mv;         // vector length in shared memory
   int R;          // rows per CTA, a multiple of four (rows past the matrix are zero rows)
@@ -208,7 +212,7 @@ __device__ __forceinline__ int argmax_xi(const Slab& s) {
   const int lane = threadIdx.x & 31;
   uint32_t best = 0, bi = 0;
   for (int c = lane; c < (s.Mp >> 2); c += 32) {
-    const float4 x = reinterpret_cast<const float4*>(s.xi2)[c];
+    const float4 x = reinterpret_cast<const float4*>(csm + s.xi2)[c];
 #define FW_CAND(X, o)                                                                                     \
     {                                                                                                     \
       const uint32_t k = (X) >= 0.f && 4 * c + (o) < s.M ? __float_as_uint(X) + 1u : 0u;                   \
@@ -226,7 +230,7 @@ __device__ __forceinline__ int argmax_xi(const Slab& s) {
 // rows reads the row where it is.
 __device__ __forceinline__ const float* row_exchange(Slab& s, const Link& l, int mp, uint32_t e) {
   const int owner = mp / s.R;
-  const float* row = s.phi + (size_t)(mp - owner * s.R) * s.Mp;
+  const float* row = csm + (mp - owner * s.R) * s.Mp;
   if (l.n == 1) return row;
   arm(l, e, (uint32_t)s.Mp * 4u);
   if (owner == s.sub) {
@@ -235,22 +239,22 @@ __device__ __forceinline__ const float* row_exchange(Slab& s, const Link& l, int
     for (int c = threadIdx.x >> 5; c < (s.Mp >> 2); c += l.active >> 5) {
       // a lane per peer: the lanes' copies of one float4 go out together
       const float4 v = reinterpret_cast<const float4*>(row)[c];
-      if (lane < l.n) st_async_v4(smem_u32(s.wvec + 4 * c) + l.rdelta, v, bar + l.rdelta);
+      if (lane < l.n) st_async_v4(smem_u32(csm + s.wvec + 4 * c) + l.rdelta, v, bar + l.rdelta);
     }
   }
   wait_exchange(l, e, &s.fail);
-  return s.wvec;
+  return csm + s.wvec;
 }
 
 // Weights of the coherent set into wvec (Eqs. 48-49); returns the size of the set
 __device__ __forceinline__ int align_weights(Slab& s, const Link& l, int mp) {
   if (s.maxcol) {
     rows_sync(l);                     // wvec may still be read by a slower warp
-    for (int m = threadIdx.x; m < s.Mp; m += l.active) s.wvec[m] = (m == mp) ? 1.f : 0.f;
+    for (int m = threadIdx.x; m < s.Mp; m += l.active) csm[s.wvec + m] = (m == mp) ? 1.f : 0.f;
     rows_sync(l);
     return 1;
   }
-  const float xi_mp = sqrtf(s.xi2[mp]), c_rel = s.c_rel, c_abs = s.c_abs;
+  const float xi_mp = sqrtf(csm[s.xi2 + mp]), c_rel = s.c_rel, c_abs = s.c_abs;
   int cnt = 0;
   for (int base = 0; base < s.Mp; base += l.active) {
     const int m = base + (int)threadIdx.x;
@@ -258,12 +262,12 @@ __device__ __forceinline__ int align_weights(Slab& s, const Link& l, int mp) {
     if (m < s.Mp) {
       float wv = 0.f;
       if (m < s.M) {
-        const float c = s.cvec[m];
-        const float thr = fmaxf(c_rel * xi_mp * sqrtf(s.xi2[m]), c_abs);
+        const float c = csm[s.cvec + m];
+        const float thr = fmaxf(c_rel * xi_mp * sqrtf(csm[s.xi2 + m]), c_abs);
         in = fabsf(c) >= thr;       // false for NaN
         wv = in ? (1.f / c) : 0.f;
       }
-      s.wvec[m] = wv;
+      csm[s.wvec + m] = wv;
     }
     int n;
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %1, 0;\n\tbarrier.cta.red.popc.aligned.u32 %0, 1, %2, p;\n\t}"
@@ -328,7 +332,7 @@ template <int NG, int IT, bool V4>
 __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* L, int steps, bool smooth, uint32_t e) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float4 a[4 * NG][IT];
-  float* th = s.th + s.row0 + 4 * warp;
+  float* th = csm + s.th + s.row0 + 4 * warp;
   int live = 0;
 #pragma unroll 1
   for (int k = 0; k < steps; ++k) live += s.ah[k] != 0.f ? 1 : 0;
@@ -339,7 +343,7 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
     for (int k = 0; k < steps; ++k) {
       const float ak = s.ah[k];
       if (ak == 0.f) continue;
-      const float4* v4 = reinterpret_cast<const float4*>(s.vh + k * s.Mv);
+      const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + k * s.Mv);
       float acc[4 * NG][2];
 #pragma unroll
       for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
@@ -382,7 +386,7 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
       const float ak = s.ah[k];
       if (ak == 0.f) continue;
       const float aq = ak * (ak + 2.f);
-      const float* tk = s.th + k * s.Mv;
+      const float* tk = csm + s.th + k * s.Mv;
       float ti[4 * NG];
 #pragma unroll
       for (int q = 0; q < 4 * NG; ++q) ti[q] = tk[s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3)];
@@ -443,7 +447,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
   float4 a[4 * NG][IT];
 #pragma unroll
   for (int q = 0; q < 4 * NG; ++q) {
-    const float4* r4 = reinterpret_cast<const float4*>(s.phi + (size_t)(4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp);
+    const float4* r4 = reinterpret_cast<const float4*>(csm + (4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp);
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       const int c = lane + 32 * k;
@@ -453,37 +457,37 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
   for (int step = k0; step < k1; ++step) {
     // S1: squared column norms (= row norms, Phi_y is exactly symmetric)             (Eq. 45)
     arm(l, e, tx);
-    pass<PASS_SELF, NG, IT>(a, nullptr, 1.f, l, s.xi2 + slot, e);
+    pass<PASS_SELF, NG, IT>(a, nullptr, 1.f, l, csm + s.xi2 + slot, e);
     wait_exchange(l, e, &s.fail); ++e;
     // S2: m' = argmax xi, x = row m' of Phi_y, c = Phi_y x                            (Eqs. 46-47)
     const int mp = argmax_xi(s);
     const float* row = row_exchange(s, l, mp, e); ++e;
     arm(l, e, tx);
-    pass<PASS_SCALE, NG, IT>(a, row, 1.f, l, s.cvec + slot, e);
+    pass<PASS_SCALE, NG, IT>(a, row, 1.f, l, csm + s.cvec + slot, e);
     wait_exchange(l, e, &s.fail); ++e;
     // S3: coherent set and aligned average                                          (Eqs. 48-49)
     arm(l, e, tx);
     const int cnt = align_weights(s, l, mp);
-    pass<PASS_SCALE, NG, IT>(a, s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, l, s.buf0 + slot, e);
+    pass<PASS_SCALE, NG, IT>(a, csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, l, csm + s.buf0 + slot, e);
     wait_exchange(l, e, &s.fail); ++e;
     // S4: P power iterations u = Phi_y (prev / ||prev||)
-    float* x = s.buf0;
-    float* y = x + s.Mv;
+    int xo = s.buf0, yo = xo + s.Mv;
     for (int p = 0; p < P; ++p) {
       arm(l, e, tx);
-      pass<PASS_NORM, NG, IT>(a, x, 0.f, l, y + slot, e);
+      pass<PASS_NORM, NG, IT>(a, csm + xo, 0.f, l, csm + yo + slot, e);
       wait_exchange(l, e, &s.fail); ++e;
-      float* t = x; x = y; y = t;
+      const int t = xo; xo = yo; yo = t;
     }
     // S5: v = prev/||prev|| (Eq. 50), u = Phi_y v, lambda_e = v.u (Eq. 36)
+    const float* x = csm + xo;
     arm(l, e, tx);
-    const float n2 = pass<PASS_NORM, NG, IT>(a, x, 0.f, l, s.uvec + slot, e);
+    const float n2 = pass<PASS_NORM, NG, IT>(a, x, 0.f, l, csm + s.uvec + slot, e);
     const float inv = inv_norm(n2);
-    float* vh = s.vh + (step - k0) * s.Mv;
+    float* vh = csm + s.vh + (step - k0) * s.Mv;
     wait_exchange(l, e, &s.fail); ++e;
     float l0 = 0.f, l1 = 0.f;
     const float4* x4 = reinterpret_cast<const float4*>(x);
-    const float4* u4 = reinterpret_cast<const float4*>(s.uvec);
+    const float4* u4 = reinterpret_cast<const float4*>(csm + s.uvec);
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       const float4 xv = x4[lane + 32 * k], uv = u4[lane + 32 * k];
@@ -510,7 +514,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
       for (int q = 0; q < 4 * NG; ++q) {
         const int i = slot + 4 * CW * (q >> 2) + (q & 3);
         vi[q] = x[i] * inv;
-        wi[q] = __fadd_rn(__fmul_rn(aa, s.uvec[i]), __fmul_rn(hl, vi[q]));
+        wi[q] = __fadd_rn(__fmul_rn(aa, csm[s.uvec + i]), __fmul_rn(hl, vi[q]));
       }
 #pragma unroll
       for (int k = 0; k < IT; ++k) {
@@ -526,7 +530,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
           a[q][k].z = __fadd_rn(a[q][k].z, __fadd_rn(__fmul_rn(vi[q], wj.z), __fmul_rn(wi[q], vj.z)));
           a[q][k].w = __fadd_rn(a[q][k].w, __fadd_rn(__fmul_rn(vi[q], wj.w), __fmul_rn(wi[q], vj.w)));
           if (c < (s.Mp >> 2))
-            reinterpret_cast<float4*>(s.phi + (size_t)(4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp)[c] = a[q][k];
+            reinterpret_cast<float4*>(csm + (4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp)[c] = a[q][k];
         }
       }
     }
@@ -553,10 +557,6 @@ __device__ __forceinline__ int warp_groups(int R) {
   const int warp = threadIdx.x >> 5, ng = R >> 2;
   return ng > warp ? (ng - warp + CW - 1) / CW : 0;
 }
-
-// dynamic shared memory: [phi slab R x Mp][xi2][cvec][wvec][two power-iteration vectors][uvec][vh: KH][th: KH], vectors
-// of Mv floats: what n slices of R results fill, and at least whole trips of a warp over the columns
-extern __shared__ __align__(16) float csm[];
 
 __host__ __device__ inline int slab_rows(int M, int n) { return (((M + n - 1) / n) + 3) & ~3; }
 __host__ __device__ inline int slab_trips(int M) { return (((M + 3) >> 2) + 31) / 32; }
@@ -603,8 +603,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     s.sub = (int)blockIdx.x - a.first_cta[layer];
     s.row0 = s.sub * s.R;
     s.nrows = max(0, min(s.R, M - s.row0));
-    s.phi = csm;
-    s.xi2 = csm + (size_t)s.R * s.Mp;
+    s.xi2 = s.R * s.Mp;
     s.cvec = s.xi2 + s.Mv; s.wvec = s.cvec + s.Mv; s.buf0 = s.wvec + s.Mv; s.uvec = s.buf0 + 2 * s.Mv;
     s.vh = s.uvec + s.Mv; s.th = s.vh + KH * s.Mv;
     s.tx = (uint32_t)n * (uint32_t)s.R * 4u;
@@ -636,13 +635,13 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
       csm[i] = (c < M && r < nrows) ? L->Phiy[(size_t)(s.row0 + r) * M + c] : 0.f;
     }
   }
-  for (int i = threadIdx.x; i < kVecs * s.Mv; i += CT) s.xi2[i] = 0.f;
+  for (int i = threadIdx.x; i < kVecs * s.Mv; i += CT) csm[s.xi2 + i] = 0.f;
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
   // A CTA's window of the cluster address space is this CTA's window shifted by a constant; the stores rely on it,
   // so it is checked on two addresses far apart before anything is sent.
   const uint32_t peer_rank = (uint32_t)(rank - s.sub + min(lane, l.n - 1));
   l.rdelta = map_cluster(l.bar0, peer_rank) - l.bar0;
-  const bool linear = (map_cluster(smem_u32(s.th), peer_rank) - smem_u32(s.th)) == l.rdelta;
+  const bool linear = (map_cluster(smem_u32(csm + s.th), peer_rank) - smem_u32(csm + s.th)) == l.rdelta;
   const bool usable = __syncthreads_or(!linear) == 0;
   cluster.sync();   // every barrier is initialised before the first remote store can arrive
 
@@ -676,7 +675,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     if (threadIdx.x == 0) L->iscal[IS_STATUS_TIMEOUT] = 1;
   } else {
     if (s.sub == 0 && !s.maxcol)
-      for (int m = threadIdx.x; m < M; m += CT) L->wvec[m] = s.wvec[m];    // alignment weights of the last step
+      for (int m = threadIdx.x; m < M; m += CT) L->wvec[m] = csm[s.wvec + m];    // alignment weights of the last step
     if ((M & 3) == 0) {
       float4* dst = reinterpret_cast<float4*>(L->Phiy + (size_t)s.row0 * M);
       for (int i = threadIdx.x; i < nrows * (M >> 2); i += CT) dst[i] = reinterpret_cast<const float4*>(csm)[i];

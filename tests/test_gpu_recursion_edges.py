@@ -71,3 +71,42 @@ def test_groups(env, dims):
     group_reduce_with_replay(Ls, Los, 2, 4, B, torch)
     for L, Lo in zip(Ls, Los):
         check(L, Lo, B)
+
+
+# ---- layers past the on-chip kernel: teams of CTAs, rows in shared memory or (4001) partly streamed ----
+@pytest.mark.parametrize("M,K", [(625, 18), (626, 2), (900, 2), (1153, 2), (1284, 2), (4001, 1)])
+def test_team_edges(env, M, K):
+    torch, B = env
+    Phi = spd32(M, 1e2, 900 + M)
+    La, Lb = B.Layer(M, 4, beta=0.2, gamma=1.0), B.Layer(M, 4, beta=0.2, gamma=1.0)
+    Lo = O.Layer(M, 4, oracle_hyper(La.desc))
+    for L in (La, Lb):
+        L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda())
+    Lo.set_phix(Phi)
+    reduce_with_replay(La, Lo, min(K, 2), 3, B, torch)
+    check(La, Lo, B)
+    for _ in range(K - 2):
+        La.cond_reduce(1, 3)
+    Lb.cond_reduce(K, 3)                     # 18 steps: T and Q take them in batches of 16 and 2
+    for f in (B.FW_F_T, B.FW_F_Q, B.FW_F_PHIY, B.FW_F_ALIGN_W):
+        assert torch.equal(La.get(f), Lb.get(f))
+    assert La.sync_status() == B.FW_OK
+
+
+def test_team_waves(env):
+    torch, B = env
+    dims = [1152] * 7 + [700, 640, 2048, 2048, 100]      # more rows than the chip holds at once, and an on-chip layer
+    Ls = []
+    for i, M in enumerate(dims):
+        L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+        L.set(B.FW_F_PHIX, torch.from_numpy(spd32(M, 1e2, 40 + i)).cuda())
+        Ls.append(L)
+    for _ in range(2):
+        B.fw_group_cond_reduce([L.handle for L in Ls], 2, 4)
+    for i in (0, 6, 7, 8, 10, 11):
+        L = B.Layer(dims[i], 4, beta=0.0, gamma=1.0)
+        L.set(B.FW_F_PHIX, torch.from_numpy(spd32(dims[i], 1e2, 40 + i)).cuda())
+        L.cond_reduce(2, 4)
+        L.cond_reduce(2, 4)
+        assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), t2n(L.get(B.FW_F_T))) <= TOL_FP32
+        assert Ls[i].sync_status() == B.FW_OK
