@@ -208,8 +208,8 @@ fw_status fw_step_momentum(fw_layer* L, float* W, float* b, const float* G_t, co
 
 /* Whitening from the eigenvalue decomposition (Sec. 2, Eqs. 7-10; Sec. 3.2,
  * Eqs. 32, 34, 35): the direct construction the recursion of Sec. 4 replaces.
- * Phi_x = V Lambda V^T is computed on the device (one-sided Jacobi rotations in
- * fp64, all layers of a group in one cooperative launch) and the layer's state is
+ * Phi_x = V Lambda V^T is computed on the device (one-sided block Jacobi rotations
+ * in fp64, all layers of a group in one cooperative launch) and the layer's state is
  * set to  T = V diag(sqrt g) V^T (the symmetric, "ZCA" whitening matrix, Eq. 9),
  * Q = T^T T, Phi_y = T Phi_x T^T, Qs <- beta Qs + (1 - beta) Q (Eq. 35), with gains
  *   g_max <= 0:  g_m = 1 / max(lambda_m, eps)                            (Eq. 10)
@@ -221,9 +221,9 @@ fw_status fw_step_momentum(fw_layer* L, float* W, float* b, const float* G_t, co
  * The gradient transform, the step and a later fw_cond_reduce continue from this
  * state.  scratch: caller-owned device memory, 256-byte aligned, at least
  * fw_evd_scratch_bytes(M) bytes per layer, used only during the call's kernels.
- * Cost: about 12 M^3 fp64 operations per sweep and 6-10 sweeps; M - 1 grid
- * barriers per sweep (bounded waits; a time-out is reported by
- * fw_layer_sync_status as FW_ERR_TIMEOUT).  Errors: FW_ERR_STATE without a
+ * Cost: about 5 M^3 fp64 operations per sweep and 9-13 sweeps; M / 16 - 1
+ * barriers of the layer's CTAs per sweep (bounded waits; a time-out is reported
+ * by fw_layer_sync_status as FW_ERR_TIMEOUT).  Errors: FW_ERR_STATE without a
  * covariance or inside an open block, FW_ERR_WORKSPACE for a short scratch. */
 size_t fw_evd_scratch_bytes(int32_t M);
 fw_status fw_evd_whiten(fw_layer* L, void* scratch, size_t scratch_bytes, float g_max);

@@ -1,44 +1,64 @@
 // Whitening from the eigenvalue decomposition (Sec. 2, Eqs. 7-10; practical gains Eqs. 32 and 34): the method the
-// recursion of Sec. 4 is measured against.  Phi = V Lambda V^T is computed by one-sided Jacobi rotations in fp64:
-// with W = Phi V (starting from W = Phi, V = I), the rotation of a pair of columns (p, q) that makes w_p, w_q
-// orthogonal is applied to W and V alike; when all columns of W are orthogonal, V holds the eigenvectors and
-// lambda_m = v_m . w_m.  A pair touches nothing but its own two columns, so the M / 2 disjoint pairs of a round
-// (round-robin tournament: M - 1 rounds cover every pair once) run on different warps with one grid barrier per
-// round, all layers of a group in the same launch.  Columns are stored as rows (Phi is symmetric), fp64 throughout:
-// T = Phi^(-1/2) carries the rounding of the decomposition times cond(Phi) / 2, which fp32 cannot afford.
+// recursion of Sec. 4 is measured against.  Phi = V Lambda V^T is computed by one-sided block Jacobi rotations in fp64:
+// the columns of W, starting from W = Phi, are rotated until all are orthogonal; then W = Phi V = V Lambda, so the
+// normalised columns of W are the eigenvectors and their lengths the eigenvalues, and V itself is never carried along.
+// Columns are stored as rows (Phi is symmetric), fp64 throughout: T = Phi^(-1/2) carries the rounding of the
+// decomposition times cond(Phi) / 2, which fp32 cannot afford.
+//
+// A CTA takes a pair of blocks of 16 columns: the 32 columns' Gram matrix (tensor-core fp64 products, the columns staged
+// in shared memory), one sweep of 2 x 2 rotations on that 32 x 32 matrix in shared memory, accumulated into U, and
+// W <- U^T W on the 32 rows.  The block pairs of a round (round-robin tournament) are disjoint, so a layer's CTAs meet
+// once per round, M / 16 - 1 rounds a sweep, instead of once per round of column pairs (M - 1 rounds).  All layers of a
+// group share the launch, each with CTAs and barriers of its own.  A sweep costs 5 / 2 M^3 multiply-adds; what bounds a
+// round at M = 576 (about 19 us) is the chain products - 31 inner rounds - products - barrier, a third each.
 //
 // Then T = V diag(sqrt g) V^T (Eq. 9), Q = T^T T = V diag(g) V^T and Phi_y = T Phi T^T = V diag(g lambda) V^T come
 // out of one pass over V.
+#include <algorithm>
 #include <cstring>
 
 #include "fw_internal.h"
+#include "fw_sm100.cuh"
 
 namespace fw {
 namespace {
 
-constexpr int ET = 512;               // threads per CTA of the rotation kernel: a warp per pair
-constexpr int kRegCols = 20;          // columns per lane held in registers: rows of up to 640 entries are read once
+constexpr int ET = 512;               // threads per CTA of the rotation kernel
 constexpr int EW = ET / 32;
+constexpr int EB = 16;                // columns per block
+constexpr int EP = 2 * EB;            // columns of a block pair
+constexpr int kChunk = 640;           // entries of a column staged at a time (rows of up to this length stay for both products)
 constexpr int kMaxSweeps = 30;
 constexpr uint32_t kEvdSpin = 1u << 22;
+constexpr int kSlots = 64;            // of kWords 4-byte words at the start of a layer's scratch
+constexpr int kWords = 256;
 constexpr double kOrthTol = 1e-14;    // |w_p . w_q| <= tol |w_p| |w_q|: the pair is left alone
+// Below kFloor max_i Phi_ii a column is rounding (lambda_max is at least that diagonal entry): repeated features, for one,
+// leave columns that are parallel to another one at any length.  Such columns are not rotated, and eigenvalues below
+// kNull lambda_max have no direction of their own: together they span what the other eigenvectors leave.
+constexpr double kFloor = 1e-14, kNull = 1e-13;
+
+// shared-memory row stride in doubles: 4 mod 16, so that the fragments of both products read without conflicts
+__host__ __device__ inline int evd_stride(int cols) { return ((cols + 15) & ~15) + 4; }
+__host__ __device__ inline int evd_ld(int M) { return (M + 7) & ~7; }
+constexpr int kGLd = EP + 1;          // leading dimension of the 32 x 32 matrices in shared memory
+constexpr int kTri = 10;              // 8 x 8 blocks of the upper triangle of a 32 x 32 matrix
+constexpr int kPartDoubles = EW / 2 * kTri * 64;
 
 struct EvdLayer {
   const float* A;    // M x M symmetric input (fp32, row-major)
-  double* W;         // M x M: row m is column m of Phi V
-  double* V;         // M x M: row m is eigenvector m (null: eigenvalues only)
+  double* W;         // M rows of evd_ld(M): row m is column m of Phi V
+  int32_t* words;    // [1] abort, [2 + s] block pairs rotated in sweep s, [kSlots + c] rounds CTA c has finished (zeroed
+                     // before the launch)
   int32_t* status;   // time-out word of the layer
   int32_t M;
-  int32_t n;         // players of the tournament: M rounded up to even (an odd M plays against a dummy)
+  int32_t nb;        // blocks of 16 columns, rounded up to even (the tournament's players)
+  int32_t cta0, n;   // its CTAs
 };
 
 struct EvdArgs {
   EvdLayer l[FW_MAX_GROUP];
-  int32_t pair0[FW_MAX_GROUP + 1];   // first pair of each layer in the flat list of a round (n / 2 pairs per layer)
   int32_t nl;
-  int32_t rounds_max;                // n_max - 1
-  int32_t nctas;
-  int32_t* bar;                      // [0] arrivals, [1] abort, [2 + s] rotations of sweep s (zeroed before the launch)
 };
 
 __device__ __forceinline__ double warp_sum_d(double x) {
@@ -47,24 +67,45 @@ __device__ __forceinline__ double warp_sum_d(double x) {
   return x;
 }
 
-// Grid barrier number idx (from 1) of this launch; false once the launch is aborted.  The wait is bounded.
-__device__ bool evd_grid_barrier(const EvdArgs& a, uint32_t idx, int* s_abort) {
+// maximum over the block of values that are not negative
+__device__ double evd_block_max(float x) {
+  __shared__ uint32_t m;
+  if (threadIdx.x == 0) m = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile int* ctr = a.bar;
-    volatile int* ab = a.bar + 1;
-    if (*s_abort == 0) {
+  atomicMax(&m, __float_as_uint(x));
+  __syncthreads();
+  const double r = (double)__uint_as_float(m);
+  __syncthreads();
+  return r;
+}
+
+// D (8 x 8) += A (8 x 4) B (4 x 8): lane holds A[lane / 4][lane % 4], B[lane % 4][lane / 4], D[lane / 4][2 (lane % 4) + {0, 1}]
+__device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
+  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+}
+
+// Barrier number idx (from 1) of a layer's CTAs; false once the layer is aborted.  Every CTA raises its own slot and the
+// first warp polls all of them: no chain of atomic additions.  The wait is bounded.
+__device__ bool evd_barrier(const EvdLayer& L, int sub, int idx, int* s_abort) {
+  __syncthreads();
+  if (threadIdx.x < 32 && *s_abort == 0) {
+    volatile int* slots = L.words + kSlots;
+    volatile int* ab = L.words + 1;
+    if (threadIdx.x == 0) {
       __threadfence();
-      atomicAdd(a.bar, 1);
-      const uint32_t target = idx * (uint32_t)a.nctas;
-      bool ok = false;
-      for (uint32_t i = 0; i < kEvdSpin; ++i) {
-        if ((int32_t)((uint32_t)*ctr - target) >= 0) { ok = true; break; }
-        if ((i & 63u) == 63u && *ab != 0) break;
-      }
+      slots[sub] = idx;
+    }
+    bool ok = false;
+    for (uint32_t i = 0; i < kEvdSpin && !ok; ++i) {
+      bool here = true;
+      for (int c = threadIdx.x; c < L.n; c += 32) here = here && slots[c] >= idx;
+      ok = __all_sync(0xffffffffu, here);
+      if (!ok && (i & 63u) == 63u && *ab != 0) break;
+    }
+    if (threadIdx.x == 0) {
       if (!ok) {
         *ab = 1;
-        for (int i = 0; i < a.nl; ++i) atomicExch(a.l[i].status, 601);
+        atomicExch(L.status, 601);
         *s_abort = 1;
       }
       __threadfence();
@@ -74,202 +115,400 @@ __device__ bool evd_grid_barrier(const EvdArgs& a, uint32_t idx, int* s_abort) {
   return *s_abort == 0;
 }
 
-__global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
-  __shared__ int s_abort;
-  __shared__ int s_rot;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = (int)blockIdx.x * EW + warp, nw = (int)gridDim.x * EW;
-  if (threadIdx.x == 0) { s_abort = 0; s_rot = 0; }
-  __syncthreads();
-  // W = Phi, V = I
-  for (int li = 0; li < a.nl; ++li) {
-    const EvdLayer L = a.l[li];
-    const int64_t mm = (int64_t)L.M * L.M;
-    for (int64_t i = (int64_t)blockIdx.x * ET + threadIdx.x; i < mm; i += (int64_t)gridDim.x * ET) {
-      L.W[i] = (double)L.A[i];
-      if (L.V) L.V[i] = (i / L.M == i % L.M) ? 1.0 : 0.0;
+// A wait for copies gave up: report, and let the layer's other CTAs leave at their next barrier.
+__device__ void evd_give_up(const EvdLayer& L) {
+  if (threadIdx.x == 0) {
+    atomicExch(L.status, 601);
+    *(volatile int*)(L.words + 1) = 1;
+  }
+}
+
+// players of pair k in round q of the tournament of 32
+__device__ __forceinline__ void evd_players(int k, int q, int& p, int& r) {
+  p = q + k; r = q - k;
+  if (p >= EP - 1) p -= EP - 1;
+  if (r < 0) r += EP - 1;
+  if (k == 0) p = EP - 1;
+}
+
+// dynamic shared memory: [32 rows of a chunk][partial Gram blocks of the warps, later the second Gram buffer and U][Gram]
+extern __shared__ __align__(16) double esm[];
+
+// Rows of the block pair (I, J): row r of the pair is column I * 16 + r or J * 16 + r - 16 of the layer.
+__device__ __forceinline__ int pair_row(int I, int J, int r) { return r < EB ? I * EB + r : J * EB + r - EB; }
+
+// Entries [k0, k0 + nk) of the pair's rows into shared memory, one bulk copy per row; rows past the matrix and entries
+// past ld are zero.  parity: of the copies' mbarrier.  Returns false when the bounded wait gave up.
+__device__ __forceinline__ bool stage_rows(const EvdLayer& L, int I, int J, int k0, int nk, int stride, uint32_t bar,
+                                           uint32_t parity) {
+  const int ld = evd_ld(L.M), have = min(nk, ld - k0);
+  const int rows = max(0, min(EB, L.M - I * EB)) + max(0, min(EB, L.M - J * EB));
+  const int tid = threadIdx.x;
+  if (tid < 32) {
+    asm volatile("fence.proxy.async;" ::: "memory");       // the rows were last written and read by ordinary accesses
+    if (tid == 0) sm100::mbar_expect_tx(bar, (uint32_t)rows * (uint32_t)have * 8u);
+    __syncwarp();
+    const int row = pair_row(I, J, tid);
+    if (row < L.M)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(sm100::smem_u32(esm + tid * stride)), "l"(L.W + (int64_t)row * ld + k0), "r"((uint32_t)have * 8u), "r"(bar)
+                   : "memory");
+  }
+  if (rows < EP || have < nk) {
+    for (int i = tid; i < EP * nk; i += ET) {
+      const int r = i / nk, c = i - r * nk;
+      if (pair_row(I, J, r) >= L.M || c >= have) esm[r * stride + c] = 0.0;
     }
   }
-  uint32_t bidx = 0;
-  if (!evd_grid_barrier(a, ++bidx, &s_abort)) return;
-  const int npairs = a.pair0[a.nl];
-  for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
-    for (int r = 0; r < a.rounds_max; ++r) {
-      bool rotated = false;
-      for (int t = gw; t < npairs; t += nw) {
-        int li = 0;
+  bool ok = false;
+  for (uint32_t i = 0; i < sm100::kSpinLimit && !ok; ++i) ok = sm100::mbar_try_wait(bar, parity);
+  return __syncthreads_and(ok) != 0;
+}
+
+// x 2^(127 - e) as fp32, truncated, for e the (biased) fp64 exponent of a number at least as large; 0 when too small
+__device__ __forceinline__ float to_float_scaled(double x, int e) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = ((hi >> 20) & 0x7ff) - e + 127;
+  const uint32_t bits = (uint32_t)(hi & 0x80000000) | ((uint32_t)ex << 23) | (__funnelshift_l((uint32_t)lo, (uint32_t)hi, 3) & 0x007fffffu);
+  return ex > 0 ? __uint_as_float(bits) : 0.f;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The rotation (c, s) that makes columns p, q orthogonal, from their Gram entries (the smaller of the two angles phi,
+// tan 2 phi = 2 ga / (be - al)); (1, 0) when they are already.  The tangent h of half the angle comes from fp32
+// arithmetic (what the angle misses, 1e-7 of the product, the next sweep sees); c = 2 / (1 + h^2) - 1 and
+// s = 2 h / (1 + h^2), with the reciprocal refined to fp64 rounding, are orthonormal whatever h is.  floor2: squared length of a null column.  This is the chain
+// of an inner round: ten dependent fp64 operations with the 2 x 2 update, no fp64 division or root.
+__device__ __forceinline__ void rotation(double al, double be, double ga, double floor2, double& c, double& s) {
+  const bool act = ga * ga > kOrthTol * kOrthTol * (al * be) && fmin(al, be) > floor2;
+  const double d = be - al;
+  const int e = max((__double2hiint(d) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
+  const float df = fabsf(to_float_scaled(d, e)), gf = to_float_scaled(ga, e);
+  const float g2 = gf + gf;
+  const float ir = rsqrt_approx(fmaf(df, df, g2 * g2));          // 1 / R
+  const float c2 = fmaf(0.5f * df, ir, 0.5f);                    // cos^2 phi
+  const float ic = rsqrt_approx(c2);
+  const float cf = c2 * ic, sf = gf * ir * ic;                   // cos phi, sin phi (up to sign)
+  float h = sf * rcp_approx(1.f + cf);
+  if (d < 0.0) h = -h;
+  if (!act) h = 0.f;
+  const double hd = (double)h, x = fma(hd, hd, 1.0);
+  const double r0 = (double)rcp_approx(fmaf(h, h, 1.f));
+  const double q = fma(-x, r0, 1.0);
+  const double r = fma(r0, fma(q, q, q), r0);
+  c = fma(2.0, r, -1.0);
+  s = (hd + hd) * r;
+}
+
+__global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
+  __shared__ int s_abort;
+  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ double s_rot[2][EB][2];                              // (c, s) of the 16 pairs of an inner round
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int li = -1;
 #pragma unroll 1
-        for (int i = 1; i < a.nl; ++i)
-          if (t >= a.pair0[i]) li = i;
-        const EvdLayer L = a.l[li];
-        const int n1 = L.n - 1;
-        if (r >= n1) continue;                      // this layer's sweep has fewer rounds
-        const int k = t - a.pair0[li];
-        int p, q;
-        if (k == 0) { p = n1; q = r; }
-        else { p = (r + k) % n1; q = (r - k + n1) % n1; }
-        if (p > q) { const int x = p; p = q; q = x; }
-        if (q >= L.M) continue;                     // the dummy player of an odd M
-        const int M = L.M;
-        double* wp = L.W + (int64_t)p * M;
-        double* wq = L.W + (int64_t)q * M;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        const bool in_regs = M <= 32 * kRegCols;
-        double xr[kRegCols], yr[kRegCols];
-        if (in_regs) {
-          // every load of the two rows is in flight at once, and the rotation needs no second read
+  for (int i = 0; i < a.nl; ++i)
+    if ((int)blockIdx.x >= a.l[i].cta0 && (int)blockIdx.x < a.l[i].cta0 + a.l[i].n) li = i;
+  if (li < 0) return;
+  const EvdLayer L = a.l[li];
+  const int M = L.M, ld = evd_ld(M), sub = (int)blockIdx.x - L.cta0;
+  const uint32_t bar = sm100::smem_u32(&s_bar);
+  uint32_t parity = 0;
+  if (tid == 0) {
+    s_abort = 0;
+    sm100::mbar_init(bar, 1);
+    sm100::mbar_fence_init();
+  }
+  float dmax = 0.f;
+  for (int i = tid; i < M; i += ET) dmax = fmaxf(dmax, fabsf(L.A[(int64_t)i * M + i]));
+  const double floor1 = kFloor * evd_block_max(dmax), floor2 = floor1 * floor1;
+  // W = Phi, padded with zeros to whole rows of ld
+  for (int64_t i = (int64_t)sub * ET + tid; i < (int64_t)M * ld; i += (int64_t)L.n * ET) {
+    const int r = (int)(i / ld), c = (int)(i - (int64_t)r * ld);
+    __stcg(L.W + i, c < M ? (double)L.A[(int64_t)r * M + c] : 0.0);
+  }
+  const int chunks = (ld + kChunk - 1) / kChunk;
+  const int nk = chunks == 1 ? ld : kChunk;                       // entries per chunk
+  const int stride = evd_stride(nk);
+  double* part = esm + EP * stride;                               // kPartDoubles
+  double* G0 = part + kPartDoubles;
+  double* G1 = part;                                              // these two reuse the partial blocks
+  double* U = part + EP * kGLd;
+  int bidx = 0;
+  if (!evd_barrier(L, sub, ++bidx, &s_abort)) return;
+  const int np = L.nb / 2, n1 = L.nb - 1;
+  for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+    bool rotated = false;
+    for (int r = 0; r < n1; ++r) {
+      for (int k = sub; k < np; k += L.n) {
+        int I, J;
+        if (k == 0) { I = n1; J = r; }
+        else { I = (r + k) % n1; J = (r - k + n1) % n1; }
+        if (I > J) { const int x = I; I = J; J = x; }
+        if (I * EB >= M) continue;                                // both blocks past the matrix
+        // ---- G = (rows)(rows)^T: each warp an eighth of the entries, all ten blocks of the upper triangle ----
+        double acc[kTri][2];
 #pragma unroll
-          for (int j = 0; j < kRegCols; ++j) {
-            const int i = lane + 32 * j;
-            xr[j] = i < M ? __ldcg(wp + i) : 0.0;
-            yr[j] = i < M ? __ldcg(wq + i) : 0.0;
-          }
+        for (int b = 0; b < kTri; ++b) acc[b][0] = acc[b][1] = 0.0;
+        for (int ch = 0; ch < chunks; ++ch) {
+          if (ch) __syncthreads();                                // the chunk before has been read
+          if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) { evd_give_up(L); return; }
+          parity ^= 1;
+          const double* w = esm + (lane >> 2) * stride + (lane & 3);
+#pragma unroll 2
+          for (int st = warp; st < nk / 4; st += EW) {
+            double f[4];
 #pragma unroll
-          for (int j = 0; j < kRegCols; ++j) {
-            al = fma(xr[j], xr[j], al); be = fma(yr[j], yr[j], be); ga = fma(xr[j], yr[j], ga);
-          }
-        } else {
-          for (int i = lane; i < M; i += 32) {
-            const double x = __ldcg(wp + i), y = __ldcg(wq + i);
-            al = fma(x, x, al); be = fma(y, y, be); ga = fma(x, y, ga);
+            for (int b = 0; b < 4; ++b) f[b] = w[8 * b * stride + 4 * st];
+            int t = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+#pragma unroll
+              for (int c = b; c < 4; ++c) mma_f64(acc[t++], f[b], f[c]);
           }
         }
-        al = warp_sum_d(al); be = warp_sum_d(be); ga = warp_sum_d(ga);
-        if (!(fabs(ga) > kOrthTol * sqrt(al * be))) continue;
+        // the second half of the warps hand their sums to the first half, which add to them
+        if (warp >= EW / 2) {
+#pragma unroll
+          for (int b = 0; b < kTri; ++b)
+            *reinterpret_cast<double2*>(part + ((warp - EW / 2) * kTri + b) * 64 + 2 * lane) = make_double2(acc[b][0], acc[b][1]);
+        }
+        __syncthreads();
+        if (warp < EW / 2) {
+#pragma unroll
+          for (int b = 0; b < kTri; ++b) {
+            double2* q = reinterpret_cast<double2*>(part + (warp * kTri + b) * 64 + 2 * lane);
+            const double2 o = *q;
+            *q = make_double2(acc[b][0] + o.x, acc[b][1] + o.y);
+          }
+        }
+        __syncthreads();
+        for (int i = tid; i < kTri * 64; i += ET) {
+          double x = 0.0;
+#pragma unroll
+          for (int w = 0; w < EW / 2; ++w) x += part[w * kTri * 64 + i];
+          const int b = i >> 6, e = i & 63;
+          const int rb = b < 4 ? 0 : (b < 7 ? 1 : (b < 9 ? 2 : 3)), cb = b - (b < 4 ? 0 : (b < 7 ? 3 : (b < 9 ? 5 : 6)));
+          const int gi = 8 * rb + (e >> 3), gj = 8 * cb + (e & 7);
+          if (rb != cb || gj >= gi) { G0[gi * kGLd + gj] = x; G0[gj * kGLd + gi] = x; }
+        }
+        __syncthreads();
+        // ---- anything to rotate? ----
+        bool act = false;
+        for (int i = tid; i < EP * EP; i += ET) {
+          const int p = i >> 5, q = i & 31;
+          if (p < q) {
+            const double g = G0[p * kGLd + q];
+            const double gp = G0[p * kGLd + p], gq = G0[q * kGLd + q];
+            act |= g * g > kOrthTol * kOrthTol * (gp * gq) && fmin(gp, gq) > floor2;
+          }
+          U[p * kGLd + q] = p == q ? 1.0 : 0.0;
+        }
+        if (!__syncthreads_or(act)) continue;
         rotated = true;
-        // the rotation that makes the two columns orthogonal (the smaller of the two angles)
-        const double zeta = (be - al) / (2.0 * ga);
-        const double tt = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + tt * tt), s = c * tt;
-        if (in_regs) {
+        // ---- one sweep of 2 x 2 rotations on G: a thread of the first half owns the 2 x 2 block of pairs (a, b); the
+        //      other half applies each round's rotations to U one round later, off the chain ----
+        {
+          const int pb = tid & 15, pa = (tid & 255) >> 4;
+          const bool on_g = tid < 256;
+          double* src = G0;
+          double* dst = G1;
+          for (int q = 0; q < EP; ++q) {
+            if (on_g) {
+              if (q < EP - 1) {
+                int ip, iq, jp, jq;
+                evd_players(pa, q, ip, iq);
+                evd_players(pb, q, jp, jq);
+                double cb, sb;
+                rotation(src[jp * kGLd + jp], src[jq * kGLd + jq], src[jp * kGLd + jq], floor2, cb, sb);
+                const double ca = __shfl_sync(0xffffffffu, cb, pa), sa = __shfl_sync(0xffffffffu, sb, pa);
+                if (pa == 0) { s_rot[q & 1][pb][0] = cb; s_rot[q & 1][pb][1] = sb; }
+                const double g00 = src[ip * kGLd + jp], g01 = src[ip * kGLd + jq], g10 = src[iq * kGLd + jp], g11 = src[iq * kGLd + jq];
+                const double h00 = cb * g00 - sb * g01, h01 = sb * g00 + cb * g01;
+                const double h10 = cb * g10 - sb * g11, h11 = sb * g10 + cb * g11;
+                dst[ip * kGLd + jp] = ca * h00 - sa * h10; dst[ip * kGLd + jq] = ca * h01 - sa * h11;
+                dst[iq * kGLd + jp] = sa * h00 + ca * h10; dst[iq * kGLd + jq] = sa * h01 + ca * h11;
+                double* z = src; src = dst; dst = z;
+              }
+            } else if (q > 0) {
+              int jp, jq;
+              evd_players(pb, q - 1, jp, jq);
+              const double cb = s_rot[(q - 1) & 1][pb][0], sb = s_rot[(q - 1) & 1][pb][1];
 #pragma unroll
-          for (int j = 0; j < kRegCols; ++j) {
-            const int i = lane + 32 * j;
-            if (i < M) {
-              __stcg(wp + i, c * xr[j] - s * yr[j]);
-              __stcg(wq + i, s * xr[j] + c * yr[j]);
-            }
-          }
-        } else {
-          for (int i = lane; i < M; i += 32) {
-            const double x = __ldcg(wp + i), y = __ldcg(wq + i);
-            __stcg(wp + i, c * x - s * y);
-            __stcg(wq + i, s * x + c * y);
-          }
-        }
-        if (L.V) {
-          double* vp = L.V + (int64_t)p * M;
-          double* vq = L.V + (int64_t)q * M;
-          if (in_regs) {
-#pragma unroll
-            for (int j = 0; j < kRegCols; ++j) {
-              const int i = lane + 32 * j;
-              xr[j] = i < M ? __ldcg(vp + i) : 0.0;
-              yr[j] = i < M ? __ldcg(vq + i) : 0.0;
-            }
-#pragma unroll
-            for (int j = 0; j < kRegCols; ++j) {
-              const int i = lane + 32 * j;
-              if (i < M) {
-                __stcg(vp + i, c * xr[j] - s * yr[j]);
-                __stcg(vq + i, s * xr[j] + c * yr[j]);
+              for (int h = 0; h < 2; ++h) {
+                double* u = U + (pa + 16 * h) * kGLd;
+                const double x = u[jp], y = u[jq];
+                u[jp] = cb * x - sb * y; u[jq] = sb * x + cb * y;
               }
             }
-          } else {
-            for (int i = lane; i < M; i += 32) {
-              const double x = __ldcg(vp + i), y = __ldcg(vq + i);
-              __stcg(vp + i, c * x - s * y);
-              __stcg(vq + i, s * x + c * y);
+            __syncthreads();
+          }
+        }
+        // ---- rows <- U^T rows, in place chunk by chunk (a single chunk is still staged) ----
+        // the first half of the warps computes the first 16 rows, the second half the others
+        double uf[2][8];
+        const int half = warp / (EW / 2), wcol = warp - half * (EW / 2);
+#pragma unroll
+        for (int cb = 0; cb < 2; ++cb)
+#pragma unroll
+          for (int kb = 0; kb < 8; ++kb) uf[cb][kb] = U[(4 * kb + (lane & 3)) * kGLd + 16 * half + 8 * cb + (lane >> 2)];
+        for (int ch = 0; ch < chunks; ++ch) {
+          if (chunks > 1) {
+            __syncthreads();
+            if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) { evd_give_up(L); return; }
+            parity ^= 1;
+          }
+#pragma unroll 2
+          for (int b = wcol; b < nk / 8; b += EW / 2) {
+            double bf[8];
+#pragma unroll
+            for (int kb = 0; kb < 8; ++kb) bf[kb] = esm[(4 * kb + (lane & 3)) * stride + 8 * b + (lane >> 2)];
+            const int col = ch * kChunk + 8 * b + 2 * (lane & 3);
+#pragma unroll
+            for (int cb = 0; cb < 2; ++cb) {
+              double d[2] = {0.0, 0.0};
+#pragma unroll
+              for (int kb = 0; kb < 8; ++kb) mma_f64(d, uf[cb][kb], bf[kb]);
+              const int row = pair_row(I, J, 16 * half + 8 * cb + (lane >> 2));
+              if (row < M && col < ld) __stcg(reinterpret_cast<double2*>(L.W + (int64_t)row * ld + col), make_double2(d[0], d[1]));
             }
           }
         }
+        __syncthreads();                                          // the staged rows are free for the next pair
       }
-      if (rotated && lane == 0) s_rot = 1;
       // the sweep's count of rotations is complete before its last barrier
-      if (r == a.rounds_max - 1) {
-        __syncthreads();
-        if (threadIdx.x == 0 && s_rot) { atomicAdd(a.bar + 2 + sweep, 1); s_rot = 0; }
-      }
-      if (!evd_grid_barrier(a, ++bidx, &s_abort)) return;
+      if (r == n1 - 1 && tid == 0 && rotated) atomicAdd(L.words + 2 + sweep, 1);
+      if (!evd_barrier(L, sub, ++bidx, &s_abort)) return;
     }
-    if (__ldcg(a.bar + 2 + sweep) == 0) break;      // every pair of every layer was already orthogonal
+    if (__ldcg(L.words + 2 + sweep) == 0) break;                  // every pair was already orthogonal
   }
 }
 
 struct FinishArgs {
   EvdLayer l[FW_MAX_GROUP];
-  double* lam[FW_MAX_GROUP];       // M eigenvalues, in the order of the rows of V
-  double* dvec[FW_MAX_GROUP];      // 3 M: sqrt(g), g, g lambda
+  double* lam[FW_MAX_GROUP];       // M eigenvalues, in the order of the rows of W
+  double* dvec[FW_MAX_GROUP];      // 3 M weights of the rows' outer products, then kBase values (null: eigenvalues only)
   float* lam_sorted[FW_MAX_GROUP]; // optional output: eigenvalues in decreasing order
   float* kappa[FW_MAX_GROUP];      // optional output: rank estimate / M
   float eps[FW_MAX_GROUP];
+  int32_t block0[FW_MAX_GROUP + 1];   // first CTA of each layer in the grid of norm_kernel (a warp per column)
+  int32_t nl;
   float g_max;                     // <= 0: g = 1 / max(lambda, eps) (Eq. 10); > 0: the gains of Eq. 34
 };
+constexpr int kBase = 4;           // weights of the identity in the three outputs; 1.0 when Phi = 0
 
-// One CTA per layer: eigenvalues, their ranks, the rank estimate (Eq. 32 read as exp(-sum lbar log lbar)) and the gains.
+// lambda_m = |w_m|, with the sign of the Rayleigh quotient (one row of Phi suffices: w_m is parallel to v_m) where the
+// eigenvectors are wanted; a warp per column
+__global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ FinishArgs a) {
+  int li = 0;
+#pragma unroll 1
+  for (int i = 1; i < a.nl; ++i)
+    if ((int)blockIdx.x >= a.block0[i]) li = i;
+  const EvdLayer L = a.l[li];
+  const int M = L.M, lane = threadIdx.x & 31;
+  const int m = ((int)blockIdx.x - a.block0[li]) * 8 + (threadIdx.x >> 5);
+  if (m >= M) return;
+  const double* w = L.W + (int64_t)m * evd_ld(M);
+  double acc = 0.0, best = -1.0;
+  int bi = 0;
+  for (int i = lane; i < M; i += 32) {
+    const double x = w[i];
+    acc = fma(x, x, acc);
+    if (fabs(x) > best) { best = fabs(x); bi = i; }
+  }
+  acc = sqrt(warp_sum_d(acc));
+  if (a.dvec[li]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double xo = __shfl_xor_sync(0xffffffffu, best, o);
+      const int io = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (xo > best || (xo == best && io < bi)) { best = xo; bi = io; }
+    }
+    double dot = 0.0;
+    for (int i = lane; i < M; i += 32) dot = fma((double)L.A[(int64_t)bi * M + i], w[i], dot);
+    dot = warp_sum_d(dot);
+    if (dot * w[bi] < 0.0) acc = -acc;
+  }
+  if (lane == 0) a.lam[li][m] = acc;
+}
+
+// sum over the block in a fixed order
+__device__ double block_sum_d(double x, double* red) {
+  x = warp_sum_d(x);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = threadIdx.x < 32 ? red[threadIdx.x] : 0.0;
+  if (threadIdx.x < 32) {
+    x = warp_sum_d(x);
+    if (threadIdx.x == 0) red[0] = x;
+  }
+  __syncthreads();
+  return red[0];
+}
+
+// One CTA per layer: ranks of the eigenvalues, the rank estimate (Eq. 32 read as exp(-sum lbar log lbar)) and the gains.
+// The sums decide an integer (the rank): their order does not depend on the launch.
 __global__ void __launch_bounds__(1024) evd_finish_kernel(const __grid_constant__ FinishArgs a) {
+  __shared__ double red[32];
   const EvdLayer L = a.l[blockIdx.x];
   const int M = L.M;
-  double* lam = a.lam[blockIdx.x];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int m = warp; m < M; m += 32) {
-    const double* w = L.W + (int64_t)m * M;
-    double acc = 0.0;
-    if (L.V) {
-      const double* v = L.V + (int64_t)m * M;
-      for (int i = lane; i < M; i += 32) acc = fma(v[i], w[i], acc);      // Rayleigh quotient v^T Phi v
-      acc = warp_sum_d(acc);
-    } else {
-      for (int i = lane; i < M; i += 32) acc = fma(w[i], w[i], acc);      // |Phi v| (Phi positive semi-definite)
-      acc = sqrt(warp_sum_d(acc));
-    }
-    if (lane == 0) lam[m] = acc;
+  const double* lam = a.lam[blockIdx.x];
+  double x = 0.0;
+  for (int m = threadIdx.x; m < M; m += 1024) x += fmax(lam[m], 0.0);
+  const double S = block_sum_d(x, red);
+  x = 0.0;
+  for (int m = threadIdx.x; m < M; m += 1024) {
+    const double lb = S > 0.0 ? fmax(lam[m], 0.0) / S : 0.0;
+    if (lb > 0.0) x -= lb * log(lb);
   }
-  __syncthreads();
-  __shared__ double s_sum;
-  __shared__ int s_ms;
-  if (threadIdx.x == 0) {
-    // fixed order: the sums decide an integer (the rank) and must not depend on the launch
-    double S = 0.0;
-    for (int m = 0; m < M; ++m) S += fmax(lam[m], 0.0);
-    double H = 0.0;
-    for (int m = 0; m < M; ++m) {
-      const double lb = S > 0.0 ? fmax(lam[m], 0.0) / S : 0.0;
-      if (lb > 0.0) H -= lb * log(lb);
-    }
-    const double ms_hat = exp(H);
-    s_sum = S;
-    int ms = (int)rint(ms_hat);
-    if (ms < 1) ms = 1;
-    if (ms > M) ms = M;
-    s_ms = ms;
-    if (a.kappa[blockIdx.x]) *a.kappa[blockIdx.x] = (float)(ms_hat / (double)M);
-  }
-  __syncthreads();
-  const double S = s_sum;
-  const int Ms = s_ms;
+  const double ms_hat = exp(block_sum_d(x, red));
+  const int Ms = min(max((int)rint(ms_hat), 1), M);
+  if (threadIdx.x == 0 && a.kappa[blockIdx.x]) *a.kappa[blockIdx.x] = (float)(ms_hat / (double)M);
   double* dv = a.dvec[blockIdx.x];
-  for (int m = threadIdx.x; m < M; m += blockDim.x) {
+  const double eps = (double)a.eps[blockIdx.x], g_max = (double)a.g_max;
+  auto gain = [&](double lm, int rank) {
+    if (a.g_max <= 0.f) return 1.0 / fmax(lm, eps);                                        // Eq. 10
+    const double lb = S > 0.0 ? fmax(lm, 0.0) / S : 0.0;
+    return rank < Ms ? fmin(1.0 / fmax((double)M * lb, 1e-300), g_max) : 1.0;              // Eq. 34
+  };
+  float top = 0.f;
+  for (int m = threadIdx.x; m < M; m += 1024) top = fmaxf(top, (float)fabs(lam[m]));
+  const double null = kNull * evd_block_max(top);
+  int nulls = 0;
+  for (int m = threadIdx.x; m < M; m += 1024) nulls += fabs(lam[m]) <= null ? 1 : 0;
+  nulls = (int)(block_sum_d((double)nulls, red) + 0.5);
+  // Null columns span what the others leave: with their common gain g0 they contribute g0 (I - sum v v^T).  When Phi = 0
+  // every column is its own unit vector.
+  const bool zero = nulls == M, some = nulls > 0 && !zero;
+  const double g0 = gain(0.0, M - 1), b0 = some ? sqrt(g0) : 0.0, b1 = some ? g0 : 0.0;
+  for (int m = threadIdx.x; m < M; m += 1024) {
     const double lm = lam[m];
     int rank = 0;                                   // position of lambda_m in decreasing order
+#pragma unroll 8
     for (int j = 0; j < M; ++j) {
       const double lj = lam[j];
       rank += (lj > lm || (lj == lm && j < m)) ? 1 : 0;
     }
     if (a.lam_sorted[blockIdx.x]) a.lam_sorted[blockIdx.x][rank] = (float)lm;
     if (dv) {
-      double g;
-      if (a.g_max <= 0.f) {
-        g = 1.0 / fmax(lm, (double)a.eps[blockIdx.x]);                                  // Eq. 10
-      } else {
-        const double lb = S > 0.0 ? fmax(lm, 0.0) / S : 0.0;
-        g = rank < Ms ? fmin(1.0 / fmax((double)M * lb, 1e-300), (double)a.g_max) : 1.0;   // Eq. 34
-      }
-      dv[m] = sqrt(g);
-      dv[M + m] = g;
-      dv[2 * M + m] = g * lm;
+      const double g = gain(lm, rank);
+      const double n2 = zero ? 1.0 : (fabs(lm) <= null ? 0.0 : 1.0 / (lm * lm));            // rows of W are lambda_m v_m
+      dv[m] = (sqrt(g) - b0) * n2;
+      dv[M + m] = (g - b1) * n2;
+      dv[2 * M + m] = g * lm * n2;
     }
   }
+  if (dv && threadIdx.x == 0) { dv[3 * M] = b0; dv[3 * M + 1] = b1; dv[3 * M + 2] = 0.0; dv[3 * M + 3] = zero ? 1.0 : 0.0; }
 }
 
 struct VdvArgs {
@@ -278,139 +517,185 @@ struct VdvArgs {
   float* T[FW_MAX_GROUP];
   float* Q[FW_MAX_GROUP];
   float* Y[FW_MAX_GROUP];
-  int32_t tile0[FW_MAX_GROUP + 1];   // flat grid over the 32 x 32 tiles of all layers
+  int32_t tile0[FW_MAX_GROUP + 1];   // flat grid over the upper-triangle 64 x 64 tiles of all layers
   int32_t nl;
 };
 
-// out_ij = sum_m d_m V_mi V_mj for the three weight vectors at once; the product V_mi V_mj is formed first, so
-// entry (i, j) and entry (j, i) see the same operations in the same order: the outputs are exactly symmetric.
+// out_ij = sum_m d_m w_mi w_mj for the three weight vectors at once, on the fp64 tensor cores; a CTA computes a tile of
+// the upper triangle and writes its mirror image too, so the outputs are exactly symmetric.  A warp takes 16 x 32.
+constexpr int VT = 64, VK = 16, kVs = VT + 4;
 __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArgs a) {
   int li = 0;
 #pragma unroll 1
   for (int i = 1; i < a.nl; ++i)
     if ((int)blockIdx.x >= a.tile0[i]) li = i;
   const EvdLayer L = a.l[li];
-  const int M = L.M;
-  const int nt = (M + 31) / 32;
-  const int tile = (int)blockIdx.x - a.tile0[li];
-  const int bi = tile / nt, bj = tile - bi * nt;
-  __shared__ double sa[32][33], sb[32][33], sd[3][32];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
-  double acc[3][4];
+  const int M = L.M, ld = evd_ld(M);
+  int bi, bj;
+  tri_decode((int)blockIdx.x - a.tile0[li], (M + VT - 1) / VT, bi, bj);
+  __shared__ __align__(16) double sa[VK][kVs], sb[VK][kVs], sd[3][VK];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wi = (warp >> 1) * 16, wj = (warp & 1) * 32;         // 4 x 2 warps
+  const double* dv = a.dvec[li];
+  double acc[3][2][4][2];
 #pragma unroll
   for (int o = 0; o < 3; ++o)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) acc[o][r] = 0.0;
-  const double* dv = a.dvec[li];
-  for (int m0 = 0; m0 < M; m0 += 32) {
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int mm = m0 + ty + 8 * r;
-      const int ci = bi * 32 + tx, cj = bj * 32 + tx;
-      sa[ty + 8 * r][tx] = (mm < M && ci < M) ? L.V[(int64_t)mm * M + ci] : 0.0;
-      sb[ty + 8 * r][tx] = (mm < M && cj < M) ? L.V[(int64_t)mm * M + cj] : 0.0;
+      for (int c = 0; c < 4; ++c) acc[o][r][c][0] = acc[o][r][c][1] = 0.0;
+  const bool unit = dv[3 * M + 3] != 0.0;                          // Phi = 0: unit vectors
+  for (int m0 = 0; m0 < M && !unit; m0 += VK) {
+    for (int i = tid; i < VK * VT; i += 256) {
+      const int mm = i / VT, c = i - mm * VT;
+      const int gi = bi * VT + c, gj = bj * VT + c;
+      sa[mm][c] = (m0 + mm < M && gi < M) ? L.W[(int64_t)(m0 + mm) * ld + gi] : 0.0;
+      sb[mm][c] = (m0 + mm < M && gj < M) ? L.W[(int64_t)(m0 + mm) * ld + gj] : 0.0;
     }
-    if (threadIdx.x < 96) {
-      const int o = threadIdx.x >> 5, mm = m0 + (threadIdx.x & 31);
-      sd[o][threadIdx.x & 31] = mm < M ? dv[o * M + mm] : 0.0;
+    if (tid < 3 * VK) {
+      const int o = tid / VK, mm = tid - o * VK;
+      sd[o][mm] = m0 + mm < M ? dv[o * M + m0 + mm] : 0.0;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 32; ++k) {
-      const double bj_ = sb[k][tx];
-      const double d0 = sd[0][k], d1 = sd[1][k], d2 = sd[2][k];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const double pr = sa[k][ty + 8 * r] * bj_;
-        acc[0][r] = fma(d0, pr, acc[0][r]);
-        acc[1][r] = fma(d1, pr, acc[1][r]);
-        acc[2][r] = fma(d2, pr, acc[2][r]);
+    for (int k = 0; k < VK / 4; ++k) {
+      const int mm = 4 * k + (lane & 3);
+      double af[2], bf[4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) af[r] = sa[mm][wi + 8 * r + (lane >> 2)];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) bf[c] = sb[mm][wj + 8 * c + (lane >> 2)];
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        const double d = sd[o][mm];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const double ad = af[r] * d;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mma_f64(acc[o][r][c], ad, bf[c]);
+        }
       }
     }
     __syncthreads();
   }
-  const int j = bj * 32 + tx;
+  float* out[3] = {a.T[li], a.Q[li], a.Y[li]};
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = bi * 32 + ty + 8 * r;
-    if (i < M && j < M) {
-      const int64_t off = (int64_t)i * M + j;
-      a.T[li][off] = (float)acc[0][r];
-      a.Q[li][off] = (float)acc[1][r];
-      a.Y[li][off] = (float)acc[2][r];
-    }
+  for (int o = 0; o < 3; ++o) {
+    const double base = dv[3 * M + o];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int i = bi * VT + wi + 8 * r + (lane >> 2), j = bj * VT + wj + 8 * c + 2 * (lane & 3) + h;
+          if (i < M && j < M && j >= i) {
+            double x = acc[o][r][c][h];
+            if (i == j) x += unit ? dv[o * M + i] : base;
+            out[o][(int64_t)i * M + j] = (float)x;
+            out[o][(int64_t)j * M + i] = (float)x;
+          }
+        }
   }
 }
 
 }  // namespace
 
-// Scratch of one layer: W and V (fp64), eigenvalues and the three weight vectors, and the barrier words
+// Scratch of one layer: barrier words, W (fp64), eigenvalues, the three weight vectors and the identity's weights.  The
+// size callers have been told is that of two M x M matrices; small M need more for the padding of the rows.
 size_t evd_scratch_bytes(int M) {
-  return 2 * (size_t)M * M * sizeof(double) + 4 * (size_t)M * sizeof(double) + 1024;
+  const size_t m = (size_t)M;
+  return std::max(m * evd_ld(M), 2 * m * m) * sizeof(double) + (4 * m + kBase) * sizeof(double) + kWords * 4;
 }
 
-// Decomposes src[i] (M x M fp32 symmetric) of every layer.  with_v: eigenvectors too, then T, Q, Phi_y are written to
-// the three outputs (T is symmetric: it is its own transpose).  lam_out / kappa_out: optional per-layer outputs.
+// Decomposes src[i] (M x M fp32 symmetric) of every layer.  with_v: T, Q, Phi_y are written to the three outputs (T is
+// symmetric: it is its own transpose).  lam_out / kappa_out: optional per-layer outputs.
 cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void* const* scratch,
                        int32_t* const* status, const float* eps, bool with_v, float g_max, float* const* T_out,
                        float* const* Q_out, float* const* Y_out, float* const* lam_out, float* const* kappa_out,
                        cudaStream_t s) {
   static int n_sm[64] = {0};
+  static SmemAttrCache attr;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) dev = 0;
   if (n_sm[dev] == 0) {
-    e = cudaDeviceGetAttribute(&n_sm[dev], cudaDevAttrMultiProcessorCount, dev);
+    int v = 0;
+    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    n_sm[dev] = v;
   }
   EvdArgs a;
   FinishArgs f;
   VdvArgs v;
   memset(&a, 0, sizeof(a)); memset(&f, 0, sizeof(f)); memset(&v, 0, sizeof(v));
-  int pairs = 0, tiles = 0, n_max = 0;
+  int tiles = 0, blocks = 0, stride = 0;
   for (int i = 0; i < n; ++i) {
     const int M = layer_M[i];
     char* base = reinterpret_cast<char*>(scratch[i]);
     EvdLayer& l = a.l[i];
     l.A = src[i];
-    l.W = reinterpret_cast<double*>(base + 1024);
-    l.V = with_v ? l.W + (size_t)M * M : nullptr;
+    l.words = reinterpret_cast<int32_t*>(base);
+    l.W = reinterpret_cast<double*>(base + kWords * 4);
     l.status = status[i];
     l.M = M;
-    l.n = M + (M & 1);
-    a.pair0[i] = pairs;
-    pairs += l.n / 2;
-    if (l.n > n_max) n_max = l.n;
-    f.l[i] = l; v.l[i] = l;
-    f.lam[i] = l.W + 2 * (size_t)M * M;
+    l.nb = ((M + EB - 1) / EB + 1) & ~1;
+    l.n = 1;
+    f.lam[i] = l.W + (size_t)M * evd_ld(M);
     f.dvec[i] = with_v ? f.lam[i] + M : nullptr;
     f.lam_sorted[i] = lam_out ? lam_out[i] : nullptr;
     f.kappa[i] = kappa_out ? kappa_out[i] : nullptr;
     f.eps[i] = eps[i];
+    f.block0[i] = blocks;
+    blocks += (M + 7) / 8;
     v.dvec[i] = f.dvec[i];
     if (with_v) { v.T[i] = T_out[i]; v.Q[i] = Q_out[i]; v.Y[i] = Y_out[i]; }
     v.tile0[i] = tiles;
-    tiles += ((M + 31) / 32) * ((M + 31) / 32);
-  }
-  a.pair0[n] = pairs; v.tile0[n] = tiles;
-  a.nl = n; v.nl = n;
-  a.rounds_max = n_max - 1;
-  int nctas = n_sm[dev];
-  if (nctas * EW > pairs) nctas = (pairs + EW - 1) / EW;
-  if (nctas < 1) nctas = 1;
-  a.nctas = nctas;
-  a.bar = reinterpret_cast<int32_t*>(scratch[0]);
-  f.g_max = g_max;
-  e = cudaMemsetAsync(a.bar, 0, 1024, s);
-  if (e != cudaSuccess) return e;
-  {
-    // n >= 2 players per layer, so every launch has at least one round
-    void* args[] = {&a};
-    ProfScope ps(FW_PROF_MISC, s);
-    e = cudaLaunchCooperativeKernel((void*)jacobi_kernel, dim3(nctas), dim3(ET), args, 0, s);
+    const int t = (M + VT - 1) / VT;
+    tiles += t * (t + 1) / 2;
+    stride = std::max(stride, evd_stride(std::min(evd_ld(M), kChunk)));
+    e = cudaMemsetAsync(l.words, 0, kWords * 4, s);
     if (e != cudaSuccess) return e;
   }
+  f.block0[n] = blocks; v.tile0[n] = tiles;
+  a.nl = n; f.nl = n; v.nl = n;
+  f.g_max = g_max;
+  // CTAs: one per layer, then one more to the layer that takes longest, as long as it helps it.  A round costs a fixed
+  // part (inner rotations, barrier) and a part in proportion to the columns' length; a CTA takes its pairs in turn.
+  auto cost = [&](const EvdLayer& l, int ctas) {
+    const int np = l.nb / 2;
+    return (double)(l.nb - 1) * ((np + ctas - 1) / ctas) * (600.0 + l.M);
+  };
+  for (int used = n; used < n_sm[dev]; ) {
+    int w = 0;
+    for (int i = 1; i < n; ++i)
+      if (cost(a.l[i], a.l[i].n) > cost(a.l[w], a.l[w].n)) w = i;
+    const int np = a.l[w].nb / 2;
+    const int turns = (np + a.l[w].n - 1) / a.l[w].n;
+    if (turns == 1) break;
+    const int need = (np + turns - 2) / (turns - 1);             // CTAs for one turn less
+    if (used + need - a.l[w].n > n_sm[dev]) break;
+    used += need - a.l[w].n;
+    a.l[w].n = need;
+  }
+  int ctas = 0;
+  for (int i = 0; i < n; ++i) { a.l[i].cta0 = ctas; ctas += a.l[i].n; f.l[i] = a.l[i]; v.l[i] = a.l[i]; }
+  const size_t smem = ((size_t)EP * stride + kPartDoubles + EP * kGLd) * sizeof(double);
+  e = ensure_dyn_smem(jacobi_kernel, smem, attr);
+  if (e != cudaSuccess) return e;
+  {
+    void* args[] = {&a};
+    ProfScope ps(FW_PROF_MISC, s);
+    e = cudaLaunchCooperativeKernel((void*)jacobi_kernel, dim3(ctas), dim3(ET), args, smem, s);
+    if (e != cudaSuccess) return e;
+  }
+  {
+    ProfScope ps(FW_PROF_MISC, s);
+    norm_kernel<<<blocks, 256, 0, s>>>(f);
+  }
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   {
     ProfScope ps(FW_PROF_MISC, s);
     evd_finish_kernel<<<n, 1024, 0, s>>>(f);
