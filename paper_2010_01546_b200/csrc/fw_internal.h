@@ -152,7 +152,8 @@ struct GemmProblem {
   int32_t m, n;
   int64_t k;
   int32_t a_kmajor, sym, splits, epi;
-  int32_t tiles_m, tiles_n, ntiles, first_cta;   // filled by the launcher
+  int32_t tiles_m, tiles_n, ntiles, first_cta;   // filled by the launcher, with
+  int32_t vec_a, vec_b, vec_c;                   // 16-byte accesses to A, B, C
   float lr;
   int32_t in_bf16;         // A and B elements are bf16 (Gram on bf16 X)
   int32_t* nonfinite;      // optional: set to 1 when the product holds a NaN or Inf
