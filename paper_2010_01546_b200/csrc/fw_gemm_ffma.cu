@@ -4,9 +4,10 @@
 //   - the re-sync products T Phix and (T Phix) T^T.
 // One launch covers every problem of a group; a CTA finds its problem, tile and K-split from its block index.
 //
-// A group of 128 threads computes a 64 x 64 tile, 8 x 4 accumulators per thread, from 16-deep slabs staged through
-// registers (where the Gram pass subtracts its shift) into two shared-memory buffers.  It is bound by the FP32 pipe when
-// the tiles fill the machine; when they do not, what counts is the length of the chain of slabs, so 2 or 4 groups of a
+// A group of 64 threads computes a 64 x 64 tile, 8 x 8 accumulators per thread (packed fp32 pairs: one instruction for two
+// products), from 16-deep slabs copied asynchronously
+// into three shared-memory buffers, where the thread that copied an element subtracts the Gram pass's shift from it.  It is bound by the FP32 pipe when
+// the tiles fill the machine; when they do not, what counts is the length of the chain of slabs, so 2, 4 or 8 groups of a
 // CTA share the tile, each a contiguous part of K, and their sums are added in order at the end: the chain is that much
 // shorter and the SM has that many more warps to hide it.  Products of the ResNet-20-shaped set at batch 32 (Gram /
 // re-sync / G Qs): 1028 / 310 / 101 us with 4 x 4 accumulators, scalar loads and one group; see launch_gemm_ffma.
@@ -18,10 +19,11 @@ namespace fw {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 128;   // tile, slab, threads of a group
-constexpr int TM = 8, TN = 4;                        // accumulators per thread: 8 x 16 threads
-constexpr int LDA = BM + 4, LDB = BN + 4;            // shared-memory rows
-constexpr int kSlab = BK * (LDA + LDB);              // floats of one buffer
+constexpr int BM = 64, BN = 64, BK = 16;             // tile, slab
+constexpr int TM = 8;                                // rows per thread
+constexpr int LDA = BM + 4;                          // shared-memory rows of both operands
+constexpr int kSlab = 2 * BK * LDA;                  // floats of one stage
+constexpr int kStages = 3;
 
 // The kernel's argument block carries as many problems as the launch needs: a launch costs 0.7 us per KB of arguments.
 template <int CAP>
@@ -30,85 +32,116 @@ struct GemmBlock {
   GemmProblem p[CAP];
 };
 
-__device__ __forceinline__ float ld_elem(const void* base, int64_t idx, int bf16) {
-  if (bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[idx]);
-  return reinterpret_cast<const float*>(base)[idx];
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(u64 r, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r)); }
+__device__ __forceinline__ void fma2(u64& c, u64 a, u64 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
+
+__device__ __forceinline__ void cp_async16(float* d, const float* p, bool in) {
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(d);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(p), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async4(float* d, const float* p, bool in) {
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(d);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sa), "l"(p), "r"(in ? 4 : 0) : "memory");
 }
 
-// A slab of a matrix stored k x n (row-major, n contiguous): element (k, n) at P[k ld + n]; 64 columns from n0.  Thread t
-// of a group holds entries (k, n) as two float4 of one column quad (vec) or eight scalars.
-struct SlabRegs { float v[8]; };
-__device__ __forceinline__ void load_kmajor(SlabRegs& r, const void* P, int64_t ld, int64_t k0, int64_t ke, int n0, int n, int t,
-                                            bool vec, int bf16) {
+// A group's shape: TN columns per thread, so 64 (TN = 8) or 128 (TN = 4) threads.
+template <int TN>
+struct Shape {
+  static constexpr int NT = BM * BN / (TM * TN);
+  static constexpr int KV = NT / 16, KS = NT / 64;   // rows of a slab a pass of the group covers: quads, single columns
+};
+
+// One operand's slab into shared memory (row k of the slab at S + k LDA), asynchronously.  A thread copies
+// quads of columns 4 (t % 16) ... of rows k = t / 16 + KV e, or (not vec) column t % 64 of rows k = t / 64 + KS e from p, its
+// first element of the slab; `left` rows of K are inside the matrix, the rest becomes zero (base: an address inside the
+// matrix for the copies that read nothing).
+template <int TN>
+__device__ __forceinline__ void stage_kmajor(float* S, const float* p, const float* base, int64_t ld, int left, bool in, int t,
+                                             bool vec) {
   if (vec) {
-    const int c = n0 + 4 * (t & 15);
+    constexpr int KV = Shape<TN>::KV;
+    const int k0 = t >> 4;
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int64_t k = k0 + (t >> 4) + 8 * e;
-      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k < ke && c < n) q = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(P) + k * ld + c);
-      *reinterpret_cast<float4*>(r.v + 4 * e) = q;
+    for (int e = 0; e < BK / KV; ++e) {
+      const bool ok = in && k0 + KV * e < left;
+      cp_async16(S + (k0 + KV * e) * LDA + 4 * (t & 15), ok ? p + KV * e * ld : base, ok);
     }
   } else {
-    const int c = n0 + (t & 63);
+    constexpr int KS = Shape<TN>::KS;
+    const int k0 = t >> 6;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int64_t k = k0 + (t >> 6) + 2 * e;
-      r.v[e] = (k < ke && c < n) ? ld_elem(P, k * ld + c, bf16) : 0.f;
+    for (int e = 0; e < BK / KS; ++e) {
+      const bool ok = in && k0 + KS * e < left;
+      cp_async4(S + (k0 + KS * e) * LDA + (t & 63), ok ? p + KS * e * ld : base, ok);
     }
   }
 }
-// shift: subtracted from the elements inside the matrix (zero for the padding)
-__device__ __forceinline__ void store_kmajor(float* S, int lds, const SlabRegs& r, const float (&sh)[4], int64_t k0, int64_t ke,
-                                             int t, bool vec) {
-  if (vec) {
+template <int TN>
+__device__ __forceinline__ void stage_bf16(float* S, const __nv_bfloat16* p, int64_t ld, int left, bool in, int t) {
+  constexpr int KS = Shape<TN>::KS;
+  const int k0 = t >> 6;
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int kk = (t >> 4) + 8 * e;
-      float4 q = *reinterpret_cast<const float4*>(r.v + 4 * e);
-      if (k0 + kk < ke) { q.x -= sh[0]; q.y -= sh[1]; q.z -= sh[2]; q.w -= sh[3]; }
-      *reinterpret_cast<float4*>(S + kk * lds + 4 * (t & 15)) = q;
+  for (int e = 0; e < BK / KS; ++e)
+    S[(k0 + KS * e) * LDA + (t & 63)] = (in && k0 + KS * e < left) ? __bfloat162float(p[KS * e * ld]) : 0.f;
+}
+// The shift, subtracted from the elements inside the matrix by the thread that copied them
+template <int TN>
+__device__ __forceinline__ void centre(float* S, const float (&sh)[4], int left, int t, bool vec) {
+  if (vec) {
+    constexpr int KV = Shape<TN>::KV;
+#pragma unroll
+    for (int e = 0; e < BK / KV; ++e) {
+      const int kk = (t >> 4) + KV * e;
+      float4* q = reinterpret_cast<float4*>(S + kk * LDA + 4 * (t & 15));
+      if (kk < left) { float4 x = *q; x.x -= sh[0]; x.y -= sh[1]; x.z -= sh[2]; x.w -= sh[3]; *q = x; }
     }
   } else {
+    constexpr int KS = Shape<TN>::KS;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int kk = (t >> 6) + 2 * e;
-      S[kk * lds + (t & 63)] = k0 + kk < ke ? r.v[e] - sh[0] : r.v[e];
+    for (int e = 0; e < BK / KS; ++e) {
+      const int kk = (t >> 6) + KS * e;
+      if (kk < left) S[kk * LDA + (t & 63)] -= sh[0];
     }
   }
 }
-// A stored m x k (row-major, k contiguous): a thread takes quads of k of row t % 64, stored transposed
-__device__ __forceinline__ void load_mmajor(SlabRegs& r, const float* P, int64_t ld, int64_t k0, int64_t ke, int m0, int m, int t,
-                                            bool vec) {
-  const int row = m0 + (t & 63);
-  const float* p = P + (int64_t)row * ld;
+// An M-major operand (stored m x k) is transposed on its way: a thread (TN = 4) takes quads of k = 4 (t / 64) + 8 e of row
+// t % 64 through registers, loaded before a slab's products and stored after them.
+struct QuadRegs { float4 q[2]; };
+__device__ __forceinline__ void load_mmajor(QuadRegs& r, const float* p, int left, bool in, int t, bool vec) {
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
-    const int64_t k = k0 + 4 * ((t >> 6) + 2 * e);
-    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row < m) {
-      if (vec && k + 4 <= ke) q = *reinterpret_cast<const float4*>(p + k);
-      else {
-        if (k < ke) q.x = p[k];
-        if (k + 1 < ke) q.y = p[k + 1];
-        if (k + 2 < ke) q.z = p[k + 2];
-        if (k + 3 < ke) q.w = p[k + 3];
-      }
+    const int k = 4 * (t >> 6) + 8 * e;
+    r.q[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!in) continue;
+    if (vec && k + 4 <= left) r.q[e] = *reinterpret_cast<const float4*>(p + k);
+    else {
+      if (k < left) r.q[e].x = p[k];
+      if (k + 1 < left) r.q[e].y = p[k + 1];
+      if (k + 2 < left) r.q[e].z = p[k + 2];
+      if (k + 3 < left) r.q[e].w = p[k + 3];
     }
-    *reinterpret_cast<float4*>(r.v + 4 * e) = q;
   }
 }
-__device__ __forceinline__ void store_mmajor(float* S, const SlabRegs& r, int t) {
+__device__ __forceinline__ void store_mmajor(float* S, const QuadRegs& r, int t) {
 #pragma unroll
-  for (int e = 0; e < 2; ++e)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) S[(4 * ((t >> 6) + 2 * e) + i) * LDA + (t & 63)] = r.v[4 * e + i];
+  for (int e = 0; e < 2; ++e) {
+    float* d = S + (4 * (t >> 6) + 8 * e) * LDA + (t & 63);
+    d[0] = r.q[e].x; d[LDA] = r.q[e].y; d[2 * LDA] = r.q[e].z; d[3 * LDA] = r.q[e].w;
+  }
 }
 
 extern __shared__ __align__(16) float gsm[];
 
-template <int KG, int CAP>
-__global__ void __launch_bounds__(NT * KG) gemm_ffma_kernel(const __grid_constant__ GemmBlock<CAP> g) {
+// AKM: A is K-major (copied asynchronously); else M-major, TN = 4
+template <int TN, bool AKM, int KG, int CAP>
+__global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm_ffma_kernel(const __grid_constant__ GemmBlock<CAP> g) {
+  constexpr int NT = Shape<TN>::NT;
   // locate the problem this CTA works on
   const int cta = blockIdx.x;
   int pi = 0;
@@ -131,83 +164,130 @@ __global__ void __launch_bounds__(NT * KG) gemm_ffma_kernel(const __grid_constan
   const int64_t gper = (max(se - sb, (int64_t)0) + KG - 1) / KG;
   const int64_t kb = (sb + grp * gper) * BK, ke = min(min(sb + (grp + 1) * gper, se) * BK, pr.k);
 
-  float* slab = gsm + grp * 2 * kSlab;
-  const int tx = t & 15, ty = t >> 4;
-  float acc[TM][TN];
+  float* slab = gsm + grp * kStages * kSlab;
+  const int tx = t % (BN / TN), ty = t / (BN / TN);
+  u64 acc2[TM / 2][TN];      // rows 8 ty + 2 i, + 1; columns 4 tx + j (and 32 + 4 tx + j - 4)
 #pragma unroll
-  for (int i = 0; i < TM; ++i)
+  for (int i = 0; i < TM / 2; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-  const bool a_km = pr.a_kmajor != 0;
-  const bool same = a_km && pr.A == pr.B && pr.lda == pr.ldb && m0 == n0;        // diagonal Gram tile: one operand
+    for (int j = 0; j < TN; ++j) acc2[i][j] = 0;
+  const bool same = AKM && pr.A == pr.B && pr.lda == pr.ldb && m0 == n0;        // diagonal Gram tile: one operand
   const bool vec_a = pr.vec_a != 0, vec_b = pr.vec_b != 0;
+  const int bf16 = pr.in_bf16;
   const bool want_colsum = pr.colsum != nullptr && tm == tn;
-  float colacc = 0.f;        // thread t < BM of a group: column m0 + t
-  float sha[4], shb[4];
+  float colacc = 0.f;        // column m0 + t
+  // my column (or row) of each operand, and whether it is inside the matrix
+  const int ca = AKM && vec_a ? m0 + 4 * (t & 15) : m0 + (t & 63), cb = vec_b ? n0 + 4 * (t & 15) : n0 + (t & 63);
+  const bool in_a = ca < pr.m, in_b = cb < pr.n;
+  float sha[4] = {0.f, 0.f, 0.f, 0.f}, shb[4] = {0.f, 0.f, 0.f, 0.f};
+  if (pr.shift) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int ca = vec_a ? m0 + 4 * (t & 15) + i : m0 + (t & 63), cb = vec_b ? n0 + 4 * (t & 15) + i : n0 + (t & 63);
-    sha[i] = pr.shift && ca < pr.m ? pr.shift[ca] : 0.f;
-    shb[i] = pr.shift && cb < pr.n ? pr.shift[cb] : 0.f;
+    for (int i = 0; i < 4; ++i) {
+      if (ca + i < pr.m) sha[i] = pr.shift[ca + i];
+      if (cb + i < pr.n) shb[i] = pr.shift[cb + i];
+    }
   }
-  SlabRegs ra, rb;
-  auto load = [&](int64_t k0) {
-    if (a_km) load_kmajor(ra, pr.A, pr.lda, k0, ke, m0, pr.m, t, vec_a, pr.in_bf16);
-    else load_mmajor(ra, reinterpret_cast<const float*>(pr.A), pr.lda, k0, ke, m0, pr.m, t, vec_a);
-    if (!same) load_kmajor(rb, pr.B, pr.ldb, k0, ke, n0, pr.n, t, vec_b, pr.in_bf16);
+  const int64_t lda = pr.lda, ldb = pr.ldb;
+  const float* pa = reinterpret_cast<const float*>(pr.A);
+  const float* pb = reinterpret_cast<const float*>(pr.B);
+  {
+    const int64_t oa = AKM ? (kb + (vec_a ? t >> 4 : t >> 6)) * lda + ca : (int64_t)ca * lda + kb;
+    const int64_t ob = (kb + (vec_b ? t >> 4 : t >> 6)) * ldb + cb;
+    if (bf16) {
+      pa = reinterpret_cast<const float*>(reinterpret_cast<const __nv_bfloat16*>(pr.A) + oa);
+      pb = reinterpret_cast<const float*>(reinterpret_cast<const __nv_bfloat16*>(pr.B) + ob);
+    } else {
+      pa += oa; pb += ob;
+    }
+  }
+  const int64_t step_a = AKM ? BK * lda : BK, step_b = BK * ldb;
+  QuadRegs rq;
+  auto stage = [&](int left, int buf) {
+    float* S = slab + buf * kSlab;
+    if (bf16) {
+      stage_bf16<TN>(S, reinterpret_cast<const __nv_bfloat16*>(pa), lda, left, in_a, t);
+      if (!same) stage_bf16<TN>(S + BK * LDA, reinterpret_cast<const __nv_bfloat16*>(pb), ldb, left, in_b, t);
+      pa = reinterpret_cast<const float*>(reinterpret_cast<const __nv_bfloat16*>(pa) + step_a);
+      pb = reinterpret_cast<const float*>(reinterpret_cast<const __nv_bfloat16*>(pb) + step_b);
+    } else {
+      if (AKM) stage_kmajor<TN>(S, pa, reinterpret_cast<const float*>(pr.A), lda, left, in_a, t, vec_a);
+      else load_mmajor(rq, pa, left, in_a, t, vec_a);
+      if (!same) stage_kmajor<TN>(S + BK * LDA, pb, reinterpret_cast<const float*>(pr.B), ldb, left, in_b, t, vec_b);
+      pa += step_a; pb += step_b;
+    }
   };
-  auto store = [&](int64_t k0, int buf) {
-    float* As = slab + buf * kSlab;
-    if (a_km) store_kmajor(As, LDA, ra, sha, k0, ke, t, vec_a);
-    else store_mmajor(As, ra, t);
-    if (!same) store_kmajor(As + BK * LDA, LDB, rb, shb, k0, ke, t, vec_b);
-  };
+  auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
   auto sync = [&] {
     if (KG == 1) __syncthreads();
     else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(NT) : "memory");
   };
 
-  int buf = 0;
-  if (kb < ke) {
-    load(kb);
-    store(kb, 0);
+  int64_t left64 = ke - kb;      // rows of K from the current slab on
+  auto rows = [&](int ahead) { return (int)max((int64_t)0, min(left64 - ahead * BK, (int64_t)BK)); };
+#pragma unroll
+  for (int i = 0; i < kStages - 1; ++i) {
+    if (rows(i) > 0) {
+      stage(rows(i), i);
+      if (!AKM) store_mmajor(slab + i * kSlab, rq, t);
+    }
+    commit();
   }
-  sync();
-  for (int64_t k0 = kb; k0 < ke; k0 += BK) {
-    const bool more = k0 + BK < ke;
-    if (more) load(k0 + BK);
+  int buf = 0;
+  for (; left64 > 0; left64 -= BK) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+    if (pr.shift) {
+      float* S = slab + buf * kSlab;
+      centre<TN>(S, sha, rows(0), t, vec_a);
+      if (!same) centre<TN>(S + BK * LDA, shb, rows(0), t, vec_b);
+    }
+    sync();                      // the slab is complete, and the one before it is free
+    const int nb = buf == 0 ? kStages - 1 : buf - 1;
+    const bool more = rows(kStages - 1) > 0;
+    if (more) stage(rows(kStages - 1), nb);
+    commit();
     const float* As = slab + buf * kSlab;
     const float* Bs = same ? As : As + BK * LDA;
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(As + kk * LDA + TM * ty);
-      const float4 a1 = *reinterpret_cast<const float4*>(As + kk * LDA + TM * ty + 4);
-      const float4 b4 = *reinterpret_cast<const float4*>(Bs + kk * LDB + TN * tx);
-      const float a[TM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[TN] = {b4.x, b4.y, b4.z, b4.w};
+      const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(As + kk * LDA + TM * ty);
+      const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(As + kk * LDA + TM * ty + 4);
+      const float4 b0 = *reinterpret_cast<const float4*>(Bs + kk * LDA + 4 * tx);
+      const float4 b1 = TN == 8 ? *reinterpret_cast<const float4*>(Bs + kk * LDA + 32 + 4 * tx) : b0;
+      const u64 a[TM / 2] = {a0.x, a0.y, a1.x, a1.y};
+      const float bs[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-      for (int i = 0; i < TM; ++i)
+      for (int j = 0; j < TN; ++j) {
+        const u64 b = pack2(bs[j], bs[j]);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int i = 0; i < TM / 2; ++i) fma2(acc2[i][j], a[i], b);
+      }
     }
     if (want_colsum && t < BM) {
 #pragma unroll
       for (int kk = 0; kk < BK; ++kk) colacc += As[kk * LDA + t];
     }
-    if (more) store(k0 + BK, buf ^ 1);
-    sync();
-    buf ^= 1;
+    if (!AKM && more) store_mmajor(slab + nb * kSlab, rq, t);
+    buf = buf == kStages - 1 ? 0 : buf + 1;
   }
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) unpack2(acc2[i][j], acc[2 * i][j], acc[2 * i + 1][j]);
 
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   // the groups' sums, added in order by the first one (thread t of every group holds the same entries)
   if (KG > 1) {
     __syncthreads();
-    float4* part = reinterpret_cast<float4*>(gsm);                                // [group - 1][8][NT] float4, then column sums
+    float4* part = reinterpret_cast<float4*>(gsm);                                // [group - 1][TN / 4 TM][NT] float4, then column sums
     float* cols = gsm + (KG - 1) * TM * TN * NT;
     if (grp > 0) {
 #pragma unroll
       for (int i = 0; i < TM; ++i)
-        part[((grp - 1) * TM + i) * NT + t] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+#pragma unroll
+        for (int h = 0; h < TN / 4; ++h)
+          part[((grp - 1) * (TN / 4) * TM + (TN / 4) * i + h) * NT + t] =
+              make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
       if (want_colsum && t < BM) cols[(grp - 1) * BM + t] = colacc;
     }
     __syncthreads();
@@ -216,8 +296,11 @@ __global__ void __launch_bounds__(NT * KG) gemm_ffma_kernel(const __grid_constan
     for (int q = 0; q < KG - 1; ++q) {
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        const float4 o = part[(q * TM + i) * NT + t];
-        acc[i][0] += o.x; acc[i][1] += o.y; acc[i][2] += o.z; acc[i][3] += o.w;
+#pragma unroll
+        for (int h = 0; h < TN / 4; ++h) {
+          const float4 o = part[(q * (TN / 4) * TM + (TN / 4) * i + h) * NT + t];
+          acc[i][4 * h] += o.x; acc[i][4 * h + 1] += o.y; acc[i][4 * h + 2] += o.z; acc[i][4 * h + 3] += o.w;
+        }
       }
       if (want_colsum && t < BM) colacc += cols[q * BM + t];
     }
@@ -226,51 +309,57 @@ __global__ void __launch_bounds__(NT * KG) gemm_ffma_kernel(const __grid_constan
   // epilogue
   float* C = pr.C + (int64_t)split * pr.c_split_stride;
   const bool vec_c = pr.vec_c != 0;
-  const int ng0 = n0 + TN * tx, mg0 = m0 + TM * ty;
+  const int mg0 = m0 + TM * ty;
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int mg = mg0 + i;
-    if (mg >= pr.m || ng0 >= pr.n) continue;
-    float* c = C + (int64_t)mg * pr.ldc + ng0;
-    const bool quad = vec_c && ng0 + TN <= pr.n;
-    float o[TN] = {0.f, 0.f, 0.f, 0.f};
-    if (pr.epi == EPI_SGD) {
-      if (quad) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(c);
+  for (int h = 0; h < TN / 4; ++h) {
+    const int ng0 = n0 + 32 * h + 4 * tx;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+      const int mg = mg0 + i;
+      if (mg >= pr.m || ng0 >= pr.n) continue;
+      float* c = C + (int64_t)mg * pr.ldc + ng0;
+      const bool quad = vec_c && ng0 + 4 <= pr.n;
+      float o[4] = {0.f, 0.f, 0.f, 0.f};
+      if (pr.epi == EPI_SGD) {
+        if (quad) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(c);
+        else
+#pragma unroll
+          for (int j = 0; j < 4; ++j) if (ng0 + j < pr.n) o[j] = c[j];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float x = acc[i][4 * h + j];
+        bad |= ng0 + j < pr.n && !isfinite(x);
+        if (pr.epi == EPI_SGD) o[j] = fmaf(-pr.lr, x, o[j]);
+        else o[j] = pr.colbias && ng0 + j < pr.n ? x - pr.colbias[ng0 + j] : x;
+      }
+      if (pr.epi == EPI_SYMM && tm == tn) {
+        // both images of a diagonal tile come from its upper triangle
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (ng0 + j < pr.n && ng0 + j >= mg) { c[j] = o[j]; C[(int64_t)(ng0 + j) * pr.ldc + mg] = o[j]; }
+        continue;
+      }
+      if (quad) *reinterpret_cast<float4*>(c) = *reinterpret_cast<const float4*>(o);
       else
 #pragma unroll
-        for (int j = 0; j < TN; ++j) if (ng0 + j < pr.n) o[j] = c[j];
+        for (int j = 0; j < 4; ++j) if (ng0 + j < pr.n) c[j] = o[j];
     }
+    if (pr.epi == EPI_SYMM && tm != tn) {
+      // the mirror image: a thread's eight rows are eight consecutive entries of each of its columns' rows
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      bad |= ng0 + j < pr.n && !isfinite(acc[i][j]);
-      if (pr.epi == EPI_SGD) o[j] = fmaf(-pr.lr, acc[i][j], o[j]);
-      else o[j] = pr.colbias && ng0 + j < pr.n ? acc[i][j] - pr.colbias[ng0 + j] : acc[i][j];
-    }
-    if (pr.epi == EPI_SYMM && tm == tn) {
-      // both images of a diagonal tile come from its upper triangle
+      for (int j = 0; j < 4; ++j) {
+        if (ng0 + j >= pr.n) continue;
+        float* c = C + (int64_t)(ng0 + j) * pr.ldc + mg0;
+        const int q = 4 * h + j;
+        if (vec_c && mg0 + TM <= pr.m) {
+          *reinterpret_cast<float4*>(c) = make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
+          *reinterpret_cast<float4*>(c + 4) = make_float4(acc[4][q], acc[5][q], acc[6][q], acc[7][q]);
+        } else {
 #pragma unroll
-      for (int j = 0; j < TN; ++j)
-        if (ng0 + j < pr.n && ng0 + j >= mg) { c[j] = o[j]; C[(int64_t)(ng0 + j) * pr.ldc + mg] = o[j]; }
-      continue;
-    }
-    if (quad) *reinterpret_cast<float4*>(c) = *reinterpret_cast<const float4*>(o);
-    else
-#pragma unroll
-      for (int j = 0; j < TN; ++j) if (ng0 + j < pr.n) c[j] = o[j];
-  }
-  if (pr.epi == EPI_SYMM && tm != tn) {
-    // the mirror image: a thread's eight rows are eight consecutive entries of each of its four columns' rows
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      if (ng0 + j >= pr.n) continue;
-      float* c = C + (int64_t)(ng0 + j) * pr.ldc + mg0;
-      if (vec_c && mg0 + TM <= pr.m) {
-        *reinterpret_cast<float4*>(c) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
-        *reinterpret_cast<float4*>(c + 4) = make_float4(acc[4][j], acc[5][j], acc[6][j], acc[7][j]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < TM; ++i) if (mg0 + i < pr.m) c[i] = acc[i][j];
+          for (int i = 0; i < TM; ++i) if (mg0 + i < pr.m) c[i] = acc[i][q];
+        }
       }
     }
   }
@@ -278,24 +367,24 @@ __global__ void __launch_bounds__(NT * KG) gemm_ffma_kernel(const __grid_constan
   if (bad && pr.nonfinite) *pr.nonfinite = 1;
 }
 
-template <int KG, int CAP>
+template <int TN, bool AKM, int KG, int CAP>
 cudaError_t launch(const GemmGroup& g, int total, cudaStream_t s) {
   static SmemAttrCache attr;
-  const size_t part = (KG - 1) * (size_t)(TM * TN * NT + BM), slabs = (size_t)KG * 2 * kSlab;
+  const size_t part = (KG - 1) * (size_t)(BM * BN + BM), slabs = (size_t)KG * kStages * kSlab;
   const size_t smem = (part > slabs ? part : slabs) * sizeof(float);
-  cudaError_t e = ensure_dyn_smem(gemm_ffma_kernel<KG, CAP>, smem, attr);
+  cudaError_t e = ensure_dyn_smem(gemm_ffma_kernel<TN, AKM, KG, CAP>, smem, attr);
   if (e != cudaSuccess) return e;
   GemmBlock<CAP> b;
   b.n = g.n;
   memcpy(b.p, g.p, g.n * sizeof(GemmProblem));
-  gemm_ffma_kernel<KG, CAP><<<total, NT * KG, smem, s>>>(b);
+  gemm_ffma_kernel<TN, AKM, KG, CAP><<<total, Shape<TN>::NT * KG, smem, s>>>(b);
   return cudaGetLastError();
 }
-template <int KG>
+template <int TN, bool AKM, int KG>
 cudaError_t launch_cap(const GemmGroup& g, int total, cudaStream_t s) {
-  if (g.n <= 2) return launch<KG, 2>(g, total, s);
-  if (g.n <= 16) return launch<KG, 16>(g, total, s);
-  return launch<KG, FW_MAX_GROUP>(g, total, s);
+  if (g.n <= 2) return launch<TN, AKM, KG, 2>(g, total, s);
+  if (g.n <= 16) return launch<TN, AKM, KG, 16>(g, total, s);
+  return launch<TN, AKM, KG, FW_MAX_GROUP>(g, total, s);
 }
 
 bool quads(const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; }
@@ -319,11 +408,17 @@ cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class) {
   g.total_ctas = total;
   if (total == 0) return cudaSuccess;
   ProfScope ps(prof_class, s);
-  // groups per tile: with six resident CTAs of one group an SM has all the warps it can use, so from four CTAs per SM on
-  // one group suffices; below, the tile's chain is shared
-  if (total >= 4 * 148) return launch_cap<1>(g, total, s);
-  if (total >= 2 * 148) return launch_cap<2>(g, total, s);
-  return launch_cap<4>(g, total, s);
+  // A launch's problems all have the same kind of A.  Groups per tile: an SM holds eight groups of 64 threads (four of
+  // 128); with fewer tiles than that the chain of a tile is shared, and below one tile per SM it is what counts, so the
+  // groups have 128 threads there.
+  if (!g.p[0].a_kmajor) {
+    if (total >= 4 * 148) return launch_cap<4, false, 1>(g, total, s);
+    return launch_cap<4, false, 4>(g, total, s);
+  }
+  if (total >= 6 * 148) return launch_cap<8, true, 1>(g, total, s);
+  if (total >= 3 * 148) return launch_cap<8, true, 2>(g, total, s);
+  if (total >= 148) return launch_cap<8, true, 4>(g, total, s);
+  return launch_cap<4, true, 4>(g, total, s);
 }
 
 }  // namespace fw

@@ -201,6 +201,8 @@ struct ProfScope {
 // ---------------------------------------------------------------------------
 // launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
+// CTAs of a launch of the FFMA GEMM that are resident together on a B200 (eight groups of 64 threads per SM)
+constexpr int kFfmaResident = 8 * 148;
 cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class);
 // to_pmean != 0: the means go to the layers' pmean vectors instead of their shift vectors
 cudaError_t launch_pilot_mean(const GroupDev& g, const PtrTable& X, const Rows64& rows, const Rows64& ldx,
