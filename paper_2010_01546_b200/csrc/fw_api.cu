@@ -782,8 +782,7 @@ fw_status fw_whiten_backward(fw_layer* L, const float* dY, int64_t rows, float* 
 fw_status fw_step(fw_layer* L, float* W, float* b, const float* G_t, const float* g_b, float lr) {
   if (!L || !W || !G_t) return FW_ERR_INVALID_ARG;
   if ((b == nullptr) != (g_b == nullptr)) return FW_ERR_INVALID_ARG;
-  FW_CUDA(launch_axpy_step(W, G_t, lr, (int64_t)L->d.N * L->d.M, L->stream), "step W");
-  if (b) FW_CUDA(launch_sgd_bias(b, g_b, lr, L->d.N, L->stream), "step b");
+  FW_CUDA(launch_sgd_step(W, G_t, (int64_t)L->d.N * L->d.M, b, g_b, L->d.N, lr, L->stream), "step");
   return FW_OK;
 }
 
@@ -792,9 +791,8 @@ fw_status fw_step_momentum(fw_layer* L, float* W, float* b, const float* G_t, co
   if (!L || !W || !G_t || !vW) return FW_ERR_INVALID_ARG;
   if (!((b == nullptr) == (g_b == nullptr) && (b == nullptr) == (vb == nullptr))) return FW_ERR_INVALID_ARG;
   if (!(momentum >= 0.f && momentum < 1.f) || !(weight_decay >= 0.f)) return FW_ERR_INVALID_ARG;
-  FW_CUDA(launch_momentum_step(W, G_t, vW, lr, momentum, weight_decay, (int64_t)L->d.N * L->d.M, L->stream),
-          "momentum step W");
-  if (b) FW_CUDA(launch_momentum_step(b, g_b, vb, lr, momentum, 0.f, L->d.N, L->stream), "momentum step b");
+  FW_CUDA(launch_momentum_step(W, G_t, vW, (int64_t)L->d.N * L->d.M, b, g_b, vb, L->d.N, lr, momentum, weight_decay, L->stream),
+          "momentum step");
   return FW_OK;
 }
 

@@ -250,13 +250,13 @@ cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s
 // out[j] = sum_k A[k][j] x[k] for a row-major M x M matrix A (A^T x)
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s);
 cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s);
-cudaError_t launch_sgd_bias(float* b, const float* gb, float lr, int N, cudaStream_t s);
 cudaError_t launch_sgd_bias_group(const GroupDev& g, const PtrTable& b, const PtrTable& gb, float lr, int max_N,
                                   cudaStream_t s);
-cudaError_t launch_axpy_step(float* W, const float* G, float lr, int64_t n, cudaStream_t s);
-// v <- momentum v + (G + wd W); W <- W - lr v
-cudaError_t launch_momentum_step(float* W, const float* G, float* v, float lr, float momentum, float wd, int64_t n,
-                                 cudaStream_t s);
+// W <- W - lr G; b <- b - lr gb unless b is null
+cudaError_t launch_sgd_step(float* W, const float* G, int64_t n, float* b, const float* gb, int N, float lr, cudaStream_t s);
+// v <- momentum v + (G + wd W); W <- W - lr v; the same with wd = 0 for b, gb, vb unless b is null
+cudaError_t launch_momentum_step(float* W, const float* G, float* v, int64_t n, float* b, const float* gb, float* vb, int N,
+                                 float lr, float momentum, float wd, cudaStream_t s);
 // rho = M / sum_ij A_ij^2 / (A_ii A_jj) of a symmetric M x M matrix, one float
 cudaError_t launch_whiteness(const float* A, int M, float* out, cudaStream_t s);
 

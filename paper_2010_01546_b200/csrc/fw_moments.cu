@@ -289,33 +289,44 @@ __device__ __forceinline__ void bias_comp_rows(const LayerDev* L, const float* W
   if (lane == 0) bp[row] += acc;
 }
 
-// Zero-padded copies of NHWC activations: dst[b][y + 1][x + 1][:] = src[b][y][x][:], one pixel of zeros all round,
-// for every layer of a group in one launch.  One thread per 16 bytes of the destinations (flat over the layers).
+// Zero-padded copies of NHWC activations: dst[b][y + 1][x + 1][:] = src[b][y][x][:], one pixel of zeros all round, for
+// every layer of a group in one launch.  A warp takes a padded image row at a time, so that its place in the tensors is
+// found once per row; all 16-byte loads of four trips are in flight before the first store.
 struct PadGroup {
   const float4* src[FW_MAX_GROUP];
   float4* dst[FW_MAX_GROUP];
-  int64_t first4[FW_MAX_GROUP + 1];   // first 16-byte unit of each layer in the flat index space
-  int32_t B[FW_MAX_GROUP], H[FW_MAX_GROUP], W[FW_MAX_GROUP], C4[FW_MAX_GROUP];
+  int32_t row0[FW_MAX_GROUP + 1];     // first padded row of each layer in the flat list of rows
+  int32_t H[FW_MAX_GROUP], W4[FW_MAX_GROUP], C4[FW_MAX_GROUP];   // W4: 16-byte units of an unpadded row
+  int32_t tail[FW_MAX_GROUP];         // units past the padded tensor that the last window may read: zeros
   int32_t n;
 };
 __global__ void __launch_bounds__(256) pad_nhwc_kernel(const __grid_constant__ PadGroup g) {
-  const int64_t total4 = g.first4[g.n];
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total4; e += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31, nw = gridDim.x * 8, total = g.row0[g.n];
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int w = blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += nw) {
     int li = 0;
 #pragma unroll 1
     for (int i = 1; i < g.n; ++i)
-      if (e >= g.first4[i]) li = i;
-    const int64_t l = e - g.first4[li];
-    const int C4 = g.C4[li], W = g.W[li], H = g.H[li];
-    const int c = (int)(l % C4);
-    int64_t p = l / C4;
-    const int xp = (int)(p % (W + 2)); p /= (W + 2);
-    const int yp = (int)(p % (H + 2));
-    const int64_t b = p / (H + 2);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (xp >= 1 && xp <= W && yp >= 1 && yp <= H && b < g.B[li])
-      v = g.src[li][((b * H + (yp - 1)) * W + (xp - 1)) * C4 + c];
-    g.dst[li][l] = v;
+      if (w >= g.row0[i]) li = i;
+    const int r = w - g.row0[li], H = g.H[li], W4 = g.W4[li], C4 = g.C4[li];
+    const int b = r / (H + 2), y = r - b * (H + 2);
+    const int len = W4 + 2 * C4;
+    float4* d = g.dst[li] + (int64_t)r * len;
+    const bool border = y == 0 || y == H + 1;
+    const float4* s = g.src[li] + ((int64_t)b * H + (y - 1)) * W4 - C4;      // unit c of the padded row is s[c] inside
+    for (int c0 = lane; c0 < len; c0 += 128) {
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = c0 + 32 * u;
+        v[u] = !border && c >= C4 && c < len - C4 ? __ldg(s + c) : z;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (c0 + 32 * u < len) d[c0 + 32 * u] = v[u];
+    }
+    if (w + 1 == g.row0[li + 1])
+      for (int c = lane; c < g.tail[li]; c += 32) d[len + c] = z;
   }
 }
 
@@ -358,14 +369,24 @@ __global__ void transpose_kernel(const float* __restrict__ src, float* __restric
   }
 }
 
-// out = A^T x: one thread per column, rows in order (coalesced across the columns)
-__global__ void __launch_bounds__(256) matT_vec_kernel(const float* __restrict__ A, const float* __restrict__ x,
-                                                       float* __restrict__ out, int M) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= M) return;
+// out = A^T x: 32 columns per CTA, the rows dealt to its 32 warps and their sums added in order
+__global__ void __launch_bounds__(1024) matT_vec_kernel(const float* __restrict__ A, const float* __restrict__ x,
+                                                        float* __restrict__ out, int M) {
+  __shared__ float sm[32][33];
+  const int j = blockIdx.x * 32 + threadIdx.x;
   float acc = 0.f;
-  for (int k = 0; k < M; ++k) acc = fmaf(A[(int64_t)k * M + j], x[k], acc);
-  out[j] = acc;
+  if (j < M) {
+#pragma unroll 4
+    for (int k = threadIdx.y; k < M; k += 32) acc = fmaf(A[(int64_t)k * M + j], x[k], acc);
+  }
+  sm[threadIdx.y][threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.y == 0 && j < M) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) t += sm[i][threadIdx.x];
+    out[j] = t;
+  }
 }
 
 // lam_bar = trace(Phix) / M after a covariance has been injected
@@ -383,11 +404,6 @@ __global__ void __launch_bounds__(256) trace_lambda_kernel(const LayerDev* L) {
   if (threadIdx.x == 0) L->scal[SC_LAMBDA_BAR] = red[0] / (float)M;
 }
 
-__global__ void sgd_bias_kernel(float* b, const float* gb, float lr, int N) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < N) b[i] = fmaf(-lr, gb[i], b[i]);
-}
-
 // b <- b - lr g_b for every layer of a group; grid (ceil(max N / 256), layers)
 __global__ void sgd_bias_group_kernel(const __grid_constant__ GroupDev g, const __grid_constant__ PtrTable b,
                                       const __grid_constant__ PtrTable gb, float lr) {
@@ -398,19 +414,31 @@ __global__ void sgd_bias_group_kernel(const __grid_constant__ GroupDev g, const 
   if (bp && gp && i < L->N) bp[i] = fmaf(-lr, gp[i], bp[i]);
 }
 
-__global__ void axpy_step_kernel(float* __restrict__ W, const float* __restrict__ G, float lr, int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    W[e] = fmaf(-lr, G[e], W[e]);
+// W <- W - lr G and b <- b - lr g_b (b may be null) in one launch
+__global__ void __launch_bounds__(256) sgd_step_kernel(float* __restrict__ W, const float* __restrict__ G, int64_t n,
+                                                       float* __restrict__ b, const float* __restrict__ gb, int N, float lr) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = first; e < n; e += step) W[e] = fmaf(-lr, G[e], W[e]);
+  if (b)
+    for (int64_t e = first; e < N; e += step) b[e] = fmaf(-lr, gb[e], b[e]);
 }
 
-__global__ void momentum_step_kernel(float* __restrict__ W, const float* __restrict__ G, float* __restrict__ v,
-                                     float lr, float momentum, float wd, int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const float w = W[e];
-    const float vn = fmaf(momentum, v[e], fmaf(wd, w, G[e]));
-    v[e] = vn;
-    W[e] = fmaf(-lr, vn, w);
-  }
+// v <- momentum v + (G + wd W), W <- W - lr v, and the same without decay for the bias (may be null), in one launch
+__device__ __forceinline__ void momentum_entry(float* __restrict__ W, const float* __restrict__ G, float* __restrict__ v,
+                                               int64_t e, float lr, float momentum, float wd) {
+  const float w = W[e];
+  const float vn = fmaf(momentum, v[e], fmaf(wd, w, G[e]));
+  v[e] = vn;
+  W[e] = fmaf(-lr, vn, w);
+}
+__global__ void __launch_bounds__(256) momentum_step_kernel(float* __restrict__ W, const float* __restrict__ G,
+                                                            float* __restrict__ v, int64_t n, float* __restrict__ b,
+                                                            const float* __restrict__ gb, float* __restrict__ vb, int N,
+                                                            float lr, float momentum, float wd) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = first; e < n; e += step) momentum_entry(W, G, v, e, lr, momentum, wd);
+  if (b)
+    for (int64_t e = first; e < N; e += step) momentum_entry(b, gb, vb, e, lr, momentum, 0.f);
 }
 
 // Eq. 51 over all index pairs.  One CTA; every thread sums its rows in fp64, fixed-order tree over the block.
@@ -437,13 +465,15 @@ __global__ void __launch_bounds__(1024) whiteness_kernel(const float* __restrict
 
 }  // namespace
 
-cudaError_t launch_momentum_step(float* W, const float* G, float* v, float lr, float momentum, float wd, int64_t n,
-                                 cudaStream_t s) {
-  int blocks = (int)((n + 1023) / 1024);
-  if (blocks > 2368) blocks = 2368;
-  if (blocks < 1) blocks = 1;
+static int step_blocks(int64_t n) {
+  const int64_t blocks = (n + 255) / 256;
+  return (int)(blocks > 2368 ? 2368 : (blocks < 1 ? 1 : blocks));
+}
+
+cudaError_t launch_momentum_step(float* W, const float* G, float* v, int64_t n, float* b, const float* gb, float* vb, int N,
+                                 float lr, float momentum, float wd, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  momentum_step_kernel<<<blocks, 256, 0, s>>>(W, G, v, lr, momentum, wd, n);
+  momentum_step_kernel<<<step_blocks(n), 256, 0, s>>>(W, G, v, n, b, gb, vb, N, lr, momentum, wd);
   return cudaGetLastError();
 }
 
@@ -498,19 +528,20 @@ cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, c
   // dst_floats covers the padded tensor plus the slack the last window may read past it: all of it is written
   PadGroup g;
   memset(&g, 0, sizeof(g));
-  int64_t total4 = 0;
+  int rows = 0;
   for (int i = 0; i < n; ++i) {
     g.src[i] = reinterpret_cast<const float4*>(src[i]); g.dst[i] = reinterpret_cast<float4*>(dst[i]);
-    g.B[i] = B[i]; g.H[i] = H[i]; g.W[i] = W[i]; g.C4[i] = C[i] / 4;
-    g.first4[i] = total4;
-    total4 += dst_floats[i] / 4;
+    g.H[i] = H[i]; g.C4[i] = C[i] / 4; g.W4[i] = W[i] * (C[i] / 4);
+    g.tail[i] = (int)(dst_floats[i] / 4 - (int64_t)B[i] * (H[i] + 2) * (g.W4[i] + 2 * g.C4[i]));
+    g.row0[i] = rows;
+    rows += B[i] * (H[i] + 2);
   }
-  g.first4[n] = total4;
+  g.row0[n] = rows;
   g.n = n;
-  int64_t blocks = (total4 + 255) / 256;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  int blocks = (rows + 7) / 8;
+  if (blocks > 148 * 8) blocks = 148 * 8;
   ProfScope ps(FW_PROF_PILOT, s);
-  pad_nhwc_kernel<<<(int)blocks, 256, 0, s>>>(g);
+  pad_nhwc_kernel<<<blocks, 256, 0, s>>>(g);
   return cudaGetLastError();
 }
 
@@ -532,7 +563,7 @@ cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s
 
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  matT_vec_kernel<<<(M + 255) / 256, 256, 0, s>>>(A, x, out, M);
+  matT_vec_kernel<<<(M + 31) / 32, dim3(32, 32), 0, s>>>(A, x, out, M);
   return cudaGetLastError();
 }
 
@@ -543,12 +574,6 @@ cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_sgd_bias(float* b, const float* gb, float lr, int N, cudaStream_t s) {
-  ProfScope ps(FW_PROF_MISC, s);
-  sgd_bias_kernel<<<(N + 255) / 256, 256, 0, s>>>(b, gb, lr, N);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_sgd_bias_group(const GroupDev& g, const PtrTable& b, const PtrTable& gb, float lr, int max_N,
                                   cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
@@ -556,12 +581,9 @@ cudaError_t launch_sgd_bias_group(const GroupDev& g, const PtrTable& b, const Pt
   return cudaGetLastError();
 }
 
-cudaError_t launch_axpy_step(float* W, const float* G, float lr, int64_t n, cudaStream_t s) {
-  int blocks = (int)((n + 1023) / 1024);
-  if (blocks > 2368) blocks = 2368;
-  if (blocks < 1) blocks = 1;
+cudaError_t launch_sgd_step(float* W, const float* G, int64_t n, float* b, const float* gb, int N, float lr, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  axpy_step_kernel<<<blocks, 256, 0, s>>>(W, G, lr, n);
+  sgd_step_kernel<<<step_blocks(n), 256, 0, s>>>(W, G, n, b, gb, N, lr);
   return cudaGetLastError();
 }
 

@@ -552,6 +552,227 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
   }
 }
 
+// ---- layers of at most 64 features: one CTA, a row on 8 lanes ----
+// No exchange leaves the CTA, so a pass is its own latency: a row on 8 lanes takes three shuffle rounds instead of five,
+// every lane has work, and one block barrier ends it (M = 64: 0.26 us a power iteration, 0.46 with four rows per warp;
+// at 128 features, 4 lanes per row were no faster than that).
+constexpr int LPR = 8;                           // lanes per row: 64 rows on 512 threads
+__device__ __forceinline__ float row_sum(float x) {
+#pragma unroll
+  for (int o = LPR / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+__device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int K, int P, bool smooth) {
+  constexpr int KM = 64 / (4 * LPR);             // float4 per lane
+  const int tid = threadIdx.x, row = tid / LPR, sub = tid % LPR;
+  const int M = s.M, M4 = s.Mp >> 2;
+  float4 a[KM];
+#pragma unroll
+  for (int k = 0; k < KM; ++k) {
+    const int c = sub + LPR * k;
+    a[k] = row < s.R && c < M4 ? reinterpret_cast<const float4*>(csm + row * s.Mp)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // y = scale (row . x) into dst; NORM: scale = 1 / ||x||, returns ||x||^2
+  auto dot = [&](const float* x, float scale, bool norm, float* dst) {
+    const float4* x4 = reinterpret_cast<const float4*>(x);
+    float d0 = 0.f, d1 = 0.f, n0 = 0.f, n1 = 0.f;
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      const float4 b = x4[sub + LPR * k];
+      d0 = fmaf(a[k].x, b.x, d0); d1 = fmaf(a[k].y, b.y, d1); d0 = fmaf(a[k].z, b.z, d0); d1 = fmaf(a[k].w, b.w, d1);
+      if (norm) { n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1); n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1); }
+    }
+    float n2 = 0.f;
+    if (norm) { n2 = row_sum(n0 + n1); scale = inv_norm(n2); }
+    const float d = row_sum(d0 + d1);
+    if (sub == 0) dst[row] = d * scale;
+    return n2;
+  };
+  for (int k0 = 0; k0 < K; k0 += KH) {
+    const int k1 = min(K, k0 + KH);
+    for (int step = k0; step < k1; ++step) {
+      // squared norms (Eq. 45), m' (Eq. 46): every warp finds it for itself
+      float q0 = 0.f, q1 = 0.f;
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        q0 = fmaf(a[k].x, a[k].x, q0); q1 = fmaf(a[k].y, a[k].y, q1); q0 = fmaf(a[k].z, a[k].z, q0); q1 = fmaf(a[k].w, a[k].w, q1);
+      }
+      q0 = row_sum(q0 + q1);
+      if (sub == 0) csm[s.xi2 + row] = q0;
+      __syncthreads();
+      const int mp = argmax_xi(s);
+      if (row == mp) {
+#pragma unroll
+        for (int k = 0; k < KM; ++k) reinterpret_cast<float4*>(csm + s.wvec)[sub + LPR * k] = a[k];
+      }
+      __syncthreads();
+      dot(csm + s.wvec, 1.f, false, csm + s.cvec);                       // Eq. 47
+      __syncthreads();
+      // coherent set, aligned average (Eqs. 48-49)
+      int cnt = 1;
+      {
+        float wv = 0.f;
+        bool in = false;
+        if (s.maxcol) {
+          wv = tid == mp ? 1.f : 0.f;
+        } else if (tid < M) {
+          const float c = csm[s.cvec + tid];
+          const float thr = fmaxf(s.c_rel * sqrtf(csm[s.xi2 + mp]) * sqrtf(csm[s.xi2 + tid]), s.c_abs);
+          in = fabsf(c) >= thr;       // false for NaN
+          wv = in ? (1.f / c) : 0.f;
+        }
+        if (tid < 64) csm[s.wvec + tid] = wv;
+        const int n = __syncthreads_count(in);
+        if (!s.maxcol) cnt = n;
+      }
+      int xo = s.buf0, yo = xo + s.Mv;
+      dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, false, csm + xo);
+      __syncthreads();
+      for (int p = 0; p < P; ++p) {
+        dot(csm + xo, 0.f, true, csm + yo);
+        __syncthreads();
+        const int t = xo; xo = yo; yo = t;
+      }
+      const float n2 = dot(csm + xo, 0.f, true, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
+      const float inv = inv_norm(n2);
+      __syncthreads();
+      const float4* x4 = reinterpret_cast<const float4*>(csm + xo);
+      const float4* u4 = reinterpret_cast<const float4*>(csm + s.uvec);
+      float l0 = 0.f, l1 = 0.f;
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const float4 x = x4[sub + LPR * k], u = u4[sub + LPR * k];
+        l0 = fmaf(x.x * inv, u.x, l0); l1 = fmaf(x.y * inv, u.y, l1); l0 = fmaf(x.z * inv, u.z, l0); l1 = fmaf(x.w * inv, u.w, l1);
+      }
+      const float lam_e = row_sum(l0 + l1);                         // Eq. 36
+      const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
+      float g_e = 1.f, aa = 0.f;
+      if (ok) {
+        g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);                 // Eqs. 40-41
+        aa = sqrtf(g_e) - 1.f;
+      }
+      // Phi_y += v w^T + w v^T, w = a u + (a^2 lambda_e / 2) v, as in run_steps
+      if (aa != 0.f) {
+        const float hl = 0.5f * aa * aa * lam_e;
+        const float vi = csm[xo + row] * inv, wi = __fadd_rn(__fmul_rn(aa, csm[s.uvec + row]), __fmul_rn(hl, vi));
+#pragma unroll
+        for (int k = 0; k < KM; ++k) {
+          float4 v = x4[sub + LPR * k], w = u4[sub + LPR * k];
+          v.x *= inv; v.y *= inv; v.z *= inv; v.w *= inv;
+          w.x = __fadd_rn(__fmul_rn(aa, w.x), __fmul_rn(hl, v.x)); w.y = __fadd_rn(__fmul_rn(aa, w.y), __fmul_rn(hl, v.y));
+          w.z = __fadd_rn(__fmul_rn(aa, w.z), __fmul_rn(hl, v.z)); w.w = __fadd_rn(__fmul_rn(aa, w.w), __fmul_rn(hl, v.w));
+          a[k].x = __fadd_rn(a[k].x, __fadd_rn(__fmul_rn(vi, w.x), __fmul_rn(wi, v.x)));
+          a[k].y = __fadd_rn(a[k].y, __fadd_rn(__fmul_rn(vi, w.y), __fmul_rn(wi, v.y)));
+          a[k].z = __fadd_rn(a[k].z, __fadd_rn(__fmul_rn(vi, w.z), __fmul_rn(wi, v.z)));
+          a[k].w = __fadd_rn(a[k].w, __fadd_rn(__fmul_rn(vi, w.w), __fmul_rn(wi, v.w)));
+        }
+      }
+      if (tid < 64) csm[s.vh + (step - k0) * s.Mv + tid] = csm[xo + tid] * inv;
+      if (tid == 0) {
+        s.ah[step - k0] = aa;
+        if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
+        if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
+        if (tr) {
+          tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
+        }
+        if (step + 1 == K) {
+          L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
+          L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
+        }
+      }
+      __syncthreads();
+    }
+    // ---- the recorded steps in T, then Q (Eqs. 42, 44), as in apply_steps ----
+    const bool last = k1 == K;
+    float4 t[KM];
+    auto load = [&](float4 (&r)[KM], const float* G) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const int c = 4 * (sub + LPR * k);
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        if (row < M && c < M) {
+          const float* p = G + (size_t)row * M + c;
+          if ((M & 3) == 0) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(p);
+          else
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (c + e < M) x[e] = p[e];
+        }
+        r[k] = make_float4(x[0], x[1], x[2], x[3]);
+      }
+    };
+    auto save = [&](const float4 (&r)[KM], float* G) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const int c = 4 * (sub + LPR * k);
+        if (row < M && c < M) {
+          float* p = G + (size_t)row * M + c;
+          if ((M & 3) == 0) *reinterpret_cast<float4*>(p) = r[k];
+          else {
+            p[0] = r[k].x;
+            if (c + 1 < M) p[1] = r[k].y;
+            if (c + 2 < M) p[2] = r[k].z;
+            if (c + 3 < M) p[3] = r[k].w;
+          }
+        }
+      }
+    };
+    load(t, L->Tt);
+#pragma unroll 1
+    for (int j = 0; j < k1 - k0; ++j) {
+      const float ak = s.ah[j];
+      if (ak == 0.f) continue;
+      const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + j * s.Mv);
+      float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const float4 b = v4[sub + LPR * k];
+        d0 = fmaf(t[k].x, b.x, d0); d1 = fmaf(t[k].y, b.y, d1); d0 = fmaf(t[k].z, b.z, d0); d1 = fmaf(t[k].w, b.w, d1);
+      }
+      const float d = row_sum(d0 + d1), at = ak * d;
+      if (sub == 0) csm[s.th + j * s.Mv + row] = d;
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const float4 b = v4[sub + LPR * k];
+        t[k].x = fmaf(at, b.x, t[k].x); t[k].y = fmaf(at, b.y, t[k].y); t[k].z = fmaf(at, b.z, t[k].z); t[k].w = fmaf(at, b.w, t[k].w);
+      }
+    }
+    save(t, L->Tt);
+    load(t, L->Q);
+    __syncthreads();
+#pragma unroll 1
+    for (int j = 0; j < k1 - k0; ++j) {
+      const float ak = s.ah[j];
+      if (ak == 0.f) continue;
+      const float aq = ak * (ak + 2.f), ti = csm[s.th + j * s.Mv + row];
+      const float4* t4 = reinterpret_cast<const float4*>(csm + s.th + j * s.Mv);
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        const float4 b = t4[sub + LPR * k];
+        t[k].x = __fadd_rn(t[k].x, __fmul_rn(aq, __fmul_rn(ti, b.x))); t[k].y = __fadd_rn(t[k].y, __fmul_rn(aq, __fmul_rn(ti, b.y)));
+        t[k].z = __fadd_rn(t[k].z, __fmul_rn(aq, __fmul_rn(ti, b.z))); t[k].w = __fadd_rn(t[k].w, __fmul_rn(aq, __fmul_rn(ti, b.w)));
+      }
+    }
+    save(t, L->Q);
+    if (last && smooth) {
+      const float beta = L->beta, ob = 1.f - beta;
+      float4 o[KM];
+      load(o, L->Qs);
+#pragma unroll
+      for (int k = 0; k < KM; ++k) {
+        o[k].x = fmaf(beta, o[k].x, ob * t[k].x); o[k].y = fmaf(beta, o[k].y, ob * t[k].y);
+        o[k].z = fmaf(beta, o[k].z, ob * t[k].z); o[k].w = fmaf(beta, o[k].w, ob * t[k].w);
+      }
+      save(o, L->Qs);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < KM; ++k) {
+    const int c = sub + LPR * k;
+    if (row < s.R && c < M4) reinterpret_cast<float4*>(csm + row * s.Mp)[c] = a[k];
+  }
+}
+
 // groups of four rows this warp owns in a slab of R rows
 __device__ __forceinline__ int warp_groups(int R) {
   const int warp = threadIdx.x >> 5, ng = R >> 2;
@@ -565,6 +786,8 @@ __host__ __device__ inline int slab_vec(int M, int n) {
   return a > b ? a : b;
 }
 constexpr int kVecs = 6 + 2 * KH;
+// one CTA with a row on 8 lanes
+__host__ __device__ inline bool solo(int M, int n) { return n == 1 && M <= 64; }
 
 template <int NG, int IT>
 __device__ __forceinline__ void run_chunk(Slab& s, const Link& l, const LayerDev* L, float* tr, int k0, int k1, int P,
@@ -647,6 +870,10 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
 
   if (usable) {
     float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
+    if (solo(M, l.n)) {
+      const bool smooth = L->Qs != L->Q;
+      run_solo(s, L, tr, a.K, a.P, smooth);
+    } else {
     const int it = slab_trips(M), ng = warp_groups(R);
     uint32_t e = 0;                        // exchanges so far
     for (int k0 = 0; k0 < a.K; k0 += KH) {
@@ -667,6 +894,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
         }
       }
       e += (uint32_t)(k1 - k0) * (uint32_t)(a.P + 5) + 1u;
+    }
     }
   }
   __syncthreads();
@@ -702,6 +930,7 @@ bool cluster_fits(int M, int n) {
 // the work of the busiest of the four SM partitions, and the fixed part of an exchange (less within one CTA).
 int cluster_cost(int M, int n) {
   const int groups = slab_rows(M, n) / 4;
+  if (solo(M, n)) return 4;
   return ((groups + 3) / 4) * slab_trips(M) + (n > 1 ? 20 : 8);
 }
 
