@@ -409,6 +409,7 @@ constexpr int kBase = 4;           // weights of the identity in the three outpu
 // lambda_m = |w_m|, with the sign of the Rayleigh quotient (one row of Phi suffices: w_m is parallel to v_m) where the
 // eigenvectors are wanted; a warp per column
 __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ FinishArgs a) {
+  dep_sync();
   int li = 0;
 #pragma unroll 1
   for (int i = 1; i < a.nl; ++i)
@@ -459,6 +460,7 @@ __device__ double block_sum_d(double x, double* red) {
 // One CTA per layer: ranks of the eigenvalues, the rank estimate (Eq. 32 read as exp(-sum lbar log lbar)) and the gains.
 // The sums decide an integer (the rank): their order does not depend on the launch.
 __global__ void __launch_bounds__(1024) evd_finish_kernel(const __grid_constant__ FinishArgs a) {
+  dep_sync();
   __shared__ double red[32];
   const EvdLayer L = a.l[blockIdx.x];
   const int M = L.M;
@@ -525,6 +527,7 @@ struct VdvArgs {
 // the upper triangle and writes its mirror image too, so the outputs are exactly symmetric.  A warp takes 16 x 32.
 constexpr int VT = 64, VK = 16, kVs = VT + 4;
 __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArgs a) {
+  dep_sync();
   int li = 0;
 #pragma unroll 1
   for (int i = 1; i < a.nl; ++i)
@@ -692,19 +695,19 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
   }
   {
     ProfScope ps(FW_PROF_MISC, s);
-    norm_kernel<<<blocks, 256, 0, s>>>(f);
+    launch_dep(norm_kernel, blocks, 256, 0, s, f);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   {
     ProfScope ps(FW_PROF_MISC, s);
-    evd_finish_kernel<<<n, 1024, 0, s>>>(f);
+    launch_dep(evd_finish_kernel, n, 1024, 0, s, f);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (with_v) {
     ProfScope ps(FW_PROF_MISC, s);
-    vdv_kernel<<<tiles, 256, 0, s>>>(v);
+    launch_dep(vdv_kernel, tiles, 256, 0, s, v);
     e = cudaGetLastError();
   }
   return e;

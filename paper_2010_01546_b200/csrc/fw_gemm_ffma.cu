@@ -141,6 +141,7 @@ extern __shared__ __align__(16) float gsm[];
 // AKM: A is K-major (copied asynchronously); else M-major, TN = 4
 template <int TN, bool AKM, int KG, int CAP>
 __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm_ffma_kernel(const __grid_constant__ GemmBlock<CAP> g) {
+  dep_sync();
   constexpr int NT = Shape<TN>::NT;
   // locate the problem this CTA works on
   const int cta = blockIdx.x;
@@ -377,7 +378,7 @@ cudaError_t launch(const GemmGroup& g, int total, cudaStream_t s) {
   GemmBlock<CAP> b;
   b.n = g.n;
   memcpy(b.p, g.p, g.n * sizeof(GemmProblem));
-  gemm_ffma_kernel<TN, AKM, KG, CAP><<<total, Shape<TN>::NT * KG, smem, s>>>(b);
+  launch_dep(gemm_ffma_kernel<TN, AKM, KG, CAP>, total, Shape<TN>::NT * KG, smem, s, b);
   return cudaGetLastError();
 }
 template <int TN, bool AKM, int KG>

@@ -19,6 +19,7 @@ constexpr int kPilotTY = 16;        // row lanes per block
 __global__ void pilot_mean_kernel(const __grid_constant__ GroupDev g, const __grid_constant__ PtrTable X,
                                   const __grid_constant__ Rows64 rows, const __grid_constant__ Rows64 ldx,
                                   int in_bf16, int to_pmean) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.y];
   const int M = L->M;
   const int col = blockIdx.x * 32 + threadIdx.x;
@@ -61,6 +62,7 @@ struct MomentArgs {
 __global__ void __launch_bounds__(1024) moments_vec_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.x];
   const int M = L->M;
   const int S = a.splits[blockIdx.x];
@@ -160,6 +162,7 @@ __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant_
                                                           const __grid_constant__ MomentArgs a,
                                                           const __grid_constant__ PtrTable W,
                                                           const __grid_constant__ PtrTable b) {
+  dep_sync();
   const int nbias = a.bias_blocks * g.n;
   if ((int)blockIdx.x < nbias) {
     // the first CTAs carry the bias compensation (Eq. 31), which needs the means only: long rows of W start early
@@ -241,6 +244,7 @@ __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant_
 // upper-triangle 32x32 tiles as moments_mat_kernel; the CTAs of a layer's first tile row also carry the column sums.
 __global__ void __launch_bounds__(256) accumulate_kernel(const __grid_constant__ GroupDev g,
                                                          const __grid_constant__ MomentArgs a) {
+  dep_sync();
   const int tile_id = (int)blockIdx.x;
   int li = 0;
 #pragma unroll 1
@@ -301,6 +305,7 @@ struct PadGroup {
   int32_t n;
 };
 __global__ void __launch_bounds__(256) pad_nhwc_kernel(const __grid_constant__ PadGroup g) {
+  dep_sync();
   const int lane = threadIdx.x & 31, nw = gridDim.x * 8, total = g.row0[g.n];
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int w = blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += nw) {
@@ -331,6 +336,7 @@ __global__ void __launch_bounds__(256) pad_nhwc_kernel(const __grid_constant__ P
 }
 
 __global__ void init_identity_kernel(const LayerDev* L) {
+  dep_sync();
   const int M = L->M;
   const int64_t n = (int64_t)M * M;
   const bool alias = (L->Qs == L->Q);
@@ -354,6 +360,7 @@ __global__ void init_identity_kernel(const LayerDev* L) {
 }
 
 __global__ void transpose_kernel(const float* __restrict__ src, float* __restrict__ dst, int M) {
+  dep_sync();
   __shared__ float tile[32][33];
   const int bi = blockIdx.y * 32, bj = blockIdx.x * 32;
 #pragma unroll
@@ -372,6 +379,7 @@ __global__ void transpose_kernel(const float* __restrict__ src, float* __restric
 // out = A^T x: 32 columns per CTA, the rows dealt to its 32 warps and their sums added in order
 __global__ void __launch_bounds__(1024) matT_vec_kernel(const float* __restrict__ A, const float* __restrict__ x,
                                                         float* __restrict__ out, int M) {
+  dep_sync();
   __shared__ float sm[32][33];
   const int j = blockIdx.x * 32 + threadIdx.x;
   float acc = 0.f;
@@ -391,6 +399,7 @@ __global__ void __launch_bounds__(1024) matT_vec_kernel(const float* __restrict_
 
 // lam_bar = trace(Phix) / M after a covariance has been injected
 __global__ void __launch_bounds__(256) trace_lambda_kernel(const LayerDev* L) {
+  dep_sync();
   const int M = L->M;
   float s = 0.f;
   for (int m = threadIdx.x; m < M; m += blockDim.x) s += L->Phix[(int64_t)m * M + m];
@@ -407,6 +416,7 @@ __global__ void __launch_bounds__(256) trace_lambda_kernel(const LayerDev* L) {
 // b <- b - lr g_b for every layer of a group; grid (ceil(max N / 256), layers)
 __global__ void sgd_bias_group_kernel(const __grid_constant__ GroupDev g, const __grid_constant__ PtrTable b,
                                       const __grid_constant__ PtrTable gb, float lr) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.y];
   float* bp = const_cast<float*>(reinterpret_cast<const float*>(b.p[blockIdx.y]));
   const float* gp = reinterpret_cast<const float*>(gb.p[blockIdx.y]);
@@ -417,6 +427,7 @@ __global__ void sgd_bias_group_kernel(const __grid_constant__ GroupDev g, const 
 // W <- W - lr G and b <- b - lr g_b (b may be null) in one launch
 __global__ void __launch_bounds__(256) sgd_step_kernel(float* __restrict__ W, const float* __restrict__ G, int64_t n,
                                                        float* __restrict__ b, const float* __restrict__ gb, int N, float lr) {
+  dep_sync();
   const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = first; e < n; e += step) W[e] = fmaf(-lr, G[e], W[e]);
   if (b)
@@ -435,6 +446,7 @@ __global__ void __launch_bounds__(256) momentum_step_kernel(float* __restrict__ 
                                                             float* __restrict__ v, int64_t n, float* __restrict__ b,
                                                             const float* __restrict__ gb, float* __restrict__ vb, int N,
                                                             float lr, float momentum, float wd) {
+  dep_sync();
   const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
   for (int64_t e = first; e < n; e += step) momentum_entry(W, G, v, e, lr, momentum, wd);
   if (b)
@@ -443,6 +455,7 @@ __global__ void __launch_bounds__(256) momentum_step_kernel(float* __restrict__ 
 
 // Eq. 51 over all index pairs.  One CTA; every thread sums its rows in fp64, fixed-order tree over the block.
 __global__ void __launch_bounds__(1024) whiteness_kernel(const float* __restrict__ A, int M, float* __restrict__ out) {
+  dep_sync();
   double acc = 0.0;
   for (int i = threadIdx.x >> 5; i < M; i += 32) {          // a warp per row
     const double dii = A[(int64_t)i * M + i];
@@ -473,13 +486,13 @@ static int step_blocks(int64_t n) {
 cudaError_t launch_momentum_step(float* W, const float* G, float* v, int64_t n, float* b, const float* gb, float* vb, int N,
                                  float lr, float momentum, float wd, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  momentum_step_kernel<<<step_blocks(n), 256, 0, s>>>(W, G, v, n, b, gb, vb, N, lr, momentum, wd);
+  launch_dep(momentum_step_kernel, step_blocks(n), 256, 0, s, W, G, v, n, b, gb, vb, N, lr, momentum, wd);
   return cudaGetLastError();
 }
 
 cudaError_t launch_whiteness(const float* A, int M, float* out, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  whiteness_kernel<<<1, 1024, 0, s>>>(A, M, out);
+  launch_dep(whiteness_kernel, 1, 1024, 0, s, A, M, out);
   return cudaGetLastError();
 }
 
@@ -487,7 +500,7 @@ cudaError_t launch_pilot_mean(const GroupDev& g, const PtrTable& X, const Rows64
                               int in_bf16, int max_M, int to_pmean, cudaStream_t s) {
   dim3 grid((max_M + 31) / 32, g.n), block(32, kPilotTY);
   ProfScope ps(FW_PROF_PILOT, s);
-  pilot_mean_kernel<<<grid, block, 0, s>>>(g, X, rows, ldx, in_bf16, to_pmean);
+  launch_dep(pilot_mean_kernel, grid, block, 0, s, g, X, rows, ldx, in_bf16, to_pmean);
   return cudaGetLastError();
 }
 
@@ -498,7 +511,7 @@ cudaError_t launch_accumulate(const GroupDev& g, const int32_t* splits, const in
   for (int i = 0; i < g.n; ++i) { a.splits[i] = splits[i]; a.use_acc[i] = fresh[i] ? 0 : 1; a.corr[i] = corr[i]; }
   const int total = fill_tile_table(a.tt, layer_M, g.n);
   ProfScope ps(FW_PROF_MOMENTS, s);
-  accumulate_kernel<<<total, dim3(32, 8), 0, s>>>(g, a);
+  launch_dep(accumulate_kernel, total, dim3(32, 8), 0, s, g, a);
   return cudaGetLastError();
 }
 
@@ -511,14 +524,14 @@ cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t*
   for (int i = 0; i < g.n; ++i) {
     a.splits[i] = splits[i]; a.first[i] = first[i]; a.use_acc[i] = use_acc[i]; a.corr[i] = corr[i];
   }
-  { ProfScope ps(FW_PROF_MOMENTS, s); moments_vec_kernel<<<g.n, 1024, 0, s>>>(g, rows, a); }
+  { ProfScope ps(FW_PROF_MOMENTS, s); launch_dep(moments_vec_kernel, g.n, 1024, 0, s, g, rows, a); }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int total = fill_tile_table(a.tt, layer_M, g.n);
   a.bias_blocks = any_params ? (max_N + 7) / 8 : 0;
   {
     ProfScope ps(FW_PROF_MOMENTS, s);
-    moments_mat_kernel<<<total + a.bias_blocks * g.n, dim3(32, 8), 0, s>>>(g, rows, a, W, b);
+    launch_dep(moments_mat_kernel, total + a.bias_blocks * g.n, dim3(32, 8), 0, s, g, rows, a, W, b);
   }
   return cudaGetLastError();
 }
@@ -541,7 +554,7 @@ cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, c
   int blocks = (rows + 7) / 8;
   if (blocks > 148 * 8) blocks = 148 * 8;
   ProfScope ps(FW_PROF_PILOT, s);
-  pad_nhwc_kernel<<<blocks, 256, 0, s>>>(g);
+  launch_dep(pad_nhwc_kernel, blocks, 256, 0, s, g);
   return cudaGetLastError();
 }
 
@@ -550,40 +563,40 @@ cudaError_t launch_init_identity(const LayerDev* dev, int M, cudaStream_t s) {
   int blocks = (int)((n + 255) / 256);
   if (blocks > 1184) blocks = 1184;
   ProfScope ps(FW_PROF_MISC, s);
-  init_identity_kernel<<<blocks, 256, 0, s>>>(dev);
+  launch_dep(init_identity_kernel, blocks, 256, 0, s, dev);
   return cudaGetLastError();
 }
 
 cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s) {
   const int t = (M + 31) / 32;
   ProfScope ps(FW_PROF_MISC, s);
-  transpose_kernel<<<dim3(t, t), dim3(32, 8), 0, s>>>(src, dst, M);
+  launch_dep(transpose_kernel, dim3(t, t), dim3(32, 8), 0, s, src, dst, M);
   return cudaGetLastError();
 }
 
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  matT_vec_kernel<<<(M + 31) / 32, dim3(32, 32), 0, s>>>(A, x, out, M);
+  launch_dep(matT_vec_kernel, (M + 31) / 32, dim3(32, 32), 0, s, A, x, out, M);
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s) {
   (void)M;
   ProfScope ps(FW_PROF_MISC, s);
-  trace_lambda_kernel<<<1, 256, 0, s>>>(dev);
+  launch_dep(trace_lambda_kernel, 1, 256, 0, s, dev);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sgd_bias_group(const GroupDev& g, const PtrTable& b, const PtrTable& gb, float lr, int max_N,
                                   cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  sgd_bias_group_kernel<<<dim3((max_N + 255) / 256, g.n), 256, 0, s>>>(g, b, gb, lr);
+  launch_dep(sgd_bias_group_kernel, dim3((max_N + 255) / 256, g.n), 256, 0, s, g, b, gb, lr);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sgd_step(float* W, const float* G, int64_t n, float* b, const float* gb, int N, float lr, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  sgd_step_kernel<<<step_blocks(n), 256, 0, s>>>(W, G, n, b, gb, N, lr);
+  launch_dep(sgd_step_kernel, step_blocks(n), 256, 0, s, W, G, n, b, gb, N, lr);
   return cudaGetLastError();
 }
 

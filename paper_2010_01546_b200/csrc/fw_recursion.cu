@@ -121,6 +121,7 @@ extern __shared__ __align__(16) float smem_x[];
 template <int PASS, int R, int C>
 __global__ void __launch_bounds__(kGemvThreads, (C == 1) ? 4 : 2) recursion_pass_kernel(const __grid_constant__ GroupDev g,
                                                                       int src_slot, int dst_slot) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.y];
   const int M = L->M;
   constexpr int RBk = WARPS * R;                // rows per CTA of this shape
@@ -313,6 +314,7 @@ __global__ void __launch_bounds__(kGemvThreads, (C == 1) ? 4 : 2) recursion_pass
 __global__ void __launch_bounds__(kGemvThreads) recursion_scalars_kernel(const __grid_constant__ GroupDev g,
                                                                          const __grid_constant__ PtrTable traces,
                                                                          int step, int pass_rows) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.x];
   const int nblk = (L->M + pass_rows - 1) / pass_rows;   // partials of lambda_e: one per CTA of the FINAL pass
   __shared__ float red[WARPS];
@@ -344,6 +346,7 @@ __global__ void __launch_bounds__(kGemvThreads) recursion_scalars_kernel(const _
 // T + T^T and P + P^T need the transposed element, so a CTA owns the pair of 32x32 tiles (bi, bj), (bj, bi).
 // Q and Phiy are computed for the upper tile and mirrored, which keeps them exactly symmetric.
 __global__ void __launch_bounds__(256) recursion_update_leaky_kernel(const __grid_constant__ GroupDev g) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.z];
   const float gm = L->gamma;
   const int M = L->M;
@@ -415,6 +418,7 @@ __global__ void __launch_bounds__(256) recursion_update_leaky_kernel(const __gri
 
 // Qs <- beta Qs + (1 - beta) Q   (Eq. 35)
 __global__ void __launch_bounds__(256) smooth_kernel(const __grid_constant__ GroupDev g) {
+  dep_sync();
   const LayerDev* L = g.layer[blockIdx.y];
   if (L->Qs == L->Q) return;
   const int64_t n = (int64_t)L->M * L->M;
@@ -432,22 +436,22 @@ static cudaError_t recursion_step_launches(const GroupDev& g, int P, int step, c
   const int nblk = (max_M + RBk - 1) / RBk;
   const size_t shm = (size_t)((max_M + 3) & ~3) * sizeof(float);
   dim3 grid(nblk, g.n), block(kGemvThreads);
-  { ProfScope ps(FW_PROF_RECUR_MV, s); recursion_pass_kernel<PASS_ROWNORM, R, C><<<grid, block, shm, s>>>(g, 0, 0); }
-  { ProfScope ps(FW_PROF_RECUR_MV, s); recursion_pass_kernel<PASS_CORR, R, C><<<grid, block, shm, s>>>(g, 0, 0); }
-  { ProfScope ps(FW_PROF_RECUR_MV, s); recursion_pass_kernel<PASS_ALIGN, R, C><<<grid, block, shm, s>>>(g, 0, 0); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_ROWNORM, R, C>, grid, block, shm, s, g, 0, 0); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_CORR, R, C>, grid, block, shm, s, g, 0, 0); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_ALIGN, R, C>, grid, block, shm, s, g, 0, 0); }
   int cur = 0;
   for (int p = 0; p < P; ++p) {
     ProfScope ps(FW_PROF_RECUR_MV, s);
-    recursion_pass_kernel<PASS_POWER, R, C><<<grid, block, shm, s>>>(g, cur, cur ^ 1);
+    launch_dep(recursion_pass_kernel<PASS_POWER, R, C>, grid, block, shm, s, g, cur, cur ^ 1);
     cur ^= 1;
   }
   dim3 grid2(nblk, g.n, 3);
-  { ProfScope ps(FW_PROF_RECUR_MV, s); recursion_pass_kernel<PASS_FINAL, R, C><<<grid2, block, shm, s>>>(g, cur, 0); }
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); recursion_scalars_kernel<<<g.n, block, 0, s>>>(g, traces, step, RBk); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_FINAL, R, C>, grid2, block, shm, s, g, cur, 0); }
+  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(recursion_scalars_kernel, g.n, block, 0, s, g, traces, step, RBk); }
   {
     const int t32 = (max_M + 31) / 32;
     ProfScope ps(FW_PROF_RECUR_UPD, s);
-    recursion_update_leaky_kernel<<<dim3(t32, t32, g.n), dim3(32, 8), 0, s>>>(g);
+    launch_dep(recursion_update_leaky_kernel, dim3(t32, t32, g.n), dim3(32, 8), 0, s, g);
   }
   return cudaGetLastError();
 }
@@ -471,7 +475,7 @@ cudaError_t launch_smooth(const GroupDev& g, int max_M, cudaStream_t s) {
   if (bx > 1184) bx = 1184;
   if (bx < 1) bx = 1;
   ProfScope ps(FW_PROF_SMOOTH, s);
-  smooth_kernel<<<dim3(bx, g.n), 256, 0, s>>>(g);
+  launch_dep(smooth_kernel, dim3(bx, g.n), 256, 0, s, g);
   return cudaGetLastError();
 }
 

@@ -107,6 +107,7 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
 
 // rows of M <= 1280 take a warp each; longer rows a CTA each
 __global__ void __launch_bounds__(AT) apply_t_kernel(const __grid_constant__ ApplyArgs a) {
+  dep_sync();
   __shared__ double red[AWARPS];
   const int li = apply_layer(a, (int)blockIdx.x);
   const LayerDev* L = a.g.layer[li];
@@ -191,6 +192,7 @@ __device__ __forceinline__ void q_tile(const LayerDev* L, int row0, int c, int K
 }
 
 __global__ void __launch_bounds__(AT) apply_q_kernel(const __grid_constant__ ApplyArgs a) {
+  dep_sync();
   const int li = apply_layer(a, (int)blockIdx.x);
   const LayerDev* L = a.g.layer[li];
   const int M = L->M;
@@ -222,7 +224,7 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
     n += layer_M[i] > kWarpRowMax ? layer_M[i] : (layer_M[i] + AWARPS - 1) / AWARPS;
   }
   a.block0[g.n] = n;
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); apply_t_kernel<<<n, AT, 0, s>>>(a); }
+  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(apply_t_kernel, n, AT, 0, s, a); }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   n = 0;
@@ -237,7 +239,7 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
     }
   }
   a.block0[g.n] = n;
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); apply_q_kernel<<<n, AT, 0, s>>>(a); }
+  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(apply_q_kernel, n, AT, 0, s, a); }
   return cudaGetLastError();
 }
 

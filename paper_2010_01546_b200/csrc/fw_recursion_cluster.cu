@@ -799,6 +799,7 @@ __device__ __forceinline__ void run_chunk(Slab& s, const Link& l, const LayerDev
 }
 
 __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
+  dep_sync();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int lane = threadIdx.x & 31;
@@ -1017,10 +1018,12 @@ cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, 
     cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = smem; cfg.stream = s;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // as launch_dep
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 2;
   };
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   {
     std::lock_guard<std::mutex> lock(mu);
     if (resident[dev][0] == 0) {

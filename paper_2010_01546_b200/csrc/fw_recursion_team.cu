@@ -591,6 +591,7 @@ __host__ __device__ inline int team_cache(int M, int R) {
 }
 
 __global__ void __launch_bounds__(PT, 1) recursion_team_kernel(const __grid_constant__ TeamArgs a) {
+  dep_sync();
   __shared__ Shared sh;
   if (threadIdx.x == 0) sh.fail = 0;
   for (int w = 0; w < a.nwaves; ++w) {

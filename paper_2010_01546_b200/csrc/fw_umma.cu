@@ -258,6 +258,7 @@ __device__ __forceinline__ float tf32_rna(float x) {
 // their loops is on the critical path of the pipeline.
 template <bool BF>
 __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_constant__ GramGroup g) {
+  dep_sync();
   constexpr int RB = BF ? 64 : 128;               // bytes per chunk row
   constexpr int KROWS = BF ? 16 : 8;              // rows of X one MMA contracts over
   constexpr uint64_t LAYOUT = BF ? kSwizzle64B : kSwizzle128B32;
@@ -1018,8 +1019,8 @@ fw_status umma_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
     }
     g.n = cnt;
     ProfScope ps(FW_PROF_GRAM, s);
-    if (group_bf16) gram_umma_kernel<true><<<total_ctas, GR_THREADS, smem, s>>>(g);
-    else gram_umma_kernel<false><<<total_ctas, GR_THREADS, smem, s>>>(g);
+    if (group_bf16) launch_dep(gram_umma_kernel<true>, total_ctas, GR_THREADS, smem, s, g);
+    else launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_umma_kernel launch: %s\n", cudaGetErrorString(e));
@@ -1097,7 +1098,7 @@ fw_status umma_atb_launch(const UmmaAtbItem* items, int n, cudaStream_t s) {
     }
     g.n = cnt;
     ProfScope ps(FW_PROF_RESYNC, s);
-    gram_umma_kernel<false><<<total_ctas, GR_THREADS, smem, s>>>(g);
+    launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_umma_kernel (A^T B) launch: %s\n", cudaGetErrorString(e));

@@ -77,6 +77,7 @@ struct QpGroup {
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(QP_THREADS, 1)
 gq_pair_kernel(const __grid_constant__ QpGroup g) {
+  dep_sync();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[QP_STAGES], bar_empty[QP_STAGES], bar_accum;
   __shared__ uint32_t tmem_base_sh;
@@ -262,6 +263,7 @@ struct QrProblem {
 struct QrGroup { QrProblem p[QP_MAX_PROBLEMS]; int32_t n; int32_t pad; int64_t total4; };
 
 __global__ void __launch_bounds__(256) gq_reduce_kernel(const __grid_constant__ QrGroup g) {
+  dep_sync();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < g.total4; e += (int64_t)gridDim.x * blockDim.x) {
     int pi = 0;
 #pragma unroll 1
@@ -411,7 +413,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     g.n = cnt; g.nitems = (int)nitems;
     {
       ProfScope ps(prof_class, s);
-      gq_pair_kernel<<<2 * g.nitems, QP_THREADS, smem, s>>>(g);
+      launch_dep(gq_pair_kernel, 2 * g.nitems, QP_THREADS, smem, s, g);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -422,7 +424,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
       int64_t blocks = (gr.total4 + 255) / 256;
       if (blocks > 148 * 8) blocks = 148 * 8;
       ProfScope ps(prof_class, s);
-      gq_reduce_kernel<<<(int)blocks, 256, 0, s>>>(gr);
+      launch_dep(gq_reduce_kernel, (int)blocks, 256, 0, s, gr);
       e = cudaGetLastError();
       if (e != cudaSuccess) {
         fprintf(stderr, "[fw] gq_reduce_kernel launch: %s\n", cudaGetErrorString(e));

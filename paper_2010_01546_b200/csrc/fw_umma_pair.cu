@@ -116,6 +116,7 @@ __device__ __forceinline__ float tf32_rna(float x) {
 template <bool BF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 gram_pair_kernel(const __grid_constant__ PairGroup g) {
+  dep_sync();
   // Chunk rows are 128 bytes for both element types (TMA fetches whole 128-byte lines):
   //   fp32: 32 columns, 128-byte swizzle with 32-byte atoms, K-atoms of 4 rows;
   //   bf16: 64 columns, 128-byte swizzle (16-byte units), K-atoms of 8 rows.
@@ -715,8 +716,8 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
     for (size_t i = 0; i < items.size(); ++i) g.item[i] = items[i].code;
     g.n = cnt; g.nitems = (int)items.size();
     ProfScope ps(prof_class, s);
-    if (specs[base].bf16) gram_pair_kernel<true><<<2 * g.nitems, GP_THREADS, smem, s>>>(g);
-    else gram_pair_kernel<false><<<2 * g.nitems, GP_THREADS, smem, s>>>(g);
+    if (specs[base].bf16) launch_dep(gram_pair_kernel<true>, 2 * g.nitems, GP_THREADS, smem, s, g);
+    else launch_dep(gram_pair_kernel<false>, 2 * g.nitems, GP_THREADS, smem, s, g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_pair_kernel launch: %s\n", cudaGetErrorString(e));
