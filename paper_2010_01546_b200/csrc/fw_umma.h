@@ -28,7 +28,7 @@ struct UmmaGqItem {
   int64_t part_floats;
   const float* colbias;  // optional, length M: subtracted from every row of the product
 };
-// out = G Qs on CTA pairs (256 x 512 tiles, K split with a fixed-order reduction); M a multiple of 4, >= 16
+// out = G Qs on CTA pairs (256 x 256 tiles, K split with a fixed-order reduction); M a multiple of 4, >= 16
 bool umma_gq_pair_supported(int M);
 fw_status umma_gq_pair_launch(const UmmaGqItem* items, int n, int epi, float lr, int prof_class, cudaStream_t s);
 // K-major fp32 operand: 2-D row-major [outer][inner] tensor, boxes of box_inner (32) floats x box_outer rows,

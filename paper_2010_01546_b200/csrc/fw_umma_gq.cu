@@ -4,19 +4,23 @@
 //
 // Shape of the problem.  out[n][m] = sum_k G[n][k] B[k][m]; N (rows of G) runs from 16 to hundreds of thousands,
 // M from 64 to 4608.  The tile is computed as D = B^T G^T: the MMA's 256 rows (128 per CTA of the pair) are 256
-// values of m, its columns are up to 512 values of n in two accumulators of up to 256 (all 512 TMEM columns of
-// both CTAs), the contraction runs over k.
+// values of m, its columns are up to 256 values of n, the contraction runs over k.
 //   A operand: B[k][m], m contiguous: MN-major chunks of 32 columns laid down by TMA (as in the Gram kernels);
 //              each CTA stages its own 128 values of m: 16 KB per 32-row stage.
 //   B operand: G[n][k], k contiguous: K-major, 128-byte swizzle, rows of 32 floats; each CTA stages its half of
-//              each panel (up to 128 rows of G): 16 KB per accumulator per stage.
-// A CTA therefore stages 48 KB for 128 x 512 x 32 multiply-adds -- the 48 bytes per tensor clock that the TMA
-// sustains -- where one CTA per 128 x 256 tile staged twice that per multiply-add.
+//              the tile's rows of G (up to 128): 16 KB per stage.
+// What bounds it: with K = M of a few hundred a tile is 10-20 k steps, no longer than its set-up and epilogue.  The
+// grid is one CTA pair per pair of SMs, each walking over its items; half of tensor memory holds the tile the tensor
+// cores work on, the other half the tile before it, which the epilogue warps store meanwhile, and the producer runs
+// up to six stages ahead across tiles.  (Tiles of 256 x 512, one per launched pair and all of tensor memory, moved
+// less through L2 -- 48 bytes staged per tensor clock against 64 -- but had nothing to overlap their epilogue with:
+// 32768 rows at M = 576 took 100 us, and take 56.)  What bounds it then is the traffic between L2 and the SMs, about
+// 45 of its 64 bytes a clock per SM: 8 us a tile at M = 512, of which the tensor cores work 4.3.
 //
 // K is split over `ksplit` items per tile when the tiles alone would not fill the machine; split s writes its
 // partial tile to a scratch buffer and a second kernel adds the partials in split order (the same order in every
 // run) and applies the epilogue.  Items are numbered problem-major, the problems in order of decreasing item
-// length, and a CTA pair finds its (problem, tile, split) from its index.
+// length; pair c of C takes items c, c + C, ... and finds the (problem, tile, split) of each from its number.
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (even CTA only) and TMEM owner, warps 2..9 epilogue.
 // Both CTAs' loads complete on the even CTA's "full" barrier; tcgen05.commit multicasts the "stage free" and
@@ -28,6 +32,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <vector>
 
 #include "fw_sm100.cuh"
@@ -42,13 +47,15 @@ namespace {
 constexpr int QP_SR = 32;                 // k rows per stage
 constexpr int QP_KSTEPS = QP_SR / 8;      // TF32 MMAs contract over 8
 constexpr int QP_A_BYTES = 4 * QP_SR * 128;       // 4 chunks of 32 columns: 16 KB
-constexpr int QP_B_BYTES = 128 * QP_SR * 4;       // 128 rows of G x 32 floats: 16 KB per accumulator
-constexpr int QP_STAGE = QP_A_BYTES + 2 * QP_B_BYTES;   // 48 KB
-constexpr int QP_STAGES = 4;
+constexpr int QP_NT = 256;                // rows of G per tile: half of tensor memory
+constexpr int QP_B_BYTES = QP_NT / 2 * QP_SR * 4; // 128 rows of G x 32 floats: 16 KB
+constexpr int QP_STAGE = QP_A_BYTES + QP_B_BYTES; // 32 KB
+constexpr int QP_STAGES = 6;
 constexpr int QP_THREADS = 64 + 8 * 32;
 constexpr int QP_SMEM = QP_STAGES * QP_STAGE;
 constexpr int QP_MAX_PROBLEMS = 16;
-constexpr int QP_MAX_ITEMS = 1 << 20;    // items of one launch (the grid is twice that)
+constexpr int QP_PAIRS = 74;              // CTA pairs of a full grid
+constexpr int QP_MAX_ITEMS = 1 << 20;    // items of one launch
 constexpr int QP_MAX_KSPLIT = 8;
 
 struct QpProblem {
@@ -60,7 +67,8 @@ struct QpProblem {
   int64_t N;               // rows of G
   int32_t M;
   int32_t ksplit, kb_per;  // splits, k blocks (of 32) per split
-  int32_t ntiles_n;        // tiles along n (512 rows of G each)
+  int32_t ntiles_n;        // tiles along n (QP_NT rows of G each)
+  int32_t ntiles_m;        // tiles along m; 0: tiles are numbered along n first
   int32_t epi;             // EPI_STORE / EPI_SGD
   int32_t use3d;           // mapA is the chunked 3-D view (M a multiple of 32), else one-chunk 2-D boxes
   float lr;
@@ -75,45 +83,59 @@ struct QpGroup {
   int32_t n, nitems;
 };
 
+// what one CTA does for item `item`
+struct QpItem {
+  int pi, split, kb0, nk;  // problem, K split, first k block and number of k blocks
+  int m_cta;               // first value of m this CTA holds
+  int nall;                // columns of the tile, a multiple of 16
+  int64_t n_base;          // first row of G of the tile
+};
+__device__ __forceinline__ QpItem qp_item(const QpGroup& g, int item, int rank) {
+  QpItem r;
+  r.pi = 0;
+#pragma unroll 1
+  for (int i = 1; i < g.n; ++i)
+    if (item >= g.p[i].first_item) r.pi = i;
+  const QpProblem& pr = g.p[r.pi];
+  const int local = item - pr.first_item;
+  const int tile = local / pr.ksplit;
+  r.split = local - tile * pr.ksplit;
+  const int I = pr.ntiles_m > 0 ? tile % pr.ntiles_m : tile / pr.ntiles_n;
+  const int t = pr.ntiles_m > 0 ? tile / pr.ntiles_m : tile - I * pr.ntiles_n;
+  r.n_base = (int64_t)t * QP_NT;
+  const int64_t nrem = pr.N - r.n_base;
+  r.nall = ((int)(nrem < QP_NT ? nrem : QP_NT) + 15) & ~15;
+  r.m_cta = 256 * I + 128 * rank;
+  const int nkb_all = (pr.M + QP_SR - 1) / QP_SR;
+  r.kb0 = r.split * pr.kb_per;
+  r.nk = min(nkb_all, r.kb0 + pr.kb_per) - r.kb0;      // at least 1
+  return r;
+}
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(QP_THREADS, 1)
 gq_pair_kernel(const __grid_constant__ QpGroup g) {
-  dep_sync();
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bar_full[QP_STAGES], bar_empty[QP_STAGES], bar_accum;
+  __shared__ __align__(8) uint64_t bar_full[QP_STAGES], bar_empty[QP_STAGES], bar_accum[2], bar_drained[2];
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const int item = (int)(blockIdx.x >> 1);
-  int pi = 0;
-#pragma unroll 1
-  for (int i = 1; i < g.n; ++i)
-    if (item >= g.p[i].first_item) pi = i;
-  const QpProblem& pr = g.p[pi];
-  const int local = item - pr.first_item;
-  const int tile = local / pr.ksplit, split = local - tile * pr.ksplit;
-  const int M = pr.M;
-  const int I = tile / pr.ntiles_n, t = tile - I * pr.ntiles_n;
-  const int64_t n_base = (int64_t)t * 512;
-  int64_t nrem = pr.N - n_base;
-  if (nrem > 512) nrem = 512;
-  const int nall = ((int)nrem + 15) & ~15;          // columns of this tile, a multiple of 16
-  const int n0 = nall < 256 ? nall : 256;
-  const int n1 = nall - n0;
-  const int m_cta = 256 * I + 128 * (int)rank;       // first value of m this CTA holds
-  uint32_t ncols = 32;
-  while ((int)ncols < nall) ncols <<= 1;
+  const int item0 = (int)(blockIdx.x >> 1), step = (int)(gridDim.x >> 1);
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < QP_STAGES; ++s) { mbar_init(smem_u32(&bar_full[s]), 1); mbar_init(smem_u32(&bar_empty[s]), 1); }
-    mbar_init(smem_u32(&bar_accum), 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&bar_accum[b]), 1);
+      mbar_init(smem_u32(&bar_drained[b]), 16);        // the epilogue warps of both CTAs, on the even CTA's barrier
+    }
     mbar_fence_init();
   }
+  dep_sync();
   __syncthreads();
   if (warp == 1) {
-    tmem_alloc_pair(smem_u32(&tmem_base_sh), ncols);
+    tmem_alloc_pair(smem_u32(&tmem_base_sh), 2 * QP_NT);
     tmem_relinquish_pair();
   }
   tc_fence_before();
@@ -128,120 +150,134 @@ gq_pair_kernel(const __grid_constant__ QpGroup g) {
   do {                                      \
     abort_flag = 1;                         \
     st_cluster_u32(peer_abort, 1u);         \
-    atomicExch(pr.status, (code));          \
+    atomicExch(g.p[it.pi].status, (code));  \
   } while (0)
 
-  // k blocks of this split
-  const int nkb_all = (M + QP_SR - 1) / QP_SR;
-  const int kb0 = min(nkb_all, split * pr.kb_per), kb1 = min(nkb_all, kb0 + pr.kb_per);
-  const int nk = kb1 - kb0;
-  // bytes both CTAs deliver per stage: A always, one or two B panels
-  const uint32_t tx_cta = (uint32_t)QP_A_BYTES + (uint32_t)QP_B_BYTES * (n1 > 0 ? 2u : 1u);
-
   if (warp == 0) {
-    // ---- TMA producer (both CTAs).  Lane 0..3: the A chunks (or lane 0 alone with the 3-D map), lanes 4, 5: the
-    //      two B panels; all loads of a stage are issued together ----
-    if (lane == 0) {
-      tma_prefetch_desc(&g.mapA[pi]);
-      tma_prefetch_desc(&g.mapB[pi]);
-    }
-    const bool issue_a = pr.use3d ? (lane == 0) : (lane < 4);
-    const bool issue_b = (lane == 4) || (lane == 5 && n1 > 0);
-    // rows of G this CTA stages for the panel: its half of the panel's n0 (n1) rows
-    const int64_t brow = n_base + (lane == 4 ? (int64_t)rank * (n0 / 2) : 256 + (int64_t)rank * (n1 / 2));
+    // ---- TMA producer (both CTAs).  Lane 0..3: the A chunks (or lane 0 alone with the 3-D map), lane 4: the rows
+    //      of G; all loads of a stage are issued together ----
     int s = 0;
     uint32_t ph = 0, sb = smem_base;
-    for (int kb = 0; kb < nk; ++kb) {
-      const bool got = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1, abortp);
-      if (!__all_sync(0xffffffffu, got)) { if (lane == 0) QP_ABORT(401); break; }
-      const uint32_t bar = mapa_shared(smem_u32(&bar_full[s]), 0u);       // counted on the even CTA's barrier
-      if (lane == 0 && rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * tx_cta);
-      const int k = (kb0 + kb) * QP_SR;
-      if (issue_a) {
-        if (pr.use3d) tma_load_3d_pair(sb, &g.mapA[pi], 0, k, m_cta / 32, bar);
-        else tma_load_2d_pair(sb + (uint32_t)lane * (QP_SR * 128), &g.mapA[pi], m_cta + lane * 32, k, bar);
+    bool ok = true;
+    for (int item = item0; item < g.nitems && ok; item += step) {
+      const QpItem it = qp_item(g, item, (int)rank);
+      const bool use3d = g.p[it.pi].use3d != 0;
+      const bool issue_a = use3d ? (lane == 0) : (lane < 4);
+      const int64_t brow = it.n_base + (int64_t)rank * (it.nall / 2);     // this CTA's half of the tile's rows of G
+      for (int kb = 0; kb < it.nk; ++kb) {
+        const bool got = mbar_wait(smem_u32(&bar_empty[s]), ph ^ 1, abortp);
+        if (!__all_sync(0xffffffffu, got)) { if (lane == 0) QP_ABORT(401); ok = false; break; }
+        const uint32_t bar = mapa_shared(smem_u32(&bar_full[s]), 0u);       // counted on the even CTA's barrier
+        if (lane == 0 && rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * (uint32_t)QP_STAGE);
+        const int k = (it.kb0 + kb) * QP_SR;
+        if (issue_a) {
+          if (use3d) tma_load_3d_pair(sb, &g.mapA[it.pi], 0, k, it.m_cta / 32, bar);
+          else tma_load_2d_pair(sb + (uint32_t)lane * (QP_SR * 128), &g.mapA[it.pi], it.m_cta + lane * 32, k, bar);
+        }
+        if (lane == 4) tma_load_2d_pair(sb + QP_A_BYTES, &g.mapB[it.pi], k, (int)brow, bar);
+        sb += QP_STAGE;
+        if (++s == QP_STAGES) { s = 0; ph ^= 1; sb = smem_base; }
       }
-      if (issue_b) tma_load_2d_pair(sb + QP_A_BYTES + (lane == 5 ? QP_B_BYTES : 0), &g.mapB[pi], k, (int)brow, bar);
-      sb += QP_STAGE;
-      if (++s == QP_STAGES) { s = 0; ph ^= 1; sb = smem_base; }
     }
   } else if (warp == 1) {
     // ---- MMA issuer: one thread of the even CTA drives the tensor cores of both SMs ----
     if (rank == 0 && elect_one()) {
       const uint64_t ad = make_smem_desc(smem_base, QP_SR * 128, 512, kSwizzle128B32);           // MN-major chunks
-      const uint64_t bd0 = make_smem_desc(smem_base + QP_A_BYTES, 16, 1024, kSwizzle128B);        // K-major rows
-      const uint64_t bd1 = make_smem_desc(smem_base + QP_A_BYTES + QP_B_BYTES, 16, 1024, kSwizzle128B);
-      const uint32_t id0 = make_idesc(2, (uint32_t)n0, 1, 0, 256u);
-      const uint32_t id1 = make_idesc(2, (uint32_t)(n1 > 0 ? n1 : 16), 1, 0, 256u);
-      int s = 0;
-      uint32_t ph = 0, soff16 = 0;
-      uint32_t accum = 0;
-      for (int kb = 0; kb < nk; ++kb) {
-        if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { QP_ABORT(402); break; }
+      const uint64_t bd = make_smem_desc(smem_base + QP_A_BYTES, 16, 1024, kSwizzle128B);         // K-major rows
+      int s = 0, b = 0;
+      uint32_t ph = 0, soff16 = 0, bph = 0;
+      bool ok = true;
+      for (int item = item0; item < g.nitems && ok; item += step) {
+        const QpItem it = qp_item(g, item, 0);
+        const uint32_t id = make_idesc(2, (uint32_t)it.nall, 1, 0, 256u);
+        const uint32_t acc = tmem_base + (uint32_t)(b * QP_NT);
+        if (!mbar_wait(smem_u32(&bar_drained[b]), bph ^ 1, abortp)) { QP_ABORT(404); break; }
         tc_fence_after();
+        for (int kb = 0; kb < it.nk; ++kb) {
+          if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { QP_ABORT(402); ok = false; break; }
+          tc_fence_after();
 #pragma unroll
-        for (int ks = 0; ks < QP_KSTEPS; ++ks) {
-          const uint64_t aoff = (uint64_t)(soff16 + ks * 64);     // 8 rows of 128 bytes
-          const uint64_t boff = (uint64_t)(soff16 + ks * 2);      // 8 floats inside the swizzled 128-byte rows
-          mma_tf32_pair(tmem_base, ad + aoff, bd0 + boff, id0, accum);
-          if (n1 > 0) mma_tf32_pair(tmem_base + 256u, ad + aoff, bd1 + boff, id1, accum);
-          accum = 1;
+          for (int ks = 0; ks < QP_KSTEPS; ++ks) {
+            const uint64_t aoff = (uint64_t)(soff16 + ks * 64);     // 8 rows of 128 bytes
+            const uint64_t boff = (uint64_t)(soff16 + ks * 2);      // 8 floats inside the swizzled 128-byte rows
+            mma_tf32_pair(acc, ad + aoff, bd + boff, id, (uint32_t)(kb + ks > 0));
+          }
+          mma_commit_pair(smem_u32(&bar_empty[s]), (uint16_t)3);
+          soff16 += QP_STAGE >> 4;
+          if (++s == QP_STAGES) { s = 0; ph ^= 1; soff16 = 0; }
         }
-        mma_commit_pair(smem_u32(&bar_empty[s]), (uint16_t)3);
-        soff16 += QP_STAGE >> 4;
-        if (++s == QP_STAGES) { s = 0; ph ^= 1; soff16 = 0; }
+        mma_commit_pair(smem_u32(&bar_accum[b]), (uint16_t)3);
+        b ^= 1;
+        if (b == 0) bph ^= 1;
       }
-      mma_commit_pair(smem_u32(&bar_accum), (uint16_t)3);
     }
   } else {
     // ---- epilogue: this CTA's 128 values of m (TMEM lanes) x the tile's columns n ----
-    const int w = warp - 2;
-    const int q = warp & 3, half = w >> 2;
-    const int m = m_cta + q * 32 + lane;
-    const bool have = nk > 0;
-    bool bad = false;
-    if (!have || mbar_wait(smem_u32(&bar_accum), 0, abortp)) {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    int b = 0;
+    uint32_t bph = 0;
+    for (int item = item0; item < g.nitems; item += step) {
+      const QpItem it = qp_item(g, item, (int)rank);
+      const QpProblem& pr = g.p[it.pi];
+      const int M = pr.M, nall = it.nall, m = it.m_cta + q * 32 + lane;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_accum[b]), bph, abortp))) { QP_ABORT(403); break; }
       tc_fence_after();
+      const uint32_t acc = tmem_base + (uint32_t)(b * QP_NT) + ((uint32_t)(q * 32) << 16);
+      const uint32_t drained = mapa_shared(smem_u32(&bar_drained[b]), 0u);
       const bool direct = pr.ksplit == 1;
-      float* dst = direct ? pr.out : pr.part + (int64_t)split * pr.N * M;
+      float* dst = direct ? pr.out : pr.part + (int64_t)it.split * pr.N * M;
       const float cb = (direct && pr.colbias && m < M) ? pr.colbias[m] : 0.f;
+      float z = 0.f;                     // 0 as long as every value so far is finite, NaN after
       // 32 columns per trip: both TMEM loads, then (SGD) all 32 loads of W, are in flight before anything is
       // used -- a read-modify-write one element at a time is a chain of global-memory round trips
       const bool sgd = direct && pr.epi == EPI_SGD;
       for (int c0 = 32 * half; c0 < nall; c0 += 64) {
         uint32_t ra[16], rb[16];
         const bool second = c0 + 16 < nall;
-        if (have) {
-          tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, ra);
-          if (second) tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c0 + 16), rb);
-          tmem_ld_wait();
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) { ra[j] = 0u; rb[j] = 0u; }
+        tmem_ld16(acc + (uint32_t)c0, ra);
+        if (second) tmem_ld16(acc + (uint32_t)(c0 + 16), rb);
+        tmem_ld_wait();
+        if (c0 + 64 >= nall) {                 // this warp's last read of the tile: the buffer goes back before the stores
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(drained);
         }
         if (m < M) {
-          float* d0 = dst + (n_base + c0) * M + m;
-          const int64_t nleft = pr.N - (n_base + c0);          // rows of the result from this column on
-          const int ncol = second ? 32 : 16;
+          float* d0 = dst + (it.n_base + c0) * M + m;
+          const int nleft = (int)min((int64_t)32, pr.N - (it.n_base + c0));      // rows of the result in this trip
           float w[32];
-          if (sgd) {
+          if (nleft == 32) {
+            if (sgd) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) w[j] = (j < ncol && j < nleft) ? d0[(int64_t)j * M] : 0.f;
-          }
+              for (int j = 0; j < 32; ++j) w[j] = d0[(int64_t)j * M];
+            }
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < ncol && j < nleft) {
+            for (int j = 0; j < 32; ++j) {
               const float v = __uint_as_float(j < 16 ? ra[j & 15] : rb[j & 15]) - cb;
-              if (direct) bad |= !isfinite(v);
+              z = fmaf(v, 0.f, z);
               d0[(int64_t)j * M] = sgd ? fmaf(-pr.lr, v, w[j]) : v;
+            }
+          } else {
+            if (sgd) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) w[j] = j < nleft ? d0[(int64_t)j * M] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              if (j < nleft) {
+                const float v = __uint_as_float(j < 16 ? ra[j & 15] : rb[j & 15]) - cb;
+                z = fmaf(v, 0.f, z);
+                d0[(int64_t)j * M] = sgd ? fmaf(-pr.lr, v, w[j]) : v;
+              }
             }
           }
         }
       }
-    } else {
-      QP_ABORT(403);
+      if (32 * half >= nall && lane == 0) mbar_arrive_cluster(drained);   // no column of a narrow tile is this warp's
+      if (direct && z != 0.f && pr.nonfinite) *pr.nonfinite = 1;
+      b ^= 1;
+      if (b == 0) bph ^= 1;
     }
-    if (bad && pr.nonfinite) *pr.nonfinite = 1;
   }
 #undef QP_ABORT
   tc_fence_before();
@@ -249,7 +285,7 @@ gq_pair_kernel(const __grid_constant__ QpGroup g) {
   cluster_wait();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc_pair(tmem_base, ncols);
+    tmem_dealloc_pair(tmem_base, 2 * QP_NT);
   }
 }
 
@@ -313,19 +349,21 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     size_t tiles_total = 0;
     while (base + cnt < n && cnt < QP_MAX_PROBLEMS) {
       const UmmaGqItem& itx = items_in[base + cnt];
-      const size_t tiles = (size_t)((itx.M + 255) / 256) * (size_t)((itx.N + 511) / 512);
+      const size_t tiles = (size_t)((itx.M + 255) / 256) * (size_t)((itx.N + QP_NT - 1) / QP_NT);
       if (cnt > 0 && (tiles_total + tiles) * QP_MAX_KSPLIT > (size_t)QP_MAX_ITEMS) break;
       if (tiles * QP_MAX_KSPLIT > (size_t)QP_MAX_ITEMS) return FW_ERR_SHAPE;
       tiles_total += tiles;
       ++cnt;
     }
-    // K split per problem: the choice whose longest-first list schedule over the resident pairs ends earliest,
+    // K split per problem: the choice with which the pair that has most to do ends earliest,
     // counting what the reduction of the partial tiles costs.  Estimates in microseconds: a stage of 32 k rows
-    // takes about 0.55 us (48 KB staged against 1024 tensor clocks), two thirds of that for tiles of one panel;
-    // an item costs about 8 us besides (set-up, pipeline fill, epilogue); the reduction streams at about 4 TB/s.
+    // takes about 0.36 us (32 KB staged at 48 bytes a clock), a tile after a pair's first no less than the
+    // 4 us of the epilogue it overlaps with; a pair costs about 8 us besides (set-up, pipeline fill, last epilogue); the reduction streams at
+    // about 4 TB/s.
     std::vector<int> ks_best(cnt, 1);
     // the search costs the host a fraction of a millisecond: its result is kept per list of shapes
     static std::map<std::vector<int64_t>, std::vector<int>> memo;
+    static std::mutex memo_mu;
     std::vector<int64_t> key;
     for (int i = 0; i < cnt; ++i) {
       const UmmaGqItem& itx = items_in[base + i];
@@ -333,12 +371,13 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     }
     bool can_split = false;
     for (int i = 0; i < cnt; ++i) can_split |= items_in[base + i].part != nullptr;
-    auto hit = memo.find(key);
-    if (!can_split) {
-      // no scratch for partial tiles anywhere: nothing to choose
-    } else if (hit != memo.end()) {
-      ks_best = hit->second;
-    } else {
+    bool known = false;
+    {
+      std::lock_guard<std::mutex> lock(memo_mu);
+      auto hit = memo.find(key);
+      if (hit != memo.end()) { ks_best = hit->second; known = true; }
+    }
+    if (can_split && !known) {             // without scratch for partial tiles there is nothing to choose
       double best = 1e300;
       std::vector<int> ks_try(cnt);
       std::vector<double> costs;
@@ -349,7 +388,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
         for (int i = 0; i < cnt; ++i) {
           const UmmaGqItem& itx = items_in[base + i];
           const int nkb = (itx.M + QP_SR - 1) / QP_SR;
-          const int64_t tiles = (int64_t)((itx.M + 255) / 256) * ((itx.N + 511) / 512);
+          const int64_t tiles = (int64_t)((itx.M + 255) / 256) * ((itx.N + QP_NT - 1) / QP_NT);
           int ks = (int)((double)nkb / tau + 0.5);
           ks = std::max(1, std::min(ks, std::min(QP_MAX_KSPLIT, std::max(1, nkb / 4))));
           if (ks > 1 && (itx.part == nullptr || (double)ks * (double)itx.N * itx.M > (double)itx.part_floats))
@@ -357,17 +396,17 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
           const int per = (nkb + ks - 1) / ks;
           ks = (nkb + per - 1) / per;
           ks_try[i] = ks;
-          const double st_us = 0.55 * (itx.N > 256 ? 1.0 : 2.0 / 3.0);
           for (int64_t t = 0; t < tiles; ++t)
-            for (int k = 0; k < ks; ++k) costs.push_back(8.0 + st_us * std::min(per, nkb - k * per));
+            for (int k = 0; k < ks; ++k) costs.push_back(0.36 * std::min(per, nkb - k * per));
           if (ks > 1) extra += 3.0 + (double)(ks + 1) * (double)itx.N * itx.M * 4.0 / 4e6;
         }
         std::sort(costs.begin(), costs.end(), [](double a, double b) { return a > b; });
-        std::vector<double> slot(74, 0.0);
-        for (double c : costs) *std::min_element(slot.begin(), slot.end()) += c;
-        const double span = *std::max_element(slot.begin(), slot.end()) + extra;
+        std::vector<double> slot(QP_PAIRS, 0.0);
+        for (size_t c = 0; c < costs.size(); ++c) slot[c % QP_PAIRS] += c < QP_PAIRS ? costs[c] : std::max(4.0, costs[c]);
+        const double span = 8.0 + *std::max_element(slot.begin(), slot.end()) + extra;
         if (span < best) { best = span; ks_best = ks_try; }
       }
+      std::lock_guard<std::mutex> lock(memo_mu);
       if (memo.size() > 256) memo.clear();
       memo[key] = ks_best;
     }
@@ -377,7 +416,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     auto item_len = [&](int i) {
       const UmmaGqItem& itx = items_in[base + i];
       const int nkb = (itx.M + QP_SR - 1) / QP_SR;
-      return (double)((nkb + ks_best[i] - 1) / ks_best[i]) * (itx.N > 256 ? 1.0 : 2.0 / 3.0);
+      return (nkb + ks_best[i] - 1) / ks_best[i];
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return item_len(a) > item_len(b); });
     int64_t nitems = 0;
@@ -387,12 +426,14 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
       QpProblem& p = g.p[oi];
       const int nkb = (itx.M + QP_SR - 1) / QP_SR;
       const int tiles_m = (itx.M + 255) / 256;
-      const int64_t tiles_n = (itx.N + 511) / 512;
+      const int64_t tiles_n = (itx.N + QP_NT - 1) / QP_NT;
       int ks = ks_best[i];
       const int per = (nkb + ks - 1) / ks;
       ks = (nkb + per - 1) / per;
       p.out = itx.out; p.part = itx.part; p.colbias = itx.colbias; p.status = itx.status; p.nonfinite = itx.nonfinite;
       p.N = itx.N; p.M = itx.M; p.ksplit = ks; p.kb_per = per; p.ntiles_n = (int)tiles_n; p.epi = epi; p.lr = lr;
+      // the larger operand is streamed once: all tiles that read a part of it follow one another and find it in L2
+      p.ntiles_m = itx.N > itx.M ? tiles_m : 0;
       p.first_item = (int)nitems;
       nitems += (int64_t)tiles_m * tiles_n * ks;
       p.use3d = (itx.M % 32) == 0 &&
@@ -413,7 +454,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     g.n = cnt; g.nitems = (int)nitems;
     {
       ProfScope ps(prof_class, s);
-      launch_dep(gq_pair_kernel, 2 * g.nitems, QP_THREADS, smem, s, g);
+      launch_dep(gq_pair_kernel, 2 * std::min(g.nitems, QP_PAIRS), QP_THREADS, smem, s, g);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
