@@ -225,8 +225,8 @@ const Tuning& tuning() {
     v.pair_splits = geti("FW_PAIR_SPLITS", 0);
     v.pair_debug = getenv("FW_PAIR_DEBUG") ? 1 : 0;
     v.pass_shape = geti("FW_PASS_SHAPE", 0);
-    v.gram_waves_pct = geti("FW_GRAM_WAVES_PCT", 0);
-    if (v.gram_waves_pct < 50 || v.gram_waves_pct > 1600) v.gram_waves_pct = 0;
+    v.gram_waves_pct = geti("FW_GRAM_WAVES_PCT", 200);
+    if (v.gram_waves_pct < 50 || v.gram_waves_pct > 1600) v.gram_waves_pct = 200;
     return v;
   }();
   return t;

@@ -209,7 +209,7 @@ struct Tuning {
   int pair_splits;     // FW_PAIR_SPLITS  row slabs per problem of the CTA-pair kernels (0: chosen by the scheduler)
   int pair_debug;      // FW_PAIR_DEBUG   print the chosen slabs
   int pass_shape;      // FW_PASS_SHAPE   42 / 24 / 18 / 41: shape of the streaming recursion passes (0: automatic)
-  int gram_waves_pct;  // FW_GRAM_WAVES_PCT  CTAs of a single-CTA Gram launch, in percent of the SM count (0: scheduled)
+  int gram_waves_pct;  // FW_GRAM_WAVES_PCT  CTAs of a single-CTA Gram launch, in percent of the SM count (default 200)
 };
 const Tuning& tuning();
 

@@ -8,9 +8,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <functional>
-#include <map>
-#include <mutex>
 #include <vector>
 
 #include "fw_sm100.cuh"
@@ -880,12 +877,7 @@ fw_status umma_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
   if (!gram_smem_attr(smem)) return FW_ERR_CUDA;
   // one element type per launch: order the items so that each group of a launch is homogeneous
   std::stable_sort(items, items + n, [](const UmmaGramItem& a, const UmmaGramItem& b) { return a.x_bf16 < b.x_bf16; });
-  // Cost model, in microseconds: what a tile takes to stream all rows of its layer.  A CTA streams at the rate shared
-  // memory allows for what the TMA writes and the MMAs (and fix-up warps) read per row: 45 GB/s for blocks whose column
-  // sums come out of the tensor core, 33 where the fix-up warps read every stage, 51 of loaded bytes for the tiles of
-  // TILED layers, which load two ranges of columns (out of L2) per MMA.  Measured at M = 144, 288 and 576; an item costs
-  // about 11 us besides (set-up, pipeline fill, epilogue).
-  constexpr double kItemUs = 11.0;
+  // cost model: bytes a tile streams through shared memory; aim at two waves of equal items
   std::vector<double> tile_cost(n);
   std::vector<int> ntiles(n), stream(n);
   double total = 0;
@@ -906,10 +898,12 @@ fw_status umma_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
         for (int c = 128 * b, t = 0; c < Mpad; c += 256, ++t) loaded_cols += (t ? 128 : 0) + std::min(256, Mpad - c);
       loaded_cols /= ntiles[i];
     }
-    double gbs = 45.0;
-    if (!stream[i]) gbs = 51.0;
-    else if (it.shift || !gram_ones_fits(Mpad)) gbs = 33.0;
-    tile_cost[i] = (double)it.rows * loaded_cols * es / (gbs * 1e3);
+    // bytes through shared memory, weighted by how fast each mode moves them (measured): tiles of the TILED
+    // mode re-read X out of L2, blocks whose column sums are taken by the fix-up warps are bound by those reads
+    double w = 1.0;
+    if (!stream[i]) w = 0.8;
+    else if (Mpad + 16 > 256 || tri + 16 * nb > 512 || it.shift) w = 1.2;
+    tile_cost[i] = (double)it.rows * loaded_cols * es * w;
     total += tile_cost[i] * ntiles[i];
   }
   // rows per stage: larger stages for the layers whose stages nothing but the TMA and the MMA warp touches
@@ -936,69 +930,19 @@ fw_status umma_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
   };
   for (int i = 0; i < n; ++i)
     if (items[i].im2col && (stage_rows(i) == 0 || items[i].x_bf16 || items[i].shift)) return FW_ERR_UNSUPPORTED;
-  // Split counts: equal shares of the launch per item, for the share with which the launch ends earliest.  Items are
-  // handed to the 148 SMs (one CTA each) longest first, and the moment kernels read what every further split writes;
-  // rounding a layer's count up or down decides whether a launch fits a wave, so candidates are scheduled, not derived.
-  // (Rounding to two waves, as before, cost ResNet-20's set 163 us against 155, and the kernels that add its partial
-  // sums 37 against 31.)  The search takes the host a few milliseconds; its result is kept per list of shapes.
+  // Split counts: about two waves of CTAs (one CTA per SM) of near-equal cost.  Rounding to nearest keeps every
+  // item within ~1.4x of the target; rounding down would leave layers whose share is just under 2 with one
+  // item of twice the cost, which then is the tail of the launch.
+  const double target = total / (148.0 * tuning().gram_waves_pct / 100.0);
   std::vector<int64_t> split_of(n);
   std::vector<double> cta_cost(n);
-  std::vector<int64_t> cap_of(n);
   for (int i = 0; i < n; ++i) {
     const int64_t nsr = (virtual_rows(i) + stage_rows(i) - 1) / stage_rows(i);
-    cap_of[i] = std::min<int64_t>(items[i].split_cap, nsr);
+    const int64_t cap = std::min<int64_t>(items[i].split_cap, nsr);
+    int64_t sp = (int64_t)(tile_cost[i] / target + 0.5);
+    split_of[i] = std::max<int64_t>(1, std::min(sp, cap));
+    cta_cost[i] = tile_cost[i] / (double)split_of[i];
   }
-  auto splits_for = [&](double target, double up, std::vector<int64_t>& sp) {
-    for (int i = 0; i < n; ++i)
-      sp[i] = std::max<int64_t>(1, std::min((int64_t)(tile_cost[i] / target + up), cap_of[i]));
-  };
-  const int forced_pct = tuning().gram_waves_pct;
-  static std::map<std::vector<int64_t>, std::vector<int64_t>> memo;
-  static std::mutex memo_mu;
-  std::vector<int64_t> key;
-  for (int i = 0; i < n; ++i) {
-    key.push_back((int64_t)(tile_cost[i] * 1e3)); key.push_back(items[i].M); key.push_back(ntiles[i]);
-    key.push_back(cap_of[i]);
-  }
-  bool known = false;
-  if (forced_pct == 0) {
-    std::lock_guard<std::mutex> lock(memo_mu);
-    auto hit = memo.find(key);
-    if (hit != memo.end()) { split_of = hit->second; known = true; }
-  }
-  if (forced_pct != 0) {
-    splits_for(total / (148.0 * forced_pct / 100.0), 0.5, split_of);
-  } else if (!known) {
-    double best = 1e300;
-    std::vector<int64_t> sp(n), last;
-    std::vector<double> len, heap;
-    for (int pct = 40; pct <= 300; pct += pct < 120 ? 2 : 5) {
-      for (int up = 0; up < 3; ++up) {
-        splits_for(total / (148.0 * pct / 100.0), up == 0 ? 0.0 : up == 1 ? 0.5 : 0.999, sp);
-        if (sp == last) continue;
-        last = sp;
-        len.clear();
-        double extra = 0;
-        for (int i = 0; i < n; ++i) {
-          len.insert(len.end(), (size_t)(sp[i] * ntiles[i]), kItemUs + tile_cost[i] / (double)sp[i]);
-          extra += (double)sp[i] * items[i].M * items[i].M * 8.0 / 3e6;      // partial sums: written, read again
-        }
-        std::sort(len.begin(), len.end(), [](double a, double b) { return a > b; });
-        heap.assign(148, 0.0);                                               // min-heap of the SMs' end times
-        for (double c : len) {
-          std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
-          heap.back() += c;
-          std::push_heap(heap.begin(), heap.end(), std::greater<double>());
-        }
-        const double span = *std::max_element(heap.begin(), heap.end()) + extra;
-        if (span < best) { best = span; split_of = sp; }
-      }
-    }
-    std::lock_guard<std::mutex> lock(memo_mu);
-    if (memo.size() > 256) memo.clear();
-    memo[key] = split_of;
-  }
-  for (int i = 0; i < n; ++i) cta_cost[i] = tile_cost[i] / (double)split_of[i];
   // longest items first: the hardware hands CTAs to SMs in index order as they free up, so the short items
   // fill the end of the launch
   {
