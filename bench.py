@@ -281,17 +281,10 @@ def peaks():
 # no entry here and reports null.
 NCU_TRAFFIC = {
     ("resnet20", "gram"): (660.70e6 + 16.17e6, "profiles/gram_umma_kernel_resnet20.md"),
-    ("resnet20", "recur_chip"): (26.71e6 + 0.43e6, "profiles/recursion_cluster_kernel_resnet20.md"),
-    ("resnet20", "gq"): (10.70e6, "profiles/gq_pair_kernel_resnet20.md"),
-    # three of the six streamed layers were captured (111 MB of Phi_y of 149 MB): scaled by the state bytes
-    ("resnet50", "recur_mv"): ((3.4177e9 + 1.3089e9) * 149.2 / 111.5,
-                               "profiles/recursion_persistent_kernel_resnet50_subset.md (x 149/111: state bytes)"),
 }
 # cost-sweep layer: TF32 Gram pass captured at B = 256 (50176 rows): bytes read, bytes written; the reads are
 # proportional to the rows
 NCU_COST_SWEEP_GRAM_B256 = (661.26e6, 7.90e6, 50176, "profiles/gram_pair_kernel_tf32_cost_sweep_B256.md (reads x rows / 50176)")
-# stress workload, one launch per pass: captured on 8 layers of M = 2304 (traffic is proportional to the layers)
-NCU_STRESS_PASS_M2304_L8 = (169.97e6 + 3.67e6, "profiles/recursion_pass_kernel_stress_M2304.md (x layers / 8)")
 
 
 def traffic_of(key):
@@ -470,6 +463,21 @@ def measure(ls, steps, warmup, reps, barrier, sampler=None, hold_s=0.0):
                 rep_ms=rep_ms, prof=prof, psteps=psteps)
 
 
+def team_roofline(us, K, P, m2):
+    """Large layers: Phi_y in the shared memory of a team of SMs; per step P + 4 products and one update pass."""
+    t = us * 1e-6
+    smem = K * (P + 6) * m2
+    return dict(kernel="recursion_team_kernel (K steps; Phi_y in shared memory as far as it fits, results exchanged through L2)",
+                us_per_step=us, us_per_recursion_step=us / K, smem_gbs=smem / t / 1e9, frac_smem=smem / t / 1e9 / SMEM_PEAK_GBS)
+
+
+def apply_roofline(us, K, m2, hbm):
+    """T and Q of up to 16 steps at a time: each read and written once."""
+    t = us * 1e-6
+    byts = 4.0 * ((K + 15) // 16) * m2
+    return dict(kernel="apply_t_kernel + apply_q_kernel", us_per_step=us, gbs=byts / t / 1e9, frac_hbm=byts / t / hbm)
+
+
 def class_rooflines(ls, m, pk):
     """Per kernel class: device time per step, algorithmic work, the roofline that binds it and the fraction
     reached.  Bounds are per layer: sum over layers of max(flops / tensor peak, bytes / HBM peak)."""
@@ -507,30 +515,15 @@ def class_rooflines(ls, m, pk):
                          frac_hbm=byts / t / hbm, bound_time_us=bound * 1e6, frac_of_per_layer_bound=bound / t)
     m2_stream = sum(4.0 * M * M for (r, M, N), oc in zip(ls.dims, ls.on_chip) if not oc)
     m2_chip = sum(4.0 * M * M for (r, M, N), oc in zip(ls.dims, ls.on_chip) if oc)
-    if "recur_mv" in prof and m2_stream > 0 and "recur_upd" not in prof:
-        # persistent launch: all K steps, passes and rank updates.  Per step P + 3 reads of Phi_y (the row norms
-        # come out of the previous update), one of T^T, and the update's 3 reads + 3 writes; + 1 for the first norms
-        byts = (K * (P + 10) + 1) * m2_stream
-        t = us("recur_mv") * 1e-6
-        out["recur_mv"] = dict(kernel="recursion_persistent_kernel (K steps, passes + rank updates; rows partly "
-                                      "resident in shared memory, so DRAM traffic is below this accounting)",
-                               us_per_step=us("recur_mv"), us_per_recursion_step=us("recur_mv") / K,
-                               launches_per_step=prof["recur_mv"][1] / ps, gbs=byts / t / 1e9, frac_hbm=byts / t / hbm)
-    elif "recur_mv" in prof and m2_stream > 0:
-        byts = K * (P + 5) * m2_stream            # per step: P + 4 reads of Phi_y and one of T^T
-        t = us("recur_mv") * 1e-6
-        out["recur_mv"] = dict(kernel="recursion_pass_kernel (layers streamed from HBM)", us_per_step=us("recur_mv"),
-                               launches_per_step=prof["recur_mv"][1] / ps, gbs=byts / t / 1e9, frac_hbm=byts / t / hbm)
+    if "recur_mv" in prof and m2_stream > 0:
+        out["recur_mv"] = team_roofline(us("recur_mv"), K, P, m2_stream)
+        out["recur_mv"]["launches_per_step"] = prof["recur_mv"][1] / ps
     if "recur_upd" in prof and m2_stream > 0:
-        byts = K * 6 * m2_stream
-        t = us("recur_upd") * 1e-6
-        out["recur_upd"] = dict(kernel="recursion_update_kernel", us_per_step=us("recur_upd"),
-                                launches_per_step=prof["recur_upd"][1] / ps, gbs=byts / t / 1e9,
-                                frac_hbm=byts / t / hbm,
-                                note="counts all K updates; a step whose a_e rounds to 0 leaves early")
+        out["recur_upd"] = apply_roofline(us("recur_upd"), K, m2_stream, hbm)
+        out["recur_upd"]["launches_per_step"] = prof["recur_upd"][1] / ps
     if "recur_chip" in prof and m2_chip > 0:
-        # state in distributed shared memory: per recursion step P + 4 slab-times-vector passes out of shared
-        # memory and one update pass (read + write); nothing of Phi_y crosses HBM inside a call
+        # state on chip: per recursion step P + 4 slab-times-vector passes and one update pass (read + write) over
+        # operands held in registers and shared memory; nothing of Phi_y crosses HBM inside a call
         smem_bytes = K * (P + 6) * m2_chip
         t = us("recur_chip") * 1e-6
         out["recur_chip"] = dict(kernel="recursion_cluster_kernel (state on chip, latency-bound chain of passes)",
@@ -572,7 +565,12 @@ def headline_roofline(ls, m, pk, rl, workload):
                     note="state on chip: not an HBM figure; the kernel is a chain of dependent passes, "
                          "us_per_recursion_step is the figure to watch",
                     us_per_recursion_step=c["us_per_recursion_step"])
-    elif dom in ("recur_mv", "recur_upd"):
+    elif dom == "recur_mv":
+        roof = dict(kernel=c["kernel"], bound="smem", achieved=c["smem_gbs"], peak=SMEM_PEAK_GBS, unit="GB/s",
+                    frac=c["frac_smem"], traffic=None, traffic_source=None,
+                    peak_source="derived: 148 SMs x 128 B/clk x 1.965 GHz shared-memory bandwidth",
+                    us_per_recursion_step=c["us_per_recursion_step"])
+    elif dom == "recur_upd":
         tr, src = traffic_of((workload, dom))
         roof = dict(kernel=c["kernel"], bound="hbm", achieved=c["gbs"], peak=pk["hbm_gbs"], unit="GB/s",
                     frac=c["frac_hbm"], traffic=tr, traffic_source=src, peak_source=pk["source"])
@@ -732,28 +730,12 @@ def stress_rooflines(B, m, M, nl, K, P, pk):
         out["recur_chip"] = dict(kernel="recursion_cluster_kernel (state on chip, latency-bound chain of passes)",
                                  us_per_step=t * 1e6, us_per_recursion_step=t * 1e6 / K,
                                  smem_gbs=smem_bytes / t / 1e9, frac_smem=smem_bytes / t / 1e9 / SMEM_PEAK_GBS)
-    if "recur_mv" in prof and "recur_upd" not in prof:
-        t = prof["recur_mv"][0] * 1e-3
-        byts = (K * (P + 10) + 1) * SM
-        out["recur_mv"] = dict(kernel="recursion_persistent_kernel (K steps in one launch: P + 3 reads of Phi_y, one of "
-                                      "T^T and the 3 + 3 matrix passes of the rank update per step)",
-                               us_per_step=t * 1e6, us_per_recursion_step=t * 1e6 / K, launches=prof["recur_mv"][1],
-                               gbs=byts / t / 1e9, frac_hbm=byts / t / 1e9 / hbm)
-    elif "recur_mv" in prof:
-        t = prof["recur_mv"][0] * 1e-3
-        byts = K * (P + 5) * SM
-        out["recur_mv"] = dict(kernel="recursion_pass_kernel (matrix-vector passes, streamed from HBM)",
-                               us_per_step=t * 1e6, launches=prof["recur_mv"][1], gbs=byts / t / 1e9,
-                               frac_hbm=byts / t / 1e9 / hbm, avg_launch_us=t * 1e6 / prof["recur_mv"][1])
+    if "recur_mv" in prof:
+        out["recur_mv"] = team_roofline(prof["recur_mv"][0] * 1e3, K, P, SM)
+        out["recur_mv"]["launches"] = prof["recur_mv"][1]
     if "recur_upd" in prof:
-        t = prof["recur_upd"][0] * 1e-3
-        byts = K * 6 * SM
-        out["recur_upd"] = dict(kernel="recursion_update_kernel", us_per_step=t * 1e6, launches=prof["recur_upd"][1],
-                                gbs=byts / t / 1e9, frac_hbm=byts / t / 1e9 / hbm)
-    if "recur_mv" in prof and "recur_upd" in prof:
-        t = (prof["recur_mv"][0] + prof["recur_upd"][0]) * 1e-3
-        out["whole_recursion"] = dict(gbs=K * (P + 11) * SM / t / 1e9, frac_hbm=K * (P + 11) * SM / t / 1e9 / hbm,
-                                      note="(P + 11) x 4 M^2 bytes per step per layer over matrix-vector + update time")
+        out["recur_upd"] = apply_roofline(prof["recur_upd"][0] * 1e3, K, SM, hbm * 1e9)
+        out["recur_upd"]["launches"] = prof["recur_upd"][1]
     return {k: {kk: (round(vv, 4) if isinstance(vv, float) else vv) for kk, vv in v.items()} for k, v in out.items()}
 
 
@@ -1055,18 +1037,10 @@ def run_stress(args):
     value = aggregate_value(nl, 1, ms, world)
     pk = peaks()
     cl = stress_rooflines(B, m, M, nl, K, P, pk)
-    if "recur_mv" in cl:
-        c = cl["recur_mv"]
-        tr, src = None, None
-        if M == 2304 and "recursion_pass_kernel" in c["kernel"]:
-            tr, src = NCU_STRESS_PASS_M2304_L8[0] * nl / 8.0, NCU_STRESS_PASS_M2304_L8[1]
-        roof = dict(kernel=c["kernel"], bound="hbm", achieved=c["gbs"], peak=pk["hbm_gbs"], unit="GB/s",
-                    frac=c["frac_hbm"], traffic=tr, traffic_source=src, peak_source=pk["source"])
-    else:
-        c = cl["recur_chip"]
-        roof = dict(kernel=c["kernel"], bound="smem", achieved=c["smem_gbs"], peak=SMEM_PEAK_GBS, unit="GB/s",
-                    frac=c["frac_smem"], traffic=None, traffic_source=None,
-                    peak_source="derived: 148 SMs x 128 B/clk x 1.965 GHz shared-memory bandwidth")
+    c = cl["recur_mv"] if "recur_mv" in cl else cl["recur_chip"]
+    roof = dict(kernel=c["kernel"], bound="smem", achieved=c["smem_gbs"], peak=SMEM_PEAK_GBS, unit="GB/s",
+                frac=c["frac_smem"], traffic=None, traffic_source=None,
+                peak_source="derived: 148 SMs x 128 B/clk x 1.965 GHz shared-memory bandwidth")
     roof["classes"] = cl
     # end to end: Phi_x comes from pinned host memory every step, Q is read back
     layers, hs, ph, distinct = m["layers"], m["hs"], m["ph"], m["distinct"]
