@@ -98,6 +98,7 @@ struct Slab {
   int maxcol;     // start vector: largest column instead of the alignment
   float c_rel, c_abs, delta, eps, lam_bar;
   float ah[KH];   // a_e of the recorded steps
+  float negz;     // -0
   int fail;       // set once a bounded wait of this CTA gave up
 };
 // The parts of it every pass needs, in registers.
@@ -167,8 +168,9 @@ __device__ __forceinline__ void send4(const Link& l, float* tgt, float4 v, uint3
 
 // One pass: y = scale * (my rows) x, sent to `dst` (the slot of the warp's first
 // group in the result vector) of every CTA of the layer.  NORM: scale = 1 / ||x||, summed from
-// the values of x the pass loads anyway; returns ||x||^2.  SELF: squared norms of the rows themselves.
-enum { PASS_SELF, PASS_SCALE, PASS_NORM };
+// the values of x the pass loads anyway; returns ||x||^2.  UNIT: the rows times x / ||x||, the norm summed first.  SELF:
+// squared norms of the rows themselves.
+enum { PASS_SELF, PASS_SCALE, PASS_NORM, PASS_UNIT };
 template <int MODE, int NG, int IT>
 __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float* x, float scale, const Link& l,
                                       float* dst, uint32_t e) {
@@ -177,11 +179,22 @@ __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float
   float acc[4 * NG][2];
 #pragma unroll
   for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
-  float n0 = 0.f, n1 = 0.f;
+  float n0 = 0.f, n1 = 0.f, n2 = 0.f, inv = 1.f;
+  if (MODE == PASS_UNIT) {
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const float4 b = x4[lane + 32 * k];
+      n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
+      n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
+    }
+    n2 = warp_sum(n0 + n1);
+    inv = inv_norm(n2);
+  }
 #pragma unroll
   for (int k = 0; k < IT; ++k) {
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
     if (MODE != PASS_SELF) b = x4[lane + 32 * k];
+    if (MODE == PASS_UNIT) { b.x *= inv; b.y *= inv; b.z *= inv; b.w *= inv; }
     if (MODE == PASS_NORM) {
       n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
       n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
@@ -194,7 +207,6 @@ __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float
       acc[q][0] = fmaf(v.z, bb.z, acc[q][0]); acc[q][1] = fmaf(v.w, bb.w, acc[q][1]);
     }
   }
-  float n2 = 0.f;
   if (MODE == PASS_NORM) { n2 = warp_sum(n0 + n1); scale = inv_norm(n2); }
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
@@ -437,6 +449,30 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
   }
 }
 
+// p + (a (vi u_j + ui v_j) + a^2 lambda_e vi v_j) of four entries j, a rounding per operation, as packed fp32 pairs: half
+// the issue slots (a step's update at M = 576 is 20 float4 per lane)
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+// A product rounded by itself: the compiler fuses a packed multiplication with the addition that follows it, .rn or not, so
+// the product is an fma with z = (-0, -0), which the compiler must not know (it comes from shared memory).
+__device__ __forceinline__ u64 mul2(u64 a, u64 b, u64 z) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(z));
+  return r;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ float4 rank2(float4 p, u64 vi, u64 ui, u64 va, u64 vb, u64 ua, u64 ub, u64 a, u64 l, u64 z) {
+  const u64 x = add2(pack2(p.x, p.y), add2(mul2(a, add2(mul2(vi, ua, z), mul2(ui, va, z)), z), mul2(l, mul2(vi, va, z), z)));
+  const u64 y = add2(pack2(p.z, p.w), add2(mul2(a, add2(mul2(vi, ub, z), mul2(ui, vb, z)), z), mul2(l, mul2(vi, vb, z), z)));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(p.x), "=f"(p.y) : "l"(x));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(p.z), "=f"(p.w) : "l"(y));
+  return p;
+}
+
 // Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane.
 template <int NG, int IT>
 __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L, float* tr, int k0, int k1, int P,
@@ -481,7 +517,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
     // S5: v = prev/||prev|| (Eq. 50), u = Phi_y v, lambda_e = v.u (Eq. 36)
     const float* x = csm + xo;
     arm(l, e, tx);
-    const float n2 = pass<PASS_NORM, NG, IT>(a, x, 0.f, l, csm + s.uvec + slot, e);
+    const float n2 = pass<PASS_UNIT, NG, IT>(a, x, 1.f, l, csm + s.uvec + slot, e);
     const float inv = inv_norm(n2);
     float* vh = csm + s.vh + (step - k0) * s.Mv;
     wait_exchange(l, e, &s.fail); ++e;
@@ -505,30 +541,26 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
       g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);
       aa = sqrtf(g_e) - 1.f;
     }
-    // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T = v w^T + w v^T with w = a u + (a^2 lambda_e / 2) v: four operations
-    // an element, symmetric in (i, j)
+    // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T, symmetric in (i, j)
     if (aa != 0.f) {
-      const float hl = 0.5f * aa * aa * lam_e;
-      float vi[4 * NG], wi[4 * NG];
+      const u64 z = pack2(s.negz, s.negz), a2 = pack2(aa, aa), l2 = pack2(aa * aa * lam_e, aa * aa * lam_e);
+      u64 vi[4 * NG], ui[4 * NG];
 #pragma unroll
       for (int q = 0; q < 4 * NG; ++q) {
         const int i = slot + 4 * CW * (q >> 2) + (q & 3);
-        vi[q] = x[i] * inv;
-        wi[q] = __fadd_rn(__fmul_rn(aa, csm[s.uvec + i]), __fmul_rn(hl, vi[q]));
+        const float v = x[i] * inv, u = csm[s.uvec + i];
+        vi[q] = pack2(v, v); ui[q] = pack2(u, u);
       }
 #pragma unroll
       for (int k = 0; k < IT; ++k) {
         const int c = lane + 32 * k;
-        float4 vj = x4[c], wj = u4[c];
+        float4 vj = x4[c];
+        const float4 uj = u4[c];
         vj.x *= inv; vj.y *= inv; vj.z *= inv; vj.w *= inv;
-        wj.x = __fadd_rn(__fmul_rn(aa, wj.x), __fmul_rn(hl, vj.x)); wj.y = __fadd_rn(__fmul_rn(aa, wj.y), __fmul_rn(hl, vj.y));
-        wj.z = __fadd_rn(__fmul_rn(aa, wj.z), __fmul_rn(hl, vj.z)); wj.w = __fadd_rn(__fmul_rn(aa, wj.w), __fmul_rn(hl, vj.w));
+        const u64 va = pack2(vj.x, vj.y), vb = pack2(vj.z, vj.w), ua = pack2(uj.x, uj.y), ub = pack2(uj.z, uj.w);
 #pragma unroll
         for (int q = 0; q < 4 * NG; ++q) {
-          a[q][k].x = __fadd_rn(a[q][k].x, __fadd_rn(__fmul_rn(vi[q], wj.x), __fmul_rn(wi[q], vj.x)));
-          a[q][k].y = __fadd_rn(a[q][k].y, __fadd_rn(__fmul_rn(vi[q], wj.y), __fmul_rn(wi[q], vj.y)));
-          a[q][k].z = __fadd_rn(a[q][k].z, __fadd_rn(__fmul_rn(vi[q], wj.z), __fmul_rn(wi[q], vj.z)));
-          a[q][k].w = __fadd_rn(a[q][k].w, __fadd_rn(__fmul_rn(vi[q], wj.w), __fmul_rn(wi[q], vj.w)));
+          a[q][k] = rank2(a[q][k], vi[q], ui[q], va, vb, ua, ub, a2, l2, z);
           if (c < (s.Mp >> 2))
             reinterpret_cast<float4*>(csm + (4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp)[c] = a[q][k];
         }
@@ -572,19 +604,28 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     const int c = sub + LPR * k;
     a[k] = row < s.R && c < M4 ? reinterpret_cast<const float4*>(csm + row * s.Mp)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  // y = scale (row . x) into dst; NORM: scale = 1 / ||x||, returns ||x||^2
-  auto dot = [&](const float* x, float scale, bool norm, float* dst) {
+  // Sums are formed as the warp of a larger layer forms them (a pair of sums per float4, then a tree over the float4s), so
+  // that a layer's result does not depend on what else is in the launch.
+  auto four = [](float4 x, float4 y) {
+    return fmaf(x.z, y.z, __fmul_rn(x.x, y.x)) + fmaf(x.w, y.w, __fmul_rn(x.y, y.y));
+  };
+  // y = scale (row . x) into dst; NORM: scale = 1 / ||x||, returns ||x||^2; UNIT: row . (x / ||x||)
+  auto dot = [&](const float* x, float scale, int mode, float* dst) {
     const float4* x4 = reinterpret_cast<const float4*>(x);
-    float d0 = 0.f, d1 = 0.f, n0 = 0.f, n1 = 0.f;
+    float d = 0.f, n2 = 0.f, inv = 1.f;
+    if (mode != PASS_SCALE) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) { const float4 b = x4[sub + LPR * k]; n2 = k ? n2 + four(b, b) : four(b, b); }
+    }
+    if (mode == PASS_UNIT) { n2 = row_sum(n2); inv = inv_norm(n2); }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-      const float4 b = x4[sub + LPR * k];
-      d0 = fmaf(a[k].x, b.x, d0); d1 = fmaf(a[k].y, b.y, d1); d0 = fmaf(a[k].z, b.z, d0); d1 = fmaf(a[k].w, b.w, d1);
-      if (norm) { n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1); n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1); }
+      float4 b = x4[sub + LPR * k];
+      if (mode == PASS_UNIT) { b.x *= inv; b.y *= inv; b.z *= inv; b.w *= inv; }
+      d = k ? d + four(a[k], b) : four(a[k], b);
     }
-    float n2 = 0.f;
-    if (norm) { n2 = row_sum(n0 + n1); scale = inv_norm(n2); }
-    const float d = row_sum(d0 + d1);
+    if (mode == PASS_NORM) { n2 = row_sum(n2); scale = inv_norm(n2); }
+    d = row_sum(d);
     if (sub == 0) dst[row] = d * scale;
     return n2;
   };
@@ -592,12 +633,10 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     const int k1 = min(K, k0 + KH);
     for (int step = k0; step < k1; ++step) {
       // squared norms (Eq. 45), m' (Eq. 46): every warp finds it for itself
-      float q0 = 0.f, q1 = 0.f;
+      float q0 = four(a[0], a[0]);
 #pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        q0 = fmaf(a[k].x, a[k].x, q0); q1 = fmaf(a[k].y, a[k].y, q1); q0 = fmaf(a[k].z, a[k].z, q0); q1 = fmaf(a[k].w, a[k].w, q1);
-      }
-      q0 = row_sum(q0 + q1);
+      for (int k = 1; k < KM; ++k) q0 += four(a[k], a[k]);
+      q0 = row_sum(q0);
       if (sub == 0) csm[s.xi2 + row] = q0;
       __syncthreads();
       const int mp = argmax_xi(s);
@@ -606,7 +645,7 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
         for (int k = 0; k < KM; ++k) reinterpret_cast<float4*>(csm + s.wvec)[sub + LPR * k] = a[k];
       }
       __syncthreads();
-      dot(csm + s.wvec, 1.f, false, csm + s.cvec);                       // Eq. 47
+      dot(csm + s.wvec, 1.f, PASS_SCALE, csm + s.cvec);                       // Eq. 47
       __syncthreads();
       // coherent set, aligned average (Eqs. 48-49)
       int cnt = 1;
@@ -626,45 +665,42 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
         if (!s.maxcol) cnt = n;
       }
       int xo = s.buf0, yo = xo + s.Mv;
-      dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, false, csm + xo);
+      dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, PASS_SCALE, csm + xo);
       __syncthreads();
       for (int p = 0; p < P; ++p) {
-        dot(csm + xo, 0.f, true, csm + yo);
+        dot(csm + xo, 0.f, PASS_NORM, csm + yo);
         __syncthreads();
         const int t = xo; xo = yo; yo = t;
       }
-      const float n2 = dot(csm + xo, 0.f, true, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
+      const float n2 = dot(csm + xo, 1.f, PASS_UNIT, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
       const float inv = inv_norm(n2);
       __syncthreads();
       const float4* x4 = reinterpret_cast<const float4*>(csm + xo);
       const float4* u4 = reinterpret_cast<const float4*>(csm + s.uvec);
-      float l0 = 0.f, l1 = 0.f;
+      float l0 = 0.f;
 #pragma unroll
       for (int k = 0; k < KM; ++k) {
-        const float4 x = x4[sub + LPR * k], u = u4[sub + LPR * k];
-        l0 = fmaf(x.x * inv, u.x, l0); l1 = fmaf(x.y * inv, u.y, l1); l0 = fmaf(x.z * inv, u.z, l0); l1 = fmaf(x.w * inv, u.w, l1);
+        float4 x = x4[sub + LPR * k];
+        x.x *= inv; x.y *= inv; x.z *= inv; x.w *= inv;
+        l0 = k ? l0 + four(x, u4[sub + LPR * k]) : four(x, u4[sub + LPR * k]);
       }
-      const float lam_e = row_sum(l0 + l1);                         // Eq. 36
+      const float lam_e = row_sum(l0);                              // Eq. 36
       const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
       float g_e = 1.f, aa = 0.f;
       if (ok) {
         g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);                 // Eqs. 40-41
         aa = sqrtf(g_e) - 1.f;
       }
-      // Phi_y += v w^T + w v^T, w = a u + (a^2 lambda_e / 2) v, as in run_steps
+      // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T, as in run_steps
       if (aa != 0.f) {
-        const float hl = 0.5f * aa * aa * lam_e;
-        const float vi = csm[xo + row] * inv, wi = __fadd_rn(__fmul_rn(aa, csm[s.uvec + row]), __fmul_rn(hl, vi));
+        const float v = csm[xo + row] * inv, u = csm[s.uvec + row], l = aa * aa * lam_e;
 #pragma unroll
         for (int k = 0; k < KM; ++k) {
-          float4 v = x4[sub + LPR * k], w = u4[sub + LPR * k];
-          v.x *= inv; v.y *= inv; v.z *= inv; v.w *= inv;
-          w.x = __fadd_rn(__fmul_rn(aa, w.x), __fmul_rn(hl, v.x)); w.y = __fadd_rn(__fmul_rn(aa, w.y), __fmul_rn(hl, v.y));
-          w.z = __fadd_rn(__fmul_rn(aa, w.z), __fmul_rn(hl, v.z)); w.w = __fadd_rn(__fmul_rn(aa, w.w), __fmul_rn(hl, v.w));
-          a[k].x = __fadd_rn(a[k].x, __fadd_rn(__fmul_rn(vi, w.x), __fmul_rn(wi, v.x)));
-          a[k].y = __fadd_rn(a[k].y, __fadd_rn(__fmul_rn(vi, w.y), __fmul_rn(wi, v.y)));
-          a[k].z = __fadd_rn(a[k].z, __fadd_rn(__fmul_rn(vi, w.z), __fmul_rn(wi, v.z)));
-          a[k].w = __fadd_rn(a[k].w, __fadd_rn(__fmul_rn(vi, w.w), __fmul_rn(wi, v.w)));
+          float4 vj = x4[sub + LPR * k];
+          const float4 uj = u4[sub + LPR * k];
+          vj.x *= inv; vj.y *= inv; vj.z *= inv; vj.w *= inv;
+          a[k] = rank2(a[k], pack2(v, v), pack2(u, u), pack2(vj.x, vj.y), pack2(vj.z, vj.w), pack2(uj.x, uj.y), pack2(uj.z, uj.w),
+                       pack2(aa, aa), pack2(l, l), pack2(s.negz, s.negz));
         }
       }
       if (tid < 64) csm[s.vh + (step - k0) * s.Mv + tid] = csm[xo + tid] * inv;
@@ -722,13 +758,11 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
       const float ak = s.ah[j];
       if (ak == 0.f) continue;
       const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + j * s.Mv);
-      float d0 = 0.f, d1 = 0.f;
+      float d = four(t[0], v4[sub]);
 #pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const float4 b = v4[sub + LPR * k];
-        d0 = fmaf(t[k].x, b.x, d0); d1 = fmaf(t[k].y, b.y, d1); d0 = fmaf(t[k].z, b.z, d0); d1 = fmaf(t[k].w, b.w, d1);
-      }
-      const float d = row_sum(d0 + d1), at = ak * d;
+      for (int k = 1; k < KM; ++k) d += four(t[k], v4[sub + LPR * k]);
+      d = row_sum(d);
+      const float at = ak * d;
       if (sub == 0) csm[s.th + j * s.Mv + row] = d;
 #pragma unroll
       for (int k = 0; k < KM; ++k) {
@@ -834,7 +868,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     s.maxcol = L->init == FW_INIT_MAXCOL;
     s.c_rel = L->c_rel; s.c_abs = L->c_abs; s.delta = L->delta; s.eps = L->eps;
     s.lam_bar = L->scal[SC_LAMBDA_BAR];
-    s.fail = 0;
+    s.fail = 0; s.negz = -0.f;
     sm100::mbar_init(l.bar0, 1);
     sm100::mbar_init(l.bar0 + 8, 1);
     sm100::mbar_fence_init();
