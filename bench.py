@@ -659,12 +659,12 @@ def evd_leg(B, torch, ls, roof, reps=3):
     torch.cuda.synchronize()
     rec_us = roof.get("classes", {}).get("recur_chip", {}).get("us_per_step")
     ms = statistics.median(ts)
-    flops = sum(12.0 * M ** 3 for _, M, _ in ls.dims)            # per sweep: 3 dot products + 2 x 2 row rotations per pair
+    flops = sum(5.0 * M ** 3 for _, M, _ in ls.dims)             # per sweep: Gram matrices and rotations of the block pairs
     return dict(kernel="jacobi_kernel + evd_finish_kernel + vdv_kernel (fw_group_evd_whiten, fp64)", layers=ls.n,
                 ms_per_call=ms, ms_min=min(ts), fp64_flops_per_sweep=flops,
                 recursion_us_per_call=rec_us, ratio_to_recursion=(ms * 1e3 / rec_us) if rec_us else None,
                 note="one decomposition of every layer's Phi_x against the K recursion steps of a call; the rotation "
-                     "kernel is bound by its M - 1 grid barriers per sweep, not by arithmetic")
+                     "kernel is bound by its chain of M / 16 - 1 rounds per sweep, not by arithmetic")
 
 
 def stress_measure(B, torch, dev, M, nl, cond, K, P, steps, warmup, barrier, sampler=None):
