@@ -15,6 +15,7 @@
 // Both are bound by reading and writing their matrix once (L2 or HBM).
 #include <cstring>
 
+#include "fw_fixsum.cuh"
 #include "fw_internal.h"
 
 namespace fw {
@@ -46,27 +47,54 @@ __device__ __forceinline__ T warp_sum(T x) {
 }
 
 // One row of T^T, NV units of V floats per thread, units `t`, `t` + T, ... of the row for thread t of the T that share it.
-// D: accumulator of the dot products (double where the recursion on Phi_y accumulates in more than fp32).
-template <int NV, int V, class D, bool BLOCK>
-__device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDev* L, int i, int K, D* red) {
-  constexpr int T = BLOCK ? AT : 32;
+// Bound by issue: the conversions of an fp64 sum (16 per clock and SM) made 64 layers of M = 1152 and eight steps 470 us,
+// now 355.  FIX: the dot product as an anchored sum of two fp32 numbers (where the recursion on Phi_y accumulates in more than fp32);
+// ||v|| = 1, so ||row|| bounds it, and a step adds at most |a t| to that norm.
+template <int NV, int V, bool FIX, bool BLOCK>
+__device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDev* L, int i, int K, float2* red) {
+  constexpr int T = BLOCK ? AT : 32, H = NV * V / 2;
   const int M = L->M, MU = M / V;
   const int t = BLOCK ? (int)threadIdx.x : (int)(threadIdx.x & 31);
+  static_assert((NV * V) % 2 == 0 || !FIX, "pairs");
   float r[NV][V];
+  float* rf = &r[0][0];
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
     const int c = t + n * T;
+#pragma unroll
+    for (int e = 0; e < V; ++e) r[n][e] = 0.f;
     if (c < MU) {
       if (V == 4) *reinterpret_cast<float4*>(r[n]) = reinterpret_cast<const float4*>(row)[c];
       else r[n][0] = row[c];
     }
+  }
+  // sum over the threads of the row
+  auto total = [&](float2 y) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) y = add2(y, shfl_xor2(y, o));
+    if (BLOCK) {
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = y;
+      __syncthreads();
+      y = red[0];
+#pragma unroll
+      for (int w = 1; w < AWARPS; ++w) y = add2(y, red[w]);
+      __syncthreads();
+    }
+    return y;
+  };
+  float rn = 0.f;
+  if (FIX) {
+    float q = 0.f;
+#pragma unroll
+    for (int n = 0; n < NV * V; ++n) q = fmaf(rf[n], rf[n], q);
+    rn = sqrtf(total(make_float2(q, 0.f)).x);
   }
   for (int k = 0; k < K; ++k) {
     const float a = L->ah[k];
     if (a == 0.f) continue;                        // no step taken (uniform)
     const float* v = L->vh + (size_t)k * M;
     float x[NV][V];
-    D acc = 0;
+    float* xf = &x[0][0];
 #pragma unroll
     for (int n = 0; n < NV; ++n) {
       const int c = t + n * T;
@@ -75,25 +103,27 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
       if (c < MU) {
         if (V == 4) *reinterpret_cast<float4*>(x[n]) = __ldg(reinterpret_cast<const float4*>(v) + c);
         else x[n][0] = __ldg(v + c);
-#pragma unroll
-        for (int e = 0; e < V; ++e) acc = fma((D)r[n][e], (D)x[n][e], acc);
       }
     }
-    acc = warp_sum(acc);
-    if (BLOCK) {
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-      __syncthreads();
-      acc = 0;
+    float ti;
+    if (FIX) {
+      const float C = anchor(1.01f * rn);
+      u64 s = pack2(C, C), l = 0;
 #pragma unroll
-      for (int w = 0; w < AWARPS; ++w) acc += red[w];
-      __syncthreads();
+      for (int h = 0; h < H; ++h) fix_add(s, l, pack2(rf[2 * h], rf[2 * h + 1]), pack2(xf[2 * h], xf[2 * h + 1]));
+      const float2 y = total(fix_value(s, l, C));
+      ti = y.x + y.y;
+    } else {
+      float acc = 0.f;
+#pragma unroll
+      for (int n = 0; n < NV * V; ++n) acc = fmaf(rf[n], xf[n], acc);
+      ti = warp_sum(acc);
     }
-    const float ti = (float)acc, ati = a * ti;
+    const float ati = a * ti;
+    if (FIX) rn += fabsf(ati);
     if (t == 0) L->th[(size_t)k * M + i] = ti;
 #pragma unroll
-    for (int n = 0; n < NV; ++n)
-#pragma unroll
-      for (int e = 0; e < V; ++e) r[n][e] = fmaf(ati, x[n][e], r[n][e]);
+    for (int n = 0; n < NV * V; ++n) rf[n] = fmaf(ati, xf[n], rf[n]);
   }
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
@@ -108,7 +138,7 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
 // rows of M <= 1280 take a warp each; longer rows a CTA each
 __global__ void __launch_bounds__(AT) apply_t_kernel(const __grid_constant__ ApplyArgs a) {
   dep_sync();
-  __shared__ double red[AWARPS];
+  __shared__ float2 red[AWARPS];
   const int li = apply_layer(a, (int)blockIdx.x);
   const LayerDev* L = a.g.layer[li];
   const int M = L->M, K = a.K;
@@ -116,10 +146,10 @@ __global__ void __launch_bounds__(AT) apply_t_kernel(const __grid_constant__ App
   if (M > kWarpRowMax) {
     float* row = L->Tt + (size_t)blk * M;
     if ((M & 3) == 0) {
-      if (M <= 4 * 3 * AT) row_steps<3, 4, double, true>(row, L, blk, K, red);
-      else row_steps<8, 4, double, true>(row, L, blk, K, red);
+      if (M <= 4 * 3 * AT) row_steps<3, 4, true, true>(row, L, blk, K, red);
+      else row_steps<8, 4, true, true>(row, L, blk, K, red);
     } else {
-      row_steps<32, 1, double, true>(row, L, blk, K, red);
+      row_steps<32, 1, true, true>(row, L, blk, K, red);
     }
     return;
   }
@@ -127,66 +157,69 @@ __global__ void __launch_bounds__(AT) apply_t_kernel(const __grid_constant__ App
   if (i >= M) return;
   float* row = L->Tt + (size_t)i * M;
   if ((M & 3) == 0) {
-    if (M <= 256) row_steps<2, 4, float, false>(row, L, i, K, nullptr);
-    else if (M <= 640) row_steps<5, 4, float, false>(row, L, i, K, nullptr);
-    else row_steps<10, 4, double, false>(row, L, i, K, nullptr);
+    if (M <= 256) row_steps<2, 4, false, false>(row, L, i, K, nullptr);
+    else if (M <= 640) row_steps<5, 4, false, false>(row, L, i, K, nullptr);
+    else row_steps<10, 4, true, false>(row, L, i, K, nullptr);
   } else {
-    if (M <= 160) row_steps<5, 1, float, false>(row, L, i, K, nullptr);
-    else if (M <= 640) row_steps<20, 1, float, false>(row, L, i, K, nullptr);
-    else row_steps<40, 1, double, false>(row, L, i, K, nullptr);
+    if (M <= 160) row_steps<5, 1, false, false>(row, L, i, K, nullptr);
+    else if (M <= 640) row_steps<20, 1, false, false>(row, L, i, K, nullptr);
+    else row_steps<40, 1, true, false>(row, L, i, K, nullptr);
   }
 }
 
-// A CTA takes QR rows by 4 AT (V = 4) or AT (V = 1) columns of a layer's Q: the vectors' entries of a thread's columns
-// stay in registers across the rows.
+// A thread takes QR rows of V columns (V = 4, or 1 for rows of odd length) of a layer's Q, whose
+// loads are all in flight together, and takes them through the steps.  Threads are numbered along the
+// columns, then along the groups of rows, so a CTA is full whatever M is (64 layers of M = 1152, eight steps: 480 us with
+// a CTA per 1024 columns and two rows in flight, 240 us so, 104 at HBM rate).
 constexpr int QR = 8;
-__host__ __device__ inline int q_blocks_x(int M) { return (M & 3) == 0 ? (M / 4 + AT - 1) / AT : (M + AT - 1) / AT; }
+__host__ __device__ inline int q_units(int M) { return (M & 3) == 0 ? M / 4 : M; }
 
 template <int V>
 __device__ __forceinline__ void q_tile(const LayerDev* L, int row0, int c, int K, bool smooth) {
   const int M = L->M;
-  const bool in = c * V < M;
-  for (int k0 = 0; k0 < K; k0 += 8) {
-    float tj[8][V], aq[8];
+  float q[QR][V];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float a = k0 + k < K ? L->ah[k0 + k] : 0.f;
-      aq[k] = a * (a + 2.f);
-#pragma unroll
-      for (int e = 0; e < V; ++e) tj[k][e] = 0.f;
-      if (a != 0.f && in) {
-        const float* t = L->th + (size_t)(k0 + k) * M;
-        if (V == 4) *reinterpret_cast<float4*>(tj[k]) = __ldg(reinterpret_cast<const float4*>(t) + c);
-        else tj[k][0] = __ldg(t + c);
-      }
-    }
-    if (!in) continue;
-    const bool last = k0 + 8 >= K;
+  for (int r = 0; r < QR; ++r) {
+    if (row0 + r >= M) continue;
+    const float* qp = L->Q + (size_t)(row0 + r) * M + (size_t)c * V;
+    if (V == 4) *reinterpret_cast<float4*>(q[r]) = *reinterpret_cast<const float4*>(qp); else q[r][0] = *qp;
+  }
 #pragma unroll 2
-    for (int r = 0; r < QR; ++r) {
-      const int i = row0 + r;
-      if (i >= M) break;
-      float* qp = L->Q + (size_t)i * M + (size_t)c * V;
-      float q[V];
-      if (V == 4) *reinterpret_cast<float4*>(q) = *reinterpret_cast<const float4*>(qp); else q[0] = *qp;
+  for (int k = 0; k < K; ++k) {
+    const float a = L->ah[k], aq = a * (a + 2.f);
+    if (aq == 0.f) continue;
+    const float* t = L->th + (size_t)k * M;
+    float tj[V], ti[QR];
+    if (V == 4) {
+      *reinterpret_cast<float4*>(tj) = __ldg(reinterpret_cast<const float4*>(t) + c);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (aq[k] != 0.f) {
-          const float ti = __ldg(L->th + (size_t)(k0 + k) * M + i);
+      for (int h = 0; h < QR / 4; ++h)            // row0 and M are multiples of four
+        if (row0 + 4 * h < M) *reinterpret_cast<float4*>(ti + 4 * h) = __ldg(reinterpret_cast<const float4*>(t + row0) + h);
+    } else {
+      tj[0] = __ldg(t + c);
 #pragma unroll
-          for (int e = 0; e < V; ++e) q[e] = __fadd_rn(q[e], __fmul_rn(aq[k], __fmul_rn(ti, tj[k][e])));
-        }
-      }
-      if (V == 4) *reinterpret_cast<float4*>(qp) = *reinterpret_cast<const float4*>(q); else *qp = q[0];
-      if (last && smooth && L->Qs != L->Q) {
-        const float beta = L->beta;
-        float* sp = L->Qs + (size_t)i * M + (size_t)c * V;
-        float s[V];
-        if (V == 4) *reinterpret_cast<float4*>(s) = *reinterpret_cast<const float4*>(sp); else s[0] = *sp;
+      for (int r = 0; r < QR; ++r) ti[r] = __ldg(t + min(row0 + r, M - 1));
+    }
 #pragma unroll
-        for (int e = 0; e < V; ++e) s[e] = fmaf(beta, s[e], (1.f - beta) * q[e]);
-        if (V == 4) *reinterpret_cast<float4*>(sp) = *reinterpret_cast<const float4*>(s); else *sp = s[0];
-      }
+    for (int r = 0; r < QR; ++r)
+#pragma unroll
+      for (int e = 0; e < V; ++e) q[r][e] = __fadd_rn(q[r][e], __fmul_rn(aq, __fmul_rn(ti[r], tj[e])));
+  }
+  const float beta = L->beta;
+  smooth = smooth && L->Qs != L->Q;
+#pragma unroll
+  for (int r = 0; r < QR; ++r) {
+    if (row0 + r >= M) continue;
+    const size_t at = (size_t)(row0 + r) * M + (size_t)c * V;
+    float* qp = L->Q + at;
+    if (V == 4) *reinterpret_cast<float4*>(qp) = *reinterpret_cast<const float4*>(q[r]); else *qp = q[r][0];
+    if (smooth) {
+      float* sp = L->Qs + at;
+      float s[V];
+      if (V == 4) *reinterpret_cast<float4*>(s) = *reinterpret_cast<const float4*>(sp); else s[0] = *sp;
+#pragma unroll
+      for (int e = 0; e < V; ++e) s[e] = fmaf(beta, s[e], (1.f - beta) * q[r][e]);
+      if (V == 4) *reinterpret_cast<float4*>(sp) = *reinterpret_cast<const float4*>(s); else *sp = s[0];
     }
   }
 }
@@ -196,19 +229,12 @@ __global__ void __launch_bounds__(AT) apply_q_kernel(const __grid_constant__ App
   const int li = apply_layer(a, (int)blockIdx.x);
   const LayerDev* L = a.g.layer[li];
   const int M = L->M;
-  const int blk = (int)blockIdx.x - a.block0[li];
-  if ((M & 3) == 0 && M <= 2 * AT) {
-    // short rows: several rows side by side
-    const int M4 = M >> 2, side = AT / M4;                 // side >= 2
-    const int g = (int)threadIdx.x / M4, c = (int)threadIdx.x - g * M4;
-    if (g < side) q_tile<4>(L, (blk * side + g) * QR, c, a.K, a.smooth != 0);
-    return;
-  }
-  const int bx = q_blocks_x(M);
-  const int by = blk / bx;
-  const int c = (blk - by * bx) * AT + (int)threadIdx.x;
-  if ((M & 3) == 0) q_tile<4>(L, by * QR, c, a.K, a.smooth != 0);
-  else q_tile<1>(L, by * QR, c, a.K, a.smooth != 0);
+  const int units = q_units(M);
+  const int64_t idx = (int64_t)((int)blockIdx.x - a.block0[li]) * AT + threadIdx.x;
+  const int row0 = (int)(idx / units) * QR, c = (int)(idx % units);
+  if (row0 >= M) return;
+  if ((M & 3) == 0) q_tile<4>(L, row0, c, a.K, a.smooth != 0);
+  else q_tile<1>(L, row0, c, a.K, a.smooth != 0);
 }
 
 }  // namespace
@@ -231,12 +257,7 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
   for (int i = 0; i < g.n; ++i) {
     const int M = layer_M[i];
     a.block0[i] = n;
-    if ((M & 3) == 0 && M <= 2 * AT) {
-      const int rows = (AT / (M >> 2)) * QR;
-      n += (M + rows - 1) / rows;
-    } else {
-      n += q_blocks_x(M) * ((M + QR - 1) / QR);
-    }
+    n += (int)(((int64_t)q_units(M) * ((M + QR - 1) / QR) + AT - 1) / AT);
   }
   a.block0[g.n] = n;
   { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(apply_q_kernel, n, AT, 0, s, a); }
