@@ -141,7 +141,6 @@ extern __shared__ __align__(16) float gsm[];
 // AKM: A is K-major (copied asynchronously); else M-major, TN = 4
 template <int TN, bool AKM, int KG, int CAP>
 __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm_ffma_kernel(const __grid_constant__ GemmBlock<CAP> g) {
-  dep_sync();
   constexpr int NT = Shape<TN>::NT;
   // locate the problem this CTA works on
   const int cta = blockIdx.x;
@@ -180,6 +179,7 @@ __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm
   // my column (or row) of each operand, and whether it is inside the matrix
   const int ca = AKM && vec_a ? m0 + 4 * (t & 15) : m0 + (t & 63), cb = vec_b ? n0 + 4 * (t & 15) : n0 + (t & 63);
   const bool in_a = ca < pr.m, in_b = cb < pr.n;
+  dep_sync();                // so far: parameters only
   float sha[4] = {0.f, 0.f, 0.f, 0.f}, shb[4] = {0.f, 0.f, 0.f, 0.f};
   if (pr.shift) {
 #pragma unroll

@@ -169,11 +169,12 @@ struct GemmGroup {
 // launch accounting / optional per-class event timing (host only, fw_api.cu)
 // ---------------------------------------------------------------------------
 // Consecutive kernels of one stream as programmatic dependents: launch_dep lets the device set a grid up (parameters,
-// CTAs on free SMs) while the grid before it still runs, and dep_sync, the first statement of every kernel launched this
-// way, holds it there until that grid has completed and its writes are visible.  A kernel's own trigger goes first: it
-// fires once every CTA of the grid has started, so a dependent never takes an SM a CTA of its predecessor still needs
-// (nor tensor memory: it allocates after its wait).  A step of the small layers is a dozen kernels of 2-20 us; the gap
-// between two of them fell from about 2.5 to 1 us.
+// CTAs on free SMs) while the grid before it still runs, and dep_sync, before the first access to memory of every kernel
+// launched this way (the matrix-product kernels work out their tile before it), holds it there until that grid has
+// completed and its writes are visible.  A kernel's own trigger goes first: it fires once every CTA of the grid has
+// started, so a dependent never takes an SM a CTA of its predecessor still needs (nor tensor memory: it allocates after
+// its wait).  A step of the small layers is a dozen kernels of 2-20 us; the gap between two of them fell from about 2.5 to
+// 1 us.
 __device__ __forceinline__ void dep_sync() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }

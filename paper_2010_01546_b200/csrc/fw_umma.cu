@@ -258,7 +258,6 @@ __device__ __forceinline__ float tf32_rna(float x) {
 // their loops is on the critical path of the pipeline.
 template <bool BF>
 __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_constant__ GramGroup g) {
-  dep_sync();
   constexpr int RB = BF ? 64 : 128;               // bytes per chunk row
   constexpr int KROWS = BF ? 16 : 8;              // rows of X one MMA contracts over
   constexpr uint64_t LAYOUT = BF ? kSwizzle64B : kSwizzle128B32;
@@ -366,6 +365,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
     mbar_init(smem_u32(&bar_accum), 1);
     mbar_fence_init();
   }
+  dep_sync();                                     // so far: parameters and this CTA's own shared memory only
   __syncthreads();
   if (s_skip) return;                             // nothing allocated yet; every thread of the CTA leaves
   const int nslots = s_nslots, nops = s_nops;

@@ -116,7 +116,6 @@ __device__ __forceinline__ float tf32_rna(float x) {
 template <bool BF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 gram_pair_kernel(const __grid_constant__ PairGroup g) {
-  dep_sync();
   // Chunk rows are 128 bytes for both element types (TMA fetches whole 128-byte lines):
   //   fp32: 32 columns, 128-byte swizzle with 32-byte atoms, K-atoms of 4 rows;
   //   bf16: 64 columns, 128-byte swizzle (16-byte units), K-atoms of 8 rows.
@@ -189,6 +188,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
     mbar_init(smem_u32(&bar_accum), 1);
     mbar_fence_init();
   }
+  dep_sync();                                     // so far: parameters and this CTA's own shared memory only
   __syncthreads();
   if (s_skip) return;       // both CTAs of the pair hold the same tile: both leave before any barrier or allocation
   const int ngroups = s_ngroups;
