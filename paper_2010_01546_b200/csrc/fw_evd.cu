@@ -18,6 +18,7 @@
 #include <cstring>
 
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 #include "fw_sm100.cuh"
 
 namespace fw {
@@ -60,12 +61,6 @@ struct EvdArgs {
   EvdLayer l[FW_MAX_GROUP];
   int32_t nl;
 };
-
-__device__ __forceinline__ double warp_sum_d(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
 
 // maximum over the block of values that are not negative
 __device__ double evd_block_max(float x) {
@@ -426,7 +421,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ Finis
     acc = fma(x, x, acc);
     if (fabs(x) > best) { best = fabs(x); bi = i; }
   }
-  acc = sqrt(warp_sum_d(acc));
+  acc = sqrt(warp_sum(acc));
   if (a.dvec[li]) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -436,7 +431,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ Finis
     }
     double dot = 0.0;
     for (int i = lane; i < M; i += 32) dot = fma((double)L.A[(int64_t)bi * M + i], w[i], dot);
-    dot = warp_sum_d(dot);
+    dot = warp_sum(dot);
     if (dot * w[bi] < 0.0) acc = -acc;
   }
   if (lane == 0) a.lam[li][m] = acc;
@@ -444,13 +439,13 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ Finis
 
 // sum over the block in a fixed order
 __device__ double block_sum_d(double x, double* red) {
-  x = warp_sum_d(x);
+  x = warp_sum(x);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
   __syncthreads();
   x = threadIdx.x < 32 ? red[threadIdx.x] : 0.0;
   if (threadIdx.x < 32) {
-    x = warp_sum_d(x);
+    x = warp_sum(x);
     if (threadIdx.x == 0) red[0] = x;
   }
   __syncthreads();

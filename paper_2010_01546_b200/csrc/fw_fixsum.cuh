@@ -4,8 +4,9 @@
 #define FW_FIXSUM_CUH_
 #include <stdint.h>
 
+#include "fw_lanes.cuh"
+
 namespace fw {
-typedef unsigned long long u64;
 
 // The running sum s + l of products whose partial sums are bounded by B, two at a time (packed fp32 pairs).
 __device__ __forceinline__ float anchor(float B) {
@@ -14,12 +15,6 @@ __device__ __forceinline__ float anchor(float B) {
   const uint32_t ex = (__float_as_uint(B) >> 23) & 0xffu;
   return __uint_as_float(min((max(ex, 26u) + 2u) << 23 | 0x00400000u, 0x7f800000u));
 }
-__device__ __forceinline__ u64 pack2(float x, float y) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void unpack2(u64 r, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r)); }
 __device__ __forceinline__ void fix_add(u64& s, u64& l, u64 a, u64 x) {
   u64 n, d, e;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(n) : "l"(a), "l"(x), "l"(s));

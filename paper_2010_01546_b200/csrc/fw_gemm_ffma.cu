@@ -14,6 +14,7 @@
 #include <cstring>
 
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 
 namespace fw {
 
@@ -32,13 +33,6 @@ struct GemmBlock {
   GemmProblem p[CAP];
 };
 
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 pack2(float x, float y) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void unpack2(u64 r, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r)); }
 __device__ __forceinline__ void fma2(u64& c, u64 a, u64 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b)); }
 
 __device__ __forceinline__ void cp_async16(float* d, const float* p, bool in) {

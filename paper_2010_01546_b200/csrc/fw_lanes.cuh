@@ -1,0 +1,49 @@
+// Small device helpers that several kernels share: packed fp32 pairs, warp sums, the rank update of Phi_y.
+#ifndef FW_LANES_CUH_
+#define FW_LANES_CUH_
+
+namespace fw {
+
+// ---- two fp32 numbers in a 64-bit register ----
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(u64 r, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r)); }
+__device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+// A product rounded by itself: the compiler fuses a packed multiplication with the addition that follows it, .rn or not, so
+// the product is an fma with z = (-0, -0), which the compiler must not know (callers read it from shared memory).
+__device__ __forceinline__ u64 mul2(u64 a, u64 b, u64 z) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(z));
+  return r;
+}
+
+// p + (a (vi u_j + ui v_j) + l vi v_j) of four entries j (l = a^2 lambda_e; va, vb, ua, ub: v_j and u_j of the first and the
+// last two), a rounding per operation and symmetric in (i, j), on packed pairs: half the issue slots.
+__device__ __forceinline__ float4 rank2(float4 p, u64 vi, u64 ui, u64 va, u64 vb, u64 ua, u64 ub, u64 a, u64 l, u64 z) {
+  const u64 x = add2(pack2(p.x, p.y), add2(mul2(a, add2(mul2(vi, ua, z), mul2(ui, va, z)), z), mul2(l, mul2(vi, va, z), z)));
+  const u64 y = add2(pack2(p.z, p.w), add2(mul2(a, add2(mul2(vi, ub, z), mul2(ui, vb, z)), z), mul2(l, mul2(vi, vb, z), z)));
+  unpack2(x, p.x, p.y);
+  unpack2(y, p.z, p.w);
+  return p;
+}
+
+// sum over the warp, the same bits in every lane
+template <class T>
+__device__ __forceinline__ T warp_sum(T x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// 1/sqrt(n2) refined by one Newton step, 0 when n2 is not a positive finite number
+__device__ __forceinline__ float inv_norm(float n2) {
+  float inv = (n2 > 0.f && isfinite(n2)) ? rsqrtf(n2) : 0.f;
+  return inv > 0.f ? inv * (1.5f - 0.5f * n2 * inv * inv) : 0.f;
+}
+
+}  // namespace fw
+#endif

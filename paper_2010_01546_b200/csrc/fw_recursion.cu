@@ -16,6 +16,7 @@
 //   pass UPDATE   g_e, a_e (Eqs. 40-41); Q (Eq. 44), T (Eq. 42), Phiy rank updates
 #include <cstdlib>
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 
 namespace fw {
 namespace {
@@ -29,12 +30,6 @@ constexpr int WARPS = kGemvThreads / 32;   // 8
 //           shared-memory reads of x, which every row of a warp shares, than the extra CTAs gain.
 
 enum { PASS_ROWNORM = 0, PASS_CORR = 1, PASS_ALIGN = 2, PASS_POWER = 3, PASS_FINAL = 4 };
-
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
 
 // Sum of n per-block partials in a fixed order, computed redundantly by every CTA.
 __device__ float block_sum_partials(const float* p, int n, float* red) {

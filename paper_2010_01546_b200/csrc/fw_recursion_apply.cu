@@ -17,6 +17,7 @@
 
 #include "fw_fixsum.cuh"
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 
 namespace fw {
 namespace {
@@ -37,13 +38,6 @@ __device__ __forceinline__ int apply_layer(const ApplyArgs& a, int block) {
   for (int i = 1; i < a.g.n; ++i)
     if (block >= a.block0[i]) li = i;
   return li;
-}
-
-template <class T>
-__device__ __forceinline__ T warp_sum(T x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
 }
 
 // One row of T^T, NV units of V floats per thread, units `t`, `t` + T, ... of the row for thread t of the T that share it.

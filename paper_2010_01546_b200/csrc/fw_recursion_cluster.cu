@@ -32,6 +32,7 @@
 #include <mutex>
 
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 #include "fw_sm100.cuh"
 
 namespace cg = cooperative_groups;
@@ -108,17 +109,6 @@ struct Link {
   int n;
   int active;       // threads of the warps that own rows; the others take no part in the steps
 };
-
-// 1/sqrt(n2) refined by one Newton step, 0 when n2 is not a positive finite number
-__device__ __forceinline__ float inv_norm(float n2) {
-  float inv = (n2 > 0.f && isfinite(n2)) ? rsqrtf(n2) : 0.f;
-  return inv > 0.f ? inv * (1.5f - 0.5f * n2 * inv * inv) : 0.f;
-}
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
 
 // Sums of four values over the warp in 6 shuffles instead of 20: halves of the warp keep two of the values, quarters
 // one, and the four totals are handed to every lane.
@@ -447,30 +437,6 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
       }
     }
   }
-}
-
-// p + (a (vi u_j + ui v_j) + a^2 lambda_e vi v_j) of four entries j, a rounding per operation, as packed fp32 pairs: half
-// the issue slots (a step's update at M = 576 is 20 float4 per lane)
-typedef unsigned long long u64;
-__device__ __forceinline__ u64 pack2(float x, float y) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-// A product rounded by itself: the compiler fuses a packed multiplication with the addition that follows it, .rn or not, so
-// the product is an fma with z = (-0, -0), which the compiler must not know (it comes from shared memory).
-__device__ __forceinline__ u64 mul2(u64 a, u64 b, u64 z) {
-  u64 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(z));
-  return r;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ float4 rank2(float4 p, u64 vi, u64 ui, u64 va, u64 vb, u64 ua, u64 ub, u64 a, u64 l, u64 z) {
-  const u64 x = add2(pack2(p.x, p.y), add2(mul2(a, add2(mul2(vi, ua, z), mul2(ui, va, z)), z), mul2(l, mul2(vi, va, z), z)));
-  const u64 y = add2(pack2(p.z, p.w), add2(mul2(a, add2(mul2(vi, ub, z), mul2(ui, vb, z)), z), mul2(l, mul2(vi, vb, z), z)));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(p.x), "=f"(p.y) : "l"(x));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(p.z), "=f"(p.w) : "l"(y));
-  return p;
 }
 
 // Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane.

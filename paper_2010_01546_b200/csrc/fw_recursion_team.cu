@@ -35,6 +35,7 @@
 
 #include "fw_fixsum.cuh"
 #include "fw_internal.h"
+#include "fw_lanes.cuh"
 
 namespace fw {
 namespace {
@@ -44,8 +45,6 @@ constexpr int PW = PT / 32;          // warps
 constexpr int kMaxRows = 96;         // rows of a layer per CTA, at most
 constexpr uint32_t kPollLimit = 1u << 19;
 constexpr size_t kSmem = 227 * 1024 - 1280;   // dynamic; the static variables take the rest (48 rows of M = 1152 fit)
-
-typedef unsigned long long u64;
 
 struct TeamArgs {
   GroupDev g;
@@ -71,16 +70,6 @@ __device__ __forceinline__ u64 peek(const u64* p) {
   return w;
 }
 __device__ __forceinline__ float value_of(u64 w) { return __uint_as_float((uint32_t)w); }
-
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
-__device__ __forceinline__ float inv_norm(float n2) {
-  float inv = (n2 > 0.f && isfinite(n2)) ? rsqrtf(n2) : 0.f;
-  return inv > 0.f ? inv * (1.5f - 0.5f * n2 * inv * inv) : 0.f;
-}
 
 // (d + l) scale, rounded once
 __device__ __forceinline__ float scaled(float2 a, float scale) {
