@@ -6,9 +6,9 @@
 // Q are not needed by a step: its v_e and a_e are recorded and applied afterwards
 // (fw_recursion_apply.cu).  So a step moves no matrix through HBM, and what bounds
 // it is the chain of P + 5 dependent passes:
-//   - the products themselves: 32 matrix elements per clock and SM, both by
-//     shared-memory bandwidth and by the four operations an element costs (below);
-//     rows that do not fit are streamed from L2 / HBM instead;
+//   - the products themselves: 5 bytes of shared memory an element (four rows share a
+//     load of the vector), so 26 matrix elements per clock and SM; rows that do not fit
+//     are streamed from L2 / HBM instead;
 //   - one exchange per pass through L2.  A result is stored as one 8-byte packet
 //     {value, exchange number}; every CTA of the team polls the packets it needs
 //     until they carry the number it waits for.  No flag, no fence, no barrier
@@ -18,14 +18,12 @@
 // all of e, so nobody still reads e - 1 when its slot is written again.  The row
 // norms have a slot of their own, read again when the coherent set is formed.
 //
-// Precision of the products.  Alignment weights 1 / c_m (Eq. 49) amplify the error
-// of c_m by up to 1 / c_rel, so the products are summed in more than fp32.  fp64
-// would be bound by the conversions (16 per clock and SM).  Instead the sum is held
-// as s + l in two fp32 numbers: s starts at C = 1.5 * 2^k, at least four times the
-// bound ||row|| ||x|| on every partial sum, so fma(a, x, s) rounds each product to a
-// multiple of ulp(C) without leaving the binade; the part rounded off is exactly
-// fma(a, x, s_old - s_new) to fp32, and l collects it.  The total is (s - C) + l with
-// an error near 2^-42 ||row|| ||x||.
+// Rounding.  The set of Eq. 48 is a comparison per column and step, and at condition 1e4 a start vector with one column
+// more or less leads to another transform; so every operation is rounded in one stated way, whatever the team:
+//   - a product is the fp64 sum of its row in one order (exact_row below) rounded to fp32;
+//   - vectors are normalised in fp32, entry by entry, before they are multiplied;
+//   - norms and v.u are fp32 sums in the order given at block_sum();
+//   - the rank update has one rounding per operation (rank2).
 //
 // Every wait is bounded: a thread that gives up raises its CTA's flag, after which
 // the CTA waits for nothing, runs to the end and reports FW_ERR_TIMEOUT.
@@ -33,7 +31,6 @@
 #include <cstring>
 #include <vector>
 
-#include "fw_fixsum.cuh"
 #include "fw_internal.h"
 #include "fw_lanes.cuh"
 
@@ -71,32 +68,33 @@ __device__ __forceinline__ u64 peek(const u64* p) {
 }
 __device__ __forceinline__ float value_of(u64 w) { return __uint_as_float((uint32_t)w); }
 
-// (d + l) scale, rounded once
-__device__ __forceinline__ float scaled(float2 a, float scale) {
-  const float p = __fmul_rn(a.x, scale);
-  return __fadd_rn(p, fmaf(a.y, scale, fmaf(a.x, scale, -p)));
+// a 2^-896 as fp64: the bits moved into place.  Exact for every finite a, zero and subnormal numbers included.
+__device__ __forceinline__ double widen(float a) {
+  const int b = __float_as_int(a);
+  return __hiloint2double((b >> 3) & 0x8fffffff, b << 29);
 }
-// sums of four such values over the warp; lane 8 r holds the r-th
-__device__ __forceinline__ float2 warp_sum4(float2 y0, float2 y1, float2 y2, float2 y3) {
+constexpr double kWiden = 0x1p896;
+
+// Sums over the warp of four values per lane; lane 8 r holds the r-th.
+__device__ __forceinline__ double warp_sum4(double y0, double y1, double y2, double y3) {
   const int lane = threadIdx.x & 31;
   const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
-  const float2 u0 = add2(hi ? y2 : y0, shfl_xor2(hi ? y0 : y2, 16));
-  const float2 u1 = add2(hi ? y3 : y1, shfl_xor2(hi ? y1 : y3, 16));
-  float2 z = add2(mid ? u1 : u0, shfl_xor2(mid ? u0 : u1, 8));
-  z = add2(z, shfl_xor2(z, 4));
-  z = add2(z, shfl_xor2(z, 2));
-  return add2(z, shfl_xor2(z, 1));
+  const double u0 = (hi ? y2 : y0) + __shfl_xor_sync(0xffffffffu, hi ? y0 : y2, 16);
+  const double u1 = (hi ? y3 : y1) + __shfl_xor_sync(0xffffffffu, hi ? y1 : y3, 16);
+  double z = (mid ? u1 : u0) + __shfl_xor_sync(0xffffffffu, mid ? u0 : u1, 8);
+  z += __shfl_xor_sync(0xffffffffu, z, 4);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+  return z + __shfl_xor_sync(0xffffffffu, z, 1);
 }
 
-// dynamic shared memory: [two vectors of Mp floats][partial results][cached rows, Mp floats each].  Vectors and rows are
-// addressed by their offset from here, so that the compiler knows them to be in shared memory.
+// dynamic shared memory: [two vectors of Mp floats][partial sums][cached rows, Mp floats each].  All are addressed by their offset from here, so that the compiler knows them to be in shared memory.
 extern __shared__ __align__(16) float psm[];
 
 // One layer as its CTA sees it.
 struct Team {
   const LayerDev* L;
   int rows;           // offset of the cached rows, Mp apart
-  int part;           // offset of the partial results (float2) of the warps that share a row, kPartRows apart
+  int part;           // offset of the partial sums: fp64 of warps that share rows, fp32 of a norm (pair_partial)
   float* phiy;        // my rows in global memory
   u64* slot;          // two alternating packet slots, Me (M rounded up to even) apart
   u64* xi;            // packet slot of the squared row norms
@@ -112,12 +110,14 @@ constexpr int kPartRows = 32;   // rows per CTA up to which the columns of a row
 struct Shared {
   Team t;
   int layer, fail;
-  float red[2][PW][2];
+  float negz;            // -0
+  __align__(16) float red[2][2 * PW];
   uint32_t key[PW], idx[PW];
-  float xi2[kMaxRows], xn[kMaxRows];   // squared norms and norms of my rows
+  float xi2[kMaxRows];   // squared norms of my rows
+  float win[kMaxRows];   // what two orders of a row's product with a unit vector may differ by
 };
 
-// four consecutive entries c4, M of a row in global memory (rows of odd length are not 16-byte aligned)
+// four consecutive entries c4, M of a row in global memory (rows that are not whole float4s are not 16-byte aligned)
 __device__ __forceinline__ float4 load4(const float* row, int c, int M, bool v4) {
   if (v4) return *(reinterpret_cast<const float4*>(row) + c);
   float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -172,131 +172,221 @@ __device__ __forceinline__ void poll(const u64* slot, int p0, int M, uint32_t ep
   }
 }
 
-// block sums of two values; one barrier.  Calls alternate between two sets of slots (flip).
-__device__ __forceinline__ void block_sum2(float& a, float& b, Shared& sh, int flip) {
-  a = warp_sum(a); b = warp_sum(b);
-  float(*red)[2] = sh.red[flip & 1];
-  if ((threadIdx.x & 31) == 0) { red[threadIdx.x >> 5][0] = a; red[threadIdx.x >> 5][1] = b; }
-  __syncthreads();
-  a = b = 0.f;
+// Sum over the block of two values per thread, those of pairs of neighbouring entries.  Entry m belongs to (virtual) thread
+// m mod 1024, which adds its entries in ascending order; 32 neighbouring threads are added as a butterfly from 16 to 1 and
+// their 32 sums in ascending order.  Two neighbouring entries are a thread here, so the butterfly of 32 runs over 16 lanes and
+// ends within the thread.  One barrier; calls alternate between two sets of slots (flip).
+__device__ __forceinline__ float block_sum(float x, float y, Shared& sh, int flip) {
 #pragma unroll
-  for (int w = 0; w < PW; ++w) { a += red[w][0]; b += red[w][1]; }
+  for (int o = 8; o > 0; o >>= 1) { x += __shfl_xor_sync(0xffffffffu, x, o); y += __shfl_xor_sync(0xffffffffu, y, o); }
+  float* red = sh.red[flip & 1];
+  if ((threadIdx.x & 15) == 0) red[threadIdx.x >> 4] = x + y;
+  __syncthreads();
+  float t = 0.f;
+#pragma unroll
+  for (int w = 0; w < 2 * PW / 4; ++w) {
+    const float4 r = reinterpret_cast<const float4*>(red)[w];
+    t += r.x; t += r.y; t += r.z; t += r.w;
+  }
+  return t;
 }
-
-// The vector at offset `dst` <- the vector of exchange `epoch`; returns its squared norm and, where dot >= 0, its product
-// with the vector at `dot` in d
-__device__ __forceinline__ float receive(const u64* slot, int M, uint32_t epoch, int dst, Shared& sh, int flip, int dot,
-                                         float& d) {
-  float sq = 0.f, dt = 0.f;
+// The same for vectors that are not whole float4s, in another order: pairs of entries, eight pairs in ascending order
+// (partial sums in `part`), partial b to thread b mod 256, a butterfly over 32 threads, their eight sums in ascending order.
+// q: sum of the thread's pair p.
+__device__ __forceinline__ void pair_partial(float q, int p, float* part) {
+  float s = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += __shfl_sync(0xffffffffu, q, (threadIdx.x & 24) + w);
+  if ((threadIdx.x & 7) == 0) part[p >> 3] = s;
+}
+__device__ __forceinline__ float partial_sum(const float* part, int n, Shared& sh, int flip) {
+  __syncthreads();
+  float s = 0.f;
+  if (threadIdx.x < 256) {
+    for (int b = threadIdx.x; b < n; b += 256) s += part[b];
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sh.red[flip & 1][threadIdx.x >> 5] = s;
+  }
+  __syncthreads();
+  s = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += sh.red[flip & 1][w];
+  return s;
+}
+// The vector at offset `dst` <- the vector of exchange `epoch`.
+enum { SUM_NONE, SUM_SQUARES, SUM_DOT };
+// Returns its squared norm or, SUM_DOT, its product with xs times the vector at `dot`.
+template <bool V4>
+__device__ __forceinline__ float receive(const u64* slot, int M, uint32_t epoch, int dst, Shared& sh, int flip, int what,
+                                         int dot, float xs) {
+  float sx = 0.f, sy = 0.f;
+  float* part = psm + sh.t.part;
   for (int p0 = threadIdx.x; 2 * (p0 & ~31) < M; p0 += kPairs * PT) {
     float2 v[kPairs];
     poll(slot, p0, M, epoch, sh, v);
 #pragma unroll
     for (int j = 0; j < kPairs; ++j) {
       const int p = p0 + j * PT;
+      if (2 * (p & ~31) >= M) continue;                // uniform in the warp
+      float2 q = v[j];                                 // 0 past the vector
       if (2 * p < M) {
-        reinterpret_cast<float2*>(psm + dst)[p] = v[j];
-        sq = fmaf(v[j].x, v[j].x, sq); sq = fmaf(v[j].y, v[j].y, sq);
-        if (dot >= 0) {
-          const float2 q = reinterpret_cast<const float2*>(psm + dot)[p];
-          dt = fmaf(v[j].x, q.x, dt); dt = fmaf(v[j].y, q.y, dt);
+        reinterpret_cast<float2*>(psm + dst)[p] = q;
+        if (what == SUM_DOT) {
+          q = reinterpret_cast<const float2*>(psm + dot)[p];
+          q.x *= xs; q.y *= xs;
         }
       }
+      if (what == SUM_NONE) continue;
+      if (V4) { sx = fmaf(q.x, v[j].x, sx); sy = fmaf(q.y, v[j].y, sy); }
+      else pair_partial(fmaf(q.y, v[j].y, __fmul_rn(q.x, v[j].x)), p, part);
     }
   }
-  block_sum2(sq, dt, sh, flip);
-  d = dt;
-  return sq;
+  if (what == SUM_NONE) { __syncthreads(); return 0.f; }
+  if (V4) return block_sum(sx, sy, sh, flip);
+  return partial_sum(part, (((M + 1) >> 1) + 7) >> 3, sh, flip);
 }
 
-// Four rows times the vector at offset xo, columns c0, c0 + stride, ... of it; lane 8 r returns the r-th row's sum.
-// CACHED: the rows are in shared memory, Mp apart; else in global memory, M apart, nrows of them.
-template <bool CACHED>
-__device__ __forceinline__ float2 group_product(const float* grow, int row, int nrows, int M, int Mp, int xo, float xnorm,
-                                                const float* xn, int c0, int stride) {
-  u64 s[4], l[4];
-  float C[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    C[r] = anchor(xn[r] * xnorm);
-    s[r] = pack2(C[r], C[r]);
-    l[r] = 0;
+// Row r of mine times xs x (x at offset xo), the sum of record: in fp64, a lane takes the entries of every 32nd float4 (rows
+// that are not whole float4s: every 32nd entry) in ascending order, the lanes are added as a butterfly from 16 to 1.
+__device__ __noinline__ double exact_row(const Shared& sh, int r, int xo, float xs) {
+  const int lane = threadIdx.x & 31;
+  const int M = sh.t.M;
+  const float* row = r < sh.t.ncached ? psm + sh.t.rows + r * sh.t.Mp : sh.t.phiy + (size_t)r * M;
+  double acc = 0.0;
+  if ((M & 3) == 0) {
+#pragma unroll 4
+    for (int c = lane; c < (M >> 2); c += 32) {
+      const float4 a = reinterpret_cast<const float4*>(row)[c], x = *reinterpret_cast<const float4*>(psm + xo + 4 * c);
+      acc = fma((double)a.x, (double)(x.x * xs), acc); acc = fma((double)a.y, (double)(x.y * xs), acc);
+      acc = fma((double)a.z, (double)(x.z * xs), acc); acc = fma((double)a.w, (double)(x.w * xs), acc);
+    }
+  } else {
+#pragma unroll 4
+    for (int c = lane; c < M; c += 32) acc = fma((double)row[c], (double)(psm[xo + c] * xs), acc);
   }
-  const bool v4 = (M & 3) == 0;
+  return warp_sum(acc);
+}
+
+// Four rows times xs x, x the vector at offset xo, entries (float4s where V4) c0, c0 + stride, ... of them; lane 8 r returns
+// the r-th row's sum.  CACHED: the rows are in shared memory, Mp apart; else in global memory, M apart, nrows of them.
+// An SM converts 16 numbers per clock to fp64, which alone would bound the product; so three entries in four of a row are
+// widened by integer operations, beside the conversions of the fourth and of x.
+template <bool CACHED, bool V4, int SHIFT>
+__device__ __forceinline__ double group_product(const float* grow, int row, int nrows, int M, int Mp, int xo, float xs, int c0) {
+  constexpr int stride = 32 << SHIFT;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  if (V4) {
 #pragma unroll 2
-  for (int c = 4 * c0; c < Mp; c += 4 * stride) {
-    const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(psm + xo + c);
+    for (int c = c0; c < (M >> 2); c += stride) {
+      const float4 x = *reinterpret_cast<const float4*>(psm + xo + 4 * c);
+      const double x0 = (double)(x.x * xs) * kWiden, x1 = (double)(x.y * xs) * kWiden, x2 = (double)(x.z * xs) * kWiden,
+                   x3 = (double)(x.w * xs);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      ulonglong2 av;
-      if (CACHED) av = *reinterpret_cast<const ulonglong2*>(psm + row + r * Mp + c);
-      else { const float4 q = load4(grow + (size_t)min(r, nrows - 1) * M, c >> 2, M, v4); av.x = pack2(q.x, q.y); av.y = pack2(q.z, q.w); }
-      fix_add(s[r], l[r], av.x, xv.x);
-      fix_add(s[r], l[r], av.y, xv.y);
+      for (int r = 0; r < 4; ++r) {
+        const float4 a = CACHED ? *reinterpret_cast<const float4*>(psm + row + r * Mp + 4 * c)
+                                : *(reinterpret_cast<const float4*>(grow + (size_t)min(r, nrows - 1) * M) + c);
+        acc[r] = fma(widen(a.x), x0, acc[r]); acc[r] = fma(widen(a.y), x1, acc[r]);
+        acc[r] = fma(widen(a.z), x2, acc[r]); acc[r] = fma((double)a.w, x3, acc[r]);
+      }
+    }
+  } else {
+#pragma unroll 4
+    for (int c = c0; c < M; c += stride) {
+      const double x = (double)(psm[xo + c] * xs) * kWiden;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        acc[r] = fma(widen(CACHED ? psm[row + r * Mp + c] : grow[(size_t)min(r, nrows - 1) * M + c]), x, acc[r]);
     }
   }
-  float2 y[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) y[r] = fix_value(s[r], l[r], C[r]);
-  return warp_sum4(y[0], y[1], y[2], y[3]);
+  return warp_sum4(acc[0], acc[1], acc[2], acc[3]);
 }
-// y = scale (my rows) x, sent into `slot` as exchange `epoch`; x at offset xo, xnorm: ||x||.  One group of four rows at a
-// time per warp (or per cg warps, which split the columns).  STREAM: some rows are in global memory.
-template <bool STREAM>
-__device__ __forceinline__ void product(const Shared& sh, int xo, float xnorm, float scale, u64* slot, uint32_t epoch) {
+
+// Whether the fp64 sum y of my row lr, formed in another order, may round to another fp32 number than the sum of record.
+// sh.win[lr] xnorm is what the two sums may differ by (new_norm).
+__device__ __forceinline__ bool open_rounding(const Shared& sh, double y, int lr, float xnorm) {
+  const double w = (double)(sh.win[lr] * xnorm);
+  return (float)(y - w) != (float)(y + w);
+}
+// y = scale (my rows) (xs x), sent into `slot` as exchange `epoch`; x at offset xo, xnorm: a bound on ||xs x||.  One group of
+// four rows at a time per warp (or per cg warps, which split the columns).  STREAM: some rows are in global memory.
+template <bool STREAM, bool V4, int SHIFT>
+__device__ __forceinline__ void product_split(const Shared& sh, int xo, float xs, float xnorm, float scale, u64* slot, uint32_t epoch) {
+  constexpr int shift = SHIFT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int M = sh.t.M, Mp = sh.t.Mp, nrows = sh.t.nrows, shift = sh.t.cg_log, rows = sh.t.rows;
+  const int M = sh.t.M, Mp = sh.t.Mp, nrows = sh.t.nrows, rows = sh.t.rows;
+  slot += sh.t.row0;
   const int groups = (nrows + 3) >> 2, cached = STREAM ? sh.t.ncached >> 2 : groups;
   const int part = warp & ((1 << shift) - 1), step = PW >> shift;
-  float2* parts = reinterpret_cast<float2*>(psm + sh.t.part);
-  slot += sh.t.row0;
-  xnorm *= 1.01f;
-  for (int g = warp >> shift; g < groups; g += step) {
-    const int c0 = part * 32 + lane, stride = 32 << shift;
-    float2 y;
-    if (!STREAM || g < cached) y = group_product<true>(nullptr, rows + 4 * g * Mp, 4, M, Mp, xo, xnorm, sh.xn + 4 * g, c0, stride);
-    else y = group_product<false>(sh.t.phiy + (size_t)4 * g * M, 0, nrows - 4 * g, M, Mp, xo, xnorm, sh.xn + 4 * g, c0, stride);
+  double* parts = reinterpret_cast<double*>(psm + sh.t.part);
+  uint32_t open = 0;                                 // rows to be summed in the order of record: bit 8 r + i, row r of my i-th group
+  int i = 0;
+  for (int g = warp >> shift; g < groups; g += step, ++i) {
+    const int c0 = part * 32 + lane;
+    double y;
+    if (!STREAM || g < cached) y = group_product<true, V4, SHIFT>(nullptr, rows + 4 * g * Mp, 4, M, Mp, xo, xs, c0);
+    else y = group_product<false, V4, SHIFT>(sh.t.phiy + (size_t)4 * g * M, 0, nrows - 4 * g, M, Mp, xo, xs, c0);
     const int lr = 4 * g + (lane >> 3);
-    if ((lane & 7) == 0 && lr < nrows) {
-      if (shift == 0) put(slot + lr, scaled(y, scale), epoch);
-      else parts[part * kPartRows + lr] = y;
+    const bool mine = (lane & 7) == 0 && lr < nrows;
+    if (shift == 0) {
+      const bool o = mine && open_rounding(sh, y, lr, xnorm);
+      if (mine && !o) put(slot + lr, __fmul_rn((float)y, scale), epoch);
+      open |= __ballot_sync(0xffffffffu, o) << i;
+    } else if (mine) {
+      parts[part * kPartRows + lr] = y;
     }
   }
   if (shift) {
     __syncthreads();
-    if ((int)threadIdx.x < nrows) {
-      float2 y = parts[threadIdx.x];
-      for (int p = 1; p < (1 << shift); ++p) y = add2(y, parts[p * kPartRows + threadIdx.x]);
-      put(slot + threadIdx.x, scaled(y, scale), epoch);
+    if (warp == 0) {
+      double y = 0.0;
+      if (lane < nrows)
+        for (int p = 0; p < (1 << shift); ++p) y += parts[p * kPartRows + lane];
+      const bool o = lane < nrows && open_rounding(sh, y, lane, xnorm);
+      if (lane < nrows && !o) put(slot + lane, __fmul_rn((float)y, scale), epoch);
+      open = __ballot_sync(0xffffffffu, o);
     }
+  }
+  while (open) {
+    const int l = __ffs(open) - 1, lr = shift ? l : 4 * (warp + (l & 7) * PW) + (l >> 3);
+    open &= open - 1;
+    const double y = exact_row(sh, lr, xo, xs);
+    if (lane == 0) put(slot + lr, __fmul_rn((float)y, scale), epoch);
   }
 }
 
-// n passes y = scale Phi_y x with the vectors exchanged between them: the first with (xnorm, scale) as given, the others
-// with x normalised; x at offset xo, the results alternate between the two vectors.  A function of its own with nothing
-// else in it, so that no register of the loop lives in memory: what is left of the L1 cache beside 226 KB of shared
-// memory does not hold the spilled registers of 512 threads (measured: 5.7 us a pass instead of 2.9 at M = 1152).
-struct PassOut { float x2, y2, xy; };    // of the last pass: ||x||^2, ||y||^2, x.y
-template <bool STREAM>
+template <bool STREAM, bool V4>
+__device__ __forceinline__ void product(const Shared& sh, int xo, float xs, float xnorm, float scale, u64* slot, uint32_t epoch) {
+  const int shift = sh.t.cg_log;
+  if (shift == 0) product_split<STREAM, V4, 0>(sh, xo, xs, xnorm, scale, slot, epoch);
+  else if (shift == 1) product_split<STREAM, V4, 1>(sh, xo, xs, xnorm, scale, slot, epoch);
+  else product_split<STREAM, V4, 2>(sh, xo, xs, xnorm, scale, slot, epoch);
+}
+
+// n >= 2 passes with the vectors exchanged between them: y = scale Phi_y x, then y = Phi_y (x / ||x||); x at offset xo,
+// xnorm a bound on the first one's length, the results alternate between the two vectors.  A function of its own with nothing else in it, so that no register of the loop
+// lives in memory: what is left of the L1 cache beside 226 KB of shared memory does not hold the spilled registers of 512
+// threads (measured: 5.7 us a pass instead of 2.9 at M = 1152).
+struct PassOut { float x2, lam; };    // of the last pass: ||x||^2, y.x / ||x||
+template <bool STREAM, bool V4>
 __device__ __noinline__ PassOut passes(Shared& sh, int n, int xo, int yo, float xnorm, float scale, uint32_t epoch, int flip) {
   const int M = sh.t.M;
   u64* const slot = sh.t.slot;
   const int Me = packet_stride(M);
-  float x2 = 0.f, n2 = 0.f, dot = 0.f;
+  float xs = 1.f, x2 = 0.f, sum = 0.f;
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {
     u64* s = slot + ((epoch & 1u) ? Me : 0);
-    product<STREAM>(sh, xo, xnorm, scale, s, epoch);
-    x2 = n2;
-    if (sh.t.cg_log == 0) __syncthreads();
-    n2 = receive(s, M, epoch, yo, sh, flip, i + 1 == n ? xo : -1, dot);
-    xnorm = sqrtf(n2);
-    scale = inv_norm(n2);
+    product<STREAM, V4>(sh, xo, xs, xnorm, scale, s, epoch);
+    scale = 1.f; xnorm = 1.001f;
+    x2 = sum;
+    if (!V4 || sh.t.cg_log == 0) __syncthreads();
+    sum = receive<V4>(s, M, epoch, yo, sh, flip, i + 1 == n ? SUM_DOT : SUM_SQUARES, xo, xs);
+    xs = inv_norm(sum);
     const int z = xo; xo = yo; yo = z;
     ++epoch;
     flip ^= 1;
   }
-  return PassOut{x2, n2, dot};
+  return PassOut{x2, sum};
 }
 
 // block maximum of (key, lowest index); one barrier before the result is read
@@ -311,23 +401,32 @@ __device__ __forceinline__ int block_argmax(uint32_t key, uint32_t idx, Shared& 
   return best == 0 || b >= (uint32_t)M ? 0 : (int)b;
 }
 
+// squared norm of my row r; sent as exchange `epoch` if `send`.  In fp64 it is finite exactly where the row is.
+__device__ __forceinline__ void new_norm(Shared& sh, int r, double n2, bool send, uint32_t epoch) {
+  if ((threadIdx.x & 31) != 0) return;
+  sh.xi2[r] = (float)n2;
+  sh.win[r] = n2 == 0.0 ? 0.f : isfinite(n2) ? fmaxf(sqrtf((float)n2), 1e-19f) * 0x1p-50f : INFINITY;
+  if (send) put(sh.t.xi + sh.t.row0 + r, (float)n2, epoch);
+}
+
 // Squared norms of my rows as they are, sent as exchange `epoch` (later steps get them from the update).
 __device__ __noinline__ void row_norms(Shared& sh, uint32_t epoch) {
   const Team& t = sh.t;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int M = t.M, Mp = t.Mp, M4 = Mp >> 2;
-  const bool v4 = (M & 3) == 0;
+  const int M = t.M, Mp = t.Mp;
   for (int r = warp; r < t.nrows; r += PW) {
+    const float* row = r < t.ncached ? psm + t.rows + r * Mp : t.phiy + (size_t)r * M;
     double acc = 0.0;
-    for (int c = lane; c < M4; c += 32) {
-      const float4 q = r < t.ncached ? *reinterpret_cast<const float4*>(psm + t.rows + r * Mp + 4 * c)
-                                     : load4(t.phiy + (size_t)r * M, c, M, v4);
-      acc = fma((double)q.x, (double)q.x, acc); acc = fma((double)q.y, (double)q.y, acc);
-      acc = fma((double)q.z, (double)q.z, acc); acc = fma((double)q.w, (double)q.w, acc);
+    if ((M & 3) == 0) {
+      for (int c = lane; c < (M >> 2); c += 32) {
+        const float4 q = reinterpret_cast<const float4*>(row)[c];
+        acc = fma((double)q.x, (double)q.x, acc); acc = fma((double)q.y, (double)q.y, acc);
+        acc = fma((double)q.z, (double)q.z, acc); acc = fma((double)q.w, (double)q.w, acc);
+      }
+    } else {
+      for (int c = lane; c < M; c += 32) acc = fma((double)row[c], (double)row[c], acc);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) { sh.xi2[r] = (float)acc; sh.xn[r] = sqrtf((float)acc); put(t.xi + t.row0 + r, (float)acc, epoch); }
+    new_norm(sh, r, warp_sum(acc), true, epoch);
   }
 }
 
@@ -351,9 +450,10 @@ __device__ __noinline__ int receive_argmax(Shared& sh, uint32_t epoch) {
 }
 
 // Row m' from its owner into the vector at xo (exchange `epoch`), c = Phi_y (Phi_y e_m') (Eq. 47, exchange `epoch` + 1),
-// and the weights of the coherent set (Eqs. 48-49) into the vector at yo; returns the size of the set, and ||w||^2 in w2.
-template <bool STREAM>
-__device__ __noinline__ float2 correlate(Shared& sh, int mp, int xo, int yo, uint32_t epoch, int flip, bool keep) {
+// and the weights of the coherent set (Eqs. 48-49) into the vector at yo; returns the size of the set and a bound on ||w||.
+struct Aligned { int cnt; float wnorm; };
+template <bool STREAM, bool V4>
+__device__ __noinline__ Aligned correlate(Shared& sh, int mp, int xo, int yo, uint32_t epoch, bool keep) {
   const Team& t = sh.t;
   const LayerDev* L = t.L;
   const int tid = threadIdx.x, M = t.M;
@@ -364,12 +464,11 @@ __device__ __noinline__ float2 correlate(Shared& sh, int mp, int xo, int yo, uin
     if (r < t.ncached) for (int m = tid; m < M; m += PT) put(s + m, psm[t.rows + r * t.Mp + m], epoch);
     else for (int m = tid; m < M; m += PT) put(s + m, t.phiy[(size_t)r * M + m], epoch);
   }
-  float unused;
-  const float xi_mp = sqrtf(receive(s, M, epoch, xo, sh, flip, -1, unused));
+  receive<V4>(s, M, epoch, xo, sh, 0, SUM_NONE, 0, 0.f);
   ++epoch;
   s = t.slot + ((epoch & 1u) ? Me : 0);
-  product<STREAM>(sh, xo, xi_mp, 1.f, s, epoch);
-  float cnt = 0.f, w2 = 0.f;
+  const float xi_mx = sqrtf(value_of(peek(t.xi + mp)));
+  product<STREAM, V4>(sh, xo, 1.f, 1.001f * xi_mx, 1.f, s, epoch);
   if (L->init == FW_INIT_MAXCOL) {
     for (int m = tid; m < M; m += PT) psm[yo + m] = (m == mp) ? 1.f : 0.f;
     for (int p0 = tid; 2 * (p0 & ~31) < M; p0 += kPairs * PT) {       // received all the same: the slots alternate on that
@@ -377,10 +476,11 @@ __device__ __noinline__ float2 correlate(Shared& sh, int mp, int xo, int yo, uin
       poll(s, p0, M, epoch, sh, v);
     }
     __syncthreads();
-    return make_float2(1.f, 1.f);
+    return Aligned{1, 1.f};
   }
   const float c_rel = L->c_rel, c_abs = L->c_abs;
-  const float xi_mx = sqrtf(value_of(peek(t.xi + mp)));
+  int cnt = 0;
+  float w2 = 0.f;
   for (int p0 = tid; 2 * (p0 & ~31) < M; p0 += kPairs * PT) {
     float2 v[kPairs];
     poll(s, p0, M, epoch, sh, v);
@@ -396,7 +496,7 @@ __device__ __noinline__ float2 correlate(Shared& sh, int mp, int xo, int yo, uin
         const bool in = fabsf(v[j].X) >= thr;          /* false for NaN */           \
         const float q = in ? 1.f / v[j].X : 0.f;                                     \
         psm[yo + (i)] = q;                                                           \
-        cnt += in ? 1.f : 0.f;                                                       \
+        cnt += in ? 1 : 0;                                                           \
         w2 = fmaf(q, q, w2);                                                         \
         if (keep) L->wvec[i] = q;                                                    \
       }
@@ -405,54 +505,49 @@ __device__ __noinline__ float2 correlate(Shared& sh, int mp, int xo, int yo, uin
 #undef FW_WEIGHT
     }
   }
-  block_sum2(cnt, w2, sh, flip ^ 1);
-  return make_float2(cnt, w2);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  w2 = warp_sum(w2);
+  if ((tid & 31) == 0) { sh.key[tid >> 5] = (uint32_t)cnt; sh.idx[tid >> 5] = __float_as_uint(w2); }
+  __syncthreads();
+  cnt = (int)__reduce_add_sync(0xffffffffu, (tid & 31) < PW ? sh.key[tid & 31] : 0u);
+  w2 = warp_sum((tid & 31) < PW ? __uint_as_float(sh.idx[tid & 31]) : 0.f);
+  return Aligned{cnt, 1.001f * sqrtf(w2)};
 }
 
-// Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T = v w^T + w v^T with w = a u + (a^2 lambda_e / 2) v on my rows, exactly
-// symmetric; v = inv x.  Squared norms of the new rows, sent as exchange `epoch` if `send`.
-__device__ __noinline__ void update_rows(Shared& sh, int xo, int yo, float inv, float aa, float lam_e, float u2, bool send, uint32_t epoch) {
+// Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T on my rows, one rounding per operation and symmetric; v = inv x, x at
+// offset xo, u at yo.  Squared norms of the new rows, sent as exchange `epoch` if `send`.
+__device__ __noinline__ void update_rows(Shared& sh, int xo, int yo, float inv, float aa, float lam_e, bool send, uint32_t epoch) {
   const Team& t = sh.t;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int M = t.M, Mp = t.Mp, M4 = Mp >> 2, nrows = t.nrows, ncached = t.ncached, row0 = t.row0, rows = t.rows;
-  const bool v4 = (M & 3) == 0;
-  float* phiy = t.phiy;
-  const float hl = 0.5f * aa * aa * lam_e;
-  // ||w|| and with it a bound on the new rows' norms, which anchors their sums
-  const float wn = 1.01f * (fabsf(aa) * sqrtf(u2) + fabsf(hl));
+  const int M = t.M, Mp = t.Mp, nrows = t.nrows, row0 = t.row0;
+  const float a2l = aa * aa * lam_e;
   for (int r = warp; r < nrows; r += PW) {
-    const float vi = psm[xo + row0 + r] * inv;
-    const float wi = __fadd_rn(__fmul_rn(aa, psm[yo + row0 + r]), __fmul_rn(hl, vi));
-    const float bound = 1.01f * (sh.xn[r] + fabsf(vi) * wn + fabsf(wi));
-    const float C = anchor(bound * bound);
-    u64 s = pack2(C, C), l = 0;
-    const bool cached = r < ncached;
+    const float vi = psm[xo + row0 + r] * inv, ui = psm[yo + row0 + r];
+    float* row = r < t.ncached ? psm + t.rows + r * Mp : t.phiy + (size_t)r * M;
+    double acc = 0.0;
+    if ((M & 3) == 0) {
+      const u64 z = pack2(sh.negz, sh.negz), a2 = pack2(aa, aa), l2 = pack2(a2l, a2l), vi2 = pack2(vi, vi), ui2 = pack2(ui, ui);
 #pragma unroll 2
-    for (int c = lane; c < M4; c += 32) {
-      float4 p = cached ? *reinterpret_cast<const float4*>(psm + rows + r * Mp + 4 * c) : load4(phiy + (size_t)r * M, c, M, v4);
-      const float4 xv = *reinterpret_cast<const float4*>(psm + xo + 4 * c), uv = *reinterpret_cast<const float4*>(psm + yo + 4 * c);
-#define FW_UPD(X)                                                                                  \
-      {                                                                                            \
-        const float vj = xv.X * inv;                                                               \
-        const float wj = __fadd_rn(__fmul_rn(aa, uv.X), __fmul_rn(hl, vj));                         \
-        p.X = __fadd_rn(p.X, __fadd_rn(__fmul_rn(vi, wj), __fmul_rn(wi, vj)));                      \
+      for (int c = lane; c < (M >> 2); c += 32) {
+        float4 p = reinterpret_cast<const float4*>(row)[c];
+        float4 v = *reinterpret_cast<const float4*>(psm + xo + 4 * c);
+        const float4 u = *reinterpret_cast<const float4*>(psm + yo + 4 * c);
+        v.x *= inv; v.y *= inv; v.z *= inv; v.w *= inv;
+        p = rank2(p, vi2, ui2, pack2(v.x, v.y), pack2(v.z, v.w), pack2(u.x, u.y), pack2(u.z, u.w), a2, l2, z);
+        reinterpret_cast<float4*>(row)[c] = p;
+        acc = fma((double)p.x, (double)p.x, acc); acc = fma((double)p.y, (double)p.y, acc);
+        acc = fma((double)p.z, (double)p.z, acc); acc = fma((double)p.w, (double)p.w, acc);
       }
-      FW_UPD(x) FW_UPD(y) FW_UPD(z) FW_UPD(w)
-#undef FW_UPD
-      if (cached) *reinterpret_cast<float4*>(psm + rows + r * Mp + 4 * c) = p;
-      else store4(phiy + (size_t)r * M, c, M, v4, p);
-      const u64 p0 = pack2(p.x, p.y), p1 = pack2(p.z, p.w);
-      fix_add(s, l, p0, p0);
-      fix_add(s, l, p1, p1);
+    } else {
+      for (int c = lane; c < M; c += 32) {
+        const float vj = psm[xo + c] * inv, uj = psm[yo + c];
+        const float p = __fadd_rn(row[c], __fadd_rn(__fmul_rn(aa, __fadd_rn(__fmul_rn(vi, uj), __fmul_rn(ui, vj))),
+                                                    __fmul_rn(a2l, __fmul_rn(vi, vj))));
+        row[c] = p;
+        acc = fma((double)p, (double)p, acc);
+      }
     }
-    float2 acc = fix_value(s, l, C);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc = add2(acc, shfl_xor2(acc, o));
-    if (lane == 0) {
-      const float n2r = acc.x + acc.y;
-      sh.xi2[r] = n2r; sh.xn[r] = sqrtf(n2r);
-      if (send) put(t.xi + row0 + r, n2r, epoch);
-    }
+    new_norm(sh, r, warp_sum(acc), send, epoch);
   }
 }
 
@@ -472,7 +567,6 @@ __device__ __noinline__ void run_layer(const TeamArgs& a, Shared& sh, int li) {
           r < t.ncached ? load4(t.phiy + (size_t)r * M, c, M, v4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     for (int i = tid; i < 2 * Mp; i += PT) psm[i] = 0.f;
-    for (int i = tid; i < kMaxRows; i += PT) sh.xi2[i] = sh.xn[i] = 0.f;
   }
   __syncthreads();
   row_norms(sh, ++e);
@@ -481,19 +575,19 @@ __device__ __noinline__ void run_layer(const TeamArgs& a, Shared& sh, int li) {
   for (int step = 0; step < a.K; ++step) {
     const int mp = receive_argmax(sh, e);
     const int Mp = t.Mp, M = t.M, P = a.P;
-    const bool stream = t.ncached < t.nrows;
+    const bool stream = t.ncached < t.nrows, v4 = (M & 3) == 0;
     const bool keep = a.last && step + 1 == a.K && t.sub == 0;
-    const float2 cw = stream ? correlate<true>(sh, mp, 0, Mp, e + 1, flip, keep)
-                             : correlate<false>(sh, mp, 0, Mp, e + 1, flip, keep);
-    const int cnt = (int)(cw.x + 0.5f);
+    const Aligned al = stream ? (v4 ? correlate<true, true>(sh, mp, 0, Mp, e + 1, keep) : correlate<true, false>(sh, mp, 0, Mp, e + 1, keep))
+                           : (v4 ? correlate<false, true>(sh, mp, 0, Mp, e + 1, keep) : correlate<false, false>(sh, mp, 0, Mp, e + 1, keep));
     // aligned average, P power iterations y = Phi_y (x / ||x||), then u = Phi_y v with v = x / ||x|| (Eqs. 49-50)
+    const int cnt = al.cnt;
     const float inv_cnt = cnt > 0 ? 1.f / (float)cnt : 0.f;
-    const PassOut o = stream ? passes<true>(sh, P + 2, Mp, 0, sqrtf(cw.y), inv_cnt, e + 3, flip)
-                             : passes<false>(sh, P + 2, Mp, 0, sqrtf(cw.y), inv_cnt, e + 3, flip);
+    const PassOut o = stream ? (v4 ? passes<true, true>(sh, P + 2, Mp, 0, al.wnorm, inv_cnt, e + 3, flip) : passes<true, false>(sh, P + 2, Mp, 0, al.wnorm, inv_cnt, e + 3, flip))
+                             : (v4 ? passes<false, true>(sh, P + 2, Mp, 0, al.wnorm, inv_cnt, e + 3, flip) : passes<false, false>(sh, P + 2, Mp, 0, al.wnorm, inv_cnt, e + 3, flip));
     flip ^= P & 1;
     e += (uint32_t)P + 4u;
     const int xo = (P & 1) ? Mp : 0, yo = Mp - xo;               // x and u of the last pass
-    const float inv = inv_norm(o.x2), lam_e = o.xy * inv;          // Eq. 36
+    const float inv = inv_norm(o.x2), lam_e = o.lam;              // Eq. 36
     // ---- g_e, a_e (Eqs. 40-41) ----
     const LayerDev* L = t.L;
     const bool ok = cnt > 0 && o.x2 > 0.f && isfinite(o.x2) && isfinite(lam_e);
@@ -523,7 +617,7 @@ __device__ __noinline__ void run_layer(const TeamArgs& a, Shared& sh, int li) {
     if (more) ++e;
     if (aa != 0.f) {
       updated = true;
-      update_rows(sh, xo, yo, inv, aa, lam_e, o.y2, more, e);
+      update_rows(sh, xo, yo, inv, aa, lam_e, more, e);
     } else if (more) {
       for (int r = tid; r < t.nrows; r += PT) put(t.xi + t.row0 + r, sh.xi2[r], e);
     }
@@ -540,17 +634,18 @@ __device__ __noinline__ void run_layer(const TeamArgs& a, Shared& sh, int li) {
 }
 
 __host__ __device__ inline int team_rows(int M, int n) { return (M + n - 1) / n; }
-// rows that fit beside the two vectors and the partial results, whole groups of four; R: rows per CTA
-constexpr int kPartFloats = 4 * kPartRows * 2;   // float2 each
+// floats of the partial sums; R: rows per CTA.  Pairs of M <= 8192 entries, eight to a partial sum of a norm.
+__host__ __device__ inline int team_part(int M, int R) { return (M & 3) ? 512 : (R <= kPartRows ? 2 * 4 * kPartRows : 0); }
+// rows that fit beside the two vectors and the partial sums, whole groups of four
 __host__ __device__ inline int team_cache(int M, int R) {
   const int Mp = (M + 3) & ~3;
-  return (((int)(kSmem / sizeof(float)) - 2 * Mp - (R <= kPartRows ? kPartFloats : 0)) / Mp) & ~3;
+  return (((int)(kSmem / sizeof(float)) - 2 * Mp - team_part(M, R)) / Mp) & ~3;
 }
 
 __global__ void __launch_bounds__(PT, 1) recursion_team_kernel(const __grid_constant__ TeamArgs a) {
   dep_sync();
   __shared__ Shared sh;
-  if (threadIdx.x == 0) sh.fail = 0;
+  if (threadIdx.x == 0) { sh.fail = 0; sh.negz = -0.f; }
   for (int w = 0; w < a.nwaves; ++w) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -568,10 +663,9 @@ __global__ void __launch_bounds__(PT, 1) recursion_team_kernel(const __grid_cons
         t.row0 = min(M, t.sub * R);
         t.nrows = min(M, t.row0 + R) - t.row0;
         t.phiy = L->Phiy + (size_t)t.row0 * M;
-        const int fit = team_cache(M, R);
-        t.ncached = min(t.nrows, fit);
+        t.ncached = min(t.nrows, team_cache(M, R));
         t.part = 2 * t.Mp;
-        t.rows = 2 * t.Mp + (R <= kPartRows ? kPartFloats : 0);
+        t.rows = t.part + team_part(M, R);
         t.slot = L->px; t.xi = L->px + 2 * packet_stride(M);
         const int groups = (R + 3) / 4;
         t.cg_log = groups <= 4 ? 2 : (R <= kPartRows ? 1 : 0);
