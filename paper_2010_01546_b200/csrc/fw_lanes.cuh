@@ -39,6 +39,13 @@ __device__ __forceinline__ T warp_sum(T x) {
   return x;
 }
 
+// a 2^-896 as fp64: the bits moved into place.  Exact for every finite a, zero and subnormal numbers included.
+__device__ __forceinline__ double widen(float a) {
+  const int b = __float_as_int(a);
+  return __hiloint2double((b >> 3) & 0x8fffffff, b << 29);
+}
+constexpr double kWiden = 0x1p896;
+
 // 1/sqrt(n2) refined by one Newton step, 0 when n2 is not a positive finite number
 __device__ __forceinline__ float inv_norm(float n2) {
   float inv = (n2 > 0.f && isfinite(n2)) ? rsqrtf(n2) : 0.f;

@@ -6,16 +6,16 @@
 // (up to kHist steps) instead of once per step, and the recursion keeps its
 // shared memory for Phi_y.
 //
-//   apply_t   a row of T^T is held in registers; for each step in order
+//   apply_t   a warp holds a row of T^T; for each step in order
 //             t[i] = T^T[i, :] . v,  T^T[i, :] += a t[i] v^T.  Rows are independent.
 //             Every element sees the operations of a step-by-step update in the same order.
 //   apply_q   Q[i][j] += a (a + 2) t[i] t[j], step after step, then (last steps of a call)
 //             the smoothing of Eq. 35.
 //
-// Both are bound by reading and writing their matrix once (L2 or HBM).
+// apply_q is bound by reading and writing its matrix (L2 or HBM), apply_t by its fp64 sums.
+#include <algorithm>
 #include <cstring>
 
-#include "fw_fixsum.cuh"
 #include "fw_internal.h"
 #include "fw_lanes.cuh"
 
@@ -40,21 +40,98 @@ __device__ __forceinline__ int apply_layer(const ApplyArgs& a, int block) {
   return li;
 }
 
-// One row of T^T, NV units of V floats per thread, units `t`, `t` + T, ... of the row for thread t of the T that share it.
-// Bound by issue: the conversions of an fp64 sum (16 per clock and SM) made 64 layers of M = 1152 and eight steps 470 us,
-// now 355.  FIX: the dot product as an anchored sum of two fp32 numbers (where the recursion on Phi_y accumulates in more than fp32);
-// ||v|| = 1, so ||row|| bounds it, and a step adds at most |a t| to that norm.
-template <int NV, int V, bool FIX, bool BLOCK>
-__device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDev* L, int i, int K, float2* red) {
-  constexpr int T = BLOCK ? AT : 32, H = NV * V / 2;
-  const int M = L->M, MU = M / V;
-  const int t = BLOCK ? (int)threadIdx.x : (int)(threadIdx.x & 31);
-  static_assert((NV * V) % 2 == 0 || !FIX, "pairs");
-  float r[NV][V];
-  float* rf = &r[0][0];
+// t[i] is an fp64 sum as the products of the recursion are: a lane takes every 32nd float4 of the row (rows that are not whole
+// float4s: every 32nd entry) in ascending order, then a butterfly over the lanes.  An SM converts 16 numbers per clock to fp64
+// and both factors need it, so the row's are widened by integer operations instead, which holds for
+// finite numbers: `plain` is for rows that are or may become anything else.  64 layers of M = 1152, eight steps: 430 us, of which the
+// conversions alone are 150; sums in fp32 pairs took 350, but some rounded otherwise.
+template <bool PLAIN>
+__device__ __forceinline__ double dot4(float4 r, float4 x, double acc) {
+  if (PLAIN) {
+    acc = fma((double)r.x, (double)x.x, acc); acc = fma((double)r.y, (double)x.y, acc);
+    acc = fma((double)r.z, (double)x.z, acc); acc = fma((double)r.w, (double)x.w, acc);
+  } else {
+    acc = fma(widen(r.x), (double)x.x * kWiden, acc); acc = fma(widen(r.y), (double)x.y * kWiden, acc);
+    acc = fma(widen(r.z), (double)x.z * kWiden, acc); acc = fma(widen(r.w), (double)x.w * kWiden, acc);
+  }
+  return acc;
+}
+__device__ __forceinline__ float4 axpy4(float a, float4 x, float4 r) {
+  return make_float4(fmaf(a, x.x, r.x), fmaf(a, x.y, r.y), fmaf(a, x.z, r.z), fmaf(a, x.w, r.w));
+}
+__device__ __forceinline__ float abs4(float4 r) { return fabsf(r.x) + fabsf(r.y) + fabsf(r.z) + fabsf(r.w); }
+constexpr float kFinite = 1e37f;    // numbers whose absolute values sum to less are finite
+
+// One row of T^T of at most 32 V NV entries in the registers of a warp, in units of V = 4 or 1 floats.
+template <int NV, int V>
+__device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDev* L, int i, int K) {
+  const int M = L->M, MU = M / V, t = threadIdx.x & 31;
+  float4 r4[V == 4 ? NV : 1];
+  float r1[V == 4 ? 1 : NV];
+  float top = 0.f;
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
-    const int c = t + n * T;
+    const int c = t + 32 * n;
+    if (V == 4) {
+      r4[n] = c < MU ? reinterpret_cast<const float4*>(row)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+      top += abs4(r4[n]);
+    } else {
+      r1[n] = c < MU ? row[c] : 0.f;
+    }
+  }
+  bool plain = V == 1 || __any_sync(0xffffffffu, !(top < kFinite));
+  for (int k = 0; k < K; ++k) {
+    const float a = L->ah[k];
+    if (a == 0.f) continue;                        // no step taken (uniform)
+    const float* v = L->vh + (size_t)k * M;
+    // all of v before any of it is used: a load at a time is a chain of latencies
+    float4 x4[V == 4 ? NV : 1];
+    float x1[V == 4 ? 1 : NV];
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      const int c = t + 32 * n;
+      if (V == 4) x4[n] = c < MU ? __ldg(reinterpret_cast<const float4*>(v) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      else x1[n] = c < MU ? __ldg(v + c) : 0.f;
+    }
+    double acc = 0.0;
+    if (V == 1) {
+#pragma unroll
+      for (int n = 0; n < NV; ++n) acc = fma((double)r1[n], (double)x1[n], acc);
+    } else if (plain) {
+#pragma unroll
+      for (int n = 0; n < NV; ++n) acc = dot4<true>(r4[n], x4[n], acc);
+    } else {
+#pragma unroll
+      for (int n = 0; n < NV; ++n) acc = dot4<false>(r4[n], x4[n], acc);
+    }
+    const float ti = (float)warp_sum(acc), ati = a * ti;
+    plain = plain || !(fabsf(ati) < kFinite / kHist);
+    if (t == 0) L->th[(size_t)k * M + i] = ti;
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      if (V == 4) r4[n] = axpy4(ati, x4[n], r4[n]);
+      else r1[n] = fmaf(ati, x1[n], r1[n]);
+    }
+  }
+#pragma unroll
+  for (int n = 0; n < NV; ++n) {
+    const int c = t + 32 * n;
+    if (c >= MU) continue;
+    if (V == 4) reinterpret_cast<float4*>(row)[c] = r4[n];
+    else row[c] = r1[n];
+  }
+}
+// A longer row in the registers of a CTA, at most AT V NV entries.  The sum runs over all threads, in another order; where
+// numbers as close to it as the two orders may be round to different fp32 numbers, the first warp forms the sum of record
+// from a copy of the row in shared memory (`copy`).  rn bounds ||row|| (||v|| = 1, so a step adds at most |a t|); a row that
+// is not finite always takes that way.
+template <int NV, int V>
+__device__ __forceinline__ void long_row_steps(float* __restrict__ row, float* copy, double* red, const LayerDev* L, int i, int K) {
+  const int M = L->M, MU = M / V, t = threadIdx.x;
+  float r[NV][V];
+#pragma unroll
+  for (int n = 0; n < NV; ++n) {
+    const int c = t + AT * n;
 #pragma unroll
     for (int e = 0; e < V; ++e) r[n][e] = 0.f;
     if (c < MU) {
@@ -62,36 +139,30 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
       else r[n][0] = row[c];
     }
   }
-  // sum over the threads of the row
-  auto total = [&](float2 y) {
+  auto total = [&](double y) {
+    y = warp_sum(y);
+    if ((t & 31) == 0) red[t >> 5] = y;
+    __syncthreads();
+    y = red[0];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) y = add2(y, shfl_xor2(y, o));
-    if (BLOCK) {
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = y;
-      __syncthreads();
-      y = red[0];
-#pragma unroll
-      for (int w = 1; w < AWARPS; ++w) y = add2(y, red[w]);
-      __syncthreads();
-    }
+    for (int w = 1; w < AWARPS; ++w) y += red[w];
+    __syncthreads();
     return y;
   };
-  float rn = 0.f;
-  if (FIX) {
-    float q = 0.f;
+  float q = 0.f;
 #pragma unroll
-    for (int n = 0; n < NV * V; ++n) q = fmaf(rf[n], rf[n], q);
-    rn = sqrtf(total(make_float2(q, 0.f)).x);
-  }
+  for (int n = 0; n < NV; ++n)
+#pragma unroll
+    for (int e = 0; e < V; ++e) q = fmaf(r[n][e], r[n][e], q);
+  float rn = 1.01f * sqrtf((float)total((double)q));
   for (int k = 0; k < K; ++k) {
     const float a = L->ah[k];
-    if (a == 0.f) continue;                        // no step taken (uniform)
+    if (a == 0.f) continue;
     const float* v = L->vh + (size_t)k * M;
     float x[NV][V];
-    float* xf = &x[0][0];
 #pragma unroll
     for (int n = 0; n < NV; ++n) {
-      const int c = t + n * T;
+      const int c = t + AT * n;
 #pragma unroll
       for (int e = 0; e < V; ++e) x[n][e] = 0.f;
       if (c < MU) {
@@ -99,29 +170,43 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
         else x[n][0] = __ldg(v + c);
       }
     }
-    float ti;
-    if (FIX) {
-      const float C = anchor(1.01f * rn);
-      u64 s = pack2(C, C), l = 0;
+    double acc = 0.0;
 #pragma unroll
-      for (int h = 0; h < H; ++h) fix_add(s, l, pack2(rf[2 * h], rf[2 * h + 1]), pack2(xf[2 * h], xf[2 * h + 1]));
-      const float2 y = total(fix_value(s, l, C));
-      ti = y.x + y.y;
-    } else {
-      float acc = 0.f;
+    for (int n = 0; n < NV; ++n)
 #pragma unroll
-      for (int n = 0; n < NV * V; ++n) acc = fmaf(rf[n], xf[n], acc);
-      ti = warp_sum(acc);
+      for (int e = 0; e < V; ++e) acc = fma(widen(r[n][e]), (double)x[n][e] * kWiden, acc);
+    double y = total(acc);
+    const double w = (double)rn * 0x1p-50;
+    if ((float)(y - w) != (float)(y + w)) {          // uniform in the CTA
+#pragma unroll
+      for (int n = 0; n < NV; ++n)
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+          if (t + AT * n < MU) copy[V * (t + AT * n) + e] = r[n][e];
+      __syncthreads();
+      if (t < 32) {
+        double z = 0.0;
+        for (int c = t; c < MU; c += 32)
+#pragma unroll
+          for (int e = 0; e < V; ++e) z = fma((double)copy[V * c + e], (double)__ldg(v + V * c + e), z);
+        z = warp_sum(z);
+        if (t == 0) red[0] = z;
+      }
+      __syncthreads();
+      y = red[0];
+      __syncthreads();
     }
-    const float ati = a * ti;
-    if (FIX) rn += fabsf(ati);
+    const float ti = (float)y, ati = a * ti;
+    rn += 1.01f * fabsf(ati);
     if (t == 0) L->th[(size_t)k * M + i] = ti;
 #pragma unroll
-    for (int n = 0; n < NV * V; ++n) rf[n] = fmaf(ati, xf[n], rf[n]);
+    for (int n = 0; n < NV; ++n)
+#pragma unroll
+      for (int e = 0; e < V; ++e) r[n][e] = fmaf(ati, x[n][e], r[n][e]);
   }
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
-    const int c = t + n * T;
+    const int c = t + AT * n;
     if (c < MU) {
       if (V == 4) reinterpret_cast<float4*>(row)[c] = *reinterpret_cast<const float4*>(r[n]);
       else row[c] = r[n][0];
@@ -129,37 +214,31 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
   }
 }
 
-// rows of M <= 1280 take a warp each; longer rows a CTA each
-__global__ void __launch_bounds__(AT) apply_t_kernel(const __grid_constant__ ApplyArgs a) {
+__global__ void __launch_bounds__(AT, 2) apply_t_kernel(const __grid_constant__ ApplyArgs a) {
   dep_sync();
-  __shared__ float2 red[AWARPS];
   const int li = apply_layer(a, (int)blockIdx.x);
   const LayerDev* L = a.g.layer[li];
-  const int M = L->M, K = a.K;
-  const int blk = (int)blockIdx.x - a.block0[li];
-  if (M > kWarpRowMax) {
-    float* row = L->Tt + (size_t)blk * M;
-    if ((M & 3) == 0) {
-      if (M <= 4 * 3 * AT) row_steps<3, 4, true, true>(row, L, blk, K, red);
-      else row_steps<8, 4, true, true>(row, L, blk, K, red);
-    } else {
-      row_steps<32, 1, true, true>(row, L, blk, K, red);
-    }
-    return;
-  }
-  const int i = blk * AWARPS + (threadIdx.x >> 5);
+  const int M = L->M;
+  const int i = ((int)blockIdx.x - a.block0[li]) * AWARPS + (threadIdx.x >> 5);
   if (i >= M) return;
   float* row = L->Tt + (size_t)i * M;
-  if ((M & 3) == 0) {
-    if (M <= 256) row_steps<2, 4, false, false>(row, L, i, K, nullptr);
-    else if (M <= 640) row_steps<5, 4, false, false>(row, L, i, K, nullptr);
-    else row_steps<10, 4, true, false>(row, L, i, K, nullptr);
-  } else {
-    if (M <= 160) row_steps<5, 1, false, false>(row, L, i, K, nullptr);
-    else if (M <= 640) row_steps<20, 1, false, false>(row, L, i, K, nullptr);
-    else row_steps<40, 1, true, false>(row, L, i, K, nullptr);
-  }
+  if ((M & 3) == 0) row_steps<kWarpRowMax / 128, 4>(row, L, i, a.K);
+  else row_steps<kWarpRowMax / 32, 1>(row, L, i, a.K);
 }
+
+template <int NV, int V>
+__global__ void __launch_bounds__(AT, NV == 3 ? 4 : 2) apply_t_long_kernel(const __grid_constant__ ApplyArgs a) {
+  dep_sync();
+  extern __shared__ __align__(16) float copy[];
+  __shared__ double red[AWARPS];
+  const int li = apply_layer(a, (int)blockIdx.x);
+  const LayerDev* L = a.g.layer[li];
+  const int M = L->M, i = (int)blockIdx.x - a.block0[li];
+  long_row_steps<NV, V>(L->Tt + (size_t)i * M, copy, red, L, i, a.K);
+}
+// which kernel takes a layer's T: 0 a warp per row; a CTA per row of whole float4s, up to three or eight per thread, or of
+// single entries.  A kernel each: together they would all have the registers of the largest (16 warps per SM).
+inline int t_kind(int M) { return M <= kWarpRowMax ? 0 : (M & 3) != 0 ? 3 : M <= 4 * 3 * AT ? 1 : 2; }
 
 // A thread takes QR rows of V columns (V = 4, or 1 for rows of odd length) of a layer's Q, whose
 // loads are all in flight together, and takes them through the steps.  Threads are numbered along the
@@ -238,13 +317,24 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
   ApplyArgs a;
   memset(&a, 0, sizeof(a));
   a.g = g; a.K = K; a.smooth = smooth ? 1 : 0;
+  void (*const kernels[])(const ApplyArgs) = {apply_t_kernel, apply_t_long_kernel<3, 4>, apply_t_long_kernel<8, 4>,
+                                              apply_t_long_kernel<32, 1>};
   int n = 0;
-  for (int i = 0; i < g.n; ++i) {
-    a.block0[i] = n;
-    n += layer_M[i] > kWarpRowMax ? layer_M[i] : (layer_M[i] + AWARPS - 1) / AWARPS;
+  for (int kind = 0; kind < 4; ++kind) {
+    int longest = 0;
+    n = 0;
+    for (int i = 0; i < g.n; ++i) {
+      const int M = layer_M[i];
+      a.block0[i] = n;
+      if (t_kind(M) != kind) continue;
+      n += kind ? M : (M + AWARPS - 1) / AWARPS;
+      longest = std::max(longest, M);
+    }
+    a.block0[g.n] = n;
+    if (n == 0) continue;
+    ProfScope ps(FW_PROF_RECUR_UPD, s);
+    launch_dep(kernels[kind], n, AT, kind ? sizeof(float) * longest : 0, s, a);      // at most 32 KB
   }
-  a.block0[g.n] = n;
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(apply_t_kernel, n, AT, 0, s, a); }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   n = 0;

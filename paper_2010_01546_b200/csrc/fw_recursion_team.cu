@@ -68,13 +68,6 @@ __device__ __forceinline__ u64 peek(const u64* p) {
 }
 __device__ __forceinline__ float value_of(u64 w) { return __uint_as_float((uint32_t)w); }
 
-// a 2^-896 as fp64: the bits moved into place.  Exact for every finite a, zero and subnormal numbers included.
-__device__ __forceinline__ double widen(float a) {
-  const int b = __float_as_int(a);
-  return __hiloint2double((b >> 3) & 0x8fffffff, b << 29);
-}
-constexpr double kWiden = 0x1p896;
-
 // Sums over the warp of four values per lane; lane 8 r holds the r-th.
 __device__ __forceinline__ double warp_sum4(double y0, double y1, double y2, double y3) {
   const int lane = threadIdx.x & 31;

@@ -116,6 +116,9 @@ class Reference:
         a2l = a * a * lam
         vi, vj, ui, uj = v[:, None], v[None, :], u[:, None], u[None, :]
         self.Y = Y + (a * (vi * uj + ui * vj) + a2l * (vi * vj))
+        t = self.rows(self.T, v)
+        self.T = self.fma((a * t)[:, None], vj, self.T)
+        self.Q = self.Q + a * (a + 2.0) * (t[:, None] * t[None, :])
         return torch.stack([lam, g, f32(float(cnt)), f32(float(mp))])
 
 
@@ -130,8 +133,32 @@ def test_bits(env, M, K, P):
     L.cond_reduce(K, P, trace)
     want = torch.stack([R.step(P) for _ in range(K)])
     assert torch.equal(trace, want)
-    assert torch.equal(L.get(B.FW_F_PHIY).view(M, M), R.Y)
+    for f, ref in ((B.FW_F_PHIY, R.Y), (B.FW_F_T, R.T.T), (B.FW_F_Q, R.Q)):
+        assert torch.equal(L.get(f).view(M, M), ref)
     assert L.sync_status() == B.FW_OK
+
+
+@pytest.mark.parametrize("M", [640, 1284, 1301, 3076])
+def test_rows_of_t_in_the_order_of_record(env, M):
+    """Rows of T^T whose squares overflow fp32 (no bound on their sums' difference between orders) or that come near its
+    largest number take their sums in the order of record, as rows whose rounding is open do."""
+    torch, B = env
+    Phi = torch.from_numpy(spd32(M, 1e2, M)).cuda()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M)
+    T = torch.eye(M, device="cuda")
+    T[:, 3:6] = torch.randn((M, 3), generator=g, device="cuda") * 1e36
+    L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+    L.set(B.FW_F_PHIX, Phi)
+    L.set(B.FW_F_T, T)
+    L.set(B.FW_F_PHIY, Phi)
+    R = Reference(torch, Phi, L.get(B.FW_F_LAMBDA_BAR)[0], L.desc)
+    R.T = T.T.contiguous()
+    L.cond_reduce(2, 2)
+    for _ in range(2):
+        R.step(2)
+    got = L.get(B.FW_F_T).view(M, M)
+    assert bool(torch.isfinite(got).all()) and torch.equal(got, R.T.T)
 
 
 @pytest.mark.parametrize("bad", [float("inf"), float("nan")])
