@@ -30,6 +30,10 @@
  *    wait that gave up) are kept in a per-layer status word in the layer's own
  *    workspace, read by fw_layer_sync_status; no kernel reports through
  *    process-wide state.
+ *  - Compute calls may be captured into a CUDA graph once a call of the same
+ *    kind has run outside of it.  A replay repeats the choices that were made at
+ *    capture (first block or not, Phi_y stale or not, T still the identity or
+ *    not), so a pass is captured after the first block and the first reduction.
  *  - A layer is not thread-safe.  Calls on different layers are independent;
  *    a grouped call requires all its layers to share one stream.
  *  - There is no CPU fallback: without a CUDA device every compute call

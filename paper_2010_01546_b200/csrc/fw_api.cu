@@ -28,7 +28,6 @@ struct fw_layer {
   bool block_open;     // earlier calls of the current block left their sums in the accumulators (FW_COV_ACCUMULATE)
   bool block_shifted;  // the current block is centred on the pilot mean taken from its first call
   int64_t acc_rows;    // rows accumulated by those calls
-  uint32_t epoch;      // packet exchanges of this layer so far (recursion of large layers)
   float* W;
   float* b;
 };
@@ -329,7 +328,7 @@ fw_status fw_layer_create(const fw_layer_desc* d, void* dev_workspace, size_t by
   L->dev = (LayerDev*)dev_workspace;
   L->have_cov = false; L->first_block = true; L->phiy_stale = true; L->t_identity = true;
   L->shift_zero = false;               // cleared by init_identity, but the first block settles it either way
-  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->epoch = 0;
+  L->block_open = false; L->block_shifted = false; L->acc_rows = 0;
   cudaError_t e = cudaMemcpyAsync(L->dev, &L->h, sizeof(LayerDev), cudaMemcpyHostToDevice, L->stream);
   if (e == cudaSuccess) e = launch_init_identity(L->dev, d->M, L->stream);
   if (e != cudaSuccess) { delete L; return cuda_fail(e, "fw_layer_create"); }
@@ -348,7 +347,7 @@ fw_status fw_layer_reset(fw_layer* L) {
   FW_CUDA(launch_init_identity(L->dev, L->d.M, L->stream), "fw_layer_reset");
   L->have_cov = false; L->first_block = true; L->phiy_stale = true; L->t_identity = true;
   L->shift_zero = true;                // init_identity clears the shift vector
-  L->block_open = false; L->block_shifted = false; L->acc_rows = 0; L->epoch = 0;
+  L->block_open = false; L->block_shifted = false; L->acc_rows = 0;
   return FW_OK;
 }
 
@@ -627,7 +626,6 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
   memset(&tc, 0, sizeof(tc)); memset(&tp, 0, sizeof(tp)); memset(&tl, 0, sizeof(tl));
   gc.n = gp.n = gl.n = 0; gc.pad = gp.pad = gl.pad = 0;
   int dims_c[FW_MAX_GROUP], dims_p[FW_MAX_GROUP], ml = 0, row_blocks = 0;
-  fw_layer* team[FW_MAX_GROUP];
   // largest layers first: CTAs are handed out in launch order, so the long row blocks start early
   int order[FW_MAX_GROUP];
   for (int i = 0; i < n; ++i) order[i] = i;
@@ -643,7 +641,7 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
     } else if (recursion_cluster_supported(M)) {
       gc.layer[gc.n] = l->dev; tc.p[gc.n] = t; dims_c[gc.n] = M; ++gc.n;
     } else {
-      gp.layer[gp.n] = l->dev; tp.p[gp.n] = t; dims_p[gp.n] = M; team[gp.n] = l; ++gp.n;
+      gp.layer[gp.n] = l->dev; tp.p[gp.n] = t; dims_p[gp.n] = M; ++gp.n;
     }
   }
   if (gc.n) FW_CUDA(launch_recursion_cluster(gc, tc, dims_c, K, P, s), "recursion (cluster)");
@@ -652,10 +650,8 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
   // large layers: teams of CTAs; T and Q take the recorded steps, up to kHist at a time
   for (int k0 = 0; k0 < K && gp.n; k0 += kHist) {
     const int kc = std::min(kHist, K - k0);
-    uint32_t epoch[FW_MAX_GROUP];
-    for (int i = 0; i < gp.n; ++i) { epoch[i] = team[i]->epoch; team[i]->epoch += (uint32_t)team_exchanges(kc, P); }
-    FW_CUDA(launch_recursion_team(gp, tp, dims_p, epoch, k0, kc, P, k0 + kc == K, s), "recursion (teams)");
-    FW_CUDA(launch_recursion_apply(gp, dims_p, kc, any_beta && k0 + kc == K, s), "recursion (T, Q)");
+    FW_CUDA(launch_recursion_team(gp, tp, dims_p, k0, kc, P, k0 + kc == K, s), "recursion (teams)");
+    FW_CUDA(launch_recursion_apply(gp, dims_p, kc, any_beta && k0 + kc == K, team_exchanges(kc, P), s), "recursion (T, Q)");
   }
   // leaky layers (their update needs transposed tiles): one launch per pass
   for (int k = 0; k < K && gl.n; ++k)

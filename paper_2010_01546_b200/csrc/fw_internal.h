@@ -81,7 +81,7 @@ constexpr int kCorrEveryStages = 8;   // CTA-pair Gram: one correction MMA per a
 
 
 enum { SC_LAMBDA_BAR = 0, SC_LAMBDA_E = 1, SC_G_E = 2, SC_A_E = 3, SC_LAST_NORM2 = 4, SC_COUNT = 8 };
-enum { IS_MPRIME = 0, IS_SETSIZE = 1, IS_STATUS_NOSUB = 2, IS_STATUS_NONFINITE = 3, IS_STATUS_TIMEOUT = 4, IS_COUNT = 8 };
+enum { IS_MPRIME = 0, IS_SETSIZE = 1, IS_STATUS_NOSUB = 2, IS_STATUS_NONFINITE = 3, IS_STATUS_TIMEOUT = 4, IS_EXCHANGE = 5, IS_COUNT = 8 };
 
 constexpr int kGemvRowsPerBlock = 32;   // rows of a matrix handled by one CTA of a GEMV pass (default shape)
 constexpr int kGemvMinRowsPerBlock = 8; // smallest pass shape: sizes the per-block partial sums
@@ -258,13 +258,15 @@ int recursion_cluster_ctas(int M);
 cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
                                      cudaStream_t s);
 // Steps k0 ... k0 + K - 1 (K <= kHist) of a call for large gamma = 1 layers, as one cooperative launch; v_e, a_e of the
-// steps are left in vh, ah.  epoch[i]: number of the layer's last packet exchange, advanced by team_exchanges(K, P) a
-// launch.  last: the launch ends the call.
+// steps are left in vh, ah.  Its packet exchanges are numbered from the layer's IS_EXCHANGE on, team_exchanges(K, P) of them;
+// the launch only reads that word (CTAs start at different times), launch_recursion_apply advances it.  last: the launch
+// ends the call.
 int team_exchanges(int K, int P);
-cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, const uint32_t* epoch,
-                                  int k0, int K, int P, bool last, cudaStream_t s);
-// T, Q take the K steps recorded in vh, ah (Eqs. 42, 44), in step order; smooth: Qs <- beta Qs + (1 - beta) Q after them
-cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K, bool smooth, cudaStream_t s);
+cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
+                                  bool last, cudaStream_t s);
+// T, Q take the K steps recorded in vh, ah (Eqs. 42, 44), in step order; smooth: Qs <- beta Qs + (1 - beta) Q after them.
+// exchanges: what the team launch used up.
+cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K, bool smooth, int exchanges, cudaStream_t s);
 // zero-padded copies [B][H + 2][W + 2][C] of n NHWC fp32 activations in one launch; dst_floats[i] (a multiple of 4)
 // floats of dst[i] are written in all
 cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, const int* B, const int* H, const int* W,

@@ -30,6 +30,7 @@ struct ApplyArgs {
   GroupDev g;
   int32_t block0[FW_MAX_GROUP + 1];   // first CTA of each layer in the flat grid
   int32_t K, smooth;
+  int32_t exchanges;
 };
 
 __device__ __forceinline__ int apply_layer(const ApplyArgs& a, int block) {
@@ -305,6 +306,7 @@ __global__ void __launch_bounds__(AT) apply_q_kernel(const __grid_constant__ App
   const int units = q_units(M);
   const int64_t idx = (int64_t)((int)blockIdx.x - a.block0[li]) * AT + threadIdx.x;
   const int row0 = (int)(idx / units) * QR, c = (int)(idx % units);
+  if (idx == 0) L->iscal[IS_EXCHANGE] = (int32_t)((uint32_t)L->iscal[IS_EXCHANGE] + (uint32_t)a.exchanges);   // the team launch has ended
   if (row0 >= M) return;
   if ((M & 3) == 0) q_tile<4>(L, row0, c, a.K, a.smooth != 0);
   else q_tile<1>(L, row0, c, a.K, a.smooth != 0);
@@ -312,11 +314,11 @@ __global__ void __launch_bounds__(AT) apply_q_kernel(const __grid_constant__ App
 
 }  // namespace
 
-cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K, bool smooth, cudaStream_t s) {
+cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K, bool smooth, int exchanges, cudaStream_t s) {
   if (K < 1 || K > kHist) return cudaErrorInvalidValue;
   ApplyArgs a;
   memset(&a, 0, sizeof(a));
-  a.g = g; a.K = K; a.smooth = smooth ? 1 : 0;
+  a.g = g; a.K = K; a.smooth = smooth ? 1 : 0; a.exchanges = exchanges;
   void (*const kernels[])(const ApplyArgs) = {apply_t_kernel, apply_t_long_kernel<3, 4>, apply_t_long_kernel<8, 4>,
                                               apply_t_long_kernel<32, 1>};
   int n = 0;

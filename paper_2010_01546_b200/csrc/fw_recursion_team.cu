@@ -16,7 +16,9 @@
 //
 // Two packet slots alternate: a CTA sends exchange e + 1 only after it has received
 // all of e, so nobody still reads e - 1 when its slot is written again.  The row
-// norms have a slot of their own, read again when the coherent set is formed.
+// norms have a slot of their own, read again when the coherent set is formed.  The
+// numbers go on from launch to launch (a layer's IS_EXCHANGE, in device memory: a
+// launch replayed from a captured graph counts on as well).
 //
 // Rounding.  The set of Eq. 48 is a comparison per column and step, and at condition 1e4 a start vector with one column
 // more or less leads to another transform; so every operation is rounded in one stated way, whatever the team:
@@ -49,7 +51,6 @@ struct TeamArgs {
   int32_t wave[FW_MAX_GROUP];        // when a layer runs
   int32_t first[FW_MAX_GROUP];       // its first CTA
   int32_t n[FW_MAX_GROUP];           // its CTAs
-  uint32_t epoch[FW_MAX_GROUP];      // number of the layer's last exchange before this launch
   int32_t k0, K, P, nwaves;
   int32_t last;                      // this launch ends the call
 };
@@ -548,7 +549,7 @@ __device__ __noinline__ void update_rows(Shared& sh, int xo, int yo, float inv, 
 __device__ __noinline__ void run_layer(const TeamArgs& a, Shared& sh, int li) {
   const Team& t = sh.t;
   const int tid = threadIdx.x;
-  uint32_t e = a.epoch[li];
+  uint32_t e = (uint32_t)t.L->iscal[IS_EXCHANGE];              // the layer's last exchange
   int flip = 0;
   {
     // ---- the cached rows into shared memory, zero rows up to whole groups of four ----
@@ -726,8 +727,8 @@ void make_plan(TeamPlan& p, const int* M, int n, int ctas) {
 
 int team_exchanges(int K, int P) { return K * (P + 5); }
 
-cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, const uint32_t* epoch,
-                                  int k0, int K, int P, bool last, cudaStream_t s) {
+cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
+                                  bool last, cudaStream_t s) {
   static int n_sm[64] = {0};
   static SmemAttrCache attr;
   thread_local TeamPlan plan;
@@ -752,7 +753,7 @@ cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, con
   a.g = g; a.traces = traces; a.k0 = k0; a.K = K; a.P = P; a.nwaves = plan.waves; a.last = last ? 1 : 0;
   int ctas = 0;
   for (int i = 0; i < g.n; ++i) {
-    a.wave[i] = plan.wave[i]; a.first[i] = plan.first[i]; a.n[i] = plan.cnt[i]; a.epoch[i] = epoch[i];
+    a.wave[i] = plan.wave[i]; a.first[i] = plan.first[i]; a.n[i] = plan.cnt[i];
     ctas = std::max(ctas, plan.first[i] + plan.cnt[i]);
   }
   void* args[] = {&a};

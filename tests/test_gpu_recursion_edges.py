@@ -110,3 +110,40 @@ def test_team_waves(env):
         L.cond_reduce(2, 4)
         assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), t2n(L.get(B.FW_F_T))) <= TOL_FP32
         assert Ls[i].sync_status() == B.FW_OK
+
+
+@pytest.mark.parametrize("M,K", [(700, 3), (1153, 18), (256, 3)])
+def test_replayed_calls(env, M, K):
+    """A pass replayed from a captured graph goes on from the state the pass before left, as a call does: the packet
+    exchanges of a team carry numbers that must not come again."""
+    torch, B = env
+    X = torch.randn(4, 2 * M, M, device="cuda") * torch.logspace(0, -1, M, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    La, Lb = (B.Layer(M, 4, alpha=0.5, beta=0.2, gamma=1.0, stream=stream.cuda_stream) for _ in range(2))
+    x = X[0].clone()
+    graph = torch.cuda.CUDAGraph()
+
+    def run(L, i):
+        with torch.cuda.stream(stream):
+            x.copy_(X[i])
+            L.cov_update(x)
+            L.cond_reduce(K, 2)
+
+    for i in range(4):
+        run(La, i)
+    for i in range(2):
+        run(Lb, i)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        Lb.cov_update(x)
+        Lb.cond_reduce(K, 2)
+    for i in range(2, 4):
+        with torch.cuda.stream(stream):
+            x.copy_(X[i])
+            graph.replay()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for f in (B.FW_F_PHIX, B.FW_F_T, B.FW_F_Q, B.FW_F_QS, B.FW_F_PHIY, B.FW_F_ALIGN_W):
+            assert torch.equal(La.get(f), Lb.get(f))
+    assert La.sync_status() == Lb.sync_status() == B.FW_OK
