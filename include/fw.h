@@ -222,6 +222,10 @@ fw_status fw_step_momentum(fw_layer* L, float* W, float* b, const float* G_t, co
  *                Ms_hat = round(exp(-sum lbar log lbar)) in [1, M]      (Eqs. 32, 34;
  *                Eq. 32 in the reading that gives M for equal eigenvalues and 1
  *                for a single dominant one, as the text states).
+ * Eigenvalues of at most 1e-13 of the largest are not told from zero (the fp32
+ * Phi_x carries rounding far above that): they have no direction of their own
+ * and share, on the subspace the other eigenvectors leave, the gain of lambda = 0.
+ * With Eq. 10 that gain is 1 / eps, also where eps is smaller than they are.
  * The gradient transform, the step and a later fw_cond_reduce continue from this
  * state.  scratch: caller-owned device memory, 256-byte aligned, at least
  * fw_evd_scratch_bytes(M) bytes per layer, used only during the call's kernels.

@@ -54,3 +54,20 @@ def test_no_full_rank(env, kind):
     Phi = np.triu(Phi) + np.triu(Phi, 1).T
     for g_max in ((0.0, 10.0) if kind != "zero" else (0.0,)):
         whiten(env, Phi, g_max)
+
+
+def test_eigenvalues_not_told_from_zero(env):
+    """Up to 1e-13 of the largest eigenvalue the gain is that of zero, 1 / eps (Eq. 10), whatever eps; above, 1 / lambda."""
+    torch, B = env
+    M = 40
+    lam = np.logspace(0, -11, M)
+    lam[[7, 33]] = 1e-12, 1e-15
+    L = B.Layer(M, 4, beta=0.0, gamma=1.0, eps=1e-18)
+    L.set(B.FW_F_PHIX, torch.from_numpy(np.diag(lam).astype(np.float32)).cuda())
+    scratch, nb = scratch_for(torch, B, M)
+    B.fw_evd_whiten(L.handle, scratch, nb, 0.0)
+    want = 1.0 / np.sqrt(lam)
+    want[33] = 1e9
+    T = t2n(L.get(B.FW_F_T))
+    assert np.abs(np.diag(T) / want - 1.0).max() <= TOL_FP32 and np.abs(T - np.diag(np.diag(T))).max() == 0.0
+    assert L.sync_status() == B.FW_OK
