@@ -699,8 +699,6 @@ void make_plan(TeamPlan& p, const int* M, int n, int ctas) {
       const int fit = std::min(team_cache(M[i], kMaxRows), kMaxRows);
       int need = (M[i] + fit - 1) / fit;
       if (need > ctas) need = ctas;
-      // half the chip is enough for a layer that nearly fits it: two such layers side by side stream a row or two each
-      if (need > ctas / 2 && need <= ctas / 2 + 4) need = ctas / 2;
       if (used + need > ctas) continue;
       in.push_back(i); p.cnt[i] = need; p.wave[i] = w; used += need; done[i] = true; --left;
     }
