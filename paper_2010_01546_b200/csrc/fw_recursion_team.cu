@@ -746,6 +746,8 @@ cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, con
     make_plan(plan, layer_M, g.n, n_sm[dev]);
     plan.dev = dev;
   }
+  for (int i = 0; i < g.n; ++i)      // the tables of a CTA's rows (86 SMs are enough for the largest M)
+    if (team_rows(layer_M[i], plan.cnt[i]) > kMaxRows) return cudaErrorInvalidConfiguration;
   TeamArgs a;
   memset(&a, 0, sizeof(a));
   a.g = g; a.traces = traces; a.k0 = k0; a.K = K; a.P = P; a.nwaves = plan.waves; a.last = last ? 1 : 0;
