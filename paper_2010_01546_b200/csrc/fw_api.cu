@@ -2,6 +2,7 @@
 // Every step of the path runs in the library's own kernels; there is no CPU
 // fallback and no call into another GEMM library.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -229,6 +230,16 @@ const Tuning& tuning() {
     return v;
   }();
   return t;
+}
+int sm_count() {
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return 148; }
+  n = known[dev].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) { cudaGetLastError(); return 148; }
+  known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 void prof_open(int cls, cudaStream_t s) {
   ++g_launches;
@@ -469,10 +480,11 @@ static fw_status cov_update_impl(fw_layer* const* L, int32_t n, const void* cons
       }
       return 16 * lo;
     };
-    int64_t klen = slab_rows(kFfmaResident);
+    const int64_t resident = ffma_resident();
+    int64_t klen = slab_rows(resident);
     int64_t work = 0;
     for (int i : ffma_idx) work += tiles_of(i) * rows[i];
-    if (klen >= 512 && 10 * work < 9 * klen * kFfmaResident) klen = slab_rows(kFfmaResident * 3 / 2);
+    if (klen >= 512 && 10 * work < 9 * klen * resident) klen = slab_rows(resident * 3 / 2);
     GemmGroup gg; gg.n = 0;
     for (int i : ffma_idx) {
       const int M = L[i]->d.M;

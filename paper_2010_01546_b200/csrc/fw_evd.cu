@@ -612,18 +612,9 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
                        int32_t* const* status, const float* eps, bool with_v, float g_max, float* const* T_out,
                        float* const* Q_out, float* const* Y_out, float* const* lam_out, float* const* kappa_out,
                        cudaStream_t s) {
-  static int n_sm[64] = {0};
   static SmemAttrCache attr;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) dev = 0;
-  if (n_sm[dev] == 0) {
-    int v = 0;
-    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    n_sm[dev] = v;
-  }
+  const int sms = sm_count();
+  cudaError_t e = cudaSuccess;
   EvdArgs a;
   FinishArgs f;
   VdvArgs v;
@@ -665,7 +656,7 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
     const int np = l.nb / 2;
     return (double)(l.nb - 1) * ((np + ctas - 1) / ctas) * (600.0 + l.M);
   };
-  for (int used = n; used < n_sm[dev]; ) {
+  for (int used = n; used < sms; ) {
     int w = 0;
     for (int i = 1; i < n; ++i)
       if (cost(a.l[i], a.l[i].n) > cost(a.l[w], a.l[w].n)) w = i;
@@ -673,7 +664,7 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
     const int turns = (np + a.l[w].n - 1) / a.l[w].n;
     if (turns == 1) break;
     const int need = (np + turns - 2) / (turns - 1);             // CTAs for one turn less
-    if (used + need - a.l[w].n > n_sm[dev]) break;
+    if (used + need - a.l[w].n > sms) break;
     used += need - a.l[w].n;
     a.l[w].n = need;
   }

@@ -406,13 +406,14 @@ cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class) {
   // A launch's problems all have the same kind of A.  Groups per tile: an SM holds eight groups of 64 threads (four of
   // 128); with fewer tiles than that the chain of a tile is shared, and below one tile per SM it is what counts, so the
   // groups have 128 threads there.
+  const int sms = sm_count();
   if (!g.p[0].a_kmajor) {
-    if (total >= 4 * 148) return launch_cap<4, false, 1>(g, total, s);
+    if (total >= 4 * sms) return launch_cap<4, false, 1>(g, total, s);
     return launch_cap<4, false, 4>(g, total, s);
   }
-  if (total >= 6 * 148) return launch_cap<8, true, 1>(g, total, s);
-  if (total >= 3 * 148) return launch_cap<8, true, 2>(g, total, s);
-  if (total >= 148) return launch_cap<8, true, 4>(g, total, s);
+  if (total >= 6 * sms) return launch_cap<8, true, 1>(g, total, s);
+  if (total >= 3 * sms) return launch_cap<8, true, 2>(g, total, s);
+  if (total >= sms) return launch_cap<8, true, 4>(g, total, s);
   return launch_cap<4, true, 4>(g, total, s);
 }
 

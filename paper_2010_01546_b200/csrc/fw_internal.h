@@ -225,8 +225,10 @@ struct ProfScope {
 // ---------------------------------------------------------------------------
 // launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
-// CTAs of a launch of the FFMA GEMM that are resident together on a B200 (eight groups of 64 threads per SM)
-constexpr int kFfmaResident = 8 * 148;
+// SMs of the current device (148 on a B200; 148 too where it cannot be asked)
+int sm_count();
+// CTAs of a launch of the FFMA GEMM that are resident together (eight groups of 64 threads per SM)
+inline int ffma_resident() { return 8 * sm_count(); }
 cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class);
 // to_pmean != 0: the means go to the layers' pmean vectors instead of their shift vectors
 cudaError_t launch_pilot_mean(const GroupDev& g, const PtrTable& X, const Rows64& rows, const Rows64& ldx,

@@ -727,23 +727,16 @@ int team_exchanges(int K, int P) { return K * (P + 5); }
 
 cudaError_t launch_recursion_team(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
                                   bool last, cudaStream_t s) {
-  static int n_sm[64] = {0};
   static SmemAttrCache attr;
   thread_local TeamPlan plan;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) dev = 0;
-  if (n_sm[dev] == 0) {
-    int v = 0;
-    e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    n_sm[dev] = v;
-  }
   e = ensure_dyn_smem(recursion_team_kernel, kSmem, attr);
   if (e != cudaSuccess) return e;
   if (plan.dev != dev || plan.n != g.n || memcmp(plan.dims, layer_M, g.n * sizeof(int)) != 0) {
-    make_plan(plan, layer_M, g.n, n_sm[dev]);
+    make_plan(plan, layer_M, g.n, sm_count());
     plan.dev = dev;
   }
   for (int i = 0; i < g.n; ++i)      // the tables of a CTA's rows (86 SMs are enough for the largest M)

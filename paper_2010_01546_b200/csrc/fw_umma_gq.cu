@@ -54,7 +54,6 @@ constexpr int QP_STAGES = 6;
 constexpr int QP_THREADS = 64 + 8 * 32;
 constexpr int QP_SMEM = QP_STAGES * QP_STAGE;
 constexpr int QP_MAX_PROBLEMS = 16;
-constexpr int QP_PAIRS = 74;              // CTA pairs of a full grid
 constexpr int QP_MAX_ITEMS = 1 << 20;    // items of one launch
 constexpr int QP_MAX_KSPLIT = 8;
 
@@ -364,7 +363,8 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     // the search costs the host a fraction of a millisecond: its result is kept per list of shapes
     static std::map<std::vector<int64_t>, std::vector<int>> memo;
     static std::mutex memo_mu;
-    std::vector<int64_t> key;
+    const size_t pairs = std::max(1, sm_count() / 2);              // CTA pairs of a full grid
+    std::vector<int64_t> key(1, (int64_t)pairs);
     for (int i = 0; i < cnt; ++i) {
       const UmmaGqItem& itx = items_in[base + i];
       key.push_back(itx.M); key.push_back(itx.N); key.push_back(itx.part ? itx.part_floats : 0);
@@ -401,8 +401,8 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
           if (ks > 1) extra += 3.0 + (double)(ks + 1) * (double)itx.N * itx.M * 4.0 / 4e6;
         }
         std::sort(costs.begin(), costs.end(), [](double a, double b) { return a > b; });
-        std::vector<double> slot(QP_PAIRS, 0.0);
-        for (size_t c = 0; c < costs.size(); ++c) slot[c % QP_PAIRS] += c < QP_PAIRS ? costs[c] : std::max(4.0, costs[c]);
+        std::vector<double> slot(pairs, 0.0);
+        for (size_t c = 0; c < costs.size(); ++c) slot[c % pairs] += c < pairs ? costs[c] : std::max(4.0, costs[c]);
         const double span = 8.0 + *std::max_element(slot.begin(), slot.end()) + extra;
         if (span < best) { best = span; ks_best = ks_try; }
       }
@@ -454,7 +454,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     g.n = cnt; g.nitems = (int)nitems;
     {
       ProfScope ps(prof_class, s);
-      launch_dep(gq_pair_kernel, 2 * std::min(g.nitems, QP_PAIRS), QP_THREADS, smem, s, g);
+      launch_dep(gq_pair_kernel, 2 * std::min(g.nitems, (int)pairs), QP_THREADS, smem, s, g);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -463,7 +463,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     }
     if (gr.n > 0) {
       int64_t blocks = (gr.total4 + 255) / 256;
-      if (blocks > 148 * 8) blocks = 148 * 8;
+      if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
       ProfScope ps(prof_class, s);
       launch_dep(gq_reduce_kernel, (int)blocks, 256, 0, s, gr);
       e = cudaGetLastError();
