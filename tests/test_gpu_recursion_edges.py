@@ -6,6 +6,7 @@ import pytest
 from oracle import fw_oracle as O
 from paper_2010_01546_b200 import synth
 
+from test_gpu_recursion_rounding import Reference
 from fwtest_util import TOL_FP32, group_reduce_with_replay, oracle_hyper, reduce_with_replay, rel_fro, t2n
 
 pytestmark = pytest.mark.gpu
@@ -65,8 +66,9 @@ def test_groups(env, dims):
         for i in (0, 27, 28, 63):
             L = B.Layer(dims[i], 4, beta=0.0, gamma=1.0)
             L.set(B.FW_F_PHIX, torch.from_numpy(spd32(dims[i], 1e2, 40 + i)).cuda())
-            L.cond_reduce(2, 4)
-            assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), t2n(L.get(B.FW_F_T))) <= TOL_FP32
+            reduce_with_replay(L, Los[i], 2, 4, B, torch)
+            check(Ls[i], Los[i], B)
+            assert torch.equal(Ls[i].get(B.FW_F_T), L.get(B.FW_F_T))
         return
     group_reduce_with_replay(Ls, Los, 2, 4, B, torch)
     for L, Lo in zip(Ls, Los):
@@ -104,12 +106,19 @@ def test_team_waves(env):
     for _ in range(2):
         B.fw_group_cond_reduce([L.handle for L in Ls], 2, 4)
     for i in (0, 6, 7, 8, 10, 11):
+        Phi = torch.from_numpy(spd32(dims[i], 1e2, 40 + i)).cuda()
         L = B.Layer(dims[i], 4, beta=0.0, gamma=1.0)
-        L.set(B.FW_F_PHIX, torch.from_numpy(spd32(dims[i], 1e2, 40 + i)).cuda())
+        L.set(B.FW_F_PHIX, Phi)
         L.cond_reduce(2, 4)
         L.cond_reduce(2, 4)
-        assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), t2n(L.get(B.FW_F_T))) <= TOL_FP32
+        for f in (B.FW_F_T, B.FW_F_Q, B.FW_F_PHIY):       # whatever the team
+            assert torch.equal(Ls[i].get(f), L.get(f))
         assert Ls[i].sync_status() == B.FW_OK
+        if i in (6, 8, 10):                               # and against the operations spelled out (M > 624)
+            R = Reference(torch, Phi, L.get(B.FW_F_LAMBDA_BAR)[0], L.desc)
+            for _ in range(4):
+                R.step(4)
+            assert torch.equal(Ls[i].get(B.FW_F_T), R.T.T)
 
 
 @pytest.mark.parametrize("M,K", [(700, 3), (1153, 18), (256, 3)])
