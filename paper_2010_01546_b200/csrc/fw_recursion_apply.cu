@@ -177,7 +177,7 @@ __device__ __forceinline__ void long_row_steps(float* __restrict__ row, float* c
 #pragma unroll
       for (int e = 0; e < V; ++e) acc = fma(widen(r[n][e]), (double)x[n][e] * kWiden, acc);
     double y = total(acc);
-    const double w = (double)rn * 0x1p-50;
+    const double w = (double)(rn * kOrderWindow);
     if ((float)(y - w) != (float)(y + w)) {          // uniform in the CTA
 #pragma unroll
       for (int n = 0; n < NV; ++n)

@@ -6,13 +6,18 @@
 // Q are not needed by a step: its v_e and a_e are recorded and applied afterwards
 // (fw_recursion_apply.cu).  So a step moves no matrix through HBM, and what bounds
 // it is the chain of P + 5 dependent passes:
-//   - the products themselves: 5 bytes of shared memory an element (four rows share a
-//     load of the vector), so 26 matrix elements per clock and SM; rows that do not fit
-//     are streamed from L2 / HBM instead;
+//   - the products: 5 bytes of shared memory an element (four rows share a load of the
+//     vector), so at most 26 matrix elements per clock and SM; rows that do not fit are
+//     streamed from L2 / HBM instead;
 //   - one exchange per pass through L2.  A result is stored as one 8-byte packet
 //     {value, exchange number}; every CTA of the team polls the packets it needs
 //     until they carry the number it waits for.  No flag, no fence, no barrier
 //     counter: the exchange costs one store and one load latency.
+// Clocks of a pass (clock64 in one CTA; six layers of M = 1152, 48 rows a CTA / one of
+// M = 2304, 16 rows): product 4740 / 3830, block barrier 100 / 110, polling 1500 / 1900,
+// norm and scale 950 / 1300: 7290 = 3.7 us / 7140 = 3.6 us.  The product is about 1800
+// clocks from the first load to the last packet whatever its size, and 108 per four rows
+// by 128 columns and SM partition, where shared memory alone would take 80.
 //
 // Two packet slots alternate: a CTA sends exchange e + 1 only after it has received
 // all of e, so nobody still reads e - 1 when its slot is written again.  The row
@@ -248,11 +253,19 @@ __device__ __noinline__ double exact_row(const Shared& sh, int r, int xo, float 
   const float* row = r < sh.t.ncached ? psm + sh.t.rows + r * sh.t.Mp : sh.t.phiy + (size_t)r * M;
   double acc = 0.0;
   if ((M & 3) == 0) {
-#pragma unroll 4
-    for (int c = lane; c < (M >> 2); c += 32) {
-      const float4 a = reinterpret_cast<const float4*>(row)[c], x = *reinterpret_cast<const float4*>(psm + xo + 4 * c);
-      acc = fma((double)a.x, (double)(x.x * xs), acc); acc = fma((double)a.y, (double)(x.y * xs), acc);
-      acc = fma((double)a.z, (double)(x.z * xs), acc); acc = fma((double)a.w, (double)(x.w * xs), acc);
+    constexpr int B = 9;                           // loads in flight
+    for (int c0 = lane; c0 < (M >> 2); c0 += 32 * B) {
+      float4 a[B];
+#pragma unroll
+      for (int h = 0; h < B; ++h) a[h] = reinterpret_cast<const float4*>(row)[min(c0 + 32 * h, (M >> 2) - 1)];
+#pragma unroll
+      for (int h = 0; h < B; ++h) {
+        const int c = c0 + 32 * h;
+        if (c >= (M >> 2)) break;
+        const float4 x = *reinterpret_cast<const float4*>(psm + xo + 4 * c);
+        acc = fma((double)a[h].x, (double)(x.x * xs), acc); acc = fma((double)a[h].y, (double)(x.y * xs), acc);
+        acc = fma((double)a[h].z, (double)(x.z * xs), acc); acc = fma((double)a[h].w, (double)(x.w * xs), acc);
+      }
     }
   } else {
 #pragma unroll 4
@@ -263,8 +276,9 @@ __device__ __noinline__ double exact_row(const Shared& sh, int r, int xo, float 
 
 // Four rows times xs x, x the vector at offset xo, entries (float4s where V4) c0, c0 + stride, ... of them; lane 8 r returns
 // the r-th row's sum.  CACHED: the rows are in shared memory, Mp apart; else in global memory, M apart, nrows of them.
-// An SM converts 16 numbers per clock to fp64, which alone would bound the product; so three entries in four of a row are
-// widened by integer operations, beside the conversions of the fourth and of x.
+// An SM converts 16 numbers per clock to fp64; so three entries in four of a row are widened by integer operations, beside
+// the conversions of the fourth and of x (clocks of a product, six layers of M = 1152: 4750; 5790 with conversions alone,
+// 4930 with all four widened).
 template <bool CACHED, bool V4, int SHIFT>
 __device__ __forceinline__ double group_product(const float* grow, int row, int nrows, int M, int Mp, int xo, float xs, int c0) {
   constexpr int stride = 32 << SHIFT;
@@ -295,8 +309,8 @@ __device__ __forceinline__ double group_product(const float* grow, int row, int 
   return warp_sum4(acc[0], acc[1], acc[2], acc[3]);
 }
 
-// Whether the fp64 sum y of my row lr, formed in another order, may round to another fp32 number than the sum of record.
-// sh.win[lr] xnorm is what the two sums may differ by (new_norm).
+// Whether the fp64 sum y of my row lr, formed in another order, may round to another fp32 number than the sum of record
+// (about one row in 1e5).  sh.win[lr] xnorm: what the two sums may differ by; infinite for a row that is not finite.
 __device__ __forceinline__ bool open_rounding(const Shared& sh, double y, int lr, float xnorm) {
   const double w = (double)(sh.win[lr] * xnorm);
   return (float)(y - w) != (float)(y + w);
@@ -399,7 +413,7 @@ __device__ __forceinline__ int block_argmax(uint32_t key, uint32_t idx, Shared& 
 __device__ __forceinline__ void new_norm(Shared& sh, int r, double n2, bool send, uint32_t epoch) {
   if ((threadIdx.x & 31) != 0) return;
   sh.xi2[r] = (float)n2;
-  sh.win[r] = n2 == 0.0 ? 0.f : isfinite(n2) ? fmaxf(sqrtf((float)n2), 1e-19f) * 0x1p-50f : INFINITY;
+  sh.win[r] = n2 == 0.0 ? 0.f : isfinite(n2) ? fmaxf(sqrtf((float)n2), 1e-19f) * kOrderWindow : INFINITY;
   if (send) put(sh.t.xi + sh.t.row0 + r, (float)n2, epoch);
 }
 
@@ -678,10 +692,10 @@ struct TeamPlan {
   int32_t wave[FW_MAX_GROUP], first[FW_MAX_GROUP], cnt[FW_MAX_GROUP];
 };
 
-// clocks of a pass on n CTAs: rows in shared memory at 32 elements per clock, streamed rows at about 12
+// what a pass costs on n CTAs, to compare splits: a row from L2 or HBM takes about 2.7 times one in shared memory
 double team_cost(int M, int n) {
   const int R = team_rows(M, n), fit = team_cache(M, R), cached = std::min(R, fit);
-  return ((double)cached / 32 + (double)(R - cached) / 12) * M;
+  return (cached + 2.7 * (R - cached)) * M;
 }
 
 void make_plan(TeamPlan& p, const int* M, int n, int ctas) {
