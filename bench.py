@@ -464,9 +464,9 @@ def measure(ls, steps, warmup, reps, barrier, sampler=None, hold_s=0.0):
 
 
 def team_roofline(us, K, P, m2):
-    """Large layers: Phi_y in the shared memory of a team of SMs; per step P + 4 products and one update pass."""
+    """Large layers: Phi_y in the shared memory of a team of SMs; per step P + 3 products and one update (read and write)."""
     t = us * 1e-6
-    smem = K * (P + 6) * m2
+    smem = K * (P + 5) * m2
     return dict(kernel="recursion_team_kernel (K steps; Phi_y in shared memory as far as it fits, results exchanged through L2)",
                 us_per_step=us, us_per_recursion_step=us / K, smem_gbs=smem / t / 1e9, frac_smem=smem / t / 1e9 / SMEM_PEAK_GBS)
 

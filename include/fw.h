@@ -351,9 +351,10 @@ fw_status fw_profile_end(float* ms_per_class, int64_t* launches_per_class);
  *   FW_GRAM_WAVES_PCT  CTAs of a single-CTA Gram launch in percent of the SM count (default 200: two waves) */
 
 /* 1 when fw_cond_reduce keeps this layer's Phi_y in distributed shared memory
- * for all K steps of a call (small M, gamma = 1), 0 when it streams the state
- * from HBM pass by pass.  Reporting aid: the two paths are bound by different
- * things (latency of dependent passes vs HBM bandwidth). */
+ * for all K steps of a call (M <= 624, gamma = 1); 0 when a team of CTAs keeps it
+ * in shared memory as far as it fits and exchanges results through L2 (larger M,
+ * gamma = 1) or every pass is a launch that reads it from HBM (gamma < 1).
+ * Reporting aid: the paths are bound by different things. */
 int32_t fw_recursion_on_chip(const fw_layer_desc* d);
 
 /* Number of kernels this library has launched since it was loaded. */

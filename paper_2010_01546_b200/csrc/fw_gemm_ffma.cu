@@ -6,8 +6,9 @@
 //
 // A group of 64 threads computes a 64 x 64 tile, 8 x 8 accumulators per thread (packed fp32 pairs: one instruction for two
 // products), from 16-deep slabs copied asynchronously
-// into three shared-memory buffers, where the thread that copied an element subtracts the Gram pass's shift from it.  It is bound by the FP32 pipe when
-// the tiles fill the machine; when they do not, what counts is the length of the chain of slabs, so 2, 4 or 8 groups of a
+// into three shared-memory buffers, where the thread that copied an element subtracts the Gram pass's shift from it.  It is bound by issue and the FP32 pipe when
+// the tiles fill the machine (65536 x 576: pipe busy in 66 % of the cycles, 55 % of its rate in products of the tiles; the
+// rest are the copies that make a pair of one operand, and latencies; shared memory is at 60 % of its wavefronts); when they do not, what counts is the length of the chain of slabs, so 2, 4 or 8 groups of a
 // CTA share the tile, each a contiguous part of K, and their sums are added in order at the end: the chain is that much
 // shorter and the SM has that many more warps to hide it.  Products of the ResNet-20-shaped set at batch 32 (Gram /
 // re-sync / G Qs): 1028 / 310 / 101 us with 4 x 4 accumulators, scalar loads and one group; see launch_gemm_ffma.

@@ -46,7 +46,7 @@ constexpr int CLMAX = 16;          // largest cluster (beyond 8: non-portable si
 constexpr int CT = 512;            // threads per CTA
 constexpr int CW = CT / 32;        // warps per CTA
 constexpr int kMaxIt = 5;          // float4 columns per lane, at most
-constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take the fp64 passes
+constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take teams of CTAs and fp64 sums
 constexpr int KH = 8;              // steps between two updates of T and Q
 constexpr size_t kSmemLimit = 226 * 1024 - 512;   // plus the static variables below: within the 227 KB of a CTA
 

@@ -190,7 +190,7 @@ def test_recursion_stress_condition_number_after_every_step(env, M, cond, K):
     # the recursion stress sweep's corner: condition number 1e6, up to 32 steps of 32 power iterations, the
     # condition number of Phi_y after every step against the oracle's (both evaluated by the oracle's eigenvalue
     # routine in fp64; at 1e6 an fp32 Phi_y carries errors of a tenth of its smallest eigenvalue, hence log10
-    # within 0.1), on chip (M = 256) and through the persistent launch (M = 640)
+    # within 0.1), on chip (M = 256) and through the team launch (M = 640)
     torch, B = env
     Phi, _, _ = synth.spd_with_spectrum(M, cond, synth.layer_seed(5, 7), basis="qr" if M <= 512 else "householder")
     Phi32 = Phi.astype(np.float32); Phi32 = np.triu(Phi32) + np.triu(Phi32, 1).T

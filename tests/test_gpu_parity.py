@@ -168,7 +168,7 @@ def test_bias_compensation(env):
                                         (577, 1e3, 3, 8),      # on chip, 16 CTAs, rows not 16-byte multiples
                                         (620, 1e3, 3, 8),      # on chip, close to the largest resident size
                                         (642, 1e3, 3, 8),      # rows not 16-byte multiples: one launch per pass
-                                        (700, 1e3, 4, 8)])     # persistent launch, rows resident in shared memory
+                                        (700, 1e3, 4, 8)])     # team launch, rows resident in shared memory
 def test_recursion_injected_covariance(env, M, cond, K, P):
     torch, B = env
     Phi, _, _ = synth.spd_with_spectrum(M, cond, 500 + M, basis="qr" if M <= 300 else "householder")
