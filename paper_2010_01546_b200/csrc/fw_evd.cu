@@ -1,8 +1,10 @@
 // Whitening from the eigenvalue decomposition (Sec. 2, Eqs. 7-10; practical gains Eqs. 32 and 34): the method the
 // recursion of Sec. 4 is measured against.  Phi = V Lambda V^T is computed by one-sided block Jacobi rotations in fp64:
-// the columns of W, starting from W = Phi, are rotated until all are orthogonal; then W = Phi V = V Lambda, so the
-// normalised columns of W are the eigenvectors and their lengths the eigenvalues, and V itself is never carried along.
-// Columns are stored as rows (Phi is symmetric), fp64 throughout: T = Phi^(-1/2) carries the rounding of the
+// Phi = R^T R (Cholesky), and the columns of W = R^T Z, starting from Z = I, are rotated until all are orthogonal; then they
+// are V Lambda^(1/2): the normalised columns are the eigenvectors and their squared lengths the eigenvalues, and Z is never
+// carried along.  Where Phi is not (safely) positive definite, W starts from Phi itself and ends as V Lambda, which takes
+// sweeps more: 8 instead of 12 to 13 for the covariances of M = 576 here, 8 instead of 15 at condition 1e3.
+// Columns are stored as rows, fp64 throughout: T = Phi^(-1/2) carries the rounding of the
 // decomposition times cond(Phi) / 2, which fp32 cannot afford.
 //
 // A CTA takes a pair of blocks of 16 columns: the 32 columns' Gram matrix (tensor-core fp64 products, the columns staged
@@ -10,9 +12,10 @@
 // W <- U^T W on the 32 rows.  The block pairs of a round (round-robin tournament) are disjoint, so a layer's CTAs meet
 // once per round, M / 16 - 1 rounds a sweep, instead of once per round of column pairs (M - 1 rounds).  All layers of a
 // group share the launch, each with CTAs and barriers of its own.  A sweep costs 5 / 2 M^3 multiply-adds; what bounds a
-// round at M = 576 (26.5 us: 12.05 ms for 13 sweeps of 35 rounds) is a chain of staging (2), products (8), 31 inner rounds
-// (12) and the barrier (3).  One-sided rotations are those of Hestenes (1958), the
-// tournament of block pairs that of Brent and Luk (1985).
+// round at M = 576 (30.8 us) is a chain, in clocks: staging 3200, Gram products 8000, 31 inner rounds 31400, update 11800,
+// barrier 5500.  The 15 layers of the ResNet-20-shaped set: 12.5 ms from Phi, 9.3 from the factor (0.34 of it the
+// factorisation).  One-sided rotations are those of Hestenes (1958), the start from the Cholesky factor that of Veselic and
+// Hari (1989), the tournament of block pairs that of Brent and Luk (1985).
 //
 // Then T = V diag(sqrt g) V^T (Eq. 9), Q = T^T T = V diag(g) V^T and Phi_y = T Phi T^T = V diag(g lambda) V^T come
 // out of one pass over V.
@@ -51,8 +54,8 @@ constexpr int kPartDoubles = EW / 2 * kTri * 64;
 struct EvdLayer {
   const float* A;    // M x M symmetric input (fp32, row-major)
   double* W;         // M rows of evd_ld(M): row m is column m of Phi V
-  int32_t* words;    // [1] abort, [2 + s] block pairs rotated in sweep s, [kSlots + c] rounds CTA c has finished (zeroed
-                     // before the launch)
+  int32_t* words;    // [0] W came from a factor of Phi, [1] abort, [kSlots + c] barriers CTA c has reached and the last round
+                     // it rotated in (zeroed before the launch)
   int32_t* status;   // time-out word of the layer
   int32_t M;
   int32_t nb;        // blocks of 16 columns, rounded up to even (the tournament's players)
@@ -82,29 +85,39 @@ __device__ __forceinline__ void mma_f64(double (&d)[2], double a, double b) {
 }
 
 // Barrier number idx (from 1) of a layer's CTAs; false once the layer is aborted.  Every CTA raises its own slot and the
-// first warp polls all of them: no chain of atomic additions.  The wait is bounded.
-__device__ bool evd_barrier(const EvdLayer& L, int sub, int idx, int* s_abort) {
+// first warp polls all of them: no chain of atomic additions.  The wait is bounded.  A slot also carries the last round its
+// CTA rotated in, and *s_last is the latest of them: the same in every CTA, since none goes on to barrier idx + 1 unless
+// what it saw at idx was recent enough to go on (and the numbers only grow).
+__device__ bool evd_barrier(const EvdLayer& L, int sub, int idx, int last, int* s_abort, int* s_last) {
   __syncthreads();
   if (threadIdx.x < 32 && *s_abort == 0) {
     volatile int* slots = L.words + kSlots;
     volatile int* ab = L.words + 1;
     if (threadIdx.x == 0) {
       __threadfence();
-      slots[sub] = idx;
+      slots[sub] = (idx << 16) | last;
     }
     bool ok = false;
+    int latest = 0;
     for (uint32_t i = 0; i < kEvdSpin && !ok; ++i) {
       bool here = true;
-      for (int c = threadIdx.x; c < L.n; c += 32) here = here && slots[c] >= idx;
+      latest = 0;
+      for (int c = threadIdx.x; c < L.n; c += 32) {
+        const int v = slots[c];
+        here = here && (v >> 16) >= idx;
+        latest = max(latest, v & 0xffff);
+      }
       ok = __all_sync(0xffffffffu, here);
       if (!ok && (i & 63u) == 63u && *ab != 0) break;
     }
+    latest = __reduce_max_sync(0xffffffffu, latest);
     if (threadIdx.x == 0) {
       if (!ok) {
         *ab = 1;
         atomicExch(L.status, 601);
         *s_abort = 1;
       }
+      *s_last = latest;
       __threadfence();
     }
   }
@@ -134,32 +147,39 @@ extern __shared__ __align__(16) double esm[];
 // Rows of the block pair (I, J): row r of the pair is column I * 16 + r or J * 16 + r - 16 of the layer.
 __device__ __forceinline__ int pair_row(int I, int J, int r) { return r < EB ? I * EB + r : J * EB + r - EB; }
 
-// Entries [k0, k0 + nk) of the pair's rows into shared memory, one bulk copy per row; rows past the matrix and entries
-// past ld are zero.  parity: of the copies' mbarrier.  Returns false when the bounded wait gave up.
-__device__ __forceinline__ bool stage_rows(const EvdLayer& L, int I, int J, int k0, int nk, int stride, uint32_t bar,
-                                           uint32_t parity) {
+// Entries [k0, k0 + nk) of the first nrows rows of the pair (I, J) into shared memory at dst, one bulk copy per row; rows past
+// the matrix and entries past ld are zero.
+__device__ __forceinline__ void stage_issue(const EvdLayer& L, double* dst, int I, int J, int nrows, int k0, int nk, int stride,
+                                            uint32_t bar) {
   const int ld = evd_ld(L.M), have = min(nk, ld - k0);
-  const int rows = max(0, min(EB, L.M - I * EB)) + max(0, min(EB, L.M - J * EB));
+  const int rows = max(0, min(EB, L.M - I * EB)) + (nrows > EB ? max(0, min(EB, L.M - J * EB)) : 0);
   const int tid = threadIdx.x;
   if (tid < 32) {
     asm volatile("fence.proxy.async;" ::: "memory");       // the rows were last written and read by ordinary accesses
     if (tid == 0) sm100::mbar_expect_tx(bar, (uint32_t)rows * (uint32_t)have * 8u);
     __syncwarp();
     const int row = pair_row(I, J, tid);
-    if (row < L.M)
+    if (tid < nrows && row < L.M)
       asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   ::"r"(sm100::smem_u32(esm + tid * stride)), "l"(L.W + (int64_t)row * ld + k0), "r"((uint32_t)have * 8u), "r"(bar)
+                   ::"r"(sm100::smem_u32(dst + tid * stride)), "l"(L.W + (int64_t)row * ld + k0), "r"((uint32_t)have * 8u), "r"(bar)
                    : "memory");
   }
-  if (rows < EP || have < nk) {
-    for (int i = tid; i < EP * nk; i += ET) {
+  if (rows < nrows || have < nk) {
+    for (int i = tid; i < nrows * nk; i += ET) {
       const int r = i / nk, c = i - r * nk;
-      if (pair_row(I, J, r) >= L.M || c >= have) esm[r * stride + c] = 0.0;
+      if (pair_row(I, J, r) >= L.M || c >= have) dst[r * stride + c] = 0.0;
     }
   }
+}
+// Waits for the copies (parity: of their mbarrier) and for the block; false when the bounded wait gave up.
+__device__ __forceinline__ bool stage_wait(uint32_t bar, uint32_t parity) {
   bool ok = false;
   for (uint32_t i = 0; i < sm100::kSpinLimit && !ok; ++i) ok = sm100::mbar_try_wait(bar, parity);
   return __syncthreads_and(ok) != 0;
+}
+__device__ __forceinline__ bool stage_rows(const EvdLayer& L, int I, int J, int k0, int nk, int stride, uint32_t bar, uint32_t parity) {
+  stage_issue(L, esm, I, J, EP, k0, nk, stride, bar);
+  return stage_wait(bar, parity);
 }
 
 // x 2^(127 - e) as fp32, truncated, for e the (biased) fp64 exponent of a number at least as large; 0 when too small
@@ -206,8 +226,200 @@ __device__ __forceinline__ void rotation(double al, double be, double ga, double
   s = (hd + hd) * r;
 }
 
+// ---- Phi = R^T R (R upper triangular), in place in W ----
+// The rows of R are columns of a factor of Phi as the rows of Phi V are of Phi Phi^T = Phi^2: rotated until they are
+// orthogonal they are the eigenvectors too, with lengths sqrt(lambda).  They start closer to orthogonal (the factor's Gram
+// matrix R R^T is one step of the LR iteration on from Phi, and its condition is that of Phi, not of Phi^2).
+constexpr int kRLd = EB + 1;
+constexpr int kOwn = 8;               // block rows of a CTA updated per staging where rows come in chunks
+constexpr double kPivot = 1e-12;      // of max_i Phi_ii: with a pivot below it, Phi is taken as it is
+
+struct Factor {
+  double* R;         // [2][16][kRLd] triangular factors of the diagonal blocks, then [2][16] reciprocals of their diagonals
+  double* P;         // [kOwn][16][kRLd] blocks of the current block row of R
+};
+
+// x <- R_kk^-T x, a column of the block row
+__device__ __forceinline__ void solve_column(double (&x)[EB], const double* R, const double* inv) {
+#pragma unroll
+  for (int j = 0; j < EB; ++j) {
+    x[j] *= inv[j];
+#pragma unroll
+    for (int p = j + 1; p < EB; ++p) x[p] = fma(-R[j * kRLd + p], x[j], x[p]);
+  }
+}
+// columns [c0, c1) of the staged block row
+__device__ __forceinline__ void solve_staged(double* row, int stride, int c0, int c1, const double* R, const double* inv) {
+  for (int c = c0 + (int)threadIdx.x; c < c1; c += ET) {
+    double x[EB];
+#pragma unroll
+    for (int p = 0; p < EB; ++p) x[p] = row[p * stride + c];
+    solve_column(x, R, inv);
+#pragma unroll
+    for (int p = 0; p < EB; ++p) row[p * stride + c] = x[p];
+  }
+}
+// The 16 x 16 diagonal block k <- its triangular factor, one warp, a column per lane; false with a pivot that is too small.
+__device__ __forceinline__ bool factor_diagonal(const EvdLayer& L, int k, double pivot, double* R, double* inv) {
+  const int lane = threadIdx.x & 31, c = lane & (EB - 1), M = L.M, ld = evd_ld(M);
+  double a[EB];
+#pragma unroll
+  for (int r = 0; r < EB; ++r)
+    a[r] = (k * EB + r < M && k * EB + c < M) ? __ldcg(L.W + (int64_t)(k * EB + r) * ld + k * EB + c) : 0.0;
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < EB; ++j) {
+    double d = __shfl_sync(0xffffffffu, a[j], j);
+    if (k * EB + j >= M) d = 1.0;
+    else ok = ok && d > pivot && d <= 1e300;
+    const double q = ok ? rsqrt(d) : 1.0;
+    a[j] *= q;
+#pragma unroll
+    for (int i = j + 1; i < EB; ++i) a[i] = fma(-__shfl_sync(0xffffffffu, a[j], i), a[j], a[i]);
+    if (lane < EB) R[j * kRLd + c] = c >= j ? a[j] : 0.0;
+    if (lane == 0) inv[j] = q;
+  }
+  return ok;
+}
+// W_i -= R_ki^T (block row k of R), columns [c0, c1) of the layer; row: entry c0 of the first staged row; P: R_ki, prow apart.
+__device__ __forceinline__ void update_block_row(const EvdLayer& L, int i, int c0, int c1, const double* row, int stride,
+                                                 const double* P, int prow) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, M = L.M, ld = evd_ld(M);
+  double af[2][4];
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) af[t][q] = -P[(4 * q + (lane & 3)) * prow + 8 * t + (lane >> 2)];
+  const int r0 = i * EB + (lane >> 2);
+#pragma unroll 2
+  for (int c = max(c0, i * EB) + 8 * warp; c < c1; c += 8 * EW) {
+    double2 d[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      d[t] = r0 + 8 * t < M ? __ldcg(reinterpret_cast<const double2*>(L.W + (int64_t)(r0 + 8 * t) * ld + c + 2 * (lane & 3)))
+                            : make_double2(0.0, 0.0);
+    double acc[2][2] = {{d[0].x, d[0].y}, {d[1].x, d[1].y}};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double b = row[(4 * q + (lane & 3)) * stride + c - c0 + (lane >> 2)];
+      mma_f64(acc[0], af[0][q], b);
+      mma_f64(acc[1], af[1][q], b);
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      if (r0 + 8 * t < M)
+        __stcg(reinterpret_cast<double2*>(L.W + (int64_t)(r0 + 8 * t) * ld + c + 2 * (lane & 3)), make_double2(acc[t][0], acc[t][1]));
+  }
+}
+// columns [c0, c1) of the finished rows of block k: zeros, the diagonal factor, the solved columns (row: entry c0)
+__device__ __forceinline__ void write_block_row(const EvdLayer& L, int k, int c0, int c1, const double* row, int stride, const double* R) {
+  const int ld = evd_ld(L.M), half = (c1 - c0) >> 1;
+  for (int i = threadIdx.x; i < EB * half; i += ET) {
+    const int r = i / half, c = c0 + 2 * (i - r * half);
+    if (k * EB + r >= L.M) continue;
+    double2 v = make_double2(0.0, 0.0);
+    if (c >= (k + 1) * EB) v = make_double2(row[r * stride + c - c0], row[r * stride + c - c0 + 1]);
+    else if (c >= k * EB) v = make_double2(R[r * kRLd + c - k * EB], R[r * kRLd + c - k * EB + 1]);
+    __stcg(reinterpret_cast<double2*>(L.W + (int64_t)(k * EB + r) * ld + c), v);
+  }
+}
+
+// Block row k of a step is finished by every CTA for itself (its 16 x 16 factor, then a column per thread) and subtracted
+// from the block rows i > k with i mod n = sub, which are the CTA's own; one barrier a step.  Its owner writes it one step later,
+// when nobody reads the unfinished row any more.  All CTAs see the same pivots and give up at the same step.
+// 1: done; 0: not positive definite (W is spoilt); -1: a wait gave up.
+__device__ __noinline__ int evd_factor(const EvdLayer& L, int sub, double pivot, int nk, int stride, const Factor& f, uint32_t bar,
+                                       uint32_t& parity, int& bidx, int* s_abort, int* s_last) {
+  __shared__ int s_bad;
+  const int M = L.M, ld = evd_ld(M), nblk = (M + EB - 1) / EB, tid = threadIdx.x;
+  const bool whole = ld <= nk;
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+  for (int k = 0; k <= nblk; ++k) {
+    double* row = esm + (k & 1) * EB * stride;
+    double* R = f.R + (k & 1) * EB * kRLd;
+    double* inv = f.R + 2 * EB * kRLd + (k & 1) * EB;
+    const int i0 = k + 1 + (sub + L.n - (k + 1) % L.n) % L.n;      // my first block row after k
+    const bool any = i0 < nblk, owner = k < nblk && k % L.n == sub;
+    const int c0 = k * EB;
+    if (whole && (any || owner)) stage_issue(L, row, k, k, EB, c0, ld - c0, stride, bar);
+    if (k < nblk && tid >= 32 && tid < 64) {
+      const bool ok = factor_diagonal(L, k, pivot, R, inv);
+      if (!ok && tid == 32) s_bad = 1;
+    }
+    if (whole && (any || owner)) {
+      if (!stage_wait(bar, parity)) { evd_give_up(L); return -1; }
+      parity ^= 1;
+    } else {
+      __syncthreads();
+    }
+    if (s_bad) return evd_barrier(L, sub, ++bidx, 0, s_abort, s_last) ? 0 : -1;
+    if (whole) {
+      if (any || owner) solve_staged(row, stride, owner ? EB : (i0 - k) * EB, ld - c0, R, inv);
+      __syncthreads();
+      for (int i = i0; i < nblk; i += L.n) update_block_row(L, i, c0, ld, row, stride, row + (i - k) * EB, stride);
+    } else {
+      for (int i = i0; i < nblk; i += kOwn * L.n) {
+        const int g = tid >> 4, r = tid & (EB - 1), ig = i + g * L.n;
+        if (g < kOwn && ig < nblk) {
+          double x[EB];
+#pragma unroll
+          for (int p = 0; p < EB; ++p) x[p] = ig * EB + r < M ? __ldcg(L.W + (int64_t)(c0 + p) * ld + ig * EB + r) : 0.0;
+          solve_column(x, R, inv);
+#pragma unroll
+          for (int p = 0; p < EB; ++p) f.P[(g * EB + p) * kRLd + r] = x[p];
+        }
+        for (int c = i * EB; c < ld; c += nk) {
+          __syncthreads();                                         // P is written, the chunk before has been read
+          stage_issue(L, row, k, k, EB, c, nk, stride, bar);
+          if (!stage_wait(bar, parity)) { evd_give_up(L); return -1; }
+          parity ^= 1;
+          solve_staged(row, stride, 0, nk, R, inv);
+          __syncthreads();
+          for (int h = 0; h < kOwn && i + h * L.n < nblk; ++h)
+            update_block_row(L, i + h * L.n, c, min(c + nk, ld), row, stride, f.P + h * EB * kRLd, kRLd);
+        }
+        __syncthreads();
+      }
+    }
+    // the block row before, when it is mine: nobody reads it as it was any more
+    if (k > 0 && (k - 1) % L.n == sub) {
+      double* row1 = esm + ((k - 1) & 1) * EB * stride;
+      double* R1 = f.R + ((k - 1) & 1) * EB * kRLd;
+      const double* inv1 = f.R + 2 * EB * kRLd + ((k - 1) & 1) * EB;
+      if (whole) {
+        write_block_row(L, k - 1, 0, c0 - EB, row1, stride, R1);
+        write_block_row(L, k - 1, c0 - EB, ld, row1, stride, R1);
+      } else {
+        for (int c = 0; c < ld; c += nk) {
+          if (c + nk > c0) {
+            __syncthreads();
+            stage_issue(L, row1, k - 1, k - 1, EB, c, nk, stride, bar);
+            if (!stage_wait(bar, parity)) { evd_give_up(L); return -1; }
+            parity ^= 1;
+            solve_staged(row1, stride, max(0, c0 - c), nk, R1, inv1);
+            __syncthreads();
+          }
+          write_block_row(L, k - 1, c, min(c + nk, ld), row1, stride, R1);
+        }
+      }
+    }
+    if (!evd_barrier(L, sub, ++bidx, 0, s_abort, s_last)) return -1;
+  }
+  return 1;
+}
+
+// W = Phi, padded with zeros to whole rows of ld
+__device__ __forceinline__ void evd_load(const EvdLayer& L, int sub) {
+  const int M = L.M, ld = evd_ld(M);
+  for (int64_t i = (int64_t)sub * ET + threadIdx.x; i < (int64_t)M * ld; i += (int64_t)L.n * ET) {
+    const int r = (int)(i / ld), c = (int)(i - (int64_t)r * ld);
+    __stcg(L.W + i, c < M ? (double)L.A[(int64_t)r * M + c] : 0.0);
+  }
+}
+
 __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_last;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ double s_rot[2][EB][2];                              // (c, s) of the 16 pairs of an inner round
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -227,12 +439,8 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
   }
   float dmax = 0.f;
   for (int i = tid; i < M; i += ET) dmax = fmaxf(dmax, fabsf(L.A[(int64_t)i * M + i]));
-  const double floor1 = kFloor * evd_block_max(dmax), floor2 = floor1 * floor1;
-  // W = Phi, padded with zeros to whole rows of ld
-  for (int64_t i = (int64_t)sub * ET + tid; i < (int64_t)M * ld; i += (int64_t)L.n * ET) {
-    const int r = (int)(i / ld), c = (int)(i - (int64_t)r * ld);
-    __stcg(L.W + i, c < M ? (double)L.A[(int64_t)r * M + c] : 0.0);
-  }
+  const double top = evd_block_max(dmax);
+  evd_load(L, sub);
   const int chunks = (ld + kChunk - 1) / kChunk;
   const int nk = chunks == 1 ? ld : kChunk;                       // entries per chunk
   const int stride = evd_stride(nk);
@@ -241,11 +449,23 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
   double* G1 = part;                                              // these two reuse the partial blocks
   double* U = part + EP * kGLd;
   int bidx = 0;
-  if (!evd_barrier(L, sub, ++bidx, &s_abort)) return;
+  if (!evd_barrier(L, sub, ++bidx, 0, &s_abort, &s_last)) return;
+  const Factor f{part, part + 2 * EB * (kRLd + 1)};
+  const int fac = evd_factor(L, sub, kPivot * top, nk, stride, f, bar, parity, bidx, &s_abort, &s_last);
+  if (fac < 0) return;
+  if (fac == 0) {
+    evd_load(L, sub);
+    if (!evd_barrier(L, sub, ++bidx, 0, &s_abort, &s_last)) return;
+  } else if (sub == 0 && tid == 0) {
+    L.words[0] = 1;
+  }
+  // squared length of a column of that is rounding
+  const double floor2 = fac ? kFloor * top : kFloor * top * (kFloor * top);
   const int np = L.nb / 2, n1 = L.nb - 1;
-  for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
-    bool rotated = false;
-    for (int r = 0; r < n1; ++r) {
+  // rounds until a sweep's worth of them in a row has rotated nothing
+  int last = 0;
+  for (int round = 1, r = 0; round <= kMaxSweeps * n1; ++round, r = r + 1 == n1 ? 0 : r + 1) {
+    {
       for (int k = sub; k < np; k += L.n) {
         int I, J;
         if (k == 0) { I = n1; J = r; }
@@ -311,7 +531,7 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
           U[p * kGLd + q] = p == q ? 1.0 : 0.0;
         }
         if (!__syncthreads_or(act)) continue;
-        rotated = true;
+        last = round;
         // ---- one sweep of 2 x 2 rotations on G: a thread of the first half owns the 2 x 2 block of pairs (a, b); the
         //      other half applies each round's rotations to U one round later, off the chain ----
         {
@@ -382,11 +602,9 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
         }
         __syncthreads();                                          // the staged rows are free for the next pair
       }
-      // the sweep's count of rotations is complete before its last barrier
-      if (r == n1 - 1 && tid == 0 && rotated) atomicAdd(L.words + 2 + sweep, 1);
-      if (!evd_barrier(L, sub, ++bidx, &s_abort)) return;
     }
-    if (__ldcg(L.words + 2 + sweep) == 0) break;                  // every pair was already orthogonal
+    if (!evd_barrier(L, sub, ++bidx, last, &s_abort, &s_last)) return;
+    if (round - s_last >= n1) break;                              // every pair is orthogonal
   }
 }
 
@@ -423,8 +641,10 @@ __global__ void __launch_bounds__(256) norm_kernel(const __grid_constant__ Finis
     acc = fma(x, x, acc);
     if (fabs(x) > best) { best = fabs(x); bi = i; }
   }
-  acc = sqrt(warp_sum(acc));
-  if (a.dvec[li]) {
+  acc = warp_sum(acc);
+  const bool factored = L.words[0] != 0;                         // lambda_m = |w_m|^2 > 0
+  if (!factored) acc = sqrt(acc);
+  if (a.dvec[li] && !factored) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const double xo = __shfl_xor_sync(0xffffffffu, best, o);
@@ -462,6 +682,7 @@ __global__ void __launch_bounds__(1024) evd_finish_kernel(const __grid_constant_
   const EvdLayer L = a.l[blockIdx.x];
   const int M = L.M;
   const double* lam = a.lam[blockIdx.x];
+  const bool factored = L.words[0] != 0;
   double x = 0.0;
   for (int m = threadIdx.x; m < M; m += 1024) x += fmax(lam[m], 0.0);
   const double S = block_sum_d(x, red);
@@ -501,7 +722,8 @@ __global__ void __launch_bounds__(1024) evd_finish_kernel(const __grid_constant_
     if (a.lam_sorted[blockIdx.x]) a.lam_sorted[blockIdx.x][rank] = (float)lm;
     if (dv) {
       const double g = gain(lm, rank);
-      const double n2 = zero ? 1.0 : (fabs(lm) <= null ? 0.0 : 1.0 / (lm * lm));            // rows of W are lambda_m v_m
+      // rows of W are lambda_m v_m, or sqrt(lambda_m) v_m where Phi was factored
+      const double n2 = zero ? 1.0 : (fabs(lm) <= null ? 0.0 : 1.0 / (factored ? lm : lm * lm));
       dv[m] = (sqrt(g) - b0) * n2;
       dv[M + m] = (g - b1) * n2;
       dv[2 * M + m] = g * lm * n2;

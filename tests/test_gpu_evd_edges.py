@@ -56,6 +56,45 @@ def test_no_full_rank(env, kind):
         whiten(env, Phi, g_max)
 
 
+@pytest.mark.parametrize("M", [16, 47, 640])
+@pytest.mark.parametrize("kind", ["graded", "singular", "indefinite"])
+def test_start_from_the_factor_or_from_phi(env, M, kind):
+    """Graded matrices (D A D, D powers of two: eigenvalues over eight decades) are factored; one exact dependence, or a
+    negative eigenvalue, and the rotations start from Phi itself."""
+    rng = np.random.default_rng(M)
+    B = rng.standard_normal((M, 2 * M)) / np.sqrt(2 * M)
+    Phi = (B @ B.T).astype(np.float32).astype(np.float64)
+    if kind == "graded":
+        d = 2.0 ** -np.round(np.linspace(0, 13, M))
+        Phi = d[:, None] * Phi * d[None, :]
+    elif kind == "singular":
+        Phi[:, -1] = Phi[:, 0]
+        Phi[-1, :] = Phi[0, :]
+        Phi[-1, -1] = Phi[0, 0]
+    else:
+        Phi[M // 2, M // 2] -= 2.0
+    Phi = np.triu(Phi) + np.triu(Phi, 1).T
+    whiten(env, Phi.astype(np.float32), 3.0)
+
+
+def test_few_ctas_per_long_layer(env):
+    """64 layers of 42 block rows in two chunks each: two CTAs a layer, so more of its own block rows than are updated per
+    staging."""
+    torch, B = env
+    M, n = 657, 64
+    Phis = [spd32(M, 1e2, 40 + i) for i in range(2)]
+    Ls, scr = [], []
+    for i in range(n):
+        L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+        L.set(B.FW_F_PHIX, torch.from_numpy(Phis[i % 2]).cuda())
+        Ls.append(L); scr.append(scratch_for(torch, B, M))
+    B.fw_group_evd_whiten([L.handle for L in Ls], [s[0] for s in scr], [s[1] for s in scr], 0.0)
+    for i in (0, 1, n - 2, n - 1):
+        assert Ls[i].sync_status() == B.FW_OK
+        To, Qo, _, _ = oracle_state(Phis[i % 2], Ls[i].desc.eps, None)
+        assert rel_fro(t2n(Ls[i].get(B.FW_F_T)), To) <= TOL_FP32 and rel_fro(t2n(Ls[i].get(B.FW_F_Q)), Qo) <= TOL_FP32
+
+
 def test_eigenvalues_not_told_from_zero(env):
     """Up to 1e-13 of the largest eigenvalue the gain is that of zero, 1 / eps (Eq. 10), whatever eps; above, 1 / lambda."""
     torch, B = env
