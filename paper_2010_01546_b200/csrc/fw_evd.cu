@@ -7,14 +7,16 @@
 // Columns are stored as rows, fp64 throughout: T = Phi^(-1/2) carries the rounding of the
 // decomposition times cond(Phi) / 2, which fp32 cannot afford.
 //
-// A CTA takes a pair of blocks of 16 columns: the 32 columns' Gram matrix (tensor-core fp64 products, the columns staged
-// in shared memory), one sweep of 2 x 2 rotations on that 32 x 32 matrix in shared memory, accumulated into U, and
-// W <- U^T W on the 32 rows.  The block pairs of a round (round-robin tournament) are disjoint, so a layer's CTAs meet
-// once per round, M / 16 - 1 rounds a sweep, instead of once per round of column pairs (M - 1 rounds).  All layers of a
-// group share the launch, each with CTAs and barriers of its own.  A sweep costs 5 / 2 M^3 multiply-adds; what bounds a
-// round at M = 576 (30.8 us) is a chain, in clocks: staging 3200, Gram products 8000, 31 inner rounds 31400, update 11800,
-// barrier 5500.  The 15 layers of the ResNet-20-shaped set: 12.5 ms from Phi, 9.3 from the factor (0.34 of it the
-// factorisation).  One-sided rotations are those of Hestenes (1958), the start from the Cholesky factor that of Veselic and
+// A CTA takes a pair of blocks of 16 columns: their products (tensor-core fp64, the columns staged in shared memory), one
+// sweep of 2 x 2 rotations on that 32 x 32 matrix in fp32 (Gram32), accumulated into U in fp64, and W <- U^T W on the 32
+// rows.  The block pairs of a round (round-robin tournament) are disjoint, so a layer's CTAs meet
+// once per round, M / 16 - 1 rounds a sweep, instead of once per round of column pairs (M - 1 rounds).  The first round of a
+// sweep rotates all pairs of a visit's 32 columns, the others those of different blocks (visit).  All layers of a
+// group share the launch, each with CTAs and barriers of its own.  What bounds a round at M = 576 (17.9 us) is a chain, in
+// clocks: staging 3200, products 5300, 16 inner rounds 9400 (553 each), update 12200 (9200 at the rate of the fp64 tensor
+// cores), barrier 5000; a round that rotates nothing takes 13500.  The 15 layers of the ResNet-20-shaped set: 12.5 ms from Phi,
+// 9.3 from the factor (0.34 of it the factorisation), 6.8 with inner rounds in fp32 (31 of 1014 clocks before, products
+// 8000).  One-sided rotations are those of Hestenes (1958), the start from the Cholesky factor that of Veselic and
 // Hari (1989), the tournament of block pairs that of Brent and Luk (1985).
 //
 // Then T = V diag(sqrt g) V^T (Eq. 9), Q = T^T T = V diag(g) V^T and Phi_y = T Phi T^T = V diag(g lambda) V^T come
@@ -34,7 +36,7 @@ constexpr int EW = ET / 32;
 constexpr int EB = 16;                // columns per block
 constexpr int EP = 2 * EB;            // columns of a block pair
 constexpr int kChunk = 640;           // entries of a column staged at a time (rows of up to this length stay for both products)
-constexpr int kMaxSweeps = 30;
+constexpr int kMaxSweeps = 60;       // (30000 rounds at the largest M: the barrier packs their number into 16 bits)
 constexpr uint32_t kEvdSpin = 1u << 22;
 constexpr int kSlots = 64;            // of kWords 4-byte words at the start of a layer's scratch
 constexpr int kWords = 256;
@@ -48,8 +50,11 @@ constexpr double kFloor = 1e-14, kNull = 1e-13;
 __host__ __device__ inline int evd_stride(int cols) { return ((cols + 15) & ~15) + 4; }
 __host__ __device__ inline int evd_ld(int M) { return (M + 7) & ~7; }
 constexpr int kGLd = EP + 1;          // leading dimension of the 32 x 32 matrices in shared memory
+constexpr int kGF = 48;                // of the fp32 copies: the two rows of a warp's access lie 16 banks apart
 constexpr int kTri = 10;              // 8 x 8 blocks of the upper triangle of a 32 x 32 matrix
+constexpr int kCross = 4 * 64 + EP;    // partial sums of a warp of a cross visit: four 8 x 8 blocks and 32 squared lengths
 constexpr int kPartDoubles = EW / 2 * kTri * 64;
+static_assert(EW * kCross <= kPartDoubles, "partial sums of cross visits");
 
 struct EvdLayer {
   const float* A;    // M x M symmetric input (fp32, row-major)
@@ -133,15 +138,21 @@ __device__ void evd_give_up(const EvdLayer& L) {
   }
 }
 
-// players of pair k in round q of the tournament of 32
+// players of pair k in inner round q: a tournament of all 32, or (CROSS) of the 16 of one block against those of the other
+template <bool CROSS>
 __device__ __forceinline__ void evd_players(int k, int q, int& p, int& r) {
+  if (CROSS) {
+    p = k;
+    r = EB + ((k + q) & (EB - 1));
+    return;
+  }
   p = q + k; r = q - k;
   if (p >= EP - 1) p -= EP - 1;
   if (r < 0) r += EP - 1;
   if (k == 0) p = EP - 1;
 }
 
-// dynamic shared memory: [32 rows of a chunk][partial Gram blocks of the warps, later the second Gram buffer and U][Gram]
+// dynamic shared memory: [32 rows of a chunk][partial Gram blocks of the warps, later U][Gram]
 extern __shared__ __align__(16) double esm[];
 
 // Rows of the block pair (I, J): row r of the pair is column I * 16 + r or J * 16 + r - 16 of the layer.
@@ -182,13 +193,6 @@ __device__ __forceinline__ bool stage_rows(const EvdLayer& L, int I, int J, int 
   return stage_wait(bar, parity);
 }
 
-// x 2^(127 - e) as fp32, truncated, for e the (biased) fp64 exponent of a number at least as large; 0 when too small
-__device__ __forceinline__ float to_float_scaled(double x, int e) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int ex = ((hi >> 20) & 0x7ff) - e + 127;
-  const uint32_t bits = (uint32_t)(hi & 0x80000000) | ((uint32_t)ex << 23) | (__funnelshift_l((uint32_t)lo, (uint32_t)hi, 3) & 0x007fffffu);
-  return ex > 0 ? __uint_as_float(bits) : 0.f;
-}
 __device__ __forceinline__ float rsqrt_approx(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -199,32 +203,21 @@ __device__ __forceinline__ float rcp_approx(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }       // -127 < e < 128
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// The rotation (c, s) that makes columns p, q orthogonal, from their Gram entries (the smaller of the two angles phi,
-// tan 2 phi = 2 ga / (be - al)); (1, 0) when they are already.  The tangent h of half the angle comes from fp32
-// arithmetic (what the angle misses, 1e-7 of the product, the next sweep sees); c = 2 / (1 + h^2) - 1 and
-// s = 2 h / (1 + h^2), with the reciprocal refined to fp64 rounding, are orthonormal whatever h is.  floor2: squared length of a null column.  This is the chain
-// of an inner round: ten dependent fp64 operations with the 2 x 2 update, no fp64 division or root.
-__device__ __forceinline__ void rotation(double al, double be, double ga, double floor2, double& c, double& s) {
-  const bool act = ga * ga > kOrthTol * kOrthTol * (al * be) && fmin(al, be) > floor2;
-  const double d = be - al;
-  const int e = max((__double2hiint(d) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
-  const float df = fabsf(to_float_scaled(d, e)), gf = to_float_scaled(ga, e);
-  const float g2 = gf + gf;
-  const float ir = rsqrt_approx(fmaf(df, df, g2 * g2));          // 1 / R
-  const float c2 = fmaf(0.5f * df, ir, 0.5f);                    // cos^2 phi
-  const float ic = rsqrt_approx(c2);
-  const float cf = c2 * ic, sf = gf * ir * ic;                   // cos phi, sin phi (up to sign)
-  float h = sf * rcp_approx(1.f + cf);
-  if (d < 0.0) h = -h;
-  if (!act) h = 0.f;
-  const double hd = (double)h, x = fma(hd, hd, 1.0);
-  const double r0 = (double)rcp_approx(fmaf(h, h, 1.f));
-  const double q = fma(-x, r0, 1.0);
-  const double r = fma(r0, fma(q, q, q), r0);
-  c = fma(2.0, r, -1.0);
-  s = (hd + hd) * r;
-}
+// The 32 x 32 Gram matrix for its sweep of rotations, in fp32: the angles need no more, since what an angle misses, 1e-7 of
+// the product, the next visit sees (it starts from fp64 products again), and the rotations that are applied to the columns are
+// orthonormal in fp64 whatever their angle.  Columns are scaled by powers of two to lengths between 1 and 2, so that
+// graded columns keep their products' relative precision; the squared lengths are carried as two numbers, so that the
+// difference of two nearly equal ones, which decides the angle between them, keeps its own.
+struct Gram32 {
+  float g[2][EP][kGF];
+  float hi[2][EP], lo[2][EP];
+  int32_t e[EP];                      // column i is 2^e times its scaled self
+  float h[2][EB];                     // tangents of half the angles of an inner round
+};
+constexpr float kFrozen = 1e-5f;      // a column that has lost this much of its squared length waits for the next visit: its products are rounding
 
 // ---- Phi = R^T R (R upper triangular), in place in W ----
 // The rows of R are columns of a factor of Phi as the rows of Phi V are of Phi Phi^T = Phi^2: rotated until they are
@@ -418,11 +411,244 @@ __device__ __forceinline__ void evd_load(const EvdLayer& L, int sub) {
   }
 }
 
+// A visit to the block pair (I, J).  CROSS: rotations between columns of different blocks only, with the products within a
+// block taken as zero (all but the squared lengths): they were rotated in the sweep's first round, and what they have become
+// since enters only at second order.  That is 4 of 10 blocks of the Gram matrix and 16 of 31 inner rounds, for half a sweep
+// more.  1: rotated; 0: nothing to rotate; -1: a wait gave up.
+template <bool CROSS>
+__device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, int chunks, int stride, double floor2, Gram32& gs,
+                                     uint32_t bar, uint32_t& parity) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, M = L.M, ld = evd_ld(M);
+  double* part = esm + EP * stride;                               // kPartDoubles
+  double* G0 = part + kPartDoubles;
+  double* U = part;                                               // reuses the partial blocks
+  // ---- G = (rows)(rows)^T: each warp a sixteenth of the entries, all blocks that are wanted ----
+  constexpr int NB = CROSS ? 4 : kTri;
+  double acc[NB][2], n2[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int b = 0; b < NB; ++b) acc[b][0] = acc[b][1] = 0.0;
+  for (int ch = 0; ch < chunks; ++ch) {
+    if (ch) __syncthreads();                                // the chunk before has been read
+    if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) return -1;
+    parity ^= 1;
+    const double* w = esm + (lane >> 2) * stride + (lane & 3);
+#pragma unroll 2
+    for (int st = warp; st < nk / 4; st += EW) {
+      double f[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) f[b] = w[8 * b * stride + 4 * st];
+      if (CROSS) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          mma_f64(acc[b], f[b >> 1], f[2 + (b & 1)]);
+          n2[b] = fma(f[b], f[b], n2[b]);
+        }
+      } else {
+        int t = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int c = b; c < 4; ++c) mma_f64(acc[t++], f[b], f[c]);
+      }
+    }
+  }
+  if (CROSS) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      *reinterpret_cast<double2*>(part + warp * kCross + b * 64 + 2 * lane) = make_double2(acc[b][0], acc[b][1]);
+      n2[b] += __shfl_xor_sync(0xffffffffu, n2[b], 1);
+      n2[b] += __shfl_xor_sync(0xffffffffu, n2[b], 2);
+      if ((lane & 3) == 0) part[warp * kCross + 256 + 8 * b + (lane >> 2)] = n2[b];
+    }
+    __syncthreads();
+    if (tid < kCross) {
+      double x = 0.0, y = 0.0;
+#pragma unroll
+      for (int w = 0; w < EW; w += 2) { x += part[w * kCross + tid]; y += part[(w + 1) * kCross + tid]; }
+      x += y;
+      const int b = tid >> 6, e = tid & 63;
+      if (b < 4) G0[(8 * (b >> 1) + (e >> 3)) * kGLd + EB + 8 * (b & 1) + (e & 7)] = x;
+      else G0[e * kGLd + e] = x;
+    }
+  } else {
+    // the second half of the warps hand their sums to the first half, which add to them
+    if (warp >= EW / 2) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b)
+        *reinterpret_cast<double2*>(part + ((warp - EW / 2) * kTri + b) * 64 + 2 * lane) = make_double2(acc[b][0], acc[b][1]);
+    }
+    __syncthreads();
+    if (warp < EW / 2) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        double2* q = reinterpret_cast<double2*>(part + (warp * kTri + b) * 64 + 2 * lane);
+        const double2 o = *q;
+        *q = make_double2(acc[b][0] + o.x, acc[b][1] + o.y);
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < kTri * 64; i += ET) {
+      double x = 0.0;
+#pragma unroll
+      for (int w = 0; w < EW / 2; ++w) x += part[w * kTri * 64 + i];
+      const int b = i >> 6, e = i & 63;
+      const int rb = b < 4 ? 0 : (b < 7 ? 1 : (b < 9 ? 2 : 3)), cb = b - (b < 4 ? 0 : (b < 7 ? 3 : (b < 9 ? 5 : 6)));
+      const int gi = 8 * rb + (e >> 3), gj = 8 * cb + (e & 7);
+      if (rb != cb || gj >= gi) G0[gi * kGLd + gj] = x;
+    }
+  }
+  __syncthreads();
+  // ---- anything to rotate?  the upper triangle, or its cross block ----
+  bool act = false;
+  for (int i = tid; i < EP * EP; i += ET) {
+    const int p = i >> 5, q = i & 31;
+    U[p * kGLd + q] = p == q ? 1.0 : 0.0;
+    if (p > q) continue;
+    const double gp = G0[p * kGLd + p], gq = G0[q * kGLd + q];
+    const bool live = fmin(gp, gq) > floor2;                      // neither is a null column
+    const int ep = (((__double2hiint(gp) >> 20) & 0x7ff) - 1023) >> 1, eq = (((__double2hiint(gq) >> 20) & 0x7ff) - 1023) >> 1;
+    double x = 0.0;
+    if (!CROSS || p == q || (p < EB && q >= EB)) {
+      const double g = G0[p * kGLd + q];
+      act |= p < q && live && g * g > kOrthTol * kOrthTol * (gp * gq);
+      if (live) x = g * pow2d(-ep) * pow2d(-eq);
+    }
+    gs.g[0][p][q] = gs.g[0][q][p] = (float)x;
+    if (p == q) {
+      gs.hi[0][p] = (float)x; gs.lo[0][p] = (float)(x - (double)(float)x);
+      gs.e[p] = live ? ep : 0;
+    }
+  }
+  if (!__syncthreads_or(act)) return 0;
+  // ---- one sweep of 2 x 2 rotations on G: a thread of the first four warps owns the 2 x 2 blocks of pairs (a, b), (a + 8, b);
+  //      the next four apply each round's rotations to U, in fp64, one round later, off the chain; the ninth keeps the squared
+  //      lengths and half-angles ----
+  if (warp < 9) {
+    const int pb = tid & 15, pa = (tid & 127) >> 4;
+    constexpr int kRounds = CROSS ? EB : EP - 1;
+    int jp, jq, ip[2], iq[2], de;
+    auto players = [&](int q) {
+      evd_players<CROSS>(pb, q, jp, jq);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        evd_players<CROSS>(pa + 8 * i, q, ip[i], iq[i]);
+        ip[i] *= kGF; iq[i] *= kGF;
+      }
+      de = min(max(gs.e[jq] - gs.e[jp], -60), 60);
+    };
+    players(0);
+    for (int q = 0; q <= kRounds; ++q) {
+      if (warp < 4 || warp == 8) {
+        if (q < kRounds) {
+          const int z = q & 1;
+          const float* src = &gs.g[z][0][0];
+          float* dst = &gs.g[z ^ 1][0][0];
+          const float al = gs.hi[z][jp], be = gs.hi[z][jq], all = gs.lo[z][jp], bel = gs.lo[z][jq], ga = src[jp * kGF + jq];
+          float g[2][4];
+          int at[2][4];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            at[i][0] = ip[i] + jp; at[i][1] = ip[i] + jq; at[i][2] = iq[i] + jp; at[i][3] = iq[i] + jq;
+            if (warp < 4) {
+#pragma unroll
+              for (int h = 0; h < 4; ++h) g[i][h] = src[at[i][h]];
+            }
+          }
+          const float w = pow2f(de), wi = pow2f(-de);
+          const int kp = jp, kq = jq;
+          players(q + 1);                                                  // of the next round, while the loads are under way
+          // the smaller of the two angles phi, tan 2 phi = 2 ga / (be - al)
+          const float d = (be * w - al * wi) + (bel * w - all * wi);
+          const float g2 = ga + ga, n2 = fmaf(d, d, g2 * g2);
+          const float ir = rsqrt_approx(n2);                               // 1 / R
+          const float c2 = fmaf(0.5f * fabsf(d), ir, 0.5f);                // cos^2 phi
+          const float ic = rsqrt_approx(c2);
+          const bool rot = ga * ga > (float)(kOrthTol * kOrthTol) * (al * be) && fminf(al, be) > kFrozen;
+          const float gs2 = d < 0.f ? -ga : ga;
+          const float cb = rot ? c2 * ic : 1.f;
+          const float sb = rot ? gs2 * ir * ic : 0.f;
+          if (warp < 4) {
+            const float s1 = sb * w, s2 = sb * wi;                         // on scaled columns
+            const float keep = rot ? 0.f : ga;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int a = pa + 8 * i;
+              const float ca = __shfl_sync(0xffffffffu, cb, a), s1a = __shfl_sync(0xffffffffu, s1, a), s2a = __shfl_sync(0xffffffffu, s2, a);
+              const float h00 = cb * g[i][0] - s1 * g[i][1], h01 = s2 * g[i][0] + cb * g[i][1];
+              const float h10 = cb * g[i][2] - s1 * g[i][3], h11 = s2 * g[i][2] + cb * g[i][3];
+              const bool own = a == pb;                                    // its diagonal entries are those in hi, lo
+              dst[at[i][0]] = ca * h00 - s1a * h10; dst[at[i][1]] = own ? keep : ca * h01 - s1a * h11;
+              dst[at[i][2]] = own ? keep : s2a * h00 + ca * h10; dst[at[i][3]] = s2a * h01 + ca * h11;
+            }
+          } else if (lane < EB) {
+            const float t = rot ? 2.f * gs2 * rcp_approx(fmaf(n2, ir, fabsf(d))) : 0.f;      // tan phi, signed
+            const float x0 = -t * ga * w, x1 = t * ga * wi;
+            const float n0 = al + x0, n1 = be + x1, v0 = n0 - al, v1 = n1 - be;
+            gs.hi[z ^ 1][kp] = n0; gs.lo[z ^ 1][kp] = all + ((al - (n0 - v0)) + (x0 - v0));
+            gs.hi[z ^ 1][kq] = n1; gs.lo[z ^ 1][kq] = bel + ((be - (n1 - v1)) + (x1 - v1));
+            gs.h[z][pb] = sb * rcp_approx(1.f + cb);
+          }
+        }
+      } else if (q > 0) {
+        evd_players<CROSS>(pb, q - 1, jp, jq);
+        // c = 2 / (1 + h^2) - 1, s = 2 h / (1 + h^2), the reciprocal refined to fp64 rounding
+        const float h = gs.h[(q - 1) & 1][pb];
+        double x0[4], x1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { x0[i] = U[(pa + 8 * i) * kGLd + jp]; x1[i] = U[(pa + 8 * i) * kGLd + jq]; }
+        const double hd = (double)h, x = fma(hd, hd, 1.0);
+        const double r0 = (double)rcp_approx(fmaf(h, h, 1.f));
+        const double f1 = fma(-x, r0, 1.0);
+        const double rr = fma(r0, fma(f1, f1, f1), r0);
+        const double c = fma(2.0, rr, -1.0), sn = (hd + hd) * rr;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          U[(pa + 8 * i) * kGLd + jp] = c * x0[i] - sn * x1[i];
+          U[(pa + 8 * i) * kGLd + jq] = sn * x0[i] + c * x1[i];
+        }
+      }
+      asm volatile("bar.sync 1, 288;" ::: "memory");
+    }
+  }
+  __syncthreads();
+  // ---- rows <- U^T rows, in place chunk by chunk (a single chunk is still staged) ----
+  // the first half of the warps computes the first 16 rows, the second half the others
+  double uf[2][8];
+  const int half = warp / (EW / 2), wcol = warp - half * (EW / 2);
+#pragma unroll
+  for (int cb = 0; cb < 2; ++cb)
+#pragma unroll
+    for (int kb = 0; kb < 8; ++kb) uf[cb][kb] = U[(4 * kb + (lane & 3)) * kGLd + 16 * half + 8 * cb + (lane >> 2)];
+  for (int ch = 0; ch < chunks; ++ch) {
+    if (chunks > 1) {
+      __syncthreads();
+      if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) return -1;
+      parity ^= 1;
+    }
+#pragma unroll 3
+    for (int b = wcol; b < nk / 8; b += EW / 2) {
+      double bf[8];
+#pragma unroll
+      for (int kb = 0; kb < 8; ++kb) bf[kb] = esm[(4 * kb + (lane & 3)) * stride + 8 * b + (lane >> 2)];
+      const int col = ch * kChunk + 8 * b + 2 * (lane & 3);
+#pragma unroll
+      for (int cb = 0; cb < 2; ++cb) {
+        double d[2] = {0.0, 0.0};
+#pragma unroll
+        for (int kb = 0; kb < 8; ++kb) mma_f64(d, uf[cb][kb], bf[kb]);
+        const int row = pair_row(I, J, 16 * half + 8 * cb + (lane >> 2));
+        if (row < M && col < ld) __stcg(reinterpret_cast<double2*>(L.W + (int64_t)row * ld + col), make_double2(d[0], d[1]));
+      }
+    }
+  }
+  return 1;
+}
+
 __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
   __shared__ int s_abort, s_last;
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ double s_rot[2][EB][2];                              // (c, s) of the 16 pairs of an inner round
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ Gram32 gs;
+  const int tid = threadIdx.x;
   int li = -1;
 #pragma unroll 1
   for (int i = 0; i < a.nl; ++i)
@@ -445,9 +671,6 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
   const int nk = chunks == 1 ? ld : kChunk;                       // entries per chunk
   const int stride = evd_stride(nk);
   double* part = esm + EP * stride;                               // kPartDoubles
-  double* G0 = part + kPartDoubles;
-  double* G1 = part;                                              // these two reuse the partial blocks
-  double* U = part + EP * kGLd;
   int bidx = 0;
   if (!evd_barrier(L, sub, ++bidx, 0, &s_abort, &s_last)) return;
   const Factor f{part, part + 2 * EB * (kRLd + 1)};
@@ -472,134 +695,10 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
         else { I = (r + k) % n1; J = (r - k + n1) % n1; }
         if (I > J) { const int x = I; I = J; J = x; }
         if (I * EB >= M) continue;                                // both blocks past the matrix
-        // ---- G = (rows)(rows)^T: each warp an eighth of the entries, all ten blocks of the upper triangle ----
-        double acc[kTri][2];
-#pragma unroll
-        for (int b = 0; b < kTri; ++b) acc[b][0] = acc[b][1] = 0.0;
-        for (int ch = 0; ch < chunks; ++ch) {
-          if (ch) __syncthreads();                                // the chunk before has been read
-          if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) { evd_give_up(L); return; }
-          parity ^= 1;
-          const double* w = esm + (lane >> 2) * stride + (lane & 3);
-#pragma unroll 2
-          for (int st = warp; st < nk / 4; st += EW) {
-            double f[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) f[b] = w[8 * b * stride + 4 * st];
-            int t = 0;
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-#pragma unroll
-              for (int c = b; c < 4; ++c) mma_f64(acc[t++], f[b], f[c]);
-          }
-        }
-        // the second half of the warps hand their sums to the first half, which add to them
-        if (warp >= EW / 2) {
-#pragma unroll
-          for (int b = 0; b < kTri; ++b)
-            *reinterpret_cast<double2*>(part + ((warp - EW / 2) * kTri + b) * 64 + 2 * lane) = make_double2(acc[b][0], acc[b][1]);
-        }
-        __syncthreads();
-        if (warp < EW / 2) {
-#pragma unroll
-          for (int b = 0; b < kTri; ++b) {
-            double2* q = reinterpret_cast<double2*>(part + (warp * kTri + b) * 64 + 2 * lane);
-            const double2 o = *q;
-            *q = make_double2(acc[b][0] + o.x, acc[b][1] + o.y);
-          }
-        }
-        __syncthreads();
-        for (int i = tid; i < kTri * 64; i += ET) {
-          double x = 0.0;
-#pragma unroll
-          for (int w = 0; w < EW / 2; ++w) x += part[w * kTri * 64 + i];
-          const int b = i >> 6, e = i & 63;
-          const int rb = b < 4 ? 0 : (b < 7 ? 1 : (b < 9 ? 2 : 3)), cb = b - (b < 4 ? 0 : (b < 7 ? 3 : (b < 9 ? 5 : 6)));
-          const int gi = 8 * rb + (e >> 3), gj = 8 * cb + (e & 7);
-          if (rb != cb || gj >= gi) { G0[gi * kGLd + gj] = x; G0[gj * kGLd + gi] = x; }
-        }
-        __syncthreads();
-        // ---- anything to rotate? ----
-        bool act = false;
-        for (int i = tid; i < EP * EP; i += ET) {
-          const int p = i >> 5, q = i & 31;
-          if (p < q) {
-            const double g = G0[p * kGLd + q];
-            const double gp = G0[p * kGLd + p], gq = G0[q * kGLd + q];
-            act |= g * g > kOrthTol * kOrthTol * (gp * gq) && fmin(gp, gq) > floor2;
-          }
-          U[p * kGLd + q] = p == q ? 1.0 : 0.0;
-        }
-        if (!__syncthreads_or(act)) continue;
-        last = round;
-        // ---- one sweep of 2 x 2 rotations on G: a thread of the first half owns the 2 x 2 block of pairs (a, b); the
-        //      other half applies each round's rotations to U one round later, off the chain ----
-        {
-          const int pb = tid & 15, pa = (tid & 255) >> 4;
-          const bool on_g = tid < 256;
-          double* src = G0;
-          double* dst = G1;
-          for (int q = 0; q < EP; ++q) {
-            if (on_g) {
-              if (q < EP - 1) {
-                int ip, iq, jp, jq;
-                evd_players(pa, q, ip, iq);
-                evd_players(pb, q, jp, jq);
-                double cb, sb;
-                rotation(src[jp * kGLd + jp], src[jq * kGLd + jq], src[jp * kGLd + jq], floor2, cb, sb);
-                const double ca = __shfl_sync(0xffffffffu, cb, pa), sa = __shfl_sync(0xffffffffu, sb, pa);
-                if (pa == 0) { s_rot[q & 1][pb][0] = cb; s_rot[q & 1][pb][1] = sb; }
-                const double g00 = src[ip * kGLd + jp], g01 = src[ip * kGLd + jq], g10 = src[iq * kGLd + jp], g11 = src[iq * kGLd + jq];
-                const double h00 = cb * g00 - sb * g01, h01 = sb * g00 + cb * g01;
-                const double h10 = cb * g10 - sb * g11, h11 = sb * g10 + cb * g11;
-                dst[ip * kGLd + jp] = ca * h00 - sa * h10; dst[ip * kGLd + jq] = ca * h01 - sa * h11;
-                dst[iq * kGLd + jp] = sa * h00 + ca * h10; dst[iq * kGLd + jq] = sa * h01 + ca * h11;
-                double* z = src; src = dst; dst = z;
-              }
-            } else if (q > 0) {
-              int jp, jq;
-              evd_players(pb, q - 1, jp, jq);
-              const double cb = s_rot[(q - 1) & 1][pb][0], sb = s_rot[(q - 1) & 1][pb][1];
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                double* u = U + (pa + 16 * h) * kGLd;
-                const double x = u[jp], y = u[jq];
-                u[jp] = cb * x - sb * y; u[jq] = sb * x + cb * y;
-              }
-            }
-            __syncthreads();
-          }
-        }
-        // ---- rows <- U^T rows, in place chunk by chunk (a single chunk is still staged) ----
-        // the first half of the warps computes the first 16 rows, the second half the others
-        double uf[2][8];
-        const int half = warp / (EW / 2), wcol = warp - half * (EW / 2);
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb)
-#pragma unroll
-          for (int kb = 0; kb < 8; ++kb) uf[cb][kb] = U[(4 * kb + (lane & 3)) * kGLd + 16 * half + 8 * cb + (lane >> 2)];
-        for (int ch = 0; ch < chunks; ++ch) {
-          if (chunks > 1) {
-            __syncthreads();
-            if (!stage_rows(L, I, J, ch * kChunk, nk, stride, bar, parity)) { evd_give_up(L); return; }
-            parity ^= 1;
-          }
-#pragma unroll 2
-          for (int b = wcol; b < nk / 8; b += EW / 2) {
-            double bf[8];
-#pragma unroll
-            for (int kb = 0; kb < 8; ++kb) bf[kb] = esm[(4 * kb + (lane & 3)) * stride + 8 * b + (lane >> 2)];
-            const int col = ch * kChunk + 8 * b + 2 * (lane & 3);
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-              double d[2] = {0.0, 0.0};
-#pragma unroll
-              for (int kb = 0; kb < 8; ++kb) mma_f64(d, uf[cb][kb], bf[kb]);
-              const int row = pair_row(I, J, 16 * half + 8 * cb + (lane >> 2));
-              if (row < M && col < ld) __stcg(reinterpret_cast<double2*>(L.W + (int64_t)row * ld + col), make_double2(d[0], d[1]));
-            }
-          }
-        }
+        const int v = r == 0 ? visit<false>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity)
+                             : visit<true>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity);
+        if (v < 0) { evd_give_up(L); return; }
+        if (v > 0) last = round;
         __syncthreads();                                          // the staged rows are free for the next pair
       }
     }

@@ -57,10 +57,11 @@ def test_no_full_rank(env, kind):
 
 
 @pytest.mark.parametrize("M", [16, 47, 640])
-@pytest.mark.parametrize("kind", ["graded", "singular", "indefinite"])
+@pytest.mark.parametrize("kind", ["graded", "singular", "indefinite", "clustered"])
 def test_start_from_the_factor_or_from_phi(env, M, kind):
     """Graded matrices (D A D, D powers of two: eigenvalues over eight decades) are factored; one exact dependence, or a
-    negative eigenvalue, and the rotations start from Phi itself."""
+    negative eigenvalue, and the rotations start from Phi itself.  Clustered: eigenvalues that differ by less than the fp32
+    products of a visit can tell."""
     rng = np.random.default_rng(M)
     B = rng.standard_normal((M, 2 * M)) / np.sqrt(2 * M)
     Phi = (B @ B.T).astype(np.float32).astype(np.float64)
@@ -71,6 +72,9 @@ def test_start_from_the_factor_or_from_phi(env, M, kind):
         Phi[:, -1] = Phi[:, 0]
         Phi[-1, :] = Phi[0, :]
         Phi[-1, -1] = Phi[0, 0]
+    elif kind == "clustered":
+        q, _ = np.linalg.qr(rng.standard_normal((M, M)))
+        Phi = (q * (1.0 + 1e-7 * rng.standard_normal(M) + (np.arange(M) < M // 4))) @ q.T
     else:
         Phi[M // 2, M // 2] -= 2.0
     Phi = np.triu(Phi) + np.triu(Phi, 1).T
