@@ -29,6 +29,7 @@ struct fw_layer {
   bool block_open;     // earlier calls of the current block left their sums in the accumulators (FW_COV_ACCUMULATE)
   bool block_shifted;  // the current block is centred on the pilot mean taken from its first call
   int64_t acc_rows;    // rows accumulated by those calls
+  int device;          // of the workspace
   float* W;
   float* b;
 };
@@ -340,6 +341,8 @@ fw_status fw_layer_create(const fw_layer_desc* d, void* dev_workspace, size_t by
   L->have_cov = false; L->first_block = true; L->phiy_stale = true; L->t_identity = true;
   L->shift_zero = false;               // cleared by init_identity, but the first block settles it either way
   L->block_open = false; L->block_shifted = false; L->acc_rows = 0;
+  cudaPointerAttributes at;
+  L->device = cudaPointerGetAttributes(&at, dev_workspace) == cudaSuccess ? at.device : -1;
   cudaError_t e = cudaMemcpyAsync(L->dev, &L->h, sizeof(LayerDev), cudaMemcpyHostToDevice, L->stream);
   if (e == cudaSuccess) e = launch_init_identity(L->dev, d->M, L->stream);
   if (e != cudaSuccess) { delete L; return cuda_fail(e, "fw_layer_create"); }
@@ -934,6 +937,17 @@ fw_status fw_layer_get(fw_layer* L, fw_field f, void* dev_dst, size_t bytes) {
     FW_CUDA(launch_transpose(L->h.Tt, (float*)dev_dst, L->d.M, L->stream), "get T");
     return FW_OK;
   }
+  // A kernel of ours is set up while the launch before it drains, a copy by the driver is not: 64 matrices of M = 256 in a row
+  // 1.4 us each instead of 3.5 (M = 1152: 225 -> 100 us).  It takes whole floats of this device's own memory; anything else the
+  // driver copies.
+  cudaPointerAttributes at;
+  int dev = -1;
+  if ((reinterpret_cast<uintptr_t>(dev_dst) & 3) == 0 && cudaGetDevice(&dev) == cudaSuccess && dev == L->device &&
+      cudaPointerGetAttributes(&at, dev_dst) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
+    FW_CUDA(launch_copy(src, (float*)dev_dst, (int64_t)(need / sizeof(float)), L->stream), "fw_layer_get");
+    return FW_OK;
+  }
+  cudaGetLastError();
   FW_CUDA(cudaMemcpyAsync(dev_dst, src, need, cudaMemcpyDeviceToDevice, L->stream), "fw_layer_get");
   return FW_OK;
 }

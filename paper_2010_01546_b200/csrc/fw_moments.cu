@@ -6,6 +6,7 @@
 //                  running average into Phix, mirror to the lower triangle
 //   bias_comp      b += W (mu_new - mu_old), carried by extra CTAs of the moments_mat launch
 //   accumulate     a call that leaves its block open: its split sums are added to the block's accumulators
+#include <algorithm>
 #include <cstring>
 
 #include "fw_internal.h"
@@ -392,6 +393,22 @@ __global__ void transpose_kernel(const float* __restrict__ src, float* __restric
   }
 }
 
+// dst <- src, n floats; V4: both 16-byte aligned and whole float4s
+template <bool V4>
+__global__ void __launch_bounds__(256) copy_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t n) {
+  dep_sync();
+  const int64_t step = (int64_t)gridDim.x * 256;
+  if (V4) {
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+    float4* d4 = reinterpret_cast<float4*>(dst);
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < (n >> 2); i += step) d4[i] = s4[i];
+  } else {
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += step) dst[i] = src[i];
+  }
+}
+
 // out = A^T x: 32 columns per CTA, the rows dealt to its 32 warps and their sums added in order
 __global__ void __launch_bounds__(1024) matT_vec_kernel(const float* __restrict__ A, const float* __restrict__ x,
                                                         float* __restrict__ out, int M) {
@@ -587,6 +604,15 @@ cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s
   const int t = (M + 31) / 32;
   ProfScope ps(FW_PROF_MISC, s);
   launch_dep(transpose_kernel, dim3(t, t), dim3(32, 8), 0, s, src, dst, M);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_copy(const float* src, float* dst, int64_t n, cudaStream_t s) {
+  const bool v4 = (n & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
+  const int64_t items = v4 ? n >> 2 : n;
+  const int blocks = (int)std::min<int64_t>((items + 255) / 256, 8 * sm_count());
+  ProfScope ps(FW_PROF_MISC, s);
+  launch_dep(v4 ? copy_kernel<true> : copy_kernel<false>, blocks, 256, 0, s, src, dst, n);
   return cudaGetLastError();
 }
 

@@ -233,3 +233,21 @@ def test_momentum_step_and_whiteness(env):
     with pytest.raises(B.FwError) as e:
         B.fw_step_momentum(L.handle, Wd, bd, Gt, None, vW, vb, 0.05, 0.9, 0.0)     # bias given without its gradient
     assert e.value.status == B.FW_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("M", [1, 5, 32, 33, 258, 1026])
+@pytest.mark.parametrize("offset", [0, 1, 4])
+def test_layer_get_writes_the_field_and_nothing_else(env, M, offset):
+    """Aligned and odd destinations, rows that are whole float4s and rows that are not; what lies around stays."""
+    torch, B = env
+    L = B.Layer(M, 4)
+    A = torch.randn((M, M), device="cuda")
+    A = torch.triu(A) + torch.triu(A, 1).T
+    L.set(B.FW_F_PHIX, A)
+    for field, want in ((B.FW_F_PHIX, A.reshape(-1)), (B.FW_F_Q, torch.eye(M, device="cuda").reshape(-1)),
+                        (B.FW_F_MU, torch.zeros(M, device="cuda"))):
+        n = want.numel()
+        buf = torch.full((n + 9,), 7.0, device="cuda")
+        B.fw_layer_get(L.handle, field, buf[offset:], 4 * n)
+        assert torch.equal(buf[offset:offset + n], want)
+        assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + n:] == 7.0).all())
