@@ -661,50 +661,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
     }
     float* P = pr.gram_part + (int64_t)split * M * M;
     const int q = warp & 3, half = w >> 2;
-    if (pr.im2col) {
-      if (good) {
-        tc_fence_after();
-        for (int o = 0; o < nops; ++o) {
-          int row = ops[o].row0 + q * 32 + lane;
-          {
-            // rows and columns as staged -> rows and columns of the patch matrix; padding columns are dropped
-            // (a group of four staged columns is all real or all padding, and real ones stay adjacent)
-            const int rr_ = (row < M16) ? i2c_col(row, pr.i2c_cpr, pr.i2c_c3) : -1;
-            for (int c0 = 16 * half; c0 < ops[o].n_out; c0 += 32) {
-              uint32_t rv[16];
-              if (have) {
-                tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ops[o].tmem_col + c0), rv);
-                tmem_ld_wait();
-              } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) rv[j] = 0u;
-              }
-              if (rr_ >= 0) {
-#pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                  const int cs = ops[o].col0 + c0 + j;
-                  const int cc = (cs < M16) ? i2c_col(cs, pr.i2c_cpr, pr.i2c_c3) : -1;
-                  if (cc >= 0)
-                    *reinterpret_cast<float4*>(P + (int64_t)rr_ * M + cc) =
-                        make_float4(__uint_as_float(rv[j]), __uint_as_float(rv[j + 1]), __uint_as_float(rv[j + 2]),
-                                    __uint_as_float(rv[j + 3]));
-                }
-              }
-            }
-            if (ops[o].cs_off >= 0 && half == 0) {
-              uint32_t rv[16];
-              if (have) {
-                tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ops[o].tmem_col + ops[o].cs_off), rv);
-                tmem_ld_wait();
-              } else {
-                rv[0] = 0u;
-              }
-              if (rr_ >= 0) pr.colsum_part[(int64_t)split * M + rr_] = __uint_as_float(rv[0]);
-            }
-          }
-        }
-      }
-    } else {
+    {
       // A TMEM lane is a row of the tile, so stores straight from the registers put the 32 lanes of a warp on 32
       // different rows of the output: half-filled sectors, and an SM stores one sector per clock (7 us for a
       // 128 x 256 tile).  The tile goes through shared memory instead (the stages are free: every MMA has completed)
@@ -753,13 +710,44 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
               } else {
                 rr[0] = 0u;
               }
-              if (row < M) pr.colsum_part[(int64_t)split * M + row] = __uint_as_float(rr[0]);
+              const int rc = pr.im2col ? (row < M16 ? i2c_col(row, pr.i2c_cpr, pr.i2c_c3) : -1) : (row < M ? row : -1);
+              if (rc >= 0) pr.colsum_part[(int64_t)split * M + rc] = __uint_as_float(rr[0]);
             }
           }
           asm volatile("bar.sync 1, 256;" ::: "memory");
           // rows of the tile, four at a time per warp: every load of a batch precedes its stores
           const int n4 = n_out >> 2;
           const bool sym = pr.full == 2;
+          if (pr.im2col) {
+            // rows and columns as staged -> rows and columns of the patch matrix; padding columns are dropped (a group of
+            // four staged columns is all real or all padding, and real ones stay adjacent)
+            int cc[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const int cs = col0 + 4 * (lane + 32 * k);
+              cc[k] = lane + 32 * k < n4 && cs < M16 ? i2c_col(cs, pr.i2c_cpr, pr.i2c_c3) : -1;
+            }
+            for (int t0 = w; t0 < 128; t0 += 4 * GR_FIX_WARPS) {
+              if (row0 + t0 >= M16) break;
+              float4 v[4][2];
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                  if (cc[k] >= 0) v[i][k] = *reinterpret_cast<const float4*>(tile + (t0 + i * GR_FIX_WARPS) * TS + 4 * (lane + 32 * k));
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int row = row0 + t0 + i * GR_FIX_WARPS;
+                const int rc = row < M16 ? i2c_col(row, pr.i2c_cpr, pr.i2c_c3) : -1;
+                if (rc < 0) continue;
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                  if (cc[k] >= 0) *reinterpret_cast<float4*>(P + (int64_t)rc * M + cc[k]) = v[i][k];
+              }
+            }
+            if (o + 1 < nops) asm volatile("bar.sync 1, 256;" ::: "memory");
+            continue;
+          }
           for (int t0 = w; t0 < 128; t0 += 4 * GR_FIX_WARPS) {
             if (row0 + t0 >= M) break;
             float4 v[4][3];
