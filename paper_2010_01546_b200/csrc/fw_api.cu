@@ -149,15 +149,18 @@ fw_status resync_phiy(fw_layer* const* L, int n) {
   GemmGroup g1, g2;
   g1.n = g2.n = 0;
   std::vector<UmmaAtbItem> t1, t2, p1, p2;   // single-CTA kernel / CTA-pair kernel, first and second product
+  std::vector<const float*> from;            // copies
+  std::vector<float*> to;
+  std::vector<int64_t> floats;
+  auto add_copy = [&](const float* src, float* dst, int64_t k) { from.push_back(src); to.push_back(dst); floats.push_back(k); };
   for (int i = 0; i < n; ++i) {
     fw_layer* l = L[i];
     if (!l->phiy_stale) continue;
     const int M = l->d.M;
-    const size_t mat = (size_t)M * M * sizeof(float);
     if (l->t_identity) {
-      FW_CUDA(cudaMemcpyAsync(l->h.Phiy, l->h.Phix, mat, cudaMemcpyDeviceToDevice, l->stream), "resync copy");
-      if (l->d.gamma != 1.0f)   // Pt = (T Phix)^T = Phix at T = I
-        FW_CUDA(cudaMemcpyAsync(l->h.tmp, l->h.Phix, mat, cudaMemcpyDeviceToDevice, l->stream), "resync copy Pt");
+      // the first step of a set copies all of its layers: one launch, not a driver copy each
+      add_copy(l->h.Phix, l->h.Phiy, (int64_t)M * M);
+      if (l->d.gamma != 1.0f) add_copy(l->h.Phix, l->h.tmp, (int64_t)M * M);     // Pt = (T Phix)^T = Phix at T = I
     } else if (l->d.prec != FW_PREC_FP32 && umma_available() && M >= 16 && (M % 4) == 0) {
       const bool pair = umma_pair_atb_eligible(M);
       UmmaAtbItem it;
@@ -184,6 +187,8 @@ fw_status resync_phiy(fw_layer* const* L, int n) {
     }
     l->phiy_stale = false;
   }
+  for (size_t i = 0; i < from.size(); i += FW_MAX_GROUP)
+    FW_CUDA(launch_copies((int)std::min<size_t>(from.size() - i, FW_MAX_GROUP), &from[i], &to[i], &floats[i], L[0]->stream), "resync copy");
   if (g1.n) {
     FW_CUDA(launch_gemm_ffma(g1, L[0]->stream, FW_PROF_RESYNC), "resync gemm 1");
     FW_CUDA(launch_gemm_ffma(g2, L[0]->stream, FW_PROF_RESYNC), "resync gemm 2");
@@ -944,7 +949,9 @@ fw_status fw_layer_get(fw_layer* L, fw_field f, void* dev_dst, size_t bytes) {
   int dev = -1;
   if ((reinterpret_cast<uintptr_t>(dev_dst) & 3) == 0 && cudaGetDevice(&dev) == cudaSuccess && dev == L->device &&
       cudaPointerGetAttributes(&at, dev_dst) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
-    FW_CUDA(launch_copy(src, (float*)dev_dst, (int64_t)(need / sizeof(float)), L->stream), "fw_layer_get");
+    float* dst = (float*)dev_dst;
+    const int64_t floats = (int64_t)(need / sizeof(float));
+    FW_CUDA(launch_copies(1, &src, &dst, &floats, L->stream), "fw_layer_get");
     return FW_OK;
   }
   cudaGetLastError();

@@ -275,8 +275,8 @@ cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, c
                             const int* C, const int64_t* dst_floats, cudaStream_t s);
 cudaError_t launch_init_identity(const LayerDev* dev, int M, cudaStream_t s);
 cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s);
-// dst <- src, n floats of this device's memory
-cudaError_t launch_copy(const float* src, float* dst, int64_t n, cudaStream_t s);
+// dst[i] <- src[i], floats[i] floats of this device's memory, n <= FW_MAX_GROUP copies in one launch
+cudaError_t launch_copies(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s);
 // out[j] = sum_k A[k][j] x[k] for a row-major M x M matrix A (A^T x)
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s);
 cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s);

@@ -421,19 +421,32 @@ __global__ void transpose_kernel(const float* __restrict__ src, float* __restric
   }
 }
 
-// dst <- src, n floats; V4: both 16-byte aligned and whole float4s
-template <bool V4>
-__global__ void __launch_bounds__(256) copy_kernel(const float* __restrict__ src, float* __restrict__ dst, int64_t n) {
+// dst <- src, n floats each; the CTAs are dealt to the copies by their sizes.  v4: both 16-byte aligned and whole float4s.
+template <int N>                        // 1 or FW_MAX_GROUP: a KB of parameters costs a launch 0.7 us
+struct CopyGroup {
+  const float* src[N];
+  float* dst[N];
+  int32_t n[N];                         // floats, at most 8192 x 8192
+  int32_t v4[N];
+  int32_t first[N + 1];                 // first CTA of each copy
+  int32_t copies;
+};
+template <int N>
+__global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyGroup<N> g) {
   dep_sync();
-  const int64_t step = (int64_t)gridDim.x * 256;
-  if (V4) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    float4* d4 = reinterpret_cast<float4*>(dst);
+  int c = 0;
+#pragma unroll 1
+  for (int i = 1; i < g.copies; ++i)
+    if ((int)blockIdx.x >= g.first[i]) c = i;
+  const float* src = g.src[c];
+  float* dst = g.dst[c];
+  const int n = g.n[c], step = 256 * (g.first[c + 1] - g.first[c]), i0 = 256 * ((int)blockIdx.x - g.first[c]) + threadIdx.x;
+  if (g.v4[c]) {
 #pragma unroll 4
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < (n >> 2); i += step) d4[i] = s4[i];
+    for (int i = i0; i < (n >> 2); i += step) reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
   } else {
 #pragma unroll 4
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += step) dst[i] = src[i];
+    for (int i = i0; i < n; i += step) dst[i] = src[i];
   }
 }
 
@@ -635,13 +648,26 @@ cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t launch_copy(const float* src, float* dst, int64_t n, cudaStream_t s) {
-  const bool v4 = (n & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
-  const int64_t items = v4 ? n >> 2 : n;
-  const int blocks = (int)std::min<int64_t>((items + 255) / 256, 8 * sm_count());
+template <int N>
+static cudaError_t launch_copies_of(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
+  CopyGroup<N> g;
+  memset(&g, 0, sizeof(g));
+  int64_t total = 0;
+  for (int i = 0; i < n; ++i) total += floats[i];
+  // a 16-byte access a thread, or more where that would be more CTAs than run together
+  const int64_t per_cta = std::max<int64_t>(1024, (total + 8 * sm_count() - 1) / (8 * sm_count()));
+  g.copies = n;
+  for (int i = 0; i < n; ++i) {
+    g.src[i] = src[i]; g.dst[i] = dst[i]; g.n[i] = (int32_t)floats[i];
+    g.v4[i] = (floats[i] & 3) == 0 && ((reinterpret_cast<uintptr_t>(src[i]) | reinterpret_cast<uintptr_t>(dst[i])) & 15) == 0;
+    g.first[i + 1] = g.first[i] + (int)((floats[i] + per_cta - 1) / per_cta);
+  }
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(v4 ? copy_kernel<true> : copy_kernel<false>, blocks, 256, 0, s, src, dst, n);
+  launch_dep(copy_kernel<N>, g.first[n], 256, 0, s, g);
   return cudaGetLastError();
+}
+cudaError_t launch_copies(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
+  return n == 1 ? launch_copies_of<1>(n, src, dst, floats, s) : launch_copies_of<FW_MAX_GROUP>(n, src, dst, floats, s);
 }
 
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s) {

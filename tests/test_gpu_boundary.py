@@ -251,3 +251,20 @@ def test_layer_get_writes_the_field_and_nothing_else(env, M, offset):
         B.fw_layer_get(L.handle, field, buf[offset:], 4 * n)
         assert torch.equal(buf[offset:offset + n], want)
         assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + n:] == 7.0).all())
+
+
+@pytest.mark.parametrize("gamma", [1.0, 0.99])
+def test_first_reduction_copies_every_layer(env, gamma):
+    """T = I: Phi_y = Phi_x bit for bit, for a full group of mixed sizes (a leaky layer copies twice: more copies than one
+    launch takes)."""
+    torch, B = env
+    Ms = [1, 2, 33, 64, 130, 7, 256, 700] * 8
+    Ls, Ps = [], []
+    for i, M in enumerate(Ms):
+        A = torch.randn((M, M), generator=torch.Generator(device="cuda").manual_seed(i), device="cuda")
+        Ps.append(torch.triu(A) + torch.triu(A, 1).T)
+        Ls.append(B.Layer(M, 4, gamma=gamma))
+        Ls[-1].set(B.FW_F_PHIX, Ps[-1])
+    B.fw_group_cond_reduce([L.handle for L in Ls], 0, 0)
+    for L, P in zip(Ls, Ps):
+        assert torch.equal(L.get(B.FW_F_PHIY).reshape(P.shape), P)
