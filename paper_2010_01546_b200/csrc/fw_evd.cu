@@ -644,6 +644,12 @@ __device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, in
   return 1;
 }
 
+// the words of every layer, a CTA each
+__global__ void __launch_bounds__(kWords) evd_clear_kernel(const __grid_constant__ EvdArgs a) {
+  dep_sync();
+  a.l[blockIdx.x].words[threadIdx.x] = 0;
+}
+
 __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
   __shared__ int s_abort, s_last;
   __shared__ __align__(8) uint64_t s_bar;
@@ -843,7 +849,10 @@ struct VdvArgs {
 
 // out_ij = sum_m d_m w_mi w_mj for the three weight vectors at once, on the fp64 tensor cores; a CTA computes a tile of
 // the upper triangle and writes its mirror image too, so the outputs are exactly symmetric.  A warp takes 16 x 32.
-constexpr int VT = 64, VK = 16, kVs = VT + 4;
+// Bound by the fp64 tensor cores (24 products of 8 x 8 x 4 a warp and step); the next two slices of 16 rows are on their way
+// meanwhile.  15 layers of the ResNet-20-shaped set: 202 us, 290 with a slice loaded between two barriers, 109 at the tensor cores' rate.
+constexpr int VT = 64, VK = 16, kVs = VT + 4, VS = 3;
+struct VdvStage { double a[VK][kVs], b[VK][kVs], d[3][VK]; };
 __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArgs a) {
   dep_sync();
   int li = 0;
@@ -854,7 +863,7 @@ __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArg
   const int M = L.M, ld = evd_ld(M);
   int bi, bj;
   tri_decode((int)blockIdx.x - a.tile0[li], (M + VT - 1) / VT, bi, bj);
-  __shared__ __align__(16) double sa[VK][kVs], sb[VK][kVs], sd[3][VK];
+  VdvStage* st = reinterpret_cast<VdvStage*>(esm);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wi = (warp >> 1) * 16, wj = (warp & 1) * 32;         // 4 x 2 warps
   const double* dv = a.dvec[li];
@@ -866,29 +875,46 @@ __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArg
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[o][r][c][0] = acc[o][r][c][1] = 0.0;
   const bool unit = dv[3 * M + 3] != 0.0;                          // Phi = 0: unit vectors
-  for (int m0 = 0; m0 < M && !unit; m0 += VK) {
-    for (int i = tid; i < VK * VT; i += 256) {
-      const int mm = i / VT, c = i - mm * VT;
-      const int gi = bi * VT + c, gj = bj * VT + c;
-      sa[mm][c] = (m0 + mm < M && gi < M) ? L.W[(int64_t)(m0 + mm) * ld + gi] : 0.0;
-      sb[mm][c] = (m0 + mm < M && gj < M) ? L.W[(int64_t)(m0 + mm) * ld + gj] : 0.0;
+  const int slices = unit ? 0 : (M + VK - 1) / VK;
+  // slice s into its stage; rows and columns past the matrix as zeros (an entry past M and below ld is a zero of W)
+  auto load = [&](int s) {
+    if (s < slices) {
+      VdvStage& d = st[s % VS];
+      const int m0 = s * VK;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = tid + 256 * h, mm = i >> 5, c = 2 * (i & 31);
+        const double* w = L.W + (int64_t)min(m0 + mm, M - 1) * ld;
+        const int ca = bi * VT + c, cb = bj * VT + c;
+        const int na = m0 + mm < M && ca < ld ? 16 : 0, nb = m0 + mm < M && cb < ld ? 16 : 0;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm100::smem_u32(&d.a[mm][c])), "l"(w + min(ca, ld - 2)), "r"(na) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sm100::smem_u32(&d.b[mm][c])), "l"(w + min(cb, ld - 2)), "r"(nb) : "memory");
+      }
+      if (tid < 3 * VK) {
+        const int o = tid / VK, mm = tid - o * VK, n = m0 + mm < M ? 8 : 0;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(sm100::smem_u32(&d.d[o][mm])), "l"(dv + o * M + min(m0 + mm, M - 1)), "r"(n) : "memory");
+      }
     }
-    if (tid < 3 * VK) {
-      const int o = tid / VK, mm = tid - o * VK;
-      sd[o][mm] = m0 + mm < M ? dv[o * M + m0 + mm] : 0.0;
-    }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load(0);
+  load(1);
+  for (int s = 0; s < slices; ++s) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();                                               // slice s is here, slice s - 1 has been used
+    load(s + 2);
+    const VdvStage& t = st[s % VS];
 #pragma unroll
     for (int k = 0; k < VK / 4; ++k) {
       const int mm = 4 * k + (lane & 3);
       double af[2], bf[4];
 #pragma unroll
-      for (int r = 0; r < 2; ++r) af[r] = sa[mm][wi + 8 * r + (lane >> 2)];
+      for (int r = 0; r < 2; ++r) af[r] = t.a[mm][wi + 8 * r + (lane >> 2)];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) bf[c] = sb[mm][wj + 8 * c + (lane >> 2)];
+      for (int c = 0; c < 4; ++c) bf[c] = t.b[mm][wj + 8 * c + (lane >> 2)];
 #pragma unroll
       for (int o = 0; o < 3; ++o) {
-        const double d = sd[o][mm];
+        const double d = t.d[o][mm];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           const double ad = af[r] * d;
@@ -897,7 +923,6 @@ __global__ void __launch_bounds__(256) vdv_kernel(const __grid_constant__ VdvArg
         }
       }
     }
-    __syncthreads();
   }
   float* out[3] = {a.T[li], a.Q[li], a.Y[li]};
 #pragma unroll
@@ -967,8 +992,6 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
     const int t = (M + VT - 1) / VT;
     tiles += t * (t + 1) / 2;
     stride = std::max(stride, evd_stride(std::min(evd_ld(M), kChunk)));
-    e = cudaMemsetAsync(l.words, 0, kWords * 4, s);
-    if (e != cudaSuccess) return e;
   }
   f.block0[n] = blocks; v.tile0[n] = tiles;
   a.nl = n; f.nl = n; v.nl = n;
@@ -997,6 +1020,11 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
   e = ensure_dyn_smem(jacobi_kernel, smem, attr);
   if (e != cudaSuccess) return e;
   {
+    ProfScope ps(FW_PROF_MISC, s);
+    e = launch_dep(evd_clear_kernel, n, kWords, 0, s, a);
+    if (e != cudaSuccess) return e;
+  }
+  {
     void* args[] = {&a};
     ProfScope ps(FW_PROF_MISC, s);
     e = cudaLaunchCooperativeKernel((void*)jacobi_kernel, dim3(ctas), dim3(ET), args, smem, s);
@@ -1016,7 +1044,10 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
   if (e != cudaSuccess) return e;
   if (with_v) {
     ProfScope ps(FW_PROF_MISC, s);
-    launch_dep(vdv_kernel, tiles, 256, 0, s, v);
+    static SmemAttrCache vattr;
+    e = ensure_dyn_smem(vdv_kernel, VS * sizeof(VdvStage), vattr);
+    if (e != cudaSuccess) return e;
+    launch_dep(vdv_kernel, tiles, 256, VS * sizeof(VdvStage), s, v);
     e = cudaGetLastError();
   }
   return e;
