@@ -12,10 +12,12 @@
 // CTA share the tile, each a contiguous part of K, and their sums are added in order at the end: the chain is that much
 // shorter and the SM has that many more warps to hide it.  Products of the ResNet-20-shaped set at batch 32 (Gram /
 // re-sync / G Qs): 1028 / 310 / 101 us with 4 x 4 accumulators, scalar loads and one group; see launch_gemm_ffma.
+#include <algorithm>
 #include <cstring>
 
 #include "fw_internal.h"
 #include "fw_lanes.cuh"
+#include "fw_sm100.cuh"
 
 namespace fw {
 
@@ -43,6 +45,17 @@ __device__ __forceinline__ void cp_async16(float* d, const float* p, bool in) {
 __device__ __forceinline__ void cp_async4(float* d, const float* p, bool in) {
   const uint32_t sa = (uint32_t)__cvta_generic_to_shared(d);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sa), "l"(p), "r"(in ? 4 : 0) : "memory");
+}
+
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+  return n;
+}
+__device__ __forceinline__ float4 ld_cluster(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
 }
 
 // A group's shape: TN columns per thread, so 64 (TN = 8) or 128 (TN = 4) threads.
@@ -134,11 +147,14 @@ __device__ __forceinline__ void store_mmajor(float* S, const QuadRegs& r, int t)
 extern __shared__ __align__(16) float gsm[];
 
 // AKM: A is K-major (copied asynchronously); else M-major, TN = 4
-template <int TN, bool AKM, int KG, int CAP>
+// SHARED: the CTAs of a cluster share a tile's K (an instantiation of its own: even reading the cluster's size costs a launch of
+// M = 64 half a microsecond)
+template <int TN, bool AKM, int KG, int CAP, bool SHARED>
 __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm_ffma_kernel(const __grid_constant__ GemmBlock<CAP> g) {
   constexpr int NT = Shape<TN>::NT;
-  // locate the problem this CTA works on
-  const int cta = blockIdx.x;
+  // locate the problem this CTA, or its cluster, works on
+  const int kc = SHARED ? (int)cluster_size() : 1, rank = SHARED ? (int)sm100::cluster_ctarank() : 0;
+  const int cta = SHARED ? (int)blockIdx.x / kc : (int)blockIdx.x;
   int pi = 0;
 #pragma unroll 1
   for (int i = 1; i < g.n; ++i)
@@ -156,8 +172,9 @@ __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm
   const int64_t kslabs = (pr.k + BK - 1) / BK;
   const int64_t per = (kslabs + pr.splits - 1) / pr.splits;
   const int64_t sb = (int64_t)split * per, se = min(sb + per, kslabs);
-  const int64_t gper = (max(se - sb, (int64_t)0) + KG - 1) / KG;
-  const int64_t kb = (sb + grp * gper) * BK, ke = min(min(sb + (grp + 1) * gper, se) * BK, pr.k);
+  const int groups = KG * kc, part_of_k = rank * KG + grp;
+  const int64_t gper = (max(se - sb, (int64_t)0) + groups - 1) / groups;
+  const int64_t kb = (sb + part_of_k * gper) * BK, ke = min(min(sb + (part_of_k + 1) * gper, se) * BK, pr.k);
 
   float* slab = gsm + grp * kStages * kSlab;
   const int tx = t % (BN / TN), ty = t / (BN / TN);
@@ -287,18 +304,43 @@ __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm
       if (want_colsum && t < BM) cols[(grp - 1) * BM + t] = colacc;
     }
     __syncthreads();
-    if (grp > 0) return;
+    if (grp > 0 && kc == 1) return;
+    if (grp == 0) {
 #pragma unroll
-    for (int q = 0; q < KG - 1; ++q) {
+      for (int q = 0; q < KG - 1; ++q) {
 #pragma unroll
-      for (int i = 0; i < TM; ++i) {
+        for (int i = 0; i < TM; ++i) {
 #pragma unroll
-        for (int h = 0; h < TN / 4; ++h) {
-          const float4 o = part[(q * (TN / 4) * TM + (TN / 4) * i + h) * NT + t];
-          acc[i][4 * h] += o.x; acc[i][4 * h + 1] += o.y; acc[i][4 * h + 2] += o.z; acc[i][4 * h + 3] += o.w;
+          for (int h = 0; h < TN / 4; ++h) {
+            const float4 o = part[(q * (TN / 4) * TM + (TN / 4) * i + h) * NT + t];
+            acc[i][4 * h] += o.x; acc[i][4 * h + 1] += o.y; acc[i][4 * h + 2] += o.z; acc[i][4 * h + 3] += o.w;
+          }
+        }
+        if (want_colsum && t < BM) colacc += cols[q * BM + t];
+      }
+    }
+    if (SHARED && kc > 1) {
+      // the CTAs' sums, added in order by the first one out of the others' shared memory, which stays until it has read them
+      float4* sums = reinterpret_cast<float4*>(gsm + (KG - 1) * (BM * BN + BM));
+      if (grp == 0 && rank > 0) {
+#pragma unroll
+        for (int i = 0; i < TM; ++i) sums[i * NT + t] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      }
+      sm100::cluster_arrive();
+      sm100::cluster_wait();
+      if (grp == 0 && rank == 0) {
+        for (int r = 1; r < kc; ++r) {
+          const uint32_t p = sm100::mapa_shared((uint32_t)__cvta_generic_to_shared(sums + t), (uint32_t)r);
+          float4 o[TM];
+#pragma unroll
+          for (int i = 0; i < TM; ++i) o[i] = ld_cluster(p + (uint32_t)(i * NT * sizeof(float4)));
+#pragma unroll
+          for (int i = 0; i < TM; ++i) { acc[i][0] += o[i].x; acc[i][1] += o[i].y; acc[i][2] += o[i].z; acc[i][3] += o[i].w; }
         }
       }
-      if (want_colsum && t < BM) colacc += cols[q * BM + t];
+      sm100::cluster_arrive();
+      sm100::cluster_wait();
+      if (grp > 0 || rank > 0) return;
     }
   }
 
@@ -363,24 +405,25 @@ __global__ void __launch_bounds__(Shape<TN>::NT * KG, TN == 8 ? 8 / KG : 1) gemm
   if (bad && pr.nonfinite) *pr.nonfinite = 1;
 }
 
-template <int TN, bool AKM, int KG, int CAP>
-cudaError_t launch(const GemmGroup& g, int total, cudaStream_t s) {
+template <int TN, bool AKM, int KG, int CAP, bool SHARED>
+cudaError_t launch(const GemmGroup& g, int total, int kc, cudaStream_t s) {
   static SmemAttrCache attr;
-  const size_t part = (KG - 1) * (size_t)(BM * BN + BM), slabs = (size_t)KG * kStages * kSlab;
+  const size_t part = (KG - 1) * (size_t)(BM * BN + BM) + (SHARED ? BM * BN : 0), slabs = (size_t)KG * kStages * kSlab;
   const size_t smem = (part > slabs ? part : slabs) * sizeof(float);
-  cudaError_t e = ensure_dyn_smem(gemm_ffma_kernel<TN, AKM, KG, CAP>, smem, attr);
+  cudaError_t e = ensure_dyn_smem(gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, smem, attr);
   if (e != cudaSuccess) return e;
   GemmBlock<CAP> b;
   b.n = g.n;
   memcpy(b.p, g.p, g.n * sizeof(GemmProblem));
-  launch_dep(gemm_ffma_kernel<TN, AKM, KG, CAP>, total, Shape<TN>::NT * KG, smem, s, b);
+  if (SHARED) launch_dep_cluster(kc, gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total * kc, Shape<TN>::NT * KG, smem, s, b);
+  else launch_dep(gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total, Shape<TN>::NT * KG, smem, s, b);
   return cudaGetLastError();
 }
-template <int TN, bool AKM, int KG>
-cudaError_t launch_cap(const GemmGroup& g, int total, cudaStream_t s) {
-  if (g.n <= 2) return launch<TN, AKM, KG, 2>(g, total, s);
-  if (g.n <= 16) return launch<TN, AKM, KG, 16>(g, total, s);
-  return launch<TN, AKM, KG, FW_MAX_GROUP>(g, total, s);
+template <int TN, bool AKM, int KG, bool SHARED = false>
+cudaError_t launch_cap(const GemmGroup& g, int total, cudaStream_t s, int kc = 1) {
+  if (g.n <= 2) return launch<TN, AKM, KG, 2, SHARED>(g, total, kc, s);
+  if (g.n <= 16) return launch<TN, AKM, KG, 16, SHARED>(g, total, kc, s);
+  return launch<TN, AKM, KG, FW_MAX_GROUP, SHARED>(g, total, kc, s);
 }
 
 bool quads(const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (ld & 3) == 0; }
@@ -408,13 +451,24 @@ cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class) {
   // 128); with fewer tiles than that the chain of a tile is shared, and below one tile per SM it is what counts, so the
   // groups have 128 threads there.
   const int sms = sm_count();
+  // A tile is 64 x 64 x K products on one SM, 9.4 us of its FP32 pipe at K = 576: with few tiles a cluster of CTAs shares each, as
+  // long as a group keeps four slabs of the longest K and the clusters fill at most three quarters of the SMs (beyond that two
+  // CTAs meet on an SM, and 36 tiles of K = 576 took 30 us on four CTAs each instead of 22 on one).  G Qs, one CTA -> shared:
+  // 64 x 576 22 -> 13 us, 256 x 576 22 -> 16, 64 x 1024 36 -> 15, 16 x 2304 68 -> 38; not taken: 16 x 144 8.7 -> 9.7.
+  int kc = 1;
+  int64_t kslabs = 0;
+  bool whole = true;                  // column sums and row splits are the Gram pass's, whose partition is the caller's
+  for (int i = 0; i < g.n; ++i) { kslabs = std::max(kslabs, (g.p[i].k + BK - 1) / BK); whole = whole && !g.p[i].colsum && g.p[i].splits == 1; }
+  while (whole && kc < 8 && 8 * kc * total <= 3 * sms && kslabs >= 16 * kc) kc *= 2;
   if (!g.p[0].a_kmajor) {
     if (total >= 4 * sms) return launch_cap<4, false, 1>(g, total, s);
+    if (kc > 1) return launch_cap<4, false, 4, true>(g, total, s, kc);
     return launch_cap<4, false, 4>(g, total, s);
   }
   if (total >= 6 * sms) return launch_cap<8, true, 1>(g, total, s);
   if (total >= 3 * sms) return launch_cap<8, true, 2>(g, total, s);
   if (total >= sms) return launch_cap<8, true, 4>(g, total, s);
+  if (kc > 1) return launch_cap<4, true, 4, true>(g, total, s, kc);
   return launch_cap<4, true, 4>(g, total, s);
 }
 

@@ -192,6 +192,22 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), p);
 }
 
+// The same in clusters of cl CTAs.
+template <class... P>
+inline cudaError_t launch_dep_cluster(int cl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                      const typename SameType<P>::type&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cl; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), p);
+}
+
 // Largest dynamic shared-memory size a kernel has been opted into, per device (the attribute is per device).
 struct SmemAttrCache { size_t set[64] = {0}; };
 template <class F>

@@ -5,7 +5,7 @@ import pytest
 
 from oracle import fw_oracle as O
 
-from fwtest_util import TOL_TC, rel_fro, t2n
+from fwtest_util import TOL_FP32, TOL_TC, rel_fro, t2n
 
 pytestmark = pytest.mark.gpu
 
@@ -35,4 +35,28 @@ def test_products_over_many_tiles(env, M, rows):
     B.fw_whiten_backward(L.handle, torch.from_numpy(dY).cuda(), rows, dX)
     assert rel_fro(t2n(dX), O.whiten_backward(Lo, dY)) <= TOL_TC
     assert bool(torch.isnan(buf[rows * M:]).all())              # nothing past the last row
+    assert L.sync_status() == B.FW_OK
+
+
+@pytest.mark.parametrize("N,M", [(4, 255), (4, 256), (4, 257), (65, 300), (16, 511), (64, 576), (130, 577), (256, 640), (100, 1031), (5, 2050)])
+def test_fp32_products_shared_by_a_cluster(env, N, M):
+    """Few tiles and a long K: G Qs and the re-sync products on two, four and eight CTAs a tile, uneven shares of K among them, odd
+    sizes."""
+    torch, B = env
+    rng = np.random.default_rng(N + M)
+    Phi = rng.standard_normal((M, M)).astype(np.float32)
+    Phi = np.triu(Phi) + np.triu(Phi, 1).T
+    T = (np.eye(M) + 0.3 * rng.standard_normal((M, M)) / np.sqrt(M)).astype(np.float32)
+    G = rng.standard_normal((N, M)).astype(np.float32)
+    L = B.Layer(M, N, beta=0.0, gamma=1.0)
+    L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda())
+    L.set(B.FW_F_T, torch.from_numpy(T).cuda())
+    B.fw_group_cond_reduce([L.handle], 0, 0)
+    T64, P64 = T.astype(np.float64), Phi.astype(np.float64)
+    Q = t2n(L.get(B.FW_F_Q)).reshape(M, M)
+    Y = t2n(L.get(B.FW_F_PHIY)).reshape(M, M)
+    assert rel_fro(Q, T64.T @ T64) <= TOL_FP32 and rel_fro(Y, T64 @ P64 @ T64.T) <= TOL_FP32
+    assert np.array_equal(Y, Y.T)
+    Gt = t2n(L.grad_transform(torch.from_numpy(G).cuda()))
+    assert rel_fro(Gt, G.astype(np.float64) @ Q.astype(np.float64)) <= TOL_FP32
     assert L.sync_status() == B.FW_OK
