@@ -688,25 +688,23 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
   } else if (sub == 0 && tid == 0) {
     L.words[0] = 1;
   }
-  // squared length of a column of that is rounding
+  // squared length of a column that is rounding
   const double floor2 = fac ? kFloor * top : kFloor * top * (kFloor * top);
   const int np = L.nb / 2, n1 = L.nb - 1;
   // rounds until a sweep's worth of them in a row has rotated nothing
   int last = 0;
   for (int round = 1, r = 0; round <= kMaxSweeps * n1; ++round, r = r + 1 == n1 ? 0 : r + 1) {
-    {
-      for (int k = sub; k < np; k += L.n) {
-        int I, J;
-        if (k == 0) { I = n1; J = r; }
-        else { I = (r + k) % n1; J = (r - k + n1) % n1; }
-        if (I > J) { const int x = I; I = J; J = x; }
-        if (I * EB >= M) continue;                                // both blocks past the matrix
-        const int v = r == 0 ? visit<false>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity)
-                             : visit<true>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity);
-        if (v < 0) { evd_give_up(L); return; }
-        if (v > 0) last = round;
-        __syncthreads();                                          // the staged rows are free for the next pair
-      }
+    for (int k = sub; k < np; k += L.n) {
+      int I, J;
+      if (k == 0) { I = n1; J = r; }
+      else { I = (r + k) % n1; J = (r - k + n1) % n1; }
+      if (I > J) { const int x = I; I = J; J = x; }
+      if (I * EB >= M) continue;                                  // both blocks past the matrix
+      const int v = r == 0 ? visit<false>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity)
+                           : visit<true>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity);
+      if (v < 0) { evd_give_up(L); return; }
+      if (v > 0) last = round;
+      __syncthreads();                                            // the staged rows are free for the next pair
     }
     if (!evd_barrier(L, sub, ++bidx, last, &s_abort, &s_last)) return;
     if (round - s_last >= n1) break;                              // every pair is orthogonal

@@ -653,9 +653,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
     }
     // ---- epilogue: accumulators -> partial Gram; two warps per TMEM lane quarter ----
     const bool have = nk > 0;
-    bool good = ok;
-    if (good && have && !mbar_wait(smem_u32(&bar_accum), 0, abortp)) {
-      good = false;
+    if (ok && have && !mbar_wait(smem_u32(&bar_accum), 0, abortp)) {
       abort_flag = 1;
       atomicExch(pr.status, 204);
     }
