@@ -217,6 +217,10 @@ struct Gram32 {
   int32_t e[EP];                      // column i is 2^e times its scaled self
   float h[2][EB];                     // tangents of half the angles of an inner round
 };
+// The fp64 products say that a visit has something to rotate; the inner rounds, in fp32, then have to rotate that pair: the bound is
+// lower by more than fp32 can be off.  With the same one on both sides a cosine a part in 1e7 above it was left alone by every visit
+// and found again in every sweep, up to kMaxSweeps.
+constexpr float kRotTol2 = (float)(kOrthTol * kOrthTol * (1.0 - 1e-5));
 constexpr float kFrozen = 1e-5f;      // a column that has lost this much of its squared length waits for the next visit: its products are rounding
 
 // ---- Phi = R^T R (R upper triangular), in place in W ----
@@ -563,7 +567,7 @@ __device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, in
           const float ir = rsqrt_approx(n2);                               // 1 / R
           const float c2 = fmaf(0.5f * fabsf(d), ir, 0.5f);                // cos^2 phi
           const float ic = rsqrt_approx(c2);
-          const bool rot = ga * ga > (float)(kOrthTol * kOrthTol) * (al * be) && fminf(al, be) > kFrozen;
+          const bool rot = ga * ga > kRotTol2 * (al * be) && fminf(al, be) > kFrozen;
           const float gs2 = d < 0.f ? -ga : ga;
           const float cb = rot ? c2 * ic : 1.f;
           const float sb = rot ? gs2 * ir * ic : 0.f;

@@ -114,3 +114,34 @@ def test_eigenvalues_not_told_from_zero(env):
     T = t2n(L.get(B.FW_F_T))
     assert np.abs(np.diag(T) / want - 1.0).max() <= TOL_FP32 and np.abs(T - np.diag(np.diag(T))).max() == 0.0
     assert L.sync_status() == B.FW_OK
+
+
+# (a, b, d) of fp32 blocks [[a, b], [b, d]]: b / a, the cosine of their factor's two columns, exceeds the rotations' tolerance of
+# 1e-14 by a part in 1e7, less than fp32 products tell
+BARELY = [("0x1.4471060000000p+1", "0x1.c89c620000000p-46", "0x1.a3703c0000000p+1"),
+          ("0x1.94766e0000000p+0", "0x1.1c9d840000000p-46", "0x1.4c46580000000p+1"),
+          ("0x1.ef237e0000000p+1", "0x1.5c6c420000000p-45", "0x1.1e0fb00000000p+0")]
+
+
+@pytest.mark.parametrize("abd", BARELY)
+@pytest.mark.parametrize("M,j", [(2, 1), (34, 33)])
+def test_rounds_end_with_a_pair_at_the_tolerance(env, M, j, abd):
+    """A pair whose cosine lies at the tolerance counts as rotated only where it is rotated: otherwise it is found again in every
+    sweep, up to the last one allowed.  In a visit of all pairs (M = 2) and of blocks 0 and 2 (M = 34)."""
+    torch, B = env
+    a, b, d = (float.fromhex(x) for x in abd)
+    assert 1e-14 < b / a < 1e-14 * (1 + 1.3e-7)
+    Phi = np.diag(np.linspace(1.0, 3.0, M)).astype(np.float32)
+    Phi[0, 0], Phi[j, j], Phi[0, j], Phi[j, 0] = a, d, b, b
+    L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+    L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda())
+    scratch, nb = scratch_for(torch, B, M)
+    B.fw_evd_whiten(L.handle, scratch, nb, 0.0)
+    assert L.sync_status() == B.FW_OK
+    # the scratch starts with the barrier words: each CTA's count of barriers, one after loading, one per 16 rows of the factor
+    # and one more, then one a round
+    blocks = (M + 15) // 16
+    rounds = (int(scratch[:1024].view(torch.int32)[64]) >> 16) - 1 - (blocks + 1)
+    assert 1 <= rounds <= 3 * (((blocks + 1) & ~1) - 1), rounds
+    T = t2n(L.get(B.FW_F_T)).reshape(M, M)
+    assert rel_fro(T, np.diag(1.0 / np.sqrt(np.diag(Phi).astype(np.float64)))) <= TOL_FP32
