@@ -3,20 +3,22 @@
 // Phi = R^T R (Cholesky), and the columns of W = R^T Z, starting from Z = I, are rotated until all are orthogonal; then they
 // are V Lambda^(1/2): the normalised columns are the eigenvectors and their squared lengths the eigenvalues, and Z is never
 // carried along.  Where Phi is not (safely) positive definite, W starts from Phi itself and ends as V Lambda, which takes
-// sweeps more: 8 instead of 12 to 13 for the covariances of M = 576 here, 8 instead of 15 at condition 1e3.
+// more sweeps: 13 instead of 10 for the covariances of M = 576 here (340 to 351 rounds), 15 instead of 9 at condition 1e3.
 // Columns are stored as rows, fp64 throughout: T = Phi^(-1/2) carries the rounding of the
 // decomposition times cond(Phi) / 2, which fp32 cannot afford.
 //
 // A CTA takes a pair of blocks of 16 columns: their products (tensor-core fp64, the columns staged in shared memory), one
-// sweep of 2 x 2 rotations on that 32 x 32 matrix in fp32 (Gram32), accumulated into U in fp64, and W <- U^T W on the 32
+// sweep of 2 x 2 rotations on that 32 x 32 matrix in shared memory, accumulated into U, and W <- U^T W on the 32
 // rows.  The block pairs of a round (round-robin tournament) are disjoint, so a layer's CTAs meet
 // once per round, M / 16 - 1 rounds a sweep, instead of once per round of column pairs (M - 1 rounds).  The first round of a
 // sweep rotates all pairs of a visit's 32 columns, the others those of different blocks (visit).  All layers of a
-// group share the launch, each with CTAs and barriers of its own.  What bounds a round at M = 576 (17.9 us) is a chain, in
-// clocks: staging 3200, products 5300, 16 inner rounds 9400 (553 each), update 12200 (9200 at the rate of the fp64 tensor
-// cores), barrier 5000; a round that rotates nothing takes 13500.  The 15 layers of the ResNet-20-shaped set: 12.5 ms from Phi,
-// 9.3 from the factor (0.34 of it the factorisation), 6.8 with inner rounds in fp32 (31 of 1014 clocks before, products
-// 8000).  One-sided rotations are those of Hestenes (1958), the start from the Cholesky factor that of Veselic and
+// group share the launch, each with CTAs and barriers of its own.  What bounds a round at M = 576 (17.8 us) is a chain, in
+// clocks: staging 3500, products 4000, 16 inner rounds 9500 (592 each), update 11700 (9200 at the rate of the fp64 tensor
+// cores), barrier 5000 to 7700; a round that rotates nothing takes 13000.  An inner round is a chain too: load 71, rotation 255,
+// the 2 x 2 products 164, barrier and waiting for the slowest warp 100.  15 layers of the ResNet-20-shaped set: 12.5 ms from
+// Phi, 9.3 from the factor (0.35 of it the factorisation), 6.7 with cross visits and inner rounds of this shape (1014 clocks
+// with 256 threads on all of the matrix and as many on U, 553 with an fp32 copy of the products, which the angles alone allow).
+// One-sided rotations are those of Hestenes (1958), the start from the Cholesky factor that of Veselic and
 // Hari (1989), the tournament of block pairs that of Brent and Luk (1985).
 //
 // Then T = V diag(sqrt g) V^T (Eq. 9), Q = T^T T = V diag(g) V^T and Phi_y = T Phi T^T = V diag(g lambda) V^T come
@@ -49,8 +51,8 @@ constexpr double kFloor = 1e-14, kNull = 1e-13;
 // shared-memory row stride in doubles: 4 mod 16, so that the fragments of both products read without conflicts
 __host__ __device__ inline int evd_stride(int cols) { return ((cols + 15) & ~15) + 4; }
 __host__ __device__ inline int evd_ld(int M) { return (M + 7) & ~7; }
-constexpr int kGLd = EP + 1;          // leading dimension of the 32 x 32 matrices in shared memory
-constexpr int kGF = 48;                // of the fp32 copies: the two rows of a warp's access lie 16 banks apart
+constexpr int kULd = EP + 1;          // leading dimensions of the 32 x 32 matrices in shared memory: U, read along a row,
+constexpr int kGLd = EP + 2;          // and the products, read along wrapped diagonals (row + column, or row - column, fixed)
 constexpr int kTri = 10;              // 8 x 8 blocks of the upper triangle of a 32 x 32 matrix
 constexpr int kCross = 4 * 64 + EP;    // partial sums of a warp of a cross visit: four 8 x 8 blocks and 32 squared lengths
 constexpr int kPartDoubles = EW / 2 * kTri * 64;
@@ -152,7 +154,7 @@ __device__ __forceinline__ void evd_players(int k, int q, int& p, int& r) {
   if (k == 0) p = EP - 1;
 }
 
-// dynamic shared memory: [32 rows of a chunk][partial Gram blocks of the warps, later U][Gram]
+// dynamic shared memory: [32 rows of a chunk][partial Gram blocks of the warps, later U and the second Gram buffer][Gram]
 extern __shared__ __align__(16) double esm[];
 
 // Rows of the block pair (I, J): row r of the pair is column I * 16 + r or J * 16 + r - 16 of the layer.
@@ -198,30 +200,44 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// x 2^(127 - e) as fp32, truncated, for e the (biased) fp64 exponent of a number at least as large; 0 when too small
+__device__ __forceinline__ float to_float_scaled(double x, int e) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int ex = ((hi >> 20) & 0x7ff) - e + 127;
+  const uint32_t bits = (uint32_t)(hi & 0x80000000) | ((uint32_t)ex << 23) | (__funnelshift_l((uint32_t)lo, (uint32_t)hi, 3) & 0x007fffffu);
+  return ex > 0 ? __uint_as_float(bits) : 0.f;
 }
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }       // -127 < e < 128
-__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// The fp32 number as fp64, without the conversion unit (8 clocks a warp); 0 becomes 6e-39.
+__device__ __forceinline__ double to_double(float x) {
+  const uint32_t b = __float_as_uint(x);
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
 
-// The 32 x 32 Gram matrix for its sweep of rotations, in fp32: the angles need no more, since what an angle misses, 1e-7 of
-// the product, the next visit sees (it starts from fp64 products again), and the rotations that are applied to the columns are
-// orthonormal in fp64 whatever their angle.  Columns are scaled by powers of two to lengths between 1 and 2, so that
-// graded columns keep their products' relative precision; the squared lengths are carried as two numbers, so that the
-// difference of two nearly equal ones, which decides the angle between them, keeps its own.
-struct Gram32 {
-  float g[2][EP][kGF];
-  float hi[2][EP], lo[2][EP];
-  int32_t e[EP];                      // column i is 2^e times its scaled self
-  float h[2][EB];                     // tangents of half the angles of an inner round
-};
-// The fp64 products say that a visit has something to rotate; the inner rounds, in fp32, then have to rotate that pair: the bound is
-// lower by more than fp32 can be off.  With the same one on both sides a cosine a part in 1e7 above it was left alone by every visit
-// and found again in every sweep, up to kMaxSweeps.
-constexpr float kRotTol2 = (float)(kOrthTol * kOrthTol * (1.0 - 1e-5));
-constexpr float kFrozen = 1e-5f;      // a column that has lost this much of its squared length waits for the next visit: its products are rounding
+// Are columns with squared lengths al, be and product ga to be rotated?  floor2: squared length of a null column.  The one rule for
+// whether a visit has anything to rotate and whether a pair is: what the first finds the second has to rotate, or every
+// sweep would find it again.
+__device__ __forceinline__ bool to_rotate(double al, double be, double ga, double floor2) {
+  return ga * ga > kOrthTol * kOrthTol * (al * be) && fmin(al, be) > floor2;
+}
+
+// The rotation (c, s) that makes columns p, q orthogonal (the smaller of the two angles phi, tan 2 phi = 2 ga / (be - al)); (1, 0)
+// when it is not needed.  The angle comes from fp32 arithmetic (what it misses, 1e-7 of the product, the next visit sees);
+// then (c, s) is brought to unit length in fp64, 1 / sqrt(1 + x) = 1 - x / 2 + 3 x^2 / 8 with x below 1e-6, so the
+// rotation is orthonormal in fp64 whatever its angle.  This is the chain of an inner round: seven dependent fp64 operations and
+// four of the 2 x 2 update, no fp64 division or root.
+__device__ __forceinline__ void rotation(double al, double be, double ga, double floor2, double& c, double& s) {
+  const double d = be - al;
+  const int e = max((__double2hiint(d) >> 20) & 0x7ff, (__double2hiint(ga) >> 20) & 0x7ff);
+  const float df = fabsf(to_float_scaled(d, e)), gf = to_float_scaled(ga, e), g2 = gf + gf;
+  const float ir = rsqrt_approx(fmaf(df, df, g2 * g2));            // 1 / R
+  const float c2 = fmaf(0.5f * df, ir, 0.5f);                      // cos^2 phi
+  const float ic = rsqrt_approx(c2);
+  const double cd = to_double(c2 * ic), sd = to_double((d < 0.0 ? -gf : gf) * ir * ic);
+  const double x = fma(cd, cd, fma(sd, sd, -1.0)), y = fma(0.375, x, -0.5);
+  const bool rot = to_rotate(al, be, ga, floor2);
+  c = rot ? fma(cd * x, y, cd) : 1.0;
+  s = rot ? fma(sd * x, y, sd) : 0.0;
+}
 
 // ---- Phi = R^T R (R upper triangular), in place in W ----
 // The rows of R are columns of a factor of Phi as the rows of Phi V are of Phi Phi^T = Phi^2: rotated until they are
@@ -415,17 +431,48 @@ __device__ __forceinline__ void evd_load(const EvdLayer& L, int sub) {
   }
 }
 
+// The 2 x 2 block of products of pairs a (rows i) and b (columns), pair a's rotation in lane a, b's (cb, sb): both applied.
+// Where two entries hold one product, both are written, except in cross visits, where a pair's first column is always of the
+// first block: an entry is then met again in the same place, if products of the two blocks are always taken from the upper
+// right quarter (only those of opposite pairs, a = b + 8, of the second block change places: mirror).
+struct Block2 { int i[2]; double g[2][2]; };
+template <bool CROSS>
+__device__ __forceinline__ Block2 load_block(const double* src, int a, int q, int jp, int jq) {
+  Block2 r;
+  evd_players<CROSS>(a, q, r.i[0], r.i[1]);
+  r.g[0][0] = src[r.i[0] * kGLd + jp]; r.g[0][1] = src[r.i[0] * kGLd + jq];
+  r.g[1][0] = CROSS ? src[jp * kGLd + r.i[1]] : src[r.i[1] * kGLd + jp];
+  r.g[1][1] = src[r.i[1] * kGLd + jq];
+  return r;
+}
+template <bool CROSS>
+__device__ __forceinline__ void rotate_block(double* dst, const Block2& r, int a, int jp, int jq, double cb, double sb, bool mine,
+                                             bool mirror) {
+  const double ca = __shfl_sync(0xffffffffu, cb, a), sa = __shfl_sync(0xffffffffu, sb, a);
+  const double h00 = cb * r.g[0][0] - sb * r.g[0][1], h01 = sb * r.g[0][0] + cb * r.g[0][1];
+  const double h10 = cb * r.g[1][0] - sb * r.g[1][1], h11 = sb * r.g[1][0] + cb * r.g[1][1];
+  const double v00 = ca * h00 - sa * h10, v01 = ca * h01 - sa * h11;
+  const double v10 = sa * h00 + ca * h10, v11 = sa * h01 + ca * h11;
+  if (!mine) return;
+  dst[r.i[0] * kGLd + jp] = v00; dst[r.i[0] * kGLd + jq] = v01;
+  dst[jp * kGLd + r.i[1]] = v10; dst[r.i[1] * kGLd + jq] = v11;
+  if (!CROSS || mirror) dst[jq * kGLd + r.i[1]] = v11;
+  if (CROSS) return;
+  dst[jp * kGLd + r.i[0]] = v00; dst[jq * kGLd + r.i[0]] = v01; dst[r.i[1] * kGLd + jp] = v10;
+}
+
 // A visit to the block pair (I, J).  CROSS: rotations between columns of different blocks only, with the products within a
 // block taken as zero (all but the squared lengths): they were rotated in the sweep's first round, and what they have become
 // since enters only at second order.  That is 4 of 10 blocks of the Gram matrix and 16 of 31 inner rounds, for half a sweep
 // more.  1: rotated; 0: nothing to rotate; -1: a wait gave up.
 template <bool CROSS>
-__device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, int chunks, int stride, double floor2, Gram32& gs,
+__device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, int chunks, int stride, double floor2, double2 (*rots)[EB],
                                      uint32_t bar, uint32_t& parity) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, M = L.M, ld = evd_ld(M);
   double* part = esm + EP * stride;                               // kPartDoubles
   double* G0 = part + kPartDoubles;
-  double* U = part;                                               // reuses the partial blocks
+  double* U = part;                                               // these two reuse the partial blocks
+  double* G1 = part + EP * kULd;
   // ---- G = (rows)(rows)^T: each warp a sixteenth of the entries, all blocks that are wanted ----
   constexpr int NB = CROSS ? 4 : kTri;
   double acc[NB][2], n2[4] = {0.0, 0.0, 0.0, 0.0};
@@ -471,9 +518,15 @@ __device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, in
       for (int w = 0; w < EW; w += 2) { x += part[w * kCross + tid]; y += part[(w + 1) * kCross + tid]; }
       x += y;
       const int b = tid >> 6, e = tid & 63;
-      if (b < 4) G0[(8 * (b >> 1) + (e >> 3)) * kGLd + EB + 8 * (b & 1) + (e & 7)] = x;
-      else G0[e * kGLd + e] = x;
+      if (b < 4) {
+        const int gi = 8 * (b >> 1) + (e >> 3), gj = EB + 8 * (b & 1) + (e & 7);
+        G0[gi * kGLd + gj] = x; G0[gj * kGLd + gi] = x;
+      } else {
+        G0[e * kGLd + e] = x;
+      }
     }
+    const int p = tid >> 4, q = (p & EB) + (tid & (EB - 1));         // ET = 32 x 16: a thread for each entry within the blocks
+    if (p != q) G0[p * kGLd + q] = 0.0;
   } else {
     // the second half of the warps hand their sums to the first half, which add to them
     if (warp >= EW / 2) {
@@ -498,120 +551,62 @@ __device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, in
       const int b = i >> 6, e = i & 63;
       const int rb = b < 4 ? 0 : (b < 7 ? 1 : (b < 9 ? 2 : 3)), cb = b - (b < 4 ? 0 : (b < 7 ? 3 : (b < 9 ? 5 : 6)));
       const int gi = 8 * rb + (e >> 3), gj = 8 * cb + (e & 7);
-      if (rb != cb || gj >= gi) G0[gi * kGLd + gj] = x;
+      if (rb != cb || gj >= gi) { G0[gi * kGLd + gj] = x; G0[gj * kGLd + gi] = x; }
     }
   }
   __syncthreads();
-  // ---- anything to rotate?  the upper triangle, or its cross block ----
+  // ---- anything to rotate? ----
   bool act = false;
   for (int i = tid; i < EP * EP; i += ET) {
     const int p = i >> 5, q = i & 31;
-    U[p * kGLd + q] = p == q ? 1.0 : 0.0;
-    if (p > q) continue;
-    const double gp = G0[p * kGLd + p], gq = G0[q * kGLd + q];
-    const bool live = fmin(gp, gq) > floor2;                      // neither is a null column
-    const int ep = (((__double2hiint(gp) >> 20) & 0x7ff) - 1023) >> 1, eq = (((__double2hiint(gq) >> 20) & 0x7ff) - 1023) >> 1;
-    double x = 0.0;
-    if (!CROSS || p == q || (p < EB && q >= EB)) {
-      const double g = G0[p * kGLd + q];
-      act |= p < q && live && g * g > kOrthTol * kOrthTol * (gp * gq);
-      if (live) x = g * pow2d(-ep) * pow2d(-eq);
-    }
-    gs.g[0][p][q] = gs.g[0][q][p] = (float)x;
-    if (p == q) {
-      gs.hi[0][p] = (float)x; gs.lo[0][p] = (float)(x - (double)(float)x);
-      gs.e[p] = live ? ep : 0;
-    }
+    U[p * kULd + q] = p == q ? 1.0 : 0.0;
+    act |= p < q && to_rotate(G0[p * kGLd + p], G0[q * kGLd + q], G0[p * kGLd + q], floor2);
   }
   if (!__syncthreads_or(act)) return 0;
-  // ---- one sweep of 2 x 2 rotations on G: a thread of the first four warps owns the 2 x 2 blocks of pairs (a, b), (a + 8, b);
-  //      the next four apply each round's rotations to U, in fp64, one round later, off the chain; the ninth keeps the squared
-  //      lengths and half-angles ----
-  if (warp < 9) {
-    const int pb = tid & 15, pa = (tid & 127) >> 4;
+  // ---- one sweep of 2 x 2 rotations on G.  A half-warp of the first five warps owns the 2 x 2 blocks of pairs (b + k, b), b its
+  //      lane: k = 0 ... 7 and, for half of the b, 8.  Six more warps apply each round's rotations to U one round later, off
+  //      the chain (not warp 8: two of the five share its scheduler). ----
+  if (warp < 12 && warp != 8) {
+    const int pb = tid & 15;
     constexpr int kRounds = CROSS ? EB : EP - 1;
-    int jp, jq, ip[2], iq[2], de;
-    auto players = [&](int q) {
-      evd_players<CROSS>(pb, q, jp, jq);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        evd_players<CROSS>(pa + 8 * i, q, ip[i], iq[i]);
-        ip[i] *= kGF; iq[i] *= kGF;
-      }
-      de = min(max(gs.e[jq] - gs.e[jp], -60), 60);
-    };
-    players(0);
-    for (int q = 0; q <= kRounds; ++q) {
-      if (warp < 4 || warp == 8) {
+    if (warp < 5) {
+      const int k = min(tid >> 4, 8), pa = (pb + k) & 15;
+      const bool mine = k < 8 || tid < 8 * EB + 8;
+      double* src = G0;
+      double* dst = G1;
+      int jp, jq;
+      evd_players<CROSS>(pb, 0, jp, jq);
+      for (int q = 0; q <= kRounds; ++q) {
         if (q < kRounds) {
-          const int z = q & 1;
-          const float* src = &gs.g[z][0][0];
-          float* dst = &gs.g[z ^ 1][0][0];
-          const float al = gs.hi[z][jp], be = gs.hi[z][jq], all = gs.lo[z][jp], bel = gs.lo[z][jq], ga = src[jp * kGF + jq];
-          float g[2][4];
-          int at[2][4];
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            at[i][0] = ip[i] + jp; at[i][1] = ip[i] + jq; at[i][2] = iq[i] + jp; at[i][3] = iq[i] + jq;
-            if (warp < 4) {
-#pragma unroll
-              for (int h = 0; h < 4; ++h) g[i][h] = src[at[i][h]];
-            }
-          }
-          const float w = pow2f(de), wi = pow2f(-de);
-          const int kp = jp, kq = jq;
-          players(q + 1);                                                  // of the next round, while the loads are under way
-          // the smaller of the two angles phi, tan 2 phi = 2 ga / (be - al)
-          const float d = (be * w - al * wi) + (bel * w - all * wi);
-          const float g2 = ga + ga, n2 = fmaf(d, d, g2 * g2);
-          const float ir = rsqrt_approx(n2);                               // 1 / R
-          const float c2 = fmaf(0.5f * fabsf(d), ir, 0.5f);                // cos^2 phi
-          const float ic = rsqrt_approx(c2);
-          const bool rot = ga * ga > kRotTol2 * (al * be) && fminf(al, be) > kFrozen;
-          const float gs2 = d < 0.f ? -ga : ga;
-          const float cb = rot ? c2 * ic : 1.f;
-          const float sb = rot ? gs2 * ir * ic : 0.f;
-          if (warp < 4) {
-            const float s1 = sb * w, s2 = sb * wi;                         // on scaled columns
-            const float keep = rot ? 0.f : ga;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const int a = pa + 8 * i;
-              const float ca = __shfl_sync(0xffffffffu, cb, a), s1a = __shfl_sync(0xffffffffu, s1, a), s2a = __shfl_sync(0xffffffffu, s2, a);
-              const float h00 = cb * g[i][0] - s1 * g[i][1], h01 = s2 * g[i][0] + cb * g[i][1];
-              const float h10 = cb * g[i][2] - s1 * g[i][3], h11 = s2 * g[i][2] + cb * g[i][3];
-              const bool own = a == pb;                                    // its diagonal entries are those in hi, lo
-              dst[at[i][0]] = ca * h00 - s1a * h10; dst[at[i][1]] = own ? keep : ca * h01 - s1a * h11;
-              dst[at[i][2]] = own ? keep : s2a * h00 + ca * h10; dst[at[i][3]] = s2a * h01 + ca * h11;
-            }
-          } else if (lane < EB) {
-            const float t = rot ? 2.f * gs2 * rcp_approx(fmaf(n2, ir, fabsf(d))) : 0.f;      // tan phi, signed
-            const float x0 = -t * ga * w, x1 = t * ga * wi;
-            const float n0 = al + x0, n1 = be + x1, v0 = n0 - al, v1 = n1 - be;
-            gs.hi[z ^ 1][kp] = n0; gs.lo[z ^ 1][kp] = all + ((al - (n0 - v0)) + (x0 - v0));
-            gs.hi[z ^ 1][kq] = n1; gs.lo[z ^ 1][kq] = bel + ((be - (n1 - v1)) + (x1 - v1));
-            gs.h[z][pb] = sb * rcp_approx(1.f + cb);
-          }
+          const double al = src[jp * kGLd + jp], be = src[jq * kGLd + jq], ga = src[jp * kGLd + jq];
+          const Block2 g = load_block<CROSS>(src, pa, q, jp, jq);
+          double cb, sb;
+          rotation(al, be, ga, floor2, cb, sb);
+          rotate_block<CROSS>(dst, g, pa, jp, jq, cb, sb, mine, k == 8);
+          if (tid >= 9 * EB) rots[q & 1][pb] = make_double2(cb, sb);
+          double* z = src; src = dst; dst = z;
+          evd_players<CROSS>(pb, q + 1, jp, jq);
         }
-      } else if (q > 0) {
-        evd_players<CROSS>(pb, q - 1, jp, jq);
-        // c = 2 / (1 + h^2) - 1, s = 2 h / (1 + h^2), the reciprocal refined to fp64 rounding
-        const float h = gs.h[(q - 1) & 1][pb];
-        double x0[4], x1[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { x0[i] = U[(pa + 8 * i) * kGLd + jp]; x1[i] = U[(pa + 8 * i) * kGLd + jq]; }
-        const double hd = (double)h, x = fma(hd, hd, 1.0);
-        const double r0 = (double)rcp_approx(fmaf(h, h, 1.f));
-        const double f1 = fma(-x, r0, 1.0);
-        const double rr = fma(r0, fma(f1, f1, f1), r0);
-        const double c = fma(2.0, rr, -1.0), sn = (hd + hd) * rr;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          U[(pa + 8 * i) * kGLd + jp] = c * x0[i] - sn * x1[i];
-          U[(pa + 8 * i) * kGLd + jq] = sn * x0[i] + c * x1[i];
-        }
+        asm volatile("bar.sync 1, 352;" ::: "memory");
       }
-      asm volatile("bar.sync 1, 288;" ::: "memory");
+    } else {
+      const int row0 = 2 * (warp - (warp > 8 ? 6 : 5)) + (lane >> 4);    // and 12, 24 more
+      for (int q = 0; q <= kRounds; ++q) {
+        if (q > 0) {
+          int jp, jq;
+          evd_players<CROSS>(pb, q - 1, jp, jq);
+          const double2 r = rots[(q - 1) & 1][pb];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            double* u = U + (row0 + 12 * i) * kULd;
+            if (i == 2 && row0 >= 8) break;
+            const double x0 = u[jp], x1 = u[jq];
+            u[jp] = r.x * x0 - r.y * x1;
+            u[jq] = r.y * x0 + r.x * x1;
+          }
+        }
+        asm volatile("bar.sync 1, 352;" ::: "memory");
+      }
     }
   }
   __syncthreads();
@@ -622,7 +617,7 @@ __device__ __forceinline__ int visit(const EvdLayer& L, int I, int J, int nk, in
 #pragma unroll
   for (int cb = 0; cb < 2; ++cb)
 #pragma unroll
-    for (int kb = 0; kb < 8; ++kb) uf[cb][kb] = U[(4 * kb + (lane & 3)) * kGLd + 16 * half + 8 * cb + (lane >> 2)];
+    for (int kb = 0; kb < 8; ++kb) uf[cb][kb] = U[(4 * kb + (lane & 3)) * kULd + 16 * half + 8 * cb + (lane >> 2)];
   for (int ch = 0; ch < chunks; ++ch) {
     if (chunks > 1) {
       __syncthreads();
@@ -657,7 +652,7 @@ __global__ void __launch_bounds__(kWords) evd_clear_kernel(const __grid_constant
 __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ EvdArgs a) {
   __shared__ int s_abort, s_last;
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ Gram32 gs;
+  __shared__ double2 rots[2][EB];
   const int tid = threadIdx.x;
   int li = -1;
 #pragma unroll 1
@@ -704,8 +699,8 @@ __global__ void __launch_bounds__(ET, 1) jacobi_kernel(const __grid_constant__ E
       else { I = (r + k) % n1; J = (r - k + n1) % n1; }
       if (I > J) { const int x = I; I = J; J = x; }
       if (I * EB >= M) continue;                                  // both blocks past the matrix
-      const int v = r == 0 ? visit<false>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity)
-                           : visit<true>(L, I, J, nk, chunks, stride, floor2, gs, bar, parity);
+      const int v = r == 0 ? visit<false>(L, I, J, nk, chunks, stride, floor2, rots, bar, parity)
+                           : visit<true>(L, I, J, nk, chunks, stride, floor2, rots, bar, parity);
       if (v < 0) { evd_give_up(L); return; }
       if (v > 0) last = round;
       __syncthreads();                                            // the staged rows are free for the next pair

@@ -116,6 +116,12 @@ def test_eigenvalues_not_told_from_zero(env):
     assert L.sync_status() == B.FW_OK
 
 
+def rounds_taken(torch, scratch, M):
+    """Rounds of the last call: the scratch starts with the barrier words, each CTA's count of barriers, one after loading, one per
+    16 rows of the factor and one more, then one a round."""
+    return (int(scratch[:1024].view(torch.int32)[64]) >> 16) - 1 - ((M + 15) // 16 + 1)
+
+
 # (a, b, d) of fp32 blocks [[a, b], [b, d]]: b / a, the cosine of their factor's two columns, exceeds the rotations' tolerance of
 # 1e-14 by a part in 1e7, less than fp32 products tell
 BARELY = [("0x1.4471060000000p+1", "0x1.c89c620000000p-46", "0x1.a3703c0000000p+1"),
@@ -138,10 +144,51 @@ def test_rounds_end_with_a_pair_at_the_tolerance(env, M, j, abd):
     scratch, nb = scratch_for(torch, B, M)
     B.fw_evd_whiten(L.handle, scratch, nb, 0.0)
     assert L.sync_status() == B.FW_OK
-    # the scratch starts with the barrier words: each CTA's count of barriers, one after loading, one per 16 rows of the factor
-    # and one more, then one a round
-    blocks = (M + 15) // 16
-    rounds = (int(scratch[:1024].view(torch.int32)[64]) >> 16) - 1 - (blocks + 1)
-    assert 1 <= rounds <= 3 * (((blocks + 1) & ~1) - 1), rounds
+    assert 1 <= rounds_taken(torch, scratch, M) <= 3 * ((((M + 15) // 16 + 1) & ~1) - 1)
     T = t2n(L.get(B.FW_F_T)).reshape(M, M)
     assert rel_fro(T, np.diag(1.0 / np.sqrt(np.diag(Phi).astype(np.float64)))) <= TOL_FP32
+
+
+def sweeps_of_one_pair(Phi):
+    """Sweeps over the up to 32 columns of a pair of blocks until one finds nothing above the tolerance, products carried in
+    fp64, with the largest cosine each starts from.  Column i is row i of the Cholesky factor."""
+    W = np.zeros((32, Phi.shape[0]))
+    W[:len(Phi)] = np.linalg.cholesky(Phi.astype(np.float64)).T
+    cosines = []
+    while True:
+        G, U = W @ W.T, np.eye(32)
+        n = np.sqrt(np.maximum(np.diag(G), 1e-300))
+        cosines.append(np.abs(G / np.outer(n, n) - np.diag(np.diag(G) / n ** 2)).max())
+        if cosines[-1] <= 1e-14:
+            return cosines
+        for q in range(31):
+            R = np.eye(32)
+            for k in range(16):
+                p, r = 31 if k == 0 else (q + k) % 31, (q - k) % 31
+                if G[p, r] ** 2 > 1e-28 * G[p, p] * G[r, r]:
+                    d = G[r, r] - G[p, p]
+                    t = 0.5 * np.arctan2(np.copysign(2 * G[p, r], G[p, r] if d >= 0 else -G[p, r]), abs(d))
+                    R[p, p] = R[r, r] = np.cos(t)
+                    R[p, r], R[r, p] = np.sin(t), -np.sin(t)
+            G, U = R.T @ G @ R, U @ R
+        W = U.T @ W
+
+
+@pytest.mark.parametrize("decades,seed", [(1, 37), (2, 38), (2, 8), (4, 10)])
+def test_products_of_a_visit_are_carried_in_fp64(env, decades, seed):
+    """As many sweeps as with all of it in fp64.  The angles are fp32: they leave up to 4 x 2^-24 of a product, which is below the
+    tolerance from cosines of 4e-8 on, where these matrices are before their last sweep that rotates.  With products carried in
+    fp32 the first two take a sweep more."""
+    torch, B = env
+    M = 16
+    q, _ = np.linalg.qr(np.random.default_rng(1000 * M + seed).standard_normal((M, M)))
+    Phi = ((q * np.logspace(0, -decades, M)) @ q.T).astype(np.float32)
+    Phi = np.triu(Phi) + np.triu(Phi, 1).T
+    cosines = sweeps_of_one_pair(Phi)
+    assert cosines[-2] < 4e-8
+    L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+    L.set(B.FW_F_PHIX, torch.from_numpy(Phi).cuda())
+    scratch, nb = scratch_for(torch, B, M)
+    B.fw_evd_whiten(L.handle, scratch, nb, 0.0)
+    assert L.sync_status() == B.FW_OK
+    assert rounds_taken(torch, scratch, M) == len(cosines)
