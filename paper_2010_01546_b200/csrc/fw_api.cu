@@ -945,16 +945,23 @@ fw_status fw_layer_get(fw_layer* L, fw_field f, void* dev_dst, size_t bytes) {
   // A kernel of ours is set up while the launch before it drains, a copy by the driver is not: 64 matrices of M = 256 in a row
   // 1.4 us each instead of 3.5 (M = 1152: 225 -> 100 us).  It takes whole floats of this device's own memory; anything else the
   // driver copies.
-  cudaPointerAttributes at;
-  int dev = -1;
-  if ((reinterpret_cast<uintptr_t>(dev_dst) & 3) == 0 && cudaGetDevice(&dev) == cudaSuccess && dev == L->device &&
-      cudaPointerGetAttributes(&at, dev_dst) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev) {
+  bool own = false;
+  if ((reinterpret_cast<uintptr_t>(dev_dst) & 3) == 0) {
+    cudaPointerAttributes at;
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev == L->device) {
+      e = cudaPointerGetAttributes(&at, dev_dst);
+      own = e == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev;
+    }
+    if (e != cudaSuccess) cudaGetLastError();        // a failed query's; any other error is the caller's to read
+  }
+  if (own) {
     float* dst = (float*)dev_dst;
     const int64_t floats = (int64_t)(need / sizeof(float));
     FW_CUDA(launch_copies(1, &src, &dst, &floats, L->stream), "fw_layer_get");
     return FW_OK;
   }
-  cudaGetLastError();
   FW_CUDA(cudaMemcpyAsync(dev_dst, src, need, cudaMemcpyDeviceToDevice, L->stream), "fw_layer_get");
   return FW_OK;
 }

@@ -1029,23 +1029,20 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
   }
   {
     ProfScope ps(FW_PROF_MISC, s);
-    launch_dep(norm_kernel, blocks, 256, 0, s, f);
+    e = launch_dep(norm_kernel, blocks, 256, 0, s, f);
+    if (e != cudaSuccess) return e;
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   {
     ProfScope ps(FW_PROF_MISC, s);
-    launch_dep(evd_finish_kernel, n, 1024, 0, s, f);
+    e = launch_dep(evd_finish_kernel, n, 1024, 0, s, f);
+    if (e != cudaSuccess) return e;
   }
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   if (with_v) {
     ProfScope ps(FW_PROF_MISC, s);
     static SmemAttrCache vattr;
     e = ensure_dyn_smem(vdv_kernel, VS * sizeof(VdvStage), vattr);
     if (e != cudaSuccess) return e;
-    launch_dep(vdv_kernel, tiles, 256, VS * sizeof(VdvStage), s, v);
-    e = cudaGetLastError();
+    e = launch_dep(vdv_kernel, tiles, 256, VS * sizeof(VdvStage), s, v);
   }
   return e;
 }

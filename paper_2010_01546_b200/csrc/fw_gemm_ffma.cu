@@ -415,9 +415,8 @@ cudaError_t launch(const GemmGroup& g, int total, int kc, cudaStream_t s) {
   GemmBlock<CAP> b;
   b.n = g.n;
   memcpy(b.p, g.p, g.n * sizeof(GemmProblem));
-  if (SHARED) launch_dep_cluster(kc, gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total * kc, Shape<TN>::NT * KG, smem, s, b);
-  else launch_dep(gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total, Shape<TN>::NT * KG, smem, s, b);
-  return cudaGetLastError();
+  if (SHARED) return launch_dep_cluster(kc, gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total * kc, Shape<TN>::NT * KG, smem, s, b);
+  return launch_dep(gemm_ffma_kernel<TN, AKM, KG, CAP, SHARED>, total, Shape<TN>::NT * KG, smem, s, b);
 }
 template <int TN, bool AKM, int KG, bool SHARED = false>
 cudaError_t launch_cap(const GemmGroup& g, int total, cudaStream_t s, int kc = 1) {

@@ -178,6 +178,8 @@ struct GemmGroup {
 __device__ __forceinline__ void dep_sync() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
+// The launchers report what their launches returned, not the thread's last error: that may be of an earlier call, and it is the
+// caller's to read.
 template <class T> struct SameType { using type = T; };
 template <class... P>
 inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -192,7 +194,14 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kernel), p);
 }
 
-// The same in clusters of cl CTAs.
+// A kernel that does not wait for its predecessor itself, after it.
+template <class... P>
+inline cudaError_t launch_plain(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, const typename SameType<P>::type&... args) {
+  void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernel(reinterpret_cast<const void*>(kernel), grid, block, p, 0, s);
+}
+
+// The same as launch_dep in clusters of cl CTAs.
 template <class... P>
 inline cudaError_t launch_dep_cluster(int cl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                       const typename SameType<P>::type&... args) {

@@ -560,22 +560,19 @@ static int step_blocks(int64_t n) {
 cudaError_t launch_momentum_step(float* W, const float* G, float* v, int64_t n, float* b, const float* gb, float* vb, int N,
                                  float lr, float momentum, float wd, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(momentum_step_kernel, step_blocks(n), 256, 0, s, W, G, v, n, b, gb, vb, N, lr, momentum, wd);
-  return cudaGetLastError();
+  return launch_dep(momentum_step_kernel, step_blocks(n), 256, 0, s, W, G, v, n, b, gb, vb, N, lr, momentum, wd);
 }
 
 cudaError_t launch_whiteness(const float* A, int M, float* out, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(whiteness_kernel, 1, 1024, 0, s, A, M, out);
-  return cudaGetLastError();
+  return launch_dep(whiteness_kernel, 1, 1024, 0, s, A, M, out);
 }
 
 cudaError_t launch_pilot_mean(const GroupDev& g, const PtrTable& X, const Rows64& rows, const Rows64& ldx,
                               int in_bf16, int max_M, int to_pmean, cudaStream_t s) {
   dim3 grid((max_M + 31) / 32, g.n), block(32, kPilotTY);
   ProfScope ps(FW_PROF_PILOT, s);
-  launch_dep(pilot_mean_kernel, grid, block, 0, s, g, X, rows, ldx, in_bf16, to_pmean);
-  return cudaGetLastError();
+  return launch_dep(pilot_mean_kernel, grid, block, 0, s, g, X, rows, ldx, in_bf16, to_pmean);
 }
 
 cudaError_t launch_accumulate(const GroupDev& g, const int32_t* splits, const int32_t* fresh, const float* corr,
@@ -585,8 +582,7 @@ cudaError_t launch_accumulate(const GroupDev& g, const int32_t* splits, const in
   for (int i = 0; i < g.n; ++i) { a.splits[i] = splits[i]; a.use_acc[i] = fresh[i] ? 0 : 1; a.corr[i] = corr[i]; }
   const int total = fill_tile_table(a.tt, layer_M, g.n);
   ProfScope ps(FW_PROF_MOMENTS, s);
-  launch_dep(accumulate_kernel, total, dim3(32, 8), 0, s, g, a);
-  return cudaGetLastError();
+  return launch_dep(accumulate_kernel, total, dim3(32, 8), 0, s, g, a);
 }
 
 cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t* splits, const int32_t* first,
@@ -598,16 +594,13 @@ cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t*
   for (int i = 0; i < g.n; ++i) {
     a.splits[i] = splits[i]; a.first[i] = first[i]; a.use_acc[i] = use_acc[i]; a.corr[i] = corr[i];
   }
-  { ProfScope ps(FW_PROF_MOMENTS, s); launch_dep(moments_vec_kernel, g.n, 1024, 0, s, g, rows, a); }
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  { ProfScope ps(FW_PROF_MOMENTS, s); e = launch_dep(moments_vec_kernel, g.n, 1024, 0, s, g, rows, a); }
   if (e != cudaSuccess) return e;
   const int total = fill_tile_table(a.tt, layer_M, g.n);
   a.bias_blocks = any_params ? (max_N + 7) / 8 : 0;
-  {
-    ProfScope ps(FW_PROF_MOMENTS, s);
-    launch_dep(moments_mat_kernel, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
-  }
-  return cudaGetLastError();
+  ProfScope ps(FW_PROF_MOMENTS, s);
+  return launch_dep(moments_mat_kernel, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
 }
 
 cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, const int* B, const int* H, const int* W,
@@ -628,8 +621,7 @@ cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, c
   int blocks = (rows + 7) / 8;
   if (blocks > 148 * 8) blocks = 148 * 8;
   ProfScope ps(FW_PROF_PILOT, s);
-  launch_dep(pad_nhwc_kernel, blocks, 256, 0, s, g);
-  return cudaGetLastError();
+  return launch_dep(pad_nhwc_kernel, blocks, 256, 0, s, g);
 }
 
 cudaError_t launch_init_identity(const LayerDev* dev, int M, cudaStream_t s) {
@@ -637,15 +629,13 @@ cudaError_t launch_init_identity(const LayerDev* dev, int M, cudaStream_t s) {
   int blocks = (int)((n + 255) / 256);
   if (blocks > 1184) blocks = 1184;
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(init_identity_kernel, blocks, 256, 0, s, dev);
-  return cudaGetLastError();
+  return launch_dep(init_identity_kernel, blocks, 256, 0, s, dev);
 }
 
 cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s) {
   const int t = (M + 31) / 32;
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(transpose_kernel, dim3(t, t), dim3(32, 8), 0, s, src, dst, M);
-  return cudaGetLastError();
+  return launch_dep(transpose_kernel, dim3(t, t), dim3(32, 8), 0, s, src, dst, M);
 }
 
 template <int N>
@@ -663,8 +653,7 @@ static cudaError_t launch_copies_of(int n, const float* const* src, float* const
     g.first[i + 1] = g.first[i] + (int)((floats[i] + per_cta - 1) / per_cta);
   }
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(copy_kernel<N>, g.first[n], 256, 0, s, g);
-  return cudaGetLastError();
+  return launch_dep(copy_kernel<N>, g.first[n], 256, 0, s, g);
 }
 cudaError_t launch_copies(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
   return n == 1 ? launch_copies_of<1>(n, src, dst, floats, s) : launch_copies_of<FW_MAX_GROUP>(n, src, dst, floats, s);
@@ -672,28 +661,24 @@ cudaError_t launch_copies(int n, const float* const* src, float* const* dst, con
 
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(matT_vec_kernel, (M + 31) / 32, dim3(32, 32), 0, s, A, x, out, M);
-  return cudaGetLastError();
+  return launch_dep(matT_vec_kernel, (M + 31) / 32, dim3(32, 32), 0, s, A, x, out, M);
 }
 
 cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s) {
   (void)M;
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(trace_lambda_kernel, 1, 256, 0, s, dev);
-  return cudaGetLastError();
+  return launch_dep(trace_lambda_kernel, 1, 256, 0, s, dev);
 }
 
 cudaError_t launch_sgd_bias_group(const GroupDev& g, const PtrTable& b, const PtrTable& gb, float lr, int max_N,
                                   cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(sgd_bias_group_kernel, dim3((max_N + 255) / 256, g.n), 256, 0, s, g, b, gb, lr);
-  return cudaGetLastError();
+  return launch_dep(sgd_bias_group_kernel, dim3((max_N + 255) / 256, g.n), 256, 0, s, g, b, gb, lr);
 }
 
 cudaError_t launch_sgd_step(float* W, const float* G, int64_t n, float* b, const float* gb, int N, float lr, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  launch_dep(sgd_step_kernel, step_blocks(n), 256, 0, s, W, G, n, b, gb, N, lr);
-  return cudaGetLastError();
+  return launch_dep(sgd_step_kernel, step_blocks(n), 256, 0, s, W, G, n, b, gb, N, lr);
 }
 
 }  // namespace fw

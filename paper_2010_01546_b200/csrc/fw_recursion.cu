@@ -431,24 +431,26 @@ static cudaError_t recursion_step_launches(const GroupDev& g, int P, int step, c
   const int nblk = (max_M + RBk - 1) / RBk;
   const size_t shm = (size_t)((max_M + 3) & ~3) * sizeof(float);
   dim3 grid(nblk, g.n), block(kGemvThreads);
-  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_ROWNORM, R, C>, grid, block, shm, s, g, 0, 0); }
-  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_CORR, R, C>, grid, block, shm, s, g, 0, 0); }
-  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_ALIGN, R, C>, grid, block, shm, s, g, 0, 0); }
+  cudaError_t e = cudaSuccess;
+  auto keep = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
+  { ProfScope ps(FW_PROF_RECUR_MV, s); keep(launch_dep(recursion_pass_kernel<PASS_ROWNORM, R, C>, grid, block, shm, s, g, 0, 0)); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); keep(launch_dep(recursion_pass_kernel<PASS_CORR, R, C>, grid, block, shm, s, g, 0, 0)); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); keep(launch_dep(recursion_pass_kernel<PASS_ALIGN, R, C>, grid, block, shm, s, g, 0, 0)); }
   int cur = 0;
   for (int p = 0; p < P; ++p) {
     ProfScope ps(FW_PROF_RECUR_MV, s);
-    launch_dep(recursion_pass_kernel<PASS_POWER, R, C>, grid, block, shm, s, g, cur, cur ^ 1);
+    keep(launch_dep(recursion_pass_kernel<PASS_POWER, R, C>, grid, block, shm, s, g, cur, cur ^ 1));
     cur ^= 1;
   }
   dim3 grid2(nblk, g.n, 3);
-  { ProfScope ps(FW_PROF_RECUR_MV, s); launch_dep(recursion_pass_kernel<PASS_FINAL, R, C>, grid2, block, shm, s, g, cur, 0); }
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(recursion_scalars_kernel, g.n, block, 0, s, g, traces, step, RBk); }
+  { ProfScope ps(FW_PROF_RECUR_MV, s); keep(launch_dep(recursion_pass_kernel<PASS_FINAL, R, C>, grid2, block, shm, s, g, cur, 0)); }
+  { ProfScope ps(FW_PROF_RECUR_UPD, s); keep(launch_dep(recursion_scalars_kernel, g.n, block, 0, s, g, traces, step, RBk)); }
   {
     const int t32 = (max_M + 31) / 32;
     ProfScope ps(FW_PROF_RECUR_UPD, s);
-    launch_dep(recursion_update_leaky_kernel, dim3(t32, t32, g.n), dim3(32, 8), 0, s, g);
+    keep(launch_dep(recursion_update_leaky_kernel, dim3(t32, t32, g.n), dim3(32, 8), 0, s, g));
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // row_blocks: 32-row blocks that have rows to work on, summed over the group's layers
@@ -470,8 +472,7 @@ cudaError_t launch_smooth(const GroupDev& g, int max_M, cudaStream_t s) {
   if (bx > 1184) bx = 1184;
   if (bx < 1) bx = 1;
   ProfScope ps(FW_PROF_SMOOTH, s);
-  launch_dep(smooth_kernel, dim3(bx, g.n), 256, 0, s, g);
-  return cudaGetLastError();
+  return launch_dep(smooth_kernel, dim3(bx, g.n), 256, 0, s, g);
 }
 
 }  // namespace fw

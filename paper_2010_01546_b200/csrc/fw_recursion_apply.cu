@@ -335,10 +335,9 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
     a.block0[g.n] = n;
     if (n == 0) continue;
     ProfScope ps(FW_PROF_RECUR_UPD, s);
-    launch_dep(kernels[kind], n, AT, kind ? sizeof(float) * longest : 0, s, a);      // at most 32 KB
+    const cudaError_t e = launch_dep(kernels[kind], n, AT, kind ? sizeof(float) * longest : 0, s, a);      // at most 32 KB
+    if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
   n = 0;
   for (int i = 0; i < g.n; ++i) {
     const int M = layer_M[i];
@@ -346,8 +345,8 @@ cudaError_t launch_recursion_apply(const GroupDev& g, const int* layer_M, int K,
     n += (int)(((int64_t)q_units(M) * ((M + QR - 1) / QR) + AT - 1) / AT);
   }
   a.block0[g.n] = n;
-  { ProfScope ps(FW_PROF_RECUR_UPD, s); launch_dep(apply_q_kernel, n, AT, 0, s, a); }
-  return cudaGetLastError();
+  ProfScope ps(FW_PROF_RECUR_UPD, s);
+  return launch_dep(apply_q_kernel, n, AT, 0, s, a);
 }
 
 }  // namespace fw

@@ -156,23 +156,23 @@ extern "C" fw_status fw_cov_block_static(const float* X, int64_t rows, int64_t l
   const int sp = (int)splits;
   const float inv_rows = 1.0f / (float)rows;
   const int t = (M + 31) / 32;
+  cudaError_t e;
   {
     fw::ProfScope ps(FW_PROF_MISC, s);
-    static_colsum_kernel<<<dim3(t, sp), dim3(32, 8), 0, s>>>(X, rows, ldx, M, sp, scratch);
+    e = fw::launch_plain(static_colsum_kernel, dim3(t, sp), dim3(32, 8), s, X, rows, ldx, M, sp, scratch);
   }
-  {
+  if (e == cudaSuccess) {
     fw::ProfScope ps(FW_PROF_MISC, s);
-    static_mean_kernel<<<(M + 127) / 128, 128, 0, s>>>(scratch, sp, M, inv_rows, mu_out);
+    e = fw::launch_plain(static_mean_kernel, (M + 127) / 128, 128, s, scratch, sp, M, inv_rows, mu_out);
   }
-  {
+  if (e == cudaSuccess) {
     fw::ProfScope ps(FW_PROF_MISC, s);
-    static_gram_kernel<<<dim3(t, t, sp), dim3(32, 8), 0, s>>>(X, mu_out, rows, ldx, M, sp, scratch);
+    e = fw::launch_plain(static_gram_kernel, dim3(t, t, sp), dim3(32, 8), s, X, mu_out, rows, ldx, M, sp, scratch);
   }
-  {
+  if (e == cudaSuccess) {
     fw::ProfScope ps(FW_PROF_MISC, s);
-    static_reduce_kernel<<<dim3(t, (M + 7) / 8), dim3(32, 8), 0, s>>>(scratch, sp, M, inv_rows, phix_out);
+    e = fw::launch_plain(static_reduce_kernel, dim3(t, (M + 7) / 8), dim3(32, 8), s, scratch, sp, M, inv_rows, phix_out);
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     fprintf(stderr, "[fw] fw_cov_block_static: launch failed: %s\n", cudaGetErrorString(e));
     return FW_ERR_CUDA;

@@ -1005,9 +1005,8 @@ fw_status umma_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
     }
     g.n = cnt;
     ProfScope ps(FW_PROF_GRAM, s);
-    if (group_bf16) launch_dep(gram_umma_kernel<true>, total_ctas, GR_THREADS, smem, s, g);
-    else launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = group_bf16 ? launch_dep(gram_umma_kernel<true>, total_ctas, GR_THREADS, smem, s, g)
+                                     : launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_umma_kernel launch: %s\n", cudaGetErrorString(e));
       return FW_ERR_CUDA;
@@ -1043,8 +1042,7 @@ __global__ void wait_probe_kernel(int32_t* status, uint32_t polls) {
 
 cudaError_t launch_wait_probe(int32_t* status, uint32_t polls, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
-  wait_probe_kernel<<<1, 32, 0, s>>>(status, polls);
-  return cudaGetLastError();
+  return launch_plain(wait_probe_kernel, 1, 32, s, status, polls);
 }
 
 // D = A^T B for square fp32 matrices (TF32 inputs rounded to nearest, fp32 accumulation):
@@ -1084,8 +1082,7 @@ fw_status umma_atb_launch(const UmmaAtbItem* items, int n, cudaStream_t s) {
     }
     g.n = cnt;
     ProfScope ps(FW_PROF_RESYNC, s);
-    launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_umma_kernel (A^T B) launch: %s\n", cudaGetErrorString(e));
       return FW_ERR_CUDA;

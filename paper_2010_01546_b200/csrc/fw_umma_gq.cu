@@ -452,11 +452,11 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
     }
     if (nitems < 1 || nitems > (int64_t)QP_MAX_ITEMS) return FW_ERR_SHAPE;
     g.n = cnt; g.nitems = (int)nitems;
+    cudaError_t e;
     {
       ProfScope ps(prof_class, s);
-      launch_dep(gq_pair_kernel, 2 * std::min(g.nitems, (int)pairs), QP_THREADS, smem, s, g);
+      e = launch_dep(gq_pair_kernel, 2 * std::min(g.nitems, (int)pairs), QP_THREADS, smem, s, g);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gq_pair_kernel launch: %s\n", cudaGetErrorString(e));
       return FW_ERR_CUDA;
@@ -465,8 +465,7 @@ fw_status umma_gq_pair_launch(const UmmaGqItem* items_in, int n, int epi, float 
       int64_t blocks = (gr.total4 + 255) / 256;
       if (blocks > 8 * sm_count()) blocks = 8 * sm_count();
       ProfScope ps(prof_class, s);
-      launch_dep(gq_reduce_kernel, (int)blocks, 256, 0, s, gr);
-      e = cudaGetLastError();
+      e = launch_dep(gq_reduce_kernel, (int)blocks, 256, 0, s, gr);
       if (e != cudaSuccess) {
         fprintf(stderr, "[fw] gq_reduce_kernel launch: %s\n", cudaGetErrorString(e));
         return FW_ERR_CUDA;

@@ -716,9 +716,8 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
     for (size_t i = 0; i < items.size(); ++i) g.item[i] = items[i].code;
     g.n = cnt; g.nitems = (int)items.size();
     ProfScope ps(prof_class, s);
-    if (specs[base].bf16) launch_dep(gram_pair_kernel<true>, 2 * g.nitems, GP_THREADS, smem, s, g);
-    else launch_dep(gram_pair_kernel<false>, 2 * g.nitems, GP_THREADS, smem, s, g);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = specs[base].bf16 ? launch_dep(gram_pair_kernel<true>, 2 * g.nitems, GP_THREADS, smem, s, g)
+                                           : launch_dep(gram_pair_kernel<false>, 2 * g.nitems, GP_THREADS, smem, s, g);
     if (e != cudaSuccess) {
       fprintf(stderr, "[fw] gram_pair_kernel launch: %s\n", cudaGetErrorString(e));
       return FW_ERR_CUDA;

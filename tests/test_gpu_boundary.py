@@ -1,6 +1,8 @@
 """GPU tests of the boundary's finer points, through the C ABI: blocks spread over
 several calls (FW_COV_ACCUMULATE), the in-place gradient transform, per-layer
 device-side status (time-out, non-finite values), against the fp64 oracle."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -268,3 +270,28 @@ def test_first_reduction_copies_every_layer(env, gamma):
     B.fw_group_cond_reduce([L.handle for L in Ls], 0, 0)
     for L, P in zip(Ls, Ps):
         assert torch.equal(L.get(B.FW_F_PHIY).reshape(P.shape), P)
+
+
+def test_an_error_of_one_call_is_not_reported_by_the_next(env):
+    """Reading the status waits for the stream, which a capture does not allow: that call fails, and the runtime keeps its error as
+    the thread's last one.  The calls after it report their own launches."""
+    torch, B = env
+    runtime = ctypes.CDLL("libcudart.so.12")                            # torch's; the library has one of its own
+    M = 40
+    stream = torch.cuda.Stream()
+    raw, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    L = B.Layer(M, 4, stream=stream.cuda_stream, beta=0.0, gamma=1.0)
+    out = torch.zeros(M, M, device="cuda")
+    X = torch.randn(200, M, device="cuda")
+    torch.cuda.synchronize()
+    assert runtime.cudaStreamBeginCapture(raw, 2) == 0                  # relaxed
+    with pytest.raises(B.FwError) as e:
+        L.sync_status()
+    assert e.value.status == B.FW_ERR_CUDA
+    assert runtime.cudaStreamEndCapture(raw, ctypes.byref(graph)) != 0 and not graph.value
+    runtime.cudaGetLastError()
+    B.fw_layer_get(L.handle, B.FW_F_Q, out, M * M * 4)
+    L.cov_update(X)
+    L.cond_reduce(1, 2)
+    assert L.sync_status() == B.FW_OK
+    assert torch.equal(out, torch.eye(M, device="cuda"))
