@@ -942,11 +942,13 @@ fw_status fw_layer_get(fw_layer* L, fw_field f, void* dev_dst, size_t bytes) {
     FW_CUDA(launch_transpose(L->h.Tt, (float*)dev_dst, L->d.M, L->stream), "get T");
     return FW_OK;
   }
-  // A kernel of ours is set up while the launch before it drains, a copy by the driver is not: 64 matrices of M = 256 in a row
-  // 1.4 us each instead of 3.5 (M = 1152: 225 -> 100 us).  It takes whole floats of this device's own memory; anything else the
-  // driver copies.
+  // A kernel of ours is set up while the launch before it drains, a copy by the driver is not: matrices in a row, M = 256 1.4 us each
+  // instead of 3.1, 1152 3.6 instead of 5.1, 4608 28.4 instead of 28.9.  From M = 6144 on (144 MiB) the driver is faster: 6656 57.4 us
+  // against 59.7, 8192 84.1 against 91.0.  Where the destination is not 16-byte aligned the kernel moves single floats, and
+  // the line is 24 MiB: M = 2305 13.5 us (driver 13.9), 3001 21.1 (18.5).  The kernel takes whole floats of this device's own memory.
   bool own = false;
-  if ((reinterpret_cast<uintptr_t>(dev_dst) & 3) == 0) {
+  const uintptr_t to = reinterpret_cast<uintptr_t>(dev_dst);
+  if ((to & 3) == 0 && need < (size_t)((to & 15) == 0 ? 144 : 24) << 20) {
     cudaPointerAttributes at;
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);

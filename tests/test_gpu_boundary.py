@@ -255,6 +255,21 @@ def test_layer_get_writes_the_field_and_nothing_else(env, M, offset):
         assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + n:] == 7.0).all())
 
 
+@pytest.mark.parametrize("M,offset,kernels", [(2507, 1, 1), (2509, 1, 0), (2509, 0, 1), (6143, 0, 1), (6144, 0, 0)])
+def test_layer_get_of_large_fields(env, M, offset, kernels):
+    """The driver copies where it is the faster one: from 144 MiB on, from 24 MiB on where a destination is not 16-byte aligned."""
+    torch, B = env
+    L = B.Layer(M, 4, beta=0.0, gamma=1.0)
+    A = torch.randn((M, M), device="cuda")
+    L.set(B.FW_F_PHIX, A)
+    buf = torch.full((M * M + 9,), 7.0, device="cuda")
+    n0 = B.fw_launch_count()
+    B.fw_layer_get(L.handle, B.FW_F_PHIX, buf[offset:], 4 * M * M)
+    assert B.fw_launch_count() - n0 == kernels
+    assert torch.equal(buf[offset:offset + M * M], A.reshape(-1))
+    assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + M * M:] == 7.0).all())
+
+
 @pytest.mark.parametrize("gamma", [1.0, 0.99])
 def test_first_reduction_copies_every_layer(env, gamma):
     """T = I: Phi_y = Phi_x bit for bit, for a full group of mixed sizes (a leaky layer copies twice: more copies than one
