@@ -453,12 +453,14 @@ cudaError_t launch_gemm_ffma(GemmGroup& g, cudaStream_t s, int prof_class) {
   // A tile is 64 x 64 x K products on one SM, 9.4 us of its FP32 pipe at K = 576: with few tiles a cluster of CTAs shares each, as
   // long as a group keeps four slabs of the longest K and the clusters fill at most three quarters of the SMs (beyond that two
   // CTAs meet on an SM, and 36 tiles of K = 576 took 30 us on four CTAs each instead of 22 on one).  G Qs, one CTA -> shared:
-  // 64 x 576 22 -> 13 us, 256 x 576 22 -> 16, 64 x 1024 36 -> 15, 16 x 2304 68 -> 38; not taken: 16 x 144 8.7 -> 9.7.
+  // 64 x 576 22 -> 13 us, 256 x 576 22 -> 16, 64 x 1024 36 -> 15, 16 x 2304 68 -> 38; not taken: 16 x 144 8.7 -> 9.7.  The longest
+  // K decides for a group of several: it is the last to end, and the others' clusters fit beside it (67 x 27 and 67 x 603 16.9 us,
+  // 67 x 603 alone 17.0, both unshared 30.7).  Eight CTAs a tile would need K above 1000 in at most 13 tiles, and there are at least K / 64.
   int kc = 1;
   int64_t kslabs = 0;
   bool whole = true;                  // column sums and row splits are the Gram pass's, whose partition is the caller's
   for (int i = 0; i < g.n; ++i) { kslabs = std::max(kslabs, (g.p[i].k + BK - 1) / BK); whole = whole && !g.p[i].colsum && g.p[i].splits == 1; }
-  while (whole && kc < 8 && 8 * kc * total <= 3 * sms && kslabs >= 16 * kc) kc *= 2;
+  while (whole && kc < 4 && 8 * kc * total <= 3 * sms && kslabs >= 16 * kc) kc *= 2;
   if (!g.p[0].a_kmajor) {
     if (total >= 4 * sms) return launch_cap<4, false, 1>(g, total, s);
     if (kc > 1) return launch_cap<4, false, 4, true>(g, total, s, kc);
