@@ -229,8 +229,9 @@ fw_status fw_step_momentum(fw_layer* L, float* W, float* b, const float* G_t, co
  * The gradient transform, the step and a later fw_cond_reduce continue from this
  * state.  scratch: caller-owned device memory, 256-byte aligned, at least
  * fw_evd_scratch_bytes(M) bytes per layer, used only during the call's kernels.
- * Cost: about 5 M^3 fp64 operations per sweep and 6-10 sweeps (up to twice as many
- * where Phi_x is not positive definite: then its Cholesky factor is no start); M / 16 - 1
+ * Cost: about 5 M^3 fp64 operations per sweep and 6-14 sweeps (10 for M = 576, fewer
+ * for graded matrices; up to 40 where Phi_x is not safely positive definite: then
+ * its Cholesky factor is no start); M / 16 - 1
  * barriers of the layer's CTAs per sweep (bounded waits; a time-out is reported
  * by fw_layer_sync_status as FW_ERR_TIMEOUT).  Errors: FW_ERR_STATE without a
  * covariance or inside an open block, FW_ERR_WORKSPACE for a short scratch. */

@@ -252,8 +252,8 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
 // tiles over all layers of the group (a grid sized for the largest layer would be mostly empty CTAs when the
 // layers differ in size, and handing those out costs more than the work).  Bound by the latency of the split partials where
 // layers are small, by HBM where they are large; with a 16-byte access per row and split instead of four rows of 4 bytes one
-// after the other: 376 -> 368 us a step of the
-// ResNet-20-shaped set, 5107 -> 5046 of the ResNet-50-shaped set, 343 -> 324 of one with odd sizes.
+// after the other, and moments_vec_kernel's sums batched: 368 -> 362 us a step of the
+// ResNet-20-shaped set, 5074 -> 5005 of the ResNet-50-shaped set, 342 -> 321 of one with odd sizes.
 __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a,
