@@ -60,8 +60,8 @@ def test_no_full_rank(env, kind):
 @pytest.mark.parametrize("kind", ["graded", "singular", "indefinite", "clustered"])
 def test_start_from_the_factor_or_from_phi(env, M, kind):
     """Graded matrices (D A D, D powers of two: eigenvalues over eight decades) are factored; one exact dependence, or a
-    negative eigenvalue, and the rotations start from Phi itself.  Clustered: eigenvalues that differ by less than the fp32
-    products of a visit can tell."""
+    negative eigenvalue, and the rotations start from Phi itself.  Clustered: eigenvalues that differ by less than fp32 can
+    tell."""
     rng = np.random.default_rng(M)
     B = rng.standard_normal((M, 2 * M)) / np.sqrt(2 * M)
     Phi = (B @ B.T).astype(np.float32).astype(np.float64)
