@@ -96,6 +96,7 @@ size_t carve(const fw_layer_desc& d, char* base, LayerDev* h) {
   L.Qs = (d.beta > 0.f) ? (float*)take(mat) : L.Q;
   L.tmp = (float*)take(mat);
   L.split_cap = std::max(split_cap_for(d.M), d.prec != FW_PREC_FP32 ? umma_pair_split_cap(d.M) : 1);
+  L.round_t = d.prec != FW_PREC_FP32 && d.gamma == 1.0f && d.M >= 16 && (d.M & 3) == 0;
   L.gram_part = (float*)take((size_t)L.split_cap * mat);
   L.colsum_part = (float*)take((size_t)L.split_cap * vec);
   L.gram_acc = (float*)take(mat);
@@ -141,6 +142,20 @@ void fill_group(fw_layer* const* L, int n, GroupDev& g, int& max_M, int& max_N) 
   }
 }
 
+// tmp <- T^T rounded, for the layers that keep it
+cudaError_t round_T(fw_layer* const* L, int n) {
+  const float* src[FW_MAX_GROUP];
+  float* dst[FW_MAX_GROUP];
+  int64_t floats[FW_MAX_GROUP];
+  int k = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!L[i]->h.round_t) continue;
+    src[k] = L[i]->h.Tt; dst[k] = L[i]->h.tmp; floats[k] = (int64_t)L[i]->d.M * L[i]->d.M;
+    ++k;
+  }
+  return k ? launch_round(k, src, dst, floats, L[0]->stream) : cudaSuccess;
+}
+
 // Phiy <- T Phix T^T for the layers whose Phiy is stale (a5).  With T kept transposed
 // (Tt = T^T) both products have the form A^T B:  tmp = Phix^T Tt (= Phix T^T, Phix is
 // symmetric) and Phiy = Tt^T tmp.  Tensor-core engines run them as TF32 MMAs, the FP32
@@ -163,12 +178,17 @@ fw_status resync_phiy(fw_layer* const* L, int n) {
       if (l->d.gamma != 1.0f) add_copy(l->h.Phix, l->h.tmp, (int64_t)M * M);     // Pt = (T Phix)^T = Phix at T = I
     } else if (l->d.prec != FW_PREC_FP32 && umma_available() && M >= 16 && (M % 4) == 0) {
       const bool pair = umma_pair_atb_eligible(M);
+      // A layer without leakage keeps T^T rounded to TF32 in tmp, and its first product is wanted only as the operand of the
+      // second: it is written rounded, in the place of the partial Gram matrices.  A leaky one keeps the product in tmp.
+      const bool rounded = l->h.round_t != 0;
+      const float* const T = rounded ? l->h.tmp : l->h.Tt;
+      float* const prod = rounded ? l->h.gram_part : l->h.tmp;
       UmmaAtbItem it;
       it.status = l->h.iscal + IS_STATUS_TIMEOUT;
-      it.A = l->h.Phix; it.B = l->h.Tt; it.C = l->h.tmp; it.M = M; it.sym = 0;
+      it.A = l->h.Phix; it.B = T; it.C = prod; it.M = M; it.sym = 0; it.round_c = rounded; it.fix = rounded ? 1 : 3;
       (pair ? p1 : t1).push_back(it);
       // T (Phix T^T) is symmetric: its upper triangle is computed and mirrored by the kernel
-      it.A = l->h.Tt; it.B = l->h.tmp; it.C = l->h.Phiy; it.M = M; it.sym = 1;
+      it.A = T; it.B = prod; it.C = l->h.Phiy; it.sym = 1; it.round_c = 0; it.fix = rounded ? 0 : 3;
       (pair ? p2 : t2).push_back(it);
     } else {
       GemmProblem p;
@@ -846,6 +866,7 @@ fw_status fw_group_evd_whiten(fw_layer* const* L, int32_t n, void* const* scratc
   cudaStream_t s = L[0]->stream;
   FW_CUDA(launch_evd(n, src, dims, scratch, status, eps, true, g_max, t_out, q_out, y_out, nullptr, nullptr, s),
           "evd whitening");
+  FW_CUDA(round_T(L, n), "evd whitening: T rounded");
   GroupDev g; int max_M, max_N;
   fill_group(L, n, g, max_M, max_N);
   bool any_beta = false;
@@ -978,6 +999,7 @@ fw_status fw_layer_set(fw_layer* L, fw_field f, const void* dev_src, size_t byte
   const int M = L->d.M;
   if (f == FW_F_T) {
     FW_CUDA(launch_transpose((const float*)dev_src, L->h.Tt, M, L->stream), "set T");
+    FW_CUDA(round_T(&L, 1), "set T: rounded");
     // Q = T^T T = Tt Tt^T: A = Tt (m x k), B[k][j] = Tt[j][k] = T[k][j]
     GemmGroup g; g.n = 1;
     GemmProblem& p = g.p[0];

@@ -32,7 +32,8 @@ struct LayerDev {
   float* Tt;            // MxM T^T (stored transposed so that t = T^T v is a row GEMV)
   float* Q;             // MxM T^T T
   float* Qs;            // MxM smoothed Q (aliases Q when beta == 0)
-  float* tmp;           // MxM Pt = (T Phix)^T: re-sync intermediate, and state of the leaky (gamma < 1) update
+  float* tmp;           // MxM Pt = (T Phix)^T: re-sync intermediate, and state of the leaky (gamma < 1) update; with round_t,
+                        // T^T rounded to TF32
   // recursion vectors
   float* xi2;           // M   squared column norms
   float* cvec;          // M   correlations with column m'
@@ -50,7 +51,8 @@ struct LayerDev {
   float* gram_part;     // split_cap x M x M partial Gram matrices
   float* colsum_part;   // split_cap x M partial column sums
   int32_t split_cap;
-  int32_t pad3;
+  int32_t round_t;      // tensor-core layers without leakage: whatever writes Tt writes its values rounded to TF32 to tmp, as
+                        // operands of the re-sync products
   // a block spread over several calls (FW_COV_ACCUMULATE): sums of the calls before the committing one
   float* gram_acc;      // M x M (upper-triangle tiles)
   float* colsum_acc;    // M
@@ -302,6 +304,8 @@ cudaError_t launch_init_identity(const LayerDev* dev, int M, cudaStream_t s);
 cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s);
 // dst[i] <- src[i], floats[i] floats of this device's memory, n <= FW_MAX_GROUP copies in one launch
 cudaError_t launch_copies(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s);
+// the same, rounded to the TF32 grid (nearest, ties away): operands of a re-sync product
+cudaError_t launch_round(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s);
 // out[j] = sum_k A[k][j] x[k] for a row-major M x M matrix A (A^T x)
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s);
 cudaError_t launch_trace_lambda(const LayerDev* dev, int M, cudaStream_t s);

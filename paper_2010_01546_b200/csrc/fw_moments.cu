@@ -10,6 +10,7 @@
 #include <cstring>
 
 #include "fw_internal.h"
+#include "fw_sm100.cuh"
 
 namespace fw {
 namespace {
@@ -389,6 +390,7 @@ __global__ void init_identity_kernel(const LayerDev* L) {
     const int i = (int)(e / M), j = (int)(e - (int64_t)i * M);
     const float d = (i == j) ? 1.f : 0.f;
     L->Tt[e] = d;
+    if (L->round_t) L->tmp[e] = d;
     L->Q[e] = d;
     if (!alias) L->Qs[e] = d;
     L->Phix[e] = 0.f;
@@ -432,7 +434,8 @@ struct CopyGroup {
   int32_t first[N + 1];                 // first CTA of each copy
   int32_t copies;
 };
-template <int N>
+// ROUND: the copy is rounded to the TF32 grid (nearest, ties away)
+template <int N, bool ROUND>
 __global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyGroup<N> g) {
   dep_sync();
   int c = 0;
@@ -442,13 +445,17 @@ __global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyG
   const float* src = g.src[c];
   float* dst = g.dst[c];
   const int n = g.n[c], step = 256 * (g.first[c + 1] - g.first[c]), i0 = 256 * ((int)blockIdx.x - g.first[c]) + threadIdx.x;
+  auto val = [](float x) { return ROUND ? sm100::tf32_rna(x) : x; };
   if (g.v4[c]) {
 #pragma unroll 4
-    for (int i = i0; i < (n >> 2); i += step) reinterpret_cast<float4*>(dst)[i] = reinterpret_cast<const float4*>(src)[i];
-    if (i0 < (n & 3)) dst[(n & ~3) + i0] = src[(n & ~3) + i0];
+    for (int i = i0; i < (n >> 2); i += step) {
+      const float4 x = reinterpret_cast<const float4*>(src)[i];
+      reinterpret_cast<float4*>(dst)[i] = make_float4(val(x.x), val(x.y), val(x.z), val(x.w));
+    }
+    if (i0 < (n & 3)) dst[(n & ~3) + i0] = val(src[(n & ~3) + i0]);
   } else {
 #pragma unroll 4
-    for (int i = i0; i < n; i += step) dst[i] = src[i];
+    for (int i = i0; i < n; i += step) dst[i] = val(src[i]);
   }
 }
 
@@ -640,7 +647,7 @@ cudaError_t launch_transpose(const float* src, float* dst, int M, cudaStream_t s
   return launch_dep(transpose_kernel, dim3(t, t), dim3(32, 8), 0, s, src, dst, M);
 }
 
-template <int N>
+template <int N, bool ROUND>
 static cudaError_t launch_copies_of(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
   CopyGroup<N> g;
   memset(&g, 0, sizeof(g));
@@ -654,11 +661,14 @@ static cudaError_t launch_copies_of(int n, const float* const* src, float* const
     g.v4[i] = ((reinterpret_cast<uintptr_t>(src[i]) | reinterpret_cast<uintptr_t>(dst[i])) & 15) == 0;
     g.first[i + 1] = g.first[i] + (int)((floats[i] + per_cta - 1) / per_cta);
   }
-  ProfScope ps(FW_PROF_MISC, s);
-  return launch_dep(copy_kernel<N>, g.first[n], 256, 0, s, g);
+  ProfScope ps(ROUND ? FW_PROF_RESYNC : FW_PROF_MISC, s);
+  return launch_dep(copy_kernel<N, ROUND>, g.first[n], 256, 0, s, g);
 }
 cudaError_t launch_copies(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
-  return n == 1 ? launch_copies_of<1>(n, src, dst, floats, s) : launch_copies_of<FW_MAX_GROUP>(n, src, dst, floats, s);
+  return n == 1 ? launch_copies_of<1, false>(n, src, dst, floats, s) : launch_copies_of<FW_MAX_GROUP, false>(n, src, dst, floats, s);
+}
+cudaError_t launch_round(int n, const float* const* src, float* const* dst, const int64_t* floats, cudaStream_t s) {
+  return n == 1 ? launch_copies_of<1, true>(n, src, dst, floats, s) : launch_copies_of<FW_MAX_GROUP, true>(n, src, dst, floats, s);
 }
 
 cudaError_t launch_matT_vec(const float* A, const float* x, float* out, int M, cudaStream_t s) {

@@ -18,6 +18,7 @@
 
 #include "fw_internal.h"
 #include "fw_lanes.cuh"
+#include "fw_sm100.cuh"
 
 namespace fw {
 namespace {
@@ -59,6 +60,10 @@ __device__ __forceinline__ double dot4(float4 r, float4 x, double acc) {
 }
 __device__ __forceinline__ float4 axpy4(float a, float4 x, float4 r) {
   return make_float4(fmaf(a, x.x, r.x), fmaf(a, x.y, r.y), fmaf(a, x.z, r.z), fmaf(a, x.w, r.w));
+}
+// on the TF32 grid (the operand of the re-sync products that a layer with round_t keeps)
+__device__ __forceinline__ float4 rounded4(float4 r) {
+  return make_float4(sm100::tf32_rna(r.x), sm100::tf32_rna(r.y), sm100::tf32_rna(r.z), sm100::tf32_rna(r.w));
 }
 __device__ __forceinline__ float abs4(float4 r) { return fabsf(r.x) + fabsf(r.y) + fabsf(r.z) + fabsf(r.w); }
 constexpr float kFinite = 1e37f;    // numbers whose absolute values sum to less are finite
@@ -118,8 +123,12 @@ __device__ __forceinline__ void row_steps(float* __restrict__ row, const LayerDe
   for (int n = 0; n < NV; ++n) {
     const int c = t + 32 * n;
     if (c >= MU) continue;
-    if (V == 4) reinterpret_cast<float4*>(row)[c] = r4[n];
-    else row[c] = r1[n];
+    if (V == 4) {
+      reinterpret_cast<float4*>(row)[c] = r4[n];
+      if (L->round_t) reinterpret_cast<float4*>(L->tmp + (size_t)i * M)[c] = rounded4(r4[n]);
+    } else {
+      row[c] = r1[n];
+    }
   }
 }
 // A longer row in the registers of a CTA, at most AT V NV entries.  The sum runs over all threads, in another order; where
@@ -209,8 +218,13 @@ __device__ __forceinline__ void long_row_steps(float* __restrict__ row, float* c
   for (int n = 0; n < NV; ++n) {
     const int c = t + AT * n;
     if (c < MU) {
-      if (V == 4) reinterpret_cast<float4*>(row)[c] = *reinterpret_cast<const float4*>(r[n]);
-      else row[c] = r[n][0];
+      if (V == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(r[n]);
+        reinterpret_cast<float4*>(row)[c] = q;
+        if (L->round_t) reinterpret_cast<float4*>(L->tmp + (size_t)i * M)[c] = rounded4(q);
+      } else {
+        row[c] = r[n][0];
+      }
     }
   }
 }

@@ -304,7 +304,8 @@ __device__ __forceinline__ void load_rows(float4 (&a)[4 * NG][IT], const float* 
     }
   }
 }
-template <int NG, int IT, bool V4>
+// ROUND: rounded to the TF32 grid
+template <int NG, int IT, bool V4, bool ROUND = false>
 __device__ __forceinline__ void store_rows(const float4 (&a)[4 * NG][IT], float* G, const Slab& s) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = s.M;
@@ -317,7 +318,9 @@ __device__ __forceinline__ void store_rows(const float4 (&a)[4 * NG][IT], float*
     for (int k = 0; k < IT; ++k) {
       const int c = lane + 32 * k;
       if (V4) {
-        if (4 * c < M) reinterpret_cast<float4*>(row)[c] = a[q][k];
+        float4 v = a[q][k];
+        if (ROUND) v = make_float4(sm100::tf32_rna(v.x), sm100::tf32_rna(v.y), sm100::tf32_rna(v.z), sm100::tf32_rna(v.w));
+        if (4 * c < M) reinterpret_cast<float4*>(row)[c] = v;
       } else {
         if (4 * c < M) row[4 * c] = a[q][k].x;
         if (4 * c + 1 < M) row[4 * c + 1] = a[q][k].y;
@@ -377,6 +380,7 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
       }
     }
     store_rows<NG, IT, V4>(a, L->Tt, s);
+    if (V4 && L->round_t) store_rows<NG, IT, true, true>(a, L->tmp, s);
   } else {
     arm(l, e, 0u);
   }
@@ -686,7 +690,7 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     }
     // ---- the recorded steps in T, then Q (Eqs. 42, 44), as in apply_steps ----
     const bool last = k1 == K;
-    float4 t[KM];
+    float4 t[KM], o[KM];
     auto load = [&](float4 (&r)[KM], const float* G) {
 #pragma unroll
       for (int k = 0; k < KM; ++k) {
@@ -737,6 +741,12 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
       }
     }
     save(t, L->Tt);
+    if (L->round_t) {                    // rows of whole float4s
+#pragma unroll
+      for (int k = 0; k < KM; ++k)
+        o[k] = make_float4(sm100::tf32_rna(t[k].x), sm100::tf32_rna(t[k].y), sm100::tf32_rna(t[k].z), sm100::tf32_rna(t[k].w));
+      save(o, L->tmp);
+    }
     load(t, L->Q);
     __syncthreads();
 #pragma unroll 1
@@ -755,7 +765,6 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     save(t, L->Q);
     if (last && smooth) {
       const float beta = L->beta, ob = 1.f - beta;
-      float4 o[KM];
       load(o, L->Qs);
 #pragma unroll
       for (int k = 0; k < KM; ++k) {

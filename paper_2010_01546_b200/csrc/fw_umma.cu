@@ -2,8 +2,8 @@
 // staged in shared memory by TMA, warp-specialised (one TMA producer warp, one
 // MMA issuer warp, four epilogue warps), mbarrier pipeline with bounded waits.
 //
-//   gram_umma_kernel  X^T X with column sums (Eqs. 3, 5), and the re-sync products A^T B,
-//                     one CTA per tile.  (G Qs runs on CTA pairs: fw_umma_gq.cu.)
+//   gram_umma_kernel  X^T X with column sums (Eqs. 3, 5), one CTA per tile.  (The re-sync products: fw_umma_atb.cu;
+//                     G Qs runs on CTA pairs: fw_umma_gq.cu.)
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -160,9 +160,6 @@ struct GramProblem {
   int32_t ntiles;          // tiles per split (1 in STREAM mode)
   int32_t first_cta;
   int32_t rows_per_split;  // multiple of GR_SR
-  int32_t full;            // 1: D = A^T B with A from mapX, B from mapB, every tile of the full output;
-                           // 2: the same for a symmetric D: tiles wholly below the diagonal are skipped, the others
-                           //    write their entries on and above the diagonal and mirror those above it
   int32_t fixup;           // fp32 only. 1: subtract shift, round to TF32, write back; 0: read-only column sums
   int32_t use3d;           // 1: chunked 3-D tensor maps (map3a / map3b): one TMA instruction per column range
   int32_t box_a;           // chunks per map3a box (STREAM: all chunks; TILED: 4)
@@ -189,9 +186,8 @@ __device__ __forceinline__ int i2c_col(int mp, int cpr, int c3) {
 }
 struct GramGroup {
   CUtensorMap mapX[kMaxUmmaGroup];
-  CUtensorMap mapB[kMaxUmmaGroup];   // second source, used only by problems with full = 1
   CUtensorMap map3a[kMaxUmmaGroup];  // chunked 3-D views (use3d = 1): A-side box, and
-  CUtensorMap map3b[kMaxUmmaGroup];  // B-side box of 8 chunks (on the second source when full = 1)
+  CUtensorMap map3b[kMaxUmmaGroup];  // B-side box of 8 chunks
   GramProblem p[kMaxUmmaGroup];
   int32_t n;
 };
@@ -247,11 +243,6 @@ __device__ __forceinline__ float4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-// round-to-nearest (ties away) of an fp32 value to the TF32 grid, on the integer pipe
-__device__ __forceinline__ float tf32_rna(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
-
 // BF = true: bf16 X (kind::f16), BF = false: fp32 X (kind::tf32).  All per-stage
 // loops are free of divisions and descriptor rebuilding: the single issuing
 // threads of the producer and MMA warps run serial code, so every instruction in
@@ -269,7 +260,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
   __shared__ int abort_flag;
   __shared__ GramOp ops[GR_MAX_OPS];
   __shared__ int s_nops, s_nslots, s_r0_col, s_r0_slots, s_r1_col, s_r1_slots, s_tmem_cols, s_cs_slots, s_ones;
-  __shared__ int s_slack_chunks, s_skip;
+  __shared__ int s_slack_chunks;
   __shared__ float s_csred[GR_FIX_WARPS][GR_MAX_SLOTS * GR_CW];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -288,7 +279,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    s_skip = 0;
     int nops = 0, tcol = 0;
     int ones = 0;
     if (pr.stream) {
@@ -298,7 +288,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
       // runs on into it, so the column sums of the values as the tensor core reads them come out as 16 extra
       // accumulator columns and no thread has to read the stage.  Taken when no fix-up pass is owed and the
       // widened MMAs fit (N <= 256, 512 accumulator columns in all).
-      if (!pr.fixup && !pr.full) ones = gram_ones_fits(M16) ? 1 : 0;
+      if (!pr.fixup) ones = gram_ones_fits(M16) ? 1 : 0;
       for (int i = 0; i < nb; ++i) {
         for (int c = 128 * i; c < M16; c += 256) {
           const int n = min(256, M16 - c);
@@ -310,16 +300,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
       }
       s_r0_col = 0; s_r0_slots = ns; s_r1_col = 0; s_r1_slots = 0;
       s_cs_slots = ones ? 0 : s_r0_slots;
-    } else if (pr.full) {
-      const int np = (M16 + 255) / 256;
-      const int i = tile / np, t = tile - i * np;
-      const int pc0 = 256 * t;
-      const int pw = min(256, M16 - pc0);
-      s_r0_col = 128 * i; s_r0_slots = GR_ABL; s_r1_col = pc0; s_r1_slots = (pw + GR_CW - 1) / GR_CW;
-      ops[nops++] = GramOp{0, GR_ABL, pw, 0, 128 * i, pc0, pw, -1};
-      s_cs_slots = 0;
-      tcol = pw;
-      s_skip = (pr.full == 2 && pc0 + pw <= 128 * i) ? 1 : 0;
     } else {
       int i = 0, t = tile;
       for (;; ++i) {
@@ -367,7 +347,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
   }
   dep_sync();                                     // so far: parameters and this CTA's own shared memory only
   __syncthreads();
-  if (s_skip) return;                             // nothing allocated yet; every thread of the CTA leaves
   const int nslots = s_nslots, nops = s_nops;
   const bool ones = s_ones != 0;
   // no pass of the fix-up warps over the stages: nothing to centre and no column sums owed to them
@@ -448,7 +427,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
     // ---- TMA producer: one 32-column box per chunk ----
     if (elect_one()) {
       tma_prefetch_desc(&g.mapX[pi]);
-      if (pr.full) tma_prefetch_desc(&g.mapB[pi]);
       if (pr.use3d) { tma_prefetch_desc(&g.map3a[pi]); tma_prefetch_desc(&g.map3b[pi]); }
       int s = 0;
       uint32_t ph = 0, sb = smem_base;
@@ -470,8 +448,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
           int col = r0c;
           for (int c = 0; c < r0n; ++c, dst += CHUNK, col += GR_CW) tma_load_2d(dst, &g.mapX[pi], col, y, fb);
           col = r1c;
-          const CUtensorMap* m1 = pr.full ? &g.mapB[pi] : &g.mapX[pi];
-          for (int c = r0n; c < nslots; ++c, dst += CHUNK, col += GR_CW) tma_load_2d(dst, m1, col, y, fb);
+          for (int c = r0n; c < nslots; ++c, dst += CHUNK, col += GR_CW) tma_load_2d(dst, &g.mapX[pi], col, y, fb);
         }
         y += SR;
         sb += stage_bytes;
@@ -663,8 +640,7 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
       // A TMEM lane is a row of the tile, so stores straight from the registers put the 32 lanes of a warp on 32
       // different rows of the output: half-filled sectors, and an SM stores one sector per clock (7 us for a
       // 128 x 256 tile).  The tile goes through shared memory instead (the stages are free: every MMA has completed)
-      // and leaves as whole rows, 512 bytes per warp instruction (2 us).  The mirror image of a symmetric product
-      // leaves from the registers: there the lanes' rows are consecutive entries of one output row.
+      // and leaves as whole rows, 512 bytes per warp instruction (2 us).
       // The verdict of the waits is made common to the eight warps first: the barriers below are taken by all of
       // them or by none.
       asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -691,13 +667,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
                 *reinterpret_cast<float4*>(trow + c0 + j) =
                     make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]), __uint_as_float(rr[j + 2]),
                                 __uint_as_float(rr[j + 3]));
-              if (pr.full == 2 && row < M) {
-                // symmetric product: entry (row, c) with c > row also goes to (c, row)
-                const int col = col0 + c0;
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  if (col + j > row && col + j < M) P[(int64_t)(col + j) * M + row] = __uint_as_float(rr[j]);
-              }
             }
             if (ops[o].cs_off >= 0 && half == 0) {
               // ones mode: every one of the 16 extra columns holds the column sum of this lane's feature
@@ -715,7 +684,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
           asm volatile("bar.sync 1, 256;" ::: "memory");
           // rows of the tile, four at a time per warp: every load of a batch precedes its stores
           const int n4 = n_out >> 2;
-          const bool sym = pr.full == 2;
           if (pr.im2col) {
             // rows and columns as staged -> rows and columns of the patch matrix; padding columns are dropped (a group of
             // four staged columns is all real or all padding, and real ones stay adjacent)
@@ -766,15 +734,14 @@ __global__ void __launch_bounds__(GR_THREADS, 1) gram_umma_kernel(const __grid_c
               for (int k = 0; k < 3; ++k) {
                 const int c4 = lane + 32 * k;
                 const int col = col0 + 4 * c4;
-                // symmetric product: the entries on and above the diagonal only
-                if (c4 >= n4 || row >= M || col >= M || (sym && col + 3 < row)) continue;
-                if (col + 3 < M && (!sym || col >= row)) {
+                if (c4 >= n4 || row >= M || col >= M) continue;
+                if (col + 3 < M) {
                   *reinterpret_cast<float4*>(prow + col) = v[i][k];
                 } else {
                   const float ve[4] = {v[i][k].x, v[i][k].y, v[i][k].z, v[i][k].w};
 #pragma unroll
                   for (int e = 0; e < 4; ++e)
-                    if (col + e < M && (!sym || col + e >= row)) prow[col + e] = ve[e];
+                    if (col + e < M) prow[col + e] = ve[e];
                 }
               }
             }
@@ -1043,52 +1010,6 @@ __global__ void wait_probe_kernel(int32_t* status, uint32_t polls) {
 cudaError_t launch_wait_probe(int32_t* status, uint32_t polls, cudaStream_t s) {
   ProfScope ps(FW_PROF_MISC, s);
   return launch_plain(wait_probe_kernel, 1, 32, s, status, polls);
-}
-
-// D = A^T B for square fp32 matrices (TF32 inputs rounded to nearest, fp32 accumulation):
-// the re-sync products Phi_x T^T and T (Phi_x T^T) when T is kept transposed.
-fw_status umma_atb_launch(const UmmaAtbItem* items, int n, cudaStream_t s) {
-  const int smem = GR_SMEM_BUDGET + 1024;
-  if (!gram_smem_attr(smem)) return FW_ERR_CUDA;
-  for (int base = 0; base < n; base += kMaxUmmaGroup) {
-    GramGroup g;
-    memset(&g, 0, sizeof(g));
-    const int cnt = (n - base) < kMaxUmmaGroup ? (n - base) : kMaxUmmaGroup;
-    int total_ctas = 0;
-    for (int i = 0; i < cnt; ++i) {
-      const UmmaAtbItem& it = items[base + i];
-      GramProblem& p = g.p[i];
-      const int M16 = (it.M + 15) / 16 * 16;
-      p.shift = nullptr; p.gram_part = it.C; p.colsum_part = nullptr;
-      p.rows = it.M; p.M = it.M; p.bf16 = 0; p.stream = 0; p.full = it.sym ? 2 : 1; p.fixup = 1;
-      p.splits = 1; p.ntiles = ((M16 + 127) / 128) * ((M16 + 255) / 256); p.first_cta = total_ctas;
-      p.rows_per_split = (it.M + GR_SR - 1) / GR_SR * GR_SR;
-      p.sr = GR_SR;
-      p.status = it.status;
-      total_ctas += p.ntiles;
-      if (!encode_2d(&g.mapX[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, it.A, (uint64_t)it.M, (uint64_t)it.M,
-                     (uint64_t)it.M, GR_CW, GR_SR, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B) ||
-          !encode_2d(&g.mapB[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, it.B, (uint64_t)it.M, (uint64_t)it.M,
-                     (uint64_t)it.M, GR_CW, GR_SR, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B)) {
-        fprintf(stderr, "[fw] tensor-map encoding failed (A^T B)\n");
-        return FW_ERR_CUDA;
-      }
-      p.box_a = GR_ABL;
-      p.use3d = (it.M % GR_CW) == 0 &&
-                encode_chunked_3d(&g.map3a[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, it.A, (uint64_t)it.M, (uint64_t)it.M,
-                                  (uint64_t)it.M, GR_SR, GR_ABL, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B) &&
-                encode_chunked_3d(&g.map3b[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, it.B, (uint64_t)it.M, (uint64_t)it.M,
-                                  (uint64_t)it.M, GR_SR, 2 * GR_ABL, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B);
-    }
-    g.n = cnt;
-    ProfScope ps(FW_PROF_RESYNC, s);
-    const cudaError_t e = launch_dep(gram_umma_kernel<false>, total_ctas, GR_THREADS, smem, s, g);
-    if (e != cudaSuccess) {
-      fprintf(stderr, "[fw] gram_umma_kernel (A^T B) launch: %s\n", cudaGetErrorString(e));
-      return FW_ERR_CUDA;
-    }
-  }
-  return FW_OK;
 }
 
 }  // namespace fw

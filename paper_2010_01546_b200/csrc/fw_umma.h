@@ -71,7 +71,6 @@ bool tmap_encode_2d(CUtensorMap* m, bool bf16, const void* base, uint64_t inner,
                     uint32_t box_inner, uint32_t box_outer);
 bool tmap_encode_chunked_3d(CUtensorMap* m, bool bf16, const void* base, uint64_t cols, uint64_t rows, uint64_t ld,
                             uint32_t box_rows, uint32_t box_chunks, uint32_t chunk_cols);
-
 // ---- the same two products on CTA pairs (cta_group::2), for matrices too large for one CTA's TMEM ----
 // 256 x 512 output tiles per pair of SMs: each CTA stages its own 128 rows of A and its half of B.
 bool umma_pair_gram_eligible(const UmmaGramItem& it);
@@ -80,10 +79,14 @@ int umma_pair_split_cap(int M);
 fw_status umma_pair_gram_launch(UmmaGramItem* items, int n, cudaStream_t s);
 
 // ---- D = A^T B, square fp32 matrices (re-sync products) ----
+// The tensor core truncates fp32 operands to TF32, so they are rounded to nearest before that: in shared memory, or by whoever
+// wrote them.
 struct UmmaAtbItem {
   const float* A;   // M x M row-major
   const float* B;   // M x M row-major
-  float* C;         // M x M row-major
+  float* C;         // M x M row-major; the values rounded to TF32 if round_c
+  int32_t round_c;
+  int32_t fix;      // operands to be rounded in shared memory: 1 A, 2 B, 3 both, 0 none (they are on the TF32 grid)
   int32_t M;
   int32_t sym;      // the product is symmetric: only its upper triangle is taken from the accumulators and mirrored
   int32_t* status;  // the layer's time-out word

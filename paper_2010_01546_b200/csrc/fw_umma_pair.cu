@@ -27,12 +27,15 @@
 // fp32 (n is known to the host).
 //
 // Roles per CTA: warp 0 TMA producer, warp 1 MMA issuer (even CTA only) and TMEM
-// owner, warps 2..9 fix-up/column sums and epilogue.  Two stage protocols:
+// owner, warps 2..9 rounding, column sums and epilogue.  Two stage protocols:
 //   direct  both CTAs' loads complete on the even CTA's "full" barrier (armed with
 //           the bytes of both); the MMA thread waits on it.
-//   pass    (diagonal tiles: column sums; re-sync: rounding to TF32) each CTA's
-//           loads complete on its own barrier, its 8 warps pass over the stage and
-//           then arrive on the even CTA's "ready" barrier (16 arrivals).
+//   pass    (diagonal tiles: column sums; operands of a re-sync product that are
+//           still to be rounded to TF32) each CTA's loads complete on its own
+//           barrier, its 8 warps pass over the stage and then arrive on the even
+//           CTA's "ready" barrier (16 arrivals).  Rounding costs 32 KB of shared
+//           memory traffic per 16 KB: with both operands a stage takes 1.6 times
+//           as long, so what can be rounded where it is written is.
 // tcgen05.commit multicasts the "stage free" and "accumulator complete" arrivals
 // to both CTAs.  Every wait is bounded; a time-out raises the abort flag of both
 // CTAs, is recorded in the owning layer's status word, and all threads still meet
@@ -68,6 +71,7 @@ constexpr int GP_CONST = 12 * 1024;        // constant operand chunks of the mea
                                            // one MMA's rows (16 bf16 / 8 fp32) x 128 columns
 constexpr int GP_MAX_PROBLEMS = 16;
 constexpr int GP_MAX_ITEMS = 2048;
+constexpr int kMinPanel = 256;             // narrowest tile of a product
 constexpr int GP_CLUSTER_SLOTS = 74;       // CTA pairs resident at once if every TPC takes one (148 SMs, one CTA per SM)
 
 struct PairProblem {
@@ -77,10 +81,11 @@ struct PairProblem {
   int32_t M;
   int32_t full;          // 1: D = A^T B from two sources, every tile; 0: symmetric Gram of one source;
                          // 2: A^T B with a symmetric result: tiles below the diagonal skipped, entries mirrored
-  int32_t fixup;         // 1 (fp32 only): round every staged value to TF32 (nearest) before the product
   int32_t rows_per_split;  // multiple of the stage's rows
   int32_t use3d;         // chunked 3-D tensor maps usable (M a multiple of 64)
-  int32_t pad;
+  int32_t fix;           // products: operands rounded to TF32 (nearest) in shared memory: 1 A, 2 B
+  int32_t round_out;     // products: the result is rounded to TF32
+  int32_t panel;         // columns of a tile: 512, or fewer (a multiple of 64) where narrower tiles fill the chip better
   int32_t* status;       // time-out word of the owning layer
   const float* pmean;    // pilot mean for the mean-product correction (Gram problems), or null
 };
@@ -99,7 +104,7 @@ __host__ __device__ inline int pair_tiles_sym(int M16) {
   for (int c = 0; c < M16; c += 256) t += (M16 - c + 511) / 512;
   return t;
 }
-__host__ __device__ inline int pair_tiles_full(int M16) { return ((M16 + 255) / 256) * ((M16 + 511) / 512); }
+__host__ __device__ inline int pair_tiles_full(int M16, int panel) { return ((M16 + 255) / 256) * ((M16 + panel - 1) / panel); }
 
 __device__ __forceinline__ float4 lds128(uint32_t a) {
   float4 v;
@@ -109,8 +114,11 @@ __device__ __forceinline__ float4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-__device__ __forceinline__ float tf32_rna(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+// the first n of four neighbouring entries
+__device__ __forceinline__ void store4(float* p, const float (&v)[4], int n) {
+  if (n >= 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else
+    for (int e = 0; e < n; ++e) p[e] = v[e];
 }
 
 template <bool BF>
@@ -139,7 +147,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_flag;
   __shared__ int s_I, s_cbase, s_n0, s_n1, s_ngroups, s_bgroup, s_pass, s_cs, s_tmem_cols, s_skip;
-  __shared__ int s_gcol[GP_MAX_GROUPS], s_gsrc[GP_MAX_GROUPS];
+  __shared__ int s_gcol[GP_MAX_GROUPS], s_gsrc[GP_MAX_GROUPS], s_gchunks[GP_MAX_GROUPS];
   __shared__ float s_csred[GP_FIX_WARPS][GP_GCOLS];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -154,7 +162,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
     abort_flag = 0;
     int I = 0, t = tile;
     if (pr.full) {
-      const int np = (M16 + 511) / 512;
+      const int np = (M16 + pr.panel - 1) / pr.panel;
       I = tile / np; t = tile - I * np;
     } else {
       for (;; ++I) {
@@ -163,20 +171,22 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
         t -= np;
       }
     }
-    const int cbase = (pr.full ? 0 : 256 * I) + 512 * t;
-    const int n0 = min(256, M16 - cbase);
-    const int n1 = max(0, min(256, M16 - cbase - 256));
+    const int cbase = (pr.full ? 0 : 256 * I) + pr.panel * t;
+    const int pw = min(pr.panel, M16 - cbase);
+    const int n0 = min(256, pw);
+    const int n1 = pw - n0;
     const bool diag = !pr.full && t == 0;
     const bool shared_b0 = diag && n0 == 256;      // first panel == the A block: staged once
     int ng = 0;
-    s_gcol[ng] = 256 * I + 128 * (int)rank; s_gsrc[ng] = 0; ++ng;
+    // columns this CTA stages of each group, in whole chunks
+    s_gcol[ng] = 256 * I + 128 * (int)rank; s_gsrc[ng] = 0; s_gchunks[ng] = GC; ++ng;
     s_bgroup = shared_b0 ? 0 : ng;
-    if (!shared_b0) { s_gcol[ng] = cbase + (int)rank * (n0 / 2); s_gsrc[ng] = pr.full ? 1 : 0; ++ng; }
-    if (n1 > 0) { s_gcol[ng] = cbase + 256 + (int)rank * (n1 / 2); s_gsrc[ng] = pr.full ? 1 : 0; ++ng; }
+    if (!shared_b0) { s_gcol[ng] = cbase + (int)rank * (n0 / 2); s_gsrc[ng] = pr.full ? 1 : 0; s_gchunks[ng] = (n0 / 2 + CW - 1) / CW; ++ng; }
+    if (n1 > 0) { s_gcol[ng] = cbase + 256 + (int)rank * (n1 / 2); s_gsrc[ng] = pr.full ? 1 : 0; s_gchunks[ng] = (n1 / 2 + CW - 1) / CW; ++ng; }
     s_I = I; s_cbase = cbase; s_n0 = n0; s_n1 = n1; s_ngroups = ng;
     s_skip = (pr.full == 2 && cbase + n0 + n1 <= 256 * I) ? 1 : 0;
     s_cs = (diag && pr.colsum_part != nullptr) ? 1 : 0;
-    s_pass = (s_cs || pr.fixup) ? 1 : 0;
+    s_pass = (s_cs || pr.fix) ? 1 : 0;
     int nc = 32;
     while (nc < n0 + n1) nc <<= 1;
     s_tmem_cols = nc;
@@ -276,13 +286,16 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
       const bool mine = q < ngroups;
       const int gcol = mine ? s_gcol[q] : 0;
       const int gsrc = mine ? s_gsrc[q] : 0;
-      const bool box3 = pr.use3d && (gcol % CW) == 0;            // this group comes with one instruction
-      const bool issue = mine && (!box3 || c == 0);
+      const int chunks = mine ? s_gchunks[q] : 0;
+      const bool box3 = pr.use3d && (gcol % CW) == 0 && chunks == GC;            // this group comes with one instruction
+      const bool issue = mine && (box3 ? c == 0 : c < chunks);
       const CUtensorMap* map = box3 ? m3[gsrc] : m2[gsrc];
       const int x = box3 ? 0 : gcol + c * CW;
       const int z = gcol / CW;
       const uint32_t doff = (uint32_t)q * GROUP_BYTES + (box3 ? 0u : (uint32_t)c * CHUNK);
-      const uint32_t tx_bytes = stage_bytes;
+      int landed = 0;
+      for (int k = 0; k < ngroups; ++k) landed += s_gchunks[k];
+      const uint32_t tx_bytes = (uint32_t)landed * CHUNK;
       int s = 0;
       uint32_t ph = 0, sb = smem_base;
       int y = (int)r_begin;
@@ -359,7 +372,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
       mma_commit_pair(smem_u32(&bar_accum), (uint16_t)3);
     }
   } else {
-    // ---- fix-up / column sums over the stages (pass protocol only), then the epilogue ----
+    // ---- rounding / column sums over the stages (pass protocol only), then the epilogue ----
     const int w = warp - 2;
     // A warp pass covers 4 rows x 128 bytes of a chunk: lane -> (row lane >> 3, 16-byte unit lane & 7); warp w owns
     // rows 4w..4w+3 of every chunk of the stage.  The unit's position in its row is swizzled as the TMA wrote it.
@@ -374,26 +387,21 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
     bool ok = true;
     if (pass) {
       const uint32_t lead_ready0 = mapa_shared(smem_u32(&bar_ready[0]), 0u);
-      const bool fix = !BF && pr.fixup != 0;
-      const int nchunks = ngroups * GC;
+      const int fix = BF ? 0 : pr.fix;
       int s = 0;
       uint32_t ph = 0, sa = smem_base + off;
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(smem_u32(&bar_full[s]), ph, abortp)) { GP_ABORT(303); ok = false; break; }
         if (fix) {
-          // every staged value rounded to the TF32 grid (nearest) in place: the tensor core would truncate
 #pragma unroll
           for (int h = 0; h < GP_MAX_GROUPS; ++h) {
-            if (h * GC < nchunks) {
+            if (h < ngroups && (fix & (h ? 2 : 1))) {
               float4 v[GC];
 #pragma unroll
               for (int jj = 0; jj < GC; ++jj) v[jj] = lds128(sa + (h * GC + jj) * CHUNK);
 #pragma unroll
-              for (int jj = 0; jj < GC; ++jj) {
-                float4 x = v[jj];
-                x.x = tf32_rna(x.x); x.y = tf32_rna(x.y); x.z = tf32_rna(x.z); x.w = tf32_rna(x.w);
-                sts128(sa + (h * GC + jj) * CHUNK, x);
-              }
+              for (int jj = 0; jj < GC; ++jj)
+                sts128(sa + (h * GC + jj) * CHUNK, make_float4(tf32_rna(v[jj].x), tf32_rna(v[jj].y), tf32_rna(v[jj].z), tf32_rna(v[jj].w)));
             }
           }
           fence_proxy_async_smem();
@@ -495,14 +503,10 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
             } else if (row < M) {
 #pragma unroll
               for (int j = 0; j < 16; j += 4) {
-                if (col + j + 3 < M) {
-                  *reinterpret_cast<float4*>(P + (int64_t)row * M + col + j) =
-                      make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]), __uint_as_float(rr[j + 2]),
-                                  __uint_as_float(rr[j + 3]));
-                } else {
-                  for (int jj = j; jj < j + 4; ++jj)
-                    if (col + jj < M) P[(int64_t)row * M + col + jj] = __uint_as_float(rr[jj]);
-                }
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = pr.round_out ? tf32_rna(__uint_as_float(rr[j + e])) : __uint_as_float(rr[j + e]);
+                store4(P + (int64_t)row * M + col + j, v, M - col - j);
               }
             }
           }
@@ -526,20 +530,22 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
 // ---------------------------------------------------------------------------
 // host: work list
 // ---------------------------------------------------------------------------
-struct PairTile { int n0, n1, ngroups; bool pass; bool skip; };   // skip: wholly below the diagonal of a symmetric product
+struct PairTile { int n0, n1, cols; bool skip; };   // cols: columns a CTA stages   // skip: wholly below the diagonal of a symmetric product
 
-void pair_tiles(int M, bool full, bool colsums, bool fixup, bool sym_out, std::vector<PairTile>& out) {
+void pair_tiles(int M, bool full, int panel, bool sym_out, std::vector<PairTile>& out) {
   const int M16 = (M + 15) / 16 * 16;
   out.clear();
   for (int I = 0; 256 * I < M16; ++I) {
     const int c_first = full ? 0 : 256 * I;
-    for (int c = c_first, t = 0; c < M16; c += 512, ++t) {
+    for (int c = c_first, t = 0; c < M16; c += panel, ++t) {
       PairTile pt;
-      pt.n0 = std::min(256, M16 - c);
-      pt.n1 = std::max(0, std::min(256, M16 - c - 256));
+      const int pw = std::min(panel, M16 - c);
+      pt.n0 = std::min(256, pw);
+      pt.n1 = pw - pt.n0;
       const bool diag = !full && t == 0;
-      pt.ngroups = 1 + ((diag && pt.n0 == 256) ? 0 : 1) + (pt.n1 > 0 ? 1 : 0);
-      pt.pass = fixup || (diag && colsums);
+      // (a Gram tile counts whole groups: the row slabs chosen by this estimate fix how the sums are rounded)
+      if (full) pt.cols = GP_GCOLS + pt.n0 / 2 + pt.n1 / 2;
+      else pt.cols = GP_GCOLS * (1 + ((diag && pt.n0 == 256) ? 0 : 1) + (pt.n1 > 0 ? 1 : 0));
       pt.skip = full && sym_out && c + pt.n0 + pt.n1 <= 256 * I;
       out.push_back(pt);
     }
@@ -549,20 +555,54 @@ void pair_tiles(int M, bool full, bool colsums, bool fixup, bool sym_out, std::v
 // Estimated time of one tile over `rows` rows, microseconds: tensor time against staging time.  Staging rates
 // are what a CTA sustains with every SM busy (measured: about 40 bytes per clock for bf16 tiles and 48 for fp32
 // tiles, which then run at the TF32 tensor rate).
-double pair_tile_us(const PairTile& t, bool bf16, bool fixup, double rows) {
+double pair_tile_us(const PairTile& t, bool bf16, int fix, double rows) {
   const double clk_us = 1800.0;                                   // SM clocks per microsecond under load
   const double tensor = (t.n0 + t.n1) / 512.0 * (bf16 ? 16.0 : 32.0);
-  double load = t.ngroups * 128.0 * (bf16 ? 2.0 / 40.0 : 4.0 / 48.0);
-  if (fixup) load *= 1.6;
+  const double load = t.cols * (bf16 ? 2.0 / 40.0 : 4.0 / 48.0) * (1.0 + 0.2 * (fix & 1) + 0.4 * (fix >> 1));
   const double fixed = 4.0 + 128.0 * (t.n0 + t.n1) * 4.0 / 80e3;  // prologue, pipeline fill, epilogue stores
   return fixed + rows * std::max(tensor, load) / clk_us;
 }
 
 struct PairSpec {
-  int M; int64_t rows; bool bf16, full, fixup, colsums, sym_out = false; int split_cap;
+  int M; int64_t rows; bool bf16, full, colsums, sym_out = false; int split_cap; int panel = 512, fix = 0, round_out = 0;
   std::vector<PairTile> tiles;
   int splits; int64_t per;     // chosen: splits, stages per split
 };
+
+// When the longest-first list schedule of the items over the resident CTA pairs ends.
+double pair_makespan(std::vector<double>& items, int slots) {
+  std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
+  std::vector<double> slot(slots, 0.0);
+  for (double c : items) *std::min_element(slot.begin(), slot.end()) += c;
+  return *std::max_element(slot.begin(), slot.end());
+}
+
+// Columns of the products' tiles: 512 moves the fewest bytes per output, but one layer of M = 2304 is 45 such tiles on 74
+// pairs of SMs, or 72 of 320 columns that take three quarters of the time.  The last set a thread launched is remembered.
+int pair_choose_panel(const std::vector<PairSpec>& P, int slots) {
+  thread_local std::vector<int> last;
+  thread_local int last_panel = 512;
+  std::vector<int> key(1, slots);
+  for (const PairSpec& p : P) { key.push_back(p.M); key.push_back(p.sym_out * 4 + p.fix); }
+  if (key == last) return last_panel;
+  int panel = 512;
+  double best = 0;
+  std::vector<PairTile> tiles;
+  std::vector<double> items;
+  for (int w = 512; w >= kMinPanel; w -= 64) {
+    items.clear();
+    for (const PairSpec& p : P) {
+      pair_tiles(p.M, true, w, p.sym_out, tiles);
+      for (const PairTile& t : tiles)
+        if (!t.skip) items.push_back(pair_tile_us(t, false, p.fix, (double)p.M));
+    }
+    if (items.size() > (size_t)GP_MAX_ITEMS) break;
+    const double end = pair_makespan(items, slots);
+    if (w == 512 || end < best) { best = end; panel = w; }
+  }
+  last = key; last_panel = panel;
+  return panel;
+}
 
 // Chooses the split count of every problem so that the longest-first list schedule of all (tile, split) items
 // over the resident CTA pairs ends earliest, counting what each further split costs the reduction that follows.
@@ -575,8 +615,8 @@ void pair_choose_splits(std::vector<PairSpec>& P, int slots) {
   std::vector<int64_t> key;
   key.push_back(slots);
   for (const PairSpec& p : P) {
-    key.push_back(p.M); key.push_back(p.rows); key.push_back(p.split_cap);
-    key.push_back((p.bf16 ? 1 : 0) | (p.full ? 2 : 0) | (p.fixup ? 4 : 0) | (p.sym_out ? 8 : 0) | (p.colsums ? 16 : 0));
+    key.push_back(p.M); key.push_back(p.rows); key.push_back(p.split_cap); key.push_back(p.panel);
+    key.push_back((p.bf16 ? 1 : 0) | (p.full ? 2 : 0) | (p.fix << 5) | (p.sym_out ? 8 : 0) | (p.colsums ? 16 : 0));
   }
   auto hit = memo.find(key);
   if (hit != memo.end()) { best_s = hit->second.first; best = hit->second.second; }
@@ -590,7 +630,7 @@ void pair_choose_splits(std::vector<PairSpec>& P, int slots) {
       PairSpec& p = P[l];
       double longest = 0;
       for (const PairTile& t : p.tiles)
-        if (!t.skip) longest = std::max(longest, pair_tile_us(t, p.bf16, p.fixup, (double)p.rows));
+        if (!t.skip) longest = std::max(longest, pair_tile_us(t, p.bf16, p.fix, (double)p.rows));
       const int SRh = pair_sr(p.bf16);
       const int64_t nsr = (p.rows + SRh - 1) / SRh;
       int64_t s = (int64_t)(longest / tau + 0.5);
@@ -602,7 +642,7 @@ void pair_choose_splits(std::vector<PairSpec>& P, int slots) {
         if (t.skip) continue;
         for (int64_t k = 0; k < s; ++k) {
           const double r = (double)std::min<int64_t>(per * SRh, p.rows - k * per * SRh);
-          items.push_back(pair_tile_us(t, p.bf16, p.fixup, r));
+          items.push_back(pair_tile_us(t, p.bf16, p.fix, r));
         }
         count += (size_t)s;
       }
@@ -610,13 +650,7 @@ void pair_choose_splits(std::vector<PairSpec>& P, int slots) {
       if (!p.full) extra += (double)(s - 1) * 0.55 * 4.0 * p.M * (double)p.M / 4e6;
     }
     if (count > (size_t)GP_MAX_ITEMS) continue;
-    std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
-    std::vector<double> slot(slots, 0.0);
-    for (double c : items) {
-      auto m = std::min_element(slot.begin(), slot.end());
-      *m += c;
-    }
-    const double span = *std::max_element(slot.begin(), slot.end()) + extra;
+    const double span = pair_makespan(items, slots) + extra;
     if (span < best) { best = span; best_s = sp; }
   }
   if (hit == memo.end()) {
@@ -669,6 +703,13 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
     int cnt = 0;
     while (base + cnt < n && cnt < GP_MAX_PROBLEMS && specs[base + cnt].bf16 == specs[base].bf16) ++cnt;
     std::vector<PairSpec> grp(specs.begin() + base, specs.begin() + base + cnt);
+    if (grp[0].full) {
+      const int panel = pair_choose_panel(grp, slots);
+      for (PairSpec& p : grp) {
+        p.panel = panel;
+        pair_tiles(p.M, true, panel, p.sym_out, p.tiles);
+      }
+    }
     pair_choose_splits(grp, slots);
     std::vector<PairGroup> gbuf(1);           // 17 KB: kept off the stack; the launch copies it
     PairGroup& g = gbuf[0];
@@ -680,24 +721,29 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
       const PairSource& so = src[base + i];
       PairProblem& p = g.p[i];
       p.out = so.out; p.colsum_part = so.colsum; p.rows = sp.rows; p.M = sp.M;
-      p.status = so.status; p.pmean = so.pmean; p.full = sp.full ? (sp.sym_out ? 2 : 1) : 0; p.fixup = sp.fixup; p.rows_per_split = (int)(sp.per * pair_sr(sp.bf16));
+      p.status = so.status; p.pmean = so.pmean; p.full = sp.full ? (sp.sym_out ? 2 : 1) : 0; p.panel = sp.panel; p.fix = sp.fix; p.round_out = sp.round_out; p.rows_per_split = (int)(sp.per * pair_sr(sp.bf16));
       const bool bf = sp.bf16;
       const uint32_t cw = bf ? 64 : 32;       // chunk rows of 128 bytes
-      if (!tmap_encode_2d(&g.mapA[i], bf, so.A, (uint64_t)sp.M, (uint64_t)sp.rows, (uint64_t)so.lda, cw, (uint32_t)pair_sr(bf)) ||
-          !tmap_encode_2d(&g.mapB[i], bf, so.B, (uint64_t)sp.M, (uint64_t)sp.rows, (uint64_t)so.ldb, cw, (uint32_t)pair_sr(bf))) {
+      // one-chunk boxes, and chunked views where M allows
+      auto encode = [&](CUtensorMap* m2, CUtensorMap* m3, const void* base, int64_t ld, bool& chunked) {
+        const uint64_t M = (uint64_t)sp.M, rows = (uint64_t)sp.rows;
+        const uint32_t sr = (uint32_t)pair_sr(bf), gc = GP_GCOLS / cw;
+        chunked = chunked && tmap_encode_chunked_3d(m3, bf, base, M, rows, (uint64_t)ld, sr, gc, cw);
+        return tmap_encode_2d(m2, bf, base, M, rows, (uint64_t)ld, cw, sr);
+      };
+      bool chunked = sp.M % 64 == 0;
+      if (!encode(&g.mapA[i], &g.map3A[i], so.A, so.lda, chunked) || !encode(&g.mapB[i], &g.map3B[i], so.B, so.ldb, chunked)) {
         fprintf(stderr, "[fw] tensor-map encoding failed (pair kernel)\n");
         return FW_ERR_CUDA;
       }
-      p.use3d = (sp.M % 64) == 0 &&
-                tmap_encode_chunked_3d(&g.map3A[i], bf, so.A, (uint64_t)sp.M, (uint64_t)sp.rows, (uint64_t)so.lda, (uint32_t)pair_sr(bf), GP_GCOLS / cw, cw) &&
-                tmap_encode_chunked_3d(&g.map3B[i], bf, so.B, (uint64_t)sp.M, (uint64_t)sp.rows, (uint64_t)so.ldb, (uint32_t)pair_sr(bf), GP_GCOLS / cw, cw);
+      p.use3d = chunked;
       for (size_t t = 0; t < sp.tiles.size(); ++t) {
         if (sp.tiles[t].skip) continue;             // never launched: the mirrored entries of other tiles fill it
         for (int k = 0; k < sp.splits; ++k) {
           const double r = (double)std::min<int64_t>(sp.per * pair_sr(sp.bf16), sp.rows - (int64_t)k * sp.per * pair_sr(sp.bf16));
           Item itm;
           itm.code = ((uint32_t)i << 28) | ((uint32_t)t << 14) | (uint32_t)k;
-          itm.cost = pair_tile_us(sp.tiles[t], sp.bf16, sp.fixup, r);
+          itm.cost = pair_tile_us(sp.tiles[t], sp.bf16, sp.fix, r);
           itm.pos = (double)k / sp.splits;
           items.push_back(itm);
         }
@@ -744,7 +790,7 @@ bool umma_pair_gram_eligible(const UmmaGramItem& it) {
 
 bool umma_pair_atb_eligible(int M) {
   const int M16 = (M + 15) / 16 * 16;
-  return M16 >= std::max(pair_min_m(), 1024) && pair_tiles_full(M16) <= GP_MAX_ITEMS;
+  return M16 >= std::max(pair_min_m(), 1024) && pair_tiles_full(M16, kMinPanel) <= GP_MAX_ITEMS;
 }
 
 // Partial buffers a layer of dimension M should have for the pair kernel to balance its launch:
@@ -769,9 +815,9 @@ fw_status umma_pair_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
   for (int i = 0; i < n; ++i) {
     const UmmaGramItem& it = items[i];
     PairSpec& p = specs[i];
-    p.M = it.M; p.rows = it.rows; p.bf16 = it.x_bf16 != 0; p.full = false; p.fixup = false; p.colsums = true;
+    p.M = it.M; p.rows = it.rows; p.bf16 = it.x_bf16 != 0; p.full = false; p.colsums = true;
     p.split_cap = std::max(1, std::min(it.split_cap, 0x3fff));
-    pair_tiles(p.M, false, true, false, false, p.tiles);
+    pair_tiles(p.M, false, p.panel, false, p.tiles);
     src[i] = PairSource{it.X, it.X, it.ldx, it.ldx, it.gram_part, it.colsum_part, it.status, it.pmean};
   }
   fw_status st = pair_launch(specs, src, FW_PROF_GRAM, s);
@@ -794,7 +840,7 @@ fw_status umma_pair_gram_launch(UmmaGramItem* items, int n, cudaStream_t s) {
   return FW_OK;
 }
 
-// D = A^T B, square fp32 matrices, operands rounded to TF32 (nearest) in shared memory
+// D = A^T B, square fp32 matrices, operands on the TF32 grid or rounded to it in shared memory
 fw_status umma_pair_atb_launch(const UmmaAtbItem* items, int n, cudaStream_t s) {
   if (n <= 0) return FW_OK;
   std::vector<PairSpec> specs(n);
@@ -802,9 +848,8 @@ fw_status umma_pair_atb_launch(const UmmaAtbItem* items, int n, cudaStream_t s) 
   for (int i = 0; i < n; ++i) {
     const UmmaAtbItem& it = items[i];
     PairSpec& p = specs[i];
-    p.M = it.M; p.rows = it.M; p.bf16 = false; p.full = true; p.fixup = true; p.colsums = false; p.sym_out = it.sym != 0;
+    p.M = it.M; p.rows = it.M; p.bf16 = false; p.full = true; p.colsums = false; p.sym_out = it.sym != 0; p.fix = it.fix; p.round_out = it.round_c;
     p.split_cap = 1;
-    pair_tiles(p.M, true, false, true, it.sym != 0, p.tiles);
     src[i] = PairSource{it.A, it.B, it.M, it.M, it.C, nullptr, it.status, nullptr};
   }
   return pair_launch(specs, src, FW_PROF_RESYNC, s);
