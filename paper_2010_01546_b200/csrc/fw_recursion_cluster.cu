@@ -1,6 +1,6 @@
 // On-chip recursion for small layers (Sec. 4): a layer's whitened covariance Phi_y
-// stays on chip for all steps of a launch, each warp's rows in its registers, with
-// a copy in shared memory for the row m' a step sends round.  The launch uses
+// stays on chip for all steps of a launch, each warp's rows in its registers (row m'
+// of a step is sent round as column m', four entries a warp).  The launch uses
 // thread-block clusters; a layer takes n = 1 ... 16 consecutive CTAs of one
 // cluster (at least as many as its rows need; more while the clusters of one wave
 // allow and the layer is the launch's slowest).  CTA `sub` of a layer owns a slab
@@ -48,7 +48,7 @@ constexpr int CW = CT / 32;        // warps per CTA
 constexpr int kMaxIt = 5;          // float4 columns per lane, at most
 constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take teams of CTAs and fp64 sums
 constexpr int KH = 8;              // steps between two updates of T and Q
-constexpr size_t kSmemLimit = 226 * 1024 - 512;   // plus the static variables below: within the 227 KB of a CTA
+constexpr size_t kSmemLimit = 64 * 1024;   // the vectors of the longest row: 22 of 16 slabs of at most 43 entries
 
 // A warp owns one group of four rows (up to kMaxIt float4 columns per lane: 80 registers) or, for rows of at most 256
 // entries, two (64 registers).
@@ -76,23 +76,20 @@ __device__ __forceinline__ void st_async_v4(uint32_t raddr, float4 v, uint32_t r
                ::"r"(raddr), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
                  "r"(__float_as_uint(v.w)), "r"(rbar) : "memory");
 }
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const float* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(g) : "memory");
-}
 
-// dynamic shared memory: [phi slab R x Mp][xi2][cvec][wvec][two power-iteration vectors][uvec][vh: KH][th: KH], vectors
+// dynamic shared memory: [xi2][cvec][wvec][two power-iteration vectors][uvec][vh: KH][th: KH], vectors
 // of Mv floats: what n slices of R results fill, and at least whole trips of a warp over the columns
 extern __shared__ __align__(16) float csm[];
 
 // What a CTA knows about its layer; lives in shared memory (the threads' registers hold matrix rows).
 struct Slab {
   // offsets into the dynamic shared memory (not pointers: the compiler then knows which memory they point to)
-  int xi2, cvec, wvec, buf0, uvec;   // vectors of Mv floats; buf0: two, Mv apart.  My rows of Phi_y are at 0, Mp apart
+  int xi2, cvec, wvec, buf0, uvec;   // vectors of Mv floats; buf0: two, Mv apart
   int vh, th;     // v_e and t of the recorded steps, KH vectors each
   int M, Mp;      // matrix size, padded row length
   int Mv;         // vector length in shared memory
   int R;          // rows per CTA, a multiple of four (rows past the matrix are zero rows)
-  int row0, nrows;  // my first row; how many of my rows are rows of the matrix
+  int row0;       // my first row
   int n;          // CTAs of this layer
   int sub;        // my index among them
   uint32_t tx;    // bytes of one exchanged vector
@@ -156,10 +153,11 @@ __device__ __forceinline__ void send4(const Link& l, float* tgt, float4 v, uint3
   }
 }
 
-// One pass: y = scale * (my rows) x, sent to `dst` (the slot of the warp's first
-// group in the result vector) of every CTA of the layer.  NORM: scale = 1 / ||x||, summed from
-// the values of x the pass loads anyway; returns ||x||^2.  UNIT: the rows times x / ||x||, the norm summed first.  SELF:
-// squared norms of the rows themselves.
+// One pass: y = (my rows) x, sent to `dst` (the slot of the warp's first group in the result vector) of every CTA of the
+// layer.  SCALE: y times `scale`.  NORM and UNIT take x as it was sent times `scale`.  NORM returns ||scale x||^2, summed after y
+// has gone: a power iteration's y = Phi_y x / ||x|| is sent without the 1 / ||x||, which every receiver knows and applies to the
+// entries it loads, so that the norm's reduction and root run while the exchange does (M = 576: XXX).  UNIT: the
+// rows times scale x / ||scale x||, the norm summed first.  SELF: squared norms of the rows themselves.
 enum { PASS_SELF, PASS_SCALE, PASS_NORM, PASS_UNIT };
 template <int MODE, int NG, int IT>
 __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float* x, float scale, const Link& l,
@@ -173,7 +171,8 @@ __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float
   if (MODE == PASS_UNIT) {
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
-      const float4 b = x4[lane + 32 * k];
+      float4 b = x4[lane + 32 * k];
+      b.x *= scale; b.y *= scale; b.z *= scale; b.w *= scale;
       n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
       n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
     }
@@ -184,6 +183,7 @@ __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float
   for (int k = 0; k < IT; ++k) {
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
     if (MODE != PASS_SELF) b = x4[lane + 32 * k];
+    if (MODE == PASS_NORM || MODE == PASS_UNIT) { b.x *= scale; b.y *= scale; b.z *= scale; b.w *= scale; }
     if (MODE == PASS_UNIT) { b.x *= inv; b.y *= inv; b.z *= inv; b.w *= inv; }
     if (MODE == PASS_NORM) {
       n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
@@ -197,14 +197,14 @@ __device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float
       acc[q][0] = fmaf(v.z, bb.z, acc[q][0]); acc[q][1] = fmaf(v.w, bb.w, acc[q][1]);
     }
   }
-  if (MODE == PASS_NORM) { n2 = warp_sum(n0 + n1); scale = inv_norm(n2); }
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     float4 v = warp_sum4(acc[4 * g][0] + acc[4 * g][1], acc[4 * g + 1][0] + acc[4 * g + 1][1],
                          acc[4 * g + 2][0] + acc[4 * g + 2][1], acc[4 * g + 3][0] + acc[4 * g + 3][1]);
-    v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale;
+    if (MODE == PASS_SCALE) { v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale; }
     send4(l, dst + 4 * CW * g, v, e);
   }
+  if (MODE == PASS_NORM) n2 = warp_sum(n0 + n1);
   return n2;
 }
 
@@ -228,24 +228,27 @@ __device__ __forceinline__ int argmax_xi(const Slab& s) {
   return top == 0 || bi >= (uint32_t)s.M ? 0 : (int)bi;
 }
 
-// Row m' of Phi_y into wvec of every CTA of the layer: the CTA that owns it sends it (exchange e).  A CTA that holds all
-// rows reads the row where it is.
-__device__ __forceinline__ const float* row_exchange(Slab& s, const Link& l, int mp, uint32_t e) {
-  const int owner = mp / s.R;
-  const float* row = csm + (mp - owner * s.R) * s.Mp;
-  if (l.n == 1) return row;
-  arm(l, e, (uint32_t)s.Mp * 4u);
-  if (owner == s.sub) {
-    const uint32_t bar = l.bar0 + ((e & 1) << 3);
-    const int lane = threadIdx.x & 31;
-    for (int c = threadIdx.x >> 5; c < (s.Mp >> 2); c += l.active >> 5) {
-      // a lane per peer: the lanes' copies of one float4 go out together
-      const float4 v = reinterpret_cast<const float4*>(row)[c];
-      if (lane < l.n) st_async_v4(smem_u32(csm + s.wvec + 4 * c) + l.rdelta, v, bar + l.rdelta);
+// Row m' of Phi_y into wvec of every CTA of the layer (exchange e).  Phi_y is exactly symmetric, so every warp sends the entries of
+// its rows in column m': a message of four entries a warp like any other exchange, where the owner of row m' sending it to
+// all alone took 4900 clocks (M = 576 on 12 CTAs: 1728 messages of one SM).
+template <int NG, int IT>
+__device__ __forceinline__ void send_column(const float4 (&a)[4 * NG][IT], int mp, const Link& l, float* dst, uint32_t e) {
+  const int k0 = mp >> 7, from = (mp >> 2) & 31, c = mp & 3;
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    float y[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float x = 0.f;
+#pragma unroll
+      for (int k = 0; k < IT; ++k) {
+        const float4 v = a[4 * g + q][k];
+        if (k == k0) x = c < 2 ? (c == 0 ? v.x : v.y) : (c == 2 ? v.z : v.w);
+      }
+      y[q] = __shfl_sync(0xffffffffu, x, from);
     }
+    send4(l, dst + 4 * CW * g, make_float4(y[0], y[1], y[2], y[3]), e);
   }
-  wait_exchange(l, e, &s.fail);
-  return csm + s.wvec;
 }
 
 // Weights of the coherent set into wvec (Eqs. 48-49); returns the size of the set
@@ -443,7 +446,8 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
   }
 }
 
-// Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane.
+// Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane; from Phi_y in global
+// memory and back.
 template <int NG, int IT>
 __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L, float* tr, int k0, int k1, int P,
                                        bool last, uint32_t e) {
@@ -451,15 +455,9 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
   const int slot = s.row0 + 4 * warp;       // the warp's first group in a result vector
   const uint32_t tx = s.tx;
   float4 a[4 * NG][IT];
-#pragma unroll
-  for (int q = 0; q < 4 * NG; ++q) {
-    const float4* r4 = reinterpret_cast<const float4*>(csm + (4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp);
-#pragma unroll
-    for (int k = 0; k < IT; ++k) {
-      const int c = lane + 32 * k;
-      a[q][k] = c < (s.Mp >> 2) ? r4[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
+  if ((s.M & 3) == 0) load_rows<NG, IT, true>(a, L->Phiy, s);
+  else load_rows<NG, IT, false>(a, L->Phiy, s);
+  if (k0 == 0) sm100::cluster_wait();          // every CTA is ready to receive
   for (int step = k0; step < k1; ++step) {
     // S1: squared column norms (= row norms, Phi_y is exactly symmetric)             (Eq. 45)
     arm(l, e, tx);
@@ -467,27 +465,30 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
     wait_exchange(l, e, &s.fail); ++e;
     // S2: m' = argmax xi, x = row m' of Phi_y, c = Phi_y x                            (Eqs. 46-47)
     const int mp = argmax_xi(s);
-    const float* row = row_exchange(s, l, mp, e); ++e;
     arm(l, e, tx);
-    pass<PASS_SCALE, NG, IT>(a, row, 1.f, l, csm + s.cvec + slot, e);
+    send_column<NG, IT>(a, mp, l, csm + s.wvec + slot, e);
+    wait_exchange(l, e, &s.fail); ++e;
+    arm(l, e, tx);
+    pass<PASS_SCALE, NG, IT>(a, csm + s.wvec, 1.f, l, csm + s.cvec + slot, e);
     wait_exchange(l, e, &s.fail); ++e;
     // S3: coherent set and aligned average                                          (Eqs. 48-49)
     arm(l, e, tx);
     const int cnt = align_weights(s, l, mp);
     pass<PASS_SCALE, NG, IT>(a, csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, l, csm + s.buf0 + slot, e);
     wait_exchange(l, e, &s.fail); ++e;
-    // S4: P power iterations u = Phi_y (prev / ||prev||)
+    // S4: P power iterations u = Phi_y (prev / ||prev||); prev is sc times the vector at xo
     int xo = s.buf0, yo = xo + s.Mv;
+    float sc = 1.f;
     for (int p = 0; p < P; ++p) {
       arm(l, e, tx);
-      pass<PASS_NORM, NG, IT>(a, csm + xo, 0.f, l, csm + yo + slot, e);
+      sc = inv_norm(pass<PASS_NORM, NG, IT>(a, csm + xo, sc, l, csm + yo + slot, e));
       wait_exchange(l, e, &s.fail); ++e;
       const int t = xo; xo = yo; yo = t;
     }
     // S5: v = prev/||prev|| (Eq. 50), u = Phi_y v, lambda_e = v.u (Eq. 36)
     const float* x = csm + xo;
     arm(l, e, tx);
-    const float n2 = pass<PASS_UNIT, NG, IT>(a, x, 1.f, l, csm + s.uvec + slot, e);
+    const float n2 = pass<PASS_UNIT, NG, IT>(a, x, sc, l, csm + s.uvec + slot, e);
     const float inv = inv_norm(n2);
     float* vh = csm + s.vh + (step - k0) * s.Mv;
     wait_exchange(l, e, &s.fail); ++e;
@@ -497,7 +498,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       const float4 xv = x4[lane + 32 * k], uv = u4[lane + 32 * k];
-      const float4 vv = make_float4(xv.x * inv, xv.y * inv, xv.z * inv, xv.w * inv);
+      const float4 vv = make_float4(xv.x * sc * inv, xv.y * sc * inv, xv.z * sc * inv, xv.w * sc * inv);
       l0 = fmaf(vv.x, uv.x, l0); l1 = fmaf(vv.y, uv.y, l1);
       l0 = fmaf(vv.z, uv.z, l0); l1 = fmaf(vv.w, uv.w, l1);
       if (warp == 0) reinterpret_cast<float4*>(vh)[lane + 32 * k] = vv;      // every CTA records the whole vector
@@ -518,7 +519,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
 #pragma unroll
       for (int q = 0; q < 4 * NG; ++q) {
         const int i = slot + 4 * CW * (q >> 2) + (q & 3);
-        const float v = x[i] * inv, u = csm[s.uvec + i];
+        const float v = x[i] * sc * inv, u = csm[s.uvec + i];
         vi[q] = pack2(v, v); ui[q] = pack2(u, u);
       }
 #pragma unroll
@@ -526,14 +527,10 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
         const int c = lane + 32 * k;
         float4 vj = x4[c];
         const float4 uj = u4[c];
-        vj.x *= inv; vj.y *= inv; vj.z *= inv; vj.w *= inv;
+        vj.x = vj.x * sc * inv; vj.y = vj.y * sc * inv; vj.z = vj.z * sc * inv; vj.w = vj.w * sc * inv;
         const u64 va = pack2(vj.x, vj.y), vb = pack2(vj.z, vj.w), ua = pack2(uj.x, uj.y), ub = pack2(uj.z, uj.w);
 #pragma unroll
-        for (int q = 0; q < 4 * NG; ++q) {
-          a[q][k] = rank2(a[q][k], vi[q], ui[q], va, vb, ua, ub, a2, l2, z);
-          if (c < (s.Mp >> 2))
-            reinterpret_cast<float4*>(csm + (4 * (warp + CW * (q >> 2)) + (q & 3)) * s.Mp)[c] = a[q][k];
-        }
+        for (int q = 0; q < 4 * NG; ++q) a[q][k] = rank2(a[q][k], vi[q], ui[q], va, vb, ua, ub, a2, l2, z);
       }
     }
     if (threadIdx.x == 0) {
@@ -550,8 +547,12 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
         }
       }
     }
-    rows_sync(l);       // the slab is complete (any warp may send its row m' next), ah and vh for apply_steps
   }
+  if (!*(volatile int*)&s.fail) {
+    if ((s.M & 3) == 0) store_rows<NG, IT, true>(a, L->Phiy, s);
+    else store_rows<NG, IT, false>(a, L->Phiy, s);
+  }
+  rows_sync(l);         // ah and vh for apply_steps
 }
 
 // ---- layers of at most 64 features: one CTA, a row on 8 lanes ----
@@ -567,36 +568,67 @@ __device__ __forceinline__ float row_sum(float x) {
 __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int K, int P, bool smooth) {
   constexpr int KM = 64 / (4 * LPR);             // float4 per lane
   const int tid = threadIdx.x, row = tid / LPR, sub = tid % LPR;
-  const int M = s.M, M4 = s.Mp >> 2;
-  float4 a[KM];
+  const int M = s.M;
+  auto load = [&](float4 (&r)[KM], const float* G) {
 #pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    const int c = sub + LPR * k;
-    a[k] = row < s.R && c < M4 ? reinterpret_cast<const float4*>(csm + row * s.Mp)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+    for (int k = 0; k < KM; ++k) {
+      const int c = 4 * (sub + LPR * k);
+      float x[4] = {0.f, 0.f, 0.f, 0.f};
+      if (row < M && c < M) {
+        const float* p = G + (size_t)row * M + c;
+        if ((M & 3) == 0) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(p);
+        else
+#pragma unroll
+          for (int e = 0; e < 4; ++e) if (c + e < M) x[e] = p[e];
+      }
+      r[k] = make_float4(x[0], x[1], x[2], x[3]);
+    }
+  };
+  auto save = [&](const float4 (&r)[KM], float* G) {
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      const int c = 4 * (sub + LPR * k);
+      if (row < M && c < M) {
+        float* p = G + (size_t)row * M + c;
+        if ((M & 3) == 0) *reinterpret_cast<float4*>(p) = r[k];
+        else {
+          p[0] = r[k].x;
+          if (c + 1 < M) p[1] = r[k].y;
+          if (c + 2 < M) p[2] = r[k].z;
+          if (c + 3 < M) p[3] = r[k].w;
+        }
+      }
+    }
+  };
+  float4 a[KM];
+  load(a, L->Phiy);
   // Sums are formed as the warp of a larger layer forms them (a pair of sums per float4, then a tree over the float4s), so
   // that a layer's result does not depend on what else is in the launch.
   auto four = [](float4 x, float4 y) {
     return fmaf(x.z, y.z, __fmul_rn(x.x, y.x)) + fmaf(x.w, y.w, __fmul_rn(x.y, y.y));
   };
-  // y = scale (row . x) into dst; NORM: scale = 1 / ||x||, returns ||x||^2; UNIT: row . (x / ||x||)
+  // y = row . x into dst, as pass() does it: SCALE times scale; NORM: row . (scale x), returns ||scale x||^2 of the next scale;
+  // UNIT: row . (scale x / ||scale x||)
   auto dot = [&](const float* x, float scale, int mode, float* dst) {
     const float4* x4 = reinterpret_cast<const float4*>(x);
     float d = 0.f, n2 = 0.f, inv = 1.f;
-    if (mode != PASS_SCALE) {
+    float4 b[KM];
 #pragma unroll
-      for (int k = 0; k < KM; ++k) { const float4 b = x4[sub + LPR * k]; n2 = k ? n2 + four(b, b) : four(b, b); }
+    for (int k = 0; k < KM; ++k) {
+      b[k] = x4[sub + LPR * k];
+      if (mode == PASS_SCALE) continue;
+      b[k].x *= scale; b[k].y *= scale; b[k].z *= scale; b[k].w *= scale;
+      n2 = k ? n2 + four(b[k], b[k]) : four(b[k], b[k]);
     }
     if (mode == PASS_UNIT) { n2 = row_sum(n2); inv = inv_norm(n2); }
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
-      float4 b = x4[sub + LPR * k];
-      if (mode == PASS_UNIT) { b.x *= inv; b.y *= inv; b.z *= inv; b.w *= inv; }
-      d = k ? d + four(a[k], b) : four(a[k], b);
+      if (mode == PASS_UNIT) { b[k].x *= inv; b[k].y *= inv; b[k].z *= inv; b[k].w *= inv; }
+      d = k ? d + four(a[k], b[k]) : four(a[k], b[k]);
     }
-    if (mode == PASS_NORM) { n2 = row_sum(n2); scale = inv_norm(n2); }
     d = row_sum(d);
-    if (sub == 0) dst[row] = d * scale;
+    if (sub == 0) dst[row] = mode == PASS_SCALE ? d * scale : d;
+    if (mode == PASS_NORM) n2 = row_sum(n2);
     return n2;
   };
   for (int k0 = 0; k0 < K; k0 += KH) {
@@ -637,12 +669,14 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
       int xo = s.buf0, yo = xo + s.Mv;
       dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, PASS_SCALE, csm + xo);
       __syncthreads();
+      float sc = 1.f;                                                         // x is sc times the vector at xo
       for (int p = 0; p < P; ++p) {
-        dot(csm + xo, 0.f, PASS_NORM, csm + yo);
+        const float n2 = dot(csm + xo, sc, PASS_NORM, csm + yo);
         __syncthreads();
+        sc = inv_norm(n2);
         const int t = xo; xo = yo; yo = t;
       }
-      const float n2 = dot(csm + xo, 1.f, PASS_UNIT, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
+      const float n2 = dot(csm + xo, sc, PASS_UNIT, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
       const float inv = inv_norm(n2);
       __syncthreads();
       const float4* x4 = reinterpret_cast<const float4*>(csm + xo);
@@ -651,7 +685,7 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
 #pragma unroll
       for (int k = 0; k < KM; ++k) {
         float4 x = x4[sub + LPR * k];
-        x.x *= inv; x.y *= inv; x.z *= inv; x.w *= inv;
+        x.x = x.x * sc * inv; x.y = x.y * sc * inv; x.z = x.z * sc * inv; x.w = x.w * sc * inv;
         l0 = k ? l0 + four(x, u4[sub + LPR * k]) : four(x, u4[sub + LPR * k]);
       }
       const float lam_e = row_sum(l0);                              // Eq. 36
@@ -663,17 +697,17 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
       }
       // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T, as in run_steps
       if (aa != 0.f) {
-        const float v = csm[xo + row] * inv, u = csm[s.uvec + row], l = aa * aa * lam_e;
+        const float v = csm[xo + row] * sc * inv, u = csm[s.uvec + row], l = aa * aa * lam_e;
 #pragma unroll
         for (int k = 0; k < KM; ++k) {
           float4 vj = x4[sub + LPR * k];
           const float4 uj = u4[sub + LPR * k];
-          vj.x *= inv; vj.y *= inv; vj.z *= inv; vj.w *= inv;
+          vj.x = vj.x * sc * inv; vj.y = vj.y * sc * inv; vj.z = vj.z * sc * inv; vj.w = vj.w * sc * inv;
           a[k] = rank2(a[k], pack2(v, v), pack2(u, u), pack2(vj.x, vj.y), pack2(vj.z, vj.w), pack2(uj.x, uj.y), pack2(uj.z, uj.w),
                        pack2(aa, aa), pack2(l, l), pack2(s.negz, s.negz));
         }
       }
-      if (tid < 64) csm[s.vh + (step - k0) * s.Mv + tid] = csm[xo + tid] * inv;
+      if (tid < 64) csm[s.vh + (step - k0) * s.Mv + tid] = csm[xo + tid] * sc * inv;
       if (tid == 0) {
         s.ah[step - k0] = aa;
         if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
@@ -691,37 +725,6 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     // ---- the recorded steps in T, then Q (Eqs. 42, 44), as in apply_steps ----
     const bool last = k1 == K;
     float4 t[KM], o[KM];
-    auto load = [&](float4 (&r)[KM], const float* G) {
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const int c = 4 * (sub + LPR * k);
-        float x[4] = {0.f, 0.f, 0.f, 0.f};
-        if (row < M && c < M) {
-          const float* p = G + (size_t)row * M + c;
-          if ((M & 3) == 0) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(p);
-          else
-#pragma unroll
-            for (int e = 0; e < 4; ++e) if (c + e < M) x[e] = p[e];
-        }
-        r[k] = make_float4(x[0], x[1], x[2], x[3]);
-      }
-    };
-    auto save = [&](const float4 (&r)[KM], float* G) {
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const int c = 4 * (sub + LPR * k);
-        if (row < M && c < M) {
-          float* p = G + (size_t)row * M + c;
-          if ((M & 3) == 0) *reinterpret_cast<float4*>(p) = r[k];
-          else {
-            p[0] = r[k].x;
-            if (c + 1 < M) p[1] = r[k].y;
-            if (c + 2 < M) p[2] = r[k].z;
-            if (c + 3 < M) p[3] = r[k].w;
-          }
-        }
-      }
-    };
     load(t, L->Tt);
 #pragma unroll 1
     for (int j = 0; j < k1 - k0; ++j) {
@@ -775,11 +778,7 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    const int c = sub + LPR * k;
-    if (row < s.R && c < M4) reinterpret_cast<float4*>(csm + row * s.Mp)[c] = a[k];
-  }
+  save(a, L->Phiy);
 }
 
 // groups of four rows this warp owns in a slab of R rows
@@ -835,8 +834,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     s.Mv = slab_vec(M, n);
     s.sub = (int)blockIdx.x - a.first_cta[layer];
     s.row0 = s.sub * s.R;
-    s.nrows = max(0, min(s.R, M - s.row0));
-    s.xi2 = s.R * s.Mp;
+    s.xi2 = 0;
     s.cvec = s.xi2 + s.Mv; s.wvec = s.cvec + s.Mv; s.buf0 = s.wvec + s.Mv; s.uvec = s.buf0 + 2 * s.Mv;
     s.vh = s.uvec + s.Mv; s.th = s.vh + KH * s.Mv;
     s.tx = (uint32_t)n * (uint32_t)s.R * 4u;
@@ -849,42 +847,29 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     sm100::mbar_fence_init();
   }
   __syncthreads();
-  const int M = s.M, R = s.R, nrows = s.nrows;
+  const int M = s.M, R = s.R;
   l.active = 32 * min(CW, R >> 2);
 
-  // ---- load my rows of Phi_y (padded with zeros to R rows of Mp); clear the vectors ----
-  if ((M & 3) == 0) {
-    // 16-byte asynchronous copies, every one of a thread in flight at once: one trip to memory
-    const int M4 = M >> 2;
-    for (int i = threadIdx.x; i < R * M4; i += CT) {
-      const int r = i / M4, c = i - r * M4;
-      float* d = csm + (size_t)r * M + 4 * c;
-      if (r < nrows) cp_async16(smem_u32(d), L->Phiy + (size_t)(s.row0 + r) * M + 4 * c);
-      else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  } else {
-    for (int i = threadIdx.x; i < R * s.Mp; i += CT) {
-      const int r = i / s.Mp, c = i - r * s.Mp;
-      csm[i] = (c < M && r < nrows) ? L->Phiy[(size_t)(s.row0 + r) * M + c] : 0.f;
-    }
-  }
-  for (int i = threadIdx.x; i < kVecs * s.Mv; i += CT) csm[s.xi2 + i] = 0.f;
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  // what no exchange fills of the vectors stays zero (rows past the matrix are zero rows)
+  const int filled = l.n * R, tail = s.Mv - filled;
+  for (int i = threadIdx.x; i < kVecs * tail; i += CT) csm[i / tail * s.Mv + filled + i % tail] = 0.f;
   // A CTA's window of the cluster address space is this CTA's window shifted by a constant; the stores rely on it,
   // so it is checked on two addresses far apart before anything is sent.
   const uint32_t peer_rank = (uint32_t)(rank - s.sub + min(lane, l.n - 1));
   l.rdelta = map_cluster(l.bar0, peer_rank) - l.bar0;
   const bool linear = (map_cluster(smem_u32(csm + s.th), peer_rank) - smem_u32(csm + s.th)) == l.rdelta;
   const bool usable = __syncthreads_or(!linear) == 0;
-  cluster.sync();   // every barrier is initialised before the first remote store can arrive
+  sm100::cluster_arrive();   // every barrier is initialised before the first remote store can arrive: waited for in run_steps
 
+  const int ng = solo(M, l.n) ? 0 : warp_groups(R);
+  if (!usable || ng == 0 || a.K < 1) sm100::cluster_wait();
   if (usable) {
     float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
     if (solo(M, l.n)) {
       const bool smooth = L->Qs != L->Q;
       run_solo(s, L, tr, a.K, a.P, smooth);
     } else {
-    const int it = slab_trips(M), ng = warp_groups(R);
+    const int it = slab_trips(M);
     uint32_t e = 0;                        // exchanges so far
     for (int k0 = 0; k0 < a.K; k0 += KH) {
       const int k1 = min(a.K, k0 + KH);
@@ -914,21 +899,12 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
   } else {
     if (s.sub == 0 && !s.maxcol)
       for (int m = threadIdx.x; m < M; m += CT) L->wvec[m] = csm[s.wvec + m];    // alignment weights of the last step
-    if ((M & 3) == 0) {
-      float4* dst = reinterpret_cast<float4*>(L->Phiy + (size_t)s.row0 * M);
-      for (int i = threadIdx.x; i < nrows * (M >> 2); i += CT) dst[i] = reinterpret_cast<const float4*>(csm)[i];
-    } else {
-      for (int i = threadIdx.x; i < nrows * s.Mp; i += CT) {
-        const int r = i / s.Mp, c = i - r * s.Mp;
-        if (c < M) L->Phiy[(size_t)(s.row0 + r) * M + c] = csm[i];
-      }
-    }
   }
   cluster.sync();   // no CTA leaves while a peer may still read or write its shared memory
 }
 
 size_t cluster_smem(int M, int n) {
-  return ((size_t)slab_rows(M, n) * ((M + 3) & ~3) + (size_t)kVecs * slab_vec(M, n)) * sizeof(float);
+  return (size_t)kVecs * slab_vec(M, n) * sizeof(float);
 }
 
 bool cluster_fits(int M, int n) {
