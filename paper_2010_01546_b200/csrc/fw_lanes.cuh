@@ -13,6 +13,13 @@ __device__ __forceinline__ u64 pack2(float x, float y) {
 }
 __device__ __forceinline__ void unpack2(u64 r, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r)); }
 __device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ u64 fmadd2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// (not for a product that is added to: see mul2)
+__device__ __forceinline__ u64 times2(u64 a, u64 b) { u64 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 // A product rounded by itself: the compiler fuses a packed multiplication with the addition that follows it, .rn or not, so
 // the product is an fma with z = (-0, -0), which the compiler must not know (callers read it from shared memory).
 __device__ __forceinline__ u64 mul2(u64 a, u64 b, u64 z) {
@@ -21,14 +28,35 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b, u64 z) {
   return r;
 }
 
-// p + (a (vi u_j + ui v_j) + l vi v_j) of four entries j (l = a^2 lambda_e; va, vb, ua, ub: v_j and u_j of the first and the
-// last two), a rounding per operation and symmetric in (i, j), on packed pairs: half the issue slots.
+// p + (a (vi u_j + ui v_j) + l vi v_j) of two or four entries j (l = a^2 lambda_e; va, vb, ua, ub: v_j and u_j of the first and
+// the last two), a rounding per operation and symmetric in (i, j), on packed pairs: half the issue slots.
+__device__ __forceinline__ u64 rank2(u64 p, u64 vi, u64 ui, u64 vj, u64 uj, u64 a, u64 l, u64 z) {
+  return add2(p, add2(mul2(a, add2(mul2(vi, uj, z), mul2(ui, vj, z)), z), mul2(l, mul2(vi, vj, z), z)));
+}
 __device__ __forceinline__ float4 rank2(float4 p, u64 vi, u64 ui, u64 va, u64 vb, u64 ua, u64 ub, u64 a, u64 l, u64 z) {
-  const u64 x = add2(pack2(p.x, p.y), add2(mul2(a, add2(mul2(vi, ua, z), mul2(ui, va, z)), z), mul2(l, mul2(vi, va, z), z)));
-  const u64 y = add2(pack2(p.z, p.w), add2(mul2(a, add2(mul2(vi, ub, z), mul2(ui, vb, z)), z), mul2(l, mul2(vi, vb, z), z)));
+  const u64 x = rank2(pack2(p.x, p.y), vi, ui, va, ua, a, l, z), y = rank2(pack2(p.z, p.w), vi, ui, vb, ub, a, l, z);
   unpack2(x, p.x, p.y);
   unpack2(y, p.z, p.w);
   return p;
+}
+
+struct Quad { u64 lo, hi; };       // four neighbouring entries of a row, as packed pairs
+
+// Sums of four values over the warp in 6 shuffles instead of 20: halves of the warp keep two of the values, quarters
+// one, and the four totals are handed to every lane.
+__device__ __forceinline__ float4 warp_sum4(float y0, float y1, float y2, float y3) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
+  float u0 = hi ? y2 : y0, u1 = hi ? y3 : y1;
+  u0 += __shfl_xor_sync(0xffffffffu, hi ? y0 : y2, 16);
+  u1 += __shfl_xor_sync(0xffffffffu, hi ? y1 : y3, 16);
+  float z = mid ? u1 : u0;
+  z += __shfl_xor_sync(0xffffffffu, mid ? u0 : u1, 8);
+  z += __shfl_xor_sync(0xffffffffu, z, 4);
+  z += __shfl_xor_sync(0xffffffffu, z, 2);
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
+  return make_float4(__shfl_sync(0xffffffffu, z, 0), __shfl_sync(0xffffffffu, z, 8), __shfl_sync(0xffffffffu, z, 16),
+                     __shfl_sync(0xffffffffu, z, 24));
 }
 
 // sum over the warp, the same bits in every lane

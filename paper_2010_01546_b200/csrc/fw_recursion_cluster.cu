@@ -9,10 +9,9 @@
 // CTAs' copies of the vector with asynchronous remote stores that count bytes on
 // the receiver's mbarrier, and every warp waits on its own CTA's barrier -- no
 // block or cluster barrier separates the power iterations.  T and Q are not
-// needed by a step, so a step only records its v_e and a_e; after the last step
-// (or every KH) each warp loads its rows of T^T, forms t = T^T v_e step by step,
-// and T and Q take the rank-one terms (Eqs. 42, 44) in step order: the product
-// T^T v is out of the chain and the rows of T^T out of shared memory.
+// needed by a step, so a step only records its v_e and a_e; after the last one
+// each warp loads its rows of T^T, forms t = T^T v_e step by step (t goes round on a
+// barrier of its own), and T and Q take the rank-one terms in step order (Eqs. 42, 44).
 //
 // What bounds it: the chain of P + 5 dependent exchanges per step.  A pass reads
 // only the vector from shared memory (rows in registers: at M = 576 the slab's 83
@@ -47,7 +46,8 @@ constexpr int CT = 512;            // threads per CTA
 constexpr int CW = CT / 32;        // warps per CTA
 constexpr int kMaxIt = 5;          // float4 columns per lane, at most
 constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take teams of CTAs and fp64 sums
-constexpr int KH = 8;              // steps between two updates of T and Q
+constexpr int kSolo = 64;          // largest layer that takes one CTA and eight lanes a row
+constexpr int KH = kChipSteps;     // steps of a launch, all of which T and Q take at its end
 constexpr size_t kSmemLimit = 64 * 1024;   // the vectors of the longest row: 22 of 16 slabs of at most 43 entries
 
 // A warp owns one group of four rows (up to kMaxIt float4 columns per lane: 80 registers) or, for rows of at most 256
@@ -59,7 +59,8 @@ struct ClusterArgs {
   PtrTable traces;
   int32_t first_cta[FW_MAX_GROUP];   // first CTA of each layer (a layer never straddles a cluster)
   int32_t ncta[FW_MAX_GROUP];        // CTAs of each layer: 1 ... cluster size
-  int32_t K, P;
+  int32_t k0, K, P;                  // first step of the call in this launch, steps, power iterations
+  int32_t last;                      // this launch ends the call
 };
 
 // shared-memory address of the same variable in CTA `rank` of the cluster
@@ -85,7 +86,7 @@ extern __shared__ __align__(16) float csm[];
 struct Slab {
   // offsets into the dynamic shared memory (not pointers: the compiler then knows which memory they point to)
   int xi2, cvec, wvec, buf0, uvec;   // vectors of Mv floats; buf0: two, Mv apart
-  int vh, th;     // v_e and t of the recorded steps, KH vectors each
+  int vh, th;     // v_e and t of the steps, KH vectors each
   int M, Mp;      // matrix size, padded row length
   int Mv;         // vector length in shared memory
   int R;          // rows per CTA, a multiple of four (rows past the matrix are zero rows)
@@ -95,34 +96,17 @@ struct Slab {
   uint32_t tx;    // bytes of one exchanged vector
   int maxcol;     // start vector: largest column instead of the alignment
   float c_rel, c_abs, delta, eps, lam_bar;
-  float ah[KH];   // a_e of the recorded steps
+  float ah[KH];   // a_e of the steps
   float negz;     // -0
   int fail;       // set once a bounded wait of this CTA gave up
 };
 // The parts of it every pass needs, in registers.
 struct Link {
   uint32_t rdelta;  // lane p < n: cluster address of CTA p's shared memory minus this CTA's own
-  uint32_t bar0;    // two exchange barriers, 8 bytes apart
+  uint32_t bar0;    // two exchange barriers and the one of all steps' t, 8 bytes apart
   int n;
   int active;       // threads of the warps that own rows; the others take no part in the steps
 };
-
-// Sums of four values over the warp in 6 shuffles instead of 20: halves of the warp keep two of the values, quarters
-// one, and the four totals are handed to every lane.
-__device__ __forceinline__ float4 warp_sum4(float y0, float y1, float y2, float y3) {
-  const int lane = threadIdx.x & 31;
-  const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
-  float u0 = hi ? y2 : y0, u1 = hi ? y3 : y1;
-  u0 += __shfl_xor_sync(0xffffffffu, hi ? y0 : y2, 16);
-  u1 += __shfl_xor_sync(0xffffffffu, hi ? y1 : y3, 16);
-  float z = mid ? u1 : u0;
-  z += __shfl_xor_sync(0xffffffffu, mid ? u0 : u1, 8);
-  z += __shfl_xor_sync(0xffffffffu, z, 4);
-  z += __shfl_xor_sync(0xffffffffu, z, 2);
-  z += __shfl_xor_sync(0xffffffffu, z, 1);
-  return make_float4(__shfl_sync(0xffffffffu, z, 0), __shfl_sync(0xffffffffu, z, 8), __shfl_sync(0xffffffffu, z, 16),
-                     __shfl_sync(0xffffffffu, z, 24));
-}
 
 // barriers among the warps that own rows
 __device__ __forceinline__ void rows_sync(const Link& l) { asm volatile("bar.sync 1, %0;" ::"r"(l.active) : "memory"); }
@@ -134,14 +118,16 @@ __device__ __forceinline__ void arm(const Link& l, uint32_t e, uint32_t bytes) {
 // Bounded wait for exchange e.  Every warp waits for itself.  Once a wait has given up no later wait of the CTA
 // blocks: the CTA runs on with stale data to the end of the call, so that its block barriers and its peers stay in
 // step, and reports the time-out there.  A layer on one CTA exchanges through its own shared memory.
-__device__ __forceinline__ void wait_exchange(const Link& l, uint32_t e, int* fail) {
-  if (l.n == 1) { rows_sync(l); return; }
-  const uint32_t bar = l.bar0 + ((e & 1) << 3), parity = (e >> 1) & 1;
+__device__ __forceinline__ void wait_bar(uint32_t bar, uint32_t parity, int* fail) {
   if (sm100::mbar_try_wait(bar, parity)) return;
   if (*(volatile int*)fail) return;
   for (uint32_t i = 0; i < sm100::kSpinLimit; ++i)
     if (sm100::mbar_try_wait(bar, parity)) return;
   *(volatile int*)fail = 1;
+}
+__device__ __forceinline__ void wait_exchange(const Link& l, uint32_t e, int* fail) {
+  if (l.n == 1) rows_sync(l);
+  else wait_bar(l.bar0 + ((e & 1) << 3), (e >> 1) & 1, fail);
 }
 // four results of a group into `tgt` of every CTA of the layer
 __device__ __forceinline__ void send4(const Link& l, float* tgt, float4 v, uint32_t e) {
@@ -154,57 +140,72 @@ __device__ __forceinline__ void send4(const Link& l, float* tgt, float4 v, uint3
 }
 
 // One pass: y = (my rows) x, sent to `dst` (the slot of the warp's first group in the result vector) of every CTA of the
-// layer.  SCALE: y times `scale`.  NORM and UNIT take x as it was sent times `scale`.  NORM returns ||scale x||^2, summed after y
-// has gone: a power iteration's y = Phi_y x / ||x|| is sent without the 1 / ||x||, which every receiver knows and applies to the
-// entries it loads, so that the norm's reduction and root run while the exchange does (M = 576: XXX).  UNIT: the
-// rows times scale x / ||scale x||, the norm summed first.  SELF: squared norms of the rows themselves.
+// layer.  SCALE: y times `scale`.  NORM and UNIT take x as it was sent times `scale`: a power iteration's y = Phi_y x / ||x|| is
+// sent without the 1 / ||x||, which a receiver applies to the entries it loads.  NORM returns ||scale x||^2, reduced once y has gone,
+// so that the norm's reduction and root run beside the exchange.  UNIT: the rows times scale x / ||scale x||, the norm first;
+// returns its square.  SELF: squared norms of the rows themselves.  Sums are packed pairs: half the instructions, every
+// product and sum rounded as before.  Recursion of the ResNet-20-shaped set (K = 4, P = 16): 124 us with scalar sums, 107
+// packed; 64 layers of M = 256, K = 8, P = 32: 292 and 262.  One warp's norm for the whole CTA, arming the exchange's barrier
+// when it is there, took 114 and 296.
 enum { PASS_SELF, PASS_SCALE, PASS_NORM, PASS_UNIT };
 template <int MODE, int NG, int IT>
-__device__ __forceinline__ float pass(const float4 (&a)[4 * NG][IT], const float* x, float scale, const Link& l,
+__device__ __forceinline__ float pass(const Quad (&a)[4 * NG][IT], const float* x, float scale, const Link& l,
                                       float* dst, uint32_t e) {
   const int lane = threadIdx.x & 31;
   const float4* x4 = reinterpret_cast<const float4*>(x);
-  float acc[4 * NG][2];
+  u64 acc[4 * NG], nn = pack2(0.f, 0.f);
 #pragma unroll
-  for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
-  float n0 = 0.f, n1 = 0.f, n2 = 0.f, inv = 1.f;
+  for (int q = 0; q < 4 * NG; ++q) acc[q] = pack2(0.f, 0.f);
+  const u64 sc = pack2(scale, scale);
+  float n2 = 0.f;
+  u64 inv = 0;
   if (MODE == PASS_UNIT) {
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
-      float4 b = x4[lane + 32 * k];
-      b.x *= scale; b.y *= scale; b.z *= scale; b.w *= scale;
-      n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
-      n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
+      const float4 b = x4[lane + 32 * k];
+      const u64 lo = times2(pack2(b.x, b.y), sc), hi = times2(pack2(b.z, b.w), sc);
+      nn = fmadd2(hi, hi, fmadd2(lo, lo, nn));
     }
+    float n0, n1;
+    unpack2(nn, n0, n1);
     n2 = warp_sum(n0 + n1);
-    inv = inv_norm(n2);
+    const float i = inv_norm(n2);
+    inv = pack2(i, i);
   }
 #pragma unroll
   for (int k = 0; k < IT; ++k) {
-    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (MODE != PASS_SELF) b = x4[lane + 32 * k];
-    if (MODE == PASS_NORM || MODE == PASS_UNIT) { b.x *= scale; b.y *= scale; b.z *= scale; b.w *= scale; }
-    if (MODE == PASS_UNIT) { b.x *= inv; b.y *= inv; b.z *= inv; b.w *= inv; }
-    if (MODE == PASS_NORM) {
-      n0 = fmaf(b.x, b.x, n0); n1 = fmaf(b.y, b.y, n1);
-      n0 = fmaf(b.z, b.z, n0); n1 = fmaf(b.w, b.w, n1);
+    u64 lo = 0, hi = 0;
+    if (MODE != PASS_SELF) {
+      const float4 b = x4[lane + 32 * k];
+      lo = pack2(b.x, b.y); hi = pack2(b.z, b.w);
     }
+    if (MODE == PASS_NORM || MODE == PASS_UNIT) { lo = times2(lo, sc); hi = times2(hi, sc); }
+    if (MODE == PASS_UNIT) { lo = times2(lo, inv); hi = times2(hi, inv); }
+    if (MODE == PASS_NORM) nn = fmadd2(hi, hi, fmadd2(lo, lo, nn));
 #pragma unroll
     for (int q = 0; q < 4 * NG; ++q) {
-      const float4 v = a[q][k];
-      const float4 bb = MODE == PASS_SELF ? v : b;
-      acc[q][0] = fmaf(v.x, bb.x, acc[q][0]); acc[q][1] = fmaf(v.y, bb.y, acc[q][1]);
-      acc[q][0] = fmaf(v.z, bb.z, acc[q][0]); acc[q][1] = fmaf(v.w, bb.w, acc[q][1]);
+      const Quad v = a[q][k];
+      acc[q] = fmadd2(v.hi, MODE == PASS_SELF ? v.hi : hi, fmadd2(v.lo, MODE == PASS_SELF ? v.lo : lo, acc[q]));
     }
   }
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    float4 v = warp_sum4(acc[4 * g][0] + acc[4 * g][1], acc[4 * g + 1][0] + acc[4 * g + 1][1],
-                         acc[4 * g + 2][0] + acc[4 * g + 2][1], acc[4 * g + 3][0] + acc[4 * g + 3][1]);
+    float y[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float y0, y1;
+      unpack2(acc[4 * g + q], y0, y1);
+      y[q] = y0 + y1;
+    }
+    float4 v = warp_sum4(y[0], y[1], y[2], y[3]);
     if (MODE == PASS_SCALE) { v.x *= scale; v.y *= scale; v.z *= scale; v.w *= scale; }
     send4(l, dst + 4 * CW * g, v, e);
   }
-  if (MODE == PASS_NORM) n2 = warp_sum(n0 + n1);
+  if (MODE == PASS_NORM) {
+    float n0, n1;
+    unpack2(nn, n0, n1);
+    n2 = warp_sum(n0 + n1);
+  }
   return n2;
 }
 
@@ -232,7 +233,7 @@ __device__ __forceinline__ int argmax_xi(const Slab& s) {
 // its rows in column m': a message of four entries a warp like any other exchange, where the owner of row m' sending it to
 // all alone took 4900 clocks (M = 576 on 12 CTAs: 1728 messages of one SM).
 template <int NG, int IT>
-__device__ __forceinline__ void send_column(const float4 (&a)[4 * NG][IT], int mp, const Link& l, float* dst, uint32_t e) {
+__device__ __forceinline__ void send_column(const Quad (&a)[4 * NG][IT], int mp, const Link& l, float* dst, uint32_t e) {
   const int k0 = mp >> 7, from = (mp >> 2) & 31, c = mp & 3;
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
@@ -242,8 +243,11 @@ __device__ __forceinline__ void send_column(const float4 (&a)[4 * NG][IT], int m
       float x = 0.f;
 #pragma unroll
       for (int k = 0; k < IT; ++k) {
-        const float4 v = a[4 * g + q][k];
-        if (k == k0) x = c < 2 ? (c == 0 ? v.x : v.y) : (c == 2 ? v.z : v.w);
+        if (k == k0) {
+          float even, odd;
+          unpack2(c < 2 ? a[4 * g + q][k].lo : a[4 * g + q][k].hi, even, odd);
+          x = c & 1 ? odd : even;
+        }
       }
       y[q] = __shfl_sync(0xffffffffu, x, from);
     }
@@ -284,7 +288,7 @@ __device__ __forceinline__ int align_weights(Slab& s, const Link& l, int mp) {
 
 // rows of a row-major matrix in global memory <-> the registers of the warp that owns them; V4: rows of whole float4s
 template <int NG, int IT, bool V4>
-__device__ __forceinline__ void load_rows(float4 (&a)[4 * NG][IT], const float* G, const Slab& s) {
+__device__ __forceinline__ void load_rows(Quad (&a)[4 * NG][IT], const float* G, const Slab& s) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = s.M;
 #pragma unroll
@@ -294,22 +298,24 @@ __device__ __forceinline__ void load_rows(float4 (&a)[4 * NG][IT], const float* 
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       const int c = lane + 32 * k;
-      a[q][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i >= M) continue;
-      if (V4) {
-        if (4 * c < M) a[q][k] = reinterpret_cast<const float4*>(row)[c];
-      } else {
-        if (4 * c < M) a[q][k].x = row[4 * c];
-        if (4 * c + 1 < M) a[q][k].y = row[4 * c + 1];
-        if (4 * c + 2 < M) a[q][k].z = row[4 * c + 2];
-        if (4 * c + 3 < M) a[q][k].w = row[4 * c + 3];
+      float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < M) {
+        if (V4) {
+          if (4 * c < M) r = reinterpret_cast<const float4*>(row)[c];
+        } else {
+          if (4 * c < M) r.x = row[4 * c];
+          if (4 * c + 1 < M) r.y = row[4 * c + 1];
+          if (4 * c + 2 < M) r.z = row[4 * c + 2];
+          if (4 * c + 3 < M) r.w = row[4 * c + 3];
+        }
       }
+      a[q][k].lo = pack2(r.x, r.y); a[q][k].hi = pack2(r.z, r.w);
     }
   }
 }
 // ROUND: rounded to the TF32 grid
 template <int NG, int IT, bool V4, bool ROUND = false>
-__device__ __forceinline__ void store_rows(const float4 (&a)[4 * NG][IT], float* G, const Slab& s) {
+__device__ __forceinline__ void store_rows(const Quad (&a)[4 * NG][IT], float* G, const Slab& s) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = s.M;
 #pragma unroll
@@ -320,94 +326,110 @@ __device__ __forceinline__ void store_rows(const float4 (&a)[4 * NG][IT], float*
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       const int c = lane + 32 * k;
+      float4 r;
+      unpack2(a[q][k].lo, r.x, r.y);
+      unpack2(a[q][k].hi, r.z, r.w);
+      if (ROUND) r = make_float4(sm100::tf32_rna(r.x), sm100::tf32_rna(r.y), sm100::tf32_rna(r.z), sm100::tf32_rna(r.w));
       if (V4) {
-        float4 v = a[q][k];
-        if (ROUND) v = make_float4(sm100::tf32_rna(v.x), sm100::tf32_rna(v.y), sm100::tf32_rna(v.z), sm100::tf32_rna(v.w));
-        if (4 * c < M) reinterpret_cast<float4*>(row)[c] = v;
+        if (4 * c < M) reinterpret_cast<float4*>(row)[c] = r;
       } else {
-        if (4 * c < M) row[4 * c] = a[q][k].x;
-        if (4 * c + 1 < M) row[4 * c + 1] = a[q][k].y;
-        if (4 * c + 2 < M) row[4 * c + 2] = a[q][k].z;
-        if (4 * c + 3 < M) row[4 * c + 3] = a[q][k].w;
+        if (4 * c < M) row[4 * c] = r.x;
+        if (4 * c + 1 < M) row[4 * c + 1] = r.y;
+        if (4 * c + 2 < M) row[4 * c + 2] = r.z;
+        if (4 * c + 3 < M) row[4 * c + 3] = r.w;
       }
     }
   }
 }
 
-// The recorded steps in T and Q, one exchange in all.  T first (t of step k comes from T after step k - 1), then Q, with
-// the operations on every element in step order; smooth: Qs <- beta Qs + (1 - beta) Q (Eq. 35).
+// The K recorded steps in T and Q: T first (t of step k comes from T after step k - 1), then Q, with the operations on every
+// element in step order; smooth: Qs <- beta Qs + (1 - beta) Q (Eq. 35).
 template <int NG, int IT, bool V4>
-__device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* L, int steps, bool smooth, uint32_t e) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float4 a[4 * NG][IT];
-  float* th = csm + s.th + s.row0 + 4 * warp;
+__device__ __forceinline__ void apply_steps(Slab& s, const Link& l, const LayerDev* L, int K, bool smooth) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, M = s.M;
   int live = 0;
 #pragma unroll 1
-  for (int k = 0; k < steps; ++k) live += s.ah[k] != 0.f ? 1 : 0;
+  for (int k = 0; k < K; ++k) live += s.ah[k] != 0.f ? 1 : 0;
+  if (!live && !smooth) return;
+  Quad a[4 * NG][IT];
   if (live) {
     load_rows<NG, IT, V4>(a, L->Tt, s);
-    arm(l, e, (uint32_t)live * s.tx);
 #pragma unroll 1
-    for (int k = 0; k < steps; ++k) {
+    for (int k = 0; k < K; ++k) {
       const float ak = s.ah[k];
       if (ak == 0.f) continue;
       const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + k * s.Mv);
-      float acc[4 * NG][2];
+      u64 acc[4 * NG];
 #pragma unroll
-      for (int q = 0; q < 4 * NG; ++q) acc[q][0] = acc[q][1] = 0.f;
+      for (int q = 0; q < 4 * NG; ++q) acc[q] = pack2(0.f, 0.f);
 #pragma unroll
       for (int it = 0; it < IT; ++it) {
         const float4 b = v4[lane + 32 * it];
+        const u64 lo = pack2(b.x, b.y), hi = pack2(b.z, b.w);
 #pragma unroll
-        for (int q = 0; q < 4 * NG; ++q) {
-          acc[q][0] = fmaf(a[q][it].x, b.x, acc[q][0]); acc[q][1] = fmaf(a[q][it].y, b.y, acc[q][1]);
-          acc[q][0] = fmaf(a[q][it].z, b.z, acc[q][0]); acc[q][1] = fmaf(a[q][it].w, b.w, acc[q][1]);
-        }
+        for (int q = 0; q < 4 * NG; ++q) acc[q] = fmadd2(a[q][it].hi, hi, fmadd2(a[q][it].lo, lo, acc[q]));
       }
-      float at[4 * NG];
+      u64 at[4 * NG];
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
-        const float4 t = warp_sum4(acc[4 * g][0] + acc[4 * g][1], acc[4 * g + 1][0] + acc[4 * g + 1][1],
-                                   acc[4 * g + 2][0] + acc[4 * g + 2][1], acc[4 * g + 3][0] + acc[4 * g + 3][1]);
-        send4(l, th + k * s.Mv + 4 * CW * g, t, e);
-        at[4 * g] = ak * t.x; at[4 * g + 1] = ak * t.y; at[4 * g + 2] = ak * t.z; at[4 * g + 3] = ak * t.w;
+        float y[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float y0, y1;
+          unpack2(acc[4 * g + q], y0, y1);
+          y[q] = y0 + y1;
+        }
+        const float4 t = warp_sum4(y[0], y[1], y[2], y[3]);
+        float* tgt = csm + s.th + k * s.Mv + s.row0 + 4 * (warp + CW * g);
+        if (l.n == 1) {
+          if (lane == 0) *reinterpret_cast<float4*>(tgt) = t;
+        } else if (lane < l.n) {
+          st_async_v4(smem_u32(tgt) + l.rdelta, t, l.bar0 + 16 + l.rdelta);
+        }
+        at[4 * g] = pack2(ak * t.x, ak * t.x); at[4 * g + 1] = pack2(ak * t.y, ak * t.y);
+        at[4 * g + 2] = pack2(ak * t.z, ak * t.z); at[4 * g + 3] = pack2(ak * t.w, ak * t.w);
       }
 #pragma unroll
       for (int it = 0; it < IT; ++it) {
         const float4 b = v4[lane + 32 * it];
+        const u64 lo = pack2(b.x, b.y), hi = pack2(b.z, b.w);
 #pragma unroll
-        for (int q = 0; q < 4 * NG; ++q) {
-          a[q][it].x = fmaf(at[q], b.x, a[q][it].x); a[q][it].y = fmaf(at[q], b.y, a[q][it].y);
-          a[q][it].z = fmaf(at[q], b.z, a[q][it].z); a[q][it].w = fmaf(at[q], b.w, a[q][it].w);
-        }
+        for (int q = 0; q < 4 * NG; ++q) { a[q][it].lo = fmadd2(at[q], lo, a[q][it].lo); a[q][it].hi = fmadd2(at[q], hi, a[q][it].hi); }
       }
     }
     store_rows<NG, IT, V4>(a, L->Tt, s);
     if (V4 && L->round_t) store_rows<NG, IT, true, true>(a, L->tmp, s);
-  } else {
-    arm(l, e, 0u);
   }
   load_rows<NG, IT, V4>(a, L->Q, s);
-  wait_exchange(l, e, &s.fail);
   if (live) {
+    if (l.n == 1) {
+      rows_sync(l);
+    } else {
+      if (threadIdx.x == 0) sm100::mbar_expect_tx(l.bar0 + 16, (uint32_t)live * s.tx);
+      wait_bar(l.bar0 + 16, 0, &s.fail);
+    }
+    const u64 z = pack2(s.negz, s.negz);
 #pragma unroll 1
-    for (int k = 0; k < steps; ++k) {
+    for (int k = 0; k < K; ++k) {
       const float ak = s.ah[k];
       if (ak == 0.f) continue;
       const float aq = ak * (ak + 2.f);
+      const u64 aq2 = pack2(aq, aq);
       const float* tk = csm + s.th + k * s.Mv;
-      float ti[4 * NG];
+      u64 ti[4 * NG];
 #pragma unroll
-      for (int q = 0; q < 4 * NG; ++q) ti[q] = tk[s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3)];
+      for (int q = 0; q < 4 * NG; ++q) {
+        const float t = tk[s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3)];
+        ti[q] = pack2(t, t);
+      }
 #pragma unroll
       for (int it = 0; it < IT; ++it) {
         const float4 b = reinterpret_cast<const float4*>(tk)[lane + 32 * it];
+        const u64 lo = pack2(b.x, b.y), hi = pack2(b.z, b.w);
 #pragma unroll
         for (int q = 0; q < 4 * NG; ++q) {
-          a[q][it].x = __fadd_rn(a[q][it].x, __fmul_rn(aq, __fmul_rn(ti[q], b.x)));
-          a[q][it].y = __fadd_rn(a[q][it].y, __fmul_rn(aq, __fmul_rn(ti[q], b.y)));
-          a[q][it].z = __fadd_rn(a[q][it].z, __fmul_rn(aq, __fmul_rn(ti[q], b.z)));
-          a[q][it].w = __fadd_rn(a[q][it].w, __fmul_rn(aq, __fmul_rn(ti[q], b.w)));
+          a[q][it].lo = add2(a[q][it].lo, mul2(aq2, mul2(ti[q], lo, z), z));
+          a[q][it].hi = add2(a[q][it].hi, mul2(aq2, mul2(ti[q], hi, z), z));
         }
       }
     }
@@ -415,50 +437,48 @@ __device__ __noinline__ void apply_steps(Slab& s, const Link l, const LayerDev* 
   }
   if (smooth) {
     const float beta = L->beta, ob = 1.f - beta;
-    const int M = s.M;
     float* Qs = L->Qs;
 #pragma unroll
     for (int q = 0; q < 4 * NG; ++q) {
       const int i = s.row0 + 4 * (warp + CW * (q >> 2)) + (q & 3);
       if (i >= M) continue;
       float* row = Qs + (size_t)i * M;
-      if (V4) {
-#pragma unroll
-        for (int it = 0; it < IT; ++it) {
-          const int c = lane + 32 * it;
-          if (4 * c >= M) continue;
-          float4 o = reinterpret_cast<float4*>(row)[c];
-          o.x = fmaf(beta, o.x, ob * a[q][it].x); o.y = fmaf(beta, o.y, ob * a[q][it].y);
-          o.z = fmaf(beta, o.z, ob * a[q][it].z); o.w = fmaf(beta, o.w, ob * a[q][it].w);
-          reinterpret_cast<float4*>(row)[c] = o;
-        }
-      } else {
 #pragma unroll
       for (int it = 0; it < IT; ++it) {
         const int c = 4 * (lane + 32 * it);
-        if (c < M) row[c] = fmaf(beta, row[c], ob * a[q][it].x);
-        if (c + 1 < M) row[c + 1] = fmaf(beta, row[c + 1], ob * a[q][it].y);
-        if (c + 2 < M) row[c + 2] = fmaf(beta, row[c + 2], ob * a[q][it].z);
-        if (c + 3 < M) row[c + 3] = fmaf(beta, row[c + 3], ob * a[q][it].w);
-      }
+        if (c >= M) continue;
+        float4 r;
+        unpack2(a[q][it].lo, r.x, r.y);
+        unpack2(a[q][it].hi, r.z, r.w);
+        if (V4) {
+          float4 o = *reinterpret_cast<float4*>(row + c);
+          o.x = fmaf(beta, o.x, ob * r.x); o.y = fmaf(beta, o.y, ob * r.y);
+          o.z = fmaf(beta, o.z, ob * r.z); o.w = fmaf(beta, o.w, ob * r.w);
+          *reinterpret_cast<float4*>(row + c) = o;
+        } else {
+          row[c] = fmaf(beta, row[c], ob * r.x);
+          if (c + 1 < M) row[c + 1] = fmaf(beta, row[c + 1], ob * r.y);
+          if (c + 2 < M) row[c + 2] = fmaf(beta, row[c + 2], ob * r.z);
+          if (c + 3 < M) row[c + 3] = fmaf(beta, row[c + 3], ob * r.w);
+        }
       }
     }
   }
 }
 
-// Steps [k0, k1) of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane; from Phi_y in global
-// memory and back.
+// All steps of a launch for a warp that owns NG groups of four rows of IT float4 columns per lane; from Phi_y in global
+// memory and back.  tr: where the trace of the launch's first step goes, or null.
 template <int NG, int IT>
-__device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L, float* tr, int k0, int k1, int P,
-                                       bool last, uint32_t e) {
+__device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L, float* tr, int K, int P, bool last) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int slot = s.row0 + 4 * warp;       // the warp's first group in a result vector
   const uint32_t tx = s.tx;
-  float4 a[4 * NG][IT];
+  Quad a[4 * NG][IT];
   if ((s.M & 3) == 0) load_rows<NG, IT, true>(a, L->Phiy, s);
   else load_rows<NG, IT, false>(a, L->Phiy, s);
-  if (k0 == 0) sm100::cluster_wait();          // every CTA is ready to receive
-  for (int step = k0; step < k1; ++step) {
+  sm100::cluster_wait();                       // every CTA is ready to receive
+  uint32_t e = 0;                              // exchanges so far
+  for (int step = 0; step < K; ++step) {
     // S1: squared column norms (= row norms, Phi_y is exactly symmetric)             (Eq. 45)
     arm(l, e, tx);
     pass<PASS_SELF, NG, IT>(a, nullptr, 1.f, l, csm + s.xi2 + slot, e);
@@ -490,7 +510,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
     arm(l, e, tx);
     const float n2 = pass<PASS_UNIT, NG, IT>(a, x, sc, l, csm + s.uvec + slot, e);
     const float inv = inv_norm(n2);
-    float* vh = csm + s.vh + (step - k0) * s.Mv;
+    float* vh = csm + s.vh + step * s.Mv;
     wait_exchange(l, e, &s.fail); ++e;
     float l0 = 0.f, l1 = 0.f;
     const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -501,7 +521,7 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
       const float4 vv = make_float4(xv.x * sc * inv, xv.y * sc * inv, xv.z * sc * inv, xv.w * sc * inv);
       l0 = fmaf(vv.x, uv.x, l0); l1 = fmaf(vv.y, uv.y, l1);
       l0 = fmaf(vv.z, uv.z, l0); l1 = fmaf(vv.w, uv.w, l1);
-      if (warp == 0) reinterpret_cast<float4*>(vh)[lane + 32 * k] = vv;      // every CTA records the whole vector
+      if (warp == 0) reinterpret_cast<float4*>(vh)[lane + 32 * k] = vv;      // every CTA keeps the whole vector for T
     }
     const float lam_e = warp_sum(l0 + l1);
     // S6: g_e, a_e (Eqs. 40-41), rank update of Phi_y.  All warps of all CTAs sum in the same order, so they hold the
@@ -530,29 +550,34 @@ __device__ __noinline__ void run_steps(Slab& s, const Link l, const LayerDev* L,
         vj.x = vj.x * sc * inv; vj.y = vj.y * sc * inv; vj.z = vj.z * sc * inv; vj.w = vj.w * sc * inv;
         const u64 va = pack2(vj.x, vj.y), vb = pack2(vj.z, vj.w), ua = pack2(uj.x, uj.y), ub = pack2(uj.z, uj.w);
 #pragma unroll
-        for (int q = 0; q < 4 * NG; ++q) a[q][k] = rank2(a[q][k], vi[q], ui[q], va, vb, ua, ub, a2, l2, z);
-      }
-    }
-    if (threadIdx.x == 0) {
-      s.ah[step - k0] = aa;
-      if (s.sub == 0) {
-        if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
-        if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
-        if (tr) {
-          tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
-        }
-        if (last && step + 1 == k1) {
-          L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
-          L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
+        for (int q = 0; q < 4 * NG; ++q) {
+          a[q][k].lo = rank2(a[q][k].lo, vi[q], ui[q], va, ua, a2, l2, z);
+          a[q][k].hi = rank2(a[q][k].hi, vi[q], ui[q], vb, ub, a2, l2, z);
         }
       }
     }
+    if (threadIdx.x == 0) s.ah[step] = aa;
+    if (threadIdx.x == 0 && s.sub == 0) {
+      if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
+      if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
+      if (tr) {
+        tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
+      }
+      if (last && step + 1 == K) {
+        L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
+        L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
+      }
+    }
   }
-  if (!*(volatile int*)&s.fail) {
-    if ((s.M & 3) == 0) store_rows<NG, IT, true>(a, L->Phiy, s);
-    else store_rows<NG, IT, false>(a, L->Phiy, s);
+  rows_sync(l);                                // v_e and a_e of the steps
+  const bool smooth = last && L->Qs != L->Q;
+  if ((s.M & 3) == 0) {
+    if (!*(volatile int*)&s.fail) store_rows<NG, IT, true>(a, L->Phiy, s);
+    apply_steps<NG, IT, true>(s, l, L, K, smooth);
+  } else {
+    if (!*(volatile int*)&s.fail) store_rows<NG, IT, false>(a, L->Phiy, s);
+    apply_steps<NG, IT, false>(s, l, L, K, smooth);
   }
-  rows_sync(l);         // ah and vh for apply_steps
 }
 
 // ---- layers of at most 64 features: one CTA, a row on 8 lanes ----
@@ -565,7 +590,7 @@ __device__ __forceinline__ float row_sum(float x) {
   for (int o = LPR / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
 }
-__device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int K, int P, bool smooth) {
+__device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int K, int P, bool last) {
   constexpr int KM = 64 / (4 * LPR);             // float4 per lane
   const int tid = threadIdx.x, row = tid / LPR, sub = tid % LPR;
   const int M = s.M;
@@ -631,153 +656,149 @@ __device__ __noinline__ void run_solo(Slab& s, const LayerDev* L, float* tr, int
     if (mode == PASS_NORM) n2 = row_sum(n2);
     return n2;
   };
-  for (int k0 = 0; k0 < K; k0 += KH) {
-    const int k1 = min(K, k0 + KH);
-    for (int step = k0; step < k1; ++step) {
-      // squared norms (Eq. 45), m' (Eq. 46): every warp finds it for itself
-      float q0 = four(a[0], a[0]);
+  for (int step = 0; step < K; ++step) {
+    // squared norms (Eq. 45), m' (Eq. 46): every warp finds it for itself
+    float q0 = four(a[0], a[0]);
 #pragma unroll
-      for (int k = 1; k < KM; ++k) q0 += four(a[k], a[k]);
-      q0 = row_sum(q0);
-      if (sub == 0) csm[s.xi2 + row] = q0;
-      __syncthreads();
-      const int mp = argmax_xi(s);
-      if (row == mp) {
-#pragma unroll
-        for (int k = 0; k < KM; ++k) reinterpret_cast<float4*>(csm + s.wvec)[sub + LPR * k] = a[k];
-      }
-      __syncthreads();
-      dot(csm + s.wvec, 1.f, PASS_SCALE, csm + s.cvec);                       // Eq. 47
-      __syncthreads();
-      // coherent set, aligned average (Eqs. 48-49)
-      int cnt = 1;
-      {
-        float wv = 0.f;
-        bool in = false;
-        if (s.maxcol) {
-          wv = tid == mp ? 1.f : 0.f;
-        } else if (tid < M) {
-          const float c = csm[s.cvec + tid];
-          const float thr = fmaxf(s.c_rel * sqrtf(csm[s.xi2 + mp]) * sqrtf(csm[s.xi2 + tid]), s.c_abs);
-          in = fabsf(c) >= thr;       // false for NaN
-          wv = in ? (1.f / c) : 0.f;
-        }
-        if (tid < 64) csm[s.wvec + tid] = wv;
-        const int n = __syncthreads_count(in);
-        if (!s.maxcol) cnt = n;
-      }
-      int xo = s.buf0, yo = xo + s.Mv;
-      dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, PASS_SCALE, csm + xo);
-      __syncthreads();
-      float sc = 1.f;                                                         // x is sc times the vector at xo
-      for (int p = 0; p < P; ++p) {
-        const float n2 = dot(csm + xo, sc, PASS_NORM, csm + yo);
-        __syncthreads();
-        sc = inv_norm(n2);
-        const int t = xo; xo = yo; yo = t;
-      }
-      const float n2 = dot(csm + xo, sc, PASS_UNIT, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
-      const float inv = inv_norm(n2);
-      __syncthreads();
-      const float4* x4 = reinterpret_cast<const float4*>(csm + xo);
-      const float4* u4 = reinterpret_cast<const float4*>(csm + s.uvec);
-      float l0 = 0.f;
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        float4 x = x4[sub + LPR * k];
-        x.x = x.x * sc * inv; x.y = x.y * sc * inv; x.z = x.z * sc * inv; x.w = x.w * sc * inv;
-        l0 = k ? l0 + four(x, u4[sub + LPR * k]) : four(x, u4[sub + LPR * k]);
-      }
-      const float lam_e = row_sum(l0);                              // Eq. 36
-      const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
-      float g_e = 1.f, aa = 0.f;
-      if (ok) {
-        g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);                 // Eqs. 40-41
-        aa = sqrtf(g_e) - 1.f;
-      }
-      // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T, as in run_steps
-      if (aa != 0.f) {
-        const float v = csm[xo + row] * sc * inv, u = csm[s.uvec + row], l = aa * aa * lam_e;
-#pragma unroll
-        for (int k = 0; k < KM; ++k) {
-          float4 vj = x4[sub + LPR * k];
-          const float4 uj = u4[sub + LPR * k];
-          vj.x = vj.x * sc * inv; vj.y = vj.y * sc * inv; vj.z = vj.z * sc * inv; vj.w = vj.w * sc * inv;
-          a[k] = rank2(a[k], pack2(v, v), pack2(u, u), pack2(vj.x, vj.y), pack2(vj.z, vj.w), pack2(uj.x, uj.y), pack2(uj.z, uj.w),
-                       pack2(aa, aa), pack2(l, l), pack2(s.negz, s.negz));
-        }
-      }
-      if (tid < 64) csm[s.vh + (step - k0) * s.Mv + tid] = csm[xo + tid] * sc * inv;
-      if (tid == 0) {
-        s.ah[step - k0] = aa;
-        if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
-        if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
-        if (tr) {
-          tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
-        }
-        if (step + 1 == K) {
-          L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
-          L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
-        }
-      }
-      __syncthreads();
-    }
-    // ---- the recorded steps in T, then Q (Eqs. 42, 44), as in apply_steps ----
-    const bool last = k1 == K;
-    float4 t[KM], o[KM];
-    load(t, L->Tt);
-#pragma unroll 1
-    for (int j = 0; j < k1 - k0; ++j) {
-      const float ak = s.ah[j];
-      if (ak == 0.f) continue;
-      const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + j * s.Mv);
-      float d = four(t[0], v4[sub]);
-#pragma unroll
-      for (int k = 1; k < KM; ++k) d += four(t[k], v4[sub + LPR * k]);
-      d = row_sum(d);
-      const float at = ak * d;
-      if (sub == 0) csm[s.th + j * s.Mv + row] = d;
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        const float4 b = v4[sub + LPR * k];
-        t[k].x = fmaf(at, b.x, t[k].x); t[k].y = fmaf(at, b.y, t[k].y); t[k].z = fmaf(at, b.z, t[k].z); t[k].w = fmaf(at, b.w, t[k].w);
-      }
-    }
-    save(t, L->Tt);
-    if (L->round_t) {                    // rows of whole float4s
-#pragma unroll
-      for (int k = 0; k < KM; ++k)
-        o[k] = make_float4(sm100::tf32_rna(t[k].x), sm100::tf32_rna(t[k].y), sm100::tf32_rna(t[k].z), sm100::tf32_rna(t[k].w));
-      save(o, L->tmp);
-    }
-    load(t, L->Q);
+    for (int k = 1; k < KM; ++k) q0 += four(a[k], a[k]);
+    q0 = row_sum(q0);
+    if (sub == 0) csm[s.xi2 + row] = q0;
     __syncthreads();
-#pragma unroll 1
-    for (int j = 0; j < k1 - k0; ++j) {
-      const float ak = s.ah[j];
-      if (ak == 0.f) continue;
-      const float aq = ak * (ak + 2.f), ti = csm[s.th + j * s.Mv + row];
-      const float4* t4 = reinterpret_cast<const float4*>(csm + s.th + j * s.Mv);
+    const int mp = argmax_xi(s);
+    if (row == mp) {
+#pragma unroll
+      for (int k = 0; k < KM; ++k) reinterpret_cast<float4*>(csm + s.wvec)[sub + LPR * k] = a[k];
+    }
+    __syncthreads();
+    dot(csm + s.wvec, 1.f, PASS_SCALE, csm + s.cvec);                       // Eq. 47
+    __syncthreads();
+    // coherent set, aligned average (Eqs. 48-49)
+    int cnt = 1;
+    {
+      float wv = 0.f;
+      bool in = false;
+      if (s.maxcol) {
+        wv = tid == mp ? 1.f : 0.f;
+      } else if (tid < M) {
+        const float c = csm[s.cvec + tid];
+        const float thr = fmaxf(s.c_rel * sqrtf(csm[s.xi2 + mp]) * sqrtf(csm[s.xi2 + tid]), s.c_abs);
+        in = fabsf(c) >= thr;       // false for NaN
+        wv = in ? (1.f / c) : 0.f;
+      }
+      if (tid < 64) csm[s.wvec + tid] = wv;
+      const int n = __syncthreads_count(in);
+      if (!s.maxcol) cnt = n;
+    }
+    int xo = s.buf0, yo = xo + s.Mv;
+    dot(csm + s.wvec, cnt > 0 ? 1.f / (float)cnt : 0.f, PASS_SCALE, csm + xo);
+    __syncthreads();
+    float sc = 1.f;                                                         // x is sc times the vector at xo
+    for (int p = 0; p < P; ++p) {
+      const float n2 = dot(csm + xo, sc, PASS_NORM, csm + yo);
+      __syncthreads();
+      sc = inv_norm(n2);
+      const int t = xo; xo = yo; yo = t;
+    }
+    const float n2 = dot(csm + xo, sc, PASS_UNIT, csm + s.uvec);           // u = Phi_y v, v = x / ||x|| (Eq. 50)
+    const float inv = inv_norm(n2);
+    __syncthreads();
+    const float4* x4 = reinterpret_cast<const float4*>(csm + xo);
+    const float4* u4 = reinterpret_cast<const float4*>(csm + s.uvec);
+    float l0 = 0.f;
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      float4 x = x4[sub + LPR * k];
+      x.x = x.x * sc * inv; x.y = x.y * sc * inv; x.z = x.z * sc * inv; x.w = x.w * sc * inv;
+      l0 = k ? l0 + four(x, u4[sub + LPR * k]) : four(x, u4[sub + LPR * k]);
+    }
+    const float lam_e = row_sum(l0);                              // Eq. 36
+    const bool ok = cnt > 0 && n2 > 0.f && isfinite(n2) && isfinite(lam_e);
+    float g_e = 1.f, aa = 0.f;
+    if (ok) {
+      g_e = s.delta * s.lam_bar / fmaxf(lam_e, s.eps);                 // Eqs. 40-41
+      aa = sqrtf(g_e) - 1.f;
+    }
+    // Phi_y += a (v u^T + u v^T) + a^2 lambda_e v v^T, as in run_steps
+    if (aa != 0.f) {
+      const float v = csm[xo + row] * sc * inv, u = csm[s.uvec + row], l = aa * aa * lam_e;
 #pragma unroll
       for (int k = 0; k < KM; ++k) {
-        const float4 b = t4[sub + LPR * k];
-        t[k].x = __fadd_rn(t[k].x, __fmul_rn(aq, __fmul_rn(ti, b.x))); t[k].y = __fadd_rn(t[k].y, __fmul_rn(aq, __fmul_rn(ti, b.y)));
-        t[k].z = __fadd_rn(t[k].z, __fmul_rn(aq, __fmul_rn(ti, b.z))); t[k].w = __fadd_rn(t[k].w, __fmul_rn(aq, __fmul_rn(ti, b.w)));
+        float4 vj = x4[sub + LPR * k];
+        const float4 uj = u4[sub + LPR * k];
+        vj.x = vj.x * sc * inv; vj.y = vj.y * sc * inv; vj.z = vj.z * sc * inv; vj.w = vj.w * sc * inv;
+        a[k] = rank2(a[k], pack2(v, v), pack2(u, u), pack2(vj.x, vj.y), pack2(vj.z, vj.w), pack2(uj.x, uj.y), pack2(uj.z, uj.w),
+                     pack2(aa, aa), pack2(l, l), pack2(s.negz, s.negz));
       }
     }
-    save(t, L->Q);
-    if (last && smooth) {
-      const float beta = L->beta, ob = 1.f - beta;
-      load(o, L->Qs);
-#pragma unroll
-      for (int k = 0; k < KM; ++k) {
-        o[k].x = fmaf(beta, o[k].x, ob * t[k].x); o[k].y = fmaf(beta, o[k].y, ob * t[k].y);
-        o[k].z = fmaf(beta, o[k].z, ob * t[k].z); o[k].w = fmaf(beta, o[k].w, ob * t[k].w);
+    if (tid < 64) csm[s.vh + step * s.Mv + tid] = csm[xo + tid] * sc * inv;
+    if (tid == 0) {
+      s.ah[step] = aa;
+      if (!ok) L->iscal[IS_STATUS_NOSUB] = 1;
+      if (!isfinite(n2) || !isfinite(lam_e)) L->iscal[IS_STATUS_NONFINITE] = 1;
+      if (tr) {
+        tr[4 * step] = lam_e; tr[4 * step + 1] = g_e; tr[4 * step + 2] = (float)cnt; tr[4 * step + 3] = (float)mp;
       }
-      save(o, L->Qs);
+      if (last && step + 1 == K) {
+        L->scal[SC_LAMBDA_E] = lam_e; L->scal[SC_G_E] = g_e; L->scal[SC_A_E] = aa;
+        L->iscal[IS_MPRIME] = mp; L->iscal[IS_SETSIZE] = cnt;
+      }
     }
     __syncthreads();
   }
+  // ---- the recorded steps in T, then Q (Eqs. 42, 44), as in apply_steps ----
+  float4 t[KM], o[KM];
+  load(t, L->Tt);
+#pragma unroll 1
+  for (int j = 0; j < K; ++j) {
+    const float ak = s.ah[j];
+    if (ak == 0.f) continue;
+    const float4* v4 = reinterpret_cast<const float4*>(csm + s.vh + j * s.Mv);
+    float d = four(t[0], v4[sub]);
+#pragma unroll
+    for (int k = 1; k < KM; ++k) d += four(t[k], v4[sub + LPR * k]);
+    d = row_sum(d);
+    const float at = ak * d;
+    if (sub == 0) csm[s.th + j * s.Mv + row] = d;
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      const float4 b = v4[sub + LPR * k];
+      t[k].x = fmaf(at, b.x, t[k].x); t[k].y = fmaf(at, b.y, t[k].y); t[k].z = fmaf(at, b.z, t[k].z); t[k].w = fmaf(at, b.w, t[k].w);
+    }
+  }
+  save(t, L->Tt);
+  if (L->round_t) {                    // rows of whole float4s
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      o[k] = make_float4(sm100::tf32_rna(t[k].x), sm100::tf32_rna(t[k].y), sm100::tf32_rna(t[k].z), sm100::tf32_rna(t[k].w));
+    save(o, L->tmp);
+  }
+  load(t, L->Q);
+  __syncthreads();
+#pragma unroll 1
+  for (int j = 0; j < K; ++j) {
+    const float ak = s.ah[j];
+    if (ak == 0.f) continue;
+    const float aq = ak * (ak + 2.f), ti = csm[s.th + j * s.Mv + row];
+    const float4* t4 = reinterpret_cast<const float4*>(csm + s.th + j * s.Mv);
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      const float4 b = t4[sub + LPR * k];
+      t[k].x = __fadd_rn(t[k].x, __fmul_rn(aq, __fmul_rn(ti, b.x))); t[k].y = __fadd_rn(t[k].y, __fmul_rn(aq, __fmul_rn(ti, b.y)));
+      t[k].z = __fadd_rn(t[k].z, __fmul_rn(aq, __fmul_rn(ti, b.z))); t[k].w = __fadd_rn(t[k].w, __fmul_rn(aq, __fmul_rn(ti, b.w)));
+    }
+  }
+  save(t, L->Q);
+  if (last && L->Qs != L->Q) {            // Eq. 35
+    const float beta = L->beta, ob = 1.f - beta;
+    load(o, L->Qs);
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+      o[k].x = fmaf(beta, o[k].x, ob * t[k].x); o[k].y = fmaf(beta, o[k].y, ob * t[k].y);
+      o[k].z = fmaf(beta, o[k].z, ob * t[k].z); o[k].w = fmaf(beta, o[k].w, ob * t[k].w);
+    }
+    save(o, L->Qs);
+  }
+  __syncthreads();
   save(a, L->Phiy);
 }
 
@@ -794,17 +815,6 @@ __host__ __device__ inline int slab_vec(int M, int n) {
   return a > b ? a : b;
 }
 constexpr int kVecs = 6 + 2 * KH;
-// one CTA with a row on 8 lanes
-__host__ __device__ inline bool solo(int M, int n) { return n == 1 && M <= 64; }
-
-template <int NG, int IT>
-__device__ __forceinline__ void run_chunk(Slab& s, const Link& l, const LayerDev* L, float* tr, int k0, int k1, int P,
-                                          bool last, bool smooth, uint32_t e) {
-  run_steps<NG, IT>(s, l, L, tr, k0, k1, P, last, e);
-  e += (uint32_t)(k1 - k0) * (uint32_t)(P + 5);
-  if ((s.M & 3) == 0) apply_steps<NG, IT, true>(s, l, L, k1 - k0, smooth, e);
-  else apply_steps<NG, IT, false>(s, l, L, k1 - k0, smooth, e);
-}
 
 __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
   dep_sync();
@@ -822,12 +832,12 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     return;
   }
   const LayerDev* L = a.g.layer[layer];
-  __shared__ __align__(8) uint64_t xbar[2];
+  __shared__ __align__(8) uint64_t xbar[3];
   __shared__ Slab s;
   Link l;
   l.n = a.ncta[layer];
   l.active = 0;
-  l.bar0 = smem_u32(&xbar[0]);                       // the two barriers are 8 bytes apart
+  l.bar0 = smem_u32(&xbar[0]);                       // the three barriers are 8 bytes apart
   if (threadIdx.x == 0) {
     const int M = L->M, n = l.n;
     s.M = M; s.Mp = (M + 3) & ~3; s.R = slab_rows(M, n); s.n = n;
@@ -844,6 +854,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     s.fail = 0; s.negz = -0.f;
     sm100::mbar_init(l.bar0, 1);
     sm100::mbar_init(l.bar0 + 8, 1);
+    sm100::mbar_init(l.bar0 + 16, 1);
     sm100::mbar_fence_init();
   }
   __syncthreads();
@@ -852,7 +863,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
 
   // what no exchange fills of the vectors stays zero (rows past the matrix are zero rows)
   const int filled = l.n * R, tail = s.Mv - filled;
-  for (int i = threadIdx.x; i < kVecs * tail; i += CT) csm[i / tail * s.Mv + filled + i % tail] = 0.f;
+  for (int i = threadIdx.x; i < kVecs * tail; i += CT) csm[s.xi2 + i / tail * s.Mv + filled + i % tail] = 0.f;
   // A CTA's window of the cluster address space is this CTA's window shifted by a constant; the stores rely on it,
   // so it is checked on two addresses far apart before anything is sent.
   const uint32_t peer_rank = (uint32_t)(rank - s.sub + min(lane, l.n - 1));
@@ -861,35 +872,27 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
   const bool usable = __syncthreads_or(!linear) == 0;
   sm100::cluster_arrive();   // every barrier is initialised before the first remote store can arrive: waited for in run_steps
 
-  const int ng = solo(M, l.n) ? 0 : warp_groups(R);
+  const int ng = M <= kSolo ? 0 : warp_groups(R), it = slab_trips(M);
   if (!usable || ng == 0 || a.K < 1) sm100::cluster_wait();
-  if (usable) {
+  if (usable && a.K > 0) {
     float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
-    if (solo(M, l.n)) {
-      const bool smooth = L->Qs != L->Q;
-      run_solo(s, L, tr, a.K, a.P, smooth);
-    } else {
-    const int it = slab_trips(M);
-    uint32_t e = 0;                        // exchanges so far
-    for (int k0 = 0; k0 < a.K; k0 += KH) {
-      const int k1 = min(a.K, k0 + KH);
-      const bool last = k1 == a.K, smooth = last && L->Qs != L->Q;
-      if (ng == 1) {
-        switch (it) {
-          case 1: run_chunk<1, 1>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-          case 2: run_chunk<1, 2>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-          case 3: run_chunk<1, 3>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-          case 4: run_chunk<1, 4>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-          default: run_chunk<1, 5>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-        }
-      } else if (ng == 2) {
-        switch (it) {
-          case 1: run_chunk<2, 1>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-          default: run_chunk<2, 2>(s, l, L, tr, k0, k1, a.P, last, smooth, e); break;
-        }
+    if (tr) tr += 4 * a.k0;
+    const bool last = a.last != 0;
+    if (M <= kSolo) {
+      run_solo(s, L, tr, a.K, a.P, last);
+    } else if (ng == 1) {
+      switch (it) {
+        case 1: run_steps<1, 1>(s, l, L, tr, a.K, a.P, last); break;
+        case 2: run_steps<1, 2>(s, l, L, tr, a.K, a.P, last); break;
+        case 3: run_steps<1, 3>(s, l, L, tr, a.K, a.P, last); break;
+        case 4: run_steps<1, 4>(s, l, L, tr, a.K, a.P, last); break;
+        default: run_steps<1, 5>(s, l, L, tr, a.K, a.P, last); break;
       }
-      e += (uint32_t)(k1 - k0) * (uint32_t)(a.P + 5) + 1u;
-    }
+    } else if (ng == 2) {
+      switch (it) {
+        case 1: run_steps<2, 1>(s, l, L, tr, a.K, a.P, last); break;
+        default: run_steps<2, 2>(s, l, L, tr, a.K, a.P, last); break;
+      }
     }
   }
   __syncthreads();
@@ -916,7 +919,7 @@ bool cluster_fits(int M, int n) {
 // the work of the busiest of the four SM partitions, and the fixed part of an exchange (less within one CTA).
 int cluster_cost(int M, int n) {
   const int groups = slab_rows(M, n) / 4;
-  if (solo(M, n)) return 4;
+  if (M <= kSolo) return 4;         // one CTA, and no gain from more
   return ((groups + 3) / 4) * slab_trips(M) + (n > 1 ? 20 : 8);
 }
 
@@ -990,8 +993,9 @@ int recursion_cluster_ctas(int M) {
 
 bool recursion_cluster_supported(int M) { return recursion_cluster_ctas(M) > 0; }
 
-cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
-                                     cudaStream_t s) {
+cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
+                                     bool last, cudaStream_t s) {
+  if (K < 1 || K > KH) return cudaErrorInvalidValue;
   static SmemAttrCache attr;
   static std::mutex mu;
   static int resident[64][5];        // clusters of 1, 2, 4, 8, 16 CTAs that run together (16: 7 on a B200)
@@ -1046,7 +1050,7 @@ cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, 
   }
   ClusterArgs a;
   memset(&a, 0, sizeof(a));
-  a.g = g; a.traces = traces; a.K = K; a.P = P;
+  a.g = g; a.traces = traces; a.k0 = k0; a.K = K; a.P = P; a.last = last ? 1 : 0;
   size_t smem = 0;
   for (int i = 0; i < g.n; ++i) {
     a.first_cta[i] = plan.first[i]; a.ncta[i] = plan.cnt[i];
