@@ -114,13 +114,6 @@ __device__ __forceinline__ float4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-// the first n of four neighbouring entries
-__device__ __forceinline__ void store4(float* p, const float (&v)[4], int n) {
-  if (n >= 4) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-  else
-    for (int e = 0; e < n; ++e) p[e] = v[e];
-}
-
 template <bool BF>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GP_THREADS, 1)
 gram_pair_kernel(const __grid_constant__ PairGroup g) {
@@ -476,6 +469,10 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) rr[j] = 0u;
             }
+            if (!BF && pr.round_out) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(tf32_rna(__uint_as_float(rr[j])));
+            }
             const int col = cb + c0;
             if (pr.full == 2) {
               // symmetric output: (row, c) for c >= row and its mirror image (c, row) for c > row
@@ -503,10 +500,14 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
             } else if (row < M) {
 #pragma unroll
               for (int j = 0; j < 16; j += 4) {
-                float v[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = pr.round_out ? tf32_rna(__uint_as_float(rr[j + e])) : __uint_as_float(rr[j + e]);
-                store4(P + (int64_t)row * M + col + j, v, M - col - j);
+                if (col + j + 3 < M) {
+                  *reinterpret_cast<float4*>(P + (int64_t)row * M + col + j) =
+                      make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]), __uint_as_float(rr[j + 2]),
+                                  __uint_as_float(rr[j + 3]));
+                } else {
+                  for (int jj = j; jj < j + 4; ++jj)
+                    if (col + jj < M) P[(int64_t)row * M + col + jj] = __uint_as_float(rr[jj]);
+                }
               }
             }
           }
