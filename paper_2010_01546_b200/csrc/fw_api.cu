@@ -745,7 +745,9 @@ static fw_status grad_transform_impl(fw_layer* const* L, int32_t n, const float*
     }
     // longest K first: items start in list order
     std::stable_sort(items.begin(), items.end(), [](const UmmaGqItem& a, const UmmaGqItem& b) { return a.M > b.M; });
-    fw_status st = umma_gq_pair_launch(items.data(), (int)items.size(), epi, lr, FW_PROF_GQ, s);
+    const fw_status st = gq_small_eligible(items.data(), (int)items.size())
+                             ? gq_small_launch(items.data(), (int)items.size(), epi, lr, FW_PROF_GQ, s)
+                             : umma_gq_pair_launch(items.data(), (int)items.size(), epi, lr, FW_PROF_GQ, s);
     if (st != FW_OK) return st;
   }
   return FW_OK;

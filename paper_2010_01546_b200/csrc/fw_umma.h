@@ -31,6 +31,9 @@ struct UmmaGqItem {
 // out = G Qs on CTA pairs (256 x 256 tiles, K split with a fixed-order reduction); M a multiple of 4, >= 16
 bool umma_gq_pair_supported(int M);
 fw_status umma_gq_pair_launch(const UmmaGqItem* items, int n, int epi, float lr, int prof_class, cudaStream_t s);
+// The same for small layers, latency instead of rate: tiles of 64 x 32 with K shared by a cluster (fw_gq_small.cu)
+bool gq_small_eligible(const UmmaGqItem* items, int n);
+fw_status gq_small_launch(const UmmaGqItem* items, int n, int epi, float lr, int prof_class, cudaStream_t s);
 // K-major fp32 operand: 2-D row-major [outer][inner] tensor, boxes of box_inner (32) floats x box_outer rows,
 // 128-byte swizzle
 bool tmap_encode_kmajor_f32(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t ld,
