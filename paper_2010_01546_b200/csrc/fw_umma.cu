@@ -243,11 +243,6 @@ __device__ __forceinline__ float4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
-// shared -> global memory, both 16-byte aligned, bytes a multiple of 16
-__device__ __forceinline__ void bulk_store(float* dst, const float* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
-}
-
 // BF = true: bf16 X (kind::f16), BF = false: fp32 X (kind::tf32).  All per-stage
 // loops are free of divisions and descriptor rebuilding: the single issuing
 // threads of the producer and MMA warps run serial code, so every instruction in

@@ -139,6 +139,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
   __shared__ __align__(8) uint64_t bar_full[GP_MAX_STAGES], bar_ready[GP_MAX_STAGES], bar_empty[GP_MAX_STAGES], bar_accum;
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_flag;
+  __shared__ int s_store;
   __shared__ int s_I, s_cbase, s_n0, s_n1, s_ngroups, s_bgroup, s_pass, s_cs, s_tmem_cols, s_skip;
   __shared__ int s_gcol[GP_MAX_GROUPS], s_gsrc[GP_MAX_GROUPS], s_gchunks[GP_MAX_GROUPS];
   __shared__ float s_csred[GP_FIX_WARPS][GP_GCOLS];
@@ -449,72 +450,74 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
         if (col0 + i < M) cs_out[col0 + i] = t;
       }
     }
-    // ---- epilogue: this CTA's 128 rows of both accumulators -> partial output ----
-    if (ok) {
+    // ---- epilogue: this CTA's 128 rows of both accumulators -> partial output, 128 columns at a time through shared memory (the
+    //      stages are free: every MMA has completed) and on as one bulk copy a row, while the next columns are read.  Stores
+    //      from the registers, where a lane is a row, took 14 us for 512 columns.  The mirror image of a symmetric product does
+    //      leave from the registers: there the lanes are neighbours in an output row.  The verdict of the waits is made
+    //      common first: the barriers below are taken by all eight warps or by none. ----
+    const bool have = nk > 0;
+    if (ok && have && !mbar_wait(smem_u32(&bar_accum), 0, abortp)) GP_ABORT(304);
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (threadIdx.x == 64) s_store = *abortp == 0;
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (s_store) {
+      tc_fence_after();
       float* P = pr.out + (int64_t)split * M * M;
-      const bool have = nk > 0;
-      if (!have || mbar_wait(smem_u32(&bar_accum), 0, abortp)) {
-        tc_fence_after();
-        const int q = warp & 3, half = w >> 2;
-        const int row = 256 * s_I + 128 * (int)rank + q * 32 + lane;
-        for (int o = 0; o < 2; ++o) {
-          const int n = o ? s_n1 : s_n0;
-          const int cb = s_cbase + 256 * o;
-          for (int c0 = 16 * half; c0 < n; c0 += 32) {
-            uint32_t rr[16];
-            if (have) {
-              tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(256 * o + c0), rr);
-              tmem_ld_wait();
-            } else {
+      constexpr int EC = 128, TS = EC + 4;         // columns of a piece, row pitch in floats: rows on distinct banks
+      float* const room = reinterpret_cast<float*>(smem_raw) + ((smem_base - smem_u32(smem_raw)) >> 2);
+      const int q = warp & 3, half = w >> 2, first = 256 * s_I + 128 * (int)rank;
+      const int row = first + q * 32 + lane, n = s_n0 + s_n1;
+      const int r = (int)threadIdx.x - 64, rrow = first + r;                // the row whose copies this thread issues
+      for (int cc = 0, piece = 0; cc < n; cc += EC) {
+        const int col0 = s_cbase + cc, width = min(EC, n - cc);
+        // symmetric output: (row, c) for c >= row and its mirror image; pieces below the diagonal are other tiles' images
+        if (pr.full == 2 && col0 + width <= first) continue;
+        const bool whole = pr.full != 2 || col0 >= first + 128;
+        float* tile = room + (piece & 1) * 128 * TS;
+        if (piece >= 2) {
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          asm volatile("bar.sync 1, 256;" ::: "memory");
+        }
+        ++piece;
+        float* trow = tile + (q * 32 + lane) * TS;
+        for (int c0 = 16 * half; c0 < width; c0 += 32) {
+          uint32_t rr[16];
+          if (have) {
+            tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(cc + c0), rr);
+            tmem_ld_wait();
+          } else {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) rr[j] = 0u;
-            }
-            if (!BF && pr.round_out) {
+            for (int j = 0; j < 16; ++j) rr[j] = 0u;
+          }
+          if (!BF && pr.round_out) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(tf32_rna(__uint_as_float(rr[j])));
-            }
-            const int col = cb + c0;
-            if (pr.full == 2) {
-              // symmetric output: (row, c) for c >= row and its mirror image (c, row) for c > row
-              if (row < M && col + 15 >= row) {
-                if (col > row && col + 15 < M) {
-                  // wholly above the diagonal: the direct stores go out as 16-byte vectors
+            for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(tf32_rna(__uint_as_float(rr[j])));
+          }
+          const int col = col0 + c0;
+          if (whole) {
 #pragma unroll
-                  for (int j = 0; j < 16; j += 4)
-                    *reinterpret_cast<float4*>(P + (int64_t)row * M + col + j) =
-                        make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]), __uint_as_float(rr[j + 2]),
-                                    __uint_as_float(rr[j + 3]));
+            for (int j = 0; j < 16; j += 4)
+              *reinterpret_cast<float4*>(trow + c0 + j) = make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]),
+                                                                      __uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3]));
+          }
+          if (pr.full == 2 && row < M) {
 #pragma unroll
-                  for (int j = 0; j < 16; ++j) P[(int64_t)(col + j) * M + row] = __uint_as_float(rr[j]);
-                } else {
-#pragma unroll
-                  for (int j = 0; j < 16; ++j) {
-                    const int c = col + j;
-                    if (c < M && c >= row) {
-                      P[(int64_t)row * M + c] = __uint_as_float(rr[j]);
-                      if (c > row) P[(int64_t)c * M + row] = __uint_as_float(rr[j]);
-                    }
-                  }
-                }
-              }
-            } else if (row < M) {
-#pragma unroll
-              for (int j = 0; j < 16; j += 4) {
-                if (col + j + 3 < M) {
-                  *reinterpret_cast<float4*>(P + (int64_t)row * M + col + j) =
-                      make_float4(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1]), __uint_as_float(rr[j + 2]),
-                                  __uint_as_float(rr[j + 3]));
-                } else {
-                  for (int jj = j; jj < j + 4; ++jj)
-                    if (col + jj < M) P[(int64_t)row * M + col + jj] = __uint_as_float(rr[jj]);
-                }
-              }
+            for (int j = 0; j < 16; ++j) {
+              const int c = col + j;
+              if (c >= M || c < row) continue;
+              if (!whole) P[(int64_t)row * M + c] = __uint_as_float(rr[j]);
+              if (c > row) P[(int64_t)c * M + row] = __uint_as_float(rr[j]);
             }
           }
         }
-      } else {
-        GP_ABORT(304);
+        fence_proxy_async_smem();                  // written by ordinary stores -> the bulk copies' reads
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (r < 128) {
+          if (whole && rrow < M && col0 < M) bulk_store(P + (int64_t)rrow * M + col0, tile + r * TS, (uint32_t)min(width, M - col0) * 4u);
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
       }
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");        // no thread leaves before its copies have read
     }
   }
 #undef GP_ABORT
