@@ -280,7 +280,7 @@ def peaks():
 # profiles/ (not measured in this run: `traffic_source` names the file); a kernel changed since its capture has
 # no entry here and reports null.
 NCU_TRAFFIC = {
-    ("resnet20", "gram"): (660.70e6 + 16.17e6, "profiles/gram_umma_kernel_resnet20.md"),
+    ("resnet20", "gram"): (660.69e6 + 16.34e6, "profiles/counters_recursion_products.md"),
 }
 # cost-sweep layer: TF32 Gram pass captured at B = 256 (50176 rows): bytes read, bytes written; the reads are
 # proportional to the rows
