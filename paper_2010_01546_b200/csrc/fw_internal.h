@@ -180,6 +180,10 @@ struct GemmGroup {
 __device__ __forceinline__ void dep_sync() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
+// The two halves, for a kernel and its dependent that share a predecessor: a kernel that waits first and triggers then lets its
+// dependent start on what the predecessor left (it has completed, and its writes are visible), before it waits itself.
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The launchers report what their launches returned, not the thread's last error: that may be of an earlier call, and it is the
 // caller's to read.
 template <class T> struct SameType { using type = T; };

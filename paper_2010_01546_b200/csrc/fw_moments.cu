@@ -73,6 +73,7 @@ struct MomentArgs {
                                      // 0 = overwrite the accumulators, 1 = add to them)
   float corr[FW_MAX_GROUP];          // > 0: corr c c^T was taken out of this call's Gram sums (c = rounded pmean)
   TileTable tt;                      // flat grid over the upper-triangle 32x32 tiles of all layers
+  int32_t early;                     // moments_mat_kernel adds its partial sums while moments_vec_kernel runs
   int32_t bias_blocks;               // CTAs per layer placed before the tiles for b += W (mu_new - mu_old); 0: none
 };
 
@@ -95,7 +96,8 @@ __device__ __forceinline__ void split_sums(const float* cp, const float* gp, int
 __global__ void __launch_bounds__(1024) moments_vec_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a) {
-  dep_sync();
+  if (a.early) { dep_wait(); dep_trigger(); }         // the Gram pass has completed: moments_mat_kernel may add its partial sums
+  else dep_sync();
   const LayerDev* L = g.layer[blockIdx.x];
   const int M = L->M;
   const int S = a.splits[blockIdx.x];
@@ -192,7 +194,8 @@ __device__ __forceinline__ void store_quad(float* p, int j, int M, float4 v) {
 __device__ __forceinline__ void bias_comp_rows(const LayerDev* L, const float* Wp, float* bp, int blk, int tid);
 
 // One 32 x 32 tile (bi <= bj) of one layer, a thread four entries of a row; the mirror image leaves through shared memory.
-template <bool V4>
+// EARLY: the partial sums before the wait for moments_vec_kernel.
+template <bool V4, bool EARLY>
 __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs& a, int li, float inv_rows, int bi, int bj,
                                              float (&tile)[32][33]) {
   const int M = L->M, S = a.splits[li], tid = threadIdx.x;
@@ -203,8 +206,13 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
   if (i < M && j < M) {
     const int64_t off = (int64_t)i * M + j, MM = (int64_t)M * M;
     const float4 old = first ? make_float4(0.f, 0.f, 0.f, 0.f) : load_quad<V4>(L->Phix + off, j, M);
-    const float mh_i = L->pv[0][i], nu_i = L->pv[1][i];           // batch mean - shift, new running mean - shift
-    const float4 mh_j = load_quad<V4>(L->pv[0] + j, j, M), nu_j = load_quad<V4>(L->pv[1] + j, j, M);
+    float mh_i, nu_i;                                             // batch mean - shift, new running mean - shift
+    float4 mh_j, nu_j;
+    auto means = [&] {
+      mh_i = L->pv[0][i]; nu_i = L->pv[1][i];
+      mh_j = load_quad<V4>(L->pv[0] + j, j, M); nu_j = load_quad<V4>(L->pv[1] + j, j, M);
+    };
+    if (!EARLY) means();
     // split partials added in split order, eight loads in flight at a time, the last ones too
     float4 s2 = make_float4(0.f, 0.f, 0.f, 0.f);
     const float* gp = L->gram_part + off;
@@ -227,6 +235,7 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
       const float4 g4 = load_quad<V4>(L->gram_acc + off, j, M);
       s2.x += g4.x; s2.y += g4.y; s2.z += g4.z; s2.w += g4.w;
     }
+    if (EARLY) { dep_wait(); means(); }
     // (1/rows) sum (x-mu)(x-mu)^T with x - mu = (x - c) - nu, written symmetrically in i, j so that the result mirrors exactly
     auto entry = [&](float s, float mhj, float nuj, float o) {
       const float cross = __fadd_rn(__fmul_rn(mh_i, nuj), __fmul_rn(nu_i, mhj));
@@ -238,6 +247,7 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
     if (bi != bj) store_quad<V4>(L->Phix + off, j, M, out);
     tile[ii][qc] = out.x; tile[ii][qc + 1] = out.y; tile[ii][qc + 2] = out.z; tile[ii][qc + 3] = out.w;
   }
+  if (EARLY) dep_wait();                                           // (threads past the matrix)
   __syncthreads();
   // element (r, c) of the tile goes to (c, r); in a diagonal tile the entries on and above the diagonal stay where they are
   const int jg = bj * 32 + ii, ig = bi * 32 + qc;
@@ -255,16 +265,19 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
 // layers are small, by HBM where they are large; with a 16-byte access per row and split instead of four rows of 4 bytes one
 // after the other, and moments_vec_kernel's sums batched: 368 -> 362 us a step of the
 // ResNet-20-shaped set, 5074 -> 5005 of the ResNet-50-shaped set, 342 -> 321 of one with odd sizes.
+template <bool EARLY>
 __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a,
                                                           const __grid_constant__ PtrTable W,
                                                           const __grid_constant__ PtrTable b) {
-  dep_sync();
+  if (EARLY) dep_trigger();
+  else dep_sync();
   const int nbias = a.bias_blocks * g.n;
   if ((int)blockIdx.x < nbias) {
     // the first CTAs carry the bias compensation (Eq. 31), which needs the means only: long rows of W start early
     // and the tiles fill in behind them
+    if (EARLY) dep_wait();
     const int layer = (int)blockIdx.x / a.bias_blocks, blk = (int)blockIdx.x - layer * a.bias_blocks;
     bias_comp_rows(g.layer[layer], reinterpret_cast<const float*>(W.p[layer]),
                    const_cast<float*>(reinterpret_cast<const float*>(b.p[layer])), blk, threadIdx.x);
@@ -281,8 +294,8 @@ __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant_
   tri_decode(tile_id - a.tt.tile0[li], (M + 31) / 32, bi, bj);
   __shared__ float tile[32][33];
   const float inv_rows = 1.0f / (float)rows.v[li];
-  if ((M & 3) == 0) moments_tile<true>(L, a, li, inv_rows, bi, bj, tile);
-  else moments_tile<false>(L, a, li, inv_rows, bi, bj, tile);
+  if ((M & 3) == 0) moments_tile<true, EARLY>(L, a, li, inv_rows, bi, bj, tile);
+  else moments_tile<false, EARLY>(L, a, li, inv_rows, bi, bj, tile);
 }
 
 // A call that leaves its block open (FW_COV_ACCUMULATE): the split sums of this call are added, in split order,
@@ -603,13 +616,21 @@ cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t*
   for (int i = 0; i < g.n; ++i) {
     a.splits[i] = splits[i]; a.first[i] = first[i]; a.use_acc[i] = use_acc[i]; a.corr[i] = corr[i];
   }
+  const int total = fill_tile_table(a.tt, layer_M, g.n);
+  a.bias_blocks = any_params ? (max_N + 7) / 8 : 0;
+  // Side by side where both fit the chip at once, a CTA an SM: covariance update of 64 x 128 rows 15.1 -> 13.4 us, 147 x 3000 52 -> 35,
+  // 400 x 2000 44 -> 32, 402 x 6000 127 -> 96.  Not with few tiles that have many splits to add (75 x 7504 109 -> 119 us a step,
+  // M = 27 beside other sizes 173 -> 187): there the CTAs of the tiles, started later, are what the launch waits for.
+  a.early = total + a.bias_blocks * g.n + g.n <= sm_count();
+  for (int i = 0; i < g.n; ++i) {
+    const int t = (layer_M[i] + 31) / 32;
+    if (splits[i] > 8 && t * (t + 1) / 2 < 12) a.early = 0;
+  }
   cudaError_t e;
   { ProfScope ps(FW_PROF_MOMENTS, s); e = launch_dep(moments_vec_kernel, g.n, 1024, 0, s, g, rows, a); }
   if (e != cudaSuccess) return e;
-  const int total = fill_tile_table(a.tt, layer_M, g.n);
-  a.bias_blocks = any_params ? (max_N + 7) / 8 : 0;
   ProfScope ps(FW_PROF_MOMENTS, s);
-  return launch_dep(moments_mat_kernel, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
+  return launch_dep(a.early ? moments_mat_kernel<true> : moments_mat_kernel<false>, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
 }
 
 cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, const int* B, const int* H, const int* W,
