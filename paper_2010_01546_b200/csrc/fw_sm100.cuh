@@ -91,9 +91,13 @@ __device__ __forceinline__ void bulk_store(float* dst, const float* src, uint32_
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes) : "memory");
 }
 
-// round-to-nearest (ties away) of an fp32 value to the TF32 grid, on the integer pipe
+// round-to-nearest (ties away) of an fp32 value to the TF32 grid.  The instruction keeps a NaN, where an integer addition and a mask turn
+// the one the GPU makes (all mantissa bits set) into a zero; the two agree for every number.  (Addition and mask with a test
+// for NaN: step of the ResNet-20-shaped set 326.9 -> 329.0 us, of which the instruction takes 0.8.)
 __device__ __forceinline__ float tf32_rna(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return __uint_as_float(r);
 }
 
 // ---- TMEM / tcgen05 --------------------------------------------------------------
