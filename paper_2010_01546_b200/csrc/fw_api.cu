@@ -230,7 +230,7 @@ struct ProfRec { int cls; cudaEvent_t a, b; };
 bool g_prof_on = false;
 std::vector<ProfRec> g_prof;
 std::vector<cudaEvent_t> g_event_pool;
-int64_t g_launches = 0;
+std::atomic<int64_t> g_launches{0};
 
 cudaEvent_t prof_event() {
   if (!g_event_pool.empty()) { cudaEvent_t e = g_event_pool.back(); g_event_pool.pop_back(); return e; }

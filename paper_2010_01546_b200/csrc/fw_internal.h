@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <mutex>
 #include "fw.h"
 
 namespace fw {
@@ -224,11 +225,12 @@ inline cudaError_t launch_dep_cluster(int cl, void (*kernel)(P...), dim3 grid, d
 }
 
 // Largest dynamic shared-memory size a kernel has been opted into, per device (the attribute is per device).
-struct SmemAttrCache { size_t set[64] = {0}; };
+struct SmemAttrCache { std::mutex mu; size_t set[64] = {0}; };
 template <class F>
 inline cudaError_t ensure_dyn_smem(F* func, size_t bytes, SmemAttrCache& c) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); dev = -1; }
+  std::lock_guard<std::mutex> lock(c.mu);       // a smaller size set late by another thread would undo a larger one
   if (dev >= 0 && dev < 64 && bytes <= c.set[dev]) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess && dev >= 0 && dev < 64) c.set[dev] = bytes;

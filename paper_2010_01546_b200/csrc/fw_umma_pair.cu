@@ -41,13 +41,12 @@
 // CTAs, is recorded in the owning layer's status word, and all threads still meet
 // at the final cluster barrier before TMEM is freed.
 #include <algorithm>
-#include <cmath>
 #include <cstdio>
-#include <cstdlib>
 #include <cstring>
-#include <map>
+#include <mutex>
 #include <vector>
 
+#include "fw_pair_plan.h"
 #include "fw_sm100.cuh"
 #include "fw_umma.h"
 
@@ -57,11 +56,6 @@ using namespace sm100;
 
 namespace {
 
-constexpr int GP_SR_F32 = 32;              // rows of X per stage, fp32 (48 KB stages, 4 in flight)
-constexpr int GP_SR_BF16 = 64;             // bf16: the same 48 KB and 1024 tensor cycles per stage as fp32; with 32 rows
-                                           // (512 cycles) the per-stage hand-offs left the tensor pipe idle a third of the time
-__host__ __device__ constexpr int pair_sr(bool bf16) { return bf16 ? GP_SR_BF16 : GP_SR_F32; }
-constexpr int GP_GCOLS = 128;              // columns per column group (chunks of 32 fp32 or 64 bf16 columns)
 constexpr int GP_MAX_GROUPS = 3;           // A block, first and second B panel halves
 constexpr int GP_MAX_STAGES = 8;
 constexpr int GP_FIX_WARPS = 8;
@@ -70,8 +64,6 @@ constexpr int GP_SMEM = 192 * 1024;
 constexpr int GP_CONST = 12 * 1024;        // constant operand chunks of the mean-product correction: 3 column groups x
                                            // one MMA's rows (16 bf16 / 8 fp32) x 128 columns
 constexpr int GP_MAX_PROBLEMS = 16;
-constexpr int GP_MAX_ITEMS = 2048;
-constexpr int kMinPanel = 256;             // narrowest tile of a product
 constexpr int GP_CLUSTER_SLOTS = 74;       // CTA pairs resident at once if every TPC takes one (148 SMs, one CTA per SM)
 
 struct PairProblem {
@@ -99,13 +91,6 @@ struct PairGroup {
   uint32_t item[GP_MAX_ITEMS];           // problem << 28 | tile << 14 | split, longest first
 };
 
-__host__ __device__ inline int pair_tiles_sym(int M16) {
-  int t = 0;
-  for (int c = 0; c < M16; c += 256) t += (M16 - c + 511) / 512;
-  return t;
-}
-__host__ __device__ inline int pair_tiles_full(int M16, int panel) { return ((M16 + 255) / 256) * ((M16 + panel - 1) / panel); }
-
 __device__ __forceinline__ float4 lds128(uint32_t a) {
   float4 v;
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
@@ -122,7 +107,7 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
   //   bf16: 64 columns, 128-byte swizzle (16-byte units), K-atoms of 8 rows.
   constexpr int CW = BF ? 64 : 32;                // columns per chunk
   constexpr int GC = GP_GCOLS / CW;               // chunks per column group
-  constexpr int SR = pair_sr(BF);                 // rows per stage
+  constexpr int SR = BF ? GP_SR_BF16 : GP_SR_F32; // rows per stage
   constexpr int KSTEPS = SR / (BF ? 16 : 8);      // MMAs along K per stage (16 / 8 rows each)
   constexpr int CHUNK = SR * 128;                 // bytes per chunk
   constexpr int GROUP_BYTES = GC * CHUNK;         // bytes per column group per stage
@@ -532,162 +517,18 @@ gram_pair_kernel(const __grid_constant__ PairGroup g) {
 }
 
 // ---------------------------------------------------------------------------
-// host: work list
+// host: work list (fw_pair_plan.h) and launch
 // ---------------------------------------------------------------------------
-struct PairTile { int n0, n1, cols; bool skip; };   // cols: columns a CTA stages   // skip: wholly below the diagonal of a symmetric product
-
-void pair_tiles(int M, bool full, int panel, bool sym_out, std::vector<PairTile>& out) {
-  const int M16 = (M + 15) / 16 * 16;
-  out.clear();
-  for (int I = 0; 256 * I < M16; ++I) {
-    const int c_first = full ? 0 : 256 * I;
-    for (int c = c_first, t = 0; c < M16; c += panel, ++t) {
-      PairTile pt;
-      const int pw = std::min(panel, M16 - c);
-      pt.n0 = std::min(256, pw);
-      pt.n1 = pw - pt.n0;
-      const bool diag = !full && t == 0;
-      // (a Gram tile counts whole groups: the row slabs chosen by this estimate fix how the sums are rounded)
-      if (full) pt.cols = GP_GCOLS + pt.n0 / 2 + pt.n1 / 2;
-      else pt.cols = GP_GCOLS * (1 + ((diag && pt.n0 == 256) ? 0 : 1) + (pt.n1 > 0 ? 1 : 0));
-      pt.skip = full && sym_out && c + pt.n0 + pt.n1 <= 256 * I;
-      out.push_back(pt);
-    }
-  }
-}
-
-// Estimated time of one tile over `rows` rows, microseconds: tensor time against staging time.  Staging rates
-// are what a CTA sustains with every SM busy (measured: about 40 bytes per clock for bf16 tiles and 48 for fp32
-// tiles, which then run at the TF32 tensor rate).
-double pair_tile_us(const PairTile& t, bool bf16, int fix, double rows) {
-  const double clk_us = 1800.0;                                   // SM clocks per microsecond under load
-  const double tensor = (t.n0 + t.n1) / 512.0 * (bf16 ? 16.0 : 32.0);
-  const double load = t.cols * (bf16 ? 2.0 / 40.0 : 4.0 / 48.0) * (1.0 + 0.2 * (fix & 1) + 0.4 * (fix >> 1));
-  const double fixed = 4.0 + 128.0 * (t.n0 + t.n1) * 4.0 / 80e3;  // prologue, pipeline fill, epilogue stores
-  return fixed + rows * std::max(tensor, load) / clk_us;
-}
-
-struct PairSpec {
-  int M; int64_t rows; bool bf16, full, colsums, sym_out = false; int split_cap; int panel = 512, fix = 0, round_out = 0;
-  std::vector<PairTile> tiles;
-  int splits; int64_t per;     // chosen: splits, stages per split
-};
-
-// When the longest-first list schedule of the items over the resident CTA pairs ends.
-double pair_makespan(std::vector<double>& items, int slots) {
-  std::sort(items.begin(), items.end(), [](double a, double b) { return a > b; });
-  std::vector<double> slot(slots, 0.0);
-  for (double c : items) *std::min_element(slot.begin(), slot.end()) += c;
-  return *std::max_element(slot.begin(), slot.end());
-}
-
-// Columns of the products' tiles: 512 moves the fewest bytes per output, but one layer of M = 2304 is 45 such tiles on 74
-// pairs of SMs, or 72 of 320 columns that take three quarters of the time.  The last set a thread launched is remembered.
-int pair_choose_panel(const std::vector<PairSpec>& P, int slots) {
-  thread_local std::vector<int> last;
-  thread_local int last_panel = 512;
-  std::vector<int> key(1, slots);
-  for (const PairSpec& p : P) { key.push_back(p.M); key.push_back(p.sym_out * 4 + p.fix); }
-  if (key == last) return last_panel;
-  int panel = 512;
-  double best = 0;
-  std::vector<PairTile> tiles;
-  std::vector<double> items;
-  for (int w = 512; w >= kMinPanel; w -= 64) {
-    items.clear();
-    for (const PairSpec& p : P) {
-      pair_tiles(p.M, true, w, p.sym_out, tiles);
-      for (const PairTile& t : tiles)
-        if (!t.skip) items.push_back(pair_tile_us(t, false, p.fix, (double)p.M));
-    }
-    if (items.size() > (size_t)GP_MAX_ITEMS) break;
-    const double end = pair_makespan(items, slots);
-    if (w == 512 || end < best) { best = end; panel = w; }
-  }
-  last = key; last_panel = panel;
-  return panel;
-}
-
-// Chooses the split count of every problem so that the longest-first list schedule of all (tile, split) items
-// over the resident CTA pairs ends earliest, counting what each further split costs the reduction that follows.
-void pair_choose_splits(std::vector<PairSpec>& P, int slots) {
-  double best = 1e300;
-  std::vector<int> best_s(P.size(), 1);
-  std::vector<double> items;
-  // the search costs the host a fraction of a millisecond: its result is kept per list of problems
-  static std::map<std::vector<int64_t>, std::pair<std::vector<int>, double>> memo;
-  std::vector<int64_t> key;
-  key.push_back(slots);
-  for (const PairSpec& p : P) {
-    key.push_back(p.M); key.push_back(p.rows); key.push_back(p.split_cap); key.push_back(p.panel);
-    key.push_back((p.bf16 ? 1 : 0) | (p.full ? 2 : 0) | (p.fix << 5) | (p.sym_out ? 8 : 0) | (p.colsums ? 16 : 0));
-  }
-  auto hit = memo.find(key);
-  if (hit != memo.end()) { best_s = hit->second.first; best = hit->second.second; }
-  for (int step = 0; hit == memo.end() && step < 64; ++step) {
-    const double tau = 6.0 * std::pow(1.12, step);                // target item time, 6 us .. 7.5 ms
-    double extra = 0;
-    size_t count = 0;
-    items.clear();
-    std::vector<int> sp(P.size());
-    for (size_t l = 0; l < P.size(); ++l) {
-      PairSpec& p = P[l];
-      double longest = 0;
-      for (const PairTile& t : p.tiles)
-        if (!t.skip) longest = std::max(longest, pair_tile_us(t, p.bf16, p.fix, (double)p.rows));
-      const int SRh = pair_sr(p.bf16);
-      const int64_t nsr = (p.rows + SRh - 1) / SRh;
-      int64_t s = (int64_t)(longest / tau + 0.5);
-      s = std::max<int64_t>(1, std::min<int64_t>(s, std::min<int64_t>(p.split_cap, nsr)));
-      const int64_t per = (nsr + s - 1) / s;
-      s = (nsr + per - 1) / per;
-      sp[l] = (int)s;
-      for (const PairTile& t : p.tiles) {
-        if (t.skip) continue;
-        for (int64_t k = 0; k < s; ++k) {
-          const double r = (double)std::min<int64_t>(per * SRh, p.rows - k * per * SRh);
-          items.push_back(pair_tile_us(t, p.bf16, p.fix, r));
-        }
-        count += (size_t)s;
-      }
-      // the reduction reads every partial once (upper triangle), at about 4 TB/s
-      if (!p.full) extra += (double)(s - 1) * 0.55 * 4.0 * p.M * (double)p.M / 4e6;
-    }
-    if (count > (size_t)GP_MAX_ITEMS) continue;
-    const double span = pair_makespan(items, slots) + extra;
-    if (span < best) { best = span; best_s = sp; }
-  }
-  if (hit == memo.end()) {
-    if (memo.size() > 256) memo.clear();
-    memo[key] = std::make_pair(best_s, best);
-  }
-  const int forced = tuning().pair_splits;   // tuning aid
-  for (size_t l = 0; l < P.size(); ++l) {
-    PairSpec& p = P[l];
-    const int64_t nsr = (p.rows + pair_sr(p.bf16) - 1) / pair_sr(p.bf16);
-    int64_t s = best_s[l];
-    if (forced > 0) s = std::max<int64_t>(1, std::min<int64_t>(forced, std::min<int64_t>(p.split_cap, nsr)));
-    if (tuning().pair_debug) fprintf(stderr, "[fw] pair: M=%d rows=%lld tiles=%zu splits=%lld (cap %d) est %.1f us\n", p.M, (long long)p.rows, p.tiles.size(), (long long)s, p.split_cap, best);
-    const int64_t per = (nsr + s - 1) / s;
-    p.splits = (int)((nsr + per - 1) / per);
-    p.per = per;
-  }
-}
-
 struct PairSource { const void* A; const void* B; int64_t lda, ldb; float* out; float* colsum; int32_t* status; const float* pmean; };
 
-fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource>& src, int prof_class, cudaStream_t s) {
-  static bool attr_set = false;
-  static int slots = GP_CLUSTER_SLOTS;
-  static SmemAttrCache attr_f32, attr_bf16;
-  const int smem = GP_SMEM + GP_CONST + 1024;
-  if (ensure_dyn_smem(gram_pair_kernel<false>, smem, attr_f32) != cudaSuccess ||
-      ensure_dyn_smem(gram_pair_kernel<true>, smem, attr_bf16) != cudaSuccess) {
-    cudaGetLastError();
-    return FW_ERR_CUDA;
-  }
-  if (!attr_set) {
-    // how many pairs the device really keeps resident (fewer than SMs / 2 when a GPC has an odd SM out)
+// How many CTA pairs the device really keeps resident (fewer than SMs / 2 when a GPC has an odd SM out)
+int resident_pairs(int smem) {
+  static std::mutex mu;
+  static int known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return GP_CLUSTER_SLOTS; }
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[dev] == 0) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(2 * GP_MAX_ITEMS); cfg.blockDim = dim3(GP_THREADS); cfg.dynamicSmemBytes = smem;
@@ -696,11 +537,22 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, gram_pair_kernel<false>, &cfg) == cudaSuccess && nc > 0) slots = nc;
-    else cudaGetLastError();
-    if (tuning().pair_debug) fprintf(stderr, "[fw] pair: %d resident CTA pairs\n", slots);
-    attr_set = true;
+    if (cudaOccupancyMaxActiveClusters(&nc, gram_pair_kernel<false>, &cfg) != cudaSuccess || nc < 1) { cudaGetLastError(); nc = GP_CLUSTER_SLOTS; }
+    known[dev] = nc;
+    if (tuning().pair_debug) fprintf(stderr, "[fw] pair: %d resident CTA pairs\n", nc);
   }
+  return known[dev];
+}
+
+fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource>& src, int prof_class, cudaStream_t s) {
+  static SmemAttrCache attr_f32, attr_bf16;
+  const int smem = GP_SMEM + GP_CONST + 1024;
+  if (ensure_dyn_smem(gram_pair_kernel<false>, smem, attr_f32) != cudaSuccess ||
+      ensure_dyn_smem(gram_pair_kernel<true>, smem, attr_bf16) != cudaSuccess) {
+    cudaGetLastError();
+    return FW_ERR_CUDA;
+  }
+  const int slots = resident_pairs(smem);
   const int n = (int)specs.size();
   for (int base = 0; base < n;) {
     // one element type per launch, at most GP_MAX_PROBLEMS problems
@@ -714,7 +566,7 @@ fw_status pair_launch(std::vector<PairSpec>& specs, const std::vector<PairSource
         pair_tiles(p.M, true, panel, p.sym_out, p.tiles);
       }
     }
-    pair_choose_splits(grp, slots);
+    pair_choose_splits(grp, slots, tuning().pair_splits, tuning().pair_debug != 0);
     std::vector<PairGroup> gbuf(1);           // 17 KB: kept off the stack; the launch copies it
     PairGroup& g = gbuf[0];
     memset(&g, 0, sizeof(g));
