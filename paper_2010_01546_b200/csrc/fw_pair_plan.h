@@ -97,14 +97,14 @@ inline double pair_makespan(std::vector<double>& items, int slots) {
 }
 
 // Columns of the products' tiles: 512 moves the fewest bytes per output, but one layer of M = 2304 is 45 such tiles on 74
-// pairs of SMs, or 72 of 320 columns that take three quarters of the time.  The last set a thread launched is remembered.
+// pairs of SMs, or 72 of 320 columns that take three quarters of the time.  The search takes the host 1 ms for 16 layers of M = 1024 to 2500 and is made
+// once per list of problems: every re-sync asks for two, one a product.
 inline int pair_choose_panel(const std::vector<PairSpec>& P, int slots) {
-  thread_local std::vector<int> last;
-  thread_local int last_panel = 512;
-  std::vector<int> key(1, slots);
+  static PlanMemo<int> memo;
+  std::vector<int64_t> key(1, slots);
   for (const PairSpec& p : P) { key.push_back(p.M); key.push_back(p.sym_out * 4 + p.fix); }
-  if (key == last) return last_panel;
   int panel = 512;
+  if (memo.find(key, panel)) return panel;
   double best = 0;
   std::vector<PairTile> tiles;
   std::vector<double> items;
@@ -119,7 +119,7 @@ inline int pair_choose_panel(const std::vector<PairSpec>& P, int slots) {
     const double end = pair_makespan(items, slots);
     if (w == 512 || end < best) { best = end; panel = w; }
   }
-  last = key; last_panel = panel;
+  memo.keep(key, panel);
   return panel;
 }
 

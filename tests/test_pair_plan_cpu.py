@@ -9,6 +9,8 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 PROGRAM = r"""
+#include <chrono>
+#include <cstdio>
 #include <thread>
 #include "fw_pair_plan.h"
 using namespace fw;
@@ -30,7 +32,7 @@ static long plan(int k, bool second, int layers) {
   for (const PairSpec& p : v) sum = sum * 31 + p.splits * 1000 + p.per;
   return sum;
 }
-int main() {
+static int threads() {
   const int T = 8, N = 80;
   std::vector<std::vector<long>> got(T, std::vector<long>(N));
   std::vector<std::thread> th;
@@ -42,6 +44,22 @@ int main() {
       if (got[t][k] != plan(N * t / 2 + k, k & 1, 2)) return 1;
   return 0;
 }
+// microseconds of choosing the width of both products' tiles, the first time and at best later
+static int repeated() {
+  const std::vector<PairSpec> a = list_of(3, false, 16), b = list_of(3, true, 16);
+  double first = 0, later = 1e300;
+  for (int i = 0; i < 20; ++i) {
+    const auto t0 = std::chrono::steady_clock::now();
+    pair_choose_panel(a, 74);
+    pair_choose_panel(b, 74);
+    const double us = std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count();
+    if (i == 0) first = us;
+    else later = std::min(later, us);
+  }
+  std::printf("%.1f %.1f\n", first, later);
+  return 0;
+}
+int main(int argc, char**) { return argc > 1 ? repeated() : threads(); }
 """
 
 
@@ -63,3 +81,10 @@ def compiled(tmp_path, flags):
 def test_plans_of_several_threads(tmp_path):
     r = subprocess.run([compiled(tmp_path, ["-O1", "-g", "-fsanitize=thread"])], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-3000:]
+
+
+def test_a_step_does_not_search_again(tmp_path):
+    """A re-sync asks for the tiles of its first product, then for those of its second, every step."""
+    r = subprocess.run([compiled(tmp_path, ["-O2"]), "repeated"], capture_output=True, text=True, timeout=300)
+    first, later = map(float, r.stdout.split())
+    assert 10 * later < first, (first, later)
