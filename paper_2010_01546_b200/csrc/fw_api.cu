@@ -684,10 +684,7 @@ fw_status fw_group_cond_reduce(fw_layer* const* L, int32_t n, int32_t K, int32_t
       gp.layer[gp.n] = l->dev; tp.p[gp.n] = t; dims_p[gp.n] = M; ++gp.n;
     }
   }
-  for (int k0 = 0; k0 < K && gc.n; k0 += kChipSteps) {
-    const int kc = std::min(kChipSteps, K - k0);
-    FW_CUDA(launch_recursion_cluster(gc, tc, dims_c, k0, kc, P, k0 + kc == K, s), "recursion (cluster)");
-  }
+  if (gc.n) FW_CUDA(launch_recursion_cluster(gc, tc, dims_c, K, P, s), "recursion (cluster)");
   bool any_beta = false;
   for (int i = 0; i < n; ++i) any_beta |= (L[i]->d.beta > 0.f);
   // large layers: teams of CTAs; T and Q take the recorded steps, up to kHist at a time

@@ -289,11 +289,8 @@ cudaError_t launch_evd(int n, const float* const* src, const int* layer_M, void*
 bool recursion_cluster_supported(int M);
 // CTAs of a 16-CTA cluster the on-chip recursion gives a layer of size M (1, 2, 4, 8, 16; 0: not on chip)
 int recursion_cluster_ctas(int M);
-// Steps k0 ... k0 + K - 1 (K <= kChipSteps) of a call for layers that fit on chip, T, Q and Qs included.  last: the launch ends
-// the call.
-constexpr int kChipSteps = 8;
-cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
-                                     bool last, cudaStream_t s);
+// All K steps of a call for layers that fit on chip, T, Q and Qs included
+cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P, cudaStream_t s);
 // Steps k0 ... k0 + K - 1 (K <= kHist) of a call for large gamma = 1 layers, as one cooperative launch; v_e, a_e of the
 // steps are left in vh, ah.  Its packet exchanges are numbered from the layer's IS_EXCHANGE on, team_exchanges(K, P) of them;
 // the launch only reads that word (CTAs start at different times), launch_recursion_apply advances it.  last: the launch

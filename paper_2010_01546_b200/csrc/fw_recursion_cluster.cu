@@ -47,7 +47,7 @@ constexpr int CW = CT / 32;        // warps per CTA
 constexpr int kMaxIt = 5;          // float4 columns per lane, at most
 constexpr int kMaxM = 624;         // longest row whose products are summed in fp32; longer ones take teams of CTAs and fp64 sums
 constexpr int kSolo = 64;          // largest layer that takes one CTA and eight lanes a row
-constexpr int KH = kChipSteps;     // steps of a launch, all of which T and Q take at its end
+constexpr int KH = 8;              // steps that T and Q take together
 constexpr size_t kSmemLimit = 64 * 1024;   // the vectors of the longest row: 22 of 16 slabs of at most 43 entries
 
 // A warp owns one group of four rows (up to kMaxIt float4 columns per lane: 80 registers) or, for rows of at most 256
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     if (tr) tr += 4 * a.k0;
     const bool last = a.last != 0;
     if (M <= kSolo) {
-      run_solo(s, L, tr, a.K, a.P, last);
+      for (int k = 0; k < a.K; k += KH) run_solo(s, L, tr ? tr + 4 * k : nullptr, min(KH, a.K - k), a.P, last && k + KH >= a.K);
     } else if (ng == 1) {
       switch (it) {
         case 1: run_steps<1, 1>(s, l, L, tr, a.K, a.P, last); break;
@@ -993,9 +993,8 @@ int recursion_cluster_ctas(int M) {
 
 bool recursion_cluster_supported(int M) { return recursion_cluster_ctas(M) > 0; }
 
-cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int k0, int K, int P,
-                                     bool last, cudaStream_t s) {
-  if (K < 1 || K > KH) return cudaErrorInvalidValue;
+cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
+                                     cudaStream_t s) {
   static SmemAttrCache attr;
   static std::mutex mu;
   static int resident[64][5];        // clusters of 1, 2, 4, 8, 16 CTAs that run together (16: 7 on a B200)
@@ -1050,15 +1049,27 @@ cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, 
   }
   ClusterArgs a;
   memset(&a, 0, sizeof(a));
-  a.g = g; a.traces = traces; a.k0 = k0; a.K = K; a.P = P; a.last = last ? 1 : 0;
+  a.g = g; a.traces = traces; a.P = P;
   size_t smem = 0;
+  bool solo = true;
   for (int i = 0; i < g.n; ++i) {
     a.first_cta[i] = plan.first[i]; a.ncta[i] = plan.cnt[i];
     smem = std::max(smem, cluster_smem(layer_M[i], plan.cnt[i]));
+    solo &= layer_M[i] <= kSolo;
   }
   config(cfg, at, plan.cl, plan.bins * plan.cl, smem);
-  ProfScope ps(FW_PROF_RECUR_CHIP, s);
-  return cudaLaunchKernelEx(&cfg, recursion_cluster_kernel, a);
+  // A launch is KH steps.  Layers of one CTA each take all of the call's in one: a launch of theirs costs as much as two steps
+  // without power iterations (M = 64, K = 32, P = 0: 93 us in four launches, 77 in one).  Where a cluster exchanges, the steps
+  // are long and the same loop in the kernel costs each of them more registers than it saves launches (M = 576, K = 8, P = 16:
+  // 160 us, with the loop 172; K = 64, P = 4: 559 and 560).
+  const int most = solo ? K : KH;
+  for (int k0 = 0; k0 < K; k0 += most) {
+    a.k0 = k0; a.K = std::min(most, K - k0); a.last = k0 + a.K == K;
+    ProfScope ps(FW_PROF_RECUR_CHIP, s);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, recursion_cluster_kernel, a);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace fw
