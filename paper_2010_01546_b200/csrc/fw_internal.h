@@ -55,7 +55,7 @@ struct LayerDev {
   int32_t round_t;      // tensor-core layers without leakage: whatever writes Tt writes its values rounded to TF32 to tmp, as
                         // operands of the re-sync products
   // a block spread over several calls (FW_COV_ACCUMULATE): sums of the calls before the committing one
-  float* gram_acc;      // M x M (upper-triangle tiles)
+  float* gram_acc;      // M x M (upper-triangle tiles); between blocks, the added split partials of a committing call
   float* colsum_acc;    // M
   // G Qs formed here when the caller asks for it in place
   float* gq_tmp;        // N x M
@@ -181,10 +181,6 @@ struct GemmGroup {
 __device__ __forceinline__ void dep_sync() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
-// The two halves, for a kernel and its dependent that share a predecessor: a kernel that waits first and triggers then lets its
-// dependent start on what the predecessor left (it has completed, and its writes are visible), before it waits itself.
-__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The launchers report what their launches returned, not the thread's last error: that may be of an earlier call, and it is the
 // caller's to read.
 template <class T> struct SameType { using type = T; };

@@ -73,7 +73,8 @@ struct MomentArgs {
                                      // 0 = overwrite the accumulators, 1 = add to them)
   float corr[FW_MAX_GROUP];          // > 0: corr c c^T was taken out of this call's Gram sums (c = rounded pmean)
   TileTable tt;                      // flat grid over the upper-triangle 32x32 tiles of all layers
-  int32_t early;                     // moments_mat_kernel adds its partial sums while moments_vec_kernel runs
+  int32_t sum_blocks;                // CTAs of moments_vec_kernel behind its one per layer that add the split partials of a tile each into
+                                     // gram_acc; 0: moments_mat_kernel adds them
   int32_t bias_blocks;               // CTAs per layer placed before the tiles for b += W (mu_new - mu_old); 0: none
 };
 
@@ -92,12 +93,105 @@ __device__ __forceinline__ void split_sums(const float* cp, const float* gp, int
   }
 }
 
-// One CTA per layer, 1024 threads (one column each for M <= 1024).
+// Four consecutive entries of a row, i fixed: V4 in one access (rows of whole float4s), else one by one below M.
+template <bool V4>
+__device__ __forceinline__ float4 load_quad(const float* p, int j, int M) {
+  if (V4) return *reinterpret_cast<const float4*>(p);
+  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+  r.x = p[0];
+  if (j + 1 < M) r.y = p[1];
+  if (j + 2 < M) r.z = p[2];
+  if (j + 3 < M) r.w = p[3];
+  return r;
+}
+template <bool V4>
+__device__ __forceinline__ void store_quad(float* p, int j, int M, float4 v) {
+  if (V4) { *reinterpret_cast<float4*>(p) = v; return; }
+  p[0] = v.x;
+  if (j + 1 < M) p[1] = v.y;
+  if (j + 2 < M) p[2] = v.z;
+  if (j + 3 < M) p[3] = v.w;
+}
+
+// Entries (i, j) ... (i, j + 3) of a layer's Gram sums: split partials in split order, eight loads in flight at a time, the last
+// ones too; then what was taken out of them and the block's earlier calls.
+template <bool V4>
+__device__ __forceinline__ float4 gram_quad(const LayerDev* L, const MomentArgs& a, int li, int i, int j) {
+  const int M = L->M, S = a.splits[li];
+  const int64_t off = (int64_t)i * M + j, MM = (int64_t)M * M;
+  float4 s2 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* gp = L->gram_part + off;
+  for (int k0 = 0; k0 < S; k0 += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k0 + u < S) v[u] = load_quad<V4>(gp + (int64_t)(k0 + u) * MM, j, M);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k0 + u < S) { s2.x += v[u].x; s2.y += v[u].y; s2.z += v[u].z; s2.w += v[u].w; }
+  }
+  const float corr = a.corr[li];
+  if (corr > 0.f) {                                                // symmetric in (i, j)
+    const int xbf = L->x_dtype == FW_BF16;
+    const float ci = corr_round(L->pmean[i], xbf);
+    const float4 pm = load_quad<V4>(L->pmean + j, j, M);
+    s2.x = fmaf(corr, __fmul_rn(ci, corr_round(pm.x, xbf)), s2.x); s2.y = fmaf(corr, __fmul_rn(ci, corr_round(pm.y, xbf)), s2.y);
+    s2.z = fmaf(corr, __fmul_rn(ci, corr_round(pm.z, xbf)), s2.z); s2.w = fmaf(corr, __fmul_rn(ci, corr_round(pm.w, xbf)), s2.w);
+  }
+  if (a.use_acc[li]) {
+    const float4 g4 = load_quad<V4>(L->gram_acc + off, j, M);
+    s2.x += g4.x; s2.y += g4.y; s2.z += g4.z; s2.w += g4.w;
+  }
+  return s2;
+}
+
+// One entry, by the same operations in the same order; sixteen loads in flight.
+__device__ __forceinline__ float gram_sum(const LayerDev* L, const MomentArgs& a, int li, int i, int j) {
+  const int M = L->M, S = a.splits[li];
+  const int64_t off = (int64_t)i * M + j, MM = (int64_t)M * M;
+  const float* gp = L->gram_part + off;
+  float s2 = 0.f;
+  for (int k0 = 0; k0 < S; k0 += 16) {
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (k0 + u < S) v[u] = gp[(int64_t)(k0 + u) * MM];
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (k0 + u < S) s2 += v[u];
+  }
+  const float corr = a.corr[li];
+  if (corr > 0.f) {
+    const int xbf = L->x_dtype == FW_BF16;
+    s2 = fmaf(corr, __fmul_rn(corr_round(L->pmean[i], xbf), corr_round(L->pmean[j], xbf)), s2);
+  }
+  return s2;
+}
+
+// the layer and the 32 x 32 tile (bi <= bj) of its upper triangle that a place in the flat list of tiles stands for
+__device__ __forceinline__ int find_tile(const GroupDev& g, const MomentArgs& a, int tile_id, int& bi, int& bj) {
+  int li = 0;
+#pragma unroll 1
+  for (int i = 1; i < g.n; ++i)
+    if (tile_id >= a.tt.tile0[i]) li = i;
+  tri_decode(tile_id - a.tt.tile0[li], (g.layer[li]->M + 31) / 32, bi, bj);
+  return li;
+}
+
+// One CTA per layer, 1024 threads (one column each for M <= 1024), and a.sum_blocks CTAs that meanwhile add the split partials
+// of a tile each, a thread an entry.
 __global__ void __launch_bounds__(1024) moments_vec_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a) {
-  if (a.early) { dep_wait(); dep_trigger(); }         // the Gram pass has completed: moments_mat_kernel may add its partial sums
-  else dep_sync();
+  dep_sync();
+  if ((int)blockIdx.x >= g.n) {
+    int bi, bj;
+    const int li = find_tile(g, a, (int)blockIdx.x - g.n, bi, bj);
+    const LayerDev* L = g.layer[li];
+    const int i = bi * 32 + ((int)threadIdx.x >> 5), j = bj * 32 + ((int)threadIdx.x & 31);
+    if (i < L->M && j < L->M) L->gram_acc[(int64_t)i * L->M + j] = gram_sum(L, a, li, i, j);
+    return;
+  }
   const LayerDev* L = g.layer[blockIdx.x];
   const int M = L->M;
   const int S = a.splits[blockIdx.x];
@@ -171,71 +265,23 @@ __global__ void __launch_bounds__(1024) moments_vec_kernel(const __grid_constant
   if (bad) L->iscal[IS_STATUS_NONFINITE] = 1;
 }
 
-// Four consecutive entries of a row, i fixed: V4 in one access (rows of whole float4s), else one by one below M.
-template <bool V4>
-__device__ __forceinline__ float4 load_quad(const float* p, int j, int M) {
-  if (V4) return *reinterpret_cast<const float4*>(p);
-  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-  r.x = p[0];
-  if (j + 1 < M) r.y = p[1];
-  if (j + 2 < M) r.z = p[2];
-  if (j + 3 < M) r.w = p[3];
-  return r;
-}
-template <bool V4>
-__device__ __forceinline__ void store_quad(float* p, int j, int M, float4 v) {
-  if (V4) { *reinterpret_cast<float4*>(p) = v; return; }
-  p[0] = v.x;
-  if (j + 1 < M) p[1] = v.y;
-  if (j + 2 < M) p[2] = v.z;
-  if (j + 3 < M) p[3] = v.w;
-}
-
 __device__ __forceinline__ void bias_comp_rows(const LayerDev* L, const float* Wp, float* bp, int blk, int tid);
 
 // One 32 x 32 tile (bi <= bj) of one layer, a thread four entries of a row; the mirror image leaves through shared memory.
-// EARLY: the partial sums before the wait for moments_vec_kernel.
-template <bool V4, bool EARLY>
+// SUMMED: the split partials have been added, into gram_acc.
+template <bool V4, bool SUMMED>
 __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs& a, int li, float inv_rows, int bi, int bj,
                                              float (&tile)[32][33]) {
-  const int M = L->M, S = a.splits[li], tid = threadIdx.x;
+  const int M = L->M, tid = threadIdx.x;
   const bool first = a.first[li] != 0;
-  const float alpha = L->alpha, corr = a.corr[li];
-  const int xbf = L->x_dtype == FW_BF16;
+  const float alpha = L->alpha;
   const int ii = tid >> 3, qc = 4 * (tid & 7), i = bi * 32 + ii, j = bj * 32 + qc;
   if (i < M && j < M) {
-    const int64_t off = (int64_t)i * M + j, MM = (int64_t)M * M;
+    const int64_t off = (int64_t)i * M + j;
     const float4 old = first ? make_float4(0.f, 0.f, 0.f, 0.f) : load_quad<V4>(L->Phix + off, j, M);
-    float mh_i, nu_i;                                             // batch mean - shift, new running mean - shift
-    float4 mh_j, nu_j;
-    auto means = [&] {
-      mh_i = L->pv[0][i]; nu_i = L->pv[1][i];
-      mh_j = load_quad<V4>(L->pv[0] + j, j, M); nu_j = load_quad<V4>(L->pv[1] + j, j, M);
-    };
-    if (!EARLY) means();
-    // split partials added in split order, eight loads in flight at a time, the last ones too
-    float4 s2 = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float* gp = L->gram_part + off;
-    for (int k0 = 0; k0 < S; k0 += 8) {
-      float4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k0 + u < S) v[u] = load_quad<V4>(gp + (int64_t)(k0 + u) * MM, j, M);
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (k0 + u < S) { s2.x += v[u].x; s2.y += v[u].y; s2.z += v[u].z; s2.w += v[u].w; }
-    }
-    if (corr > 0.f) {                                              // symmetric in (i, j)
-      const float ci = corr_round(L->pmean[i], xbf);
-      const float4 pm = load_quad<V4>(L->pmean + j, j, M);
-      s2.x = fmaf(corr, __fmul_rn(ci, corr_round(pm.x, xbf)), s2.x); s2.y = fmaf(corr, __fmul_rn(ci, corr_round(pm.y, xbf)), s2.y);
-      s2.z = fmaf(corr, __fmul_rn(ci, corr_round(pm.z, xbf)), s2.z); s2.w = fmaf(corr, __fmul_rn(ci, corr_round(pm.w, xbf)), s2.w);
-    }
-    if (a.use_acc[li]) {
-      const float4 g4 = load_quad<V4>(L->gram_acc + off, j, M);
-      s2.x += g4.x; s2.y += g4.y; s2.z += g4.z; s2.w += g4.w;
-    }
-    if (EARLY) { dep_wait(); means(); }
+    const float mh_i = L->pv[0][i], nu_i = L->pv[1][i];           // batch mean - shift, new running mean - shift
+    const float4 mh_j = load_quad<V4>(L->pv[0] + j, j, M), nu_j = load_quad<V4>(L->pv[1] + j, j, M);
+    const float4 s2 = SUMMED ? load_quad<V4>(L->gram_acc + off, j, M) : gram_quad<V4>(L, a, li, i, j);
     // (1/rows) sum (x-mu)(x-mu)^T with x - mu = (x - c) - nu, written symmetrically in i, j so that the result mirrors exactly
     auto entry = [&](float s, float mhj, float nuj, float o) {
       const float cross = __fadd_rn(__fmul_rn(mh_i, nuj), __fmul_rn(nu_i, mhj));
@@ -247,7 +293,6 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
     if (bi != bj) store_quad<V4>(L->Phix + off, j, M, out);
     tile[ii][qc] = out.x; tile[ii][qc + 1] = out.y; tile[ii][qc + 2] = out.z; tile[ii][qc + 3] = out.w;
   }
-  if (EARLY) dep_wait();                                           // (threads past the matrix)
   __syncthreads();
   // element (r, c) of the tile goes to (c, r); in a diagonal tile the entries on and above the diagonal stay where they are
   const int jg = bj * 32 + ii, ig = bi * 32 + qc;
@@ -265,37 +310,29 @@ __device__ __forceinline__ void moments_tile(const LayerDev* L, const MomentArgs
 // layers are small, by HBM where they are large; with a 16-byte access per row and split instead of four rows of 4 bytes one
 // after the other, and moments_vec_kernel's sums batched: 368 -> 362 us a step of the
 // ResNet-20-shaped set, 5074 -> 5005 of the ResNet-50-shaped set, 342 -> 321 of one with odd sizes.
-template <bool EARLY>
+template <bool SUMMED>
 __global__ void __launch_bounds__(256) moments_mat_kernel(const __grid_constant__ GroupDev g,
                                                           const __grid_constant__ Rows64 rows,
                                                           const __grid_constant__ MomentArgs a,
                                                           const __grid_constant__ PtrTable W,
                                                           const __grid_constant__ PtrTable b) {
-  if (EARLY) dep_trigger();
-  else dep_sync();
+  dep_sync();
   const int nbias = a.bias_blocks * g.n;
   if ((int)blockIdx.x < nbias) {
     // the first CTAs carry the bias compensation (Eq. 31), which needs the means only: long rows of W start early
     // and the tiles fill in behind them
-    if (EARLY) dep_wait();
     const int layer = (int)blockIdx.x / a.bias_blocks, blk = (int)blockIdx.x - layer * a.bias_blocks;
     bias_comp_rows(g.layer[layer], reinterpret_cast<const float*>(W.p[layer]),
                    const_cast<float*>(reinterpret_cast<const float*>(b.p[layer])), blk, threadIdx.x);
     return;
   }
-  const int tile_id = (int)blockIdx.x - nbias;
-  int li = 0;
-#pragma unroll 1
-  for (int i = 1; i < g.n; ++i)
-    if (tile_id >= a.tt.tile0[i]) li = i;
-  const LayerDev* L = g.layer[li];
-  const int M = L->M;
   int bi, bj;
-  tri_decode(tile_id - a.tt.tile0[li], (M + 31) / 32, bi, bj);
+  const int li = find_tile(g, a, (int)blockIdx.x - nbias, bi, bj);
+  const LayerDev* L = g.layer[li];
   __shared__ float tile[32][33];
   const float inv_rows = 1.0f / (float)rows.v[li];
-  if ((M & 3) == 0) moments_tile<true, EARLY>(L, a, li, inv_rows, bi, bj, tile);
-  else moments_tile<false, EARLY>(L, a, li, inv_rows, bi, bj, tile);
+  if ((L->M & 3) == 0) moments_tile<true, SUMMED>(L, a, li, inv_rows, bi, bj, tile);
+  else moments_tile<false, SUMMED>(L, a, li, inv_rows, bi, bj, tile);
 }
 
 // A call that leaves its block open (FW_COV_ACCUMULATE): the split sums of this call are added, in split order,
@@ -618,19 +655,19 @@ cudaError_t launch_moments(const GroupDev& g, const Rows64& rows, const int32_t*
   }
   const int total = fill_tile_table(a.tt, layer_M, g.n);
   a.bias_blocks = any_params ? (max_N + 7) / 8 : 0;
-  // Side by side where both fit the chip at once, a CTA an SM: covariance update of 64 x 128 rows 15.1 -> 13.4 us, 147 x 3000 52 -> 35,
-  // 400 x 2000 44 -> 32, 402 x 6000 127 -> 96.  Not with few tiles that have many splits to add (75 x 7504 109 -> 119 us a step,
-  // M = 27 beside other sizes 173 -> 187): there the CTAs of the tiles, started later, are what the launch waits for.
-  a.early = total + a.bias_blocks * g.n + g.n <= sm_count();
-  for (int i = 0; i < g.n; ++i) {
-    const int t = (layer_M[i] + 31) / 32;
-    if (splits[i] > 8 && t * (t + 1) / 2 < 12) a.early = 0;
-  }
+  // The tiles' split partials are added beside the vectors where the CTAs of both are on the chip at once, two of 1024 threads an SM.
+  // fp32 sums, all in moments_mat_kernel and side by side: covariance update of 64 x 128 rows 16.0 and 15.4 us, 147 x 3000 53 and 29,
+  // 75 x 7504 49 and 43, 27 x 30000 62 and 51, 402 x 6000 128 and 107, 576 x 6000 109 and 83; tensor cores 64 x 20000 34.7 and
+  // 32.7, 700 x 3000 50 and 42.  (1000 x 2000, 530 tiles: 47.4, side by side 43.7, but such a launch is no longer one wave.)  A block of
+  // several calls holds its sums in gram_acc, of which moments_vec_kernel reads the diagonal.
+  bool side = g.n + total <= 2 * sm_count();
+  for (int i = 0; i < g.n; ++i) side = side && !use_acc[i];
+  a.sum_blocks = side ? total : 0;
   cudaError_t e;
-  { ProfScope ps(FW_PROF_MOMENTS, s); e = launch_dep(moments_vec_kernel, g.n, 1024, 0, s, g, rows, a); }
+  { ProfScope ps(FW_PROF_MOMENTS, s); e = launch_dep(moments_vec_kernel, g.n + a.sum_blocks, 1024, 0, s, g, rows, a); }
   if (e != cudaSuccess) return e;
   ProfScope ps(FW_PROF_MOMENTS, s);
-  return launch_dep(a.early ? moments_mat_kernel<true> : moments_mat_kernel<false>, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
+  return launch_dep(side ? moments_mat_kernel<true> : moments_mat_kernel<false>, total + a.bias_blocks * g.n, 256, 0, s, g, rows, a, W, b);
 }
 
 cudaError_t launch_pad_nhwc(int n, const float* const* src, float* const* dst, const int* B, const int* H, const int* W,
