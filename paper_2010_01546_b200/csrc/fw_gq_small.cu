@@ -4,8 +4,8 @@
 // 32 columns and its K is shared by a cluster of one, two, four or eight CTAs, at most 168 each: a CTA brings its whole share of both
 // operands to shared memory in one go (one trip to memory), multiplies it with warp-level TF32 instructions, and the
 // cluster's partial tiles are added in rank order out of shared memory.  With so little to do for each CTA the start-up of tcgen05
-// (allocation, descriptors, commit and read-back) costs more than its rate gains.  (The instruction reads
-// the leading 19 bits of its operands, as tcgen05 does.)
+// (allocation, descriptors, commit and read-back) costs more than its rate gains.  (Operands go in as they are.  PTX leaves the
+// low 13 bits of a TF32 operand open; measured, the instruction ignores them, as tcgen05 does.)
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -159,18 +159,33 @@ __global__ void __launch_bounds__(GS_THREADS) gq_small_kernel(const __grid_const
 
 }  // namespace
 
-// Small layers whose tiles, counted by their rows, come to no more than a CTA an SM: one product of 64 x 576 takes 6.8 us here and
-// 8.0 by CTA pairs, 32 x 288 4.9 and 6.9, 128 x 576 7.0 and 8.9, 20 x 1000 5.8 and 9.2; but 64 x 1024 9.8 and 8.4, the fifteen of
-// a ResNet-20-shaped set 19 and 13.5.  16-byte accesses throughout: rows of whole float4s and aligned matrices.
+// Every problem of a launch gets the cluster of the longest (a launch for each size of cluster took longer: 300 x 64 three times beside 144 x
+// 32 and 576 x 16, eight layers, 16.0 us for 9.7, by CTA pairs 12.0), so three things are asked for:
+// - rows: tiles with the K that they need, counted by their rows, come to no more than 64 rows an SM.  One product of 64 x 576 takes
+//   6.8 us here and 8.0 by CTA pairs, 32 x 288 4.9 and 6.9, 128 x 576 7.0 and 8.9, 20 x 1000 5.8 and 9.2; but 64 x 1024 9.8 and 8.4, the
+//   fifteen of a ResNet-20-shaped set 19 and 13.5.
+// - where K is shared by four CTAs or more, no more tiles than nine to ten SMs for each launch that the pairs need (sixteen layers), however few
+//   rows they have: 10 x 576 six times 9.7 and 11.7 us, eight times 12.6 and 11.8, twelve times 17.6 and 11.9; 1 x 1000 four times 13.5 and
+//   18.4, eight times 25.3 and 18.7, sixteen times 53 and 20.  (Below that 10 x 300 64 times: 34.9 and 39.9.)
+// - CTAs beyond those that the layers' own K takes: no more than one an SM.  10 x 1000 beside fifteen of 16 x 144 is 856 for 331: 14.3 and
+//   11.4 us; beside 32 x 576, 32 x 300 and 32 x 64, 496 for 350: 10.1 and 13.6.
+// 16-byte accesses throughout: rows of whole float4s and aligned matrices.
 bool gq_small_eligible(const UmmaGqItem* items, int n) {
-  int64_t rows = 0;
+  int64_t rows = 0, tiles = 0, ctas = 0;
+  int cl = 1;
   for (int i = 0; i < n; ++i) {
     const UmmaGqItem& it = items[i];
     const uintptr_t p = (uintptr_t)it.Qs | (uintptr_t)it.G | (uintptr_t)it.out;
     if (it.N > GS_MAX_N || it.M > GS_MAX_M || it.M % 4 != 0 || (p & 15) != 0 || it.colbias) return false;
-    rows += (int64_t)((it.M + GS_M - 1) / GS_M) * it.N * gs_cluster(it.M);
+    const int64_t wide = (it.M + GS_M - 1) / GS_M, t = wide * ((it.N + GS_N - 1) / GS_N);
+    const int c = gs_cluster(it.M);
+    rows += wide * it.N * c; tiles += t; ctas += t * c;
+    cl = std::max(cl, c);
   }
-  return rows <= (int64_t)GS_N * sm_count();
+  const int64_t sms = sm_count();
+  if (rows > GS_N * sms) return false;
+  if (cl >= 4 && 10 * tiles > 9 * sms * ((n + GS_MAX - 1) / GS_MAX)) return false;
+  return cl * tiles - ctas <= sms;
 }
 
 fw_status gq_small_launch(const UmmaGqItem* items, int n, int epi, float lr, int prof_class, cudaStream_t s) {
