@@ -816,6 +816,9 @@ __host__ __device__ inline int slab_vec(int M, int n) {
 }
 constexpr int kVecs = 6 + 2 * KH;
 
+// SOLO: all layers take one CTA and eight lanes a row; any number of steps.  (A kernel of its own: the loop round run_solo costs
+// run_steps registers where both are called, M = 576, K = 8, P = 16 160 -> 162 us.)
+template <bool SOLO>
 __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_constant__ ClusterArgs a) {
   dep_sync();
   cg::cluster_group cluster = cg::this_cluster();
@@ -878,8 +881,10 @@ __global__ void __launch_bounds__(CT, 1) recursion_cluster_kernel(const __grid_c
     float* tr = const_cast<float*>(reinterpret_cast<const float*>(a.traces.p[layer]));
     if (tr) tr += 4 * a.k0;
     const bool last = a.last != 0;
-    if (M <= kSolo) {
+    if (SOLO) {
       for (int k = 0; k < a.K; k += KH) run_solo(s, L, tr ? tr + 4 * k : nullptr, min(KH, a.K - k), a.P, last && k + KH >= a.K);
+    } else if (M <= kSolo) {
+      run_solo(s, L, tr, a.K, a.P, last);
     } else if (ng == 1) {
       switch (it) {
         case 1: run_steps<1, 1>(s, l, L, tr, a.K, a.P, last); break;
@@ -995,7 +1000,7 @@ bool recursion_cluster_supported(int M) { return recursion_cluster_ctas(M) > 0; 
 
 cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, const int* layer_M, int K, int P,
                                      cudaStream_t s) {
-  static SmemAttrCache attr;
+  static SmemAttrCache attr, solo_attr;
   static std::mutex mu;
   static int resident[64][5];        // clusters of 1, 2, 4, 8, 16 CTAs that run together (16: 7 on a B200)
   thread_local ClusterPlan plan;
@@ -1016,13 +1021,15 @@ cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, 
     std::lock_guard<std::mutex> lock(mu);
     if (resident[dev][0] == 0) {
       // clusters of 16 CTAs are beyond the portable size of 8
-      cudaError_t e = cudaFuncSetAttribute(recursion_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e == cudaSuccess) e = ensure_dyn_smem(recursion_cluster_kernel, kSmemLimit, attr);
+      cudaError_t e = cudaFuncSetAttribute(recursion_cluster_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(recursion_cluster_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) e = ensure_dyn_smem(recursion_cluster_kernel<false>, kSmemLimit, attr);
+      if (e == cudaSuccess) e = ensure_dyn_smem(recursion_cluster_kernel<true>, kSmemLimit, solo_attr);
       if (e != cudaSuccess) return e;
       for (int b = 4; b >= 0; --b) {
         int nc = 0;
         config(cfg, at, 1 << b, CLMAX * 64, kSmemLimit);
-        if (cudaOccupancyMaxActiveClusters(&nc, recursion_cluster_kernel, &cfg) != cudaSuccess || nc < 1) {
+        if (cudaOccupancyMaxActiveClusters(&nc, recursion_cluster_kernel<false>, &cfg) != cudaSuccess || nc < 1) {
           cudaGetLastError();
           nc = 1;
         }
@@ -1060,13 +1067,14 @@ cudaError_t launch_recursion_cluster(const GroupDev& g, const PtrTable& traces, 
   config(cfg, at, plan.cl, plan.bins * plan.cl, smem);
   // A launch is KH steps.  Layers of one CTA each take all of the call's in one: a launch of theirs costs as much as two steps
   // without power iterations (M = 64, K = 32, P = 0: 93 us in four launches, 77 in one).  Where a cluster exchanges, the steps
-  // are long and the same loop in the kernel costs each of them more registers than it saves launches (M = 576, K = 8, P = 16:
-  // 160 us, with the loop 172; K = 64, P = 4: 559 and 560).
+  // are long and a loop round run_steps costs each of them more than it saves launches (M = 576, K = 8, P = 16: 160 us, with the
+  // loop 172; K = 64, P = 4: 559 and 560).
   const int most = solo ? K : KH;
   for (int k0 = 0; k0 < K; k0 += most) {
     a.k0 = k0; a.K = std::min(most, K - k0); a.last = k0 + a.K == K;
     ProfScope ps(FW_PROF_RECUR_CHIP, s);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, recursion_cluster_kernel, a);
+    const cudaError_t e = solo ? cudaLaunchKernelEx(&cfg, recursion_cluster_kernel<true>, a)
+                               : cudaLaunchKernelEx(&cfg, recursion_cluster_kernel<false>, a);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
